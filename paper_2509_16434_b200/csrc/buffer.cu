@@ -151,33 +151,44 @@ struct CopySeg {
     const char *src;
     char *dst;
     unsigned long long bytes;
-    int vec;  // 16 when both ends and the size allow 128-bit accesses, else 1
+    uint32_t block_end;  // blocks of the segments up to and including this one
+    uint32_t vec;        // 16 or 4 when both ends and the size allow such accesses, else 1
 };
 struct CopySegs {
     CopySeg s[7];
 };
 
-// blockIdx.y selects the segment; blocks stride over it with 128-bit (or byte) accesses.
-__global__ void __launch_bounds__(256) write_step_kernel(CopySegs segs) {
-    const CopySeg sg = segs.s[blockIdx.y];
-    const unsigned long long tid = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const unsigned long long nth = (unsigned long long)gridDim.x * blockDim.x;
-    if (sg.vec == 16) {
-        const uint4 *s = reinterpret_cast<const uint4 *>(sg.src);
-        uint4 *d = reinterpret_cast<uint4 *>(sg.dst);
-        const unsigned long long n = sg.bytes >> 4;
-        unsigned long long i = tid;
-        for (; i + 3 * nth < n; i += 4 * nth) {
-            uint4 a = __ldcs(s + i), b = __ldcs(s + i + nth), c = __ldcs(s + i + 2 * nth), e = __ldcs(s + i + 3 * nth);
-            d[i] = a;
-            d[i + nth] = b;
-            d[i + 2 * nth] = c;
-            d[i + 3 * nth] = e;
-        }
-        for (; i < n; i += nth) d[i] = __ldcs(s + i);
-    } else {
-        for (unsigned long long i = tid; i < sg.bytes; i += nth) sg.dst[i] = sg.src[i];
+constexpr uint32_t kCopyBlockBytes = 16384;  // per block: four 128-bit accesses in flight per thread
+
+template <typename V>
+__device__ __forceinline__ void copy_strided(const char *src, char *dst, uint32_t bytes) {
+    const V *s = reinterpret_cast<const V *>(src);
+    V *d = reinterpret_cast<V *>(dst);
+    const uint32_t n = bytes / sizeof(V);
+    uint32_t i = threadIdx.x;
+    for (; i + 3 * 256 < n; i += 4 * 256) {
+        const V a = __ldcs(s + i), b = __ldcs(s + i + 256), c = __ldcs(s + i + 512), e = __ldcs(s + i + 768);
+        __stcs(d + i, a);
+        __stcs(d + i + 256, b);
+        __stcs(d + i + 512, c);
+        __stcs(d + i + 768, e);
     }
+    for (; i < n; i += 256) __stcs(d + i, __ldcs(s + i));
+}
+
+// A pure copy, bound by HBM.  Every block moves one 16 KB piece of one segment: the blocks are dealt out in proportion
+// to the segments' sizes (a grid with one row of blocks per segment spends most of its time starting the empty blocks
+// of the six small ones: 36 us instead of 14 us for the 39 MB of a 1024-env step of 160 x 120 frames).
+__global__ void __launch_bounds__(256) write_step_kernel(const __grid_constant__ CopySegs segs) {
+    uint32_t k = 0, first = 0;
+    while (blockIdx.x >= segs.s[k].block_end) first = segs.s[k++].block_end;
+    const CopySeg &sg = segs.s[k];
+    const unsigned long long off = (unsigned long long)(blockIdx.x - first) * kCopyBlockBytes;
+    const unsigned long long left = sg.bytes - off;
+    const uint32_t bytes = left < kCopyBlockBytes ? (uint32_t)left : kCopyBlockBytes;
+    if (sg.vec == 16) copy_strided<uint4>(sg.src + off, sg.dst + off, bytes);
+    else if (sg.vec == 4) copy_strided<uint32_t>(sg.src + off, sg.dst + off, bytes);
+    else copy_strided<uint8_t>(sg.src + off, sg.dst + off, bytes);
 }
 
 // Copies up to 7 per-env arrays of one step into slab row t (null sources are skipped).
@@ -189,25 +200,24 @@ static int write_fields(ppo_buffer *b, int t, const void *const srcs[7], void *s
     const size_t per_env[7] = {(size_t)d.H * d.W * 2, (size_t)d.P * 4, (size_t)d.A * 4, 4, 4, 4, 1};
     CopySegs segs;
     int n = 0;
-    size_t largest = 0;
+    unsigned long long blocks = 0;
     for (int i = 0; i < 7; ++i) {
         if (!srcs[i]) continue;
         size_t bytes = N * per_env[i];
         char *dst = b->base + b->field_off[fields[i]] + (size_t)t * bytes;
+        const uintptr_t bits = reinterpret_cast<uintptr_t>(srcs[i]) | reinterpret_cast<uintptr_t>(dst) | bytes;
+        blocks += (bytes + kCopyBlockBytes - 1) / kCopyBlockBytes;
+        if (blocks > 0x7fffffffull) return PPO_ERR_UNSUPPORTED;
         segs.s[n].src = static_cast<const char *>(srcs[i]);
         segs.s[n].dst = dst;
         segs.s[n].bytes = bytes;
-        segs.s[n].vec = (ppo_aligned(srcs[i], 16) && ppo_aligned(dst, 16) && bytes % 16 == 0) ? 16 : 1;
-        largest = bytes > largest ? bytes : largest;
+        segs.s[n].block_end = (uint32_t)blocks;
+        segs.s[n].vec = bits % 16 == 0 ? 16u : (bits % 4 == 0 ? 4u : 1u);
         ++n;
     }
     b->gae_valid = false;
     if (n == 0) return PPO_OK;
-    // enough blocks to cover the largest segment with ~4 x 16 B per thread, capped at a few waves
-    long long units = (long long)(largest / 16 / 4 / 256) + 1;
-    int gx = (int)(units < (long long)ppo_num_sms() * 16 ? units : (long long)ppo_num_sms() * 16);
-    dim3 grid(gx, n);
-    write_step_kernel<<<grid, 256, 0, static_cast<cudaStream_t>(stream)>>>(segs);
+    write_step_kernel<<<(unsigned)blocks, 256, 0, static_cast<cudaStream_t>(stream)>>>(segs);
     PPO_LAUNCH_CHECK();
     return PPO_OK;
 }
