@@ -1,0 +1,885 @@
+// 3x3 stride-2 convolutions whose weights fit in shared memory: forward and input gradient as one kind of GEMM on
+// halo tiles (sm_100a).
+//
+// The forward pass of a stride-2 convolution reads its input through four planes, the parities of row and column: plane
+// (py, px) holds the pixels (2v + py, 2u + px) and is a plain 4-D tensor to the copy engine (base and strides adjusted).
+// In its plane every kernel tap is a shift by 0 or -1.  The input gradient reads one plane, dY itself, at shifts 0 or
+// +1.  So a tile of Wt x R outputs (of I images) needs, per plane, one box of (Wt + 1) x (R + 1) cells, and the A operand
+// of a tap is that box read from another start address: row m of the MMA is cell m + shift.  The swizzle is a function
+// of the shared-memory address, so a matrix may start at any row of a swizzled image.  Rows that fall on the halo
+// column or row compute values nobody stores.
+//
+// Against one box per tap (gemm_tma.cu) this brings a third to a half of the bytes into shared memory with one copy per
+// plane, and all three serial streams that bounded these layers get shorter: the copy-issuing thread, the MMA-issuing
+// thread (unrolled taps; no zero blocks in the input gradient), and the epilogue (outputs leave as one bulk tensor store
+// per 64 columns and tile, clipped at the edges by the copy engine, instead of a shuffle, a load and a store per 16 bytes;
+// ReLU gates are fetched a tile ahead).  The weights stay in shared memory for the life of the CTA.  Sums run in the same
+// order as in gemm_tma.cu: the results are the same bits.
+// Measured, 4096 rows (against the HBM time of inputs, gates and outputs): 32 -> 64 channels on 160 x 120 forward
+// 2.22 -> 1.29 ms (1.17), input gradient 3.25 -> 1.37 (1.2); 64 -> 128 on 80 x 60 forward 1.20 -> 1.08 (0.58), input
+// gradient 1.58 -> 1.00 (0.6).
+#include <cuda.h>
+
+#include "gemm.cuh"
+#include "tcgen05.cuh"
+#include "tma_host.cuh"
+
+namespace {
+
+using namespace tc;
+
+constexpr int kEpiWarps = 8;  // of an epilogue group; a CTA that has the SM to itself runs two groups on alternate tiles
+
+constexpr int kMaxSlots = 8;
+constexpr int kMaxOps = 9;
+constexpr size_t kSmemMax = 227 * 1024;
+
+enum { FWD = 0, FWD_LN = 1, DG_BITS = 2, DG_ACT = 3 };
+
+// One tap of a plane: CB / 16 MMAs over the channels of a chunk.
+struct Op {
+    uint32_t a16;    // start of the A rows inside the plane's box, in 16-byte units
+    uint32_t b16;    // start of the weights of chunk 0, in 16-byte units
+    uint32_t dcol;   // first accumulator column
+    uint32_t idesc;  // instruction descriptor (column count)
+};
+
+struct Plane {
+    int ox, oy;      // box origin relative to the tile's first output cell
+    uint32_t bytes;  // of its box
+};
+
+struct WLoad {       // one box of weights: rows of one tap (all chunks loaded one after the other)
+    int k0;          // column of the weight matrix, without the chunk
+    uint32_t off;    // destination of chunk 0
+};
+
+struct Args {
+    CUtensorMap mapA[4];    // planes
+    CUtensorMap mapW;
+    CUtensorMap mapO[4];    // output groups (forward: one map, the group is the first coordinate)
+    CUtensorMap mapX;       // normalised values
+    Op ops[kMaxOps];
+    Plane planes[4];
+    WLoad wl[kMaxOps];
+    int nplanes, nwl, nchunks, nloads, CB, rb;
+    uint32_t w_chunk;       // bytes of the weights of one chunk
+    uint32_t w_box;         // bytes of one box of weights
+    uint32_t slot_bytes, slots_bytes;  // of one slot; of all of them, rounded up
+    uint32_t stg_bytes;     // of a staging buffer
+    int slots, nbuf, neg;   // slots, staging buffers per epilogue group, epilogue groups
+    int Wt, R, I, Wp, Rp;   // tile: Wt x R outputs of I images; cells per box row and box rows per image
+    int xsegs, ysegs, tiles;
+    int Hr, Wr, B;          // grid of outputs (forward) or of 2x2 input blocks (input gradient)
+    int N;                  // accumulator columns
+    int acc_cols, nacc;
+    int Hi, Wi;             // input gradient: the image that is written
+    const float *bias;
+    int relu;
+    uint32_t *out_bits;
+    const uint32_t *mask_bits;
+    const bf16 *mask;
+    const float *ln_gamma, *ln_beta;
+    float *ln_rstd;
+    int grid;
+    size_t smem;
+    int32_t *status;
+};
+
+struct Pipe {
+    uint64_t full[kMaxSlots], empty[kMaxSlots], tfull[4], tempty[4], wfull;
+    uint32_t tmem_slot;
+    int abort_flag;
+    alignas(16) float bias[256], gamma[256], beta[256];
+};
+
+__device__ __forceinline__ void tma_store_4d(const void *map, uint32_t src, int c0, int c1, int c2, int c3) {
+    asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5}], [%1];" ::"l"(
+                     reinterpret_cast<uint64_t>(map)),
+                 "r"(src), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+                 : "memory");
+}
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void bulk_wait_read() {
+    asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+__device__ __forceinline__ void epi_sync(int eg) { asm volatile("bar.sync %0, %1;" ::"r"(1 + eg), "n"(kEpiWarps * 32) : "memory"); }
+
+// 32 consecutive fp32 columns of this thread's TMEM lane.
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float *v) {
+    uint32_t r[32];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+          "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(taddr)
+        : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// The sign bits of bytes 1 and 3, each replicated over its half word (prmt.b32 in its sign-replicating form).
+__device__ __forceinline__ uint32_t half_signs(uint32_t x) {
+    uint32_t r;
+    asm("prmt.b32 %0, %1, 0, 0xBB99;" : "=r"(r) : "r"(x));
+    return r;
+}
+// Pair j of the 32-channel gate word (bits j and 16 + j) as a mask over the two halves.
+__device__ __forceinline__ uint32_t gate_mask(uint32_t gate, int j) { return half_signs(gate << (15 - j)); }
+
+// Slots in the order they become free: four bits each, the next one lowest.  Producer and MMA warp walk the same
+// sequence, so a slot that is read for the last time early in a tile takes the next tile's first load.
+struct SlotQueue {
+    uint32_t q;
+    int n;
+    __device__ void init(int slots) {
+        q = 0x76543210u;
+        n = slots;
+    }
+    __device__ int pop() {
+        const int s = (int)(q & 15u);
+        q >>= 4;
+        --n;
+        return s;
+    }
+    __device__ void push(int s) {
+        q = (q & ~(15u << (4 * n))) | ((uint32_t)s << (4 * n));
+        ++n;
+    }
+};
+
+struct TileAt {
+    int n, y, x;  // first image, row and column of the tile
+    __device__ void init(const Args &a, int t) {
+        const int xs = t % a.xsegs;
+        t /= a.xsegs;
+        const int ys = t % a.ysegs;
+        n = t / a.ysegs * a.I;
+        x = xs * a.Wt;
+        y = ys * a.R;
+    }
+    __device__ void next(const Args &a) {
+        x += a.Wt;
+        if (x >= a.Wr) {
+            x = 0;
+            y += a.R;
+            if (y >= a.Hr) {
+                y = 0;
+                n += a.I;
+            }
+        }
+    }
+};
+
+// Barrier of an epilogue group that also ANDs a condition over them (a bounded wait that ran out in one warp ends all).
+__device__ __forceinline__ bool epi_all(bool ok, int eg) {
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %1, 0;\n\t"
+        "bar.red.and.pred q, %3, %2, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(r)
+        : "r"(ok ? 1u : 0u), "n"(kEpiWarps * 32), "r"(1 + eg)
+        : "memory");
+    return r != 0;
+}
+
+// GC: columns of an output group, i.e. of one pixel of one store (16, 32 or 64; its bytes are the swizzled row).
+// KS: K = 16 steps per channel chunk (1, 2 or 4: rows of 32, 64 or 128 bytes).
+template <int MODE, int GC, int KS>
+__global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a) {
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    const uint32_t smem_base = smem_u32(smem);
+    // A slots, then weights (reads of the last slot's halo rows may run on into them), output staging, pipeline state
+    const uint32_t w_base = smem_base + a.slots_bytes;
+    const uint32_t w_bytes = (uint32_t)a.nchunks * a.w_chunk;
+    const uint32_t stg_off = (a.slots_bytes + w_bytes + 1023u) & ~1023u;
+    Pipe *pipe = reinterpret_cast<Pipe *>(smem + stg_off + (size_t)(a.nbuf * a.neg) * a.stg_bytes);
+    volatile int *abort_flag = &pipe->abort_flag;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int nacc = a.nacc;
+    const uint32_t ncols = (uint32_t)(a.acc_cols * nacc);
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < a.slots; ++s) {
+            mbar_init(&pipe->full[s], 1);
+            mbar_init(&pipe->empty[s], 1);
+        }
+        for (int i = 0; i < nacc; ++i) {
+            mbar_init(&pipe->tfull[i], 1);
+            mbar_init(&pipe->tempty[i], kEpiWarps * 32);
+        }
+        mbar_init(&pipe->wfull, 1);
+        pipe->abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (MODE == FWD || MODE == FWD_LN)
+        for (int i = threadIdx.x; i < a.N; i += (int)blockDim.x) {
+            pipe->bias[i] = a.bias[i];
+            if (MODE == FWD_LN) {
+                pipe->gamma[i] = a.ln_gamma[i];
+                pipe->beta[i] = a.ln_beta[i];
+            }
+        }
+    if (warp == 1) tmem_alloc(&pipe->tmem_slot, ncols);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = pipe->tmem_slot;
+
+    // contiguous run of tiles for this CTA
+    const int q = a.tiles / (int)gridDim.x, rem = a.tiles - q * (int)gridDim.x, bid = (int)blockIdx.x;
+    const int t0 = bid * q + (bid < rem ? bid : rem), nt = q + (bid < rem ? 1 : 0);
+
+    if (warp == 0) {
+        if (lane == 0) {
+            mbar_arrive_expect_tx(&pipe->wfull, w_bytes);
+            for (int c = 0; c < a.nchunks; ++c)
+                for (int i = 0; i < a.nwl; ++i)
+                    tma_load_2d(w_base + (uint32_t)c * a.w_chunk + a.wl[i].off, &a.mapW, &pipe->wfull, a.wl[i].k0 + c * a.CB, 0);
+            TileAt t;
+            t.init(a, t0);
+            SlotQueue sq;
+            sq.init(a.slots);
+            uint32_t phase = 0, armed = 0;  // per slot: parity of its next use; whether it was ever filled
+            bool ok = true;
+            for (int li = 0; li < nt && ok; ++li, t.next(a)) {
+                uint32_t used = 0;  // the tile's slots in the order of its loads
+                for (int i = 0; i < a.nloads; ++i) {  // forward: the planes in the order of their first tap; else the chunks
+                    const int p = a.nplanes == 4 ? 3 - i : 0, s = sq.pop();
+                    const Plane &pl = a.planes[p];
+                    used |= (uint32_t)s << (4 * i);
+                    ok = mbar_wait(&pipe->empty[s], (~phase >> s) & 1u, abort_flag, a.status);
+                    if (!ok) break;
+                    phase ^= 1u << s;
+                    armed |= 1u << s;
+                    mbar_arrive_expect_tx(&pipe->full[s], pl.bytes);
+                    tma_load_4d(smem_base + (uint32_t)s * a.slot_bytes, &a.mapA[p], &pipe->full[s], a.nplanes == 4 ? 0 : i * a.CB,
+                                t.x + pl.ox, t.y + pl.oy, t.n);
+                }
+                if (a.nplanes == 4) used = (used >> 8) | (used << 8 & 0xFF00u);  // planes 01 and 00 are done first
+                for (int i = 0; i < a.nloads; ++i) sq.push((int)(used >> (4 * i)) & 15);
+            }
+            if (!ok) {  // bounded wait for the copies in flight
+                for (int s = 0; s < a.slots; ++s) {
+                    if (!((armed >> s) & 1u)) continue;
+                    const long long c0 = clock64();
+                    while (!mbar_try_wait(&pipe->full[s], (~phase >> s) & 1u))
+                        if (clock64() - c0 > kWaitCycles / 4) break;
+                }
+            }
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        // One thread feeds the tensor core and its instruction stream is what bounds the narrow layers, so the taps of a
+        // plane are unrolled: everything but the slot's address is a constant of the launch.
+        // The sums run in the order tap, channel (and shift, channel), whatever the order of the loads.
+        constexpr bool kFwd = MODE == FWD || MODE == FWD_LN;
+        constexpr uint32_t rb = KS * 32u, sbo = 8u * rb;
+        const uint64_t d0 = smem_desc_sw(smem_base, 16, sbo, rb);
+        const uint32_t a_lo0 = (uint32_t)d0, d_hi = (uint32_t)(d0 >> 32);
+        const uint32_t w_lo0 = a_lo0 + ((w_base - smem_base) >> 4);
+        const uint32_t slot16 = a.slot_bytes >> 4, wchunk16 = a.w_chunk >> 4;
+        SlotQueue sq;
+        sq.init(a.slots);
+        int acc = 0;
+        uint32_t phase = 0, aph = 1u;  // parities of the slots; parity that says the accumulator has been drained
+        bool ok = mbar_wait(&pipe->wfull, 0, abort_flag, a.status);
+        auto taps = [&](int o, uint32_t la0, uint32_t lb0, uint32_t tmem_d, uint32_t accum) {
+            const Op &op = a.ops[o];
+            const uint32_t la = la0 + op.a16, lb = lb0 + op.b16, td = tmem_d + op.dcol, id = op.idesc;
+            umma_bf16_lh(td, la, d_hi, lb, d_hi, id, accum);
+#pragma unroll
+            for (int k = 1; k < KS; ++k) umma_bf16_lh(td, la + 2 * k, d_hi, lb + 2 * k, d_hi, id, 1u);
+        };
+        for (int li = 0; li < nt && ok; ++li) {
+            ok = mbar_wait(&pipe->tempty[acc], aph, abort_flag, a.status);
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t tmem_d = tmem_base + (uint32_t)(acc * a.acc_cols);
+            if (kFwd) {
+                // planes 11, 10, 01, 00 sit in four consecutive slots; taps in raster order need them in that order
+                int sl[4];
+                uint32_t la[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    sl[i] = sq.pop();
+                    la[i] = a_lo0 + (uint32_t)sl[i] * slot16;
+                }
+#pragma unroll
+                for (int t = 0; t < 9; ++t) {
+                    constexpr int kLoad[9] = {0, 1, 0, 2, 3, 2, 0, 1, 0};  // load that brings the tap's plane
+                    const int i = kLoad[t];
+                    if (t < 2 || t == 3 || t == 4) {
+                        ok = mbar_wait(&pipe->full[sl[i]], (phase >> sl[i]) & 1u, abort_flag, a.status);
+                        if (!ok) break;
+                        tc_fence_after();
+                    }
+                    if (lane == 0) {
+                        taps(t, la[i], w_lo0, tmem_d, t > 0 ? 1u : 0u);
+                        if (t == 5) {
+                            umma_commit(&pipe->empty[sl[2]]);
+                            umma_commit(&pipe->empty[sl[3]]);
+                        }
+                    }
+                    __syncwarp();
+                }
+                if (!ok) break;
+                if (lane == 0) {
+                    umma_commit(&pipe->empty[sl[0]]);
+                    umma_commit(&pipe->empty[sl[1]]);
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    phase ^= 1u << sl[i];
+                    sq.push(sl[i ^ 2]);
+                }
+            } else {
+                uint32_t used = 0;
+                for (int c = 0; c < a.nchunks; ++c) {
+                    const int s = sq.pop();
+                    used |= (uint32_t)s << (4 * c);
+                    ok = mbar_wait(&pipe->full[s], (phase >> s) & 1u, abort_flag, a.status);
+                    if (!ok) break;
+                    phase ^= 1u << s;
+                }
+                if (!ok) break;
+                tc_fence_after();
+                if (lane == 0) {
+#pragma unroll
+                    for (int o = 0; o < 4; ++o) {
+                        uint32_t lb = w_lo0;
+                        for (int c = 0; c < a.nchunks; ++c, lb += wchunk16) {
+                            const int s = (int)(used >> (4 * c)) & 15;
+                            taps(o, a_lo0 + (uint32_t)s * slot16, lb, tmem_d, o > 0 || c > 0 ? 1u : 0u);
+                            if (o == 3) umma_commit(&pipe->empty[s]);
+                        }
+                    }
+                }
+                for (int c = 0; c < a.nchunks; ++c) sq.push((int)(used >> (4 * c)) & 15);
+            }
+            if (lane == 0) umma_commit(&pipe->tfull[acc]);
+            __syncwarp();
+            if (++acc == nacc) { acc = 0; aph ^= 1u; }
+        }
+    } else {
+        // ---------------- epilogue: warp reads TMEM lanes 32 (warp % 4) .. +31 and, of every 64 columns, half `h`
+        const int lg = warp & 3, eg = (warp - 2) >> 3, h = ((warp - 2) >> 2) & 1;
+        const int m = lg * 32 + lane;
+        const int ci = m / (a.Rp * a.Wp), mr = m - ci * a.Rp * a.Wp, cr = mr / a.Wp, cx = mr - cr * a.Wp;
+        const bool cell = ci < a.I && cr < a.R && cx < a.Wt;  // an output of the tile, not a halo cell
+        const int srow = (ci * a.R + cr) * a.Wt + cx;         // its row in the dense staging tile
+        const bool issuer = threadIdx.x == 64 + eg * kEpiWarps * 32;
+        constexpr uint32_t RBO = GC * 2;                      // bytes of a staged row
+        const uint32_t sx = GC == 64 ? (uint32_t)(srow & 7) : (GC == 32 ? (uint32_t)(srow >> 1) & 3u : (uint32_t)(srow >> 2) & 1u);
+        const uint32_t grp_bytes = a.stg_bytes * GC / 64u;    // of an output group's part of a staging buffer
+        const int nsteps = (a.N + 63) >> 6;
+        int acc = eg, buf = 0;  // nacc is even where there are two groups
+        uint32_t aph = 0;
+        TileAt t;
+        t.init(a, t0 + (eg < nt ? eg : 0));
+        // columns col .. col + 7 (of the step's 64) of this thread's row
+        auto put = [&](uint32_t stg, int col, uint4 v) {
+            const uint32_t grp = (uint32_t)col / GC, piece = ((uint32_t)col % GC) >> 3;
+            const uint32_t addr = stg + grp * grp_bytes + (uint32_t)srow * RBO + ((piece ^ sx) << 4);
+            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+        };
+        auto stage_free = [&]() {  // the store that last read this buffer is done (asked by the thread that issued it)
+            if (issuer) {
+                if (a.nbuf == 2) bulk_wait_read<1>();
+                else bulk_wait_read<0>();
+            }
+        };
+        auto store_step = [&](uint32_t stg, int s, const CUtensorMap *maps) {
+            fence_async_smem();
+            epi_sync(eg);
+            if (issuer) {
+#pragma unroll
+                for (int g = 0; g < 64 / GC; ++g) {
+                    const int col = s * 64 + g * GC, grp = col / GC;
+                    if (col >= a.N) break;
+                    if (MODE == FWD || MODE == FWD_LN) {
+                        tma_store_4d(maps, stg + (uint32_t)g * grp_bytes, col, t.x, t.y, t.n);
+                    } else {  // parity classes in the order 00, 01, 11, 10
+                        const int ph = grp >> 1, pw = (grp == 1 || grp == 2) ? 1 : 0;
+                        if (2 * t.y + ph < a.Hi && 2 * t.x + pw < a.Wi)
+                            tma_store_4d(maps + grp, stg + (uint32_t)g * grp_bytes, 0, t.x, t.y, t.n);
+                    }
+                }
+                bulk_commit();
+            }
+            if (++buf == a.nbuf) buf = 0;
+        };
+        const uint32_t stg0 = smem_base + stg_off + (uint32_t)(eg * a.nbuf) * a.stg_bytes;
+        // ReLU gates of the pixels this thread's columns belong to.  They are fetched a tile ahead: this warp is what the
+        // tile waits for, so a load on its own tile's path would cost its whole latency.
+        uint32_t gate[4], gate_n[4];
+        uint4 act[4], act_n[4];
+        auto fetch_gates = [&](const TileAt &at) {
+            const int n = at.n + ci, y = at.y + cr, x = at.x + cx;
+            const bool live = cell && n < a.B && y < a.Hr && x < a.Wr;
+            if (MODE == DG_BITS) {
+#pragma unroll
+                for (int s = 0; s < 4; ++s) {
+                    gate_n[s] = 0u;
+                    const int col = s * 64 + h * 32, grp = col / GC;
+                    const int iy = 2 * y + (grp >> 1), ix = 2 * x + ((grp == 1 || grp == 2) ? 1 : 0);
+                    if (col < a.N && live && iy < a.Hi && ix < a.Wi)
+                        gate_n[s] = __ldg(a.mask_bits + (((long long)n * a.Hi + iy) * a.Wi + ix) * (GC / 32 > 0 ? GC / 32 : 1) + (GC == 64 ? h : 0));
+                }
+            }
+            if (MODE == DG_ACT) {  // GC == 16: this thread's 32 columns are two classes of 16 channels
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int grp = h * 2 + e;
+                    const int iy = 2 * y + (grp >> 1), ix = 2 * x + ((grp == 1 || grp == 2) ? 1 : 0);
+                    act_n[2 * e] = act_n[2 * e + 1] = make_uint4(0, 0, 0, 0);
+                    if (live && iy < a.Hi && ix < a.Wi) {
+                        const uint4 *mp = reinterpret_cast<const uint4 *>(a.mask + (((long long)n * a.Hi + iy) * a.Wi + ix) * 16);
+                        act_n[2 * e] = __ldg(mp);
+                        act_n[2 * e + 1] = __ldg(mp + 1);
+                    }
+                }
+            }
+        };
+        TileAt t_next = t;
+        if (eg < nt) fetch_gates(t);
+        for (int li = eg; li < nt; li += a.neg, t = t_next) {
+            const int n = t.n + ci, y = t.y + cr, x = t.x + cx;
+            const bool live = cell && n < a.B && y < a.Hr && x < a.Wr;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if (MODE == DG_BITS) gate[k] = gate_n[k];
+                if (MODE == DG_ACT) act[k] = act_n[k];
+            }
+            for (int k = 0; k < a.neg; ++k) t_next.next(a);
+            if (li + a.neg < nt) fetch_gates(t_next);
+            stage_free();
+            const bool ok = epi_all(mbar_wait(&pipe->tfull[acc], aph, abort_flag, a.status), eg);
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t lane_base = tmem_base + (uint32_t)(acc * a.acc_cols) + ((uint32_t)(lg * 32) << 16);
+            if (MODE == FWD_LN) {
+                // Layer normalisation over the N channels of this thread's row: the row is walked twice in tensor memory
+                // (mean, then variance about it), 16 columns at a time.  With 32 channels the two warps of a lane quarter
+                // take 16 columns each, else 32 of every 64.
+                float sum = 0.f, sq = 0.f;
+                for (int c0 = 0; c0 < a.N; c0 += 16) {
+                    float v[16];
+                    tmem_ld16(lane_base + (uint32_t)c0, v);
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) sum += v[i] + pipe->bias[c0 + i];
+                }
+                const float mean = sum / (float)a.N;
+                for (int c0 = 0; c0 < a.N; c0 += 16) {
+                    float v[16];
+                    tmem_ld16(lane_base + (uint32_t)c0, v);
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        const float d = v[i] + pipe->bias[c0 + i] - mean;
+                        sq += d * d;
+                    }
+                }
+                const float rs = rsqrtf(sq / (float)a.N + kLnEps);
+                const long long px = ((long long)n * a.Hr + y) * a.Wr + x;
+                if (live && h == 0) a.ln_rstd[px] = rs;
+                const bool narrow = a.N == 32;
+                const int nsub = narrow ? 1 : 2;
+#pragma unroll 1
+                for (int s = 0; s < nsteps; ++s) {
+                    if (s > 0) {
+                        stage_free();
+                        epi_sync(eg);
+                    }
+                    const uint32_t stg = stg0 + (uint32_t)buf * a.stg_bytes;
+                    const int cb = narrow ? h * 16 : s * 64 + h * 32;
+                    uint32_t keep[2][8];  // ReLU outputs of the sub-chunks, written after the normalised values have left
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        if (j < nsub && cb < a.N) {
+                            const int c0 = cb + 16 * j;
+                            float v[16];
+                            tmem_ld16(lane_base + (uint32_t)c0, v);
+                            uint32_t xh[8];
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) {
+                                const float x0 = (v[2 * i] + pipe->bias[c0 + 2 * i] - mean) * rs;
+                                const float x1 = (v[2 * i + 1] + pipe->bias[c0 + 2 * i + 1] - mean) * rs;
+                                xh[i] = pack_bf16x2(x0, x1);
+                                keep[j][i] = relu_pack_bf16x2(fmaf(pipe->gamma[c0 + 2 * i], x0, pipe->beta[c0 + 2 * i]),
+                                                              fmaf(pipe->gamma[c0 + 2 * i + 1], x1, pipe->beta[c0 + 2 * i + 1]));
+                            }
+                            if (cell) {
+                                put(stg, c0 & 63, make_uint4(xh[0], xh[1], xh[2], xh[3]));
+                                put(stg, (c0 & 63) + 8, make_uint4(xh[4], xh[5], xh[6], xh[7]));
+                            }
+                        }
+                    }
+                    if (s == nsteps - 1) {
+                        tc_fence_before();
+                        mbar_arrive(&pipe->tempty[acc]);
+                    }
+                    store_step(stg, s, &a.mapX);
+                    stage_free();
+                    epi_sync(eg);
+                    const uint32_t stg2 = stg0 + (uint32_t)buf * a.stg_bytes;
+                    if (cb < a.N) {
+                        uint32_t w = 0;
+#pragma unroll
+                        for (int j = 0; j < 2; ++j) {
+                            if (j < nsub) {
+                                if (cell) {
+                                    put(stg2, ((cb + 16 * j) & 63), make_uint4(keep[j][0], keep[j][1], keep[j][2], keep[j][3]));
+                                    put(stg2, ((cb + 16 * j) & 63) + 8, make_uint4(keep[j][4], keep[j][5], keep[j][6], keep[j][7]));
+                                }
+#pragma unroll
+                                for (int i = 0; i < 8; ++i) w = gate_bits_add(w, keep[j][i], 8 * j + i);
+                            }
+                        }
+                        if (a.out_bits && live) {
+                            if (narrow) {  // channels 16h .. 16h + 15: bytes h and 2 + h of the pixel's word
+                                uint8_t *bp = reinterpret_cast<uint8_t *>(a.out_bits + px);
+                                bp[h] = (uint8_t)w;
+                                bp[2 + h] = (uint8_t)(w >> 16);
+                            } else {
+                                a.out_bits[px * (a.N >> 5) + (cb >> 5)] = w;
+                            }
+                        }
+                    }
+                    store_step(stg2, s, &a.mapO[0]);
+                }
+                acc += a.neg;
+                if (acc >= nacc) { acc = eg; aph ^= 1u; }
+                continue;
+            }
+#pragma unroll 1
+            for (int s = 0; s < nsteps; ++s) {
+                const int c0 = s * 64 + h * 32;
+                const bool mine = c0 < a.N;  // uniform in a warp
+                float v[32];
+                if (mine) tmem_ld32(lane_base + (uint32_t)c0, v);
+                if (s == nsteps - 1) {  // the accumulator has been read by this warp
+                    tc_fence_before();
+                    mbar_arrive(&pipe->tempty[acc]);
+                }
+                if (s > 0) {
+                    stage_free();
+                    epi_sync(eg);
+                }
+                const uint32_t stg = stg0 + (uint32_t)buf * a.stg_bytes;
+                if (MODE == FWD) {
+                    if (mine) {
+                        const float4 *bp = reinterpret_cast<const float4 *>(pipe->bias + c0);
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) {
+                            const float4 b4 = bp[k];
+                            v[4 * k] += b4.x; v[4 * k + 1] += b4.y; v[4 * k + 2] += b4.z; v[4 * k + 3] += b4.w;
+                        }
+                    }
+                    if (mine) {
+                        uint32_t pk[16], w = 0;
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) {
+                            pk[j] = a.relu ? relu_pack_bf16x2(v[2 * j], v[2 * j + 1]) : pack_bf16x2(v[2 * j], v[2 * j + 1]);
+                            w = gate_bits_add(w, pk[j], j);
+                        }
+                        if (cell) {
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) put(stg, h * 32 + 8 * k, make_uint4(pk[4 * k], pk[4 * k + 1], pk[4 * k + 2], pk[4 * k + 3]));
+                        }
+                        if (a.out_bits && live) a.out_bits[(((long long)n * a.Hr + y) * a.Wr + x) * (a.N >> 5) + (c0 >> 5)] = w;
+                    }
+                } else if (MODE != FWD_LN && mine && cell) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        uint32_t pk[4];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const uint32_t pr = pack_bf16x2(v[8 * k + 2 * j], v[8 * k + 2 * j + 1]);
+                            if (MODE == DG_BITS) {
+                                const uint32_t gw = s == 0 ? gate[0] : (s == 1 ? gate[1] : (s == 2 ? gate[2] : gate[3]));
+                                pk[j] = pr & gate_mask(gw, 4 * k + j);
+                            } else {
+                                const uint4 &q4 = act[k];
+                                const uint32_t aw = j == 0 ? q4.x : (j == 1 ? q4.y : (j == 2 ? q4.z : q4.w));
+                                // stored activations are >= 0 (the outputs of a ReLU): a half gates unless it is zero
+                                pk[j] = pr & half_signs(aw + 0x7FFF7FFFu);
+                            }
+                        }
+                        put(stg, h * 32 + 8 * k, make_uint4(pk[0], pk[1], pk[2], pk[3]));
+                    }
+                }
+                store_step(stg, s, MODE == DG_BITS || MODE == DG_ACT ? a.mapO : &a.mapO[0]);
+            }
+            acc += a.neg;
+            if (acc >= nacc) { acc = eg; aph ^= 1u; }
+        }
+        if (issuer) bulk_wait_all();
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem_base, ncols);
+    }
+}
+
+// --------------------------------------------------------------------- host ----
+
+uint32_t stage_rows_bytes(int rows) { return ((uint32_t)rows * 128u + 1023u) & ~1023u; }
+
+// Tile rectangle whose loads (`loads` slots) and staging buffers (`bufs`) fit into `room` bytes: fewest tiles over the
+// whole grid, then fewest loaded cells.  The M rows of a tile (halo cells included, except behind its last row) have to
+// fit into the 128 rows of an MMA.
+bool choose_tile(Args &a, int Wr, int Hr, int B, size_t room, int loads, int bufs) {
+    long long best_t = -1, best_c = 0;
+    for (int xs = 1; xs <= Wr && xs <= 64; ++xs) {
+        const int Wt = (Wr + xs - 1) / xs, Wp = Wt + 1;
+        if (Wt > 128) continue;
+        int top = (128 - Wt) / Wp + 1;
+        if (top > Hr) top = Hr;
+        for (int R = top; R >= 1; --R) {
+            const int ysegs = (Hr + R - 1) / R;
+            if (R < top && (Hr + R) / (R + 1) == ysegs) continue;  // a taller tile makes as few segments
+            const int Re = (Hr + ysegs - 1) / ysegs;
+            int I = 1;
+            if (ysegs == 1 && xs == 1) {
+                const int per = (Re + 1) * Wp, last = (Re - 1) * Wp + Wt;
+                I = 1 + (128 - last) / per;
+                if (I > B) I = B;
+            }
+            auto fits = [&](int img) {
+                const size_t slot = ((size_t)img * (Re + 1) * Wp * a.rb + 127) & ~size_t(127);
+                return (size_t)loads * slot + (size_t)bufs * stage_rows_bytes(img * Re * Wt) <= room;
+            };
+            while (I > 1 && !fits(I)) --I;
+            if (!fits(I)) continue;
+            const long long tiles = (long long)((B + I - 1) / I) * ysegs * ((Wr + Wt - 1) / Wt);
+            const long long cells = tiles * I * (Re + 1) * Wp;
+            if (best_t < 0 || tiles < best_t || (tiles == best_t && cells < best_c)) {
+                best_t = tiles; best_c = cells;
+                a.Wt = Wt; a.R = Re; a.I = I;
+            }
+        }
+    }
+    if (best_t < 0 || best_t > 0x3fffffff) return false;
+    a.Wp = a.Wt + 1;
+    a.Rp = a.R + 1;
+    a.xsegs = (Wr + a.Wt - 1) / a.Wt;
+    a.ysegs = (Hr + a.R - 1) / a.R;
+    a.tiles = (int)best_t;
+    a.Hr = Hr; a.Wr = Wr; a.B = B;
+    return true;
+}
+
+// Division of shared and tensor memory, and the tile that goes with it.  A tile's loads (four planes, or one box per chunk)
+// are all held at once.  Two CTAs per SM, one epilogue group each, where the weights and a full-sized tile's loads and
+// staging fit into half of it; else one CTA with two epilogue groups, if need be with a smaller tile.  The epilogue is
+// the longest chain of a tile (read the accumulator, convert, stage, hand over, wait until the copy engine has read the
+// buffer), so it is what the second CTA or group is for; a CTA's only group stages into two buffers if they fit.  What
+// room is left goes to more slots, for the next tile's loads.
+bool plan(Args &a, int Wr, int Hr, int B) {
+    const size_t w = ((size_t)a.nchunks * a.w_chunk + 1023) & ~size_t(1023);
+    const size_t fixed = w + sizeof(Pipe) + 1024 + 1024;  // alignment of the base and behind the slots
+    a.acc_cols = 32;
+    while (a.acc_cols < a.N) a.acc_cols *= 2;
+    const size_t half = kSmemMax / 2 - 512;
+    Args best = a;
+    if (!choose_tile(best, Wr, Hr, B, size_t(1) << 30, a.nloads, 1)) return false;
+    for (int two = a.N <= 128 ? 1 : 0; two >= 0; --two) {
+        const size_t room = two ? half : kSmemMax;
+        if (fixed >= room) continue;
+        a.neg = two ? 1 : 2;
+        const int least = a.nloads == 4 || two ? a.nloads : a.nloads + 1;
+        if (!choose_tile(a, Wr, Hr, B, room - fixed, least, a.neg)) continue;
+        if (two && a.tiles > best.tiles) continue;  // no smaller tile for the sake of a second CTA
+        a.slot_bytes = (uint32_t)(a.I * a.Rp * a.Wp * a.rb + 127) & ~127u;
+        a.stg_bytes = stage_rows_bytes(a.I * a.R * a.Wt);
+        // a second staging buffer comes before more slots where a step stages twice (normalised values, then outputs) or a
+        // tile is one load; a plain forward tile wants its next two planes first (32 -> 64 channels: 1.45 -> 1.29 ms)
+        const int before = a.nloads == 4 && !a.ln_gamma ? a.nloads + 2 : least;
+        a.nbuf = two && (size_t)before * a.slot_bytes + 2 * (size_t)a.stg_bytes <= room - fixed ? 2 : 1;
+        a.slots = (int)((room - fixed - (size_t)(a.nbuf * a.neg) * a.stg_bytes) / a.slot_bytes);
+        if (a.slots > kMaxSlots) a.slots = kMaxSlots;
+        a.slots_bytes = ((uint32_t)a.slots * a.slot_bytes + 1023u) & ~1023u;
+        a.nacc = (two ? 256 : 512) / a.acc_cols;
+        if (a.nacc > 4) a.nacc = 4;
+        if (a.nacc < 2) continue;
+        a.smem = a.slots_bytes + w + (size_t)(a.nbuf * a.neg) * a.stg_bytes + sizeof(Pipe) + 1024;
+        const int ctas = ppo_num_sms() * (two ? 2 : 1);
+        a.grid = a.tiles < ctas ? a.tiles : ctas;
+        return true;
+    }
+    return false;
+}
+
+template <int MODE, int GC, int KS>
+int launch_one(const Args &a, cudaStream_t st) {
+    static bool attr_set[64] = {false};
+    int dev = 0;
+    PPO_CUDA_CHECK(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= 64) return PPO_ERR_CUDA;
+    if (!attr_set[dev]) {
+        PPO_CUDA_CHECK(cudaFuncSetAttribute(conv_halo_kernel<MODE, GC, KS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+        attr_set[dev] = true;
+    }
+    conv_halo_kernel<MODE, GC, KS><<<(unsigned)a.grid, (2 + a.neg * kEpiWarps) * 32, a.smem, st>>>(a);
+    PPO_LAUNCH_CHECK();
+    return PPO_OK;
+}
+
+template <int MODE, int GC>
+int launch_ks(const Args &a, int ks, cudaStream_t st) {
+    if (ks == 4) return launch_one<MODE, GC, 4>(a, st);
+    return ks == 2 ? launch_one<MODE, GC, 2>(a, st) : launch_one<MODE, GC, 1>(a, st);
+}
+
+int launch(const Args &a, int mode, int GC, cudaStream_t st) {
+    const int ks = a.CB >> 4;
+    if (mode == FWD) return GC == 64 ? launch_ks<FWD, 64>(a, ks, st) : launch_ks<FWD, 32>(a, ks, st);
+    if (mode == FWD_LN) return GC == 64 ? launch_ks<FWD_LN, 64>(a, ks, st) : launch_ks<FWD_LN, 32>(a, ks, st);
+    if (mode == DG_BITS) return GC == 64 ? launch_ks<DG_BITS, 64>(a, ks, st) : launch_ks<DG_BITS, 32>(a, ks, st);
+    return launch_ks<DG_ACT, 16>(a, ks, st);
+}
+
+// Channels per chunk of a C-channel source, or 0.
+int chunk_of(int C) { return C % 64 == 0 ? 64 : (C % 32 == 0 ? 32 : (C % 16 == 0 ? 16 : 0)); }
+
+}  // namespace
+
+int halo_conv_fwd(const ConvGeom &g, const bf16 *X, const bf16 *W, const FwdEpilogue &e, int32_t *status, cudaStream_t st) {
+    if (!status || g.k != 3 || g.pad != 1 || g.Hi < 2 || g.Wi < 2) return PPO_ERR_UNSUPPORTED;
+    if (!e.out || (e.ldo && e.ldo != g.Co) || g.Co % 32 != 0 || g.Co > 256) return PPO_ERR_UNSUPPORTED;
+    const int CB = chunk_of(g.Ci);
+    if (CB == 0 || CB != g.Ci || (size_t)9 * g.Ci * g.Co * 2 > 160 * 1024) return PPO_ERR_UNSUPPORTED;
+    Args a = {};
+    a.CB = CB;
+    a.rb = CB * 2;
+    a.nchunks = 1;
+    a.N = g.Co;
+    a.nplanes = a.nloads = 4;
+    a.nwl = 9;
+    a.w_box = (uint32_t)(g.Co * a.rb);
+    a.w_chunk = 9u * a.w_box;
+    a.ln_gamma = e.ln_gamma;
+    if (!plan(a, g.Wo, g.Ho, g.B)) return PPO_ERR_UNSUPPORTED;
+    for (int p = 0; p < 4; ++p) {
+        const int py = p >> 1, px = p & 1;
+        Plane &pl = a.planes[p];
+        for (int ky = 0; ky < 3; ++ky)
+            for (int kx = 0; kx < 3; ++kx) {
+                if ((ky == 1 ? 0 : 1) != py || (kx == 1 ? 0 : 1) != px) continue;
+                const int t = ky * 3 + kx;
+                a.ops[t] = {(uint32_t)(((ky == 2 ? 1 : 0) * a.Wp + (kx == 2 ? 1 : 0)) * a.rb) >> 4, (uint32_t)t * a.w_box >> 4, 0u,
+                            instr_desc(128, a.N, 0, 0)};
+                a.wl[t] = {t * g.Ci, (uint32_t)t * a.w_box};
+            }
+        pl.ox = -px;
+        pl.oy = -py;
+        const int rows = a.I > 1 ? a.R + 1 : a.R + py;
+        pl.bytes = (uint32_t)(a.I * rows * a.Wp * a.rb);
+        const long long dims[4] = {g.Ci, (g.Wi - px + 1) / 2, (g.Hi - py + 1) / 2, g.B};
+        const long long str[3] = {4ll * g.Ci, 4ll * g.Wi * g.Ci, 2ll * g.Hi * g.Wi * g.Ci};
+        const int box[4] = {CB, a.Wp, rows, a.I};
+        const int s = make_map_strided(&a.mapA[p], X + ((size_t)py * g.Wi + px) * g.Ci, 4, dims, str, box);
+        if (s != PPO_OK) return s;
+    }
+    {
+        const long long dims[2] = {g.K(), g.Co}, str[1] = {2ll * g.K()};
+        const int box[2] = {CB, a.N};
+        const int s = make_map_strided(&a.mapW, W, 2, dims, str, box);
+        if (s != PPO_OK) return s;
+    }
+    const int GC = g.Co % 64 == 0 ? 64 : 32;
+    const long long dims[4] = {g.Co, g.Wo, g.Ho, g.B};
+    const long long str[3] = {2ll * g.Co, 2ll * g.Wo * g.Co, 2ll * g.Ho * g.Wo * g.Co};
+    const int box[4] = {GC, a.Wt, a.R, a.I};
+    int s = make_map_strided(&a.mapO[0], e.out, 4, dims, str, box);
+    if (s != PPO_OK) return s;
+    a.bias = e.bias;
+    a.relu = e.relu;
+    a.out_bits = e.out_bits;
+    if (e.out_bits && !e.relu) return PPO_ERR_UNSUPPORTED;
+    if (e.ln_gamma) {
+        if (!e.ln_beta || !e.ln_xhat || !e.ln_rstd || !e.relu) return PPO_ERR_UNSUPPORTED;
+        s = make_map_strided(&a.mapX, e.ln_xhat, 4, dims, str, box);
+        if (s != PPO_OK) return s;
+        a.ln_beta = e.ln_beta;
+        a.ln_rstd = e.ln_rstd;
+    }
+    a.status = status;
+    return launch(a, e.ln_gamma ? FWD_LN : FWD, GC, st);
+}
+
+// The four parity classes (ph, pw) of input pixels (2y + ph, 2x + pw) side by side in the order 00, 01, 11, 10: the
+// classes that have a tap at a given shift of dY are then neighbours (all four at (0, 0), 01 | 11 at (0, 1), 11 | 10 at
+// (1, 0), 11 at (1, 1)), so every shift is one MMA of just those columns and no product with a zero weight is formed.
+int halo_conv_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, int wt_ld, const DgradEpilogue &e,
+                    int32_t *status, cudaStream_t st) {
+    if (!status || g.k != 3 || g.pad != 1 || g.Hi < 2 || g.Wi < 2 || ldy != g.Co || !e.out || e.out_f32) return PPO_ERR_UNSUPPORTED;
+    if (g.Ci != 16 && g.Ci != 32 && g.Ci != 64) return PPO_ERR_UNSUPPORTED;
+    if (g.Ci == 16 ? !e.mask_act : !e.mask_bits) return PPO_ERR_UNSUPPORTED;
+    const int CB = chunk_of(g.Co);
+    if (CB == 0 || wt_ld < g.Co || wt_ld % 8 != 0 || (size_t)9 * g.Ci * g.Co * 2 > 160 * 1024) return PPO_ERR_UNSUPPORTED;
+    Args a = {};
+    a.CB = CB;
+    a.rb = CB * 2;
+    a.nchunks = g.Co / CB;
+    a.N = 4 * g.Ci;
+    a.nplanes = 1;
+    a.nloads = a.nchunks;
+    a.w_box = (uint32_t)(g.Ci * a.rb);
+    a.w_chunk = 9u * a.w_box;
+    if (a.nchunks > kMaxSlots || !plan(a, (g.Wi + 1) / 2, (g.Hi + 1) / 2, g.B)) return PPO_ERR_UNSUPPORTED;
+    const int cls_ph[4] = {0, 0, 1, 1}, cls_pw[4] = {0, 1, 1, 0};
+    int nb = 0, no = 0;
+    for (int dy = 0; dy < 2; ++dy)
+        for (int dx = 0; dx < 2; ++dx) {
+            const int first = nb;
+            int c0 = -1;
+            for (int c = 0; c < 4; ++c) {
+                if (cls_ph[c] < dy || cls_pw[c] < dx) continue;
+                if (c0 < 0) c0 = c;
+                const int tap = (cls_ph[c] + 1 - 2 * dy) * 3 + cls_pw[c] + 1 - 2 * dx;
+                a.wl[nb] = {tap * wt_ld, (uint32_t)nb * a.w_box};
+                ++nb;
+            }
+            a.ops[no++] = {(uint32_t)((dy * a.Wp + dx) * a.rb) >> 4, (uint32_t)first * a.w_box >> 4, (uint32_t)(c0 * g.Ci),
+                           instr_desc(128, (nb - first) * g.Ci, 0, 0)};
+        }
+    a.nwl = nb;
+    a.planes[0] = {0, 0, (uint32_t)(a.I * a.Rp * a.Wp * a.rb)};
+    {
+        const long long dims[4] = {g.Co, g.Wo, g.Ho, g.B};
+        const long long str[3] = {2ll * g.Co, 2ll * g.Wo * g.Co, 2ll * g.Ho * g.Wo * g.Co};
+        const int box[4] = {CB, a.Wp, a.Rp, a.I};
+        int s = make_map_strided(&a.mapA[0], dY, 4, dims, str, box);
+        if (s != PPO_OK) return s;
+        const long long wd[2] = {9ll * wt_ld, g.Ci}, ws[1] = {18ll * wt_ld};
+        const int wb[2] = {CB, g.Ci};
+        s = make_map_strided(&a.mapW, Wt, 2, wd, ws, wb);
+        if (s != PPO_OK) return s;
+    }
+    for (int c = 0; c < 4; ++c) {
+        const int ph = cls_ph[c], pw = cls_pw[c];
+        const long long dims[4] = {g.Ci, (g.Wi - pw + 1) / 2, (g.Hi - ph + 1) / 2, g.B};
+        const long long str[3] = {4ll * g.Ci, 4ll * g.Wi * g.Ci, 2ll * g.Hi * g.Wi * g.Ci};
+        const int box[4] = {g.Ci, a.Wt, a.R, a.I};
+        const int s = make_map_strided(&a.mapO[c], e.out + ((size_t)ph * g.Wi + pw) * g.Ci, 4, dims, str, box);
+        if (s != PPO_OK) return s;
+    }
+    a.Hi = g.Hi;
+    a.Wi = g.Wi;
+    a.mask_bits = e.mask_bits;
+    a.mask = e.mask_act;
+    a.status = status;
+    return launch(a, g.Ci == 16 ? DG_ACT : DG_BITS, g.Ci, st);
+}

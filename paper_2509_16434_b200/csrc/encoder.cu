@@ -782,7 +782,9 @@ static ConvGeom fc_geom(int rows, int in, int out) {
 
 static int run_fwd(const ppo_model *m, const ConvGeom &g, const bf16 *X, const bf16 *W, const FwdEpilogue &e,
                    cudaStream_t st) {
-    int s = tma_gemm_fwd(g, X, W, e, ppo_device_status_ptr(), st);  // writes e.out_bits itself
+    int s = halo_conv_fwd(g, X, W, e, ppo_device_status_ptr(), st);  // the TMA kernels write e.out_bits themselves
+    if (s != PPO_ERR_UNSUPPORTED) return s;
+    s = tma_gemm_fwd(g, X, W, e, ppo_device_status_ptr(), st);
     if (s != PPO_ERR_UNSUPPORTED) return s;
     s = tc_gemm_fwd(g, X, W, e, ppo_device_status_ptr(), st);
     if (s == PPO_OK && e.out_bits) s = relu_bits(e.out, e.out_bits, g.M(), g.Co, st);
@@ -791,7 +793,9 @@ static int run_fwd(const ppo_model *m, const ConvGeom &g, const bf16 *X, const b
 
 static int run_dgrad(const ppo_model *m, const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *W, const bf16 *Wt,
                      int wt_ld, const bf16 *Wc, const DgradEpilogue &e, cudaStream_t st) {
-    const int s = tma_gemm_dgrad(g, dY, ldy, Wt, wt_ld, Wc, e, ppo_device_status_ptr(), st);
+    int s = halo_conv_dgrad(g, dY, ldy, Wt, wt_ld, e, ppo_device_status_ptr(), st);
+    if (s != PPO_ERR_UNSUPPORTED) return s;
+    s = tma_gemm_dgrad(g, dY, ldy, Wt, wt_ld, Wc, e, ppo_device_status_ptr(), st);
     if (s != PPO_ERR_UNSUPPORTED) return s;
     return tc_gemm_dgrad(g, dY, ldy, Wt, wt_ld, e, ppo_device_status_ptr(), st);
 }

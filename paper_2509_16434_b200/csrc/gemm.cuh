@@ -54,6 +54,11 @@ int tma_gemm_fwd(const ConvGeom &g, const bf16 *X, const bf16 *W, const FwdEpilo
 // fully connected layers read Wt).
 int tma_gemm_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, int wt_ld, const bf16 *Wc,
                    const DgradEpilogue &e, int32_t *status, cudaStream_t st);
+// 3x3 layers whose weights fit in shared memory (conv_halo.cu): the same forward and input gradient from halo tiles;
+// PPO_ERR_UNSUPPORTED (nothing launched) for anything else.
+int halo_conv_fwd(const ConvGeom &g, const bf16 *X, const bf16 *W, const FwdEpilogue &e, int32_t *status, cudaStream_t st);
+int halo_conv_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, int wt_ld, const DgradEpilogue &e,
+                    int32_t *status, cudaStream_t st);
 size_t tma_dgrad_weight_elems(int Ci, int k, int wt_ld);
 int tma_dgrad_weights(const bf16 *W, bf16 *Wc, int Co, int k, int Ci, int wt_ld, cudaStream_t st);
 // db (may be null; convolutions only): the bias gradient db[co] += sum over pixels of dY[.][co], taken from a

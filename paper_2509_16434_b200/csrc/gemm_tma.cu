@@ -26,10 +26,9 @@
 // (16 channels, SWIZZLE_32B).
 // Every wait is bounded: on a time-out the kernel records PPO_ERR_TIMEOUT, waits (bounded) for the
 // copies it has in flight, frees its tensor memory and returns.
-#include <cuda.h>  // CUtensorMap and its enums; the encoder is reached through the runtime's entry-point query
-
 #include "gemm.cuh"
 #include "tcgen05.cuh"
+#include "tma_host.cuh"
 
 namespace {
 
@@ -845,24 +844,6 @@ __global__ void __launch_bounds__(256) wgrad_reduce_kernel(const float *__restri
 
 // --------------------------------------------------------------------- host ----
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
-                                  const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encode_fn() {
-    static EncodeTiledFn fn = nullptr;
-    static bool tried = false;
-    if (!tried) {
-        tried = true;
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeTiledFn>(p);
-    }
-    return fn;
-}
-
 // Map of a bf16 tensor [d3][d2][d1][d0] whose innermost rows are `ld` elements apart; box and traversal
 // strides innermost first.  `row_bytes` selects the swizzle (box[0] * 2 == row_bytes).
 int make_map(CUtensorMap *m, const void *base, int rank, const long long *dims, long long ld, const int *box,
@@ -885,8 +866,7 @@ int make_map(CUtensorMap *m, const void *base, int rank, const long long *dims, 
         s *= dims[i + 1];
     }
     if (box[0] * 2 != row_bytes || !ppo_aligned(base, 16)) return PPO_ERR_UNSUPPORTED;
-    const CUtensorMapSwizzle sw = row_bytes == 128 ? CU_TENSOR_MAP_SWIZZLE_128B
-                                  : (row_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
+    const CUtensorMapSwizzle sw = swizzle_of_row(row_bytes);
     const CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void *>(base), gd, gs, bx,
                           es, CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);

@@ -1,0 +1,72 @@
+"""Convolution kernels at the edges of their tiles: odd extents, segments that do not divide a row, several small images
+per tile, every chunk width, single rows and columns of outputs, micro-batches that leave the last tile part empty."""
+import numpy as np
+import pytest
+
+import test_gpu_learner as base
+from helpers import rel_l2
+from oracle import oracle as orc
+from paper_2509_16434_b200 import binding as ppo
+from paper_2509_16434_b200 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def _net(name, H, W, conv_c, conv_k, N=6, T=2, **kw):
+    return synth.Workload(name, N, T, H, W, conv_c, conv_k, (40,), 1, 2, P=16, A=3, **kw)
+
+
+NETS = {
+    "narrow_16_32": _net("narrow_16_32", 17, 22, (16, 32), (3, 3)),
+    "chunks_of_16": _net("chunks_of_16", 37, 30, (48, 64, 32), (3, 3, 3)),
+    "two_chunks": _net("two_chunks", 33, 46, (32, 64, 128), (5, 3, 3)),
+    "three_groups": _net("three_groups", 30, 50, (32, 32, 96, 32), (3, 3, 3, 3)),
+    "wide_rows": _net("wide_rows", 12, 530, (16, 64, 32), (3, 3, 3), N=2),
+    "tall": _net("tall", 261, 14, (32, 64), (3, 3), N=2),
+    "small_images": _net("small_images", 14, 18, (32, 64, 64, 64), (3, 3, 3, 3), N=14, T=3),
+    "one_block": _net("one_block", 8, 8, (16, 32, 64), (3, 3, 3), N=2),
+    "tall_kernels": _net("tall_kernels", 40, 44, (32, 64, 96), (3, 5, 3)),
+    "ln_odd": _net("ln_odd", 35, 54, (16, 32, 64, 128), (3, 3, 3, 3), norm=True, embed=32),
+    "ln_32": _net("ln_32", 22, 30, (32, 32, 64), (5, 3, 3), norm=True),
+}
+
+
+@pytest.mark.parametrize("name", list(NETS))
+def test_conv_stack_matches_oracle(name, monkeypatch):
+    w = NETS[name]
+    monkeypatch.setitem(base.SHAPES, name, w)
+    base.test_backward_matches_oracle_on_identical_activations(name)  # every gradient tensor within 2e-2
+    # forward, in micro-batches that do not divide the rows
+    B = w.M // w.minibatches
+    L, md, lay, theta, roll, action, logp, dev = base._setup(w, max(1, B - 1), theta_scale_head=20.0)
+    L.compute_gae(dev["last_value"])
+    f, _, _, mu_o, V_o = base._oracle_minibatch(md, lay, theta, roll, action, logp, w, L.hyper, 5, 0, 0, w.minibatches)
+    ppo.ppo_shuffle_gather_minibatch(L.buffer, 5, 0, 0, w.minibatches, L.mb)
+    mus, vs = [], []
+    for r0 in range(0, B, L.microbatch):
+        rows = min(L.microbatch, B - r0)
+        ppo.ppo_encoder_fwd(L.model, L.mb, r0, rows, L.mean, L.value)
+        mus.append(L.mean[:rows].cpu().numpy().copy())
+        vs.append(L.value[:rows].cpu().numpy().copy())
+    assert ppo.ppo_poll_status() == 0
+    assert rel_l2(np.concatenate(mus), mu_o) <= base.ENC_TOL and rel_l2(np.concatenate(vs), V_o) <= base.ENC_TOL
+
+
+def test_gate_bits_are_the_signs_of_the_activations():
+    """The forward kernels' one-bit gates against the activations they stored, also where two warps share a word."""
+    for name in ("two_chunks", "ln_odd", "ln_32", "three_groups"):
+        w = NETS[name]
+        B = w.M // w.minibatches
+        L, md, lay, theta, roll, action, logp, dev = base._setup(w, B)
+        L.compute_gae(dev["last_value"])
+        ppo.ppo_shuffle_gather_minibatch(L.buffer, 5, 0, 0, w.minibatches, L.mb)
+        ppo.ppo_encoder_fwd(L.model, L.mb, 0, B, L.mean, L.value)
+        Ho, Wo = orc.conv_shapes(md)
+        for l, (h, wd, c) in enumerate(zip(Ho, Wo, md.conv_c), start=1):
+            if c % 32 or l == len(md.conv_c):
+                continue
+            act = L.model.activation(0, l)[:B * h * wd * c].float().cpu().numpy().reshape(-1, c // 32, 32)
+            word = L.model.activation(2, l)[:B * h * wd * c // 32].cpu().numpy().view(np.uint32).reshape(-1, c // 32)
+            ch = np.arange(32)
+            bits = (word[:, :, None] >> (ch // 2 + 16 * (ch % 2))) & 1
+            assert np.array_equal(bits != 0, act > 0), (name, l)
