@@ -4,6 +4,7 @@
 #include <new>
 
 #include "common.cuh"
+#include "launch.cuh"
 
 // ------------------------------------------------------------------ status ----
 
@@ -180,6 +181,7 @@ __device__ __forceinline__ void copy_strided(const char *src, char *dst, uint32_
 // to the segments' sizes (a grid with one row of blocks per segment spends most of its time starting the empty blocks
 // of the six small ones: 36 us instead of 14 us for the 39 MB of a 1024-env step of 160 x 120 frames).
 __global__ void __launch_bounds__(256) write_step_kernel(const __grid_constant__ CopySegs segs) {
+    grid_wait();
     uint32_t k = 0, first = 0;
     while (blockIdx.x >= segs.s[k].block_end) first = segs.s[k++].block_end;
     const CopySeg &sg = segs.s[k];
@@ -217,8 +219,7 @@ static int write_fields(ppo_buffer *b, int t, const void *const srcs[7], void *s
     }
     b->gae_valid = false;
     if (n == 0) return PPO_OK;
-    write_step_kernel<<<(unsigned)blocks, 256, 0, static_cast<cudaStream_t>(stream)>>>(segs);
-    PPO_LAUNCH_CHECK();
+    PPO_TRY(ppo_launch(write_step_kernel, dim3((unsigned)blocks), dim3(256), 0, static_cast<cudaStream_t>(stream), segs));
     return PPO_OK;
 }
 
@@ -278,6 +279,7 @@ __global__ void __launch_bounds__(128) gae_scan_kernel(const float *__restrict__
                                                        float gamma_lambda, float *__restrict__ adv,
                                                        float *__restrict__ ret, int T, int N,
                                                        double *__restrict__ partials) {
+    grid_wait();
     __shared__ double sh[32];
     const int n = blockIdx.x * blockDim.x + threadIdx.x;
     double s1 = 0.0, s2 = 0.0;
@@ -336,6 +338,7 @@ __global__ void __launch_bounds__(128) gae_scan_kernel(const float *__restrict__
 __global__ void __launch_bounds__(256) adv_normalize_kernel(float *__restrict__ adv, long long M,
                                                             const double *__restrict__ partials, int nparts,
                                                             float *__restrict__ stats_out) {
+    grid_wait();
     __shared__ double sh[32];
     __shared__ float s_mean, s_inv;
     double s1 = 0.0, s2 = 0.0;
@@ -386,6 +389,7 @@ __global__ void __launch_bounds__(128) gae_fused_kernel(const float *__restrict_
                                                         float *__restrict__ ret, int T, int N, double *partials,
                                                         unsigned int *barrier /*[2]: counter, generation*/,
                                                         float *__restrict__ stats_out, int32_t *status) {
+    grid_wait();
     __shared__ double sh[32];
     __shared__ float s_mean, s_inv;
     __shared__ int s_ok;
@@ -516,19 +520,17 @@ extern "C" int ppo_compute_gae(ppo_buffer *b, const float *last_value, float gam
         b->gae_blocks = blocks;
         return PPO_OK;
     }
-    gae_scan_kernel<8><<<blocks, threads, 0, st>>>(slab<float>(b, PPO_FIELD_REWARD), slab<float>(b, PPO_FIELD_VALUE),
+    PPO_TRY(ppo_launch(gae_scan_kernel<8>, dim3(blocks), dim3(threads), 0, st, slab<float>(b, PPO_FIELD_REWARD), slab<float>(b, PPO_FIELD_VALUE),
                                                    slab<uint8_t>(b, PPO_FIELD_DONE), last_value, gamma,
                                                    gamma * lambda, slab<float>(b, PPO_FIELD_ADV),
-                                                   slab<float>(b, PPO_FIELD_RET), T, N, partials);
-    PPO_LAUNCH_CHECK();
+                                                   slab<float>(b, PPO_FIELD_RET), T, N, partials));
     if (normalize) {
         const long long M = (long long)N * T;
         int nb = ppo_cdiv(M, 256 * 4 * 4);
         int cap = ppo_num_sms() * 8;
         if (nb > cap) nb = cap;
         if (nb < 1) nb = 1;
-        adv_normalize_kernel<<<nb, 256, 0, st>>>(slab<float>(b, PPO_FIELD_ADV), M, partials, blocks, stats_out);
-        PPO_LAUNCH_CHECK();
+        PPO_TRY(ppo_launch(adv_normalize_kernel, dim3(nb), dim3(256), 0, st, slab<float>(b, PPO_FIELD_ADV), M, partials, blocks, stats_out));
     }
     b->gae_valid = true;
     b->gae_blocks = blocks;
@@ -569,16 +571,14 @@ extern "C" int ppo_gae_static(const float *reward, const float *value, const uin
     if (!partials) return PPO_ERR_CUDA;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // every partial a later pass reads is written by this launch first: nothing has to start at zero
-    gae_scan_kernel<8><<<blocks, threads, 0, st>>>(reward, value, done, last_value, gamma, gamma * lambda, adv, ret, T, N,
-                                                   partials);
-    PPO_LAUNCH_CHECK();
+    PPO_TRY(ppo_launch(gae_scan_kernel<8>, dim3(blocks), dim3(threads), 0, st, reward, value, done, last_value, gamma, gamma * lambda, adv, ret, T, N,
+                                                   partials));
     if (normalize) {
         const long long M = (long long)N * T;
         int nb = ppo_cdiv(M, 256 * 4 * 4);
         const int cap = ppo_num_sms() * 8;
         nb = nb > cap ? cap : (nb < 1 ? 1 : nb);
-        adv_normalize_kernel<<<nb, 256, 0, st>>>(adv, M, partials, blocks, stats_out);
-        PPO_LAUNCH_CHECK();
+        PPO_TRY(ppo_launch(adv_normalize_kernel, dim3(nb), dim3(256), 0, st, adv, M, partials, blocks, stats_out));
     }
     return PPO_OK;
 }
@@ -694,6 +694,7 @@ constexpr uint32_t kGatherUnits = 1024;  // 16-byte units a CTA moves: four per 
 // against a pixel per access.
 template <bool RAGGED>
 __global__ void __launch_bounds__(256) gather_kernel(const __grid_constant__ GatherArgs g, const __grid_constant__ PermParams p) {
+    grid_wait();
     const uint32_t row = blockIdx.x / g.chunks, chunk = blockIdx.x - row * g.chunks;
     __shared__ uint32_t s_sample;
     if (threadIdx.x < 32) {
@@ -811,8 +812,7 @@ static int gather_impl(const ppo_buffer *b, uint64_t seed, uint32_t epoch, int m
     const long long ctas = B * g.chunks;
     if (ctas > 0x7fffffffll || frame > 0x7fffffffull) return PPO_ERR_UNSUPPORTED;
     PermParams p = make_perm(seed, epoch, (uint32_t)M);
-    if (vec16) gather_kernel<false><<<(unsigned)ctas, 256, 0, static_cast<cudaStream_t>(stream)>>>(g, p);
-    else gather_kernel<true><<<(unsigned)ctas, 256, 0, static_cast<cudaStream_t>(stream)>>>(g, p);
-    PPO_LAUNCH_CHECK();
+    if (vec16) PPO_TRY(ppo_launch(gather_kernel<false>, dim3((unsigned)ctas), dim3(256), 0, static_cast<cudaStream_t>(stream), g, p));
+    else PPO_TRY(ppo_launch(gather_kernel<true>, dim3((unsigned)ctas), dim3(256), 0, static_cast<cudaStream_t>(stream), g, p));
     return PPO_OK;
 }

@@ -25,6 +25,12 @@ typedef __nv_bfloat16 bf16;
         PPO_CUDA_CHECK(cudaGetLastError()); \
     } while (0)
 
+#define PPO_TRY(...)                 \
+    do {                             \
+        const int _s = (__VA_ARGS__); \
+        if (_s != PPO_OK) return _s; \
+    } while (0)
+
 static inline bool ppo_aligned(const void *p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 static inline size_t ppo_align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 static inline int ppo_cdiv(long long a, long long b) { return (int)((a + b - 1) / b); }
@@ -56,6 +62,8 @@ struct ConvGeom {
 struct ppo_tensor {
     int64_t off, size;
 };
+
+struct ppo_plans;  // recorded launches of a model (launch.cuh)
 
 struct ppo_model {
     ppo_model_desc d;
@@ -115,9 +123,13 @@ struct ppo_model {
     float *act_mean;               // [mb][A]: Gaussian mean of ppo_policy_act before sampling
     int loss_partial_blocks;
     bool wT_valid;
+    bool wC_valid[PPO_MAX_CONV + 1];
+    unsigned int *loss_ticket;     // blocks of the loss kernel that are done (0 between launches)
+    bool ticket_zeroed;
     // forward/backward pairing
     int last_row0, last_rows;
     bool fwd_valid;
+    ppo_plans *plans = nullptr;
     // second stream of the backward pass with its fork and join events (made on first use)
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;

@@ -16,6 +16,7 @@
 // Frames must hold finite values (an Inf or NaN beside a window would meet a zero weight) and have an even
 // width.
 #include "gemm.cuh"
+#include "launch.cuh"
 #include "tcgen05.cuh"
 
 namespace {
@@ -117,6 +118,16 @@ __global__ void __launch_bounds__(kThreads, 1) conv1_tc_kernel(const __grid_cons
         pipe->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    // The constant part of every im2col row of every stage: the two bias slots hold 1.0 (as fp16), the padding behind
+    // them zero.  The producers' copies only ever write the window words in front of it.
+    for (int i = threadIdx.x; i < S * T * 128; i += kThreads) {
+        uint8_t *row = smem + (size_t)(i >> 7) * kTileBytes;
+#pragma unroll
+        for (int k = KW; k < KP / 2; ++k)
+            *reinterpret_cast<uint32_t *>(row + core_offset(i & 127, k >> 2, KP) + (k & 3) * 4) = k == KW ? 0x3C003C00u : 0u;
+    }
+    if (warp == kProdWarps) tmem_alloc(&pipe->tmem_slot, ncols);
+    grid_wait();
     // filters in the K layout of the window, bias parts in the two slots behind it, zeros elsewhere
     for (int i = threadIdx.x; i < N * KP; i += kThreads) {
         const int n = i / KP, k = i - n * KP;
@@ -131,20 +142,11 @@ __global__ void __launch_bounds__(kThreads, 1) conv1_tc_kernel(const __grid_cons
         }
         *reinterpret_cast<__half *>(bsm + core_offset(n, k >> 3, KP) + (k & 7) * 2) = __float2half_rn(f);
     }
-    // The constant part of every im2col row of every stage: the two bias slots hold 1.0 (as fp16), the padding behind
-    // them zero.  The producers' copies only ever write the window words in front of it.
-    for (int i = threadIdx.x; i < S * T * 128; i += kThreads) {
-        uint8_t *row = smem + (size_t)(i >> 7) * kTileBytes;
-#pragma unroll
-        for (int k = KW; k < KP / 2; ++k)
-            *reinterpret_cast<uint32_t *>(row + core_offset(i & 127, k >> 2, KP) + (k & 3) * 4) = k == KW ? 0x3C003C00u : 0u;
-    }
     if (a.ln_gamma && threadIdx.x < 32) {
         pipe->gamma[threadIdx.x] = (int)threadIdx.x < N ? a.ln_gamma[threadIdx.x] : 0.f;
         pipe->beta[threadIdx.x] = (int)threadIdx.x < N ? a.ln_beta[threadIdx.x] : 0.f;
     }
     fence_async_smem();
-    if (warp == kProdWarps) tmem_alloc(&pipe->tmem_slot, ncols);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -349,8 +351,7 @@ int launch(Args &a, cudaStream_t st) {
     if (smem > 200 * 1024) return PPO_ERR_UNSUPPORTED;
     const int sms = ppo_num_sms();
     const int nstage = (a.tiles + a.T - 1) / a.T;
-    conv1_tc_kernel<KS><<<nstage < sms ? nstage : sms, kThreads, smem, st>>>(a);
-    PPO_LAUNCH_CHECK();
+    PPO_TRY(ppo_launch(conv1_tc_kernel<KS>, dim3(nstage < sms ? nstage : sms), dim3(kThreads), smem, st, a));
     return PPO_OK;
 }
 

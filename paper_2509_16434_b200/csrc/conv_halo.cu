@@ -21,6 +21,7 @@
 #include <cuda.h>
 
 #include "gemm.cuh"
+#include "launch.cuh"
 #include "tcgen05.cuh"
 #include "tma_host.cuh"
 
@@ -221,6 +222,8 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
         pipe->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (warp == 1) tmem_alloc(&pipe->tmem_slot, ncols);
+    grid_wait();
     if (MODE == FWD || MODE == FWD_LN)
         for (int i = threadIdx.x; i < a.N; i += (int)blockDim.x) {
             pipe->bias[i] = a.bias[i];
@@ -229,7 +232,6 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
                 pipe->beta[i] = a.ln_beta[i];
             }
         }
-    if (warp == 1) tmem_alloc(&pipe->tmem_slot, ncols);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -731,8 +733,7 @@ int launch_one(const Args &a, cudaStream_t st) {
         PPO_CUDA_CHECK(cudaFuncSetAttribute(conv_halo_kernel<MODE, GC, KS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
         attr_set[dev] = true;
     }
-    conv_halo_kernel<MODE, GC, KS><<<(unsigned)a.grid, (2 + a.neg * kEpiWarps) * 32, a.smem, st>>>(a);
-    PPO_LAUNCH_CHECK();
+    PPO_TRY(ppo_launch(conv_halo_kernel<MODE, GC, KS>, dim3((unsigned)a.grid), dim3((2 + a.neg * kEpiWarps) * 32), a.smem, st, a));
     return PPO_OK;
 }
 
@@ -819,17 +820,13 @@ int halo_conv_fwd(const ConvGeom &g, const bf16 *X, const bf16 *W, const FwdEpil
     return launch(a, e.ln_gamma ? FWD_LN : FWD, GC, st);
 }
 
-// The four parity classes (ph, pw) of input pixels (2y + ph, 2x + pw) side by side in the order 00, 01, 11, 10: the
-// classes that have a tap at a given shift of dY are then neighbours (all four at (0, 0), 01 | 11 at (0, 1), 11 | 10 at
-// (1, 0), 11 at (1, 1)), so every shift is one MMA of just those columns and no product with a zero weight is formed.
-int halo_conv_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, int wt_ld, const DgradEpilogue &e,
-                    int32_t *status, cudaStream_t st) {
-    if (!status || g.k != 3 || g.pad != 1 || g.Hi < 2 || g.Wi < 2 || ldy != g.Co || !e.out || e.out_f32) return PPO_ERR_UNSUPPORTED;
-    if (g.Ci != 16 && g.Ci != 32 && g.Ci != 64) return PPO_ERR_UNSUPPORTED;
-    if (g.Ci == 16 ? !e.mask_act : !e.mask_bits) return PPO_ERR_UNSUPPORTED;
+// Shape part of the input gradient's arguments; false where the layer is not covered.
+static bool plan_dgrad(Args &a, const ConvGeom &g, int ldy, int wt_ld, const DgradEpilogue &e) {
+    if (g.k != 3 || g.pad != 1 || g.Hi < 2 || g.Wi < 2 || ldy != g.Co || !e.out || e.out_f32 || e.ksplit > 1) return false;
+    if (g.Ci != 16 && g.Ci != 32 && g.Ci != 64) return false;
+    if (g.Ci == 16 ? !e.mask_act : !e.mask_bits) return false;
     const int CB = chunk_of(g.Co);
-    if (CB == 0 || wt_ld < g.Co || wt_ld % 8 != 0 || (size_t)9 * g.Ci * g.Co * 2 > 160 * 1024) return PPO_ERR_UNSUPPORTED;
-    Args a = {};
+    if (CB == 0 || wt_ld < g.Co || wt_ld % 8 != 0 || (size_t)9 * g.Ci * g.Co * 2 > 160 * 1024) return false;
     a.CB = CB;
     a.rb = CB * 2;
     a.nchunks = g.Co / CB;
@@ -838,7 +835,23 @@ int halo_conv_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, 
     a.nloads = a.nchunks;
     a.w_box = (uint32_t)(g.Ci * a.rb);
     a.w_chunk = 9u * a.w_box;
-    if (a.nchunks > kMaxSlots || !plan(a, (g.Wi + 1) / 2, (g.Hi + 1) / 2, g.B)) return PPO_ERR_UNSUPPORTED;
+    return a.nchunks <= kMaxSlots && plan(a, (g.Wi + 1) / 2, (g.Hi + 1) / 2, g.B);
+}
+
+bool halo_dgrad_covers(const ConvGeom &g, int ldy, int wt_ld, const DgradEpilogue &e) {
+    if (g.k != 3) return false;
+    Args a = {};
+    return plan_dgrad(a, g, ldy, wt_ld, e);
+}
+
+// The four parity classes (ph, pw) of input pixels (2y + ph, 2x + pw) side by side in the order 00, 01, 11, 10: the
+// classes that have a tap at a given shift of dY are then neighbours (all four at (0, 0), 01 | 11 at (0, 1), 11 | 10 at
+// (1, 0), 11 at (1, 1)), so every shift is one MMA of just those columns and no product with a zero weight is formed.
+int halo_conv_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, int wt_ld, const DgradEpilogue &e,
+                    int32_t *status, cudaStream_t st) {
+    Args a = {};
+    if (!status || !plan_dgrad(a, g, ldy, wt_ld, e)) return PPO_ERR_UNSUPPORTED;
+    const int CB = a.CB;
     const int cls_ph[4] = {0, 0, 1, 1}, cls_pw[4] = {0, 1, 1, 0};
     int nb = 0, no = 0;
     for (int dy = 0; dy < 2; ++dy)

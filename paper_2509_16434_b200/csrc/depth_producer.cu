@@ -7,6 +7,7 @@
 // ((u + 0.5 - W/2) / f, (v + 0.5 - H/2) / f, 1), f = (W/2) / tan(hfov/2).  With the ray's z component equal to 1 the
 // ray parameter of a hit is its depth.  Depths outside [near, far] and rays that hit nothing give 0 (no return).
 #include "common.cuh"
+#include "launch.cuh"
 
 namespace {
 
@@ -78,6 +79,7 @@ __device__ __forceinline__ float hit_capsule(float dx, float dy, float dz, const
 __global__ void __launch_bounds__(256) depth_render_kernel(__half *__restrict__ depth, int H, int W, float inv_f,
                                                            float near, float far, const float *__restrict__ plane,
                                                            int n_prims, const float *__restrict__ prims, int chunks) {
+    grid_wait();
     __shared__ float sp[kMaxPrims * 8];
     __shared__ float spl[4];
     const int n = blockIdx.x / chunks, chunk = blockIdx.x - n * chunks;
@@ -136,8 +138,7 @@ extern "C" int ppo_buffer_render_depth(ppo_buffer *b, int t, float hfov, float n
     __half *depth = reinterpret_cast<__half *>(b->base + b->field_off[PPO_FIELD_DEPTH]) + (size_t)t * d.N * HW;
     const float inv_f = tanf(0.5f * hfov) / (0.5f * (float)d.W);
     b->gae_valid = false;
-    depth_render_kernel<<<(unsigned)(d.N * chunks), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        depth, d.H, d.W, inv_f, near, far, plane, n_prims, prims, chunks);
-    PPO_LAUNCH_CHECK();
+    PPO_TRY(ppo_launch(depth_render_kernel, dim3((unsigned)(d.N * chunks)), dim3(256), 0, static_cast<cudaStream_t>(stream), 
+        depth, d.H, d.W, inv_f, near, far, plane, n_prims, prims, chunks));
     return PPO_OK;
 }

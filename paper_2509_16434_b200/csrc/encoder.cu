@@ -1,6 +1,9 @@
 // Encoder forward/backward: the direct first convolution (C_in = 1), pooling, the small
 // element-wise kernels, and the orchestration of the implicit GEMMs of the deeper layers.
+#include <new>
+
 #include "common.cuh"
+#include "launch.cuh"
 #include "gemm.cuh"
 
 // -------------------------------------------------------------------- conv1 ----
@@ -16,6 +19,7 @@ __global__ void __launch_bounds__(128) conv1_fwd_kernel(const __half *__restrict
                                                         const bf16 *__restrict__ W, const float *__restrict__ bias,
                                                         bf16 *__restrict__ out, uint32_t *__restrict__ bits,
                                                         int rows, int Hi, int Wi, int Ho, int Wo, int C1) {
+    grid_wait();
     extern __shared__ __align__(16) float sm[];  // w[tap][co], then bias[co], then (STAGE) 4 warps x 32 pixels x C1 bf16
     float *w = sm, *bs = sm + KS * KS * C1;
     for (int i = threadIdx.x; i < KS * KS * C1; i += blockDim.x) {
@@ -107,6 +111,7 @@ __global__ void __launch_bounds__(128) conv1_wgrad_kernel(const __half *__restri
                                                           const bf16 *__restrict__ dZ, float *__restrict__ part,
                                                           int rows, int Hi, int Wi, int Ho,
                                                           int Wo, int C1, long long px_per_warp) {
+    grid_wait();
     constexpr int K2 = KS * KS, P = KS / 2;
     extern __shared__ float sm[];  // [4 warps][C1 * (K2 + 1)]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -231,6 +236,7 @@ __global__ void __launch_bounds__(256) conv1_wgrad_mma_kernel(const __half *__re
                                                               const bf16 *__restrict__ dZ, float *__restrict__ part,
                                                               int rows, int Hi, int Wi,
                                                               int Ho, int Wo, long long px_per_warp) {
+    grid_wait();
     constexpr int K2 = KS * KS, P = KS / 2, ODD = P & 1, NP = (KS + ODD + 1) / 2, KW = KS * NP;
     constexpr int TP = (2 * KW + 1 + 15) / 16 * 16, MB = TP / 16, C1 = NB * 8;
     constexpr int PX = 32;  // pixels per trip: one per lane, two K = 16 steps of the MMA
@@ -378,6 +384,7 @@ __global__ void __launch_bounds__(256) conv1_wgrad_mma_kernel(const __half *__re
 // gate_bit_of_channel(c).
 __global__ void __launch_bounds__(256) relu_bits_kernel(const bf16 *__restrict__ act, uint32_t *__restrict__ bits,
                                                         long long words) {
+    grid_wait();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= words) return;
     const uint4 *p = reinterpret_cast<const uint4 *>(act + i * 32);
@@ -400,8 +407,7 @@ int relu_bits(const bf16 *act, uint32_t *bits, long long M, int C, cudaStream_t 
     if (C % 32 != 0) return PPO_ERR_UNSUPPORTED;
     const long long words = M * (C / 32);
     if (words <= 0) return PPO_OK;
-    relu_bits_kernel<<<ppo_cdiv(words, 256), 256, 0, st>>>(act, bits, words);
-    PPO_LAUNCH_CHECK();
+    PPO_TRY(ppo_launch(relu_bits_kernel, dim3(ppo_cdiv(words, 256)), dim3(256), 0, st, act, bits, words));
     return PPO_OK;
 }
 
@@ -411,6 +417,7 @@ int relu_bits(const bf16 *act, uint32_t *bits, long long M, int C, cudaStream_t 
 __global__ void __launch_bounds__(256) pool_concat_kernel(const bf16 *__restrict__ act,
                                                           const float *__restrict__ proprio, bf16 *__restrict__ h0,
                                                           int rows, int npx, int C, int P) {
+    grid_wait();
     const int b = blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (b >= rows) return;
@@ -441,6 +448,7 @@ __global__ void __launch_bounds__(256) pool_concat_kernel(const bf16 *__restrict
 __global__ void __launch_bounds__(256) unpool_kernel(const float *__restrict__ dh0, const bf16 *__restrict__ act,
                                                      bf16 *__restrict__ dact, long long total8, int npx, int C,
                                                      int ld_h0) {
+    grid_wait();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= total8) return;
     const int c8n = C >> 3;
@@ -465,6 +473,7 @@ __global__ void __launch_bounds__(256) unpool_kernel(const float *__restrict__ d
 __global__ void __launch_bounds__(256) pack_dout_kernel(const float *__restrict__ dmean,
                                                         const float *__restrict__ dvalue, bf16 *__restrict__ out,
                                                         int rows, int A) {
+    grid_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= rows * 16) return;
     const int r = i / 16, j = i % 16;
@@ -474,16 +483,11 @@ __global__ void __launch_bounds__(256) pack_dout_kernel(const float *__restrict_
     out[i] = __float2bfloat16_rn(v);
 }
 
-#define PPO_TRY(expr)                 \
-    do {                              \
-        int _s = (expr);              \
-        if (_s != PPO_OK) return _s;  \
-    } while (0)
-
 // dst[i] (i < nA: dstA[i], else dstB[i - nA]) += part[0][i] + part[1][i] + ... in that order: the second stage of the
 // reductions whose blocks leave partial sums instead of adding to the result with atomics (reproducible results).
 __global__ void __launch_bounds__(256) sum_partials_kernel(const float *__restrict__ part, int nparts, int nA,
                                                            float *__restrict__ dstA, int nB, float *__restrict__ dstB) {
+    grid_wait();
     // 32 results per block; eight threads share a result, thread j adding the partials b = j, j + 8, ... in order, and
     // the eight sums are added in the order of j: fixed, whatever the launch.
     __shared__ float sh[8][32];
@@ -493,8 +497,18 @@ __global__ void __launch_bounds__(256) sum_partials_kernel(const float *__restri
     part += (size_t)blockIdx.y * nparts * n;  // blockIdx.y: one of several independent reductions of nA results (nB = 0)
     dstA += (size_t)blockIdx.y * nA;
     float acc = 0.f;
-    if (i < n)
-        for (int b = j; b < nparts; b += 8) acc += part[(size_t)b * n + i];
+    if (i < n) {
+        // the loads of eight partials are in flight while the sum stays in order
+        int b = j;
+        for (; b + 56 < nparts; b += 64) {
+            float v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = part[(size_t)(b + 8 * u) * n + i];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) acc += v[u];
+        }
+        for (; b < nparts; b += 8) acc += part[(size_t)b * n + i];
+    }
     sh[j][o] = acc;
     __syncthreads();
     if (j == 0 && i < n) {
@@ -508,8 +522,7 @@ __global__ void __launch_bounds__(256) sum_partials_kernel(const float *__restri
 
 static int sum_partials(const float *part, int nparts, int nA, float *dstA, int nB, float *dstB, cudaStream_t st,
                         int slabs = 1) {
-    sum_partials_kernel<<<dim3(ppo_cdiv(nA + nB, 32), slabs), 256, 0, st>>>(part, nparts, nA, dstA, nB, dstB);
-    PPO_LAUNCH_CHECK();
+    PPO_TRY(ppo_launch(sum_partials_kernel, dim3(ppo_cdiv(nA + nB, 32), slabs), dim3(256), 0, st, part, nparts, nA, dstA, nB, dstB));
     return PPO_OK;
 }
 
@@ -517,6 +530,7 @@ static int sum_partials(const float *part, int nparts, int nA, float *dstA, int 
 // walk (row, 8-column chunk) pairs with 128-bit loads; threads that share a chunk are folded through shared memory.
 __global__ void __launch_bounds__(256) colsum_kernel(const bf16 *__restrict__ dZ, int ld, long long M, int N,
                                                      float *__restrict__ part) {
+    grid_wait();
     __shared__ float sh[256][9];
     const int chunks = N >> 3;                    // 16-byte chunks per row
     const int rows_per_pass = 256 / chunks;       // whole rows covered by one pass of the block
@@ -550,40 +564,72 @@ __global__ void __launch_bounds__(256) colsum_kernel(const bf16 *__restrict__ dZ
     }
 }
 
-// The same first stage for any N <= ld (used for the head, whose 13 columns sit in rows of 16).
+// The same first stage for any N <= ld (used for the head, whose 13 columns sit in rows of 16): blockIdx.y is the column.
 __global__ void __launch_bounds__(256) colsum_small_kernel(const bf16 *__restrict__ dZ, int ld, long long M, int N,
                                                            float *__restrict__ part) {
+    grid_wait();
     __shared__ float sh[256];
-    for (int n = 0; n < N; ++n) {
-        float v = 0.f;
-        for (long long m = (long long)blockIdx.x * 256 + threadIdx.x; m < M; m += (long long)gridDim.x * 256)
-            v += bf2f(dZ[m * ld + n]);
-        sh[threadIdx.x] = v;
-        __syncthreads();
-        for (int o = 128; o > 0; o >>= 1) {
-            if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) part[(size_t)blockIdx.x * N + n] = sh[0];
+    const int n = blockIdx.y;
+    float v = 0.f;
+    for (long long m = (long long)blockIdx.x * 256 + threadIdx.x; m < M; m += (long long)gridDim.x * 256) v += bf2f(dZ[m * ld + n]);
+    sh[threadIdx.x] = v;
+    __syncthreads();
+    for (int o = 128; o > 0; o >>= 1) {
+        if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
         __syncthreads();
     }
+    if (threadIdx.x == 0) part[(size_t)blockIdx.x * N + n] = sh[0];
 }
 
-// Wt[ci][tap][co (row stride ld)] = W[co][tap][ci], zero in the padding co >= Co.
-__global__ void __launch_bounds__(256) transpose_weights_kernel(const bf16 *__restrict__ W, bf16 *__restrict__ Wt,
-                                                                int Co, int taps, int Ci, int ld) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long total = (long long)Ci * taps * ld;
-    if (i >= total) return;
-    const int co = (int)(i % ld);
-    const long long r = i / ld;
-    const int tap = (int)(r % taps), ci = (int)(r / taps);
-    Wt[i] = (co < Co) ? W[((size_t)co * taps + tap) * Ci + ci] : __float2bfloat16_rn(0.f);
+// Wt[ci][tap][co (row stride ld)] = W[co][tap][ci], zero in the padding co >= Co, for every weight matrix in one launch.
+struct TransposeJob {
+    long long src, dst;  // element offsets
+    int Co, taps, Ci, ld;
+    int block_end;       // blocks of the jobs up to and including this one
+};
+struct TransposeJobs {
+    TransposeJob j[PPO_MAX_TENSORS];
+};
+
+// A block turns a tile of 64 output channels x 64 columns (tap, input channel) of the row-major weight matrix through
+// shared memory: both sides move whole 128-byte lines.  One launch for all matrices: a launch per matrix spent more time
+// between the kernels than in them (two LSTM layers, 14 M weights: 364 -> 90 us per 4 minibatches; small networks: a
+// dozen launches of 2 us).
+__global__ void __launch_bounds__(256) transpose_weights_kernel(const bf16 *__restrict__ W0, bf16 *__restrict__ Wt0,
+                                                                const __grid_constant__ TransposeJobs jobs) {
+    grid_wait();
+    __shared__ uint16_t tile[64][66];
+    int k = 0, first = 0;
+    while ((int)blockIdx.x >= jobs.j[k].block_end) first = jobs.j[k++].block_end;
+    const TransposeJob &jb = jobs.j[k];
+    const int J = jb.taps * jb.Ci, jt = (J + 63) >> 6;
+    const int b = (int)blockIdx.x - first, co0 = b / jt * 64, j0 = (b - b / jt * jt) * 64;
+    const uint16_t *W = reinterpret_cast<const uint16_t *>(W0) + jb.src;
+    uint16_t *Wt = reinterpret_cast<uint16_t *>(Wt0) + jb.dst;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int r = warp * 8 + i, co = co0 + r, j = j0 + 2 * lane;
+        uint32_t v = 0u;
+        if (co < jb.Co && j < J) v = *reinterpret_cast<const uint32_t *>(W + (size_t)co * J + j);  // J is even
+        tile[r][2 * lane] = (uint16_t)v;
+        tile[r][2 * lane + 1] = (uint16_t)(v >> 16);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int c = warp * 8 + i, j = j0 + c, co = co0 + 2 * lane;
+        if (j >= J || co >= jb.ld) continue;  // ld is a multiple of 8
+        const int tap = j / jb.Ci, ci = j - tap * jb.Ci;
+        *reinterpret_cast<uint32_t *>(Wt + ((size_t)ci * jb.taps + tap) * jb.ld + co) =
+            (uint32_t)tile[2 * lane][c] | ((uint32_t)tile[2 * lane + 1][c] << 16);
+    }
 }
 
 // h0[b][E .. E+P) = proprio[b] as bf16 (the embedding occupies the first E columns of a row of ld elements).
 __global__ void __launch_bounds__(256) concat_proprio_kernel(const float *__restrict__ proprio, bf16 *__restrict__ h0,
                                                              int rows, int E, int P, int ld) {
+    grid_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= rows * P) return;
     const int b = i / P, j = i - b * P;
@@ -593,6 +639,7 @@ __global__ void __launch_bounds__(256) concat_proprio_kernel(const float *__rest
 // dz[b][e] = dh0[b][e] where the embedding h0[b][e] is > 0, else 0 (back through its ReLU), as a bf16 GEMM operand.
 __global__ void __launch_bounds__(256) embed_dz_kernel(const float *__restrict__ dh0, const bf16 *__restrict__ h0,
                                                        bf16 *__restrict__ dz, int rows, int E, int ld) {
+    grid_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= rows * E) return;
     const int b = i / E, e = i - b * E;
@@ -608,6 +655,7 @@ __global__ void __launch_bounds__(256) embed_dz_kernel(const float *__restrict__
 __global__ void __launch_bounds__(256) ln_bwd_kernel(bf16 *__restrict__ d, const bf16 *__restrict__ xhat,
                                                      const float *__restrict__ rstd, const float *__restrict__ gamma,
                                                      long long M, int C, float *__restrict__ part) {
+    grid_wait();
     __shared__ float sh[16][256];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int lpp = C >> 3, ppw = 32 / lpp;
@@ -684,6 +732,7 @@ __device__ __forceinline__ float sigmoidf_(float x) { return 1.f / (1.f + __expf
 // State the first step of a sequence starts from: h_prev[0] = bf16(h_init), c_prev[0] = c_init (rows of one step, Be x H).
 __global__ void __launch_bounds__(256) lstm_init_kernel(const float *__restrict__ h_init, const float *__restrict__ c_init,
                                                         bf16 *__restrict__ hprev, float *__restrict__ cprev, int n) {
+    grid_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     hprev[i] = __float2bfloat16_rn(h_init[i]);
@@ -700,6 +749,7 @@ __global__ void __launch_bounds__(256) lstm_cell_fwd_kernel(const float *__restr
                                                             float *__restrict__ c, bf16 *__restrict__ h,
                                                             bf16 *__restrict__ hprev_next, float *__restrict__ cprev_next,
                                                             int Be, int H) {
+    grid_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= Be * H) return;
     const int e = i / H, j = i - e * H;
@@ -734,6 +784,7 @@ __global__ void __launch_bounds__(256) lstm_cell_bwd_kernel(const float *__restr
                                                             const float *__restrict__ gates, const float *__restrict__ c,
                                                             const float *__restrict__ cprev, bf16 *__restrict__ dg,
                                                             int Be, int H, int last, int nsplit) {
+    grid_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= Be * H) return;
     const int e = i / H, j = i - e * H;
@@ -780,42 +831,94 @@ static ConvGeom fc_geom(int rows, int in, int out) {
     return g;
 }
 
-static int run_fwd(const ppo_model *m, const ConvGeom &g, const bf16 *X, const bf16 *W, const FwdEpilogue &e,
-                   cudaStream_t st) {
-    int s = halo_conv_fwd(g, X, W, e, ppo_device_status_ptr(), st);  // the TMA kernels write e.out_bits themselves
-    if (s != PPO_ERR_UNSUPPORTED) return s;
-    s = tma_gemm_fwd(g, X, W, e, ppo_device_status_ptr(), st);
-    if (s != PPO_ERR_UNSUPPORTED) return s;
-    s = tc_gemm_fwd(g, X, W, e, ppo_device_status_ptr(), st);
-    if (s == PPO_OK && e.out_bits) s = relu_bits(e.out, e.out_bits, g.M(), g.Co, st);
+// Runs `make` the first time an operation is called with this key and remembers its launches; later calls only enqueue
+// them.
+template <typename F>
+static int recorded(ppo_model *m, const PlanKey &key, cudaStream_t st, F &&make) {
+    if (!m->plans) m->plans = new (std::nothrow) ppo_plans();
+    if (!m->plans) return make();
+    if (const PlanEntry *e = ppo_find_plan(m->plans, key)) return ppo_replay(*e, st);
+    std::vector<LaunchRecord> launches, *outer = ppo_recording;
+    ppo_recording = &launches;
+    const int s = make();
+    ppo_recording = outer;
+    if (s == PPO_OK) ppo_store_plan(m->plans, key, std::move(launches));
     return s;
 }
 
-static int run_dgrad(const ppo_model *m, const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *W, const bf16 *Wt,
-                     int wt_ld, const bf16 *Wc, const DgradEpilogue &e, cudaStream_t st) {
-    int s = halo_conv_dgrad(g, dY, ldy, Wt, wt_ld, e, ppo_device_status_ptr(), st);
-    if (s != PPO_ERR_UNSUPPORTED) return s;
-    s = tma_gemm_dgrad(g, dY, ldy, Wt, wt_ld, Wc, e, ppo_device_status_ptr(), st);
-    if (s != PPO_ERR_UNSUPPORTED) return s;
-    return tc_gemm_dgrad(g, dY, ldy, Wt, wt_ld, e, ppo_device_status_ptr(), st);
+enum { OP_FWD = 1, OP_DGRAD, OP_WGRAD };
+
+static PlanKey plan_key(int op, const ConvGeom &g) {
+    PlanKey k;
+    memset(&k, 0, sizeof(k));
+    k.op = op;
+    k.g = g;
+    return k;
+}
+
+static int run_fwd(ppo_model *m, const ConvGeom &g, const bf16 *X, const bf16 *W, const FwdEpilogue &e, cudaStream_t st) {
+    PlanKey k = plan_key(OP_FWD, g);
+    const void *p[] = {X, W, e.bias, e.out, e.out_mean, e.out_value, e.out_bits, e.ln_gamma, e.ln_beta, e.ln_xhat, e.ln_rstd};
+    memcpy(k.p, p, sizeof(p));
+    k.v[0] = e.relu; k.v[1] = e.A; k.v[2] = e.ldo;
+    return recorded(m, k, st, [&]() -> int {
+        int s = halo_conv_fwd(g, X, W, e, ppo_device_status_ptr(), st);  // the TMA kernels write e.out_bits themselves
+        if (s != PPO_ERR_UNSUPPORTED) return s;
+        s = tma_gemm_fwd(g, X, W, e, ppo_device_status_ptr(), st);
+        if (s != PPO_ERR_UNSUPPORTED) return s;
+        s = tc_gemm_fwd(g, X, W, e, ppo_device_status_ptr(), st);
+        if (s == PPO_OK && e.out_bits) s = relu_bits(e.out, e.out_bits, g.M(), g.Co, st);
+        return s;
+    });
+}
+
+// layer: conv layer (>= 2) whose regrouped weights the generic TMA kernel reads, made when it first needs them after an
+// update; 0 for a flat product.
+static int run_dgrad(ppo_model *m, const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, int wt_ld, int layer,
+                     const DgradEpilogue &e, cudaStream_t st) {
+    PlanKey k = plan_key(OP_DGRAD, g);
+    const void *p[] = {dY, Wt, nullptr, e.mask_act, e.out, e.out_f32, e.mask_bits};
+    memcpy(k.p, p, sizeof(p));
+    k.v[0] = ldy; k.v[1] = wt_ld; k.v[2] = e.ksplit;
+    if (m->plans)
+        if (const PlanEntry *pe = ppo_find_plan(m->plans, k)) return ppo_replay(*pe, st);
+    const bool halo = halo_dgrad_covers(g, ldy, wt_ld, e);
+    const bf16 *Wc = layer > 0 && !halo ? m->wC + m->wC_off[layer] : nullptr;
+    if (Wc && !m->wC_valid[layer]) {
+        PPO_TRY(tma_dgrad_weights(m->shadow + m->tensors[m->ti_conv[layer]].off, m->wC + m->wC_off[layer], g.Co, g.k, g.Ci, wt_ld, st));
+        m->wC_valid[layer] = true;
+    }
+    k.p[2] = Wc;  // null: the plan does not depend on the regrouped weights and is found above
+    return recorded(m, k, st, [&]() -> int {
+        if (halo) return halo_conv_dgrad(g, dY, ldy, Wt, wt_ld, e, ppo_device_status_ptr(), st);
+        const int s = tma_gemm_dgrad(g, dY, ldy, Wt, wt_ld, Wc, e, ppo_device_status_ptr(), st);
+        if (s != PPO_ERR_UNSUPPORTED) return s;
+        return e.ksplit > 1 ? s : tc_gemm_dgrad(g, dY, ldy, Wt, wt_ld, e, ppo_device_status_ptr(), st);
+    });
 }
 
 static int run_colsum(const bf16 *dZ, int ld, long long M, int N, float *db, float *part, cudaStream_t st);
 
 // Weight and bias gradients of the layer whose weight matrix is tensor ti.  The TMA kernel of a convolution sums
 // the bias gradient on the tensor core on its way; everything else reduces dY in a pass of its own.
-static int run_wgrad(const ppo_model *m, int ti, const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *X,
+static int run_wgrad(ppo_model *m, int ti, const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *X,
                      cudaStream_t st, bool with_bias = true) {
     float *dW = m->grad + m->tensors[ti].off, *db = with_bias ? m->grad + m->tensors[ti + 1].off : nullptr;
     float *part = m->wg_part[ti];
     const size_t cap = m->wg_cap[ti];
     const bool conv = g.k > 1;
-    int s = tma_gemm_wgrad(g, dY, ldy, X, dW, conv ? db : nullptr, part, cap, ppo_device_status_ptr(), st);
-    if (s == PPO_OK && conv) return s;
-    if (s == PPO_ERR_UNSUPPORTED && conv) s = tma_gemm_wgrad(g, dY, ldy, X, dW, nullptr, part, cap, ppo_device_status_ptr(), st);
-    if (s == PPO_ERR_UNSUPPORTED) s = tc_gemm_wgrad(g, dY, ldy, X, dW, part, cap, ppo_device_status_ptr(), st);
-    if (s != PPO_OK || !with_bias) return s;
-    return run_colsum(dY, ldy, g.M(), g.Co, db, m->cs_part[ti], st);
+    PlanKey key = plan_key(OP_WGRAD, g);
+    const void *p[] = {dY, X, dW, db, part};
+    memcpy(key.p, p, sizeof(p));
+    key.v[0] = ldy; key.v[1] = with_bias;
+    return recorded(m, key, st, [&]() -> int {
+        int s = tma_gemm_wgrad(g, dY, ldy, X, dW, conv ? db : nullptr, part, cap, ppo_device_status_ptr(), st);
+        if (s == PPO_OK && conv) return s;
+        if (s == PPO_ERR_UNSUPPORTED && conv) s = tma_gemm_wgrad(g, dY, ldy, X, dW, nullptr, part, cap, ppo_device_status_ptr(), st);
+        if (s == PPO_ERR_UNSUPPORTED) s = tc_gemm_wgrad(g, dY, ldy, X, dW, part, cap, ppo_device_status_ptr(), st);
+        if (s != PPO_OK || !with_bias) return s;
+        return run_colsum(dY, ldy, g.M(), g.Co, db, m->cs_part[ti], st);
+    });
 }
 
 // Blocks a column sum of M rows is cut into (first stage), at most 4 per SM.
@@ -830,21 +933,18 @@ static int run_colsum(const bf16 *dZ, int ld, long long M, int N, float *db, flo
     if (N % 8 == 0 && N <= 256 && ld % 8 == 0) {
         const int rows_per_pass = 256 / (N / 8);
         const int blocks = colsum_blocks(M, (long long)rows_per_pass * 8);
-        colsum_kernel<<<blocks, 256, 0, st>>>(dZ, ld, M, N, part);
-        PPO_LAUNCH_CHECK();
+        PPO_TRY(ppo_launch(colsum_kernel, dim3(blocks), dim3(256), 0, st, dZ, ld, M, N, part));
         return sum_partials(part, blocks, N, db, 0, nullptr, st);
     }
     if (N > 256 && N % 256 == 0) {
         // wide layers: slabs of 256 columns along the grid's second axis
         const int blocks = colsum_blocks(M, 64);
-        colsum_kernel<<<dim3(blocks, N / 256), 256, 0, st>>>(dZ, ld, M, 256, part);
-        PPO_LAUNCH_CHECK();
+        PPO_TRY(ppo_launch(colsum_kernel, dim3(blocks, N / 256), dim3(256), 0, st, dZ, ld, M, 256, part));
         return sum_partials(part, blocks, 256, db, 0, nullptr, st, N / 256);
     }
     int blocks = ppo_cdiv(M, 2048);
     blocks = blocks > 64 ? 64 : (blocks < 1 ? 1 : blocks);
-    colsum_small_kernel<<<blocks, 256, 0, st>>>(dZ, ld, M, N, part);
-    PPO_LAUNCH_CHECK();
+    PPO_TRY(ppo_launch(colsum_small_kernel, dim3(blocks, N), dim3(256), 0, st, dZ, ld, M, N, part));
     return sum_partials(part, blocks, N, db, 0, nullptr, st);
 }
 
@@ -871,13 +971,12 @@ static int wt_ld_of(int Co) { return (Co + 7) / 8 * 8; }
 // contraction of the recurrent trunk, through the flat (1x1-image) input-gradient GEMM.
 // ksplit > 1: the reduction is cut into that many slabs and `out` receives their partial products one after another
 // (rows * N floats each), for the reader to add in order.
-static int gemm_nt_f32(const ppo_model *m, int rows, int N, int K, const bf16 *A, int lda, const bf16 *Wn, float *out,
+static int gemm_nt_f32(ppo_model *m, int rows, int N, int K, const bf16 *A, int lda, const bf16 *Wn, float *out,
                        cudaStream_t st, int ksplit = 1) {
     ConvGeom g = fc_geom(rows, N, K);
     DgradEpilogue e = {nullptr, nullptr, out};
     e.ksplit = ksplit;
-    if (ksplit > 1) return tma_gemm_dgrad(g, A, lda, Wn, K, nullptr, e, ppo_device_status_ptr(), st);
-    return run_dgrad(m, g, A, lda, Wn, Wn, K, nullptr, e, st);
+    return run_dgrad(m, g, A, lda, Wn, K, 0, e, st);
 }
 
 // Forward of the recurrent trunk over the announced sequence (rows = T * Be, time-major): per layer one GEMM for
@@ -891,19 +990,17 @@ static int lstm_forward(ppo_model *m, int rows, cudaStream_t st) {
         const bf16 *X = l == 0 ? m->h[0] : m->lstm_hs[l - 1];
         float *cprev = m->lstm_c[l] + (size_t)m->mbmax * H;
         PPO_TRY(gemm_nt_f32(m, rows, 4 * H, in, X, in, m->shadow + m->tensors[ti].off, m->lstm_xg, st));
-        lstm_init_kernel<<<ppo_cdiv((long long)Be * H, 256), 256, 0, st>>>(m->seq_h_init + (size_t)l * Be * H,
+        PPO_TRY(ppo_launch(lstm_init_kernel, dim3(ppo_cdiv((long long)Be * H, 256)), dim3(256), 0, st, m->seq_h_init + (size_t)l * Be * H,
                                                                           m->seq_c_init + (size_t)l * Be * H,
-                                                                          m->lstm_hprev[l], cprev, Be * H);
-        PPO_LAUNCH_CHECK();
+                                                                          m->lstm_hprev[l], cprev, Be * H));
         for (int t = 0; t < T; ++t) {
             const size_t r0 = (size_t)t * Be;
             PPO_TRY(gemm_nt_f32(m, Be, 4 * H, H, m->lstm_hprev[l] + r0 * H, H, m->shadow + m->tensors[ti + 1].off, m->lstm_hg, st));
             const bool last = t == T - 1;
-            lstm_cell_fwd_kernel<<<ppo_cdiv((long long)Be * H, 256), 256, 0, st>>>(
+            PPO_TRY(ppo_launch(lstm_cell_fwd_kernel, dim3(ppo_cdiv((long long)Be * H, 256)), dim3(256), 0, st, 
                 m->lstm_xg + r0 * 4 * H, m->lstm_hg, m->master + m->tensors[ti + 2].off, cprev + r0 * H, m->seq_done + r0,
                 m->lstm_gates[l] + r0 * 4 * H, m->lstm_c[l] + r0 * H, m->lstm_hs[l] + r0 * H,
-                last ? nullptr : m->lstm_hprev[l] + (r0 + Be) * H, last ? nullptr : cprev + (r0 + Be) * H, Be, H);
-            PPO_LAUNCH_CHECK();
+                last ? nullptr : m->lstm_hprev[l] + (r0 + Be) * H, last ? nullptr : cprev + (r0 + Be) * H, Be, H));
         }
     }
     return PPO_OK;
@@ -924,10 +1021,9 @@ static int lstm_backward(ppo_model *m, int rows, cudaStream_t st) {
         int nsplit = (T >= 4 && Be <= 512) ? 4 : 1;
         for (int t = T - 1; t >= 0; --t) {
             const size_t r0 = (size_t)t * Be;
-            lstm_cell_bwd_kernel<<<ppo_cdiv((long long)Be * H, 256), 256, 0, st>>>(
+            PPO_TRY(ppo_launch(lstm_cell_bwd_kernel, dim3(ppo_cdiv((long long)Be * H, 256)), dim3(256), 0, st, 
                 m->lstm_dtop + r0 * H, m->lstm_dhc, m->lstm_dcc, m->seq_done + r0, m->lstm_gates[l] + r0 * 4 * H,
-                m->lstm_c[l] + r0 * H, cprev + r0 * H, m->lstm_dg + r0 * 4 * H, Be, H, t == T - 1 ? 1 : 0, nsplit);
-            PPO_LAUNCH_CHECK();
+                m->lstm_c[l] + r0 * H, cprev + r0 * H, m->lstm_dg + r0 * 4 * H, Be, H, t == T - 1 ? 1 : 0, nsplit));
             if (t > 0) {  // raw gradient of the state this step started from: dg W_h
                 int s = PPO_ERR_UNSUPPORTED;
                 if (nsplit > 1)
@@ -975,11 +1071,11 @@ extern "C" int ppo_encoder_fwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
 #define PPO_CONV1(KS_)                                                                                              \
     do {                                                                                                            \
         if (stage)                                                                                                  \
-            conv1_fwd_kernel<KS_, true><<<blocks, 128, smem, st>>>(depth, W, bias, m->act[1], m->abits[1], rows, d.H, d.W,       \
-                                                                   m->Hs[1], m->Ws[1], C1);                         \
+            PPO_TRY(ppo_launch(conv1_fwd_kernel<KS_, true>, dim3(blocks), dim3(128), smem, st, depth, W, bias, m->act[1], m->abits[1], rows, d.H, d.W,       \
+                                                                   m->Hs[1], m->Ws[1], C1));                         \
         else                                                                                                        \
-            conv1_fwd_kernel<KS_, false><<<blocks, 128, smem, st>>>(depth, W, bias, m->act[1], m->abits[1], rows, d.H, d.W,      \
-                                                                    m->Hs[1], m->Ws[1], C1);                        \
+            PPO_TRY(ppo_launch(conv1_fwd_kernel<KS_, false>, dim3(blocks), dim3(128), smem, st, depth, W, bias, m->act[1], m->abits[1], rows, d.H, d.W,      \
+                                                                    m->Hs[1], m->Ws[1], C1));                        \
     } while (0)
         if (tcs == PPO_OK) { /* done on the tensor cores */ }
         else if (KS == 1) PPO_CONV1(1);
@@ -987,7 +1083,6 @@ extern "C" int ppo_encoder_fwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
         else if (KS == 5) PPO_CONV1(5);
         else PPO_CONV1(7);
 #undef PPO_CONV1
-        PPO_LAUNCH_CHECK();
     }
     for (int l = 2; l <= m->L; ++l) {
         ConvGeom g = conv_geom(m, l, rows);
@@ -1008,13 +1103,12 @@ extern "C" int ppo_encoder_fwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
         FwdEpilogue e = {m->master + m->tensors[m->ti_embed + 1].off, 1, m->h[0], nullptr, nullptr, 0};
         e.ldo = m->hw[0];
         PPO_TRY(run_fwd(m, g, m->act[m->L], m->shadow + m->tensors[m->ti_embed].off, e, st));
-        concat_proprio_kernel<<<ppo_cdiv((long long)rows * d.P, 256), 256, 0, st>>>(mb->proprio + (size_t)row0 * d.P, m->h[0],
-                                                                                  rows, d.embed, d.P, m->hw[0]);
+        PPO_TRY(ppo_launch(concat_proprio_kernel, dim3(ppo_cdiv((long long)rows * d.P, 256)), dim3(256), 0, st, mb->proprio + (size_t)row0 * d.P, m->h[0],
+                                                                                  rows, d.embed, d.P, m->hw[0]));
     } else {
-        pool_concat_kernel<<<ppo_cdiv(rows, 8), 256, 0, st>>>(m->act[m->L], mb->proprio + (size_t)row0 * d.P, m->h[0], rows,
-                                                              m->Hs[m->L] * m->Ws[m->L], m->Cs[m->L], d.P);
+        PPO_TRY(ppo_launch(pool_concat_kernel, dim3(ppo_cdiv(rows, 8)), dim3(256), 0, st, m->act[m->L], mb->proprio + (size_t)row0 * d.P, m->h[0], rows,
+                                                              m->Hs[m->L] * m->Ws[m->L], m->Cs[m->L], d.P));
     }
-    PPO_LAUNCH_CHECK();
     if (d.n_lstm > 0) PPO_TRY(lstm_forward(m, rows, st));
     int ti = m->ti_fc[1];
     for (int l = 1; l <= m->F; ++l, ti += 2) {
@@ -1035,41 +1129,29 @@ extern "C" int ppo_encoder_fwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
 
 static int refresh_transposed(ppo_model *m, cudaStream_t st) {
     if (m->wT_valid) return PPO_OK;
-    for (int l = 2; l <= m->L; ++l) {
-        const int Co = m->Cs[l], Ci = m->Cs[l - 1], taps = m->d.conv_k[l - 1] * m->d.conv_k[l - 1];
-        const int tc = m->ti_conv[l];
-        const long long total = (long long)Ci * taps * wt_ld_of(Co);
-        transpose_weights_kernel<<<ppo_cdiv(total, 256), 256, 0, st>>>(m->shadow + m->tensors[tc].off,
-                                                                     m->wT + m->wT_off[tc], Co, taps, Ci, wt_ld_of(Co));
-        PPO_LAUNCH_CHECK();
-        PPO_TRY(tma_dgrad_weights(m->shadow + m->tensors[tc].off, m->wC + m->wC_off[l], Co, m->d.conv_k[l - 1], Ci,
-                                  wt_ld_of(Co), st));
-    }
-    if (m->ti_embed >= 0) {
-        const int Ci = m->Hs[m->L] * m->Ws[m->L] * m->Cs[m->L], Co = m->d.embed;
-        const long long total = (long long)Ci * wt_ld_of(Co);
-        transpose_weights_kernel<<<ppo_cdiv(total, 256), 256, 0, st>>>(m->shadow + m->tensors[m->ti_embed].off,
-                                                                     m->wT + m->wT_off[m->ti_embed], Co, 1, Ci, wt_ld_of(Co));
-        PPO_LAUNCH_CHECK();
-    }
+    TransposeJobs jobs;
+    int n = 0;
+    long long blocks = 0;
+    auto add = [&](int ti, int Co, int taps, int Ci) {
+        TransposeJob &j = jobs.j[n++];
+        j.src = m->tensors[ti].off;
+        j.dst = m->wT_off[ti];
+        j.Co = Co; j.taps = taps; j.Ci = Ci;
+        j.ld = wt_ld_of(Co);
+        blocks += (long long)((j.ld + 63) / 64) * (((long long)taps * Ci + 63) / 64);
+        j.block_end = (int)blocks;
+    };
+    for (int l = 2; l <= m->L; ++l) add(m->ti_conv[l], m->Cs[l], m->d.conv_k[l - 1] * m->d.conv_k[l - 1], m->Cs[l - 1]);
+    if (m->ti_embed >= 0) add(m->ti_embed, m->d.embed, 1, m->Hs[m->L] * m->Ws[m->L] * m->Cs[m->L]);
     for (int l = 0; l < m->d.n_lstm; ++l) {
-        const int H = m->d.lstm_h, in = l == 0 ? m->hw[0] : H, tl = m->ti_lstm[l];
-        transpose_weights_kernel<<<ppo_cdiv((long long)in * 4 * H, 256), 256, 0, st>>>(m->shadow + m->tensors[tl].off,
-                                                                                     m->wT + m->wT_off[tl], 4 * H, 1, in, 4 * H);
-        PPO_LAUNCH_CHECK();
-        transpose_weights_kernel<<<ppo_cdiv((long long)H * 4 * H, 256), 256, 0, st>>>(m->shadow + m->tensors[tl + 1].off,
-                                                                                    m->wT + m->wT_off[tl + 1], 4 * H, 1, H, 4 * H);
-        PPO_LAUNCH_CHECK();
+        add(m->ti_lstm[l], 4 * m->d.lstm_h, 1, l == 0 ? m->hw[0] : m->d.lstm_h);
+        add(m->ti_lstm[l] + 1, 4 * m->d.lstm_h, 1, m->d.lstm_h);
     }
-    int ti = m->ti_fc[1];
-    for (int l = 1; l <= m->F + 1; ++l, ti += 2) {
-        const int Ci = fc_input_width(m, l), Co = (l <= m->F) ? m->hw[l] : m->d.A + 1;
-        const long long total = (long long)Ci * wt_ld_of(Co);
-        transpose_weights_kernel<<<ppo_cdiv(total, 256), 256, 0, st>>>(m->shadow + m->tensors[ti].off,
-                                                                     m->wT + m->wT_off[ti], Co, 1, Ci, wt_ld_of(Co));
-        PPO_LAUNCH_CHECK();
-    }
+    for (int l = 1; l <= m->F + 1; ++l) add(m->ti_fc[l], l <= m->F ? m->hw[l] : m->d.A + 1, 1, fc_input_width(m, l));
+    if (blocks > 0x7fffffffll) return PPO_ERR_UNSUPPORTED;
+    PPO_TRY(ppo_launch(transpose_weights_kernel, dim3((unsigned)blocks), dim3(256), 0, st, m->shadow, m->wT, jobs));
     m->wT_valid = true;
+    for (int l = 2; l <= m->L; ++l) m->wC_valid[l] = false;
     return PPO_OK;
 }
 
@@ -1115,8 +1197,8 @@ static int conv1_wgrad(ppo_model *m, const ppo_minibatch *mb, int row0, int rows
         if (smem > 48 * 1024)                                                                                \
             PPO_CUDA_CHECK(cudaFuncSetAttribute(conv1_wgrad_mma_kernel<KS_, NB_>,                            \
                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));    \
-        conv1_wgrad_mma_kernel<KS_, NB_><<<blocks, 256, smem, st>>>(depth, m->dact[1], m->c1_part, rows, d.H, \
-                                                                    d.W, m->Hs[1], m->Ws[1], per_warp);      \
+        PPO_TRY(ppo_launch(conv1_wgrad_mma_kernel<KS_, NB_>, dim3(blocks), dim3(256), smem, st, depth, m->dact[1], m->c1_part, rows, d.H, \
+                                                                    d.W, m->Hs[1], m->Ws[1], per_warp));      \
     } while (0)
         const int nb = C1 / 8;
         if (KS == 3 && nb == 2) PPO_C1W(3, 2);
@@ -1128,7 +1210,6 @@ static int conv1_wgrad(ppo_model *m, const ppo_minibatch *mb, int row0, int rows
         else if (KS == 5 && nb == 6) PPO_C1W(5, 6);
         else PPO_C1W(5, 8);
 #undef PPO_C1W
-        PPO_LAUNCH_CHECK();
         return sum_partials(m->c1_part, blocks, C1 * KS * KS, dW, C1, db, st);
     }
     const int cpt = KS <= 3 ? 8 : (KS == 5 ? 4 : 2);
@@ -1144,8 +1225,8 @@ static int conv1_wgrad(ppo_model *m, const ppo_minibatch *mb, int row0, int rows
     float *dW = m->grad + m->tensors[0].off, *db = m->grad + m->tensors[1].off;
     if ((size_t)blocks * C1 * (KS * KS + 1) > m->c1_cap) return PPO_ERR_SHAPE;
 #define PPO_CONV1W(KS_, CPT_, U_)                                                                                 \
-    conv1_wgrad_kernel<KS_, CPT_, U_><<<blocks, 128, smem, st>>>(depth, m->dact[1], m->c1_part, rows, d.H, d.W,  \
-                                                             m->Hs[1], m->Ws[1], C1, per_warp)
+    PPO_TRY(ppo_launch(conv1_wgrad_kernel<KS_, CPT_, U_>, dim3(blocks), dim3(128), smem, st, depth, m->dact[1], m->c1_part, rows, d.H, d.W,  \
+                                                             m->Hs[1], m->Ws[1], C1, per_warp))
     if (smem > 48 * 1024) {
         if (KS == 5) PPO_CUDA_CHECK(cudaFuncSetAttribute(conv1_wgrad_kernel<5, 4, 1>,
                                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -1157,7 +1238,6 @@ static int conv1_wgrad(ppo_model *m, const ppo_minibatch *mb, int row0, int rows
     else if (KS == 5) PPO_CONV1W(5, 4, 1);
     else PPO_CONV1W(7, 2, 1);
 #undef PPO_CONV1W
-    PPO_LAUNCH_CHECK();
     return sum_partials(m->c1_part, blocks, C1 * KS * KS, dW, C1, db, st);
 }
 
@@ -1176,8 +1256,7 @@ extern "C" int ppo_encoder_bwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
     }
     PPO_TRY(refresh_transposed(m, st));
 
-    pack_dout_kernel<<<ppo_cdiv((long long)rows * 16, 256), 256, 0, st>>>(dmean, dvalue, m->dh[F + 1], rows, d.A);
-    PPO_LAUNCH_CHECK();
+    PPO_TRY(ppo_launch(pack_dout_kernel, dim3(ppo_cdiv((long long)rows * 16, 256)), dim3(256), 0, st, dmean, dvalue, m->dh[F + 1], rows, d.A));
     // Weight and bias gradients are leaves of the dependency graph: only the chain of dgrads has to run in order.
     // The leaves of the FC layers (small kernels on a fraction of the SMs) and, further down, conv1's wgrad go to
     // a second stream that forks from the caller's stream whenever the gradient they read is ready and joins it
@@ -1210,7 +1289,7 @@ extern "C" int ppo_encoder_bwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
         DgradEpilogue e;
         if (l > 1) e = {m->h[l - 1], m->dh[l - 1], nullptr};
         else e = {nullptr, nullptr, d.n_lstm > 0 ? m->lstm_dtop : m->dh0_f32};
-        s = run_dgrad(m, g, dY, ldy, m->shadow + m->tensors[ti].off, m->wT + m->wT_off[ti], wt_ld_of(Co), nullptr, e, st);
+        s = run_dgrad(m, g, dY, ldy, m->wT + m->wT_off[ti], wt_ld_of(Co), 0, e, st);
         if (s == PPO_OK && l > 1) s = fork_here();  // dh[l-1] is ready for the next leaf
         if (s != PPO_OK) return join(s);
     }
@@ -1223,20 +1302,18 @@ extern "C" int ppo_encoder_bwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
         // ReLU of the last conv output, which the flattened vector is)
         const int te = m->ti_embed, E = d.embed;
         ConvGeom g = fc_geom(rows, m->Hs[L] * m->Ws[L] * m->Cs[L], E);
-        embed_dz_kernel<<<ppo_cdiv((long long)rows * E, 256), 256, 0, st>>>(m->dh0_f32, m->h[0], m->dze, rows, E, m->hw[0]);
-        PPO_LAUNCH_CHECK();
+        PPO_TRY(ppo_launch(embed_dz_kernel, dim3(ppo_cdiv((long long)rows * E, 256)), dim3(256), 0, st, m->dh0_f32, m->h[0], m->dze, rows, E, m->hw[0]));
         int s = fork_here();
         if (s == PPO_OK) s = run_wgrad(m, te, g, m->dze, E, m->act[L], leaf);
         DgradEpilogue e = {m->act[L], m->dact[L], nullptr};
         if (s == PPO_OK)
-            s = run_dgrad(m, g, m->dze, E, m->shadow + m->tensors[te].off, m->wT + m->wT_off[te], wt_ld_of(E), nullptr, e, st);
+            s = run_dgrad(m, g, m->dze, E, m->wT + m->wT_off[te], wt_ld_of(E), 0, e, st);
         if (s != PPO_OK) return join(s);
     } else {
         const int npx = m->Hs[L] * m->Ws[L], C = m->Cs[L];
         const long long total8 = (long long)rows * npx * C / 8;
-        unpool_kernel<<<ppo_cdiv(total8, 256), 256, 0, st>>>(m->dh0_f32, m->act[L], m->dact[L], total8, npx, C,
-                                                           m->hw[0]);
-        PPO_LAUNCH_CHECK();
+        PPO_TRY(ppo_launch(unpool_kernel, dim3(ppo_cdiv(total8, 256)), dim3(256), 0, st, m->dh0_f32, m->act[L], m->dact[L], total8, npx, C,
+                                                           m->hw[0]));
     }
     // With layer normalisation dact[l] arrives as the gradient of the normalised, scaled and shifted value; ln_bwd
     // turns it in place into the gradient of the convolution's output and adds the gamma and beta gradients.
@@ -1250,9 +1327,8 @@ extern "C" int ppo_encoder_bwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
         const int cap = ppo_num_sms() * 4;
         blocks = blocks > cap ? cap : (blocks < 1 ? 1 : blocks);
         if ((size_t)blocks * 2 * C > m->ln_cap) return PPO_ERR_SHAPE;
-        ln_bwd_kernel<<<blocks, 256, 0, st>>>(m->dact[l], m->xhat[l], m->rstd[l], m->master + m->tensors[tc + 2].off, M, C,
-                                              m->ln_part);
-        PPO_LAUNCH_CHECK();
+        PPO_TRY(ppo_launch(ln_bwd_kernel, dim3(blocks), dim3(256), 0, st, m->dact[l], m->xhat[l], m->rstd[l], m->master + m->tensors[tc + 2].off, M, C,
+                                              m->ln_part));
         return sum_partials(m->ln_part, blocks, C, m->grad + m->tensors[tc + 2].off, C, m->grad + m->tensors[tc + 3].off, st);
     };
     // The chain of dgrads first; then the wgrads of the GEMM layers one after the other on the caller's stream
@@ -1269,8 +1345,7 @@ extern "C" int ppo_encoder_bwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
         if (s == PPO_OK && !fork)
             s = run_wgrad(m, ti, g, m->dact[l], g.Co, m->act[l - 1], st);
         if (s == PPO_OK)
-            s = run_dgrad(m, g, m->dact[l], g.Co, m->shadow + m->tensors[ti].off, m->wT + m->wT_off[ti],
-                          wt_ld_of(g.Co), m->wC + m->wC_off[l], e, st);
+            s = run_dgrad(m, g, m->dact[l], g.Co, m->wT + m->wT_off[ti], wt_ld_of(g.Co), l, e, st);
         if (s != PPO_OK) return join(s);
     }
     {

@@ -57,6 +57,8 @@ int tma_gemm_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, i
 // 3x3 layers whose weights fit in shared memory (conv_halo.cu): the same forward and input gradient from halo tiles;
 // PPO_ERR_UNSUPPORTED (nothing launched) for anything else.
 int halo_conv_fwd(const ConvGeom &g, const bf16 *X, const bf16 *W, const FwdEpilogue &e, int32_t *status, cudaStream_t st);
+// Whether halo_conv_dgrad takes such a layer (it then does not read the regrouped weights).
+bool halo_dgrad_covers(const ConvGeom &g, int ldy, int wt_ld, const DgradEpilogue &e);
 int halo_conv_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, int wt_ld, const DgradEpilogue &e,
                     int32_t *status, cudaStream_t st);
 size_t tma_dgrad_weight_elems(int Ci, int k, int wt_ld);

@@ -15,6 +15,7 @@
 // memory descriptors name.  Read K-major, a row is one M/N index and its 64 columns are K; read
 // MN-major, a row is one K index and its 64 columns are M/N.
 #include "gemm.cuh"
+#include "launch.cuh"
 #include "tcgen05.cuh"
 
 namespace {
@@ -108,6 +109,7 @@ __global__ void __launch_bounds__(kKThreads, 1) igemm_kmajor_kernel(const __grid
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == kGatherWarps) tmem_alloc(&pipe->tmem_slot, ncols);
+    grid_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -401,6 +403,7 @@ __global__ void __launch_bounds__(kThreads) igemm_wgrad_kernel(const __grid_cons
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 4) tmem_alloc(&pipe->tmem_slot, ncols);
+    grid_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -571,8 +574,7 @@ int launch_kmajor(KArgs &a, cudaStream_t st) {
     a.stages = kmajor_stages(a.BN);
     const int sms = ppo_num_sms();
     const unsigned grid = (unsigned)(tiles < sms ? tiles : sms);
-    igemm_kmajor_kernel<<<grid, kKThreads, kmajor_smem(a.BN), st>>>(a);
-    PPO_LAUNCH_CHECK();
+    PPO_TRY(ppo_launch(igemm_kmajor_kernel, dim3(grid), dim3(kKThreads), kmajor_smem(a.BN), st, a));
     return PPO_OK;
 }
 
@@ -673,7 +675,6 @@ int tc_gemm_wgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *X, flo
     a.doh64 = (64 % (g.Ho * g.Wo)) / g.Wo;
     a.dow64 = 64 % g.Wo;
     dim3 grid((unsigned)((a.Kfwd + 127) / 128), (unsigned)((g.Co + a.BN - 1) / a.BN), (unsigned)splits);
-    igemm_wgrad_kernel<<<grid, kThreads, wgrad_smem(a.BN), st>>>(a);
-    PPO_LAUNCH_CHECK();
+    PPO_TRY(ppo_launch(igemm_wgrad_kernel, dim3(grid), dim3(kThreads), wgrad_smem(a.BN), st, a));
     return wgrad_reduce(part, jtiles, ctiles, (int)splits, a.BN, a.Kfwd, g.Co, dW, nullptr, 0, st);
 }

@@ -27,6 +27,7 @@
 // Every wait is bounded: on a time-out the kernel records PPO_ERR_TIMEOUT, waits (bounded) for the
 // copies it has in flight, frees its tensor memory and returns.
 #include "gemm.cuh"
+#include "launch.cuh"
 #include "tcgen05.cuh"
 #include "tma_host.cuh"
 
@@ -250,6 +251,8 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
         pipe->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (warp == 1) tmem_alloc(&pipe->tmem_slot, ncols);
+    grid_wait();
     if (a.mode != EPI_DGRAD)
         for (int i = threadIdx.x; i < a.tiles_n * BN; i += (int)blockDim.x) pipe->bias[i] = i < a.N ? a.bias[i] : 0.f;
     if (a.ln_gamma)
@@ -264,7 +267,6 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
             if (tap < a.cls[c].taps.n)
                 pipe->wtab[c][q] = (uint32_t)((int)a.cls[c].taps.wt[tap] * a.kchunks + kc) * (b_bytes >> 4);
         }
-    if (warp == 1) tmem_alloc(&pipe->tmem_slot, ncols);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -696,6 +698,7 @@ __global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_con
     }
     fence_async_smem();
     if (warp == 1) tmem_alloc(&pipe->tmem_slot, ncols);
+    grid_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -819,6 +822,7 @@ __global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_con
 __global__ void __launch_bounds__(256) wgrad_reduce_kernel(const float *__restrict__ part, int jtiles, int ctiles,
                                                            int splits, int BN, int Kfwd, int Co, float *__restrict__ dW,
                                                            float *__restrict__ db, int ones_row) {
+    grid_wait();
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long nW = (long long)Co * Kfwd;
     int co, jj;
@@ -838,7 +842,15 @@ __global__ void __launch_bounds__(256) wgrad_reduce_kernel(const float *__restri
     const size_t tile = (size_t)128 * BN, per_split = (size_t)ctiles * jtiles * tile;
     const float *src = part + ((size_t)y * jtiles + x) * tile + (size_t)c * 128 + p;
     float acc = 0.f;
-    for (int z = 0; z < splits; ++z) acc += src[(size_t)z * per_split];
+    int z = 0;
+    for (; z + 16 <= splits; z += 16) {  // the loads of sixteen splits are in flight while the sum stays in order
+        float v[16];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) v[u] = src[(size_t)(z + u) * per_split];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) acc += v[u];
+    }
+    for (; z < splits; ++z) acc += src[(size_t)z * per_split];
     *dst += acc;
 }
 
@@ -1021,8 +1033,7 @@ int launch_kmajor(KArgs &a, cudaStream_t st) {
     const long long ctas = two ? 2ll * sms : sms;
     const unsigned grid = (unsigned)(total < ctas ? total : ctas);
     const size_t smem = (size_t)a.stages * G * sub + (a.wres ? res : 0) + fixed;
-    tma_kmajor_kernel<<<grid, (2 + a.nepi) * 32, smem, st>>>(a);
-    PPO_LAUNCH_CHECK();
+    PPO_TRY(ppo_launch(tma_kmajor_kernel, dim3(grid), dim3((2 + a.nepi) * 32), smem, st, a));
     return PPO_OK;
 }
 
@@ -1241,6 +1252,7 @@ size_t tma_dgrad_weight_elems(int Ci, int k, int wt_ld) {
 // when that tap exists, else 0.
 __global__ void __launch_bounds__(256) dgrad_weights_kernel(const bf16 *__restrict__ W, bf16 *__restrict__ Wc, int Co,
                                                             int k, int Ci, int ld, int dmin, int n1) {
+    grid_wait();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long total = (long long)4 * Ci * n1 * n1 * ld;
     if (i >= total) return;
@@ -1259,16 +1271,14 @@ int tma_dgrad_weights(const bf16 *W, bf16 *Wc, int Co, int k, int Ci, int wt_ld,
     int dmin, n1;
     tma_dgrad_shifts(k, &dmin, &n1);
     const long long total = (long long)tma_dgrad_weight_elems(Ci, k, wt_ld);
-    dgrad_weights_kernel<<<ppo_cdiv(total, 256), 256, 0, st>>>(W, Wc, Co, k, Ci, wt_ld, dmin, n1);
-    PPO_LAUNCH_CHECK();
+    PPO_TRY(ppo_launch(dgrad_weights_kernel, dim3(ppo_cdiv(total, 256)), dim3(256), 0, st, W, Wc, Co, k, Ci, wt_ld, dmin, n1));
     return PPO_OK;
 }
 
 int wgrad_reduce(const float *part, int jtiles, int ctiles, int splits, int BN, int Kfwd, int Co, float *dW, float *db,
                  int ones_row, cudaStream_t st) {
     const long long n = (long long)Co * Kfwd + (db ? Co : 0);
-    wgrad_reduce_kernel<<<ppo_cdiv(n, 256), 256, 0, st>>>(part, jtiles, ctiles, splits, BN, Kfwd, Co, dW, db, ones_row);
-    PPO_LAUNCH_CHECK();
+    PPO_TRY(ppo_launch(wgrad_reduce_kernel, dim3(ppo_cdiv(n, 256)), dim3(256), 0, st, part, jtiles, ctiles, splits, BN, Kfwd, Co, dW, db, ones_row));
     return PPO_OK;
 }
 
@@ -1338,8 +1348,7 @@ int tma_gemm_wgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *X, fl
     a.tiles_per_split = (a.grid.tiles + splits - 1) / splits;
     splits = (a.grid.tiles + a.tiles_per_split - 1) / a.tiles_per_split;  // every split has at least one pixel tile
     dim3 grid((unsigned)jtiles, (unsigned)ctiles, (unsigned)splits);
-    tma_wgrad_kernel<<<grid, kThreads, (size_t)a.stages * stage + sizeof(Pipe) + 1024, st>>>(a);
-    PPO_LAUNCH_CHECK();
+    PPO_TRY(ppo_launch(tma_wgrad_kernel, dim3(grid), dim3(kThreads), (size_t)a.stages * stage + sizeof(Pipe) + 1024, st, a));
     return wgrad_reduce(part, jtiles, ctiles, splits, a.BN, a.Kfwd, g.Co, dW, db,
                         db ? (jtiles - 1) * 128 + a.ones_blk * CB : 0, st);
 }

@@ -5,6 +5,7 @@
 #include <new>
 
 #include "common.cuh"
+#include "launch.cuh"
 #include "gemm.cuh"
 
 static int conv_out(int in, int k) { return (in + 2 * (k / 2) - k) / 2 + 1; }
@@ -140,6 +141,7 @@ extern "C" int ppo_model_destroy(ppo_model *m) {
         cudaEventDestroy(m->ev_fork);
         cudaEventDestroy(m->ev_join);
     }
+    delete m->plans;
     delete m;
     return PPO_OK;
 }
@@ -191,7 +193,8 @@ static size_t carve(ppo_model *m, const ppo_model *shape, int mb, char *base) {
         if (m) m->wC = (bf16 *)wc;
         int blocks = ppo_cdiv(mb, kLossThreads);
         char *lp = take((size_t)blocks * 32 * sizeof(float));
-        if (m) { m->loss_partials = (float *)lp; m->loss_partial_blocks = blocks; }
+        char *lt = take(sizeof(unsigned int));
+        if (m) { m->loss_partials = (float *)lp; m->loss_partial_blocks = blocks; m->loss_ticket = (unsigned int *)lt; }
         char *am = take((size_t)mb * shape->d.A * sizeof(float));
         if (m) m->act_mean = (float *)am;
         // scratch of the two-stage gradient reductions (sizes do not depend on the micro-batch)
@@ -259,6 +262,7 @@ extern "C" int ppo_model_bind(ppo_model *m, float *master, void *shadow, float *
         !ppo_aligned(av, 16) || !ppo_aligned(ws, 256))
         return PPO_ERR_ALIGN;
     if (ws_bytes < ppo_model_workspace_bytes(m, microbatch)) return PPO_ERR_SHAPE;
+    if (m->plans) m->plans->map.clear();  // they hold the old addresses
     m->master = master;
     m->shadow = static_cast<bf16 *>(shadow);
     m->grad = grad;
@@ -270,6 +274,7 @@ extern "C" int ppo_model_bind(ppo_model *m, float *master, void *shadow, float *
     carve(m, m, microbatch, m->ws);
     m->fwd_valid = false;
     m->wT_valid = false;
+    m->ticket_zeroed = false;
     return PPO_OK;
 }
 
@@ -329,6 +334,7 @@ extern "C" int ppo_model_set_sequence(ppo_model *m, int T, int Be, const uint8_t
 __global__ void __launch_bounds__(256) lstm_read_state_kernel(const bf16 *__restrict__ h, const float *__restrict__ c,
                                                               const uint8_t *__restrict__ done, float *__restrict__ h_out,
                                                               float *__restrict__ c_out, int Be, int H) {
+    grid_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= Be * H) return;
     const bool reset = done[i / H] != 0;
@@ -342,10 +348,9 @@ extern "C" int ppo_model_read_state(const ppo_model *m, float *h_out, float *c_o
     const int Be = m->seq_Be, H = m->d.lstm_h;
     const size_t last = (size_t)(m->seq_T - 1) * Be;
     for (int l = 0; l < m->d.n_lstm; ++l) {
-        lstm_read_state_kernel<<<ppo_cdiv((long long)Be * H, 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(
+        PPO_TRY(ppo_launch(lstm_read_state_kernel, dim3(ppo_cdiv((long long)Be * H, 256)), dim3(256), 0, static_cast<cudaStream_t>(stream), 
             m->lstm_hs[l] + last * H, m->lstm_c[l] + last * H, m->seq_done + last, h_out + (size_t)l * Be * H,
-            c_out + (size_t)l * Be * H, Be, H);
-        PPO_LAUNCH_CHECK();
+            c_out + (size_t)l * Be * H, Be, H));
     }
     return PPO_OK;
 }
@@ -366,6 +371,7 @@ extern "C" int ppo_model_sync_masks(ppo_model *m, int rows, void *stream) {
 
 __global__ void __launch_bounds__(256) shadow_kernel(const float4 *__restrict__ master, uint2 *__restrict__ shadow,
                                                      size_t n4) {
+    grid_wait();
     size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n4) return;
     float4 x = master[i];
@@ -379,9 +385,8 @@ __global__ void __launch_bounds__(256) shadow_kernel(const float4 *__restrict__ 
 extern "C" int ppo_model_sync_shadow(ppo_model *m, void *stream) {
     if (!m || !m->master) return PPO_ERR_STATE;
     size_t n4 = m->arena / 4;
-    shadow_kernel<<<ppo_cdiv(n4, 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        reinterpret_cast<const float4 *>(m->master), reinterpret_cast<uint2 *>(m->shadow), n4);
-    PPO_LAUNCH_CHECK();
+    PPO_TRY(ppo_launch(shadow_kernel, dim3(ppo_cdiv(n4, 256)), dim3(256), 0, static_cast<cudaStream_t>(stream), 
+        reinterpret_cast<const float4 *>(m->master), reinterpret_cast<uint2 *>(m->shadow), n4));
     m->wT_valid = false;
     return PPO_OK;
 }
@@ -401,6 +406,7 @@ __global__ void __launch_bounds__(256) adam_kernel(float4 *__restrict__ theta, f
                                                    float4 *__restrict__ v, const float4 *__restrict__ g,
                                                    uint2 *__restrict__ shadow, size_t n4, float lr, float b1,
                                                    float b2, float eps, float inv_c1, float inv_c2) {
+    grid_wait();
     const size_t nth = (size_t)gridDim.x * blockDim.x;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += nth) {
         float4 th = theta[i], mm = m[i], vv = v[i];
@@ -435,11 +441,10 @@ extern "C" int ppo_adam_step(ppo_model *m, float lr, float beta1, float beta2, f
     int blocks = ppo_cdiv(n4, 256);
     const int cap = ppo_num_sms() * 8;
     if (blocks > cap) blocks = cap;
-    adam_kernel<<<blocks, 256, 0, static_cast<cudaStream_t>(stream)>>>(
+    PPO_TRY(ppo_launch(adam_kernel, dim3(blocks), dim3(256), 0, static_cast<cudaStream_t>(stream), 
         reinterpret_cast<float4 *>(m->master), reinterpret_cast<float4 *>(m->adam_m),
         reinterpret_cast<float4 *>(m->adam_v), reinterpret_cast<const float4 *>(m->grad),
-        reinterpret_cast<uint2 *>(m->shadow), n4, lr, beta1, beta2, eps, (float)(1.0 / c1), (float)(1.0 / c2));
-    PPO_LAUNCH_CHECK();
+        reinterpret_cast<uint2 *>(m->shadow), n4, lr, beta1, beta2, eps, (float)(1.0 / c1), (float)(1.0 / c2)));
     m->wT_valid = false;
     m->fwd_valid = false;
     return PPO_OK;
@@ -462,8 +467,11 @@ __global__ void __launch_bounds__(kLossThreads) loss_kernel(
     int rows, int A, float inv_Bt, const float *__restrict__ mean, const float *__restrict__ value,
     const float *__restrict__ logsigma, const float *__restrict__ action, const float *__restrict__ logp_old,
     const float *__restrict__ adv, const float *__restrict__ ret, float clip, float vf_coef,
-    float *__restrict__ dmean, float *__restrict__ dvalue, float *__restrict__ partials) {
+    float *__restrict__ dmean, float *__restrict__ dvalue, float *__restrict__ partials, unsigned int *ticket, float share,
+    float ent_coef, float *__restrict__ loss_out, float *__restrict__ grad_logsigma) {
+    grid_wait();
     __shared__ float sh[kLossThreads / 32][4 + PPO_MAX_A];
+    __shared__ bool s_last;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     float acc[4 + PPO_MAX_A];
 #pragma unroll
@@ -515,19 +523,27 @@ __global__ void __launch_bounds__(kLossThreads) loss_kernel(
 #pragma unroll
         for (int w = 0; w < kLossThreads / 32; ++w) v += sh[w][threadIdx.x];
         partials[(size_t)blockIdx.x * 32 + threadIdx.x] = v;
+        __threadfence();
     }
-}
-
-// Single block: fixed-order sum of the per-block partials (fp64), added into the loss
-// scalars and the log-sigma gradient.
-__global__ void __launch_bounds__(32) loss_finalize_kernel(const float *__restrict__ partials, int nblocks, int A,
-                                                           const float *__restrict__ logsigma, float share,
-                                                           float ent_coef, float *__restrict__ loss_out,
-                                                           float *__restrict__ grad_logsigma) {
-    const int j = threadIdx.x;
+    // The block that finishes last adds the blocks' sums in their order (fp64) into the loss scalars and the log-sigma
+    // gradient; the counter wraps to zero for the next launch.  (A second launch for this took 5 us, most of it waiting.)
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    const int j = threadIdx.x, nblocks = (int)gridDim.x;
     if (j >= 4 + A) return;
     double s = 0.0;
-    for (int b = 0; b < nblocks; ++b) s += (double)partials[(size_t)b * 32 + j];
+    int b = 0;
+    for (; b + 8 <= nblocks; b += 8) {
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = __ldcg(partials + (size_t)(b + u) * 32 + j);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) s += (double)v[u];
+    }
+    for (; b < nblocks; ++b) s += (double)__ldcg(partials + (size_t)b * 32 + j);
     if (j == 0) loss_out[0] += (float)s;
     if (j == 1) loss_out[1] += (float)s;
     if (j == 2) loss_out[3] += (float)s;
@@ -551,13 +567,16 @@ extern "C" int ppo_loss_fwd_bwd(ppo_model *m, const ppo_minibatch *mb, int row0,
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const float *logsigma = m->master + m->tensors.back().off;
     const int blocks = ppo_cdiv(rows, kLossThreads);
-    loss_kernel<<<blocks, kLossThreads, 0, st>>>(rows, A, 1.f / (float)B_total, mean, value, logsigma,
+    if (!m->ticket_zeroed) {
+        PPO_CUDA_CHECK(cudaMemsetAsync(m->loss_ticket, 0, sizeof(unsigned int), st));
+        ppo_count_launches(1);
+        m->ticket_zeroed = true;
+    }
+    PPO_TRY(ppo_launch(loss_kernel, dim3(blocks), dim3(kLossThreads), 0, st, rows, A, 1.f / (float)B_total, mean, value, logsigma,
                                                  mb->action + (size_t)row0 * A, mb->logp_old + row0, mb->adv + row0,
-                                                 mb->ret + row0, clip, vf_coef, dmean, dvalue, m->loss_partials);
-    PPO_LAUNCH_CHECK();
-    loss_finalize_kernel<<<1, 32, 0, st>>>(m->loss_partials, blocks, A, logsigma, (float)rows / (float)B_total,
-                                           ent_coef, loss_out, m->grad + m->tensors.back().off);
-    PPO_LAUNCH_CHECK();
+                                                 mb->ret + row0, clip, vf_coef, dmean, dvalue, m->loss_partials,
+                                                 m->loss_ticket, (float)rows / (float)B_total, ent_coef, loss_out,
+                                                 m->grad + m->tensors.back().off));
     return PPO_OK;
 }
 
@@ -567,6 +586,7 @@ __global__ void __launch_bounds__(128) sample_kernel(int rows, int A, const floa
                                                      const float *__restrict__ logsigma,
                                                      const float *__restrict__ eps, float *__restrict__ action,
                                                      float *__restrict__ logp) {
+    grid_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= rows) return;
     float lp = 0.f;
@@ -582,9 +602,8 @@ extern "C" int ppo_policy_sample(const ppo_model *m, int rows, const float *mean
                                  float *logp, void *stream) {
     if (!m || !mean || !eps || !action || !logp || rows <= 0) return PPO_ERR_INVALID_ARG;
     if (!m->master) return PPO_ERR_STATE;
-    sample_kernel<<<ppo_cdiv(rows, 128), 128, 0, static_cast<cudaStream_t>(stream)>>>(
-        rows, m->d.A, mean, m->master + m->tensors.back().off, eps, action, logp);
-    PPO_LAUNCH_CHECK();
+    PPO_TRY(ppo_launch(sample_kernel, dim3(ppo_cdiv(rows, 128)), dim3(128), 0, static_cast<cudaStream_t>(stream), 
+        rows, m->d.A, mean, m->master + m->tensors.back().off, eps, action, logp));
     return PPO_OK;
 }
 

@@ -83,6 +83,14 @@ class Learner:
         obs = ppo.Minibatch(depth.data_ptr(), proprio.data_ptr(), None, None, None, None, None, None, n)
         if self.recurrent and (self.roll_h is None or self.roll_h.shape[1] != n):
             self.reset_rollout_state(n)
+        if n <= self.microbatch:  # all envs at once: the state is read and written where it is kept
+            if self.recurrent:
+                ppo.ppo_model_set_sequence(self.model, 1, n, self.roll_done, self.roll_h, self.roll_c)
+            ppo.ppo_encoder_fwd(self.model, obs, 0, n, self.mean, value)
+            ppo.ppo_policy_sample(self.model, n, self.mean, eps, action, logp)
+            if self.recurrent:
+                ppo.ppo_model_read_state(self.model, self.roll_h, self.roll_c)
+            return action, logp, value
         for r0 in range(0, n, self.microbatch):
             rows = min(self.microbatch, n - r0)
             if self.recurrent:  # a one-step sequence from the state the envs carry
@@ -106,9 +114,9 @@ class Learner:
             self.roll_c = torch.zeros_like(self.roll_h)
             self.roll_done = torch.zeros(n, dtype=torch.uint8, device=self.device)
         else:
-            keep = (done == 0).to(torch.float32).view(1, n, 1)
-            self.roll_h *= keep
-            self.roll_c *= keep
+            ended = (done != 0).view(1, n, 1)
+            self.roll_h.masked_fill_(ended, 0.0)
+            self.roll_c.masked_fill_(ended, 0.0)
 
     def act_into_buffer(self, t: int, depth: torch.Tensor, proprio: torch.Tensor, eps: torch.Tensor):
         """One rollout step without intermediate copies: the observation goes into slab row t, the policy reads
