@@ -152,14 +152,13 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
 }
 
 // ReLU gates of a group of 32 channels as one word: channel c sits at bit (c >> 1) + 16 (c & 1), i.e. pair j of
-// packed bf16 values owns bits j (its low half, channel 2j) and 16 + j (its high half, channel 2j + 1).  With the
-// halves non-negative (they come out of a ReLU), half + 0x7fff carries into its top bit exactly when it is not
-// zero, so a pair costs an add, a shift and a logic operation; and a pair's two gates come back out as the mask
-// of its two halves with a shift, an and, and a multiply.
+// packed bf16 values owns bits j (its low half, channel 2j) and 16 + j (its high half, channel 2j + 1).  A
+// pair costs one packed comparison and one logic operation; and its two gates come back out as the mask of its two
+// halves with a shift, an and, and a multiply.
 __host__ __device__ __forceinline__ int gate_bit_of_channel(int c) { return ((c & 31) >> 1) + 16 * (c & 1); }
 __device__ __forceinline__ uint32_t gate_bits_add(uint32_t gate, uint32_t pair, int j) {
-    const uint32_t t = pair + 0x7FFF7FFFu;
-    return gate | ((t >> (15 - j)) & (0x00010001u << j));
+    const uint32_t on = __hgt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&pair), __float2bfloat162_rn(0.f));
+    return gate | (on & (0x00010001u << j));
 }
 __device__ __forceinline__ uint32_t gate_pair_mask(uint32_t gate, int j) {
     return ((gate >> j) & 0x00010001u) * 0xFFFFu;

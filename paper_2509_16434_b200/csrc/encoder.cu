@@ -241,6 +241,9 @@ __global__ void __launch_bounds__(256) conv1_wgrad_mma_kernel(const __half *__re
     constexpr int TP = (2 * KW + 1 + 15) / 16 * 16, MB = TP / 16, C1 = NB * 8;
     constexpr int PX = 32;  // pixels per trip: one per lane, two K = 16 steps of the MMA
     constexpr int kXBytes = PX * TP * 2, kZBytes = PX * C1 * 2;
+    // 16-byte piece c of row r of a tile sits at piece c ^ f(r): rows of 32, 64 or 128 bytes would otherwise put the
+    // same piece of several rows into the same banks, on the way in as on the way out (ldmatrix reads a column of pieces)
+    auto swz = [](int r, int row_bytes) { return row_bytes == 128 ? r & 7 : (row_bytes == 64 ? (r >> 1) & 3 : (row_bytes == 32 ? (r >> 2) & 1 : 0)); };
     extern __shared__ __align__(16) uint8_t smw[];  // per warp: X tile [32 px][TP], dZ tile [32 px][C1]; later the reduction
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint8_t *xs = smw + (size_t)warp * (kXBytes + kZBytes), *zs = xs + kXBytes;
@@ -312,9 +315,12 @@ __global__ void __launch_bounds__(256) conv1_wgrad_mma_kernel(const __half *__re
     if (m0 < m_end) prefetch(m0);
     for (; m0 < m_end; m0 += PX) {
 #pragma unroll
-        for (int c = 0; c < TP / 8; ++c) *reinterpret_cast<uint4 *>(xs + lane * (TP * 2) + c * 16) = xreg[c];
+        for (int c = 0; c < TP / 8; ++c) *reinterpret_cast<uint4 *>(xs + lane * (TP * 2) + ((c ^ swz(lane, TP * 2)) * 16)) = xreg[c];
 #pragma unroll
-        for (int z = 0; z < ZP; ++z) reinterpret_cast<uint4 *>(zs)[lane + 32 * z] = zreg[z];
+        for (int z = 0; z < ZP; ++z) {
+            const int i = lane + 32 * z, zr = i / (C1 / 8), zc = i % (C1 / 8);
+            reinterpret_cast<uint4 *>(zs)[zr * (C1 / 8) + (zc ^ swz(zr, C1 * 2))] = zreg[z];
+        }
         __syncwarp();
         ow += d_ow;
         if (ow >= Wo) { ow -= Wo; ++oh; }
@@ -329,15 +335,15 @@ __global__ void __launch_bounds__(256) conv1_wgrad_mma_kernel(const __half *__re
 #pragma unroll
             for (int i = 0; i < MB; ++i) {
                 // matrices: (taps 16i..+7, px 0-7), (taps 16i+8.., px 0-7), (taps 16i.., px 8-15), (taps 16i+8.., px 8-15)
-                const uint32_t addr =
-                    xs_a + (uint32_t)((16 * ks + r + (mi >= 2 ? 8 : 0)) * (TP * 2) + (16 * i + (mi & 1) * 8) * 2);
+                const int row = 16 * ks + r + (mi >= 2 ? 8 : 0);
+                const uint32_t addr = xs_a + (uint32_t)(row * (TP * 2) + ((2 * i + (mi & 1)) ^ swz(row, TP * 2)) * 16);
                 ldmatrix_x4_trans(addr, af[i][0], af[i][1], af[i][2], af[i][3]);
             }
 #pragma unroll
             for (int j = 0; j < NB; j += 2) {
                 // matrices: (px 0-7, co 8j..), (px 8-15, co 8j..), (px 0-7, co 8j+8..), (px 8-15, co 8j+8..)
-                const uint32_t addr =
-                    zs_a + (uint32_t)((16 * ks + r + (mi & 1) * 8) * (C1 * 2) + (8 * j + (mi >> 1) * 8) * 2);
+                const int row = 16 * ks + r + (mi & 1) * 8;
+                const uint32_t addr = zs_a + (uint32_t)(row * (C1 * 2) + ((j + (mi >> 1)) ^ swz(row, C1 * 2)) * 16);
                 uint32_t b0, b1, b2, b3;
                 ldmatrix_x4_trans(addr, b0, b1, b2, b3);
 #pragma unroll
@@ -412,36 +418,55 @@ int relu_bits(const bf16 *act, uint32_t *bits, long long M, int C, cudaStream_t 
 }
 
 
-// h0[b] = [mean over pixels of act[b][px][c], proprio[b]] as bf16.  One warp per row b; a lane
-// owns 8 channels at a time so that every pixel is read with 128-bit loads.
+// h0[b] = [mean over pixels of act[b][px][c], proprio[b]] as bf16.  One thread per row and 8 channels, so that narrow
+// layers fill their warps too and every pixel is read with 128-bit loads; the pixels are added in order, the loads of
+// sixteen in flight (one at a time, a warp waits for memory npx times over).  The threads behind those copy the
+// proprioception.
 __global__ void __launch_bounds__(256) pool_concat_kernel(const bf16 *__restrict__ act,
                                                           const float *__restrict__ proprio, bf16 *__restrict__ h0,
                                                           int rows, int npx, int C, int P) {
     grid_wait();
-    const int b = blockIdx.x * 8 + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (b >= rows) return;
-    const float inv = 1.f / (float)npx;
-    const bf16 *base = act + (size_t)b * npx * C;
-    bf16 *out = h0 + (size_t)b * (C + P);
-    for (int c8 = lane * 8; c8 < C; c8 += 256) {
+    const int c8n = C >> 3;
+    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < (long long)rows * c8n) {
+        const long long b = i / c8n;
+        const int c8 = (int)(i - b * c8n) * 8;
+        const float inv = 1.f / (float)npx;
+        const bf16 *base = act + b * npx * C + c8;
         float s[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) s[i] = 0.f;
-        for (int px = 0; px < npx; ++px) {
-            const uint4 raw = *reinterpret_cast<const uint4 *>(base + (size_t)px * C + c8);
+        for (int k = 0; k < 8; ++k) s[k] = 0.f;
+        auto add = [&](const uint4 &raw) {
             const __nv_bfloat162 *p2 = reinterpret_cast<const __nv_bfloat162 *>(&raw);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float2 f = __bfloat1622float2(p2[i]);
-                s[2 * i] += f.x;
-                s[2 * i + 1] += f.y;
+            for (int k = 0; k < 4; ++k) {
+                const float2 f = __bfloat1622float2(p2[k]);
+                s[2 * k] += f.x;
+                s[2 * k + 1] += f.y;
             }
-        }
+        };
+        int px = 0;
+        for (; px + 16 <= npx; px += 16) {
+            uint4 raw[16];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) out[c8 + i] = __float2bfloat16_rn(s[i] * inv);
+            for (int u = 0; u < 16; ++u) raw[u] = __ldcs(reinterpret_cast<const uint4 *>(base + (size_t)(px + u) * C));
+#pragma unroll
+            for (int u = 0; u < 16; ++u) add(raw[u]);
+        }
+        for (; px < npx; ++px) add(__ldcs(reinterpret_cast<const uint4 *>(base + (size_t)px * C)));
+        uint4 o;
+        o.x = pack_bf16x2(s[0] * inv, s[1] * inv);
+        o.y = pack_bf16x2(s[2] * inv, s[3] * inv);
+        o.z = pack_bf16x2(s[4] * inv, s[5] * inv);
+        o.w = pack_bf16x2(s[6] * inv, s[7] * inv);
+        *reinterpret_cast<uint4 *>(h0 + b * (C + P) + c8) = o;  // C + P is a multiple of 8
+        return;
     }
-    for (int j = lane; j < P; j += 32) out[C + j] = __float2bfloat16_rn(proprio[(size_t)b * P + j]);
+    i -= (long long)rows * c8n;
+    if (i >= (long long)rows * P) return;
+    const long long b = i / P;
+    const int j = (int)(i - b * P);
+    h0[b * (C + P) + C + j] = __float2bfloat16_rn(proprio[i]);
 }
 
 // dact[b][px][c] = dh0[b][c] / npx where act > 0, else 0; 8 channels per thread.
@@ -1106,7 +1131,7 @@ extern "C" int ppo_encoder_fwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
         PPO_TRY(ppo_launch(concat_proprio_kernel, dim3(ppo_cdiv((long long)rows * d.P, 256)), dim3(256), 0, st, mb->proprio + (size_t)row0 * d.P, m->h[0],
                                                                                   rows, d.embed, d.P, m->hw[0]));
     } else {
-        PPO_TRY(ppo_launch(pool_concat_kernel, dim3(ppo_cdiv(rows, 8)), dim3(256), 0, st, m->act[m->L], mb->proprio + (size_t)row0 * d.P, m->h[0], rows,
+        PPO_TRY(ppo_launch(pool_concat_kernel, dim3(ppo_cdiv((long long)rows * (m->Cs[m->L] / 8 + d.P), 256)), dim3(256), 0, st, m->act[m->L], mb->proprio + (size_t)row0 * d.P, m->h[0], rows,
                                                               m->Hs[m->L] * m->Ws[m->L], m->Cs[m->L], d.P));
     }
     if (d.n_lstm > 0) PPO_TRY(lstm_forward(m, rows, st));
