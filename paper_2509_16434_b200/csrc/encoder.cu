@@ -272,45 +272,50 @@ __global__ void __launch_bounds__(256) conv1_wgrad_mma_kernel(const __half *__re
     constexpr int ZP = PX * C1 / 8 / 32;       // 16-byte pieces of the gradient tile per lane
     uint4 xreg[TP / 8], zreg[ZP];
     // Loads of the tile that starts at pixel mt into registers; they are issued one trip ahead, so that their
-    // latency overlaps the previous tile's MMAs.
+    // latency overlaps the previous tile's MMAs.  The kernel is bound by its instructions as much as by HBM: a pair outside
+    // the frame is a predicated load that leaves its zero, a full tile takes its gradient rows without tests.
     const int Wh = Wi >> 1;  // 32-bit words per frame row
+    const uint32_t *const frames = reinterpret_cast<const uint32_t *>(depth);
     auto prefetch = [&](long long mt) {
         const bool live = mt + lane < m_end;
-        // every load is issued, from a clamped address where its pixel pair lies outside the frame, before the first
-        // conversion: the loads of a trip are then in flight together
-        const uint32_t *img = reinterpret_cast<const uint32_t *>(depth) + (live ? b : 0) * Hi * Wh;
-        uint32_t wv[TP / 2], raw[KW];
-        const int pw0 = ow - (P + ODD) / 2;
-        uint32_t okm = 0;
+        const int pw0 = ow - (P + ODD) / 2, ih0 = 2 * oh - P;
+        const uint32_t *row = frames + ((b * Hi + ih0) * Wh + pw0);
+        uint32_t raw[KW];
+        bool cok[NP];
+#pragma unroll
+        for (int q = 0; q < NP; ++q) cok[q] = live && (unsigned)(pw0 + q) < (unsigned)Wh;
 #pragma unroll
         for (int kh = 0; kh < KS; ++kh) {
-            const int ih = 2 * oh + kh - P;
-            const bool rok = live && (unsigned)ih < (unsigned)Hi;
-            const uint32_t *row = img + (rok ? ih : 0) * Wh;
+            const bool rok = (unsigned)(ih0 + kh) < (unsigned)Hi;
 #pragma unroll
             for (int q = 0; q < NP; ++q) {
-                const int pw = pw0 + q;
-                const bool ok = rok && (unsigned)pw < (unsigned)Wh;
-                raw[kh * NP + q] = __ldg(row + (ok ? pw : 0));
-                okm |= (ok ? 1u : 0u) << (kh * NP + q);
+                raw[kh * NP + q] = 0u;
+                if (rok && cok[q]) raw[kh * NP + q] = __ldg(row + q);
+            }
+            row += Wh;
+        }
+        if (mt + PX <= m_end) {
+#pragma unroll
+            for (int z = 0; z < ZP; ++z) zreg[z] = __ldcs(reinterpret_cast<const uint4 *>(dZ + mt * C1) + lane + 32 * z);
+        } else {
+#pragma unroll
+            for (int z = 0; z < ZP; ++z) {
+                const int i = lane + 32 * z;
+                zreg[z] = make_uint4(0, 0, 0, 0);
+                if (mt + i / (C1 / 8) < m_end) zreg[z] = __ldcs(reinterpret_cast<const uint4 *>(dZ + mt * C1) + i);
             }
         }
+        uint32_t wv[TP / 2];
 #pragma unroll
         for (int k = 0; k < TP / 2; ++k) wv[k] = 0u;
 #pragma unroll
         for (int k = 0; k < KW; ++k) {
             const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&raw[k]));
-            wv[k] = (okm >> k) & 1u ? pack_bf16x2(f.x, f.y) : 0u;
+            wv[k] = pack_bf16x2(f.x, f.y);
         }
         if (live) wv[KW] = 0x00003F80u;  // (1.0, 0) as bf16: the bias-gradient column
 #pragma unroll
         for (int c = 0; c < TP / 8; ++c) xreg[c] = make_uint4(wv[4 * c], wv[4 * c + 1], wv[4 * c + 2], wv[4 * c + 3]);
-#pragma unroll
-        for (int z = 0; z < ZP; ++z) {
-            const int i = lane + 32 * z;
-            zreg[z] = make_uint4(0, 0, 0, 0);
-            if (mt + i / (C1 / 8) < m_end) zreg[z] = __ldcs(reinterpret_cast<const uint4 *>(dZ + mt * C1) + i);
-        }
     };
     if (m0 < m_end) prefetch(m0);
     for (; m0 < m_end; m0 += PX) {

@@ -180,6 +180,7 @@ struct KArgs {
     RowGrid grid;
     int s_mul, s_oy, s_ox;  // source pixel of tap t: (y * s_mul + s_oy + dy[t], x * s_mul + s_ox + dx[t])
     int CB, row_bytes;      // channels per box (64, 32 or 16) and bytes of a shared-memory row
+    uint32_t a_bytes;       // room for a tile's A rows (the MMA reads 128; what lies behind belongs to rows nobody stores)
     int kchunks;            // boxes along the channels of one tap
     int w_tap;              // elements between taps in a weight row
     int G, nbmax;           // sub-blocks per stage; most A boxes a tile has
@@ -226,7 +227,7 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int BN = a.BN, S = a.stages, G = a.G;
     const uint32_t rb = (uint32_t)a.row_bytes;
-    const uint32_t a_bytes = 128u * rb, b_bytes = (uint32_t)BN * rb;
+    const uint32_t a_bytes = a.a_bytes, b_bytes = (uint32_t)BN * rb;
     const uint32_t sub_bytes = a_bytes + (a.wres ? 0u : b_bytes);
     const uint32_t stage_bytes = (uint32_t)G * sub_bytes;
     const uint32_t res_bytes = a.wres ? (uint32_t)(a.wtaps * a.kchunks) * b_bytes : 0u;
@@ -960,6 +961,22 @@ static int flat_bn(int N, long long rows) {
     return bn;
 }
 
+// Grid of a flat GEMM's rows: tiles of 128, halved (down to 32) while the tiles would leave more than half of the SMs
+// without work.  A CTA's time is the length of its reduction (copies and one MMA per 16 of K, nothing amortises them), so
+// rows are better spread over idle SMs.
+static bool make_flat_grid(RowGrid &g, long long rows, int tiles_n, int row_bytes) {
+    if (!make_grid(g, (int)rows, 1, 1, row_bytes)) return false;
+    int Wt = g.Wt;
+    while (Wt % 2 == 0 && Wt / 2 >= 32 && (Wt / 2) * row_bytes % 1024 == 0 && 2ll * g.xsegs * tiles_n <= ppo_num_sms()) {
+        Wt /= 2;
+        g.Wt = Wt;
+        g.xsegs = (int)((rows + Wt - 1) / Wt);
+        g.tiles = g.xsegs;
+        g.arows = Wt;
+    }
+    return true;
+}
+
 int ensure_smem_attrs() {
     static bool attr_set[64] = {false};
     int dev = 0;
@@ -1010,14 +1027,17 @@ int launch_kmajor(KArgs &a, cudaStream_t st) {
     // issue rate.  Wide tiles run at the tensor rate with one CTA and keep the SM to themselves.
     // A GEMM of a few row tiles gives a CTA one or two tiles: nothing amortises the copy latency, so such a CTA takes the
     // SM alone, with stages of up to 96 KB (fewer, larger hand-overs), and the narrow-tile rule below does not apply.
-    const bool small_m = a.grid.tiles <= 4 && (a.ncls == 1 || a.cls_orows != 0);
+    const bool flat = a.grid.Hr == 1 && a.grid.Nimg == 1;
+    const bool small_m = (a.grid.tiles <= 4 || (flat && total <= ppo_num_sms())) && (a.ncls == 1 || a.cls_orows != 0);
     const bool two = a.BN <= 128 && !small_m;
     a.tmem_cap = two ? 256 : 512;
     a.nepi = (!two && a.mode == EPI_DGRAD && a.mask_bits) ? 16 : 8;
     const size_t fixed = sizeof(PipeK) + (size_t)a.nepi * 2048 + 1024;  // pipeline state, epilogue staging, alignment slack
     const size_t cta_max = two ? kSmemMax / 2 : kSmemMax;
-    if (a.wres && res + fixed + 3 * (size_t)128 * a.row_bytes + 1024 > cta_max) a.wres = 0;
-    const size_t sub = (size_t)128 * a.row_bytes + (a.wres ? 0 : b_bytes);
+    // (the rows an MMA reads beyond a_bytes of the last sub-block lie in the pipeline state and staging, at least 16 KB)
+    a.a_bytes = flat ? ((uint32_t)(a.grid.arows * a.row_bytes) + 1023u) & ~1023u : 128u * (uint32_t)a.row_bytes;
+    if (a.wres && res + fixed + 3 * (size_t)a.a_bytes + 1024 > cta_max) a.wres = 0;
+    const size_t sub = (size_t)a.a_bytes + (a.wres ? 0 : b_bytes);
     const size_t budget = cta_max - 1024 - fixed - (a.wres ? res : 0);
     int G = (int)(((small_m ? 96 : 48) * 1024) / sub);  // sub-blocks per stage: fewer barrier round trips per byte
     G = G < 1 ? 1 : (G > 8 ? 8 : G);
@@ -1053,14 +1073,14 @@ int tma_gemm_fwd(const ConvGeom &g, const bf16 *X, const bf16 *W, const FwdEpilo
     a.kchunks = (g.Ci + CB - 1) / CB;
     a.w_tap = g.Ci;
     a.wtaps = g.taps();
+    a.N = g.Co;
+    a.BN = flat && e.out ? flat_bn(g.Co, g.B) : pick_bn(g.Co);
     // a fully connected layer is one image with a single row of B pixels
-    const bool ok = flat ? make_grid(a.grid, g.B, 1, 1, a.row_bytes) : make_grid(a.grid, g.Wo, g.Ho, g.B, a.row_bytes);
+    const bool ok = flat ? make_flat_grid(a.grid, g.B, (a.N + a.BN - 1) / a.BN, a.row_bytes) : make_grid(a.grid, g.Wo, g.Ho, g.B, a.row_bytes);
     if (!ok) return PPO_ERR_UNSUPPORTED;
     int s = flat ? make_act_maps(a.mapA, X, g.Ci, g.Ci, g.B, 1, 1, a.grid, CB, 1)
                  : make_act_maps(a.mapA, X, g.Ci, g.Ci, g.Wi, g.Hi, g.B, a.grid, CB, 2);
     if (s != PPO_OK) return s;
-    a.N = g.Co;
-    a.BN = flat && e.out ? flat_bn(g.Co, g.B) : pick_bn(g.Co);
     {
         const long long dims[2] = {g.K(), g.Co};
         const int box[2] = {CB, a.BN}, es[2] = {1, 1};
@@ -1131,7 +1151,10 @@ int tma_gemm_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, i
     a.kchunks = (g.Co + CB - 1) / CB;
     a.w_tap = wt_ld;
     const int Hr = flat ? 1 : (g.Hi + 1) / 2, Wr = flat ? g.B : (g.Wi + 1) / 2;
-    if (!make_grid(a.grid, Wr, Hr, flat ? 1 : g.B, a.row_bytes)) return PPO_ERR_UNSUPPORTED;
+    const int flat_n = flat ? flat_bn(g.Ci, g.B) : 0;
+    if (!(flat && e.ksplit <= 1 ? make_flat_grid(a.grid, g.B, (g.Ci + flat_n - 1) / flat_n, a.row_bytes)
+                                : make_grid(a.grid, Wr, Hr, flat ? 1 : g.B, a.row_bytes)))
+        return PPO_ERR_UNSUPPORTED;
     int s = flat ? make_act_maps(a.mapA, dY, g.Co, ldy, g.B, 1, 1, a.grid, CB, 1)
                  : make_act_maps(a.mapA, dY, g.Co, ldy, g.Wo, g.Ho, g.B, a.grid, CB, 1);
     if (s != PPO_OK) return s;
@@ -1185,7 +1208,7 @@ int tma_gemm_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, i
     }
     if (flat) {
         a.N = g.Ci;
-        a.BN = flat_bn(g.Ci, g.B);
+        a.BN = flat_n;
         a.wtaps = 1;
         const long long dims[2] = {wt_ld, g.Ci};
         const int box[2] = {CB, a.BN}, es[2] = {1, 1};
