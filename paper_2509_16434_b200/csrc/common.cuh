@@ -88,6 +88,8 @@ struct ppo_model {
     bf16 *lstm_dg;                   // gradient w.r.t. the gate pre-activations [mb][4H]
     float *lstm_dtop;                // gradient w.r.t. a layer's outputs [mb][H] (from the FC layers or the layer above)
     float *lstm_dhc, *lstm_dcc;      // gradients carried to the previous step [mb][H]
+    unsigned int *lstm_counters;     // of the persistent time loop (lstm.cuh)
+    bool counters_zeroed;
     size_t arena, nparams;
     // bound arrays
     float *master, *grad, *adam_m, *adam_v;

@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv1_tc_kernel(const __grid_cons
     const uint32_t raw_off = stg_off + (uint32_t)kEpiWarps * 2u * kStgBytes;
     Pipe *pipe = reinterpret_cast<Pipe *>(smem + raw_off + (size_t)kRaw * a.raw_bytes);
     volatile int *abort_flag = &pipe->abort_flag;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const uint32_t acc_cols = tmem_cols_for(T * N);                // T accumulators side by side
     const int nacc_log = acc_cols * 4 <= 512 ? 2 : 1, nacc = 1 << nacc_log;
     const uint32_t ncols = acc_cols * nacc;
@@ -302,12 +302,12 @@ __global__ void __launch_bounds__(kThreads, 1) conv1_tc_kernel(const __grid_cons
         uint32_t ph = 0;
         for (int li = 0; li < ns && ok; ++li) {
             const int acc = li & (nacc - 1);
-            ok = mbar_wait(&pipe->tempty[acc], ((li >> nacc_log) & 1) ^ 1, abort_flag, a.status);
+            ok = mbar_wait_warp(&pipe->tempty[acc], ((li >> nacc_log) & 1) ^ 1, abort_flag, a.status);
             if (!ok) break;
-            ok = mbar_wait(&pipe->full[s], ph, abort_flag, a.status);
+            ok = mbar_wait_warp(&pipe->full[s], ph, abort_flag, a.status);
             if (!ok) break;
             tc_fence_after();
-            if (lane == 0) {
+            if (elect_one()) {
                 uint32_t la = (uint32_t)dA0 + (uint32_t)s * (kStageBytes >> 4);
                 uint32_t td = tmem_base + acc * acc_cols;
 #pragma unroll

@@ -176,7 +176,7 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
     const uint32_t stg_off = (a.slots_bytes + w_bytes + 1023u) & ~1023u;
     Pipe *pipe = reinterpret_cast<Pipe *>(smem + stg_off + (size_t)(a.nbuf * a.neg) * a.stg_bytes);
     volatile int *abort_flag = &pipe->abort_flag;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int nacc = a.nacc;
     const uint32_t ncols = (uint32_t)(a.acc_cols * nacc);
 
@@ -213,11 +213,11 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
     const int t0 = bid * q + (bid < rem ? bid : rem), nt = q + (bid < rem ? 1 : 0);
 
     if (warp == 0) {
-        if (lane == 0) {
-            mbar_arrive_expect_tx(&pipe->wfull, w_bytes);
+        {
+            if (elect_one()) mbar_arrive_expect_tx(&pipe->wfull, w_bytes);
             for (int c = 0; c < a.nchunks; ++c)
                 for (int i = 0; i < a.nwl; ++i)
-                    tma_load_2d(w_base + (uint32_t)c * a.w_chunk + a.wl[i].off, &a.mapW, &pipe->wfull, a.wl[i].k0 + c * a.CB, 0);
+                    if (elect_one()) tma_load_2d(w_base + (uint32_t)c * a.w_chunk + a.wl[i].off, &a.mapW, &pipe->wfull, a.wl[i].k0 + c * a.CB, 0);
             TileAt t;
             t.init(a, t0);
             SlotQueue sq;
@@ -230,13 +230,16 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
                     const int p = a.nplanes == 4 ? 3 - i : 0, s = sq.pop();
                     const Plane &pl = a.planes[p];
                     used |= (uint32_t)s << (4 * i);
-                    ok = mbar_wait(&pipe->empty[s], (~phase >> s) & 1u, abort_flag, a.status);
+                    ok = mbar_wait_warp(&pipe->empty[s], (~phase >> s) & 1u, abort_flag, a.status);
                     if (!ok) break;
                     phase ^= 1u << s;
                     armed |= 1u << s;
-                    mbar_arrive_expect_tx(&pipe->full[s], pl.bytes);
-                    tma_load_4d(smem_base + (uint32_t)s * a.slot_bytes, &a.mapA[p], &pipe->full[s], a.nplanes == 4 ? 0 : i * a.CB,
-                                t.x + pl.ox, t.y + pl.oy, t.n);
+                    if (elect_one()) {
+                        mbar_arrive_expect_tx(&pipe->full[s], pl.bytes);
+                        tma_load_4d(smem_base + (uint32_t)s * a.slot_bytes, &a.mapA[p], &pipe->full[s], a.nplanes == 4 ? 0 : i * a.CB,
+                                    t.x + pl.ox, t.y + pl.oy, t.n);
+                    }
+                    __syncwarp();
                 }
                 if (a.nplanes == 4) used = (used >> 8) | (used << 8 & 0xFF00u);  // planes 01 and 00 are done first
                 for (int i = 0; i < a.nloads; ++i) sq.push((int)(used >> (4 * i)) & 15);
@@ -265,7 +268,7 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
         sq.init(a.slots);
         int acc = 0;
         uint32_t phase = 0, aph = 1u;  // parities of the slots; parity that says the accumulator has been drained
-        bool ok = mbar_wait(&pipe->wfull, 0, abort_flag, a.status);
+        bool ok = mbar_wait_warp(&pipe->wfull, 0, abort_flag, a.status);
         auto taps = [&](int o, uint32_t la0, uint32_t lb0, uint32_t tmem_d, uint32_t accum) {
             const Op &op = a.ops[o];
             const uint32_t la = la0 + op.a16, lb = lb0 + op.b16, td = tmem_d + op.dcol, id = op.idesc;
@@ -274,7 +277,7 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
             for (int k = 1; k < KS; ++k) umma_bf16_lh(td, la + 2 * k, d_hi, lb + 2 * k, d_hi, id, 1u);
         };
         for (int li = 0; li < nt && ok; ++li) {
-            ok = mbar_wait(&pipe->tempty[acc], aph, abort_flag, a.status);
+            ok = mbar_wait_warp(&pipe->tempty[acc], aph, abort_flag, a.status);
             if (!ok) break;
             tc_fence_after();
             const uint32_t tmem_d = tmem_base + (uint32_t)(acc * a.acc_cols);
@@ -292,11 +295,11 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
                     constexpr int kLoad[9] = {0, 1, 0, 2, 3, 2, 0, 1, 0};  // load that brings the tap's plane
                     const int i = kLoad[t];
                     if (t < 2 || t == 3 || t == 4) {
-                        ok = mbar_wait(&pipe->full[sl[i]], (phase >> sl[i]) & 1u, abort_flag, a.status);
+                        ok = mbar_wait_warp(&pipe->full[sl[i]], (phase >> sl[i]) & 1u, abort_flag, a.status);
                         if (!ok) break;
                         tc_fence_after();
                     }
-                    if (lane == 0) {
+                    if (elect_one()) {
                         taps(t, la[i], w_lo0, tmem_d, t > 0 ? 1u : 0u);
                         if (t == 5) {
                             umma_commit(&pipe->empty[sl[2]]);
@@ -306,7 +309,7 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
                     __syncwarp();
                 }
                 if (!ok) break;
-                if (lane == 0) {
+                if (elect_one()) {
                     umma_commit(&pipe->empty[sl[0]]);
                     umma_commit(&pipe->empty[sl[1]]);
                 }
@@ -320,13 +323,13 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
                 for (int c = 0; c < a.nchunks; ++c) {
                     const int s = sq.pop();
                     used |= (uint32_t)s << (4 * c);
-                    ok = mbar_wait(&pipe->full[s], (phase >> s) & 1u, abort_flag, a.status);
+                    ok = mbar_wait_warp(&pipe->full[s], (phase >> s) & 1u, abort_flag, a.status);
                     if (!ok) break;
                     phase ^= 1u << s;
                 }
                 if (!ok) break;
                 tc_fence_after();
-                if (lane == 0) {
+                if (elect_one()) {
 #pragma unroll
                     for (int o = 0; o < 4; ++o) {
                         uint32_t lb = w_lo0;
@@ -339,7 +342,7 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
                 }
                 for (int c = 0; c < a.nchunks; ++c) sq.push((int)(used >> (4 * c)) & 15);
             }
-            if (lane == 0) umma_commit(&pipe->tfull[acc]);
+            if (elect_one()) umma_commit(&pipe->tfull[acc]);
             __syncwarp();
             if (++acc == nacc) { acc = 0; aph ^= 1u; }
         }

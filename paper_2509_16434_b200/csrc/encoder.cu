@@ -5,6 +5,7 @@
 #include "common.cuh"
 #include "launch.cuh"
 #include "gemm.cuh"
+#include "lstm.cuh"
 
 // -------------------------------------------------------------------- conv1 ----
 
@@ -757,8 +758,6 @@ __global__ void __launch_bounds__(256) ln_bwd_kernel(bf16 *__restrict__ d, const
 
 // ------------------------------------------------------------ recurrent trunk ----
 
-__device__ __forceinline__ float sigmoidf_(float x) { return 1.f / (1.f + __expf(-x)); }
-
 // State the first step of a sequence starts from: h_prev[0] = bf16(h_init), c_prev[0] = c_init (rows of one step, Be x H).
 __global__ void __launch_bounds__(256) lstm_init_kernel(const float *__restrict__ h_init, const float *__restrict__ c_init,
                                                         bf16 *__restrict__ hprev, float *__restrict__ cprev, int n) {
@@ -784,12 +783,9 @@ __global__ void __launch_bounds__(256) lstm_cell_fwd_kernel(const float *__restr
     if (i >= Be * H) return;
     const int e = i / H, j = i - e * H;
     const size_t g0 = (size_t)e * 4 * H + j;
-    const float gi = sigmoidf_(xg[g0] + hg[g0] + bias[j]);
-    const float gf = sigmoidf_(xg[g0 + H] + hg[g0 + H] + bias[H + j]);
-    const float gg = tanhf(xg[g0 + 2 * H] + hg[g0 + 2 * H] + bias[2 * H + j]);
-    const float go = sigmoidf_(xg[g0 + 3 * H] + hg[g0 + 3 * H] + bias[3 * H + j]);
-    const float cv = gf * cprev[i] + gi * gg;
-    const float hv = go * tanhf(cv);
+    float gi, gf, gg, go, cv, hv;
+    lstm_cell(xg[g0] + hg[g0] + bias[j], xg[g0 + H] + hg[g0 + H] + bias[H + j], xg[g0 + 2 * H] + hg[g0 + 2 * H] + bias[2 * H + j],
+              xg[g0 + 3 * H] + hg[g0 + 3 * H] + bias[3 * H + j], cprev[i], gi, gf, gg, go, cv, hv);
     gates[g0] = gi;
     gates[g0 + H] = gf;
     gates[g0 + 2 * H] = gg;
@@ -823,15 +819,14 @@ __global__ void __launch_bounds__(256) lstm_cell_bwd_kernel(const float *__restr
     float dhn = 0.f;
     if (carry)
         for (int s = 0; s < nsplit; ++s) dhn += dhc[(size_t)s * Be * H + i];
-    const float dh = dtop[i] + dhn;
-    const float gi = gates[g0], gf = gates[g0 + H], gg = gates[g0 + 2 * H], go = gates[g0 + 3 * H];
-    const float tc = tanhf(c[i]);
-    const float dc = (carry ? dcc[i] : 0.f) + dh * go * (1.f - tc * tc);
-    dg[g0] = __float2bfloat16_rn(dc * gg * gi * (1.f - gi));
-    dg[g0 + H] = __float2bfloat16_rn(dc * cprev[i] * gf * (1.f - gf));
-    dg[g0 + 2 * H] = __float2bfloat16_rn(dc * gi * (1.f - gg * gg));
-    dg[g0 + 3 * H] = __float2bfloat16_rn(dh * tc * go * (1.f - go));
-    dcc[i] = dc * gf;
+    float di, df, dgg, dgo, dc_out;
+    lstm_cell_back(dtop[i] + dhn, carry ? dcc[i] : 0.f, gates[g0], gates[g0 + H], gates[g0 + 2 * H], gates[g0 + 3 * H], c[i], cprev[i], di,
+                   df, dgg, dgo, dc_out);
+    dg[g0] = __float2bfloat16_rn(di);
+    dg[g0 + H] = __float2bfloat16_rn(df);
+    dg[g0 + 2 * H] = __float2bfloat16_rn(dgg);
+    dg[g0 + 3 * H] = __float2bfloat16_rn(dgo);
+    dcc[i] = dc_out;
 }
 
 // ------------------------------------------------------------ orchestration ----
@@ -876,7 +871,7 @@ static int recorded(ppo_model *m, const PlanKey &key, cudaStream_t st, F &&make)
     return s;
 }
 
-enum { OP_FWD = 1, OP_DGRAD, OP_WGRAD };
+enum { OP_FWD = 1, OP_DGRAD, OP_WGRAD, OP_LSTM_FWD, OP_LSTM_BWD };
 
 static PlanKey plan_key(int op, const ConvGeom &g) {
     PlanKey k;
@@ -1009,6 +1004,33 @@ static int gemm_nt_f32(ppo_model *m, int rows, int N, int K, const bf16 *A, int 
     return run_dgrad(m, g, A, lda, Wn, K, 0, e, st);
 }
 
+static LstmSteps lstm_steps(const ppo_model *m, int l) {
+    LstmSteps p;
+    p.T = m->seq_T; p.Be = m->seq_Be; p.H = m->d.lstm_h;
+    p.done = m->seq_done;
+    p.gates = m->lstm_gates[l];
+    p.c = m->lstm_c[l];
+    p.cprev = m->lstm_c[l] + (size_t)m->mbmax * m->d.lstm_h;
+    p.h = m->lstm_hs[l];
+    p.hprev = m->lstm_hprev[l];
+    p.counters = m->lstm_counters;
+    return p;
+}
+
+// Runs a layer's time loop as one launch where it fits (remembered like the GEMMs' launches).
+template <typename F>
+static int lstm_persistent(ppo_model *m, int op, int l, cudaStream_t st, F &&make) {
+    if (!m->counters_zeroed) {
+        PPO_CUDA_CHECK(cudaMemsetAsync(m->lstm_counters, 0, kLstmCounters * 128, st));
+        ppo_count_launches(1);
+        m->counters_zeroed = true;
+    }
+    PlanKey k = plan_key(op, fc_geom(m->seq_Be, m->seq_T, l));
+    const void *p[] = {m->seq_done, m->seq_h_init, m->seq_c_init};
+    memcpy(k.p, p, sizeof(p));
+    return recorded(m, k, st, make);
+}
+
 // Forward of the recurrent trunk over the announced sequence (rows = T * Be, time-major): per layer one GEMM for
 // W_x x of all rows, then per step the GEMM W_h h_prev and the element-wise cell.
 static int lstm_forward(ppo_model *m, int rows, cudaStream_t st) {
@@ -1020,6 +1042,12 @@ static int lstm_forward(ppo_model *m, int rows, cudaStream_t st) {
         const bf16 *X = l == 0 ? m->h[0] : m->lstm_hs[l - 1];
         float *cprev = m->lstm_c[l] + (size_t)m->mbmax * H;
         PPO_TRY(gemm_nt_f32(m, rows, 4 * H, in, X, in, m->shadow + m->tensors[ti].off, m->lstm_xg, st));
+        const int one = lstm_persistent(m, OP_LSTM_FWD, l, st, [&]() -> int {
+            return lstm_fwd_steps(lstm_steps(m, l), m->shadow + m->tensors[ti + 1].off, m->lstm_xg, m->master + m->tensors[ti + 2].off,
+                                  m->seq_h_init + (size_t)l * Be * H, m->seq_c_init + (size_t)l * Be * H, ppo_device_status_ptr(), st);
+        });
+        if (one == PPO_OK) continue;
+        if (one != PPO_ERR_UNSUPPORTED) return one;
         PPO_TRY(ppo_launch(lstm_init_kernel, dim3(ppo_cdiv((long long)Be * H, 256)), dim3(256), 0, st, m->seq_h_init + (size_t)l * Be * H,
                                                                           m->seq_c_init + (size_t)l * Be * H,
                                                                           m->lstm_hprev[l], cprev, Be * H));
@@ -1049,7 +1077,13 @@ static int lstm_backward(ppo_model *m, int rows, cudaStream_t st) {
         // dg W_h reduces over 4H columns into few output tiles: with few envs the reduction is cut into four slabs that
         // as many CTAs work on, and the next cell kernel adds their partial products (dhc holds rows * H floats)
         int nsplit = (T >= 4 && Be <= 512) ? 4 : 1;
-        for (int t = T - 1; t >= 0; --t) {
+        int one = PPO_ERR_UNSUPPORTED;
+        if (nsplit == 4 || T == 1)
+            one = lstm_persistent(m, OP_LSTM_BWD, l, st, [&]() -> int {
+                return lstm_bwd_steps(lstm_steps(m, l), m->wT + m->wT_off[ti + 1], m->lstm_dtop, m->lstm_dg, m->lstm_dhc, ppo_device_status_ptr(), st);
+            });
+        if (one != PPO_OK && one != PPO_ERR_UNSUPPORTED) return one;
+        for (int t = T - 1; t >= 0 && one != PPO_OK; --t) {
             const size_t r0 = (size_t)t * Be;
             PPO_TRY(ppo_launch(lstm_cell_bwd_kernel, dim3(ppo_cdiv((long long)Be * H, 256)), dim3(256), 0, st, 
                 m->lstm_dtop + r0 * H, m->lstm_dhc, m->lstm_dcc, m->seq_done + r0, m->lstm_gates[l] + r0 * 4 * H,

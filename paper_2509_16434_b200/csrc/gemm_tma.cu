@@ -170,7 +170,6 @@ enum { EPI_FWD = 0, EPI_HEAD = 1, EPI_DGRAD = 2 };
 constexpr int kEpiWarps = 16;                     // at most: two or four warps per TMEM lane quarter share out the column groups
 constexpr int kKThreads = (2 + kEpiWarps) * 32;   // warp 0: TMA producer, warp 1: MMA issue and TMEM owner
 constexpr int kMaxBias = 512;
-constexpr int kMaxWtab = 64;
 
 // A pipeline stage carries G sub-blocks; sub-block q of a tile is (tap, channel chunk) = divmod(q, kchunks):
 // the A boxes of that tap (128 rows) followed, unless the weights are resident, by its BN weight rows.
@@ -216,7 +215,6 @@ struct PipeK {
     int abort_flag;
     int nboxes;
     Box boxes[kMaxBoxes];
-    uint32_t wtab[4][kMaxWtab];  // resident weights: (byte offset >> 4) of the box that sub-block q of a class reads
     alignas(16) float bias[kMaxBias];
     alignas(16) float gamma[256], beta[256];  // layer normalisation (N <= 256)
     // followed by the epilogue staging: per epilogue warp 32 rows x 32 bf16 columns (2 KB), 16-byte pieces swizzled
@@ -233,7 +231,7 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
     const uint32_t res_bytes = a.wres ? (uint32_t)(a.wtaps * a.kchunks) * b_bytes : 0u;
     PipeK *pipe = reinterpret_cast<PipeK *>(smem + (size_t)S * stage_bytes + res_bytes);
     volatile int *abort_flag = &pipe->abort_flag;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     // ring of accumulators in tensor memory: four when they fit in its 512 columns, else two
     const uint32_t acc_cols = tmem_cols_for(BN);
     const int nacc_log = acc_cols * 4 <= (uint32_t)a.tmem_cap ? 2 : 1, nacc = 1 << nacc_log;
@@ -260,13 +258,6 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
         for (int i = threadIdx.x; i < 256; i += (int)blockDim.x) {
             pipe->gamma[i] = i < a.N ? a.ln_gamma[i] : 0.f;
             pipe->beta[i] = i < a.N ? a.ln_beta[i] : 0.f;
-        }
-    if (a.wres)
-        for (int i = threadIdx.x; i < a.ncls * kMaxWtab; i += (int)blockDim.x) {
-            const int c = i / kMaxWtab, q = i - c * kMaxWtab;
-            const int tap = q / a.kchunks, kc = q - tap * a.kchunks;
-            if (tap < a.cls[c].taps.n)
-                pipe->wtab[c][q] = (uint32_t)((int)a.cls[c].taps.wt[tap] * a.kchunks + kc) * (b_bytes >> 4);
         }
     tc_fence_before();
     __syncthreads();
@@ -341,54 +332,59 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
         if (!ok && lane == 0) drain_copies(pipe->full, it, S);
         __syncwarp();
     } else if (warp == 1) {
-        // ---------------- MMA issue: one thread feeds the tensor core.  Its instruction stream is the
-        // ceiling of the whole kernel (a lone thread issues a dependent instruction only every few cycles),
-        // so the descriptors are built once and advanced by adds.
+        // ---------------- MMA issue: one elected thread feeds the tensor core; the descriptors are built once and
+        // advanced by adds
         const uint32_t idesc = instr_desc(128, BN, 0, 0);
         const uint32_t sbo = 8u * rb;
         const uint64_t d0 = smem_desc_sw(smem_base, 16, sbo, rb);
         const uint32_t d_lo0 = (uint32_t)d0, d_hi = (uint32_t)(d0 >> 32);
         const uint32_t res_lo0 = d_lo0 + ((res_base - smem_base) >> 4);
-        const uint32_t stage16 = stage_bytes >> 4, sub16 = sub_bytes >> 4, ab16 = a_bytes >> 4;
+        const uint32_t stage16 = stage_bytes >> 4, sub16 = sub_bytes >> 4, ab16 = a_bytes >> 4, b16 = b_bytes >> 4;
         const int ksteps = a.CB >> 4;  // 4, 2 or 1 K = 16 steps per box (32 bytes each along the swizzled row)
         int ti = 0, s = 0;
         uint32_t ph = 0;
         bool ok = true;
-        if (a.wres) ok = mbar_wait(&pipe->wfull, 0, abort_flag, a.status);
+        if (a.wres) ok = mbar_wait_warp(&pipe->wfull, 0, abort_flag, a.status);
         TileCursor tc_;
         for (tc_.init(a.total_tiles, a.tiles_n, a.ncls); tc_.valid() && ok; tc_.next(a.tiles_n, a.ncls), ++ti) {
             const int c = tc_.c;
             const int nsub = a.cls[c].taps.n * a.kchunks;
-            const uint32_t *tbl = pipe->wtab[c];
             const int acc = ti & (nacc - 1);
-            ok = mbar_wait(&pipe->tempty[acc], ((ti >> nacc_log) & 1) ^ 1, abort_flag, a.status);
+            ok = mbar_wait_warp(&pipe->tempty[acc], ((ti >> nacc_log) & 1) ^ 1, abort_flag, a.status);
             if (!ok) break;
             tc_fence_after();
             const uint32_t tmem_d = tmem_base + acc * acc_cols;
             uint32_t accum = 0;
+            int tap = 0, kc = 0;  // of the next sub-block (resident weights)
             for (int q0 = 0; q0 < nsub; q0 += G) {
-                ok = mbar_wait(&pipe->full[s], ph, abort_flag, a.status);
+                ok = mbar_wait_warp(&pipe->full[s], ph, abort_flag, a.status);
                 if (!ok) break;
                 tc_fence_after();
-                if (lane == 0) {
-                    const int nval = min(G, nsub - q0);
-                    uint32_t la = d_lo0 + (uint32_t)s * stage16;
-                    for (int gi = 0; gi < nval; ++gi, la += sub16) {
-                        const uint32_t lb = a.wres ? res_lo0 + tbl[q0 + gi] : la + ab16;
+                const int nval = min(G, nsub - q0);
+                uint32_t la = d_lo0 + (uint32_t)s * stage16;
+                for (int gi = 0; gi < nval; ++gi, la += sub16) {
+                    uint32_t lb = la + ab16;
+                    if (a.wres) {
+                        lb = res_lo0 + (uint32_t)((int)a.cls[c].taps.wt[tap] * a.kchunks + kc) * b16;
+                        if (++kc == a.kchunks) { kc = 0; ++tap; }
+                    }
+                    if (elect_one()) {
                         umma_bf16_lh(tmem_d, la, d_hi, lb, d_hi, idesc, accum);
                         if (ksteps >= 2) umma_bf16_lh(tmem_d, la + 2, d_hi, lb + 2, d_hi, idesc, 1u);
                         if (ksteps == 4) {
                             umma_bf16_lh(tmem_d, la + 4, d_hi, lb + 4, d_hi, idesc, 1u);
                             umma_bf16_lh(tmem_d, la + 6, d_hi, lb + 6, d_hi, idesc, 1u);
                         }
-                        accum = 1u;
                     }
+                    accum = 1u;
+                }
+                if (elect_one()) {
                     umma_commit(&pipe->empty[s]);
                 }
                 __syncwarp();
                 if (++s == S) { s = 0; ph ^= 1u; }
             }
-            if (ok && lane == 0) umma_commit(&pipe->tfull[acc]);
+            if (ok && elect_one()) umma_commit(&pipe->tfull[acc]);
             __syncwarp();
         }
     } else {
@@ -666,7 +662,7 @@ __global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_con
     const uint32_t stage_bytes = a_bytes + 128u * 2u * (uint32_t)BN;
     Pipe *pipe = reinterpret_cast<Pipe *>(smem + (size_t)S * stage_bytes);
     volatile int *abort_flag = &pipe->abort_flag;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const uint32_t ncols = tmem_cols_for(BN);
 
     if (threadIdx.x == 0) {
@@ -776,10 +772,10 @@ __global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_con
         uint32_t accum = 0, ph = 0;
         int s = 0;
         for (int kb = 0; kb < nkb && ok; ++kb) {
-            ok = mbar_wait(&pipe->full[s], ph, abort_flag, a.status);
+            ok = mbar_wait_warp(&pipe->full[s], ph, abort_flag, a.status);
             if (!ok) break;
             tc_fence_after();
-            if (lane == 0) {
+            if (elect_one()) {
                 uint32_t la = (uint32_t)dA + (uint32_t)s * (stage_bytes >> 4), lb = (uint32_t)dB + (uint32_t)s * (stage_bytes >> 4);
                 for (int k = 0; k < a.nmma; ++k, la += stepA, lb += stepB) {
                     umma_bf16_lh(tmem_d, la, a_hi, lb, b_hi, idesc, accum);
@@ -790,7 +786,7 @@ __global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_con
             __syncwarp();
             if (++s == S) { s = 0; ph ^= 1u; }
         }
-        if (ok && nkb > 0 && lane == 0) umma_commit(&pipe->tfull[0]);
+        if (ok && nkb > 0 && elect_one()) umma_commit(&pipe->tfull[0]);
         __syncwarp();
     } else if (nkb > 0) {
         // ---------------- epilogue: TMEM lane p is row p of this CTA's 128 x BN tile of dW^T; the whole tile goes
@@ -1021,7 +1017,7 @@ int launch_kmajor(KArgs &a, cudaStream_t st) {
     const size_t res = (size_t)a.wtaps * a.kchunks * b_bytes;
     // resident weights only while they leave most of the shared memory to the A stages: the bytes in flight
     // are what hides the copy latency
-    a.wres = (a.tiles_n == 1 && a.ncls == 1 && res <= kMaxResident && a.wtaps * a.kchunks <= kMaxWtab) ? 1 : 0;
+    a.wres = (a.tiles_n == 1 && a.ncls == 1 && res <= kMaxResident) ? 1 : 0;
     // Narrow tiles (BN <= 128) leave the tensor pipe mostly idle because one thread per CTA cannot issue MMAs
     // fast enough; two CTAs per SM (half the shared and tensor memory each, 8 epilogue warps each) double the
     // issue rate.  Wide tiles run at the tensor rate with one CTA and keep the SM to themselves.

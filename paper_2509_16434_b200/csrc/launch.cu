@@ -19,15 +19,20 @@ static uint64_t hash_key(const PlanKey &k) {
     return h;
 }
 
-int ppo_enqueue(const void *fn, dim3 grid, dim3 block, size_t smem, cudaStream_t st, void **argv) {
+int ppo_enqueue(const void *fn, dim3 grid, dim3 block, size_t smem, bool together, cudaStream_t st, void **argv) {
     cudaLaunchConfig_t c = {};
     c.gridDim = grid;
     c.blockDim = block;
     c.dynamicSmemBytes = smem;
     c.stream = st;
     cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
+    if (together) {
+        at[0].id = cudaLaunchAttributeCooperative;
+        at[0].val.cooperative = 1;
+    } else {
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+    }
     c.attrs = at;
     c.numAttrs = 1;
     ppo_count_launches(1);
@@ -48,7 +53,7 @@ int ppo_replay(const PlanEntry &e, cudaStream_t st) {
         const size_t n = r.offset.size();
         if (n > 32) return PPO_ERR_CUDA;
         for (size_t i = 0; i < n; ++i) argv[i] = const_cast<char *>(r.bytes.data()) + r.offset[i];
-        const int s = ppo_enqueue(r.fn, r.grid, r.block, r.smem, st, argv);
+        const int s = ppo_enqueue(r.fn, r.grid, r.block, r.smem, r.together, st, argv);
         if (s != PPO_OK) return s;
     }
     return PPO_OK;

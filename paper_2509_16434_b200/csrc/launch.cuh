@@ -5,7 +5,7 @@
 // model remember the launches they made under a key of everything the preparation read (shapes and pointers); the next
 // call with the same key only enqueues them.
 //
-// Every kernel launched here starts with grid_wait(): the launch carries the programmatic-serialization attribute, so
+// Every kernel launched by ppo_launch starts with grid_wait(): the launch carries the programmatic-serialization attribute, so
 // the next kernel of the stream may be set up while the one before it drains, and reads or writes memory only after that
 // wait.  (Letting it start earlier still, as soon as every block of the one before it runs, costs 1 to 5 %: the waiting
 // blocks take room from the second stream's kernels.)
@@ -28,6 +28,7 @@ struct LaunchRecord {
     const void *fn;
     dim3 grid, block;
     size_t smem;
+    bool together;                 // all blocks resident at once (cooperative launch)
     std::vector<char> bytes;       // argument values one after the other
     std::vector<uint32_t> offset;  // where each starts
 };
@@ -51,10 +52,10 @@ struct ppo_plans {
 // The record of the operation being prepared on this thread (null: none).
 extern thread_local std::vector<LaunchRecord> *ppo_recording;
 
-int ppo_enqueue(const void *fn, dim3 grid, dim3 block, size_t smem, cudaStream_t st, void **argv);
+int ppo_enqueue(const void *fn, dim3 grid, dim3 block, size_t smem, bool together, cudaStream_t st, void **argv);
 
 template <typename... P, typename... A>
-int ppo_launch(void (*fn)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+int ppo_launch_as(bool together, void (*fn)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
     static_assert(sizeof...(P) == sizeof...(A), "argument count");
     void *argv[sizeof...(A)];
     int n = 0;
@@ -67,6 +68,7 @@ int ppo_launch(void (*fn)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_
         r.grid = grid;
         r.block = block;
         r.smem = smem;
+        r.together = together;
         n = 0;
         const size_t sizes[] = {sizeof(P)...};
         for (size_t i = 0; i < sizeof...(P); ++i) {
@@ -76,7 +78,16 @@ int ppo_launch(void (*fn)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_
         }
         ppo_recording->push_back(std::move(r));
     }
-    return ppo_enqueue(reinterpret_cast<const void *>(fn), grid, block, smem, st, argv);
+    return ppo_enqueue(reinterpret_cast<const void *>(fn), grid, block, smem, together, st, argv);
+}
+template <typename... P, typename... A>
+int ppo_launch(void (*fn)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+    return ppo_launch_as(false, fn, grid, block, smem, st, args...);
+}
+// For kernels whose blocks wait for one another: the launch fails unless they can all be resident at once.
+template <typename... P, typename... A>
+int ppo_launch_together(void (*fn)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+    return ppo_launch_as(true, fn, grid, block, smem, st, args...);
 }
 
 // The entry of a key, or null.

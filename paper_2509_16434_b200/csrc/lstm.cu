@@ -1,0 +1,483 @@
+// The time loop of a recurrent layer as one persistent kernel per direction (sm_100a).
+//
+// A step's product with W_h is small (Be x 4H x H) and every step waits for the one before it, so launch by launch the loop
+// was a chain of 13 us GEMMs and 5 us cell kernels that mostly waited: for W_h from L2, for the pipeline to fill, for the
+// launch.  Here a CTA keeps its slice of W_h in shared memory for all steps, the cell runs on the accumulator (forward) or
+// between two exchanges (backward) with c and its gradient in registers, and the CTAs of a tile of 128 envs meet at a
+// counter in global memory once (forward) or twice (backward) per step.  What a step then costs is the 256 KB of h (or of
+// one gate's gradients) a CTA pulls through L2 (2 us), the cell's memory traffic and the exchanges.
+// The arithmetic is that of the step-by-step path, sum by sum: same bits.
+//
+// All CTAs of a launch have to be resident at once (cooperative launch, one CTA per SM); every wait is bounded: on a
+// time-out the kernel records PPO_ERR_TIMEOUT, waits (bounded) for its copies and returns, and the last CTA to leave
+// clears the counters whatever happened.
+#include "gemm.cuh"
+#include "launch.cuh"
+#include "lstm.cuh"
+#include "tcgen05.cuh"
+#include "tma_host.cuh"
+
+namespace {
+
+using namespace tc;
+
+constexpr int kCellWarps = 8;
+constexpr int kThreads = (2 + kCellWarps) * 32;  // warp 0: TMA producer, warp 1: MMA issue and TMEM owner
+constexpr int kMaxStages = 8;
+constexpr uint32_t kABytes = 128 * 128, kBBytes = 64 * 128;  // one 64-wide chunk of the reduction: 128 envs, 64 weight rows
+constexpr size_t kSmemMax = 227 * 1024;
+
+struct Args {
+    CUtensorMap mapA;  // forward: h_prev [T * Be][H]; backward: gate gradients [T * Be][4H]
+    CUtensorMap mapB;  // forward: W_h [4H][H], boxes of 16 rows; backward: W_h^T [H][4H], boxes of 64 rows
+    int T, Be, H, per_tile, stages;  // per_tile: CTAs of a tile of 128 envs
+    const uint8_t *done;
+    const float *xg, *bias, *h_init, *c_init;        // forward
+    const float *dtop;                               // backward
+    float *gates, *c, *cprev;
+    bf16 *h, *hprev, *dg;
+    float *dhc;
+    unsigned int *counters;  // one per tile, 32 words apart; the last one counts the CTAs that have left
+    int32_t *status;
+};
+
+struct Pipe {
+    uint64_t full[kMaxStages], empty[kMaxStages], tfull, wfull;
+    uint32_t tmem_slot;
+    int abort_flag;
+};
+
+__device__ __forceinline__ void cell_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kCellWarps * 32) : "memory"); }
+__device__ __forceinline__ bool cell_all(bool ok) {
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %1, 0;\n\t"
+        "bar.red.and.pred q, 1, %2, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(r)
+        : "r"(ok ? 1u : 0u), "n"(kCellWarps * 32)
+        : "memory");
+    return r != 0;
+}
+__device__ __forceinline__ void fence_proxy_all() { asm volatile("fence.proxy.async;" ::: "memory"); }
+
+// Arrival at a tile's counter, by one thread behind a barrier of the threads whose writes it publishes.
+__device__ __forceinline__ void tile_arrive(unsigned int *counter) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(counter) : "memory");
+}
+// Bounded wait until a tile's counter has reached `target`.
+__device__ bool tile_wait(const unsigned int *counter, unsigned int target, volatile int *abort_flag, int32_t *status) {
+    const long long t0 = clock64();
+    while (true) {
+        unsigned int v;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(counter) : "memory");
+        if (v >= target) return true;
+        if (*abort_flag) return false;
+        if (clock64() - t0 > kWaitCycles) {
+            *abort_flag = 1;
+            ppo_report(status, PPO_ERR_TIMEOUT);
+            return false;
+        }
+    }
+}
+
+// Eight consecutive fp32 columns of this thread's TMEM lane.
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float *v) {
+    uint32_t r[8];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr)
+                 : "memory");
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+__device__ __forceinline__ void load8(const float *p, float *v) {
+    const float4 a = *reinterpret_cast<const float4 *>(p), b = *reinterpret_cast<const float4 *>(p + 4);
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+}
+__device__ __forceinline__ void load8_l2(const float *p, float *v) {  // written by other CTAs of this launch
+    const float4 a = __ldcg(reinterpret_cast<const float4 *>(p)), b = __ldcg(reinterpret_cast<const float4 *>(p + 4));
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+}
+__device__ __forceinline__ void store8(float *p, const float *v) {
+    *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    *reinterpret_cast<float4 *>(p + 4) = make_float4(v[4], v[5], v[6], v[7]);
+}
+__device__ __forceinline__ uint4 pack8(const float *v) {
+    return make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]), pack_bf16x2(v[6], v[7]));
+}
+
+// Everything the two kernels share around the cell: barriers, tensor memory, the resident weight slice, the stream of A
+// chunks and the MMAs.
+struct Frame {
+    Pipe *pipe;
+    uint32_t smem_base, b_base, tmem;
+    int warp, lane, mt, q, chunks, S;
+};
+
+__device__ __forceinline__ Frame frame_begin(const Args &a, uint8_t *raw) {
+    Frame f;
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
+    f.chunks = a.H >> 6;
+    f.S = a.stages;
+    f.smem_base = smem_u32(smem);
+    f.b_base = f.smem_base + (uint32_t)f.S * kABytes;
+    f.pipe = reinterpret_cast<Pipe *>(smem + (size_t)f.S * kABytes + (size_t)f.chunks * kBBytes);
+    f.warp = warp_index();
+    f.lane = threadIdx.x & 31;
+    f.mt = (int)blockIdx.x / a.per_tile;
+    f.q = (int)blockIdx.x - f.mt * a.per_tile;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < f.S; ++s) {
+            mbar_init(&f.pipe->full[s], 1);
+            mbar_init(&f.pipe->empty[s], 1);
+        }
+        mbar_init(&f.pipe->tfull, 1);
+        mbar_init(&f.pipe->wfull, 1);
+        f.pipe->abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (f.warp == 1) tmem_alloc(&f.pipe->tmem_slot, 64);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    f.tmem = f.pipe->tmem_slot;
+    return f;
+}
+
+__device__ __forceinline__ void frame_end(const Args &a, const Frame &f) {
+    tc_fence_before();
+    __syncthreads();
+    if (f.warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(f.tmem, 64);
+    }
+    if (threadIdx.x == 0) {  // the last CTA to leave clears the counters for the next launch
+        const int tiles = (int)gridDim.x / a.per_tile;
+        __threadfence();
+        if (atomicAdd(a.counters + tiles * 32, 1u) == gridDim.x - 1) {
+            for (int i = 0; i <= tiles; ++i) a.counters[i * 32] = 0u;
+            __threadfence();
+        }
+    }
+}
+
+// Producer: the A chunks of one step (columns col0 .. col0 + H of rows row0 .. row0 + 127).
+__device__ __forceinline__ bool produce_step(const Args &a, const Frame &f, int col0, int row0, int &s, uint32_t &ph, int &it) {
+    for (int k = 0; k < f.chunks; ++k, ++it) {
+        if (!mbar_wait(&f.pipe->empty[s], ph ^ 1u, &f.pipe->abort_flag, a.status)) return false;
+        mbar_arrive_expect_tx(&f.pipe->full[s], kABytes);
+        tma_load_2d(f.smem_base + (uint32_t)s * kABytes, &a.mapA, &f.pipe->full[s], col0 + k * 64, row0);
+        if (++s == f.S) { s = 0; ph ^= 1u; }
+    }
+    return true;
+}
+__device__ __forceinline__ void drain(const Frame &f, int it) {
+    for (int i = max(0, it - f.S); i < it; ++i) {
+        const long long t0 = clock64();
+        while (!mbar_try_wait(&f.pipe->full[i % f.S], (i / f.S) & 1))
+            if (clock64() - t0 > kWaitCycles / 4) break;
+    }
+}
+
+// MMAs of one step into the 64 accumulator columns (warp 1).
+__device__ __forceinline__ bool mma_step(const Args &a, const Frame &f, int &s, uint32_t &ph) {
+    constexpr uint32_t idesc = instr_desc(128, 64, 0, 0);
+    const uint64_t d0 = smem_desc_sw(f.smem_base, 16, 1024, 128);
+    const uint32_t lo = (uint32_t)d0, hi = (uint32_t)(d0 >> 32), b_lo = lo + ((f.b_base - f.smem_base) >> 4);
+    for (int k = 0; k < f.chunks; ++k) {
+        if (!mbar_wait_warp(&f.pipe->full[s], ph, &f.pipe->abort_flag, a.status)) return false;
+        tc_fence_after();
+        if (elect_one()) {
+            const uint32_t la = lo + (uint32_t)s * (kABytes >> 4), lb = b_lo + (uint32_t)k * (kBBytes >> 4);
+            umma_bf16_lh(f.tmem, la, hi, lb, hi, idesc, k > 0 ? 1u : 0u);
+#pragma unroll
+            for (int j = 1; j < 4; ++j) umma_bf16_lh(f.tmem, la + 2 * j, hi, lb + 2 * j, hi, idesc, 1u);
+            umma_commit(&f.pipe->empty[s]);
+        }
+        __syncwarp();
+        if (++s == f.S) { s = 0; ph ^= 1u; }
+    }
+    if (elect_one()) umma_commit(&f.pipe->tfull);
+    __syncwarp();
+    return true;
+}
+
+// Forward over all steps of one layer.  CTA q of a tile owns units 16 q .. 16 q + 15: accumulator column 16 g + j is gate g
+// of unit 16 q + j, so that a thread of the cell holds the four gates of its eight units.
+__global__ void __launch_bounds__(kThreads, 1) lstm_fwd_kernel(const __grid_constant__ Args a) {
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    const Frame f = frame_begin(a, smem_raw);
+    unsigned int *counter = a.counters + f.mt * 32;
+    const int H = a.H, u0 = f.q * 16, row0 = f.mt * 128;
+    volatile int *abort_flag = &f.pipe->abort_flag;
+    if (f.warp == 0) {
+        if (f.lane == 0) {
+            mbar_arrive_expect_tx(&f.pipe->wfull, (uint32_t)f.chunks * kBBytes);
+            for (int k = 0; k < f.chunks; ++k)
+                for (int g = 0; g < 4; ++g)
+                    tma_load_2d(f.b_base + (uint32_t)k * kBBytes + (uint32_t)g * 2048u, &a.mapB, &f.pipe->wfull, k * 64, g * H + u0);
+            int s = 0, it = 0;
+            uint32_t ph = 0;
+            bool ok = true;
+            for (int t = 0; t < a.T && ok; ++t) {
+                ok = tile_wait(counter, (unsigned)(a.per_tile * (t + 1)), abort_flag, a.status);
+                if (!ok) break;
+                ok = produce_step(a, f, 0, t * a.Be + row0, s, ph, it);
+            }
+            if (!ok) drain(f, it);
+        }
+        __syncwarp();
+    } else if (f.warp == 1) {
+        int s = 0;
+        uint32_t ph = 0;
+        bool ok = mbar_wait_warp(&f.pipe->wfull, 0, abort_flag, a.status);
+        for (int t = 0; t < a.T && ok; ++t) ok = mma_step(a, f, s, ph);
+    } else {
+        const int lg = f.warp & 3, half = (f.warp - 2) >> 2, row = lg * 32 + f.lane, e = row0 + row;
+        const bool live = e < a.Be, issuer = threadIdx.x == 64;
+        const int j0 = u0 + 8 * half;
+        const uint32_t tm = f.tmem + ((uint32_t)(lg * 32) << 16) + (uint32_t)(8 * half);
+        float cp[8], bias[4][8];
+#pragma unroll
+        for (int g = 0; g < 4; ++g) load8(a.bias + g * H + j0, bias[g]);
+        if (live) {  // the state the first step starts from
+            const size_t i = (size_t)e * H + j0;
+            float hv[8];
+            load8(a.h_init + i, hv);
+            load8(a.c_init + i, cp);
+            *reinterpret_cast<uint4 *>(a.hprev + i) = pack8(hv);
+            store8(a.cprev + i, cp);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) cp[k] = 0.f;
+        }
+        fence_proxy_all();
+        cell_sync();
+        if (issuer) tile_arrive(counter);
+        for (int t = 0; t < a.T; ++t) {
+            const size_t r = (size_t)t * a.Be + e;
+            float xg[4][8];
+            bool reset = false;
+            if (live) {  // ahead of the wait: they do not depend on this step's product
+#pragma unroll
+                for (int g = 0; g < 4; ++g) load8(a.xg + r * 4 * H + g * H + j0, xg[g]);
+                reset = a.done[r] != 0;
+            }
+            if (!cell_all(mbar_wait(&f.pipe->tfull, t & 1, abort_flag, a.status))) break;
+            tc_fence_after();
+            float hg[4][8];
+#pragma unroll
+            for (int g = 0; g < 4; ++g) tmem_ld8(tm + 16u * g, hg[g]);
+            tmem_wait_ld();
+            tc_fence_before();
+            float gi[8], gf[8], gg[8], go[8], cv[8];
+            uint4 hb = make_uint4(0, 0, 0, 0);
+            if (live) {
+                float hv[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    lstm_cell(xg[0][k] + hg[0][k] + bias[0][k], xg[1][k] + hg[1][k] + bias[1][k], xg[2][k] + hg[2][k] + bias[2][k],
+                              xg[3][k] + hg[3][k] + bias[3][k], cp[k], gi[k], gf[k], gg[k], go[k], cv[k], hv[k]);
+                }
+                hb = pack8(hv);
+                if (t + 1 < a.T) *reinterpret_cast<uint4 *>(a.hprev + (r + a.Be) * H + j0) = reset ? make_uint4(0, 0, 0, 0) : hb;
+            }
+            if (t + 1 < a.T) {  // what the others wait for goes first, the rest behind it
+                fence_proxy_all();
+                cell_sync();
+                if (issuer) tile_arrive(counter);
+            }
+            if (live) {
+                *reinterpret_cast<uint4 *>(a.h + r * H + j0) = hb;
+                float *gp = a.gates + r * 4 * H + j0;
+                store8(gp, gi);
+                store8(gp + H, gf);
+                store8(gp + 2 * H, gg);
+                store8(gp + 3 * H, go);
+                store8(a.c + r * H + j0, cv);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) cp[k] = reset ? 0.f : cv[k];
+                if (t + 1 < a.T) store8(a.cprev + (r + a.Be) * H + j0, cp);
+            }
+        }
+    }
+    frame_end(a, f);
+}
+
+// Back-propagation through all steps of one layer: gate gradients dg of every step.  The product dg W_h of a step reduces
+// over 4 H columns in four slabs (one gate each) whose partial products are added in order: CTA q = (slab, 64 units) forms
+// one, all of them leave their partial products in global memory, and as a cell CTA q works on units 16 q .. 16 q + 15.
+__global__ void __launch_bounds__(kThreads, 1) lstm_bwd_kernel(const __grid_constant__ Args a) {
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    const Frame f = frame_begin(a, smem_raw);
+    unsigned int *counter = a.counters + f.mt * 32;
+    const int H = a.H, row0 = f.mt * 128, slices = H >> 6, slab = f.q / slices, n0 = (f.q - slab * slices) * 64;
+    volatile int *abort_flag = &f.pipe->abort_flag;
+    if (f.warp == 0) {
+        if (f.lane == 0) {
+            mbar_arrive_expect_tx(&f.pipe->wfull, (uint32_t)f.chunks * kBBytes);
+            for (int k = 0; k < f.chunks; ++k)
+                tma_load_2d(f.b_base + (uint32_t)k * kBBytes, &a.mapB, &f.pipe->wfull, slab * H + k * 64, n0);
+            int s = 0, it = 0;
+            uint32_t ph = 0;
+            bool ok = true;
+            for (int t = a.T - 1, i = 0; t > 0 && ok; --t, ++i) {
+                ok = tile_wait(counter, (unsigned)(a.per_tile * (2 * i + 1)), abort_flag, a.status);
+                if (!ok) break;
+                ok = produce_step(a, f, slab * H, t * a.Be + row0, s, ph, it);
+            }
+            if (!ok) drain(f, it);
+        }
+        __syncwarp();
+    } else if (f.warp == 1) {
+        int s = 0;
+        uint32_t ph = 0;
+        bool ok = mbar_wait_warp(&f.pipe->wfull, 0, abort_flag, a.status);
+        for (int t = a.T - 1; t > 0 && ok; --t) ok = mma_step(a, f, s, ph);
+    } else {
+        const int lg = f.warp & 3, half = (f.warp - 2) >> 2, row = lg * 32 + f.lane, e = row0 + row;
+        const bool live = e < a.Be, issuer = threadIdx.x == 64;
+        const int j0 = f.q * 16 + 8 * half;
+        const uint32_t tm = f.tmem + ((uint32_t)(lg * 32) << 16) + (uint32_t)(32 * half);
+        const size_t step = (size_t)a.Be * H;
+        float dcc[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) dcc[k] = 0.f;
+        for (int t = a.T - 1, i = 0; t >= 0; --t, ++i) {
+            const size_t r = (size_t)t * a.Be + e;
+            const bool last = t == a.T - 1;
+            float dtop[8], g4[4][8], cv[8], cp[8];
+            bool carry = false;
+            if (live) {
+                load8(a.dtop + r * H + j0, dtop);
+#pragma unroll
+                for (int g = 0; g < 4; ++g) load8(a.gates + r * 4 * H + g * H + j0, g4[g]);
+                load8(a.c + r * H + j0, cv);
+                load8(a.cprev + r * H + j0, cp);
+                carry = !last && a.done[r] == 0;
+            }
+            if (!last) {  // the partial products of the step after this one
+                bool ok = true;
+                if (issuer) ok = tile_wait(counter, (unsigned)(a.per_tile * 2 * i), abort_flag, a.status);
+                if (!cell_all(ok)) break;
+            }
+            if (live) {
+                float dhn[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) dhn[k] = 0.f;
+                if (carry) {
+                    float p[4][8];
+#pragma unroll
+                    for (int s = 0; s < 4; ++s) load8_l2(a.dhc + s * step + (size_t)e * H + j0, p[s]);
+#pragma unroll
+                    for (int s = 0; s < 4; ++s)
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) dhn[k] += p[s][k];
+                }
+                float di[8], df[8], dgg[8], dgo[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    lstm_cell_back(dtop[k] + dhn[k], carry ? dcc[k] : 0.f, g4[0][k], g4[1][k], g4[2][k], g4[3][k], cv[k], cp[k], di[k],
+                                   df[k], dgg[k], dgo[k], dcc[k]);
+                bf16 *o = a.dg + r * 4 * H + j0;
+                *reinterpret_cast<uint4 *>(o) = pack8(di);
+                *reinterpret_cast<uint4 *>(o + H) = pack8(df);
+                *reinterpret_cast<uint4 *>(o + 2 * H) = pack8(dgg);
+                *reinterpret_cast<uint4 *>(o + 3 * H) = pack8(dgo);
+            }
+            if (t == 0) break;
+            fence_proxy_all();
+            cell_sync();
+            if (issuer) tile_arrive(counter);
+            // this CTA's partial product
+            if (!cell_all(mbar_wait(&f.pipe->tfull, i & 1, abort_flag, a.status))) break;
+            tc_fence_after();
+            float v[32];
+            tmem_ld32(tm, v);
+            tc_fence_before();
+            if (live) {
+                float *o = a.dhc + slab * step + (size_t)e * H + n0 + 32 * half;
+#pragma unroll
+                for (int k = 0; k < 8; ++k) __stcg(reinterpret_cast<float4 *>(o) + k, make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]));
+            }
+            cell_sync();
+            if (issuer) tile_arrive(counter);
+        }
+    }
+    frame_end(a, f);
+}
+
+// Shape part; false where the layer or the sequence does not fit: a slice of W_h has to leave room for four chunks of A, and
+// all CTAs have to be resident at once.
+bool plan(Args &a, int T, int Be, int H, int &ctas, size_t &smem) {
+    if (H % 64 != 0 || T < 1 || Be < 1) return false;
+    a.T = T; a.Be = Be; a.H = H;
+    a.per_tile = H / 16;
+    const long long n = (long long)((Be + 127) / 128) * a.per_tile;
+    if (n > ppo_num_sms() || (Be + 127) / 128 + 1 > kLstmCounters) return false;
+    const size_t fixed = (size_t)(H / 64) * kBBytes + sizeof(Pipe) + 1024;
+    if (fixed + 4 * kABytes > kSmemMax) return false;
+    a.stages = (int)((kSmemMax - fixed) / kABytes);
+    if (a.stages > kMaxStages) a.stages = kMaxStages;
+    smem = fixed + (size_t)a.stages * kABytes;
+    ctas = (int)n;
+    return true;
+}
+
+int prepare_kernel(const void *fn, bool (&set)[64]) {
+    int dev = 0;
+    PPO_CUDA_CHECK(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= 64) return PPO_ERR_CUDA;
+    if (!set[dev]) {
+        PPO_CUDA_CHECK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+        set[dev] = true;
+    }
+    return PPO_OK;
+}
+
+}  // namespace
+
+int lstm_fwd_steps(const LstmSteps &p, const bf16 *Wh, const float *xg, const float *bias, const float *h_init, const float *c_init,
+                   int32_t *status, cudaStream_t st) {
+    Args a = {};
+    int ctas = 0;
+    size_t smem = 0;
+    if (!status || !plan(a, p.T, p.Be, p.H, ctas, smem)) return PPO_ERR_UNSUPPORTED;
+    const long long H = p.H, rows = (long long)p.T * p.Be;
+    const long long da[2] = {H, rows}, sa[1] = {2 * H}, db[2] = {H, 4 * H}, sb[1] = {2 * H};
+    const int ba[2] = {64, 128}, bb[2] = {64, 16};
+    PPO_TRY(make_map_strided(&a.mapA, p.hprev, 2, da, sa, ba));
+    PPO_TRY(make_map_strided(&a.mapB, Wh, 2, db, sb, bb));
+    a.done = p.done;
+    a.xg = xg; a.bias = bias; a.h_init = h_init; a.c_init = c_init;
+    a.gates = p.gates; a.c = p.c; a.cprev = p.cprev; a.h = p.h; a.hprev = p.hprev;
+    a.counters = p.counters;
+    a.status = status;
+    static bool set[64] = {false};
+    PPO_TRY(prepare_kernel(reinterpret_cast<const void *>(lstm_fwd_kernel), set));
+    return ppo_launch_together(lstm_fwd_kernel, dim3(ctas), dim3(kThreads), smem, st, a);
+}
+
+int lstm_bwd_steps(const LstmSteps &p, const bf16 *WhT, const float *dtop, bf16 *dg, float *dhc, int32_t *status, cudaStream_t st) {
+    Args a = {};
+    int ctas = 0;
+    size_t smem = 0;
+    if (!status || !plan(a, p.T, p.Be, p.H, ctas, smem)) return PPO_ERR_UNSUPPORTED;
+    const long long H = p.H, rows = (long long)p.T * p.Be;
+    const long long da[2] = {4 * H, rows}, sa[1] = {8 * H}, db[2] = {4 * H, H}, sb[1] = {8 * H};
+    const int ba[2] = {64, 128}, bb[2] = {64, 64};
+    PPO_TRY(make_map_strided(&a.mapA, dg, 2, da, sa, ba));
+    PPO_TRY(make_map_strided(&a.mapB, WhT, 2, db, sb, bb));
+    a.done = p.done;
+    a.dtop = dtop; a.dg = dg; a.dhc = dhc;
+    a.gates = p.gates; a.c = p.c; a.cprev = p.cprev;
+    a.counters = p.counters;
+    a.status = status;
+    static bool set[64] = {false};
+    PPO_TRY(prepare_kernel(reinterpret_cast<const void *>(lstm_bwd_kernel), set));
+    return ppo_launch_together(lstm_bwd_kernel, dim3(ctas), dim3(kThreads), smem, st, a);
+}

@@ -7,6 +7,7 @@
 #include "common.cuh"
 #include "launch.cuh"
 #include "gemm.cuh"
+#include "lstm.cuh"
 
 static int conv_out(int in, int k) { return (in + 2 * (k / 2) - k) / 2 + 1; }
 
@@ -229,10 +230,11 @@ static size_t carve(ppo_model *m, const ppo_model *shape, int mb, char *base) {
             }
             char *xg = take(4 * R * H * sizeof(float)), *hg = take(4 * R * H * sizeof(float));
             char *dg = take(4 * R * H * sizeof(bf16)), *dt = take(R * H * sizeof(float));
-            char *dh = take(R * H * sizeof(float)), *dc = take(R * H * sizeof(float));
+            char *dh = take(R * H * sizeof(float)), *dc = take(R * H * sizeof(float)), *cn = take((size_t)kLstmCounters * 128);
             if (m) {
                 m->lstm_xg = (float *)xg; m->lstm_hg = (float *)hg; m->lstm_dg = (bf16 *)dg;
                 m->lstm_dtop = (float *)dt; m->lstm_dhc = (float *)dh; m->lstm_dcc = (float *)dc;
+                m->lstm_counters = (unsigned int *)cn;
             }
         }
         if (shape->d.embed > 0) {
@@ -274,7 +276,7 @@ extern "C" int ppo_model_bind(ppo_model *m, float *master, void *shadow, float *
     carve(m, m, microbatch, m->ws);
     m->fwd_valid = false;
     m->wT_valid = false;
-    m->ticket_zeroed = false;
+    m->ticket_zeroed = m->counters_zeroed = false;
     return PPO_OK;
 }
 

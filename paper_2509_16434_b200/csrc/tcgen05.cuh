@@ -59,6 +59,26 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volati
     return mbar_wait_limit(bar, parity, abort_flag, status, kWaitCycles);
 }
 
+// Warp roles that feed the tensor core or the copy engine run with all lanes in uniform control flow and let one elected
+// lane issue: the operands of tcgen05.mma and of the bulk copies are warp-uniform registers, and the compiler keeps
+// addresses and loop state there only where it can see that they are uniform.  With the lane picked by its index instead, an
+// issue takes 87 to 130 cycles of moving operands over; this way the tensor core accepts one every 41 (N = 32), 48 (64),
+// 64 (128) or 128 (256) cycles.
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+__device__ __forceinline__ bool elect_one() {  // the same lane every time
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(p));
+    return p != 0;
+}
+// mbar_wait by a whole warp with one answer for all lanes.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity, volatile int *abort_flag, int32_t *status) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status)) != 0;
+}
+
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool valid) {
     const uint32_t n = valid ? 16u : 0u;  // 0 source bytes: the 16 destination bytes are zero-filled
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
