@@ -29,7 +29,10 @@ namespace {
 
 using namespace tc;
 
-constexpr int kEpiWarps = 8;  // of an epilogue group; a CTA that has the SM to itself runs two groups on alternate tiles
+// Warps of an epilogue group: two per TMEM lane quarter, which share out the columns; one where there are only 32 columns.
+// The groups of a CTA work on alternate tiles.
+template <bool NARROW>
+constexpr int kEpiWarps = NARROW ? 4 : 8;
 
 constexpr int kMaxSlots = 8;
 constexpr int kMaxOps = 9;
@@ -68,6 +71,8 @@ struct Args {
     uint32_t w_box;         // bytes of one box of weights
     uint32_t slot_bytes, slots_bytes;  // of one slot; of all of them, rounded up
     uint32_t stg_bytes;     // of a staging buffer
+    int stg_row;            // of a row of it, over all its output groups
+    bool narrow;
     int slots, nbuf, neg;   // slots, staging buffers per epilogue group, epilogue groups
     int Wt, R, I, Wp, Rp;   // tile: Wt x R outputs of I images; cells per box row and box rows per image
     int xsegs, ysegs, tiles;
@@ -94,7 +99,8 @@ struct Pipe {
     alignas(16) float bias[256], gamma[256], beta[256];
 };
 
-__device__ __forceinline__ void epi_sync(int eg) { asm volatile("bar.sync %0, %1;" ::"r"(1 + eg), "n"(kEpiWarps * 32) : "memory"); }
+template <int EPW>
+__device__ __forceinline__ void epi_sync(int eg) { asm volatile("bar.sync %0, %1;" ::"r"(1 + eg), "n"(EPW * 32) : "memory"); }
 
 // The sign bits of bytes 1 and 3, each replicated over its half word (prmt.b32 in its sign-replicating form).
 __device__ __forceinline__ uint32_t half_signs(uint32_t x) {
@@ -150,6 +156,7 @@ struct TileAt {
 };
 
 // Barrier of an epilogue group that also ANDs a condition over them (a bounded wait that ran out in one warp ends all).
+template <int EPW>
 __device__ __forceinline__ bool epi_all(bool ok, int eg) {
     uint32_t r;
     asm volatile(
@@ -158,15 +165,17 @@ __device__ __forceinline__ bool epi_all(bool ok, int eg) {
         "bar.red.and.pred q, %3, %2, p;\n\t"
         "selp.u32 %0, 1, 0, q;\n\t}"
         : "=r"(r)
-        : "r"(ok ? 1u : 0u), "n"(kEpiWarps * 32), "r"(1 + eg)
+        : "r"(ok ? 1u : 0u), "n"(EPW * 32), "r"(1 + eg)
         : "memory");
     return r != 0;
 }
 
 // GC: columns of an output group, i.e. of one pixel of one store (16, 32 or 64; its bytes are the swizzled row).
 // KS: K = 16 steps per channel chunk (1, 2 or 4: rows of 32, 64 or 128 bytes).
-template <int MODE, int GC, int KS>
+// NARROW: forward with 32 output channels.
+template <int MODE, int GC, int KS, bool NARROW>
 __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a) {
+    constexpr int EPW = kEpiWarps<NARROW>;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t smem_base = smem_u32(smem);
@@ -187,7 +196,7 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
         }
         for (int i = 0; i < nacc; ++i) {
             mbar_init(&pipe->tfull[i], 1);
-            mbar_init(&pipe->tempty[i], kEpiWarps * 32);
+            mbar_init(&pipe->tempty[i], EPW * 32);
         }
         mbar_init(&pipe->wfull, 1);
         pipe->abort_flag = 0;
@@ -348,15 +357,15 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
         }
     } else {
         // ---------------- epilogue: warp reads TMEM lanes 32 (warp % 4) .. +31 and, of every 64 columns, half `h`
-        const int lg = warp & 3, eg = (warp - 2) >> 3, h = ((warp - 2) >> 2) & 1;
+        const int lg = warp & 3, eg = (warp - 2) / EPW, h = NARROW ? 0 : ((warp - 2) >> 2) & 1;
         const int m = lg * 32 + lane;
         const int ci = m / (a.Rp * a.Wp), mr = m - ci * a.Rp * a.Wp, cr = mr / a.Wp, cx = mr - cr * a.Wp;
         const bool cell = ci < a.I && cr < a.R && cx < a.Wt;  // an output of the tile, not a halo cell
         const int srow = (ci * a.R + cr) * a.Wt + cx;         // its row in the dense staging tile
-        const bool issuer = threadIdx.x == 64 + eg * kEpiWarps * 32;
+        const bool issuer = threadIdx.x == 64 + eg * EPW * 32;
         constexpr uint32_t RBO = GC * 2;                      // bytes of a staged row
         const uint32_t sx = GC == 64 ? (uint32_t)(srow & 7) : (GC == 32 ? (uint32_t)(srow >> 1) & 3u : (uint32_t)(srow >> 2) & 1u);
-        const uint32_t grp_bytes = a.stg_bytes * GC / 64u;    // of an output group's part of a staging buffer
+        const uint32_t grp_bytes = a.stg_bytes / (uint32_t)a.stg_row * RBO;    // of an output group's part of a staging buffer
         const int nsteps = (a.N + 63) >> 6;
         int acc = eg, buf = 0;  // nacc is even where there are two groups
         uint32_t aph = 0;
@@ -376,7 +385,7 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
         };
         auto store_step = [&](uint32_t stg, int s, const CUtensorMap *maps) {
             fence_async_smem();
-            epi_sync(eg);
+            epi_sync<EPW>(eg);
             if (issuer) {
 #pragma unroll
                 for (int g = 0; g < 64 / GC; ++g) {
@@ -439,27 +448,81 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
             for (int k = 0; k < a.neg; ++k) t_next.next(a);
             if (li + a.neg < nt) fetch_gates(t_next);
             stage_free();
-            const bool ok = epi_all(mbar_wait(&pipe->tfull[acc], aph, abort_flag, a.status), eg);
+            const bool ok = epi_all<EPW>(mbar_wait(&pipe->tfull[acc], aph, abort_flag, a.status), eg);
             if (!ok) break;
             tc_fence_after();
             const uint32_t lane_base = tmem_base + (uint32_t)(acc * a.acc_cols) + ((uint32_t)(lg * 32) << 16);
+            if (MODE == FWD_LN && NARROW) {
+                // Layer normalisation with a row's 32 channels in registers: one walk through tensor memory, and both results
+                // leave with one hand-over.
+                const long long px = ((long long)n * a.Hr + y) * a.Wr + x;
+                float v[32];
+                tmem_ld32(lane_base, v);
+                tc_fence_before();
+                mbar_arrive(&pipe->tempty[acc]);
+                float sum = 0.f, sq = 0.f;
+#pragma unroll
+                for (int i = 0; i < 32; ++i) {
+                    v[i] += pipe->bias[i];
+                    sum += v[i];
+                }
+                const float mean = sum / 32.f;
+#pragma unroll
+                for (int i = 0; i < 32; ++i) {
+                    v[i] -= mean;
+                    sq += v[i] * v[i];
+                }
+                const float rs = rsqrtf(sq / 32.f + kLnEps);
+                const uint32_t stg = stg0 + (uint32_t)buf * a.stg_bytes;
+                uint32_t w = 0;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    uint32_t xh[4], rl[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int c = 8 * k + 2 * i;
+                        const float x0 = v[c] * rs, x1 = v[c + 1] * rs;
+                        xh[i] = pack_bf16x2(x0, x1);
+                        rl[i] = relu_pack_bf16x2(fmaf(pipe->gamma[c], x0, pipe->beta[c]), fmaf(pipe->gamma[c + 1], x1, pipe->beta[c + 1]));
+                        w = gate_bits_add(w, rl[i], 4 * k + i);
+                    }
+                    if (cell) {
+                        put(stg, 8 * k, make_uint4(xh[0], xh[1], xh[2], xh[3]));
+                        put(stg, 32 + 8 * k, make_uint4(rl[0], rl[1], rl[2], rl[3]));
+                    }
+                }
+                if (live) {
+                    a.ln_rstd[px] = rs;
+                    if (a.out_bits) a.out_bits[px] = w;
+                }
+                fence_async_smem();
+                epi_sync<EPW>(eg);
+                if (issuer) {
+                    tma_store_4d(&a.mapX, stg, 0, t.x, t.y, t.n);
+                    tma_store_4d(&a.mapO[0], stg + grp_bytes, 0, t.x, t.y, t.n);
+                    bulk_commit();
+                }
+                if (++buf == a.nbuf) buf = 0;
+                acc += a.neg;
+                if (acc >= nacc) { acc = eg; aph ^= 1u; }
+                continue;
+            }
             if (MODE == FWD_LN) {
                 // Layer normalisation over the N channels of this thread's row: the row is walked twice in tensor memory
-                // (mean, then variance about it), 16 columns at a time.  With 32 channels the two warps of a lane quarter
-                // take 16 columns each, else 32 of every 64.
+                // (mean, then variance about it), 32 columns at a time; the two warps of a lane quarter take 32 of every 64.
                 float sum = 0.f, sq = 0.f;
-                for (int c0 = 0; c0 < a.N; c0 += 16) {
-                    float v[16];
-                    tmem_ld16(lane_base + (uint32_t)c0, v);
+                for (int c0 = 0; c0 < a.N; c0 += 32) {
+                    float v[32];
+                    tmem_ld32(lane_base + (uint32_t)c0, v);
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) sum += v[i] + pipe->bias[c0 + i];
+                    for (int i = 0; i < 32; ++i) sum += v[i] + pipe->bias[c0 + i];
                 }
                 const float mean = sum / (float)a.N;
-                for (int c0 = 0; c0 < a.N; c0 += 16) {
-                    float v[16];
-                    tmem_ld16(lane_base + (uint32_t)c0, v);
+                for (int c0 = 0; c0 < a.N; c0 += 32) {
+                    float v[32];
+                    tmem_ld32(lane_base + (uint32_t)c0, v);
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) {
+                    for (int i = 0; i < 32; ++i) {
                         const float d = v[i] + pipe->bias[c0 + i] - mean;
                         sq += d * d;
                     }
@@ -467,20 +530,18 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
                 const float rs = rsqrtf(sq / (float)a.N + kLnEps);
                 const long long px = ((long long)n * a.Hr + y) * a.Wr + x;
                 if (live && h == 0) a.ln_rstd[px] = rs;
-                const bool narrow = a.N == 32;
-                const int nsub = narrow ? 1 : 2;
 #pragma unroll 1
                 for (int s = 0; s < nsteps; ++s) {
                     if (s > 0) {
                         stage_free();
-                        epi_sync(eg);
+                        epi_sync<EPW>(eg);
                     }
                     const uint32_t stg = stg0 + (uint32_t)buf * a.stg_bytes;
-                    const int cb = narrow ? h * 16 : s * 64 + h * 32;
+                    const int cb = s * 64 + h * 32;
                     uint32_t keep[2][8];  // ReLU outputs of the sub-chunks, written after the normalised values have left
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
-                        if (j < nsub && cb < a.N) {
+                        if (cb < a.N) {
                             const int c0 = cb + 16 * j;
                             float v[16];
                             tmem_ld16(lane_base + (uint32_t)c0, v);
@@ -505,30 +566,20 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
                     }
                     store_step(stg, s, &a.mapX);
                     stage_free();
-                    epi_sync(eg);
+                    epi_sync<EPW>(eg);
                     const uint32_t stg2 = stg0 + (uint32_t)buf * a.stg_bytes;
                     if (cb < a.N) {
                         uint32_t w = 0;
 #pragma unroll
                         for (int j = 0; j < 2; ++j) {
-                            if (j < nsub) {
-                                if (cell) {
-                                    put(stg2, ((cb + 16 * j) & 63), make_uint4(keep[j][0], keep[j][1], keep[j][2], keep[j][3]));
-                                    put(stg2, ((cb + 16 * j) & 63) + 8, make_uint4(keep[j][4], keep[j][5], keep[j][6], keep[j][7]));
-                                }
+                            if (cell) {
+                                put(stg2, ((cb + 16 * j) & 63), make_uint4(keep[j][0], keep[j][1], keep[j][2], keep[j][3]));
+                                put(stg2, ((cb + 16 * j) & 63) + 8, make_uint4(keep[j][4], keep[j][5], keep[j][6], keep[j][7]));
+                            }
 #pragma unroll
-                                for (int i = 0; i < 8; ++i) w = gate_bits_add(w, keep[j][i], 8 * j + i);
-                            }
+                            for (int i = 0; i < 8; ++i) w = gate_bits_add(w, keep[j][i], 8 * j + i);
                         }
-                        if (a.out_bits && live) {
-                            if (narrow) {  // channels 16h .. 16h + 15: bytes h and 2 + h of the pixel's word
-                                uint8_t *bp = reinterpret_cast<uint8_t *>(a.out_bits + px);
-                                bp[h] = (uint8_t)w;
-                                bp[2 + h] = (uint8_t)(w >> 16);
-                            } else {
-                                a.out_bits[px * (a.N >> 5) + (cb >> 5)] = w;
-                            }
-                        }
+                        if (a.out_bits && live) a.out_bits[px * (a.N >> 5) + (cb >> 5)] = w;
                     }
                     store_step(stg2, s, &a.mapO[0]);
                 }
@@ -548,7 +599,7 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
                 }
                 if (s > 0) {
                     stage_free();
-                    epi_sync(eg);
+                    epi_sync<EPW>(eg);
                 }
                 const uint32_t stg = stg0 + (uint32_t)buf * a.stg_bytes;
                 if (MODE == FWD) {
@@ -610,7 +661,7 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
 
 // --------------------------------------------------------------------- host ----
 
-uint32_t stage_rows_bytes(int rows) { return ((uint32_t)rows * 128u + 1023u) & ~1023u; }
+uint32_t stage_rows_bytes(int rows, int row_bytes) { return ((uint32_t)(rows * row_bytes) + 1023u) & ~1023u; }
 
 // Tile rectangle whose loads (`loads` slots) and staging buffers (`bufs`) fit into `room` bytes: fewest tiles over the
 // whole grid, then fewest loaded cells.  The M rows of a tile (halo cells included, except behind its last row) have to
@@ -634,7 +685,7 @@ bool choose_tile(Args &a, int Wr, int Hr, int B, size_t room, int loads, int buf
             }
             auto fits = [&](int img) {
                 const size_t slot = ((size_t)img * (Re + 1) * Wp * a.rb + 127) & ~size_t(127);
-                return (size_t)loads * slot + (size_t)bufs * stage_rows_bytes(img * Re * Wt) <= room;
+                return (size_t)loads * slot + (size_t)bufs * stage_rows_bytes(img * Re * Wt, a.stg_row) <= room;
             };
             while (I > 1 && !fits(I)) --I;
             if (!fits(I)) continue;
@@ -665,6 +716,7 @@ bool choose_tile(Args &a, int Wr, int Hr, int B, size_t room, int loads, int buf
 bool plan(Args &a, int Wr, int Hr, int B) {
     const size_t w = ((size_t)a.nchunks * a.w_chunk + 1023) & ~size_t(1023);
     const size_t fixed = w + sizeof(Pipe) + 1024 + 1024;  // alignment of the base and behind the slots
+    a.stg_row = a.narrow && !a.ln_gamma ? 64 : 128;  // narrow: 32 columns, normalised values beside the outputs
     a.acc_cols = 32;
     while (a.acc_cols < a.N) a.acc_cols *= 2;
     const size_t half = kSmemMax / 2 - 512;
@@ -673,16 +725,16 @@ bool plan(Args &a, int Wr, int Hr, int B) {
     for (int two = a.N <= 128 ? 1 : 0; two >= 0; --two) {
         const size_t room = two ? half : kSmemMax;
         if (fixed >= room) continue;
-        a.neg = two ? 1 : 2;
+        a.neg = (two ? 1 : 2) * (a.narrow ? 2 : 1);
         const int least = a.nloads == 4 || two ? a.nloads : a.nloads + 1;
         if (!choose_tile(a, Wr, Hr, B, room - fixed, least, a.neg)) continue;
         if (two && a.tiles > best.tiles) continue;  // no smaller tile for the sake of a second CTA
         a.slot_bytes = (uint32_t)(a.I * a.Rp * a.Wp * a.rb + 127) & ~127u;
-        a.stg_bytes = stage_rows_bytes(a.I * a.R * a.Wt);
+        a.stg_bytes = stage_rows_bytes(a.I * a.R * a.Wt, a.stg_row);
         // a second staging buffer comes before more slots where a step stages twice (normalised values, then outputs) or a
         // tile is one load; a plain forward tile wants its next two planes first (32 -> 64 channels: 1.45 -> 1.29 ms)
         const int before = a.nloads == 4 && !a.ln_gamma ? a.nloads + 2 : least;
-        a.nbuf = two && (size_t)before * a.slot_bytes + 2 * (size_t)a.stg_bytes <= room - fixed ? 2 : 1;
+        a.nbuf = two && (size_t)before * a.slot_bytes + 2 * (size_t)(a.neg * a.stg_bytes) <= room - fixed ? 2 : 1;
         a.slots = (int)((room - fixed - (size_t)(a.nbuf * a.neg) * a.stg_bytes) / a.slot_bytes);
         if (a.slots > kMaxSlots) a.slots = kMaxSlots;
         a.slots_bytes = ((uint32_t)a.slots * a.slot_bytes + 1023u) & ~1023u;
@@ -697,32 +749,33 @@ bool plan(Args &a, int Wr, int Hr, int B) {
     return false;
 }
 
-template <int MODE, int GC, int KS>
+template <int MODE, int GC, int KS, bool NARROW>
 int launch_one(const Args &a, cudaStream_t st) {
     static bool attr_set[64] = {false};
     int dev = 0;
     PPO_CUDA_CHECK(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64) return PPO_ERR_CUDA;
     if (!attr_set[dev]) {
-        PPO_CUDA_CHECK(cudaFuncSetAttribute(conv_halo_kernel<MODE, GC, KS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+        PPO_CUDA_CHECK(cudaFuncSetAttribute(conv_halo_kernel<MODE, GC, KS, NARROW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
         attr_set[dev] = true;
     }
-    PPO_TRY(ppo_launch(conv_halo_kernel<MODE, GC, KS>, dim3((unsigned)a.grid), dim3((2 + a.neg * kEpiWarps) * 32), a.smem, st, a));
+    PPO_TRY(ppo_launch(conv_halo_kernel<MODE, GC, KS, NARROW>, dim3((unsigned)a.grid), dim3((2 + a.neg * kEpiWarps<NARROW>) * 32), a.smem, st, a));
     return PPO_OK;
 }
 
-template <int MODE, int GC>
-int launch_ks(const Args &a, int ks, cudaStream_t st) {
-    if (ks == 4) return launch_one<MODE, GC, 4>(a, st);
-    return ks == 2 ? launch_one<MODE, GC, 2>(a, st) : launch_one<MODE, GC, 1>(a, st);
+template <int MODE, int GC, bool NARROW = false>
+int launch_ks(const Args &a, cudaStream_t st) {
+    const int ks = a.CB >> 4;
+    if (ks == 4) return launch_one<MODE, GC, 4, NARROW>(a, st);
+    return ks == 2 ? launch_one<MODE, GC, 2, NARROW>(a, st) : launch_one<MODE, GC, 1, NARROW>(a, st);
 }
 
 int launch(const Args &a, int mode, int GC, cudaStream_t st) {
-    const int ks = a.CB >> 4;
-    if (mode == FWD) return GC == 64 ? launch_ks<FWD, 64>(a, ks, st) : launch_ks<FWD, 32>(a, ks, st);
-    if (mode == FWD_LN) return GC == 64 ? launch_ks<FWD_LN, 64>(a, ks, st) : launch_ks<FWD_LN, 32>(a, ks, st);
-    if (mode == DG_BITS) return GC == 64 ? launch_ks<DG_BITS, 64>(a, ks, st) : launch_ks<DG_BITS, 32>(a, ks, st);
-    return launch_ks<DG_ACT, 16>(a, ks, st);
+    if (mode == FWD && a.narrow) return launch_ks<FWD, 32, true>(a, st);
+    if (mode == FWD) return GC == 64 ? launch_ks<FWD, 64>(a, st) : launch_ks<FWD, 32>(a, st);
+    if (mode == FWD_LN) return a.narrow ? launch_ks<FWD_LN, 32, true>(a, st) : launch_ks<FWD_LN, 64>(a, st);  // a power of two
+    if (mode == DG_BITS) return GC == 64 ? launch_ks<DG_BITS, 64>(a, st) : launch_ks<DG_BITS, 32>(a, st);
+    return launch_ks<DG_ACT, 16>(a, st);
 }
 
 // Channels per chunk of a C-channel source, or 0.
@@ -745,6 +798,8 @@ int halo_conv_fwd(const ConvGeom &g, const bf16 *X, const bf16 *W, const FwdEpil
     a.w_box = (uint32_t)(g.Co * a.rb);
     a.w_chunk = 9u * a.w_box;
     a.ln_gamma = e.ln_gamma;
+    a.narrow = g.Co == 32;
+    if (e.ln_gamma && (g.Co & (g.Co - 1)) != 0) return PPO_ERR_UNSUPPORTED;
     if (!plan(a, g.Wo, g.Ho, g.B)) return PPO_ERR_UNSUPPORTED;
     for (int p = 0; p < 4; ++p) {
         const int py = p >> 1, px = p & 1;

@@ -840,12 +840,19 @@ __global__ void __launch_bounds__(256) wgrad_reduce_kernel(const float *__restri
     const float *src = part + ((size_t)y * jtiles + x) * tile + (size_t)c * 128 + p;
     float acc = 0.f;
     int z = 0;
-    for (; z + 16 <= splits; z += 16) {  // the loads of sixteen splits are in flight while the sum stays in order
-        float v[16];
+    for (; z + 32 <= splits; z += 32) {  // the loads of 32 splits are in flight while the sum stays in order
+        float v[32];
 #pragma unroll
-        for (int u = 0; u < 16; ++u) v[u] = src[(size_t)(z + u) * per_split];
+        for (int u = 0; u < 32; ++u) v[u] = src[(size_t)(z + u) * per_split];
 #pragma unroll
-        for (int u = 0; u < 16; ++u) acc += v[u];
+        for (int u = 0; u < 32; ++u) acc += v[u];
+    }
+    for (; z + 8 <= splits; z += 8) {
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = src[(size_t)(z + u) * per_split];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) acc += v[u];
     }
     for (; z < splits; ++z) acc += src[(size_t)z * per_split];
     *dst += acc;
@@ -1139,7 +1146,9 @@ int tma_gemm_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, i
     // per-thread epilogue (16 columns = one class at a time) takes over, which needs the bf16 gate
     if (!flat && (g.k < 3 || g.Hi < 2 || g.Wi < 2 || !Wc)) return PPO_ERR_UNSUPPORTED;
     if (!flat && g.Ci % 32 != 0 && (g.Ci % 16 != 0 || !e.mask_act || e.mask_bits || !e.out)) return PPO_ERR_UNSUPPORTED;
-    const int CB = channels_per_box(g.Co, flat);
+    // at most 16 columns in rows padded to 16 (the head): one box, one MMA of K = 16
+    const bool head = flat && g.Co <= 16 && ldy == 16 && wt_ld <= 16;
+    const int CB = head ? 16 : channels_per_box(g.Co, flat);
     if (CB == 0 || g.taps() > kMaxTaps || wt_ld < g.Co) return PPO_ERR_UNSUPPORTED;
     KArgs a = {};
     a.CB = CB;
@@ -1151,7 +1160,7 @@ int tma_gemm_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, i
     if (!(flat && e.ksplit <= 1 ? make_flat_grid(a.grid, g.B, (g.Ci + flat_n - 1) / flat_n, a.row_bytes)
                                 : make_grid(a.grid, Wr, Hr, flat ? 1 : g.B, a.row_bytes)))
         return PPO_ERR_UNSUPPORTED;
-    int s = flat ? make_act_maps(a.mapA, dY, g.Co, ldy, g.B, 1, 1, a.grid, CB, 1)
+    int s = flat ? make_act_maps(a.mapA, dY, head ? 16 : g.Co, ldy, g.B, 1, 1, a.grid, CB, 1)
                  : make_act_maps(a.mapA, dY, g.Co, ldy, g.Wo, g.Ho, g.B, a.grid, CB, 1);
     if (s != PPO_OK) return s;
     a.s_mul = 1;
