@@ -29,10 +29,9 @@ namespace {
 
 using namespace tc;
 
-// Warps of an epilogue group: two per TMEM lane quarter, which share out the columns; one where there are only 32 columns.
-// The groups of a CTA work on alternate tiles.
-template <bool NARROW>
-constexpr int kEpiWarps = NARROW ? 4 : 8;
+// An epilogue group works on a tile, the groups of a CTA on alternate ones.  A group has four warps, one per TMEM lane
+// quarter: fewer meet at its barriers, and two tiles are drained at a time.  Where shared memory holds only one CTA per SM
+// and two staging buffers, a group has eight warps, two per lane quarter, which share out the columns.
 
 constexpr int kMaxSlots = 8;
 constexpr int kMaxOps = 9;
@@ -72,7 +71,8 @@ struct Args {
     uint32_t slot_bytes, slots_bytes;  // of one slot; of all of them, rounded up
     uint32_t stg_bytes;     // of a staging buffer
     int stg_row;            // of a row of it, over all its output groups
-    bool narrow;
+    int epw;                // warps of an epilogue group
+    bool wide_gate;         // gates come as 16 activations per pixel: too many registers for a whole row per thread
     int slots, nbuf, neg;   // slots, staging buffers per epilogue group, epilogue groups
     int Wt, R, I, Wp, Rp;   // tile: Wt x R outputs of I images; cells per box row and box rows per image
     int xsegs, ysegs, tiles;
@@ -172,10 +172,10 @@ __device__ __forceinline__ bool epi_all(bool ok, int eg) {
 
 // GC: columns of an output group, i.e. of one pixel of one store (16, 32 or 64; its bytes are the swizzled row).
 // KS: K = 16 steps per channel chunk (1, 2 or 4: rows of 32, 64 or 128 bytes).
-// NARROW: forward with 32 output channels.
-template <int MODE, int GC, int KS, bool NARROW>
+// EPW: warps of an epilogue group, 4 or 8.
+template <int MODE, int GC, int KS, int EPW>
 __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a) {
-    constexpr int EPW = kEpiWarps<NARROW>;
+    constexpr int NH = EPW == 4 ? 2 : 1;  // halves of 64 columns a warp works on
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t smem_base = smem_u32(smem);
@@ -357,7 +357,7 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
         }
     } else {
         // ---------------- epilogue: warp reads TMEM lanes 32 (warp % 4) .. +31 and, of every 64 columns, half `h`
-        const int lg = warp & 3, eg = (warp - 2) / EPW, h = NARROW ? 0 : ((warp - 2) >> 2) & 1;
+        const int lg = warp & 3, eg = (warp - 2) / EPW, h = EPW == 4 ? 0 : ((warp - 2) >> 2) & 1;
         const int m = lg * 32 + lane;
         const int ci = m / (a.Rp * a.Wp), mr = m - ci * a.Rp * a.Wp, cr = mr / a.Wp, cx = mr - cr * a.Wp;
         const bool cell = ci < a.I && cr < a.R && cx < a.Wt;  // an output of the tile, not a halo cell
@@ -413,12 +413,12 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
             const bool live = cell && n < a.B && y < a.Hr && x < a.Wr;
             if (MODE == DG_BITS) {
 #pragma unroll
-                for (int s = 0; s < 4; ++s) {
-                    gate_n[s] = 0u;
-                    const int col = s * 64 + h * 32, grp = col / GC;
+                for (int k = 0; k < 4; ++k) {  // step k / NH, half k % NH (EPW == 4: at most 128 columns)
+                    gate_n[k] = 0u;
+                    const int hh = EPW == 4 ? k % NH : h, col = (k / NH) * 64 + hh * 32, grp = col / GC;
                     const int iy = 2 * y + (grp >> 1), ix = 2 * x + ((grp == 1 || grp == 2) ? 1 : 0);
                     if (col < a.N && live && iy < a.Hi && ix < a.Wi)
-                        gate_n[s] = __ldg(a.mask_bits + (((long long)n * a.Hi + iy) * a.Wi + ix) * (GC / 32 > 0 ? GC / 32 : 1) + (GC == 64 ? h : 0));
+                        gate_n[k] = __ldg(a.mask_bits + (((long long)n * a.Hi + iy) * a.Wi + ix) * (GC / 32 > 0 ? GC / 32 : 1) + (GC == 64 ? hh : 0));
                 }
             }
             if (MODE == DG_ACT) {  // GC == 16: this thread's 32 columns are two classes of 16 channels
@@ -452,136 +452,78 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
             if (!ok) break;
             tc_fence_after();
             const uint32_t lane_base = tmem_base + (uint32_t)(acc * a.acc_cols) + ((uint32_t)(lg * 32) << 16);
-            if (MODE == FWD_LN && NARROW) {
-                // Layer normalisation with a row's 32 channels in registers: one walk through tensor memory, and both results
-                // leave with one hand-over.
-                const long long px = ((long long)n * a.Hr + y) * a.Wr + x;
-                float v[32];
-                tmem_ld32(lane_base, v);
-                tc_fence_before();
-                mbar_arrive(&pipe->tempty[acc]);
-                float sum = 0.f, sq = 0.f;
-#pragma unroll
-                for (int i = 0; i < 32; ++i) {
-                    v[i] += pipe->bias[i];
-                    sum += v[i];
-                }
-                const float mean = sum / 32.f;
-#pragma unroll
-                for (int i = 0; i < 32; ++i) {
-                    v[i] -= mean;
-                    sq += v[i] * v[i];
-                }
-                const float rs = rsqrtf(sq / 32.f + kLnEps);
-                const uint32_t stg = stg0 + (uint32_t)buf * a.stg_bytes;
-                uint32_t w = 0;
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    uint32_t xh[4], rl[4];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int c = 8 * k + 2 * i;
-                        const float x0 = v[c] * rs, x1 = v[c + 1] * rs;
-                        xh[i] = pack_bf16x2(x0, x1);
-                        rl[i] = relu_pack_bf16x2(fmaf(pipe->gamma[c], x0, pipe->beta[c]), fmaf(pipe->gamma[c + 1], x1, pipe->beta[c + 1]));
-                        w = gate_bits_add(w, rl[i], 4 * k + i);
-                    }
-                    if (cell) {
-                        put(stg, 8 * k, make_uint4(xh[0], xh[1], xh[2], xh[3]));
-                        put(stg, 32 + 8 * k, make_uint4(rl[0], rl[1], rl[2], rl[3]));
-                    }
-                }
-                if (live) {
-                    a.ln_rstd[px] = rs;
-                    if (a.out_bits) a.out_bits[px] = w;
-                }
-                fence_async_smem();
-                epi_sync<EPW>(eg);
-                if (issuer) {
-                    tma_store_4d(&a.mapX, stg, 0, t.x, t.y, t.n);
-                    tma_store_4d(&a.mapO[0], stg + grp_bytes, 0, t.x, t.y, t.n);
-                    bulk_commit();
-                }
-                if (++buf == a.nbuf) buf = 0;
-                acc += a.neg;
-                if (acc >= nacc) { acc = eg; aph ^= 1u; }
-                continue;
-            }
             if (MODE == FWD_LN) {
-                // Layer normalisation over the N channels of this thread's row: the row is walked twice in tensor memory
-                // (mean, then variance about it), 32 columns at a time; the two warps of a lane quarter take 32 of every 64.
+                // Layer normalisation over the N channels of this thread's row.  32 channels stay in registers; more are
+                // walked three times in tensor memory (mean, variance about it, result).  Normalised values and outputs of 32
+                // channels leave with one hand-over.
+                const long long px = ((long long)n * a.Hr + y) * a.Wr + x;
+                const bool one = a.N == 32;
+                float v[32];
                 float sum = 0.f, sq = 0.f;
-                for (int c0 = 0; c0 < a.N; c0 += 32) {
-                    float v[32];
+                auto load = [&](int c0) {
                     tmem_ld32(lane_base + (uint32_t)c0, v);
 #pragma unroll
-                    for (int i = 0; i < 32; ++i) sum += v[i] + pipe->bias[c0 + i];
+                    for (int i = 0; i < 32; ++i) v[i] += pipe->bias[c0 + i];
+                };
+                for (int c0 = 0; c0 < a.N; c0 += 32) {
+                    load(c0);
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) sum += v[i];
                 }
                 const float mean = sum / (float)a.N;
                 for (int c0 = 0; c0 < a.N; c0 += 32) {
-                    float v[32];
-                    tmem_ld32(lane_base + (uint32_t)c0, v);
+                    if (!one) load(c0);
 #pragma unroll
                     for (int i = 0; i < 32; ++i) {
-                        const float d = v[i] + pipe->bias[c0 + i] - mean;
-                        sq += d * d;
+                        v[i] -= mean;
+                        sq += v[i] * v[i];
                     }
                 }
                 const float rs = rsqrtf(sq / (float)a.N + kLnEps);
-                const long long px = ((long long)n * a.Hr + y) * a.Wr + x;
-                if (live && h == 0) a.ln_rstd[px] = rs;
+                if (live) a.ln_rstd[px] = rs;
 #pragma unroll 1
-                for (int s = 0; s < nsteps; ++s) {
-                    if (s > 0) {
+                for (int c0 = 0; c0 < a.N; c0 += 32) {
+                    if (!one) {
+                        load(c0);
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) v[i] -= mean;
+                    }
+                    if (c0 + 32 == a.N) {
+                        tc_fence_before();
+                        mbar_arrive(&pipe->tempty[acc]);
+                    }
+                    if (c0 > 0) {
                         stage_free();
                         epi_sync<EPW>(eg);
                     }
                     const uint32_t stg = stg0 + (uint32_t)buf * a.stg_bytes;
-                    const int cb = s * 64 + h * 32;
-                    uint32_t keep[2][8];  // ReLU outputs of the sub-chunks, written after the normalised values have left
+                    uint32_t w = 0;
 #pragma unroll
-                    for (int j = 0; j < 2; ++j) {
-                        if (cb < a.N) {
-                            const int c0 = cb + 16 * j;
-                            float v[16];
-                            tmem_ld16(lane_base + (uint32_t)c0, v);
-                            uint32_t xh[8];
+                    for (int k = 0; k < 4; ++k) {
+                        uint32_t xh[4], rl[4];
 #pragma unroll
-                            for (int i = 0; i < 8; ++i) {
-                                const float x0 = (v[2 * i] + pipe->bias[c0 + 2 * i] - mean) * rs;
-                                const float x1 = (v[2 * i + 1] + pipe->bias[c0 + 2 * i + 1] - mean) * rs;
-                                xh[i] = pack_bf16x2(x0, x1);
-                                keep[j][i] = relu_pack_bf16x2(fmaf(pipe->gamma[c0 + 2 * i], x0, pipe->beta[c0 + 2 * i]),
-                                                              fmaf(pipe->gamma[c0 + 2 * i + 1], x1, pipe->beta[c0 + 2 * i + 1]));
-                            }
-                            if (cell) {
-                                put(stg, c0 & 63, make_uint4(xh[0], xh[1], xh[2], xh[3]));
-                                put(stg, (c0 & 63) + 8, make_uint4(xh[4], xh[5], xh[6], xh[7]));
-                            }
+                        for (int i = 0; i < 4; ++i) {
+                            const int c = 8 * k + 2 * i;
+                            const float x0 = v[c] * rs, x1 = v[c + 1] * rs;
+                            xh[i] = pack_bf16x2(x0, x1);
+                            rl[i] = relu_pack_bf16x2(fmaf(pipe->gamma[c0 + c], x0, pipe->beta[c0 + c]),
+                                                     fmaf(pipe->gamma[c0 + c + 1], x1, pipe->beta[c0 + c + 1]));
+                            w = gate_bits_add(w, rl[i], 4 * k + i);
+                        }
+                        if (cell) {
+                            put(stg, 8 * k, make_uint4(xh[0], xh[1], xh[2], xh[3]));
+                            put(stg, 32 + 8 * k, make_uint4(rl[0], rl[1], rl[2], rl[3]));
                         }
                     }
-                    if (s == nsteps - 1) {
-                        tc_fence_before();
-                        mbar_arrive(&pipe->tempty[acc]);
-                    }
-                    store_step(stg, s, &a.mapX);
-                    stage_free();
+                    if (a.out_bits && live) a.out_bits[px * (a.N >> 5) + (c0 >> 5)] = w;
+                    fence_async_smem();
                     epi_sync<EPW>(eg);
-                    const uint32_t stg2 = stg0 + (uint32_t)buf * a.stg_bytes;
-                    if (cb < a.N) {
-                        uint32_t w = 0;
-#pragma unroll
-                        for (int j = 0; j < 2; ++j) {
-                            if (cell) {
-                                put(stg2, ((cb + 16 * j) & 63), make_uint4(keep[j][0], keep[j][1], keep[j][2], keep[j][3]));
-                                put(stg2, ((cb + 16 * j) & 63) + 8, make_uint4(keep[j][4], keep[j][5], keep[j][6], keep[j][7]));
-                            }
-#pragma unroll
-                            for (int i = 0; i < 8; ++i) w = gate_bits_add(w, keep[j][i], 8 * j + i);
-                        }
-                        if (a.out_bits && live) a.out_bits[px * (a.N >> 5) + (cb >> 5)] = w;
+                    if (issuer) {
+                        tma_store_4d(&a.mapX, stg, c0, t.x, t.y, t.n);
+                        tma_store_4d(&a.mapO[0], stg + grp_bytes, c0, t.x, t.y, t.n);
+                        bulk_commit();
                     }
-                    store_step(stg2, s, &a.mapO[0]);
+                    if (++buf == a.nbuf) buf = 0;
                 }
                 acc += a.neg;
                 if (acc >= nacc) { acc = eg; aph ^= 1u; }
@@ -589,29 +531,29 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
             }
 #pragma unroll 1
             for (int s = 0; s < nsteps; ++s) {
-                const int c0 = s * 64 + h * 32;
-                const bool mine = c0 < a.N;  // uniform in a warp
-                float v[32];
-                if (mine) tmem_ld32(lane_base + (uint32_t)c0, v);
-                if (s == nsteps - 1) {  // the accumulator has been read by this warp
-                    tc_fence_before();
-                    mbar_arrive(&pipe->tempty[acc]);
-                }
                 if (s > 0) {
                     stage_free();
                     epi_sync<EPW>(eg);
                 }
                 const uint32_t stg = stg0 + (uint32_t)buf * a.stg_bytes;
-                if (MODE == FWD) {
-                    if (mine) {
+#pragma unroll
+                for (int q = 0; q < NH; ++q) {
+                    const int hh = EPW == 4 ? q : h, c0 = s * 64 + hh * 32;
+                    const bool mine = c0 < a.N;  // uniform in a warp
+                    float v[32];
+                    if (mine) tmem_ld32(lane_base + (uint32_t)c0, v);
+                    if (s == nsteps - 1 && q == NH - 1) {  // the accumulator has been read by this warp
+                        tc_fence_before();
+                        mbar_arrive(&pipe->tempty[acc]);
+                    }
+                    if (!mine) continue;
+                    if (MODE == FWD) {
                         const float4 *bp = reinterpret_cast<const float4 *>(pipe->bias + c0);
 #pragma unroll
                         for (int k = 0; k < 8; ++k) {
                             const float4 b4 = bp[k];
                             v[4 * k] += b4.x; v[4 * k + 1] += b4.y; v[4 * k + 2] += b4.z; v[4 * k + 3] += b4.w;
                         }
-                    }
-                    if (mine) {
                         uint32_t pk[16], w = 0;
 #pragma unroll
                         for (int j = 0; j < 16; ++j) {
@@ -620,28 +562,29 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
                         }
                         if (cell) {
 #pragma unroll
-                            for (int k = 0; k < 4; ++k) put(stg, h * 32 + 8 * k, make_uint4(pk[4 * k], pk[4 * k + 1], pk[4 * k + 2], pk[4 * k + 3]));
+                            for (int k = 0; k < 4; ++k) put(stg, hh * 32 + 8 * k, make_uint4(pk[4 * k], pk[4 * k + 1], pk[4 * k + 2], pk[4 * k + 3]));
                         }
                         if (a.out_bits && live) a.out_bits[(((long long)n * a.Hr + y) * a.Wr + x) * (a.N >> 5) + (c0 >> 5)] = w;
-                    }
-                } else if (MODE != FWD_LN && mine && cell) {
+                    } else if (cell) {
+                        const int gk = s * NH + q;
+                        const uint32_t gw = gk == 0 ? gate[0] : (gk == 1 ? gate[1] : (gk == 2 ? gate[2] : gate[3]));
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        uint32_t pk[4];
+                        for (int k = 0; k < 4; ++k) {
+                            uint32_t pk[4];
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const uint32_t pr = pack_bf16x2(v[8 * k + 2 * j], v[8 * k + 2 * j + 1]);
-                            if (MODE == DG_BITS) {
-                                const uint32_t gw = s == 0 ? gate[0] : (s == 1 ? gate[1] : (s == 2 ? gate[2] : gate[3]));
-                                pk[j] = pr & gate_mask(gw, 4 * k + j);
-                            } else {
-                                const uint4 &q4 = act[k];
-                                const uint32_t aw = j == 0 ? q4.x : (j == 1 ? q4.y : (j == 2 ? q4.z : q4.w));
-                                // stored activations are >= 0 (the outputs of a ReLU): a half gates unless it is zero
-                                pk[j] = pr & half_signs(aw + 0x7FFF7FFFu);
+                            for (int j = 0; j < 4; ++j) {
+                                const uint32_t pr = pack_bf16x2(v[8 * k + 2 * j], v[8 * k + 2 * j + 1]);
+                                if (MODE == DG_BITS) {
+                                    pk[j] = pr & gate_mask(gw, 4 * k + j);
+                                } else {
+                                    const uint4 &q4 = act[k];
+                                    const uint32_t aw = j == 0 ? q4.x : (j == 1 ? q4.y : (j == 2 ? q4.z : q4.w));
+                                    // stored activations are >= 0 (the outputs of a ReLU): a half gates unless it is zero
+                                    pk[j] = pr & half_signs(aw + 0x7FFF7FFFu);
+                                }
                             }
+                            put(stg, hh * 32 + 8 * k, make_uint4(pk[0], pk[1], pk[2], pk[3]));
                         }
-                        put(stg, h * 32 + 8 * k, make_uint4(pk[0], pk[1], pk[2], pk[3]));
                     }
                 }
                 store_step(stg, s, MODE == DG_BITS || MODE == DG_ACT ? a.mapO : &a.mapO[0]);
@@ -716,7 +659,7 @@ bool choose_tile(Args &a, int Wr, int Hr, int B, size_t room, int loads, int buf
 bool plan(Args &a, int Wr, int Hr, int B) {
     const size_t w = ((size_t)a.nchunks * a.w_chunk + 1023) & ~size_t(1023);
     const size_t fixed = w + sizeof(Pipe) + 1024 + 1024;  // alignment of the base and behind the slots
-    a.stg_row = a.narrow && !a.ln_gamma ? 64 : 128;  // narrow: 32 columns, normalised values beside the outputs
+    a.stg_row = a.N == 32 && !a.ln_gamma ? 64 : 128;  // 64 columns, or 32 and the normalised values beside the outputs
     a.acc_cols = 32;
     while (a.acc_cols < a.N) a.acc_cols *= 2;
     const size_t half = kSmemMax / 2 - 512;
@@ -725,7 +668,16 @@ bool plan(Args &a, int Wr, int Hr, int B) {
     for (int two = a.N <= 128 ? 1 : 0; two >= 0; --two) {
         const size_t room = two ? half : kSmemMax;
         if (fixed >= room) continue;
-        a.neg = (two ? 1 : 2) * (a.narrow ? 2 : 1);
+        // Four-warp groups (see the top of the file) cost a second staging buffer: worth it for the input gradient (32
+        // channels: 1.49 -> 1.29 ms), a single step of 32 columns and normalised rows; a plain forward tile of 64 columns and
+        // more wants the room for its next two planes (1.30 against 1.48 ms).
+        a.epw = a.ln_gamma || (two && (a.nloads != 4 || a.N == 32)) ? 4 : 8;
+        if (a.wide_gate) a.epw = 8;
+        a.nacc = (two ? 256 : 512) / a.acc_cols;
+        if (a.nacc > 4) a.nacc = 4;
+        if (a.nacc < 2) continue;
+        a.neg = two ? 8 / a.epw : 2;
+        if (a.neg > a.nacc) a.neg = a.nacc;  // a group has accumulators of its own
         const int least = a.nloads == 4 || two ? a.nloads : a.nloads + 1;
         if (!choose_tile(a, Wr, Hr, B, room - fixed, least, a.neg)) continue;
         if (two && a.tiles > best.tiles) continue;  // no smaller tile for the sake of a second CTA
@@ -738,9 +690,6 @@ bool plan(Args &a, int Wr, int Hr, int B) {
         a.slots = (int)((room - fixed - (size_t)(a.nbuf * a.neg) * a.stg_bytes) / a.slot_bytes);
         if (a.slots > kMaxSlots) a.slots = kMaxSlots;
         a.slots_bytes = ((uint32_t)a.slots * a.slot_bytes + 1023u) & ~1023u;
-        a.nacc = (two ? 256 : 512) / a.acc_cols;
-        if (a.nacc > 4) a.nacc = 4;
-        if (a.nacc < 2) continue;
         a.smem = a.slots_bytes + w + (size_t)(a.nbuf * a.neg) * a.stg_bytes + sizeof(Pipe) + 1024;
         const int ctas = ppo_num_sms() * (two ? 2 : 1);
         a.grid = a.tiles < ctas ? a.tiles : ctas;
@@ -749,33 +698,37 @@ bool plan(Args &a, int Wr, int Hr, int B) {
     return false;
 }
 
-template <int MODE, int GC, int KS, bool NARROW>
+template <int MODE, int GC, int KS, int EPW>
 int launch_one(const Args &a, cudaStream_t st) {
     static bool attr_set[64] = {false};
     int dev = 0;
     PPO_CUDA_CHECK(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64) return PPO_ERR_CUDA;
+    const auto fn = conv_halo_kernel<MODE, GC, KS, EPW>;
     if (!attr_set[dev]) {
-        PPO_CUDA_CHECK(cudaFuncSetAttribute(conv_halo_kernel<MODE, GC, KS, NARROW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+        PPO_CUDA_CHECK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
         attr_set[dev] = true;
     }
-    PPO_TRY(ppo_launch(conv_halo_kernel<MODE, GC, KS, NARROW>, dim3((unsigned)a.grid), dim3((2 + a.neg * kEpiWarps<NARROW>) * 32), a.smem, st, a));
-    return PPO_OK;
+    return ppo_launch(fn, dim3((unsigned)a.grid), dim3((2 + a.neg * EPW) * 32), a.smem, st, a);
 }
 
-template <int MODE, int GC, bool NARROW = false>
+template <int MODE, int GC, int EPW>
 int launch_ks(const Args &a, cudaStream_t st) {
     const int ks = a.CB >> 4;
-    if (ks == 4) return launch_one<MODE, GC, 4, NARROW>(a, st);
-    return ks == 2 ? launch_one<MODE, GC, 2, NARROW>(a, st) : launch_one<MODE, GC, 1, NARROW>(a, st);
+    if (ks == 4) return launch_one<MODE, GC, 4, EPW>(a, st);
+    return ks == 2 ? launch_one<MODE, GC, 2, EPW>(a, st) : launch_one<MODE, GC, 1, EPW>(a, st);
+}
+
+template <int MODE, int GC>
+int launch_epw(const Args &a, cudaStream_t st) {
+    return a.epw == 4 ? launch_ks<MODE, GC, 4>(a, st) : launch_ks<MODE, GC, 8>(a, st);
 }
 
 int launch(const Args &a, int mode, int GC, cudaStream_t st) {
-    if (mode == FWD && a.narrow) return launch_ks<FWD, 32, true>(a, st);
-    if (mode == FWD) return GC == 64 ? launch_ks<FWD, 64>(a, st) : launch_ks<FWD, 32>(a, st);
-    if (mode == FWD_LN) return a.narrow ? launch_ks<FWD_LN, 32, true>(a, st) : launch_ks<FWD_LN, 64>(a, st);  // a power of two
-    if (mode == DG_BITS) return GC == 64 ? launch_ks<DG_BITS, 64>(a, st) : launch_ks<DG_BITS, 32>(a, st);
-    return launch_ks<DG_ACT, 16>(a, st);
+    if (mode == FWD) return GC == 64 ? launch_epw<FWD, 64>(a, st) : launch_epw<FWD, 32>(a, st);
+    if (mode == FWD_LN) return launch_ks<FWD_LN, 32, 4>(a, st);
+    if (mode == DG_BITS) return GC == 64 ? launch_epw<DG_BITS, 64>(a, st) : launch_epw<DG_BITS, 32>(a, st);
+    return launch_ks<DG_ACT, 16, 8>(a, st);
 }
 
 // Channels per chunk of a C-channel source, or 0.
@@ -798,8 +751,6 @@ int halo_conv_fwd(const ConvGeom &g, const bf16 *X, const bf16 *W, const FwdEpil
     a.w_box = (uint32_t)(g.Co * a.rb);
     a.w_chunk = 9u * a.w_box;
     a.ln_gamma = e.ln_gamma;
-    a.narrow = g.Co == 32;
-    if (e.ln_gamma && (g.Co & (g.Co - 1)) != 0) return PPO_ERR_UNSUPPORTED;
     if (!plan(a, g.Wo, g.Ho, g.B)) return PPO_ERR_UNSUPPORTED;
     for (int p = 0; p < 4; ++p) {
         const int py = p >> 1, px = p & 1;
@@ -828,7 +779,7 @@ int halo_conv_fwd(const ConvGeom &g, const bf16 *X, const bf16 *W, const FwdEpil
         const int s = make_map_strided(&a.mapW, W, 2, dims, str, box);
         if (s != PPO_OK) return s;
     }
-    const int GC = g.Co % 64 == 0 ? 64 : 32;
+    const int GC = g.Co % 64 == 0 && !e.ln_gamma ? 64 : 32;
     const long long dims[4] = {g.Co, g.Wo, g.Ho, g.B};
     const long long str[3] = {2ll * g.Co, 2ll * g.Wo * g.Co, 2ll * g.Ho * g.Wo * g.Co};
     const int box[4] = {GC, a.Wt, a.R, a.I};
@@ -864,6 +815,7 @@ static bool plan_dgrad(Args &a, const ConvGeom &g, int ldy, int wt_ld, const Dgr
     a.nloads = a.nchunks;
     a.w_box = (uint32_t)(g.Ci * a.rb);
     a.w_chunk = 9u * a.w_box;
+    a.wide_gate = g.Ci == 16;
     return a.nchunks <= kMaxSlots && plan(a, (g.Wi + 1) / 2, (g.Hi + 1) / 2, g.B);
 }
 
