@@ -274,6 +274,10 @@ int ppo_model_set_sequence(ppo_model *m, int T, int Be, const uint8_t *dev_done,
  * was announced, or a model without LSTM layers -> STATE. */
 int ppo_model_read_state(const ppo_model *m, float *dev_h_out, float *dev_c_out, void *stream);
 
+/* Rows of a carried recurrent state (dev_h, dev_c fp32 [layers][n][H], as ppo_model_read_state writes them) whose env has
+ * ended (dev_done uint8 [n], != 0) <- 0, between two rollout steps. */
+int ppo_state_reset(float *dev_h, float *dev_c, const uint8_t *dev_done, int layers, int n, int H, void *stream);
+
 /* shadow <- bf16(master) (round to nearest even); call after writing master from outside. */
 int ppo_model_sync_shadow(ppo_model *m, void *stream);
 

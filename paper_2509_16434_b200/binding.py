@@ -29,7 +29,7 @@ EXPORTS = [
     "ppo_adam_step", "ppo_policy_sample", "ppo_poll_status", "ppo_model_activation_ptr", "ppo_gae_static",
     "ppo_model_sync_masks", "ppo_buffer_write_obs", "ppo_buffer_write_outcome", "ppo_policy_act", "ppo_launch_count",
     "ppo_selftest_wait_timeout", "ppo_buffer_render_depth", "ppo_model_set_sequence", "ppo_shuffle_gather_sequences",
-    "ppo_model_read_state",
+    "ppo_model_read_state", "ppo_state_reset",
 ]
 
 
@@ -112,6 +112,7 @@ def lib():
         L.ppo_shuffle_gather_sequences.argtypes = [C.c_void_p, C.c_uint64, C.c_uint32, C.c_int, C.c_int,
                                                    C.POINTER(Minibatch), C.c_void_p, C.c_void_p]
         L.ppo_model_read_state.argtypes = [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]
+        L.ppo_state_reset.argtypes = [C.c_void_p] * 3 + [C.c_int] * 3 + [C.c_void_p]
         L.ppo_launch_count.restype = C.c_uint64
         L.ppo_launch_count.argtypes = []
         L.ppo_selftest_wait_timeout.argtypes = [C.c_longlong, C.c_void_p, C.c_void_p]
@@ -362,6 +363,12 @@ def ppo_model_set_sequence(m: Model, T: int, Be: int, done, h_init, c_init):
 def ppo_model_read_state(m: Model, h_out, c_out, stream=None):
     """fp32 [n_lstm,Be,lstm_h] each: the state after the last step of the latest forward, zero where that step was done."""
     _check(lib().ppo_model_read_state(m.handle, _ptr(h_out), _ptr(c_out), _stream(stream)), "ppo_model_read_state")
+
+
+def ppo_state_reset(h, c, done, stream=None):
+    """h, c fp32 [layers,n,H], done uint8 [n]: zeroes the state rows of the envs whose flag is set."""
+    _check(lib().ppo_state_reset(_ptr(h), _ptr(c), _ptr(done), h.shape[0], h.shape[1], h.shape[2], _stream(stream)),
+           "ppo_state_reset")
 
 
 def ppo_shuffle_gather_sequences(buf: Buffer, seed: int, epoch: int, mb_index: int, num_minibatches: int,

@@ -667,6 +667,25 @@ __global__ void __launch_bounds__(256) concat_proprio_kernel(const float *__rest
     h0[(size_t)b * ld + E + j] = __float2bfloat16_rn(proprio[i]);
 }
 
+// h0[b] = [ReLU(bias + the slabs' partial products in order), proprio[b]] as bf16: second stage of a split embedding.
+__global__ void __launch_bounds__(256) embed_finish_kernel(const float *__restrict__ part, int slabs, const float *__restrict__ bias,
+                                                           const float *__restrict__ proprio, bf16 *__restrict__ h0, int rows,
+                                                           int E, int P) {
+    grid_wait();
+    const int ld = E + P, i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= rows * ld) return;
+    const int b = i / ld, j = i - b * ld;
+    float v;
+    if (j < E) {
+        v = bias[j];
+        for (int s = 0; s < slabs; ++s) v += part[((size_t)s * rows + b) * E + j];
+        v = fmaxf(v, 0.f);
+    } else {
+        v = proprio[(size_t)b * P + j - E];
+    }
+    h0[i] = __float2bfloat16_rn(v);
+}
+
 // dz[b][e] = dh0[b][e] where the embedding h0[b][e] is > 0, else 0 (back through its ReLU), as a bf16 GEMM operand.
 __global__ void __launch_bounds__(256) embed_dz_kernel(const float *__restrict__ dh0, const bf16 *__restrict__ h0,
                                                        bf16 *__restrict__ dz, int rows, int E, int ld) {
@@ -1163,12 +1182,27 @@ extern "C" int ppo_encoder_fwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
     }
     if (m->ti_embed >= 0) {
         // flatten -> fully connected -> ReLU into the first E columns of h_0, proprio behind them
-        ConvGeom g = fc_geom(rows, m->Hs[m->L] * m->Ws[m->L] * m->Cs[m->L], d.embed);
+        const int K = m->Hs[m->L] * m->Ws[m->L] * m->Cs[m->L];
+        ConvGeom g = fc_geom(rows, K, d.embed);
+        // Acting (one step, no gradients to follow) on few rows: the long reduction of a handful of tiles is the longest link
+        // of a decision, so it is cut into slabs that as many CTAs work on (K = 10240, 16 rows: 26 -> 8 us).  Sequences
+        // keep the one sum: their passes are compared step by step.
+        const float *part = m->wg_part[m->ti_embed];
+        int slabs = 8;
+        while (slabs > 1 && K % (slabs * 64) != 0) slabs /= 2;
+        if ((m->acting || (d.n_lstm > 0 && m->seq_T == 1)) && slabs > 1 && K >= 2048 && rows <= 1024 &&
+            (size_t)slabs * rows * d.embed <= m->wg_cap[m->ti_embed]) {
+            PPO_TRY(gemm_nt_f32(m, rows, d.embed, K, m->act[m->L], K, m->shadow + m->tensors[m->ti_embed].off, m->wg_part[m->ti_embed],
+                                st, slabs));
+            PPO_TRY(ppo_launch(embed_finish_kernel, dim3(ppo_cdiv((long long)rows * m->hw[0], 256)), dim3(256), 0, st, part, slabs,
+                               m->master + m->tensors[m->ti_embed + 1].off, mb->proprio + (size_t)row0 * d.P, m->h[0], rows, d.embed, d.P));
+        } else {
         FwdEpilogue e = {m->master + m->tensors[m->ti_embed + 1].off, 1, m->h[0], nullptr, nullptr, 0};
         e.ldo = m->hw[0];
         PPO_TRY(run_fwd(m, g, m->act[m->L], m->shadow + m->tensors[m->ti_embed].off, e, st));
         PPO_TRY(ppo_launch(concat_proprio_kernel, dim3(ppo_cdiv((long long)rows * d.P, 256)), dim3(256), 0, st, mb->proprio + (size_t)row0 * d.P, m->h[0],
                                                                                   rows, d.embed, d.P, m->hw[0]));
+        }
     } else {
         PPO_TRY(ppo_launch(pool_concat_kernel, dim3(ppo_cdiv((long long)rows * (m->Cs[m->L] / 8 + d.P), 256)), dim3(256), 0, st, m->act[m->L], mb->proprio + (size_t)row0 * d.P, m->h[0], rows,
                                                               m->Hs[m->L] * m->Ws[m->L], m->Cs[m->L], d.P));

@@ -36,6 +36,7 @@ namespace {
 using namespace tc;
 
 constexpr int kMaxTaps = 49;
+constexpr int kMaxClasses = 8;
 constexpr int kMaxBoxes = 32;    // boxes per tile; rows per tile are capped at 32 so that this always holds
 constexpr int kMaxHeights = 32;  // one tensor map per box height 1 .. 32 rows (a copy costs ~100 cycles to issue,
                                  // so a tile is cut into as few boxes as the image boundaries allow)
@@ -202,7 +203,7 @@ struct KArgs {
     bf16 *ln_xhat;
     float *ln_rstd;
     int32_t *status;
-    KClass cls[4];
+    KClass cls[kMaxClasses];
 };
 
 struct PipeK {
@@ -1179,7 +1180,7 @@ int tma_gemm_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, i
         // Split reduction: the Co columns of dY are seen as an image of ks rows of Co / ks channels (row y of pixel x
         // starts at x * ldy + y * Co / ks), class s reads row s against the weight columns s * Co / ks .. and
         // leaves its product in its own copy of the output.
-        if (ks > 4 || g.Co % (ks * 64) != 0 || !e.out_f32 || e.out || e.mask_act) return PPO_ERR_UNSUPPORTED;
+        if (ks > kMaxClasses || g.Co % (ks * 64) != 0 || !e.out_f32 || e.out || e.mask_act) return PPO_ERR_UNSUPPORTED;
         const int Kc = g.Co / ks;
         a.kchunks = Kc / CB;
         a.w_tap = Kc;

@@ -332,16 +332,21 @@ extern "C" int ppo_model_set_sequence(ppo_model *m, int T, int Be, const uint8_t
     return PPO_OK;
 }
 
-// h (bf16 -> fp32) and c of the last time step, zero where done: one thread per state element of a layer.
-__global__ void __launch_bounds__(256) lstm_read_state_kernel(const bf16 *__restrict__ h, const float *__restrict__ c,
-                                                              const uint8_t *__restrict__ done, float *__restrict__ h_out,
-                                                              float *__restrict__ c_out, int Be, int H) {
+struct LstmStates {
+    const bf16 *h[PPO_MAX_LSTM];
+    const float *c[PPO_MAX_LSTM];
+};
+
+// h (bf16 -> fp32) and c of the last time step, zero where done: one thread per state element, blockIdx.y is the layer.
+__global__ void __launch_bounds__(256) lstm_read_state_kernel(const __grid_constant__ LstmStates s, const uint8_t *__restrict__ done,
+                                                              float *__restrict__ h_out, float *__restrict__ c_out, int Be, int H) {
     grid_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= Be * H) return;
     const bool reset = done[i / H] != 0;
-    h_out[i] = reset ? 0.f : __bfloat162float(h[i]);
-    c_out[i] = reset ? 0.f : c[i];
+    const size_t o = (size_t)blockIdx.y * Be * H + i;
+    h_out[o] = reset ? 0.f : __bfloat162float(s.h[blockIdx.y][i]);
+    c_out[o] = reset ? 0.f : s.c[blockIdx.y][i];
 }
 
 extern "C" int ppo_model_read_state(const ppo_model *m, float *h_out, float *c_out, void *stream) {
@@ -349,12 +354,31 @@ extern "C" int ppo_model_read_state(const ppo_model *m, float *h_out, float *c_o
     if (m->d.n_lstm == 0 || !m->ws || m->seq_T <= 0 || !m->fwd_valid) return PPO_ERR_STATE;
     const int Be = m->seq_Be, H = m->d.lstm_h;
     const size_t last = (size_t)(m->seq_T - 1) * Be;
+    LstmStates s = {};
     for (int l = 0; l < m->d.n_lstm; ++l) {
-        PPO_TRY(ppo_launch(lstm_read_state_kernel, dim3(ppo_cdiv((long long)Be * H, 256)), dim3(256), 0, static_cast<cudaStream_t>(stream), 
-            m->lstm_hs[l] + last * H, m->lstm_c[l] + last * H, m->seq_done + last, h_out + (size_t)l * Be * H,
-            c_out + (size_t)l * Be * H, Be, H));
+        s.h[l] = m->lstm_hs[l] + last * H;
+        s.c[l] = m->lstm_c[l] + last * H;
     }
-    return PPO_OK;
+    return ppo_launch(lstm_read_state_kernel, dim3(ppo_cdiv((long long)Be * H, 256), m->d.n_lstm), dim3(256), 0,
+                      static_cast<cudaStream_t>(stream), s, m->seq_done + last, h_out, c_out, Be, H);
+}
+
+// State rows of the envs whose flag is set <- 0; blockIdx.y is the layer.
+__global__ void __launch_bounds__(256) state_reset_kernel(float *__restrict__ h, float *__restrict__ c,
+                                                          const uint8_t *__restrict__ done, int n, int H) {
+    grid_wait();
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n * H || done[i / H] == 0) return;
+    const size_t o = (size_t)blockIdx.y * n * H + i;
+    h[o] = 0.f;
+    c[o] = 0.f;
+}
+
+extern "C" int ppo_state_reset(float *h, float *c, const uint8_t *done, int layers, int n, int H, void *stream) {
+    if (!h || !c || !done || layers <= 0 || layers > PPO_MAX_LSTM || n <= 0 || H <= 0 || (long long)n * H >= (1ll << 31))
+        return PPO_ERR_INVALID_ARG;
+    return ppo_launch(state_reset_kernel, dim3(ppo_cdiv((long long)n * H, 256), layers), dim3(256), 0, static_cast<cudaStream_t>(stream), h,
+                      c, done, n, H);
 }
 
 extern "C" int ppo_model_sync_masks(ppo_model *m, int rows, void *stream) {
@@ -631,7 +655,9 @@ extern "C" int ppo_policy_act(ppo_model *m, ppo_buffer *b, int t, const float *e
     b->gae_valid = false;
     for (int r0 = 0; r0 < d.N; r0 += m->mbmax) {
         const int rows = d.N - r0 < m->mbmax ? d.N - r0 : m->mbmax;
+        m->acting = true;
         int s = ppo_encoder_fwd(m, &obs, r0, rows, m->act_mean, value + r0, stream);
+        m->acting = false;
         if (s != PPO_OK) return s;
         s = ppo_policy_sample(m, rows, m->act_mean, eps + (size_t)r0 * d.A, action + (size_t)r0 * d.A, logp + r0, stream);
         if (s != PPO_OK) return s;

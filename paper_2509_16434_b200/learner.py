@@ -114,9 +114,11 @@ class Learner:
             self.roll_c = torch.zeros_like(self.roll_h)
             self.roll_done = torch.zeros(n, dtype=torch.uint8, device=self.device)
         else:
-            ended = (done != 0).view(1, n, 1)
-            self.roll_h.masked_fill_(ended, 0.0)
-            self.roll_c.masked_fill_(ended, 0.0)
+            if done.dtype != torch.uint8 or not done.is_contiguous() or done.device != self.roll_h.device:
+                done = (done != 0).to(self.roll_h.device, torch.uint8).contiguous()
+            if done.numel() != n or self.roll_h.shape[1] != n:
+                raise ValueError("one done flag per env that carries a state")
+            ppo.ppo_state_reset(self.roll_h, self.roll_c, done)
 
     def act_into_buffer(self, t: int, depth: torch.Tensor, proprio: torch.Tensor, eps: torch.Tensor):
         """One rollout step without intermediate copies: the observation goes into slab row t, the policy reads
