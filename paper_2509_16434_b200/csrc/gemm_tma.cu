@@ -37,9 +37,7 @@ using namespace tc;
 
 constexpr int kMaxTaps = 49;
 constexpr int kMaxClasses = 8;
-constexpr int kMaxBoxes = 32;    // boxes per tile; rows per tile are capped at 32 so that this always holds
-constexpr int kMaxHeights = 32;  // one tensor map per box height 1 .. 32 rows (a copy costs ~100 cycles to issue,
-                                 // so a tile is cut into as few boxes as the image boundaries allow)
+constexpr int kMaxHeights = 32;  // one tensor map per box height 1 .. 32 rows: a tile is cut at image boundaries only
 constexpr int kMaxStages = 8;
 constexpr int kThreads = 192;    // warp 0: TMA producer, warp 1: MMA issue and TMEM owner, warps 2-5: epilogue
 constexpr size_t kSmemBudget = 200 * 1024;  // operand stages of the wgrad kernel
@@ -62,38 +60,13 @@ struct RowGrid {
     int arows;  // pixel rows a tile fills in shared memory: R * Wt
 };
 
-struct Box {
-    int n, y, x;  // image, first row, first pixel
-    int hl;       // box height in rows, minus one (index of its tensor map)
-    int rowoff;   // first shared-memory row of the box
-};
-
 struct Pipe {
     uint64_t full[kMaxStages];
     uint64_t empty[kMaxStages];
-    uint64_t tfull[2];
-    uint64_t tempty[2];
+    uint64_t tfull;
     uint32_t tmem_slot;
     int abort_flag;
-    int nboxes;
-    Box boxes[kMaxBoxes];
 };
-
-// Boxes of the pixel tile whose first grid row is row y of image n and whose first pixel is x0, in
-// shared-memory row order.  Rows past the last image get an image index >= Nimg, which the copy engine
-// answers with zeros.  Called by one thread.
-__host__ __device__ inline int build_boxes_at(const RowGrid &g, int n, int y, int x0, Box *out) {
-    int left = g.R, nb = 0, off = 0;
-    while (left > 0) {
-        int seg = g.Hr - y < left ? g.Hr - y : left;
-        left -= seg;
-        out[nb++] = {n, y, x0, seg - 1, off};
-        y += seg;
-        off += seg * g.Wt;
-        if (y >= g.Hr) { y = 0; ++n; }
-    }
-    return nb;
-}
 
 // First grid row (image n, row y) and x segment xs of pixel tile mt; advanced tile by tile without divisions
 // (a lone thread pays a hundred cycles and more for each).
@@ -118,12 +91,6 @@ struct PixTile {
         }
     }
 };
-
-__host__ __device__ inline int build_boxes(const RowGrid &g, int tile, Box *out) {
-    PixTile pt;
-    pt.init(g, tile);
-    return build_boxes_at(g, pt.n, pt.y, pt.xs * g.Wt, out);
-}
 
 // After a time-out: bounded wait for the copies of the last `S` armed stages (iterations it-S .. it-1).
 __device__ void drain_copies(uint64_t *full, int it, int S) {
@@ -183,7 +150,7 @@ struct KArgs {
     uint32_t a_bytes;       // room for a tile's A rows (the MMA reads 128; what lies behind belongs to rows nobody stores)
     int kchunks;            // boxes along the channels of one tap
     int w_tap;              // elements between taps in a weight row
-    int G, nbmax;           // sub-blocks per stage; most A boxes a tile has
+    int G;                  // sub-blocks per stage
     int tmem_cap;           // tensor-memory columns this CTA may take: 512, or 256 when two CTAs share an SM
     int nepi;               // epilogue warps: 8, or 16 where the epilogue is the heavier side (dgrad with gate bits)
     int wres, wtaps;        // weights resident in shared memory (all wtaps * kchunks boxes, loaded once)
@@ -214,8 +181,6 @@ struct PipeK {
     uint64_t wfull;
     uint32_t tmem_slot;
     int abort_flag;
-    int nboxes;
-    Box boxes[kMaxBoxes];
     alignas(16) float bias[kMaxBias];
     alignas(16) float gamma[256], beta[256];  // layer normalisation (N <= 256)
     // followed by the epilogue staging: per epilogue warp 32 rows x 32 bf16 columns (2 KB), 16-byte pieces swizzled
@@ -268,7 +233,7 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
     const uint32_t res_base = smem_base + (uint32_t)S * stage_bytes;
 
     if (warp == 0) {
-        // ---------------- TMA producer: the lanes share out the copies of a stage, one thread each
+        // ---------------- TMA producer
         if (a.wres) {
             const int nw = a.wtaps * a.kchunks;
             if (lane == 0) mbar_arrive_expect_tx(&pipe->wfull, (uint32_t)nw * b_bytes);
@@ -278,12 +243,7 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
                 tma_load_2d(res_base + (uint32_t)q * b_bytes, &a.mapB, &pipe->wfull, tap * a.w_tap + kc * a.CB, 0);
             }
         }
-        // Lane l owns copy j = l % lps of sub-block slot gi = l / lps of every stage (G * lps <= 32): its
-        // A box of the tile, or the weight rows.  Per stage a lane only advances (tap, chunk) and issues.
-        const int lps = a.nbmax + (a.wres ? 0 : 1);
-        const int gi = lane / lps, j = lane - gi * lps;
-        const bool lane_on = gi < G;
-        const bool is_b = !a.wres && j == a.nbmax;
+        // All lanes walk the tiles together, one elected lane issues (see tcgen05.cuh).
         const uint32_t tx_sub = (uint32_t)a.grid.arows * rb + (a.wres ? 0u : b_bytes);
         int it = 0, s = 0;
         uint32_t ph = 0;
@@ -292,41 +252,35 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
         tc_.init(a.total_tiles, a.tiles_n, a.ncls);
         PixTile pt;
         pt.init(a.grid, tc_.mt);
-        int last_mt = -1;
-        bool have = false;
-        Box bx = {0, 0, 0, 0, 0};
-        const int tap0 = gi / a.kchunks, kc0 = gi - tap0 * a.kchunks;
         for (; tc_.valid() && ok; tc_.next(a.tiles_n, a.ncls)) {
-            const int n0 = tc_.nt * BN;
             const KClass &k = a.cls[tc_.c];
-            if (tc_.mt != last_mt) {
-                last_mt = tc_.mt;
-                pt.advance_to(a.grid, tc_.mt);
-                if (lane == 0) pipe->nboxes = build_boxes_at(a.grid, pt.n, pt.y, pt.xs * a.grid.Wt, pipe->boxes);
-                __syncwarp();
-                have = lane_on && (is_b || j < pipe->nboxes);
-                if (have && !is_b) bx = pipe->boxes[j];
-                __syncwarp();
-            }
-            const uint32_t dst_off = (uint32_t)gi * sub_bytes + (is_b ? a_bytes : (uint32_t)bx.rowoff * rb);
-            const int cx = bx.x * a.s_mul + a.s_ox, cy = bx.y * a.s_mul + a.s_oy;
-            const void *map = is_b ? (const void *)&a.mapB : (const void *)&a.mapA[bx.hl];
-            const int ntaps = k.taps.n, nsub = ntaps * a.kchunks;
-            int tap = tap0, kc = kc0;
+            pt.advance_to(a.grid, tc_.mt);
+            const int brow = tc_.nt * BN + k.b_row0, ntaps = k.taps.n, nsub = ntaps * a.kchunks;
+            const int cx = pt.xs * a.grid.Wt * a.s_mul + a.s_ox;
+            int tap = 0, kc = 0;
             for (int q0 = 0; q0 < nsub; q0 += G, ++it) {
-                int okw = 1;
-                if (lane == 0) okw = mbar_wait(&pipe->empty[s], ph ^ 1u, abort_flag, a.status) ? 1 : 0;
-                ok = __shfl_sync(0xffffffffu, okw, 0) != 0;
+                ok = mbar_wait_warp(&pipe->empty[s], ph ^ 1u, abort_flag, a.status);
                 if (!ok) break;
-                if (lane == 0) mbar_arrive_expect_tx(&pipe->full[s], (uint32_t)min(G, nsub - q0) * tx_sub);
-                __syncwarp();
-                if (have && tap < ntaps) {
-                    const uint32_t dst = smem_base + (uint32_t)s * stage_bytes + dst_off;
-                    if (is_b) tma_load_2d(dst, map, &pipe->full[s], (int)k.taps.wt[tap] * a.w_tap + kc * a.CB, n0 + k.b_row0);
-                    else tma_load_4d(dst, map, &pipe->full[s], kc * a.CB, cx + k.taps.dx[tap], cy + k.taps.dy[tap], bx.n);
+                const int nval = min(G, nsub - q0);
+                if (elect_one()) mbar_arrive_expect_tx(&pipe->full[s], (uint32_t)nval * tx_sub);
+                uint32_t dst = smem_base + (uint32_t)s * stage_bytes;
+                for (int gi = 0; gi < nval; ++gi, dst += sub_bytes) {
+                    const int dx = k.taps.dx[tap], dy = k.taps.dy[tap];
+                    int n = pt.n, y = pt.y, row = 0;
+                    while (row < a.grid.R) {  // one box per image the tile touches
+                        const int seg = min(a.grid.Hr - y, a.grid.R - row);
+                        if (elect_one())
+                            tma_load_4d(dst + (uint32_t)(row * a.grid.Wt) * rb, &a.mapA[seg - 1], &pipe->full[s], kc * a.CB, cx + dx,
+                                        y * a.s_mul + a.s_oy + dy, n);
+                        row += seg;
+                        y += seg;
+                        if (y >= a.grid.Hr) { y = 0; ++n; }
+                    }
+                    if (!a.wres && elect_one())
+                        tma_load_2d(dst + a_bytes, &a.mapB, &pipe->full[s], (int)k.taps.wt[tap] * a.w_tap + kc * a.CB, brow);
+                    if (++kc == a.kchunks) { kc = 0; ++tap; }
                 }
-                kc += G;
-                while (kc >= a.kchunks) { kc -= a.kchunks; ++tap; }
+                __syncwarp();
                 if (++s == S) { s = 0; ph ^= 1u; }
             }
         }
@@ -637,7 +591,8 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
 // -------------------------------------------------------------------- wgrad ----
 
 struct WArgs {
-    CUtensorMap mapA[kMaxHeights];  // tap boxes of X (traversal stride 2 for a convolution)
+    CUtensorMap mapA[kMaxHeights];  // tap boxes of X (traversal stride 2 for a convolution; boxes over its four parity planes
+                                    // without one are 10 to 20 % slower)
     CUtensorMap mapB[kMaxHeights];  // boxes of dY over the same pixels
     RowGrid grid;                   // output pixels
     int s_mul, pad, ksz, ntaps;
@@ -671,7 +626,7 @@ __global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_con
             mbar_init(&pipe->full[s], 1);
             mbar_init(&pipe->empty[s], 1);
         }
-        mbar_init(&pipe->tfull[0], 1);
+        mbar_init(&pipe->tfull, 1);
         pipe->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -714,50 +669,43 @@ __global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_con
     const uint32_t tx_bytes = (uint32_t)a.grid.arows * ((uint32_t)nvalid * rbA + (uint32_t)a.nblocks * rbB);
 
     if (warp == 0) {
-        // ---------------- TMA producer: the lanes share out the copies of a K block, one thread each
-        // Lane l owns copy i = l % per_box (an A column block, then the B blocks) of box l / per_box of every
-        // pixel tile; tiles with more boxes than that go round again.
-        const int per_box = nvalid + a.nblocks;
-        const int b_l = lane / per_box, i_l = lane - b_l * per_box;
-        const int boxes_per_round = 32 / per_box;
-        int tap = 0, kc = 0, kh = 0, kw = 0;
-        if (i_l < nvalid) {
-            const int jb = jb0 + i_l;
-            tap = jb / a.kchunks;
-            kc = jb - tap * a.kchunks;
-            kh = tap / a.ksz;
-            kw = tap - kh * a.ksz;
-        }
-        const bool is_a = i_l < nvalid;
-        const uint32_t rbu = is_a ? rbA : rbB;
-        const uint32_t blk_off = is_a ? (uint32_t)i_l * 128u * rbA : a_bytes + (uint32_t)(i_l - nvalid) * 128u * rbB;
-        const int c0 = is_a ? kc * a.CB : co0 + (i_l - nvalid) * a.CBn;
-        const int mul = is_a ? a.s_mul : 1, ox = is_a ? kw - a.pad : 0, oy = is_a ? kh - a.pad : 0;
-        const CUtensorMap *maps = is_a ? a.mapA : a.mapB;
+        // ---------------- TMA producer: all lanes walk the tiles together, one elected lane issues.  (The copies of a
+        // stage shared out over the lanes cost about 100 cycles each: a divergent lane's operands are moved over one by
+        // one.)  Per image a tile touches there is one box for every A column block and for the B blocks.
+        const int tap0 = jb0 / a.kchunks, kc0 = jb0 - tap0 * a.kchunks, kh0 = tap0 / a.ksz, kw0 = tap0 - kh0 * a.ksz;
         bool ok = true;
         int kb = 0, s = 0;
         uint32_t ph = 0;
         PixTile pt;
         pt.init(a.grid, t_lo);
         for (; kb < nkb; ++kb) {
-            int okw = 1;
-            if (lane == 0) okw = mbar_wait(&pipe->empty[s], ph ^ 1u, abort_flag, a.status) ? 1 : 0;
-            ok = __shfl_sync(0xffffffffu, okw, 0) != 0;
+            pt.advance_to(a.grid, t_lo + kb);
+            const uint32_t st = smem_base + (uint32_t)s * stage_bytes;
+            const int x0 = pt.xs * a.grid.Wt;
+            ok = mbar_wait_warp(&pipe->empty[s], ph ^ 1u, abort_flag, a.status);
             if (!ok) break;
-            if (lane == 0) {
-                mbar_arrive_expect_tx(&pipe->full[s], tx_bytes);
-                pt.advance_to(a.grid, t_lo + kb);
-                pipe->nboxes = build_boxes_at(a.grid, pt.n, pt.y, pt.xs * a.grid.Wt, pipe->boxes);
-            }
-            __syncwarp();
-            const int nb = pipe->nboxes;
-            const uint32_t st = smem_base + (uint32_t)s * stage_bytes + blk_off;
-            if (b_l < boxes_per_round)
-                for (int b = b_l; b < nb; b += boxes_per_round) {
-                    const Box bx = pipe->boxes[b];
-                    tma_load_4d(st + (uint32_t)bx.rowoff * rbu, &maps[bx.hl], &pipe->full[s], c0, bx.x * mul + ox,
-                                bx.y * mul + oy, bx.n);
+            if (elect_one()) mbar_arrive_expect_tx(&pipe->full[s], tx_bytes);
+            int n = pt.n, y = pt.y, row = 0;
+            while (row < a.grid.R) {
+                const int seg = min(a.grid.Hr - y, a.grid.R - row);
+                const uint32_t off = (uint32_t)(row * a.grid.Wt);
+                const int cx = x0 * a.s_mul - a.pad, cy = y * a.s_mul - a.pad;
+                int kc = kc0, kh = kh0, kw = kw0;
+                for (int i = 0; i < nvalid; ++i) {
+                    if (elect_one())
+                        tma_load_4d(st + ((uint32_t)i * 128u + off) * rbA, &a.mapA[seg - 1], &pipe->full[s], kc * a.CB, cx + kw, cy + kh, n);
+                    if (++kc == a.kchunks) {
+                        kc = 0;
+                        if (++kw == a.ksz) { kw = 0; ++kh; }
+                    }
                 }
+                for (int i = 0; i < a.nblocks; ++i)
+                    if (elect_one())
+                        tma_load_4d(st + a_bytes + ((uint32_t)i * 128u + off) * rbB, &a.mapB[seg - 1], &pipe->full[s], co0 + i * a.CBn, x0, y, n);
+                row += seg;
+                y += seg;
+                if (y >= a.grid.Hr) { y = 0; ++n; }
+            }
             __syncwarp();
             if (++s == S) { s = 0; ph ^= 1u; }
         }
@@ -784,17 +732,18 @@ __global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_con
                 }
                 umma_commit(&pipe->empty[s]);
             }
+            accum = 1u;
             __syncwarp();
             if (++s == S) { s = 0; ph ^= 1u; }
         }
-        if (ok && nkb > 0 && elect_one()) umma_commit(&pipe->tfull[0]);
+        if (ok && nkb > 0 && elect_one()) umma_commit(&pipe->tfull);
         __syncwarp();
     } else if (nkb > 0) {
         // ---------------- epilogue: TMEM lane p is row p of this CTA's 128 x BN tile of dW^T; the whole tile goes
         // to the CTA's slot of the scratch array, column by column (a warp's store covers 32 consecutive rows)
         const int lg = warp & 3;
         const int p = lg * 32 + lane;
-        if (mbar_wait(&pipe->tfull[0], 0, abort_flag, a.status)) {
+        if (mbar_wait(&pipe->tfull, 0, abort_flag, a.status)) {
             tc_fence_after();
             float *tile = a.part + ((size_t)(blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * (size_t)(128 * BN);
             const uint32_t lane_base = tmem_d + ((uint32_t)(lg * 32) << 16);
@@ -911,7 +860,7 @@ bool make_grid(RowGrid &g, int Wr, int Hr, int Nimg, int row_bytes_min) {
         Wt = (Wt + wstep - 1) / wstep * wstep;
         if (Wt > 128) continue;
         int R = 128 / Wt;
-        if (R > kMaxBoxes) R = kMaxBoxes;
+        if (R > kMaxHeights) R = kMaxHeights;
         if (R > rows) R = (int)rows;
         const int xsegs = (Wr + Wt - 1) / Wt;
         const long long util = (long long)Wr * R * 1000 / ((long long)xsegs * 128);  // useful share of tile rows
@@ -995,20 +944,6 @@ int ensure_smem_attrs() {
     return PPO_OK;
 }
 
-// Most A boxes any tile of the grid is cut into (the cut repeats with the tile's first row modulo Hr).
-int max_boxes(const RowGrid &g) {
-    Box tmp[kMaxBoxes];
-    int mx = 1;
-    const int groups = g.tiles / g.xsegs;  // the cut depends on the row group only
-    const int lim = groups < g.Hr + 1 ? groups : g.Hr + 1;
-    for (int t = 0; t < lim; ++t) {
-        const int n = build_boxes(g, t * g.xsegs, tmp);
-        mx = n > mx ? n : mx;
-    }
-    const int n = build_boxes(g, g.tiles - 1, tmp);
-    return n > mx ? n : mx;
-}
-
 // `a.wtaps` = taps of the whole weight tensor (all classes).
 int launch_kmajor(KArgs &a, cudaStream_t st) {
     int s = ensure_smem_attrs();
@@ -1020,7 +955,6 @@ int launch_kmajor(KArgs &a, cudaStream_t st) {
     if (total <= 0) return PPO_OK;
     if (total > 0x7fffffffll) return PPO_ERR_UNSUPPORTED;
     a.total_tiles = (int)total;
-    a.nbmax = max_boxes(a.grid);
     const size_t b_bytes = (size_t)a.BN * a.row_bytes;
     const size_t res = (size_t)a.wtaps * a.kchunks * b_bytes;
     // resident weights only while they leave most of the shared memory to the A stages: the bytes in flight
@@ -1046,9 +980,6 @@ int launch_kmajor(KArgs &a, cudaStream_t st) {
     int G = (int)(((small_m ? 96 : 48) * 1024) / sub);  // sub-blocks per stage: fewer barrier round trips per byte
     G = G < 1 ? 1 : (G > 8 ? 8 : G);
     while (G > 1 && budget / (G * sub) < (small_m ? 2 : 3)) --G;
-    const int lps = a.nbmax + (a.wres ? 0 : 1);  // copies per sub-block; one producer lane each
-    if (lps > 32) return PPO_ERR_UNSUPPORTED;
-    while (G > 1 && G * lps > 32) --G;
     a.G = G;
     a.stages = (int)(budget / (G * sub));
     if (a.stages > kMaxStages) a.stages = kMaxStages;
