@@ -271,17 +271,18 @@ __global__ void __launch_bounds__(256) conv1_wgrad_mma_kernel(const __half *__re
     }
     const int d_oh = PX / Wo, d_ow = PX % Wo;  // 32 pixels further (Wo >= 1)
     constexpr int ZP = PX * C1 / 8 / 32;       // 16-byte pieces of the gradient tile per lane
-    uint4 xreg[TP / 8], zreg[ZP];
+    uint32_t raw[KW];                          // this lane's window, zero outside the frame
+    bool live = false;
+    uint4 zreg[ZP];
     // Loads of the tile that starts at pixel mt into registers; they are issued one trip ahead, so that their
     // latency overlaps the previous tile's MMAs.  The kernel is bound by its instructions as much as by HBM: a pair outside
     // the frame is a predicated load that leaves its zero, a full tile takes its gradient rows without tests.
     const int Wh = Wi >> 1;  // 32-bit words per frame row
     const uint32_t *const frames = reinterpret_cast<const uint32_t *>(depth);
     auto prefetch = [&](long long mt) {
-        const bool live = mt + lane < m_end;
+        live = mt + lane < m_end;
         const int pw0 = ow - (P + ODD) / 2, ih0 = 2 * oh - P;
         const uint32_t *row = frames + ((b * Hi + ih0) * Wh + pw0);
-        uint32_t raw[KW];
         bool cok[NP];
 #pragma unroll
         for (int q = 0; q < NP; ++q) cok[q] = live && (unsigned)(pw0 + q) < (unsigned)Wh;
@@ -306,22 +307,24 @@ __global__ void __launch_bounds__(256) conv1_wgrad_mma_kernel(const __half *__re
                 if (mt + i / (C1 / 8) < m_end) zreg[z] = __ldcs(reinterpret_cast<const uint4 *>(dZ + mt * C1) + i);
             }
         }
-        uint32_t wv[TP / 2];
-#pragma unroll
-        for (int k = 0; k < TP / 2; ++k) wv[k] = 0u;
-#pragma unroll
-        for (int k = 0; k < KW; ++k) {
-            const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&raw[k]));
-            wv[k] = pack_bf16x2(f.x, f.y);
-        }
-        if (live) wv[KW] = 0x00003F80u;  // (1.0, 0) as bf16: the bias-gradient column
-#pragma unroll
-        for (int c = 0; c < TP / 8; ++c) xreg[c] = make_uint4(wv[4 * c], wv[4 * c + 1], wv[4 * c + 2], wv[4 * c + 3]);
     };
     if (m0 < m_end) prefetch(m0);
     for (; m0 < m_end; m0 += PX) {
+        {   // conversion here, a trip after the loads were issued: at their side it would wait for them on the spot
+            uint32_t wv[TP / 2];
 #pragma unroll
-        for (int c = 0; c < TP / 8; ++c) *reinterpret_cast<uint4 *>(xs + lane * (TP * 2) + ((c ^ swz(lane, TP * 2)) * 16)) = xreg[c];
+            for (int k = 0; k < TP / 2; ++k) wv[k] = 0u;
+#pragma unroll
+            for (int k = 0; k < KW; ++k) {
+                const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&raw[k]));
+                wv[k] = pack_bf16x2(f.x, f.y);
+            }
+            if (live) wv[KW] = 0x00003F80u;  // (1.0, 0) as bf16: the bias-gradient column
+#pragma unroll
+            for (int c = 0; c < TP / 8; ++c)
+                *reinterpret_cast<uint4 *>(xs + lane * (TP * 2) + ((c ^ swz(lane, TP * 2)) * 16)) =
+                    make_uint4(wv[4 * c], wv[4 * c + 1], wv[4 * c + 2], wv[4 * c + 3]);
+        }
 #pragma unroll
         for (int z = 0; z < ZP; ++z) {
             const int i = lane + 32 * z, zr = i / (C1 / 8), zc = i % (C1 / 8);
