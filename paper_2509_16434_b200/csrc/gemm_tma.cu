@@ -766,7 +766,7 @@ __global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_con
 // dW[co][jj] += sum over the splits, in their order, of the partial tiles a split-K weight-gradient kernel left
 // in `part` ([split][column tile y][row tile x][BN][128]); threads past Co * Kfwd do the same for the bias gradient,
 // whose partial sums sit in row `ones_row` of dW^T (db == null: there is none).
-__global__ void __launch_bounds__(256) wgrad_reduce_kernel(const float *__restrict__ part, int jtiles, int ctiles,
+__global__ void __launch_bounds__(128) wgrad_reduce_kernel(const float *__restrict__ part, int jtiles, int ctiles,
                                                            int splits, int BN, int Kfwd, int Co, float *__restrict__ dW,
                                                            float *__restrict__ db, int ones_row) {
     grid_wait();
@@ -790,20 +790,14 @@ __global__ void __launch_bounds__(256) wgrad_reduce_kernel(const float *__restri
     const float *src = part + ((size_t)y * jtiles + x) * tile + (size_t)c * 128 + p;
     float acc = 0.f;
     int z = 0;
-    for (; z + 32 <= splits; z += 32) {  // the loads of 32 splits are in flight while the sum stays in order
-        float v[32];
+    for (; z + 16 <= splits; z += 16) {  // the loads of 16 splits are in flight while the sum stays in order
+        float v[16];
 #pragma unroll
-        for (int u = 0; u < 32; ++u) v[u] = src[(size_t)(z + u) * per_split];
+        for (int u = 0; u < 16; ++u) v[u] = src[(size_t)(z + u) * per_split];
 #pragma unroll
-        for (int u = 0; u < 32; ++u) acc += v[u];
+        for (int u = 0; u < 16; ++u) acc += v[u];
     }
-    for (; z + 8 <= splits; z += 8) {
-        float v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = src[(size_t)(z + u) * per_split];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) acc += v[u];
-    }
+#pragma unroll 8
     for (; z < splits; ++z) acc += src[(size_t)z * per_split];
     *dst += acc;
 }
@@ -1238,7 +1232,8 @@ int tma_dgrad_weights(const bf16 *W, bf16 *Wc, int Co, int k, int Ci, int wt_ld,
 int wgrad_reduce(const float *part, int jtiles, int ctiles, int splits, int BN, int Kfwd, int Co, float *dW, float *db,
                  int ones_row, cudaStream_t st) {
     const long long n = (long long)Co * Kfwd + (db ? Co : 0);
-    PPO_TRY(ppo_launch(wgrad_reduce_kernel, dim3(ppo_cdiv(n, 256)), dim3(256), 0, st, part, jtiles, ctiles, splits, BN, Kfwd, Co, dW, db, ones_row));
+    const int threads = n < 128 * ppo_num_sms() ? 32 : 128;  // few results: a warp each on more SMs
+    PPO_TRY(ppo_launch(wgrad_reduce_kernel, dim3(ppo_cdiv(n, threads)), dim3(threads), 0, st, part, jtiles, ctiles, splits, BN, Kfwd, Co, dW, db, ones_row));
     return PPO_OK;
 }
 

@@ -417,11 +417,19 @@ extern "C" int ppo_model_sync_shadow(ppo_model *m, void *stream) {
     return PPO_OK;
 }
 
+// (A memset node between two kernels would break the chain of overlapped launches.)
+__global__ void __launch_bounds__(256) zero_kernel(float4 *__restrict__ p, size_t n4) {
+    grid_wait();
+    const size_t nth = (size_t)gridDim.x * blockDim.x;
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += nth) p[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
 extern "C" int ppo_model_zero_grad(ppo_model *m, void *stream) {
     if (!m || !m->grad) return PPO_ERR_STATE;
-    PPO_CUDA_CHECK(cudaMemsetAsync(m->grad, 0, m->arena * sizeof(float), static_cast<cudaStream_t>(stream)));
-    ppo_count_launches(1);
-    return PPO_OK;
+    const size_t n4 = m->arena / 4;  // tensors start at multiples of 64 elements
+    const long long blocks = (long long)((n4 + 1023) / 1024), cap = (long long)ppo_num_sms() * 8;
+    return ppo_launch(zero_kernel, dim3((unsigned)(blocks < cap ? blocks : cap)), dim3(256), 0, static_cast<cudaStream_t>(stream),
+                      reinterpret_cast<float4 *>(m->grad), n4);
 }
 
 // -------------------------------------------------------------------- Adam ----
