@@ -1,9 +1,9 @@
 // TMA-fed tensor-core versions of the encoder's implicit GEMMs for sm_100a.
 //
-// One elected thread moves whole operand tiles with cp.async.bulk.tensor (TMA): a box of the NHWC
+// Elected threads move whole operand tiles with cp.async.bulk.tensor (TMA): a box of the NHWC
 // activation tensor with a traversal stride of 2 along W and H *is* the im2col tile of one kernel tap
 // of a stride-2 convolution, zero padding included (out-of-range parts of a box arrive as zeros), and
-// it lands in shared memory already in the swizzled image the UMMA descriptors name.  A second thread
+// it lands in shared memory already in the swizzled image the UMMA descriptors name.  Another thread
 // issues tcgen05.mma into a ring of accumulators in tensor memory; 8 or 16 warps read them back with
 // tcgen05.ld for the epilogue.  No thread computes an address per element.
 //
@@ -39,7 +39,7 @@ constexpr int kMaxTaps = 49;
 constexpr int kMaxClasses = 8;
 constexpr int kMaxHeights = 32;  // one tensor map per box height 1 .. 32 rows: a tile is cut at image boundaries only
 constexpr int kMaxStages = 8;
-constexpr int kThreads = 192;    // warp 0: TMA producer, warp 1: MMA issue and TMEM owner, warps 2-5: epilogue
+constexpr int kThreads = 160;    // wgrad: warp 0: MMA issue and TMEM owner, warps 1-4: TMA producers, then epilogue
 constexpr size_t kSmemBudget = 200 * 1024;  // operand stages of the wgrad kernel
 constexpr size_t kSmemMax = 227 * 1024;     // dynamic shared memory a CTA may ask for
 constexpr size_t kMaxResident = 64 * 1024;
@@ -92,9 +92,19 @@ struct PixTile {
     }
 };
 
-// After a time-out: bounded wait for the copies of the last `S` armed stages (iterations it-S .. it-1).
-__device__ void drain_copies(uint64_t *full, int it, int S) {
-    for (int i = max(0, it - S); i < it; ++i) {
+// Stages are dealt out over `np` producer warps, stage `it` to warp it % np.  A copy costs the warp that issues it 110 to
+// 220 cycles (its operands pass through uniform registers), which made a lone producer the bound of every GEMM with
+// several boxes per stage: 900 to 1900 cycles per stage where the copies take 500 to 750 and the MMAs 250 to 500.
+// Measured with 4096 images: weight gradient of 64 -> 128 channels over 15 x 20 pixels 330 -> 284 us, forward of 128 -> 256
+// over 8 x 10 181 -> 170 us, GEMMs of a few microseconds 5 to 10 % shorter.
+// There are never more producers than stages: a producer that waits for use u of a slot has seen everything up to
+// np + S stages back consumed, so the phase it waits for is the barrier's current or last one (np <= S), not an older
+// one of the same parity.
+// After a time-out: bounded wait of producer `first` for the stages it has armed (first, first + np, .. below it) and whose
+// copies may be in flight.
+__device__ void drain_copies(uint64_t *full, int it, int S, int first, int np) {
+    for (int i = first; i < it; i += np) {
+        if (i < it - S) continue;
         const long long t0 = clock64();
         while (!mbar_try_wait(&full[i % S], (i / S) & 1))
             if (clock64() - t0 > kWaitCycles / 4) break;
@@ -136,7 +146,8 @@ struct KClass {
 enum { EPI_FWD = 0, EPI_HEAD = 1, EPI_DGRAD = 2 };
 
 constexpr int kEpiWarps = 16;                     // at most: two or four warps per TMEM lane quarter share out the column groups
-constexpr int kKThreads = (2 + kEpiWarps) * 32;   // warp 0: TMA producer, warp 1: MMA issue and TMEM owner
+constexpr int kProducers = 3;                     // TMA producer warps at most: warp 0 and those behind the epilogue's
+constexpr int kKThreads = (1 + kProducers + kEpiWarps) * 32;  // warp 1: MMA issue and TMEM owner
 constexpr int kMaxBias = 512;
 
 // A pipeline stage carries G sub-blocks; sub-block q of a tile is (tap, channel chunk) = divmod(q, kchunks):
@@ -153,6 +164,7 @@ struct KArgs {
     int G;                  // sub-blocks per stage
     int tmem_cap;           // tensor-memory columns this CTA may take: 512, or 256 when two CTAs share an SM
     int nepi;               // epilogue warps: 8, or 16 where the epilogue is the heavier side (dgrad with gate bits)
+    int nprod;              // producer warps: 1 .. min(kProducers, stages)
     int wres, wtaps;        // weights resident in shared memory (all wtaps * kchunks boxes, loaded once)
     int N, BN, tiles_n, total_tiles, ncls, stages;  // tile g = ((mt * tiles_n) + nt) * ncls + class
     int Hout, Wout, ldo;
@@ -232,9 +244,10 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
     const uint32_t smem_base = smem_u32(smem);
     const uint32_t res_base = smem_base + (uint32_t)S * stage_bytes;
 
-    if (warp == 0) {
-        // ---------------- TMA producer
-        if (a.wres) {
+    if (warp == 0 || warp >= 2 + a.nepi) {
+        // ---------------- TMA producers
+        const int pw = warp == 0 ? 0 : warp - 1 - a.nepi, np = a.nprod;
+        if (a.wres && pw == 0) {
             const int nw = a.wtaps * a.kchunks;
             if (lane == 0) mbar_arrive_expect_tx(&pipe->wfull, (uint32_t)nw * b_bytes);
             __syncwarp();
@@ -245,7 +258,7 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
         }
         // All lanes walk the tiles together, one elected lane issues (see tcgen05.cuh).
         const uint32_t tx_sub = (uint32_t)a.grid.arows * rb + (a.wres ? 0u : b_bytes);
-        int it = 0, s = 0;
+        int it = pw, s = pw, it0 = 0;  // it, s: this warp's next stage of the whole run and its slot; it0: first of the tile
         uint32_t ph = 0;
         bool ok = true;
         TileCursor tc_;
@@ -257,8 +270,9 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
             pt.advance_to(a.grid, tc_.mt);
             const int brow = tc_.nt * BN + k.b_row0, ntaps = k.taps.n, nsub = ntaps * a.kchunks;
             const int cx = pt.xs * a.grid.Wt * a.s_mul + a.s_ox;
-            int tap = 0, kc = 0;
-            for (int q0 = 0; q0 < nsub; q0 += G, ++it) {
+            int tap = 0, kc = (it - it0) * G;
+            while (kc >= a.kchunks) { kc -= a.kchunks; ++tap; }
+            for (int q0 = (it - it0) * G; q0 < nsub; q0 += np * G, it += np) {
                 ok = mbar_wait_warp(&pipe->empty[s], ph ^ 1u, abort_flag, a.status);
                 if (!ok) break;
                 const int nval = min(G, nsub - q0);
@@ -281,10 +295,14 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
                     if (++kc == a.kchunks) { kc = 0; ++tap; }
                 }
                 __syncwarp();
-                if (++s == S) { s = 0; ph ^= 1u; }
+                s += np;
+                if (s >= S) { s -= S; ph ^= 1u; }
+                kc += (np - 1) * G;
+                while (kc >= a.kchunks) { kc -= a.kchunks; ++tap; }
             }
+            it0 += (nsub + G - 1) / G;
         }
-        if (!ok && lane == 0) drain_copies(pipe->full, it, S);
+        if (!ok && lane == 0) drain_copies(pipe->full, it, S, pw, np);
         __syncwarp();
     } else if (warp == 1) {
         // ---------------- MMA issue: one elected thread feeds the tensor core; the descriptors are built once and
@@ -623,7 +641,7 @@ __global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_con
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
-            mbar_init(&pipe->full[s], 1);
+            mbar_init(&pipe->full[s], 2);  // one arrival for each operand
             mbar_init(&pipe->empty[s], 1);
         }
         mbar_init(&pipe->tfull, 1);
@@ -650,7 +668,7 @@ __global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_con
         }
     }
     fence_async_smem();
-    if (warp == 1) tmem_alloc(&pipe->tmem_slot, ncols);
+    if (warp == 0) tmem_alloc(&pipe->tmem_slot, ncols);
     grid_wait();
     tc_fence_before();
     __syncthreads();
@@ -666,52 +684,8 @@ __global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_con
     int nvalid = 0;
     for (int i = 0; i < a.mblocks; ++i)
         if ((jb0 + i) / a.kchunks < a.ntaps) ++nvalid;
-    const uint32_t tx_bytes = (uint32_t)a.grid.arows * ((uint32_t)nvalid * rbA + (uint32_t)a.nblocks * rbB);
 
     if (warp == 0) {
-        // ---------------- TMA producer: all lanes walk the tiles together, one elected lane issues.  (The copies of a
-        // stage shared out over the lanes cost about 100 cycles each: a divergent lane's operands are moved over one by
-        // one.)  Per image a tile touches there is one box for every A column block and for the B blocks.
-        const int tap0 = jb0 / a.kchunks, kc0 = jb0 - tap0 * a.kchunks, kh0 = tap0 / a.ksz, kw0 = tap0 - kh0 * a.ksz;
-        bool ok = true;
-        int kb = 0, s = 0;
-        uint32_t ph = 0;
-        PixTile pt;
-        pt.init(a.grid, t_lo);
-        for (; kb < nkb; ++kb) {
-            pt.advance_to(a.grid, t_lo + kb);
-            const uint32_t st = smem_base + (uint32_t)s * stage_bytes;
-            const int x0 = pt.xs * a.grid.Wt;
-            ok = mbar_wait_warp(&pipe->empty[s], ph ^ 1u, abort_flag, a.status);
-            if (!ok) break;
-            if (elect_one()) mbar_arrive_expect_tx(&pipe->full[s], tx_bytes);
-            int n = pt.n, y = pt.y, row = 0;
-            while (row < a.grid.R) {
-                const int seg = min(a.grid.Hr - y, a.grid.R - row);
-                const uint32_t off = (uint32_t)(row * a.grid.Wt);
-                const int cx = x0 * a.s_mul - a.pad, cy = y * a.s_mul - a.pad;
-                int kc = kc0, kh = kh0, kw = kw0;
-                for (int i = 0; i < nvalid; ++i) {
-                    if (elect_one())
-                        tma_load_4d(st + ((uint32_t)i * 128u + off) * rbA, &a.mapA[seg - 1], &pipe->full[s], kc * a.CB, cx + kw, cy + kh, n);
-                    if (++kc == a.kchunks) {
-                        kc = 0;
-                        if (++kw == a.ksz) { kw = 0; ++kh; }
-                    }
-                }
-                for (int i = 0; i < a.nblocks; ++i)
-                    if (elect_one())
-                        tma_load_4d(st + a_bytes + ((uint32_t)i * 128u + off) * rbB, &a.mapB[seg - 1], &pipe->full[s], co0 + i * a.CBn, x0, y, n);
-                row += seg;
-                y += seg;
-                if (y >= a.grid.Hr) { y = 0; ++n; }
-            }
-            __syncwarp();
-            if (++s == S) { s = 0; ph ^= 1u; }
-        }
-        if (!ok && lane == 0) drain_copies(pipe->full, kb, S);
-        __syncwarp();
-    } else if (warp == 1) {
         const uint32_t idesc = instr_desc(128, BN, 1, 1);
         const uint64_t dA = smem_desc_sw(smem_base, 128u * rbA, 8u * rbA, rbA);
         const uint64_t dB = smem_desc_sw(smem_base + a_bytes, 128u * rbB, 8u * rbB, rbB);
@@ -738,12 +712,60 @@ __global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_con
         }
         if (ok && nkb > 0 && elect_one()) umma_commit(&pipe->tfull);
         __syncwarp();
-    } else if (nkb > 0) {
+    } else {
+        // ---------------- TMA producers: two warps for A and two for B, each with every second stage (S >= 2).  All lanes
+        // walk the tiles together, one elected lane issues.  (The copies of a stage shared out over the lanes cost more: a
+        // divergent lane's operands are moved over one by one.)  Per image a tile touches there is one box for every A
+        // column block and for every B block.
+        constexpr int NP = 2;
+        const int pw = (warp - 1) & 1;
+        const bool sideA = warp <= NP;
+        const uint32_t tx_bytes = (uint32_t)a.grid.arows * (sideA ? (uint32_t)nvalid * rbA : (uint32_t)a.nblocks * rbB);
+        const int tap0 = jb0 / a.kchunks, kc0 = jb0 - tap0 * a.kchunks, kh0 = tap0 / a.ksz, kw0 = tap0 - kh0 * a.ksz;
+        bool ok = true;
+        int kb = pw, s = pw;
+        uint32_t ph = 0;
+        PixTile pt;
+        pt.init(a.grid, t_lo);
+        for (; kb < nkb; kb += NP) {
+            pt.advance_to(a.grid, t_lo + kb);
+            const uint32_t st = smem_base + (uint32_t)s * stage_bytes;
+            const int x0 = pt.xs * a.grid.Wt;
+            ok = mbar_wait_warp(&pipe->empty[s], ph ^ 1u, abort_flag, a.status);
+            if (!ok) break;
+            if (elect_one()) mbar_arrive_expect_tx(&pipe->full[s], tx_bytes);
+            int n = pt.n, y = pt.y, row = 0;
+            while (row < a.grid.R) {
+                const int seg = min(a.grid.Hr - y, a.grid.R - row);
+                const uint32_t off = (uint32_t)(row * a.grid.Wt);
+                const int cx = x0 * a.s_mul - a.pad, cy = y * a.s_mul - a.pad;
+                int kc = kc0, kh = kh0, kw = kw0;
+                for (int i = 0; sideA && i < nvalid; ++i) {
+                    if (elect_one())
+                        tma_load_4d(st + ((uint32_t)i * 128u + off) * rbA, &a.mapA[seg - 1], &pipe->full[s], kc * a.CB, cx + kw, cy + kh, n);
+                    if (++kc == a.kchunks) {
+                        kc = 0;
+                        if (++kw == a.ksz) { kw = 0; ++kh; }
+                    }
+                }
+                for (int i = 0; !sideA && i < a.nblocks; ++i)
+                    if (elect_one())
+                        tma_load_4d(st + a_bytes + ((uint32_t)i * 128u + off) * rbB, &a.mapB[seg - 1], &pipe->full[s], co0 + i * a.CBn, x0, y, n);
+                row += seg;
+                y += seg;
+                if (y >= a.grid.Hr) { y = 0; ++n; }
+            }
+            __syncwarp();
+            s += NP;
+            if (s >= S) { s -= S; ph ^= 1u; }
+        }
+        if (!ok && lane == 0) drain_copies(pipe->full, kb, S, pw, NP);
+        __syncwarp();
         // ---------------- epilogue: TMEM lane p is row p of this CTA's 128 x BN tile of dW^T; the whole tile goes
         // to the CTA's slot of the scratch array, column by column (a warp's store covers 32 consecutive rows)
         const int lg = warp & 3;
         const int p = lg * 32 + lane;
-        if (mbar_wait(&pipe->tfull, 0, abort_flag, a.status)) {
+        if (nkb > 0 && ok && mbar_wait(&pipe->tfull, 0, abort_flag, a.status)) {
             tc_fence_after();
             float *tile = a.part + ((size_t)(blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * (size_t)(128 * BN);
             const uint32_t lane_base = tmem_d + ((uint32_t)(lg * 32) << 16);
@@ -757,7 +779,7 @@ __global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_con
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 1) {
+    if (warp == 0) {
         tc_fence_after();
         tmem_dealloc(tmem_d, ncols);
     }
@@ -978,11 +1000,13 @@ int launch_kmajor(KArgs &a, cudaStream_t st) {
     a.stages = (int)(budget / (G * sub));
     if (a.stages > kMaxStages) a.stages = kMaxStages;
     if (a.stages < 2) return PPO_ERR_UNSUPPORTED;
+    // (two CTAs per SM have a producer each; more would not leave 96 registers per thread)
+    a.nprod = two ? 1 : (a.stages < kProducers ? a.stages : kProducers);
     const int sms = ppo_num_sms();
     const long long ctas = two ? 2ll * sms : sms;
     const unsigned grid = (unsigned)(total < ctas ? total : ctas);
     const size_t smem = (size_t)a.stages * G * sub + (a.wres ? res : 0) + fixed;
-    PPO_TRY(ppo_launch(tma_kmajor_kernel, dim3(grid), dim3((2 + a.nepi) * 32), smem, st, a));
+    PPO_TRY(ppo_launch(tma_kmajor_kernel, dim3(grid), dim3((1 + a.nprod + a.nepi) * 32), smem, st, a));
     return PPO_OK;
 }
 
