@@ -146,7 +146,7 @@ struct KClass {
 enum { EPI_FWD = 0, EPI_HEAD = 1, EPI_DGRAD = 2 };
 
 constexpr int kEpiWarps = 16;                     // at most: two or four warps per TMEM lane quarter share out the column groups
-constexpr int kProducers = 3;                     // TMA producer warps at most: warp 0 and those behind the epilogue's
+constexpr int kProducers = 2;                     // TMA producer warps at most: warp 0 and those behind the epilogue's
 constexpr int kKThreads = (1 + kProducers + kEpiWarps) * 32;  // warp 1: MMA issue and TMEM owner
 constexpr int kMaxBias = 512;
 
@@ -297,8 +297,10 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
                 __syncwarp();
                 s += np;
                 if (s >= S) { s -= S; ph ^= 1u; }
-                kc += (np - 1) * G;
-                while (kc >= a.kchunks) { kc -= a.kchunks; ++tap; }
+                if (np > 1) {
+                    kc += (np - 1) * G;
+                    while (kc >= a.kchunks) { kc -= a.kchunks; ++tap; }
+                }
             }
             it0 += (nsub + G - 1) / G;
         }
@@ -1000,8 +1002,7 @@ int launch_kmajor(KArgs &a, cudaStream_t st) {
     a.stages = (int)(budget / (G * sub));
     if (a.stages > kMaxStages) a.stages = kMaxStages;
     if (a.stages < 2) return PPO_ERR_UNSUPPORTED;
-    // (two CTAs per SM have a producer each; more would not leave 96 registers per thread)
-    a.nprod = two ? 1 : (a.stages < kProducers ? a.stages : kProducers);
+    a.nprod = two || a.ncls > 1 ? 1 : (a.stages < kProducers ? a.stages : kProducers);
     const int sms = ppo_num_sms();
     const long long ctas = two ? 2ll * sms : sms;
     const unsigned grid = (unsigned)(total < ctas ? total : ctas);

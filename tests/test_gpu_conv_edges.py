@@ -26,6 +26,7 @@ NETS = {
     "small_images": _net("small_images", 14, 18, (32, 64, 64, 64), (3, 3, 3, 3), N=14, T=3),
     "one_block": _net("one_block", 8, 8, (16, 32, 64), (3, 3, 3), N=2),
     "tall_kernels": _net("tall_kernels", 40, 44, (32, 64, 96), (3, 5, 3)),
+    "many_chunks": _net("many_chunks", 20, 26, (32, 128, 256), (3, 3, 3), N=10, T=3),
     "ln_odd": _net("ln_odd", 35, 54, (16, 32, 64, 128), (3, 3, 3, 3), norm=True, embed=32),
     "ln_32": _net("ln_32", 22, 30, (32, 32, 64), (5, 3, 3), norm=True),
 }

@@ -1,0 +1,60 @@
+"""Recurrent layers as one kernel per direction at the edges of their tiles (128 envs, 16 units per CTA), the step-by-step
+path where not all CTAs fit the GPU, and what acting does differently: the embedding in slabs and the state reset."""
+import numpy as np
+import pytest
+import torch
+
+import test_gpu_lstm as base
+from helpers import oracle_model, rel_l2
+from oracle import oracle as orc
+from paper_2509_16434_b200 import synth
+from test_gpu_learner import ENC_TOL
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+# envs per sequence group, units, steps: one env, one short / exact / one over a tile, three tiles, too many CTAs
+@pytest.mark.parametrize("Be,H,T", [(1, 64, 3), (127, 64, 3), (128, 192, 4), (129, 128, 3), (257, 448, 3), (257, 1024, 3)])
+def test_sequences_at_tile_edges_match_oracle(Be, H, T, monkeypatch):
+    w = synth.Workload("edge", 2 * Be, T, 8, 12, (16, 32), (3, 3), (24,), 1, 2, P=32, A=3, n_lstm=2, lstm_h=H)
+    monkeypatch.setitem(base.REC, "edge", w)
+    base.test_forward_through_time_matches_oracle("edge", False)
+    base.test_backward_through_time_matches_oracle_on_identical_state("edge")
+
+
+# 1024 rows and fewer take the embedding (4096 inputs) in slabs, one more does not
+@pytest.mark.parametrize("n_lstm", [0, 1])
+@pytest.mark.parametrize("n", [1, 65, 1024, 1025])
+def test_acting_matches_oracle(n, n_lstm):
+    w = synth.Workload("act", n, 1, 64, 64, (16, 32, 64), (3, 3, 3), (40,), 1, 1, P=32, A=3, embed=32, n_lstm=n_lstm, lstm_h=64)
+    md = oracle_model(w)
+    lay = orc.param_layout(md)
+    theta = synth.init_params(lay.total, lay.offsets, lay.shapes, 3)
+    roll = synth.rollout_numpy(w, 3)
+    L = base.Learner(w, n, DEV)
+    L.model.load(theta)
+    dev = {k: torch.as_tensor(v).to(DEV) for k, v in roll.items()}
+    used = orc.round_weights(md, theta)
+    if n_lstm:
+        zero = np.zeros((n_lstm, n, 64), np.float32)
+        mu, V, _, _ = orc.encoder_fwd_seq(md, used, roll["depth"], roll["proprio"], roll["done"], zero, zero, True)
+        a, lp, val = L.act(dev["depth"][0], dev["proprio"][0], dev["eps"][0])
+    else:
+        mu, V, _ = orc.encoder_fwd(md, used, roll["depth"][0], roll["proprio"][0], True)
+        L.act_into_buffer(0, dev["depth"][0], dev["proprio"][0], dev["eps"][0])
+        a, lp, val = (L.buffer.field(f)[0] for f in (base.ppo.FIELD_ACTION, base.ppo.FIELD_LOGP, base.ppo.FIELD_VALUE))
+    ls = np.asarray(theta, np.float64)[lay.offsets[-1]:lay.offsets[-1] + md.A]
+    want, lp_want = orc.sample_action(mu, ls, roll["eps"].reshape(n, md.A))
+    assert base.ppo.ppo_poll_status() == 0
+    assert rel_l2(a.cpu().numpy(), want) <= ENC_TOL and rel_l2(val.cpu().numpy(), V) <= ENC_TOL
+    assert rel_l2(lp.cpu().numpy(), lp_want) <= ENC_TOL
+
+
+@pytest.mark.parametrize("layers,n,H", [(1, 1, 64), (2, 33, 64), (2, 300, 1024)])
+def test_state_reset_clears_finished_envs_only(layers, n, H):
+    h, c = (torch.randn((layers, n, H), device=DEV) for _ in range(2))
+    done = (torch.arange(n, device=DEV) % 3 == 0).to(torch.uint8) * 7  # any non-zero flag
+    want = [torch.where(done[None, :, None] != 0, torch.zeros_like(s), s) for s in (h, c)]
+    base.ppo.ppo_state_reset(h, c, done)
+    assert torch.equal(h, want[0]) and torch.equal(c, want[1])
