@@ -33,11 +33,11 @@ sys.path.insert(0, ROOT)
 # sample row, from ncu captures of small twins of the workloads (traffic grows in proportion to the rows): workload
 # -> (bytes per row, capture).  An entry is dropped (traffic: null) as soon as a kernel it covers changes.
 NCU_DRAM_BYTES_PER_ROW = {
-    "cfg2": (2.7490e6, "ncu capture of cfg2_prof at 512 rows, scaled by rows: profiles/ncu_main_kernels_cfg2_prof.md"),
-    "cfg3": (2.7490e6, "ncu capture of cfg2_prof at 512 rows, scaled by rows: profiles/ncu_main_kernels_cfg2_prof.md"),
-    "cfg2_prof": (2.7490e6, "ncu capture of cfg2_prof at 512 rows: profiles/ncu_main_kernels_cfg2_prof.md"),
-    "cfg4": (11.4461e6, "ncu capture of cfg4_prof at 128 rows, scaled by rows: profiles/ncu_main_kernels_cfg4_prof.md"),
-    "cfg4_prof": (11.4461e6, "ncu capture of cfg4_prof at 128 rows: profiles/ncu_main_kernels_cfg4_prof.md"),
+    "cfg2": (2.5673e6, "ncu capture of cfg2_prof at 512 rows, scaled by rows: profiles/ncu_main_kernels_cfg2_prof.md"),
+    "cfg3": (2.5673e6, "ncu capture of cfg2_prof at 512 rows, scaled by rows: profiles/ncu_main_kernels_cfg2_prof.md"),
+    "cfg2_prof": (2.5673e6, "ncu capture of cfg2_prof at 512 rows: profiles/ncu_main_kernels_cfg2_prof.md"),
+    "cfg4": (10.9533e6, "ncu capture of cfg4_prof at 128 rows, scaled by rows: profiles/ncu_main_kernels_cfg4_prof.md"),
+    "cfg4_prof": (10.9533e6, "ncu capture of cfg4_prof at 128 rows: profiles/ncu_main_kernels_cfg4_prof.md"),
 }
 METRIC = "ppo_learner_env_steps_trained_per_sec"
 UNIT = "env-steps/s"
@@ -366,7 +366,7 @@ def run_ours(args):
         per_row, capture = NCU_DRAM_BYTES_PER_ROW.get(w.name, (None, "no ncu capture of the current kernels at this workload"))
         traffic = per_row * mean_rows if per_row else None
         roofline = {"bound": "tensor",
-                    "kernel": "ppo_encoder_fwd + ppo_encoder_bwd: tma_kmajor_kernel / tma_wgrad_kernel (tcgen05 implicit GEMMs) "
+                    "kernel": "ppo_encoder_fwd + ppo_encoder_bwd: conv_halo_kernel / tma_kmajor_kernel / tma_wgrad_kernel (tcgen05 implicit GEMMs) "
                               "+ conv1 kernels; flops, time and traffic per call pair",
                     "achieved": round(enc_tf, 2), "peak": peak_tf, "unit": "TFLOP/s",
                     "frac": round(enc_tf / peak_tf, 4), "traffic": traffic, "traffic_source": capture,
