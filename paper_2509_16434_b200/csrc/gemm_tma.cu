@@ -978,9 +978,9 @@ int launch_kmajor(KArgs &a, cudaStream_t st) {
     // resident weights only while they leave most of the shared memory to the A stages: the bytes in flight
     // are what hides the copy latency
     a.wres = (a.tiles_n == 1 && a.ncls == 1 && res <= kMaxResident) ? 1 : 0;
-    // Narrow tiles (BN <= 128) leave the tensor pipe mostly idle because one thread per CTA cannot issue MMAs
-    // fast enough; two CTAs per SM (half the shared and tensor memory each, 8 epilogue warps each) double the
-    // issue rate.  Wide tiles run at the tensor rate with one CTA and keep the SM to themselves.
+    // Narrow tiles (BN <= 128): a tile's copies, MMAs and epilogue are of like length, and two CTAs per SM (half the shared
+    // and tensor memory each, 8 epilogue warps each) overlap them better than one with deeper stages (input gradient
+    // 256 -> 128 channels of 4096 images of 8 x 10: 260 us, with one CTA per SM 299).  Wide tiles keep the SM to themselves.
     // A GEMM of a few row tiles gives a CTA one or two tiles: nothing amortises the copy latency, so such a CTA takes the
     // SM alone, with stages of up to 96 KB (fewer, larger hand-overs), and the narrow-tile rule below does not apply.
     const bool flat = a.grid.Hr == 1 && a.grid.Nimg == 1;
