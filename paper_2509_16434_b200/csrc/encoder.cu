@@ -895,7 +895,7 @@ static int recorded(ppo_model *m, const PlanKey &key, cudaStream_t st, F &&make)
     return s;
 }
 
-enum { OP_FWD = 1, OP_DGRAD, OP_WGRAD, OP_LSTM_FWD, OP_LSTM_BWD };
+enum { OP_FWD = 1, OP_DGRAD, OP_WGRAD, OP_CONV_WGRADS, OP_LSTM_FWD, OP_LSTM_BWD };
 
 static PlanKey plan_key(int op, const ConvGeom &g) {
     PlanKey k;
@@ -950,23 +950,43 @@ static int run_colsum(const bf16 *dZ, int ld, long long M, int N, float *db, flo
 
 // Weight and bias gradients of the layer whose weight matrix is tensor ti.  The TMA kernel of a convolution sums
 // the bias gradient on the tensor core on its way; everything else reduces dY in a pass of its own.
-static int run_wgrad(ppo_model *m, int ti, const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *X,
-                     cudaStream_t st, bool with_bias = true) {
+static int make_wgrad(ppo_model *m, int ti, const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *X, cudaStream_t st,
+                      bool with_bias) {
     float *dW = m->grad + m->tensors[ti].off, *db = with_bias ? m->grad + m->tensors[ti + 1].off : nullptr;
     float *part = m->wg_part[ti];
     const size_t cap = m->wg_cap[ti];
     const bool conv = g.k > 1;
+    int s = tma_gemm_wgrad(g, dY, ldy, X, dW, conv ? db : nullptr, part, cap, ppo_device_status_ptr(), st);
+    if (s == PPO_OK && conv) return s;
+    if (s == PPO_ERR_UNSUPPORTED && conv) s = tma_gemm_wgrad(g, dY, ldy, X, dW, nullptr, part, cap, ppo_device_status_ptr(), st);
+    if (s == PPO_ERR_UNSUPPORTED) s = tc_gemm_wgrad(g, dY, ldy, X, dW, part, cap, ppo_device_status_ptr(), st);
+    if (s != PPO_OK || !with_bias) return s;
+    return run_colsum(dY, ldy, g.M(), g.Co, db, m->cs_part[ti], st);
+}
+
+static int run_wgrad(ppo_model *m, int ti, const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *X,
+                     cudaStream_t st, bool with_bias = true) {
     PlanKey key = plan_key(OP_WGRAD, g);
-    const void *p[] = {dY, X, dW, db, part};
+    const void *p[] = {dY, X, m->grad + m->tensors[ti].off, with_bias ? m->grad + m->tensors[ti + 1].off : nullptr, m->wg_part[ti]};
     memcpy(key.p, p, sizeof(p));
     key.v[0] = ldy; key.v[1] = with_bias;
+    return recorded(m, key, st, [&]() -> int { return make_wgrad(m, ti, g, dY, ldy, X, st, with_bias); });
+}
+
+// The weight gradients of all convolutions behind the first: the GEMMs one after the other (conv2 first: the longest), then
+// one reduction.
+static int run_conv_wgrads(ppo_model *m, int rows, cudaStream_t st) {
+    PlanKey key = plan_key(OP_CONV_WGRADS, conv_geom(m, 2, rows));
+    const void *p[] = {m->grad, m->act[1], m->dact[2], m->wg_part[m->ti_conv[2]]};  // one workspace: they move together
+    memcpy(key.p, p, sizeof(p));
     return recorded(m, key, st, [&]() -> int {
-        int s = tma_gemm_wgrad(g, dY, ldy, X, dW, conv ? db : nullptr, part, cap, ppo_device_status_ptr(), st);
-        if (s == PPO_OK && conv) return s;
-        if (s == PPO_ERR_UNSUPPORTED && conv) s = tma_gemm_wgrad(g, dY, ldy, X, dW, nullptr, part, cap, ppo_device_status_ptr(), st);
-        if (s == PPO_ERR_UNSUPPORTED) s = tc_gemm_wgrad(g, dY, ldy, X, dW, part, cap, ppo_device_status_ptr(), st);
-        if (s != PPO_OK || !with_bias) return s;
-        return run_colsum(dY, ldy, g.M(), g.Co, db, m->cs_part[ti], st);
+        return wgrad_batch([&]() -> int {
+            for (int l = 2; l <= m->L; ++l) {
+                const ConvGeom g = conv_geom(m, l, rows);
+                PPO_TRY(make_wgrad(m, m->ti_conv[l], g, m->dact[l], g.Co, m->act[l - 1], st, true));
+            }
+            return PPO_OK;
+        }, st);
     });
 }
 
@@ -1461,11 +1481,7 @@ extern "C" int ppo_encoder_bwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
     if (fork && L >= 2) {
         int s = fork_here();  // dZ1 is ready
         if (s == PPO_OK) s = conv1_wgrad(m, mb, row0, rows, leaf);
-        for (int l = 2; l <= L && s == PPO_OK; ++l) {  // conv2 first: the longest, and the best partner
-            const int ti = m->ti_conv[l];
-            ConvGeom g = conv_geom(m, l, rows);
-            s = run_wgrad(m, ti, g, m->dact[l], g.Co, m->act[l - 1], st);
-        }
+        if (s == PPO_OK) s = run_conv_wgrads(m, rows, st);
         return join(s);
     }
     return join(conv1_wgrad(m, mb, row0, rows, st));

@@ -5,6 +5,8 @@
 //   wgrad : dW[co][tap][ci] += sum_m dY[m][co] * X[b, 2oh+kh-p, 2ow+kw-p, ci]
 // m = (b, oh, ow) over output pixels, m' = (b, ih, iw) over input pixels; fp32 accumulation.
 #pragma once
+#include <functional>
+
 #include "common.cuh"
 
 struct FwdEpilogue {
@@ -71,6 +73,9 @@ int tma_dgrad_weights(const bf16 *W, bf16 *Wc, int Co, int k, int Ci, int wt_ld,
 int tma_gemm_wgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *X, float *dW, float *db, float *part,
                    size_t part_elems, int32_t *status, cudaStream_t st);
 size_t wgrad_scratch_elems(const ConvGeom &g);
+// Runs `gemms` (weight-gradient GEMMs on stream st, each with scratch of its own) and then one launch that adds the partial
+// tiles of all of them.
+int wgrad_batch(const std::function<int()> &gemms, cudaStream_t st);
 int wgrad_reduce(const float *part, int jtiles, int ctiles, int splits, int BN, int Kfwd, int Co, float *dW, float *db,
                  int ones_row, cudaStream_t st);
 

@@ -39,6 +39,7 @@ constexpr int kMaxTaps = 49;
 constexpr int kMaxClasses = 8;
 constexpr int kMaxHeights = 32;  // one tensor map per box height 1 .. 32 rows: a tile is cut at image boundaries only
 constexpr int kMaxStages = 8;
+constexpr int kMaxReduceJobs = 8;
 constexpr int kThreads = 160;    // wgrad: warp 0: MMA issue and TMEM owner, warps 1-4: TMA producers, then epilogue
 constexpr size_t kSmemBudget = 200 * 1024;  // operand stages of the wgrad kernel
 constexpr size_t kSmemMax = 227 * 1024;     // dynamic shared memory a CTA may ask for
@@ -789,29 +790,45 @@ __global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_con
 
 // dW[co][jj] += sum over the splits, in their order, of the partial tiles a split-K weight-gradient kernel left
 // in `part` ([split][column tile y][row tile x][BN][128]); threads past Co * Kfwd do the same for the bias gradient,
-// whose partial sums sit in row `ones_row` of dW^T (db == null: there is none).
-__global__ void __launch_bounds__(128) wgrad_reduce_kernel(const float *__restrict__ part, int jtiles, int ctiles,
-                                                           int splits, int BN, int Kfwd, int Co, float *__restrict__ dW,
-                                                           float *__restrict__ db, int ones_row) {
+// whose partial sums sit in row `ones_row` of dW^T (db == null: there is none).  The layers of a backward pass are reduced
+// by one launch behind their last GEMM: one by one each was a link of 8 us between two GEMMs.
+struct ReduceJob {
+    const float *part;
+    float *dW, *db;
+    int jtiles, ctiles, splits, BN, Kfwd, Co, ones_row;
+    int per_block;  // results per block: 128, or 32 (a warp each on more SMs) where they are few
+    unsigned block_end;
+};
+struct ReduceJobs {
+    int n;
+    ReduceJob j[kMaxReduceJobs];
+};
+
+__global__ void __launch_bounds__(128) wgrad_reduce_kernel(const __grid_constant__ ReduceJobs jobs) {
     grid_wait();
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    int k = 0;
+    while (blockIdx.x >= jobs.j[k].block_end) ++k;
+    const ReduceJob &q = jobs.j[k];
+    if ((int)threadIdx.x >= q.per_block) return;
+    const int jtiles = q.jtiles, ctiles = q.ctiles, splits = q.splits, BN = q.BN, Kfwd = q.Kfwd, Co = q.Co;
+    const long long idx = (long long)(blockIdx.x - (k ? jobs.j[k - 1].block_end : 0u)) * q.per_block + threadIdx.x;
     const long long nW = (long long)Co * Kfwd;
     int co, jj;
     float *dst;
     if (idx < nW) {
         co = (int)(idx / Kfwd);
         jj = (int)(idx - (long long)co * Kfwd);
-        dst = dW + idx;
-    } else if (db != nullptr && idx < nW + Co) {
+        dst = q.dW + idx;
+    } else if (q.db != nullptr && idx < nW + Co) {
         co = (int)(idx - nW);
-        jj = ones_row;
-        dst = db + co;
+        jj = q.ones_row;
+        dst = q.db + co;
     } else {
         return;
     }
     const int x = jj >> 7, p = jj & 127, y = co / BN, c = co - y * BN;
     const size_t tile = (size_t)128 * BN, per_split = (size_t)ctiles * jtiles * tile;
-    const float *src = part + ((size_t)y * jtiles + x) * tile + (size_t)c * 128 + p;
+    const float *src = q.part + ((size_t)y * jtiles + x) * tile + (size_t)c * 128 + p;
     float acc = 0.f;
     int z = 0;
     for (; z + 16 <= splits; z += 16) {  // the loads of 16 splits are in flight while the sum stays in order
@@ -1254,12 +1271,38 @@ int tma_dgrad_weights(const bf16 *W, bf16 *Wc, int Co, int k, int Ci, int wt_ld,
     return PPO_OK;
 }
 
+// Reductions collected on this thread inside wgrad_batch (null: each is launched at once)
+static thread_local ReduceJobs *reduce_batch = nullptr;
+
+static int launch_reductions(const ReduceJobs &jobs, cudaStream_t st) {
+    if (jobs.n == 0) return PPO_OK;
+    return ppo_launch(wgrad_reduce_kernel, dim3(jobs.j[jobs.n - 1].block_end), dim3(128), 0, st, jobs);
+}
+
 int wgrad_reduce(const float *part, int jtiles, int ctiles, int splits, int BN, int Kfwd, int Co, float *dW, float *db,
                  int ones_row, cudaStream_t st) {
     const long long n = (long long)Co * Kfwd + (db ? Co : 0);
-    const int threads = n < 128 * ppo_num_sms() ? 32 : 128;  // few results: a warp each on more SMs
-    PPO_TRY(ppo_launch(wgrad_reduce_kernel, dim3(ppo_cdiv(n, threads)), dim3(threads), 0, st, part, jtiles, ctiles, splits, BN, Kfwd, Co, dW, db, ones_row));
-    return PPO_OK;
+    ReduceJobs one;
+    one.n = 0;
+    ReduceJobs &jobs = reduce_batch ? *reduce_batch : one;
+    if (jobs.n == kMaxReduceJobs) {
+        PPO_TRY(launch_reductions(jobs, st));
+        jobs.n = 0;
+    }
+    ReduceJob &q = jobs.j[jobs.n];
+    q = {part, dW, db, jtiles, ctiles, splits, BN, Kfwd, Co, ones_row, n < 128 * ppo_num_sms() ? 32 : 128, 0u};
+    q.block_end = (jobs.n ? jobs.j[jobs.n - 1].block_end : 0u) + (unsigned)((n + q.per_block - 1) / q.per_block);
+    ++jobs.n;
+    return reduce_batch ? PPO_OK : launch_reductions(jobs, st);
+}
+
+int wgrad_batch(const std::function<int()> &gemms, cudaStream_t st) {
+    ReduceJobs jobs, *outer = reduce_batch;
+    jobs.n = 0;
+    reduce_batch = &jobs;
+    const int s = gemms();
+    reduce_batch = outer;
+    return s == PPO_OK ? launch_reductions(jobs, st) : s;
 }
 
 int tma_gemm_wgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *X, float *dW, float *db, float *part,
