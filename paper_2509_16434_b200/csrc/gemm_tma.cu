@@ -804,6 +804,39 @@ struct ReduceJobs {
     ReduceJob j[kMaxReduceJobs];
 };
 
+// src[0] + src[stride] + .. in order, the loads of IN splits in flight.  Few results wait for memory, and a remainder read
+// one by one costs a trip for each split: there it is one more predicated round (148 splits: 13 trips -> 5).  Many results
+// wait for bandwidth and mostly have a handful of splits: predicated rounds would only cost instructions (19 -> 27 us for
+// 4 M results).
+template <int IN, bool ROUND>
+__device__ __forceinline__ float sum_splits(const float *__restrict__ src, size_t stride, int splits) {
+    float acc = 0.f;
+    int z = 0;
+    for (; z + IN <= splits; z += IN) {
+        float v[IN];
+#pragma unroll
+        for (int u = 0; u < IN; ++u) v[u] = src[(size_t)(z + u) * stride];
+#pragma unroll
+        for (int u = 0; u < IN; ++u) acc += v[u];
+    }
+    if (ROUND && z < splits) {
+        float v[IN];
+#pragma unroll
+        for (int u = 0; u < IN; ++u) v[u] = z + u < splits ? src[(size_t)(z + u) * stride] : 0.f;
+#pragma unroll
+        for (int u = 0; u < IN; ++u)
+            if (z + u < splits) acc += v[u];
+    }
+    if (!ROUND) {
+#pragma unroll 8
+        for (; z < splits; ++z) acc += src[(size_t)z * stride];
+    }
+    return acc;
+}
+
+// FEW: every job of the launch has few results (a kernel of its own: the registers of its rounds would halve the blocks
+// that fit an SM).
+template <bool FEW>
 __global__ void __launch_bounds__(128) wgrad_reduce_kernel(const __grid_constant__ ReduceJobs jobs) {
     grid_wait();
     int k = 0;
@@ -829,18 +862,7 @@ __global__ void __launch_bounds__(128) wgrad_reduce_kernel(const __grid_constant
     const int x = jj >> 7, p = jj & 127, y = co / BN, c = co - y * BN;
     const size_t tile = (size_t)128 * BN, per_split = (size_t)ctiles * jtiles * tile;
     const float *src = q.part + ((size_t)y * jtiles + x) * tile + (size_t)c * 128 + p;
-    float acc = 0.f;
-    int z = 0;
-    for (; z + 16 <= splits; z += 16) {  // the loads of 16 splits are in flight while the sum stays in order
-        float v[16];
-#pragma unroll
-        for (int u = 0; u < 16; ++u) v[u] = src[(size_t)(z + u) * per_split];
-#pragma unroll
-        for (int u = 0; u < 16; ++u) acc += v[u];
-    }
-#pragma unroll 8
-    for (; z < splits; ++z) acc += src[(size_t)z * per_split];
-    *dst += acc;
+    *dst += sum_splits<FEW ? 32 : 16, FEW>(src, per_split, splits);
 }
 
 // --------------------------------------------------------------------- host ----
@@ -1276,7 +1298,10 @@ static thread_local ReduceJobs *reduce_batch = nullptr;
 
 static int launch_reductions(const ReduceJobs &jobs, cudaStream_t st) {
     if (jobs.n == 0) return PPO_OK;
-    return ppo_launch(wgrad_reduce_kernel, dim3(jobs.j[jobs.n - 1].block_end), dim3(128), 0, st, jobs);
+    bool few = true;
+    for (int i = 0; i < jobs.n; ++i) few = few && jobs.j[i].per_block == 32;
+    return ppo_launch(few ? wgrad_reduce_kernel<true> : wgrad_reduce_kernel<false>, dim3(jobs.j[jobs.n - 1].block_end), dim3(128), 0, st,
+                      jobs);
 }
 
 int wgrad_reduce(const float *part, int jtiles, int ctiles, int splits, int BN, int Kfwd, int Co, float *dW, float *db,
