@@ -480,21 +480,23 @@ __global__ void __launch_bounds__(256) pool_concat_kernel(const bf16 *__restrict
     h0[b * (C + P) + C + j] = __float2bfloat16_rn(proprio[i]);
 }
 
-// dact[b][px][c] = dh0[b][c] / npx where act > 0, else 0; 8 channels per thread.
+// dact[b][px][c] = dh0[b][c] / npx where act > 0, else 0; 8 channels per thread.  I: index type, 32 bits where they do (two
+// 64-bit divisions per thread cost as much as its memory traffic).
+template <typename I>
 __global__ void __launch_bounds__(256) unpool_kernel(const float *__restrict__ dh0, const bf16 *__restrict__ act,
                                                      bf16 *__restrict__ dact, long long total8, int npx, int C,
                                                      int ld_h0) {
     grid_wait();
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= total8) return;
-    const int c8n = C >> 3;
+    const I i = (I)blockIdx.x * (I)256 + (I)threadIdx.x;
+    if (i >= (I)total8) return;
+    const I c8n = (I)(C >> 3);
     const int c8 = (int)(i % c8n) * 8;
-    const long long b = i / ((long long)npx * c8n);
+    const long long b = (long long)(i / ((I)npx * c8n));
     const float inv = 1.f / (float)npx;
     const float4 g0 = *reinterpret_cast<const float4 *>(dh0 + b * ld_h0 + c8);
     const float4 g1 = *reinterpret_cast<const float4 *>(dh0 + b * ld_h0 + c8 + 4);
     const float g[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
-    const uint4 raw = *reinterpret_cast<const uint4 *>(act + i * 8);
+    const uint4 raw = *reinterpret_cast<const uint4 *>(act + (size_t)i * 8);
     const __nv_bfloat162 *a2 = reinterpret_cast<const __nv_bfloat162 *>(&raw);
     __nv_bfloat162 o[4];
 #pragma unroll
@@ -502,7 +504,7 @@ __global__ void __launch_bounds__(256) unpool_kernel(const float *__restrict__ d
         const float2 f = __bfloat1622float2(a2[k]);
         o[k] = __floats2bfloat162_rn(f.x > 0.f ? g[2 * k] * inv : 0.f, f.y > 0.f ? g[2 * k + 1] * inv : 0.f);
     }
-    *reinterpret_cast<uint4 *>(dact + i * 8) = *reinterpret_cast<uint4 *>(o);
+    *reinterpret_cast<uint4 *>(dact + (size_t)i * 8) = *reinterpret_cast<uint4 *>(o);
 }
 
 // Head gradient as a bf16 GEMM operand: [rows][16] = [dmean (A), dvalue, zeros].
@@ -1438,7 +1440,7 @@ extern "C" int ppo_encoder_bwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
     } else {
         const int npx = m->Hs[L] * m->Ws[L], C = m->Cs[L];
         const long long total8 = (long long)rows * npx * C / 8;
-        PPO_TRY(ppo_launch(unpool_kernel, dim3(ppo_cdiv(total8, 256)), dim3(256), 0, st, m->dh0_f32, m->act[L], m->dact[L], total8, npx, C,
+        PPO_TRY(ppo_launch(total8 < (1ll << 31) ? unpool_kernel<uint32_t> : unpool_kernel<unsigned long long>, dim3(ppo_cdiv(total8, 256)), dim3(256), 0, st, m->dh0_f32, m->act[L], m->dact[L], total8, npx, C,
                                                            m->hw[0]));
     }
     // With layer normalisation dact[l] arrives as the gradient of the normalised, scaled and shifted value; ln_bwd

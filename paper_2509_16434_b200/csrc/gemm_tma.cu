@@ -844,13 +844,14 @@ __global__ void __launch_bounds__(128) wgrad_reduce_kernel(const __grid_constant
     const ReduceJob &q = jobs.j[k];
     if ((int)threadIdx.x >= q.per_block) return;
     const int jtiles = q.jtiles, ctiles = q.ctiles, splits = q.splits, BN = q.BN, Kfwd = q.Kfwd, Co = q.Co;
-    const long long idx = (long long)(blockIdx.x - (k ? jobs.j[k - 1].block_end : 0u)) * q.per_block + threadIdx.x;
-    const long long nW = (long long)Co * Kfwd;
+    // 32-bit indices: a 64-bit division per result took most of the time where splits are few
+    const uint32_t idx = (blockIdx.x - (k ? jobs.j[k - 1].block_end : 0u)) * (uint32_t)q.per_block + threadIdx.x;
+    const uint32_t nW = (uint32_t)Co * (uint32_t)Kfwd;
     int co, jj;
     float *dst;
     if (idx < nW) {
-        co = (int)(idx / Kfwd);
-        jj = (int)(idx - (long long)co * Kfwd);
+        co = (int)(idx / (uint32_t)Kfwd);
+        jj = (int)(idx - (uint32_t)co * (uint32_t)Kfwd);
         dst = q.dW + idx;
     } else if (q.db != nullptr && idx < nW + Co) {
         co = (int)(idx - nW);
@@ -1307,6 +1308,7 @@ static int launch_reductions(const ReduceJobs &jobs, cudaStream_t st) {
 int wgrad_reduce(const float *part, int jtiles, int ctiles, int splits, int BN, int Kfwd, int Co, float *dW, float *db,
                  int ones_row, cudaStream_t st) {
     const long long n = (long long)Co * Kfwd + (db ? Co : 0);
+    if (n > 0xffffff00ll) return PPO_ERR_UNSUPPORTED;  // 16 GB of weights in one layer
     ReduceJobs one;
     one.n = 0;
     ReduceJobs &jobs = reduce_batch ? *reduce_batch : one;
