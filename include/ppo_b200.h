@@ -16,6 +16,10 @@
  *    must provide.  *_create / *_alloc allocate only small host-side handles.
  *  - `stream` is a cudaStream_t passed as void*.  Calls only enqueue work on it and
  *    do not synchronise (ppo_poll_status is the exception).
+ *  - Calls may be captured into a CUDA graph, except ppo_poll_status and the first ppo_gae_static on a device.  The
+ *    graph repeats the call with the pointers, sizes and scalars (the Adam step number among them) of the capture.
+ *    Counters that a handle keeps cleared between launches are cleared inside each graph that uses them, so a
+ *    graph may be launched before, between or after eager calls.  A graph does not outlive ppo_model_bind.
  *  - Device pointers must be 16-byte aligned; storage handed to ppo_buffer_alloc
  *    and ppo_model_bind's workspace must be 256-byte aligned.
  *  - Samples of the buffer are numbered time-major: s = t * N + n.

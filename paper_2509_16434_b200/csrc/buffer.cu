@@ -40,6 +40,24 @@ int ppo_num_sms() {
     return sms[dev];
 }
 
+int ppo_work_sequence(cudaStream_t st, uint64_t *seq) {
+    cudaStreamCaptureStatus status;
+    unsigned long long id = 0;
+    PPO_CUDA_CHECK(cudaStreamGetCaptureInfo(st, &status, &id));
+    *seq = status == cudaStreamCaptureStatusNone ? kEagerWork : kEagerWork + 1 + id;  // ids are never given out twice
+    return PPO_OK;
+}
+
+int ppo_clear_once(uint64_t *made, void *p, size_t bytes, cudaStream_t st) {
+    uint64_t seq;
+    PPO_TRY(ppo_work_sequence(st, &seq));
+    if (*made == seq) return PPO_OK;
+    PPO_CUDA_CHECK(cudaMemsetAsync(p, 0, bytes, st));
+    ppo_count_launches(1);
+    *made = seq;
+    return PPO_OK;
+}
+
 extern "C" const char *ppo_status_string(int s) {
     switch (s) {
         case PPO_OK: return "ok";
@@ -125,7 +143,7 @@ extern "C" int ppo_buffer_alloc(const ppo_buffer_desc *d, void *dev_storage, siz
     }
     b->gae_valid = false;
     b->gae_blocks = 0;
-    b->barrier_zeroed = false;
+    b->barrier_made = kNotMade;
     *out = b;
     return PPO_OK;
 }
@@ -501,11 +519,7 @@ extern "C" int ppo_compute_gae(ppo_buffer *b, const float *last_value, float gam
     if (normalize == 2 && (blocks >= kMaxGaeBlocks || blocks > gae_fused_capacity())) return PPO_ERR_UNSUPPORTED;
     if (normalize == 2) {
         unsigned int *barrier = reinterpret_cast<unsigned int *>(partials + 2 * kMaxGaeBlocks) - 2;
-        if (!b->barrier_zeroed) {
-            PPO_CUDA_CHECK(cudaMemsetAsync(barrier, 0, 8, st));
-            ppo_count_launches(1);
-            b->barrier_zeroed = true;
-        }
+        PPO_TRY(ppo_clear_once(&b->barrier_made, barrier, 8, st));
         const float *reward = slab<float>(b, PPO_FIELD_REWARD), *value = slab<float>(b, PPO_FIELD_VALUE);
         const uint8_t *done = slab<uint8_t>(b, PPO_FIELD_DONE);
         float *adv = slab<float>(b, PPO_FIELD_ADV), *ret = slab<float>(b, PPO_FIELD_RET);

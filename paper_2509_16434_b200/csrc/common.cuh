@@ -41,6 +41,17 @@ int32_t *ppo_device_status_ptr();
 void ppo_count_launches(int n);
 int ppo_num_sms();
 
+// Device state that a handle makes once and relies on from then on (cleared counters) is remembered together with the
+// sequence of work that makes it: eager work has run by the time later eager work does, but work that is captured runs when
+// its graph is launched, which may be never, or again after anything else.  So what one capture made counts for the rest
+// of that capture only, and a graph makes everything it leans on itself.
+constexpr uint64_t kNotMade = 0, kEagerWork = 1;
+// The sequence that work enqueued on st now belongs to: kEagerWork, or a number of the capture in progress.
+int ppo_work_sequence(cudaStream_t st, uint64_t *seq);
+// Clears the words at p unless *made says that the sequence st is in has them cleared already.  The kernels that use them leave
+// them as a cleared state (a clear in front of every launch would break the chain of overlapped launches).
+int ppo_clear_once(uint64_t *made, void *p, size_t bytes, cudaStream_t st);
+
 struct ppo_buffer {
     ppo_buffer_desc d;
     char *base;
@@ -48,7 +59,7 @@ struct ppo_buffer {
     size_t field_off[PPO_NUM_FIELDS];
     bool gae_valid;
     int gae_blocks;  // partial sums held in the scratch slab
-    bool barrier_zeroed;  // the grid-barrier words at the end of the scratch slab have been cleared once
+    uint64_t barrier_made;  // where the grid-barrier words at the end of the scratch slab were cleared (ppo_clear_once)
 };
 
 // Geometry of one stride-2 convolution (an FC layer is the 1x1 image, k = 1 case).
@@ -89,7 +100,7 @@ struct ppo_model {
     float *lstm_dtop;                // gradient w.r.t. a layer's outputs [mb][H] (from the FC layers or the layer above)
     float *lstm_dhc, *lstm_dcc;      // gradients carried to the previous step [mb][H]
     unsigned int *lstm_counters;     // of the persistent time loop (lstm.cuh)
-    bool counters_zeroed;
+    uint64_t counters_made;          // where they were cleared (ppo_clear_once)
     bool acting = false;             // inside ppo_policy_act
     size_t arena, nparams;
     // bound arrays
@@ -128,7 +139,7 @@ struct ppo_model {
     bool wT_valid;
     bool wC_valid[PPO_MAX_CONV + 1];
     unsigned int *loss_ticket;     // blocks of the loss kernel that are done (0 between launches)
-    bool ticket_zeroed;
+    uint64_t ticket_made;          // where it was cleared (ppo_clear_once)
     // forward/backward pairing
     int last_row0, last_rows;
     bool fwd_valid;

@@ -1066,11 +1066,7 @@ static LstmSteps lstm_steps(const ppo_model *m, int l) {
 // Runs a layer's time loop as one launch where it fits (remembered like the GEMMs' launches).
 template <typename F>
 static int lstm_persistent(ppo_model *m, int op, int l, cudaStream_t st, F &&make) {
-    if (!m->counters_zeroed) {
-        PPO_CUDA_CHECK(cudaMemsetAsync(m->lstm_counters, 0, kLstmCounters * 128, st));
-        ppo_count_launches(1);
-        m->counters_zeroed = true;
-    }
+    PPO_TRY(ppo_clear_once(&m->counters_made, m->lstm_counters, kLstmCounters * 128, st));
     PlanKey k = plan_key(op, fc_geom(m->seq_Be, m->seq_T, l));
     const void *p[] = {m->seq_done, m->seq_h_init, m->seq_c_init};
     memcpy(k.p, p, sizeof(p));

@@ -276,7 +276,7 @@ extern "C" int ppo_model_bind(ppo_model *m, float *master, void *shadow, float *
     carve(m, m, microbatch, m->ws);
     m->fwd_valid = false;
     m->wT_valid = false;
-    m->ticket_zeroed = m->counters_zeroed = false;
+    m->ticket_made = m->counters_made = kNotMade;
     return PPO_OK;
 }
 
@@ -601,11 +601,7 @@ extern "C" int ppo_loss_fwd_bwd(ppo_model *m, const ppo_minibatch *mb, int row0,
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const float *logsigma = m->master + m->tensors.back().off;
     const int blocks = ppo_cdiv(rows, kLossThreads);
-    if (!m->ticket_zeroed) {
-        PPO_CUDA_CHECK(cudaMemsetAsync(m->loss_ticket, 0, sizeof(unsigned int), st));
-        ppo_count_launches(1);
-        m->ticket_zeroed = true;
-    }
+    PPO_TRY(ppo_clear_once(&m->ticket_made, m->loss_ticket, sizeof(unsigned int), st));
     PPO_TRY(ppo_launch(loss_kernel, dim3(blocks), dim3(kLossThreads), 0, st, rows, A, 1.f / (float)B_total, mean, value, logsigma,
                                                  mb->action + (size_t)row0 * A, mb->logp_old + row0, mb->adv + row0,
                                                  mb->ret + row0, clip, vf_coef, dmean, dvalue, m->loss_partials,
