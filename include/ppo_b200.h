@@ -18,8 +18,9 @@
  *    do not synchronise (ppo_poll_status is the exception).
  *  - Calls may be captured into a CUDA graph, except ppo_poll_status and the first ppo_gae_static on a device.  The
  *    graph repeats the call with the pointers, sizes and scalars (the Adam step number among them) of the capture.
- *    Counters that a handle keeps cleared between launches are cleared inside each graph that uses them, so a
- *    graph may be launched before, between or after eager calls.  A graph does not outlive ppo_model_bind.
+ *    What a handle keeps on the device between calls (cleared counters, transposed weights) is made inside each graph
+ *    that uses it, so a graph may be launched before, between or after eager calls.  A graph does not outlive
+ *    ppo_model_bind.
  *  - Device pointers must be 16-byte aligned; storage handed to ppo_buffer_alloc
  *    and ppo_model_bind's workspace must be 256-byte aligned.
  *  - Samples of the buffer are numbered time-major: s = t * N + n.

@@ -136,8 +136,9 @@ struct ppo_model {
     float *loss_partials;
     float *act_mean;               // [mb][A]: Gaussian mean of ppo_policy_act before sampling
     int loss_partial_blocks;
-    bool wT_valid;
-    bool wC_valid[PPO_MAX_CONV + 1];
+    uint64_t wT_made;              // where wT was made from the current weights (kNotMade: not yet)
+    bool update_captured;          // a graph holds an update of the weights: when it runs is not known here
+    bool wC_valid[PPO_MAX_CONV + 1];  // made since wT was
     unsigned int *loss_ticket;     // blocks of the loss kernel that are done (0 between launches)
     uint64_t ticket_made;          // where it was cleared (ppo_clear_once)
     // forward/backward pairing

@@ -1252,7 +1252,10 @@ extern "C" int ppo_encoder_fwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
 }
 
 static int refresh_transposed(ppo_model *m, cudaStream_t st) {
-    if (m->wT_valid) return PPO_OK;
+    uint64_t seq;
+    PPO_TRY(ppo_work_sequence(st, &seq));
+    // (behind a captured update eager calls cannot know the weights' age, and make the copies each time)
+    if (m->wT_made == seq && !(seq == kEagerWork && m->update_captured)) return PPO_OK;
     TransposeJobs jobs;
     int n = 0;
     long long blocks = 0;
@@ -1274,7 +1277,7 @@ static int refresh_transposed(ppo_model *m, cudaStream_t st) {
     for (int l = 1; l <= m->F + 1; ++l) add(m->ti_fc[l], l <= m->F ? m->hw[l] : m->d.A + 1, 1, fc_input_width(m, l));
     if (blocks > 0x7fffffffll) return PPO_ERR_UNSUPPORTED;
     PPO_TRY(ppo_launch(transpose_weights_kernel, dim3((unsigned)blocks), dim3(256), 0, st, m->shadow, m->wT, jobs));
-    m->wT_valid = true;
+    m->wT_made = seq;
     for (int l = 2; l <= m->L; ++l) m->wC_valid[l] = false;
     return PPO_OK;
 }

@@ -125,7 +125,6 @@ extern "C" int ppo_model_create(const ppo_model_desc *d, ppo_model **out) {
     m->ws_bytes = 0;
     m->mbmax = 0;
     m->fwd_valid = false;
-    m->wT_valid = false;
     m->last_row0 = m->last_rows = -1;
     m->seq_T = m->seq_Be = 0;
     m->seq_done = nullptr;
@@ -275,8 +274,8 @@ extern "C" int ppo_model_bind(ppo_model *m, float *master, void *shadow, float *
     m->mbmax = microbatch;
     carve(m, m, microbatch, m->ws);
     m->fwd_valid = false;
-    m->wT_valid = false;
-    m->ticket_made = m->counters_made = kNotMade;
+    m->ticket_made = m->counters_made = m->wT_made = kNotMade;
+    m->update_captured = false;
     return PPO_OK;
 }
 
@@ -408,13 +407,21 @@ __global__ void __launch_bounds__(256) shadow_kernel(const float4 *__restrict__ 
     shadow[i] = o;
 }
 
+// What was made from the weights is out of date.
+static int weights_changed(ppo_model *m, cudaStream_t st) {
+    m->wT_made = kNotMade;
+    uint64_t seq;
+    PPO_TRY(ppo_work_sequence(st, &seq));
+    if (seq != kEagerWork) m->update_captured = true;
+    return PPO_OK;
+}
+
 extern "C" int ppo_model_sync_shadow(ppo_model *m, void *stream) {
     if (!m || !m->master) return PPO_ERR_STATE;
     size_t n4 = m->arena / 4;
     PPO_TRY(ppo_launch(shadow_kernel, dim3(ppo_cdiv(n4, 256)), dim3(256), 0, static_cast<cudaStream_t>(stream), 
         reinterpret_cast<const float4 *>(m->master), reinterpret_cast<uint2 *>(m->shadow), n4));
-    m->wT_valid = false;
-    return PPO_OK;
+    return weights_changed(m, static_cast<cudaStream_t>(stream));
 }
 
 // (A memset node between two kernels would break the chain of overlapped launches.)
@@ -479,9 +486,8 @@ extern "C" int ppo_adam_step(ppo_model *m, float lr, float beta1, float beta2, f
         reinterpret_cast<float4 *>(m->master), reinterpret_cast<float4 *>(m->adam_m),
         reinterpret_cast<float4 *>(m->adam_v), reinterpret_cast<const float4 *>(m->grad),
         reinterpret_cast<uint2 *>(m->shadow), n4, lr, beta1, beta2, eps, (float)(1.0 / c1), (float)(1.0 / c2)));
-    m->wT_valid = false;
     m->fwd_valid = false;
-    return PPO_OK;
+    return weights_changed(m, static_cast<cudaStream_t>(stream));
 }
 
 // -------------------------------------------------------------------- loss ----
