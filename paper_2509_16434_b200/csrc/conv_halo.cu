@@ -579,8 +579,9 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
                                 } else {
                                     const uint4 &q4 = act[k];
                                     const uint32_t aw = j == 0 ? q4.x : (j == 1 ? q4.y : (j == 2 ? q4.z : q4.w));
-                                    // stored activations are >= 0 (the outputs of a ReLU): a half gates unless it is zero
-                                    pk[j] = pr & half_signs(aw + 0x7FFF7FFFu);
+                                    // a comparison, as wherever a gate is read: saved activations can be written from outside,
+                                    // and minus zero, negative numbers and NaN close it
+                                    pk[j] = pr & __hgt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&aw), __float2bfloat162_rn(0.f));
                                 }
                             }
                             put(stg, hh * 32 + 8 * k, make_uint4(pk[0], pk[1], pk[2], pk[3]));

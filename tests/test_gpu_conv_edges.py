@@ -2,6 +2,7 @@
 per tile, every chunk width, single rows and columns of outputs, micro-batches that leave the last tile part empty."""
 import numpy as np
 import pytest
+import torch
 
 import test_gpu_learner as base
 from helpers import rel_l2
@@ -71,3 +72,40 @@ def test_gate_bits_are_the_signs_of_the_activations():
             ch = np.arange(32)
             bits = (word[:, :, None] >> (ch // 2 + 16 * (ch % 2))) & 1
             assert np.array_equal(bits != 0, act > 0), (name, l)
+
+
+# layers whose gate the input gradient reads as activations in the halo kernel (16 channels), as activations in the generic
+# one (48) and as bits (32)
+@pytest.mark.parametrize("name", ["narrow_16_32", "ln_odd", "chunks_of_16", "two_chunks"])
+def test_gate_is_open_for_positive_activations_only(name):
+    """Saved activations written from outside may be anything: minus zero, negative numbers and NaN close the gate as zero
+    does, in both halves of a pair and without a trace in the neighbouring channel.  The first layer's gradients, which see
+    these activations through the gate alone, keep every bit."""
+    w = NETS[name]
+    B = w.M // w.minibatches
+    L, md, lay, theta, roll, action, logp, dev = base._setup(w, B)
+    h = L.hyper
+    L.compute_gae(dev["last_value"])
+    ppo.ppo_shuffle_gather_minibatch(L.buffer, 5, 0, 0, w.minibatches, L.mb)
+    ppo.ppo_encoder_fwd(L.model, L.mb, 0, B, L.mean, L.value)
+    L.loss.zero_()
+    ppo.ppo_loss_fwd_bwd(L.model, L.mb, 0, B, B, L.mean, L.value, h.clip, h.vf_coef, h.ent_coef, L.loss, L.dmean, L.dvalue)
+    act = L.model.activation(0, 1).view(torch.int16)
+    saved = act.clone()
+    where = torch.rand(act.shape, device=act.device, generator=torch.Generator(act.device).manual_seed(1)) < 0.3
+    closed = [0x0000, 0x8000, 0x8001, 0xBF80, 0xFF80, 0x7FC0, 0x7FFF, 0xFFC0]  # 0, -0, -tiny, -1, -inf, NaN, NaN, -NaN
+
+    def first_layer(pattern):
+        act.copy_(torch.where(where, torch.tensor(pattern - 0x10000 if pattern & 0x8000 else pattern, dtype=torch.int16,
+                                                  device=act.device), saved))
+        ppo.ppo_model_sync_masks(L.model, B)
+        ppo.ppo_model_zero_grad(L.model)
+        ppo.ppo_encoder_bwd(L.model, L.mb, 0, B, L.dmean, L.dvalue, True)
+        assert ppo.ppo_poll_status() == 0
+        (o0, s0), (o1, s1) = L.model.tensors()[:2]
+        return L.model.grad[o0:o1 + s1].clone()
+
+    want = first_layer(closed[0])
+    assert torch.isfinite(want).all() and float(want.norm()) > 0
+    for pattern in closed[1:]:
+        assert torch.equal(first_layer(pattern), want), hex(pattern)
