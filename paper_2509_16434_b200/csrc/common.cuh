@@ -101,7 +101,6 @@ struct ppo_model {
     float *lstm_dhc, *lstm_dcc;      // gradients carried to the previous step [mb][H]
     unsigned int *lstm_counters;     // of the persistent time loop (lstm.cuh)
     uint64_t counters_made;          // where they were cleared (ppo_clear_once)
-    bool acting = false;             // inside ppo_policy_act
     size_t arena, nparams;
     // bound arrays
     float *master, *grad, *adam_m, *adam_v;

@@ -1207,13 +1207,19 @@ extern "C" int ppo_encoder_fwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
         // flatten -> fully connected -> ReLU into the first E columns of h_0, proprio behind them
         const int K = m->Hs[m->L] * m->Ws[m->L] * m->Cs[m->L];
         ConvGeom g = fc_geom(rows, K, d.embed);
-        // Acting (one step, no gradients to follow) on few rows: the long reduction of a handful of tiles is the longest link
-        // of a decision, so it is cut into slabs that as many CTAs work on (K = 10240, 16 rows: 26 -> 8 us).  Sequences
-        // keep the one sum: their passes are compared step by step.
+        // One step of a recurrent policy, i.e. acting: the reduction over K of a handful of tiles is the longest link of a
+        // decision, so it is cut into slabs that as many CTAs work on.  The slabs' sum differs from the one sum in its last
+        // fp32 digits, which a bf16 rounding of the embedding can turn into a step of 2^-8, so everything else keeps the one
+        // sum, and with it the same bits whatever the call: longer sequences, and feed-forward policies, whose
+        // forward is the same call when acting and when training.
+        // The gain hardly depends on the rows; its share of the forward pass does (us, one sum -> slabs).  K = 10240: 16 rows
+        // 69.0 -> 50.6, 512 165 -> 147, 1024 256 -> 237, 2048 454 -> 434, 4096 866 -> 851 (a run's spread there: 829 .. 886).
+        // 16 rows: K = 768 48.3 -> 45.5, 1536 49.7 -> 45.9, 2048 50.7 -> 46.1, 6144 59.7 -> 48.3.  The lines lie where less than
+        // a tenth (K) or a fifteenth (rows) is left to gain.
         const float *part = m->wg_part[m->ti_embed];
         int slabs = 8;
         while (slabs > 1 && K % (slabs * 64) != 0) slabs /= 2;
-        if ((m->acting || (d.n_lstm > 0 && m->seq_T == 1)) && slabs > 1 && K >= 2048 && rows <= 1024 &&
+        if (d.n_lstm > 0 && m->seq_T == 1 && slabs > 1 && K >= 2048 && rows <= 1024 &&
             (size_t)slabs * rows * d.embed <= m->wg_cap[m->ti_embed]) {
             PPO_TRY(gemm_nt_f32(m, rows, d.embed, K, m->act[m->L], K, m->shadow + m->tensors[m->ti_embed].off, m->wg_part[m->ti_embed],
                                 st, slabs));

@@ -665,9 +665,7 @@ extern "C" int ppo_policy_act(ppo_model *m, ppo_buffer *b, int t, const float *e
     b->gae_valid = false;
     for (int r0 = 0; r0 < d.N; r0 += m->mbmax) {
         const int rows = d.N - r0 < m->mbmax ? d.N - r0 : m->mbmax;
-        m->acting = true;
         int s = ppo_encoder_fwd(m, &obs, r0, rows, m->act_mean, value + r0, stream);
-        m->acting = false;
         if (s != PPO_OK) return s;
         s = ppo_policy_sample(m, rows, m->act_mean, eps + (size_t)r0 * d.A, action + (size_t)r0 * d.A, logp + r0, stream);
         if (s != PPO_OK) return s;

@@ -23,7 +23,7 @@ def test_sequences_at_tile_edges_match_oracle(Be, H, T, monkeypatch):
     base.test_backward_through_time_matches_oracle_on_identical_state("edge")
 
 
-# 1024 rows and fewer take the embedding (4096 inputs) in slabs, one more does not
+# one step of a recurrent policy: 1024 rows and fewer take the embedding (4096 inputs) in slabs, one more does not
 @pytest.mark.parametrize("n_lstm", [0, 1])
 @pytest.mark.parametrize("n", [1, 65, 1024, 1025])
 def test_acting_matches_oracle(n, n_lstm):
@@ -58,3 +58,58 @@ def test_state_reset_clears_finished_envs_only(layers, n, H):
     want = [torch.where(done[None, :, None] != 0, torch.zeros_like(s), s) for s in (h, c)]
     base.ppo.ppo_state_reset(h, c, done)
     assert torch.equal(h, want[0]) and torch.equal(c, want[1])
+
+
+# 2048 and 4096 inputs of the embedding, few and many rows
+@pytest.mark.parametrize("H,n", [(64, 1), (64, 65), (64, 1025), (72, 300)])
+def test_feed_forward_acting_gives_the_bits_of_the_training_forward(H, n):
+    """`act`, `act_into_buffer` and the forward of a minibatch with the same frames, in one piece and in micro-batches: the
+    log-probability that acting stores belongs to the mean that training starts from."""
+    ppo = base.ppo
+    w = synth.Workload("act", n, 2, H, 64, (16, 32, 64), (3, 3, 3), (40,), 1, 1, P=32, A=3, norm=True, embed=32)
+    L, small = base.Learner(w, w.B, DEV), base.Learner(w, max(1, n // 3), DEV)
+    shapes, gammas = synth.param_shapes(w)
+    theta = synth.init_params(L.model.arena, [o for o, _ in L.model.tensors()], shapes, 3, ones=gammas)
+    r = synth.rollout_torch(w, DEV, 3)
+    depth, proprio, eps = r["depth"][0], r["proprio"][0], r["eps"][0]
+    zero = torch.zeros_like(eps)  # actions are then the means
+    got = []
+    for X in (L, small):
+        X.model.load(theta)
+        a, lp, v = X.act(depth, proprio, eps)
+        X.act_into_buffer(0, depth, proprio, eps)
+        got += [(a, lp, v), tuple(X.buffer.field(f)[0].clone() for f in (ppo.FIELD_ACTION, ppo.FIELD_LOGP, ppo.FIELD_VALUE))]
+    for other in got[1:]:
+        assert all(torch.equal(x, y) for x, y in zip(got[0], other))
+    both = ppo.Minibatch(r["depth"].data_ptr(), r["proprio"].data_ptr(), None, None, None, None, None, None, 2 * n)
+    ppo.ppo_encoder_fwd(L.model, both, 0, 2 * n, L.mean, L.value)  # 2 n rows at once, as training takes them
+    mean = L.act(depth, proprio, zero)[0]
+    ppo.ppo_encoder_fwd(L.model, both, 0, 2 * n, L.mean, L.value)
+    assert torch.equal(L.mean[:n], mean) and torch.equal(L.value[:n], got[0][2])
+    assert ppo.ppo_poll_status() == 0
+
+
+def test_recurrent_acting_stays_within_a_rounding_of_the_sequence():
+    """Steps taken one by one (embedding in slabs) against the same steps as one sequence (one sum).  The two sums of an
+    embedding differ in fp32; rounded to bf16 a value may fall to the other side, a step of at most 2^-8 of it, and what
+    follows (gates, layers of unit gain) does not enlarge a relative difference beyond that."""
+    w = synth.Workload("act_seq", 9, 3, 64, 64, (16, 32, 64), (3, 3, 3), (40,), 1, 1, P=32, A=3, norm=True, embed=32, n_lstm=2, lstm_h=128)
+    L, md, lay, theta, roll, action, logp, dev = base._setup(w, w.B)
+    ppo = base.ppo
+    steps = []
+    for t in range(w.T):
+        steps.append(L.act(dev["depth"][t], dev["proprio"][t], dev["eps"][t]))
+        L.reset_rollout_state(w.N, dev["done"][t])
+    rows = w.T * w.N
+    seq = ppo.Minibatch(dev["depth"].data_ptr(), dev["proprio"].data_ptr(), None, None, None, None, None, None, rows)
+    ppo.ppo_model_set_sequence(L.model, w.T, w.N, dev["done"], L.h_init, L.c_init)
+    ppo.ppo_encoder_fwd(L.model, seq, 0, rows, L.mean, L.value)
+    a, lp = torch.empty((rows, w.A), device=DEV), torch.empty(rows, device=DEV)
+    ppo.ppo_policy_sample(L.model, rows, L.mean, dev["eps"].reshape(rows, w.A), a, lp)
+    got_a, got_lp, got_v = (torch.cat([s[i] for s in steps]) for i in range(3))
+    # the same noise on both sides: actions differ by the means
+    d = (got_a - a).norm() / L.mean[:rows].norm(), (got_v - L.value[:rows]).norm() / L.value[:rows].norm()
+    print(f"one by one against one sequence: mean {float(d[0]):.2e}, value {float(d[1]):.2e}")
+    assert float(max(d)) <= 2.0 ** -8
+    assert torch.equal(got_lp, lp)  # of the action under its own mean: noise and log-sigma only
+    assert ppo.ppo_poll_status() == 0
