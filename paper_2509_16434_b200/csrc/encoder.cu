@@ -888,12 +888,12 @@ template <typename F>
 static int recorded(ppo_model *m, const PlanKey &key, cudaStream_t st, F &&make) {
     if (!m->plans) m->plans = new (std::nothrow) ppo_plans();
     if (!m->plans) return make();
-    if (const PlanEntry *e = ppo_find_plan(m->plans, key)) return ppo_replay(*e, st);
-    std::vector<LaunchRecord> launches, *outer = ppo_recording;
+    if (const Launches *known = m->plans->find(key)) return ppo_replay(*known, st);
+    Launches launches, *outer = ppo_recording;
     ppo_recording = &launches;
     const int s = make();
     ppo_recording = outer;
-    if (s == PPO_OK) ppo_store_plan(m->plans, key, std::move(launches));
+    if (s == PPO_OK) m->plans->put(key, std::move(launches));
     return s;
 }
 
@@ -932,7 +932,7 @@ static int run_dgrad(ppo_model *m, const ConvGeom &g, const bf16 *dY, int ldy, c
     memcpy(k.p, p, sizeof(p));
     k.v[0] = ldy; k.v[1] = wt_ld; k.v[2] = e.ksplit;
     if (m->plans)
-        if (const PlanEntry *pe = ppo_find_plan(m->plans, k)) return ppo_replay(*pe, st);
+        if (const Launches *known = m->plans->find(k)) return ppo_replay(*known, st);
     const bool halo = halo_dgrad_covers(g, ldy, wt_ld, e);
     const bf16 *Wc = layer > 0 && !halo ? m->wC + m->wC_off[layer] : nullptr;
     if (Wc && !m->wC_valid[layer]) {

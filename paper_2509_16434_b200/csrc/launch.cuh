@@ -12,14 +12,11 @@
 // Measured: host time of a forward pass of the recurrent policy 140 -> 53 us; TrainPPO of 4 x 1024 rows of 64 x 64, where
 // launches and gaps count, 1258 -> 944 us together with the launches that were merged.
 #pragma once
-#include <string.h>
-
 #include <tuple>
-
-#include <unordered_map>
 #include <vector>
 
 #include "common.cuh"
+#include "plan_store.h"
 
 // Everything the kernels in front of this one in the stream wrote is visible behind this.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -40,17 +37,14 @@ struct PlanKey {
     long long v[6];
 };
 
-struct PlanEntry {
-    PlanKey key;
-    std::vector<LaunchRecord> launches;
-};
+using Launches = std::vector<LaunchRecord>;
 
-struct ppo_plans {
-    std::unordered_multimap<uint64_t, PlanEntry> map;
+struct ppo_plans : PlanStore<PlanKey, Launches> {
+    ppo_plans() : PlanStore(1024) {}  // operations of one model; a few MB of host memory
 };
 
 // The record of the operation being prepared on this thread (null: none).
-extern thread_local std::vector<LaunchRecord> *ppo_recording;
+extern thread_local Launches *ppo_recording;
 
 int ppo_enqueue(const void *fn, dim3 grid, dim3 block, size_t smem, bool together, cudaStream_t st, void **argv);
 
@@ -90,8 +84,5 @@ int ppo_launch_together(void (*fn)(P...), dim3 grid, dim3 block, size_t smem, cu
     return ppo_launch_as(true, fn, grid, block, smem, st, args...);
 }
 
-// The entry of a key, or null.
-PlanEntry *ppo_find_plan(ppo_plans *plans, const PlanKey &key);
 // Enqueues a recorded operation.
-int ppo_replay(const PlanEntry &e, cudaStream_t st);
-void ppo_store_plan(ppo_plans *plans, const PlanKey &key, std::vector<LaunchRecord> &&launches);
+int ppo_replay(const Launches &launches, cudaStream_t st);

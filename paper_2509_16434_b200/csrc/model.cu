@@ -263,7 +263,7 @@ extern "C" int ppo_model_bind(ppo_model *m, float *master, void *shadow, float *
         !ppo_aligned(av, 16) || !ppo_aligned(ws, 256))
         return PPO_ERR_ALIGN;
     if (ws_bytes < ppo_model_workspace_bytes(m, microbatch)) return PPO_ERR_SHAPE;
-    if (m->plans) m->plans->map.clear();  // they hold the old addresses
+    if (m->plans) m->plans->clear();  // they hold the old addresses
     m->master = master;
     m->shadow = static_cast<bf16 *>(shadow);
     m->grad = grad;
