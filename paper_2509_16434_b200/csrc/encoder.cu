@@ -889,11 +889,11 @@ static int recorded(ppo_model *m, const PlanKey &key, cudaStream_t st, F &&make)
     if (!m->plans) m->plans = new (std::nothrow) ppo_plans();
     if (!m->plans) return make();
     if (const Launches *known = m->plans->find(key)) return ppo_replay(*known, st);
-    Launches launches, *outer = ppo_recording;
-    ppo_recording = &launches;
+    Recording made, *outer = ppo_recording;
+    ppo_recording = &made;
     const int s = make();
     ppo_recording = outer;
-    if (s == PPO_OK) m->plans->put(key, std::move(launches));
+    if (s == PPO_OK && made.complete) m->plans->put(key, std::move(made.launches));
     return s;
 }
 

@@ -5,8 +5,6 @@
 //   wgrad : dW[co][tap][ci] += sum_m dY[m][co] * X[b, 2oh+kh-p, 2ow+kw-p, ci]
 // m = (b, oh, ow) over output pixels, m' = (b, ih, iw) over input pixels; fp32 accumulation.
 #pragma once
-#include <functional>
-
 #include "common.cuh"
 
 struct FwdEpilogue {
@@ -75,7 +73,11 @@ int tma_gemm_wgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *X, fl
 size_t wgrad_scratch_elems(const ConvGeom &g);
 // Runs `gemms` (weight-gradient GEMMs on stream st, each with scratch of its own) and then one launch that adds the partial
 // tiles of all of them.
-int wgrad_batch(const std::function<int()> &gemms, cudaStream_t st);
+int wgrad_batch_of(int (*gemms)(void *), void *arg, cudaStream_t st);
+template <typename F>
+int wgrad_batch(F gemms, cudaStream_t st) {
+    return wgrad_batch_of([](void *f) -> int { return (*static_cast<F *>(f))(); }, &gemms, st);
+}
 int wgrad_reduce(const float *part, int jtiles, int ctiles, int splits, int BN, int Kfwd, int Co, float *dW, float *db,
                  int ones_row, cudaStream_t st);
 

@@ -1323,11 +1323,11 @@ int wgrad_reduce(const float *part, int jtiles, int ctiles, int splits, int BN, 
     return reduce_batch ? PPO_OK : launch_reductions(jobs, st);
 }
 
-int wgrad_batch(const std::function<int()> &gemms, cudaStream_t st) {
+int wgrad_batch_of(int (*gemms)(void *), void *arg, cudaStream_t st) {
     ReduceJobs jobs, *outer = reduce_batch;
     jobs.n = 0;
     reduce_batch = &jobs;
-    const int s = gemms();
+    const int s = gemms(arg);
     reduce_batch = outer;
     return s == PPO_OK ? launch_reductions(jobs, st) : s;
 }

@@ -1,7 +1,26 @@
 // Recorded launches (see launch.cuh).
 #include "launch.cuh"
 
-thread_local Launches *ppo_recording = nullptr;
+thread_local Recording *ppo_recording = nullptr;
+
+void ppo_record(const void *fn, dim3 grid, dim3 block, size_t smem, bool together, void *const *argv, const size_t *sizes, size_t n) noexcept {
+    try {
+        LaunchRecord r;
+        r.fn = fn;
+        r.grid = grid;
+        r.block = block;
+        r.smem = smem;
+        r.together = together;
+        for (size_t i = 0; i < n; ++i) {
+            r.offset.push_back((uint32_t)r.bytes.size());
+            const char *src = static_cast<const char *>(argv[i]);
+            r.bytes.insert(r.bytes.end(), src, src + sizes[i]);
+        }
+        ppo_recording->launches.push_back(std::move(r));
+    } catch (...) {
+        ppo_recording->complete = false;
+    }
+}
 
 int ppo_enqueue(const void *fn, dim3 grid, dim3 block, size_t smem, bool together, cudaStream_t st, void **argv) {
     cudaLaunchConfig_t c = {};

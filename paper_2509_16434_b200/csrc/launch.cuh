@@ -43,8 +43,13 @@ struct ppo_plans : PlanStore<PlanKey, Launches> {
     ppo_plans() : PlanStore(1024) {}  // operations of one model; a few MB of host memory
 };
 
-// The record of the operation being prepared on this thread (null: none).
-extern thread_local Launches *ppo_recording;
+// The operation being prepared on this thread.
+struct Recording {
+    Launches launches;
+    bool complete = true;  // false: memory ran out on the way; the launches were made all the same
+};
+extern thread_local Recording *ppo_recording;  // null: none
+void ppo_record(const void *fn, dim3 grid, dim3 block, size_t smem, bool together, void *const *argv, const size_t *sizes, size_t n) noexcept;
 
 int ppo_enqueue(const void *fn, dim3 grid, dim3 block, size_t smem, bool together, cudaStream_t st, void **argv);
 
@@ -57,20 +62,8 @@ int ppo_launch_as(bool together, void (*fn)(P...), dim3 grid, dim3 block, size_t
     std::tuple<std::remove_const_t<P>...> vals(static_cast<std::remove_const_t<P>>(args)...);
     std::apply([&](auto &...v) { ((argv[n++] = (void *)&v), ...); }, vals);
     if (ppo_recording) {
-        LaunchRecord r;
-        r.fn = reinterpret_cast<const void *>(fn);
-        r.grid = grid;
-        r.block = block;
-        r.smem = smem;
-        r.together = together;
-        n = 0;
         const size_t sizes[] = {sizeof(P)...};
-        for (size_t i = 0; i < sizeof...(P); ++i) {
-            r.offset.push_back((uint32_t)r.bytes.size());
-            const char *src = static_cast<const char *>(argv[i]);
-            r.bytes.insert(r.bytes.end(), src, src + sizes[i]);
-        }
-        ppo_recording->push_back(std::move(r));
+        ppo_record(reinterpret_cast<const void *>(fn), grid, block, smem, together, argv, sizes, sizeof...(P));
     }
     return ppo_enqueue(reinterpret_cast<const void *>(fn), grid, block, smem, together, st, argv);
 }

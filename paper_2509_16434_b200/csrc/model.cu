@@ -41,6 +41,12 @@ extern "C" int ppo_model_create(const ppo_model_desc *d, ppo_model **out) {
         return PPO_ERR_UNSUPPORTED;  // the trunk's input rows feed 64-channel boxes
     ppo_model *m = new (std::nothrow) ppo_model();
     if (!m) return PPO_ERR_INVALID_ARG;
+    try {
+        m->tensors.reserve(PPO_MAX_TENSORS);
+    } catch (...) {
+        delete m;
+        return PPO_ERR_INVALID_ARG;
+    }
     m->d = *d;
     m->L = d->n_conv;
     m->F = d->n_fc;
