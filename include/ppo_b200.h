@@ -290,7 +290,7 @@ int ppo_model_sync_shadow(ppo_model *m, void *stream);
  * Gaussian mean dev_mean [rows][A] and the value dev_value [rows] (fp32) and keeps the
  * activations in the workspace for ppo_encoder_bwd.  bf16 operands (weights from the
  * shadow, activations rounded to bf16 between layers), fp32 accumulation; the depth
- * frame enters as fp16.  A row's result does not depend on the other rows of the call, nor on
+ * frame enters as fp16 and has to be finite (a pixel may meet a zero weight).  A row's result does not depend on the other rows of the call, nor on
  * which call (this one or ppo_policy_act) computes it, with one exception: a one-step sequence
  * (T == 1 of ppo_model_set_sequence) of at most 1024 rows whose embedding has 2048 inputs or more
  * adds that sum up in up to eight slabs.  Such a step agrees with the same step inside a

@@ -19,7 +19,7 @@
 // What bounds it: the output's way to HBM and, on a level with it, the instructions of builders and epilogue (everything
 // about a group's shape is a template argument for that reason).  Copying every pair from global memory into its place
 // by itself (4 bytes per copy, 15 per pixel of a 5x5 window, each store a four-way bank conflict) was bound by the
-// copies.  4096 frames, before -> now (HBM time): 320x240 5x5 32 filters 2.05 -> 1.06 ms (0.88); 160x120 3x3 32 filters
+// copies.  4096 frames, 4-byte copies per pair -> rows (HBM time): 320x240 5x5 32 filters 2.05 -> 1.06 ms (0.88); 160x120 3x3 32 filters
 // 0.41 -> 0.25 (0.22); 160x120 3x3 16 filters normalised 0.51 -> 0.29 (0.22).
 // Frames must hold finite values (an Inf or NaN beside a window would meet a zero weight) and have an even
 // width.

@@ -15,9 +15,9 @@
 // per 64 columns and tile, clipped at the edges by the copy engine, instead of a shuffle, a load and a store per 16 bytes;
 // ReLU gates are fetched a tile ahead).  The weights stay in shared memory for the life of the CTA.  Sums run in the same
 // order as in gemm_tma.cu: the results are the same bits.
-// Measured, 4096 rows (against the HBM time of inputs, gates and outputs): 32 -> 64 channels on 160 x 120 forward
-// 2.22 -> 1.29 ms (1.17), input gradient 3.25 -> 1.37 (1.2); 64 -> 128 on 80 x 60 forward 1.20 -> 1.08 (0.58), input
-// gradient 1.58 -> 1.00 (0.6).
+// Measured, 4096 rows alone (tap boxes -> here; in brackets the HBM time of inputs, gates and outputs): 32 -> 64 channels on
+// 160 x 120 forward 2.22 -> 1.25 ms (1.17), input gradient 3.25 -> 1.28 (1.2); 64 -> 128 on 80 x 60 forward 1.20 -> 0.98
+// (0.58), input gradient 1.58 -> 1.01 to 1.07 (0.6).
 #include <cuda.h>
 
 #include "gemm.cuh"

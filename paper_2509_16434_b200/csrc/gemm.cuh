@@ -46,7 +46,8 @@ int tc_gemm_wgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *X, flo
                   int32_t *status, cudaStream_t st);
 
 // TMA-fed versions of the same three operations (operand tiles moved by cp.async.bulk.tensor).  They cover
-// channel counts that are multiples of 32 (any multiple of 8 that is at least 64 for a fully connected layer);
+// channel counts that are multiples of 16 (any multiple of 8 that is at least 64 for a fully connected layer; a merged
+// input gradient of 16-channel layers gates by activations, not by bits);
 // for anything else they return PPO_ERR_UNSUPPORTED without launching and the caller uses the tc_ versions.
 int tma_gemm_fwd(const ConvGeom &g, const bf16 *X, const bf16 *W, const FwdEpilogue &e, int32_t *status,
                  cudaStream_t st);

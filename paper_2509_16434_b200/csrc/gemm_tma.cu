@@ -1042,6 +1042,12 @@ int launch_kmajor(KArgs &a, cudaStream_t st) {
     a.stages = (int)(budget / (G * sub));
     if (a.stages > kMaxStages) a.stages = kMaxStages;
     if (a.stages < 2) return PPO_ERR_UNSUPPORTED;
+    // Producers.  Two CTAs on an SM are two producers already, and a second one in each costs the other CTA its place: 352
+    // threads of 96 registers do not fit twice (input gradient 256 -> 128 channels of 4096 images of 20 x 15: 252 us with one,
+    // 365 with two; forward 96 -> 128 on 40 x 30 413 and 646).  Alone on its SM a CTA of a single class takes two
+    // (forward 128 -> 256 on 20 x 15 195 us with one, 178 with two; 256 -> 256 359 and 338).  Several classes alone on an SM
+    // (merged input gradients wider than 128 columns, split reductions) keep one, which is not the faster choice: 256 -> 256 on
+    // 20 x 15 432 us with one and 416 with two, 96 -> 128 on 40 x 30 487 and 476, 8 slabs of 16 x 10240 9.1 and 8.4.
     a.nprod = two || a.ncls > 1 ? 1 : (a.stages < kProducers ? a.stages : kProducers);
     const int sms = ppo_num_sms();
     const long long ctas = two ? 2ll * sms : sms;
@@ -1126,9 +1132,9 @@ static void tma_dgrad_shifts(int k, int *dmin, int *n1) {
 // classes of input pixels are computed together.  Row (y, x) of the GEMM stands for the 2x2 block of input
 // pixels (2y + ph, 2x + pw); column class * Ci + ci; the reduction runs over the shifts (dy, dx) of the
 // output pixel (y + dy, x + dx) and its channels, with the weights Wc[class * Ci + ci][shift][co] (zero
-// where a class has no kernel tap at that shift).  One wide GEMM instead of four narrow ones: the tensor
-// core is fed by one thread, and an instruction of 64 columns or fewer occupies it as long as one of 128
-// (~55 cycles per issue at best; 128 columns run at the tensor rate of 64 cycles, 256 at 128).
+// where a class has no kernel tap at that shift).  One wide GEMM instead of four narrow ones: an instruction takes 41
+// cycles for 32 columns, 48 for 64, 64 for 128 and 128 for 256, so up to 128 columns wide ones do more per cycle,
+// and the operand rows of A are read once instead of once per class.
 int tma_gemm_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, int wt_ld, const bf16 *Wc,
                    const DgradEpilogue &e, int32_t *status, cudaStream_t st) {
     if (!status || g.Ci % 8 != 0 || ldy % 8 != 0 || wt_ld % 8 != 0 || ldy < wt_ld) return PPO_ERR_UNSUPPORTED;

@@ -1,7 +1,7 @@
 // The time loop of a recurrent layer as one persistent kernel per direction (sm_100a).
 //
-// A step's product with W_h is small (Be x 4H x H) and every step waits for the one before it, so launch by launch the loop
-// was a chain of 13 us GEMMs and 5 us cell kernels that mostly waited: for W_h from L2, for the pipeline to fill, for the
+// A step's product with W_h is small (Be x 4H x H) and every step waits for the one before it: launch by launch the loop is
+// a chain of 13 us GEMMs and 5 us cell kernels that mostly wait, for W_h from L2, for the pipeline to fill, for the
 // launch.  Here a CTA keeps its slice of W_h in shared memory for all steps, the cell runs on the accumulator (forward) or
 // between two exchanges (backward) with c and its gradient in registers, and the CTAs of a tile of 128 envs meet at a
 // counter in global memory once (forward) or twice (backward) per step.  What a step then costs is the 256 KB of h (or of
