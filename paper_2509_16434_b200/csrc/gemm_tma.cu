@@ -163,8 +163,9 @@ struct KArgs {
     int kchunks;            // boxes along the channels of one tap
     int w_tap;              // elements between taps in a weight row
     int G;                  // sub-blocks per stage
+    int batched;            // flat GEMM: one copy per operand brings all sub-blocks of a stage (channel chunks as a third axis)
     int tmem_cap;           // tensor-memory columns this CTA may take: 512, or 256 when two CTAs share an SM
-    int nepi;               // epilogue warps: 8, or 16 where the epilogue is the heavier side (dgrad with gate bits)
+    int nepi;               // epilogue warps: 8, or 16 where the epilogue is the heavier side (dgrad with gates)
     int nprod;              // producer warps: 1 .. min(kProducers, stages)
     int wres, wtaps;        // weights resident in shared memory (all wtaps * kchunks boxes, loaded once)
     int N, BN, tiles_n, total_tiles, ncls, stages;  // tile g = ((mt * tiles_n) + nt) * ncls + class
@@ -199,6 +200,16 @@ struct PipeK {
     // followed by the epilogue staging: per epilogue warp 32 rows x 32 bf16 columns (2 KB), 16-byte pieces swizzled
 };
 
+// All ones over each half of a bf16 pair that is > 0.
+__device__ __forceinline__ uint32_t gate_open(uint32_t pair) {
+    return __hgt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&pair), __float2bfloat162_rn(0.f));
+}
+
+// A kernel each for forward passes, input gradients and input gradients whose gate is the bf16 activation: in one, the
+// registers of the widest epilogue would spill the others'.
+enum { KIND_FWD = 0, KIND_DGRAD = 1, KIND_DGRAD_ACT = 2 };
+
+template <int KIND>
 __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_constant__ KArgs a) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -207,6 +218,8 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
     const uint32_t a_bytes = a.a_bytes, b_bytes = (uint32_t)BN * rb;
     const uint32_t sub_bytes = a_bytes + (a.wres ? 0u : b_bytes);
     const uint32_t stage_bytes = (uint32_t)G * sub_bytes;
+    // a stage is A and B of sub-block after sub-block, or (batched) all A and behind them all B
+    const uint32_t a_step = a.batched ? a_bytes : sub_bytes, b_off = a.batched ? (uint32_t)G * a_bytes : a_bytes;
     const uint32_t res_bytes = a.wres ? (uint32_t)(a.wtaps * a.kchunks) * b_bytes : 0u;
     PipeK *pipe = reinterpret_cast<PipeK *>(smem + (size_t)S * stage_bytes + res_bytes);
     volatile int *abort_flag = &pipe->abort_flag;
@@ -231,9 +244,9 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
     }
     if (warp == 1) tmem_alloc(&pipe->tmem_slot, ncols);
     grid_wait();
-    if (a.mode != EPI_DGRAD)
+    if (KIND == KIND_FWD)
         for (int i = threadIdx.x; i < a.tiles_n * BN; i += (int)blockDim.x) pipe->bias[i] = i < a.N ? a.bias[i] : 0.f;
-    if (a.ln_gamma)
+    if (KIND == KIND_FWD && a.ln_gamma)
         for (int i = threadIdx.x; i < 256; i += (int)blockDim.x) {
             pipe->gamma[i] = i < a.N ? a.ln_gamma[i] : 0.f;
             pipe->beta[i] = i < a.N ? a.ln_beta[i] : 0.f;
@@ -272,13 +285,18 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
             const int brow = tc_.nt * BN + k.b_row0, ntaps = k.taps.n, nsub = ntaps * a.kchunks;
             const int cx = pt.xs * a.grid.Wt * a.s_mul + a.s_ox;
             int tap = 0, kc = (it - it0) * G;
-            while (kc >= a.kchunks) { kc -= a.kchunks; ++tap; }
+            while (!a.batched && kc >= a.kchunks) { kc -= a.kchunks; ++tap; }
             for (int q0 = (it - it0) * G; q0 < nsub; q0 += np * G, it += np) {
                 ok = mbar_wait_warp(&pipe->empty[s], ph ^ 1u, abort_flag, a.status);
                 if (!ok) break;
-                const int nval = min(G, nsub - q0);
-                if (elect_one()) mbar_arrive_expect_tx(&pipe->full[s], (uint32_t)nval * tx_sub);
+                const int nval = a.batched ? 0 : min(G, nsub - q0);
+                if (elect_one()) mbar_arrive_expect_tx(&pipe->full[s], (uint32_t)(a.batched ? G : nval) * tx_sub);
                 uint32_t dst = smem_base + (uint32_t)s * stage_bytes;
+                if (a.batched) {  // chunks behind the last arrive as zeros; one kernel tap, one pixel row
+                    if (elect_one()) tma_load_4d(dst, &a.mapA[0], &pipe->full[s], 0, cx, kc, 0);
+                    if (!a.wres && elect_one()) tma_load_4d(dst + b_off, &a.mapB, &pipe->full[s], 0, brow, kc, 0);
+                    kc += G;
+                }
                 for (int gi = 0; gi < nval; ++gi, dst += sub_bytes) {
                     const int dx = k.taps.dx[tap], dy = k.taps.dy[tap];
                     int n = pt.n, y = pt.y, row = 0;
@@ -300,7 +318,7 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
                 if (s >= S) { s -= S; ph ^= 1u; }
                 if (np > 1) {
                     kc += (np - 1) * G;
-                    while (kc >= a.kchunks) { kc -= a.kchunks; ++tap; }
+                    while (!a.batched && kc >= a.kchunks) { kc -= a.kchunks; ++tap; }
                 }
             }
             it0 += (nsub + G - 1) / G;
@@ -315,7 +333,8 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
         const uint64_t d0 = smem_desc_sw(smem_base, 16, sbo, rb);
         const uint32_t d_lo0 = (uint32_t)d0, d_hi = (uint32_t)(d0 >> 32);
         const uint32_t res_lo0 = d_lo0 + ((res_base - smem_base) >> 4);
-        const uint32_t stage16 = stage_bytes >> 4, sub16 = sub_bytes >> 4, ab16 = a_bytes >> 4, b16 = b_bytes >> 4;
+        const uint32_t stage16 = stage_bytes >> 4, a16 = a_step >> 4, b16 = b_bytes >> 4;
+        const uint32_t boff16 = b_off >> 4, bstep16 = a.batched ? b16 : a16;
         const int ksteps = a.CB >> 4;  // 4, 2 or 1 K = 16 steps per box (32 bytes each along the swizzled row)
         int ti = 0, s = 0;
         uint32_t ph = 0;
@@ -337,9 +356,9 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
                 if (!ok) break;
                 tc_fence_after();
                 const int nval = min(G, nsub - q0);
-                uint32_t la = d_lo0 + (uint32_t)s * stage16;
-                for (int gi = 0; gi < nval; ++gi, la += sub16) {
-                    uint32_t lb = la + ab16;
+                uint32_t la = d_lo0 + (uint32_t)s * stage16, ls = la + boff16;
+                for (int gi = 0; gi < nval; ++gi, la += a16, ls += bstep16) {
+                    uint32_t lb = ls;
                     if (a.wres) {
                         lb = res_lo0 + (uint32_t)((int)a.cls[c].taps.wt[tap] * a.kchunks + kc) * b16;
                         if (++kc == a.kchunks) { kc = 0; ++tap; }
@@ -407,16 +426,18 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
                 return pix_ok && oy < a.Hout && ox < a.Wout;
             };
             const int ncol = a.nq_ci ? a.nq_ci : a.N;  // columns of an output row
-            const bool use_bits = a.mode == EPI_DGRAD && a.mask_bits != nullptr;
-            const bool use_mask = a.mode == EPI_DGRAD && a.mask != nullptr && !use_bits;
+            constexpr bool fwd = KIND == KIND_FWD, use_mask = KIND == KIND_DGRAD_ACT;
+            const bool use_bits = KIND == KIND_DGRAD && a.mask_bits != nullptr;
             const int acc = ti & (nacc - 1);
             const uint32_t lane_base = tmem_base + acc * acc_cols + ((uint32_t)(lg * 32) << 16);
-            if (a.out != nullptr && a.out_f32 == nullptr && a.mode != EPI_HEAD && !use_mask) {
+            if (a.out != nullptr && a.out_f32 == nullptr && (!use_mask || (a.nq_ci & 31) == 0)) {
                 // ---- bf16 outputs, staged: a thread owns a pixel (its TMEM lane), but a warp that stores 32
                 // pixels with one instruction touches 32 cache lines.  So 32-column groups pass through a small
                 // swizzled shared-memory tile: four lanes then move one pixel's 64 contiguous bytes, and an
-                // instruction covers 8 lines.  The ReLU mask comes in the same way, and the first group's mask
-                // is fetched before the accumulator is waited for, so that its latency overlaps the MMAs.
+                // instruction covers 8 lines.  Gate bits are fetched before the accumulator is waited for, so that their
+                // latency overlaps the MMAs.  Where the gate is the activation itself, the lane that stores 16 bytes reads
+                // the 16 bytes of the gate: whole lines again, a group ahead of its use (each thread reading and storing its
+                // own row touched a line for every 32 bytes: input gradient of 512 <- 512 columns, 4096 rows, 16.4 -> 12.9 us).
                 uint4 *stg = reinterpret_cast<uint4 *>(pipe + 1) + (size_t)(warp - 2) * 128;
                 const int sw = (lane >> 1) & 3;
                 const int rr0 = lane >> 2, piece = lane & 3;
@@ -434,6 +455,22 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
                         }
                     }
                 }
+                uint4 gact[4];  // this lane's pieces of the next group's gate
+                auto fetch_gate = [&](int g) {
+                    const int c0 = (ew4 + wq * g) * 32;
+                    long long orow;
+                    int col;
+                    const int okr = g < ng && locate(c0, orow, col) ? 1 : 0;
+#pragma unroll
+                    for (int ps = 0; ps < 4; ++ps) {
+                        const long long o_r = __shfl_sync(0xffffffffu, orow, ps * 8 + rr0);
+                        const int ok_r = __shfl_sync(0xffffffffu, okr, ps * 8 + rr0);
+                        gact[ps] = make_uint4(0, 0, 0, 0);
+                        if (ok_r && col + piece * 8 < ncol && c0 + piece * 8 < BN)
+                            gact[ps] = __ldg(reinterpret_cast<const uint4 *>(a.mask + o_r * a.ldo + col + piece * 8));
+                    }
+                };
+                if constexpr (use_mask) fetch_gate(0);
                 ok = mbar_wait(&pipe->tfull[acc], (ti >> nacc_log) & 1, abort_flag, a.status);
                 if (!ok) break;
                 tc_fence_after();
@@ -441,7 +478,7 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
                 // every warp of the lane quarter walks the whole row twice (mean, then variance about it) before it
                 // normalises its own column groups.
                 float ln_mean = 0.f, ln_rs = 0.f;
-                if (a.ln_gamma) {
+                if (fwd && a.ln_gamma) {
                     float sum = 0.f;
                     for (int c0 = 0; c0 < a.N; c0 += 16) {
                         float t[16];
@@ -473,14 +510,14 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
                     int col;
                     const int okr = locate(c0, orow, col) ? 1 : 0;
                     uint32_t pk[16];
-                    if (a.mode == EPI_FWD) {
+                    if (fwd) {
                         const float4 *bp = reinterpret_cast<const float4 *>(pipe->bias + n0 + c0);
 #pragma unroll
                         for (int q = 0; q < 8; ++q) {
                             const float4 bv = bp[q];
                             v[4 * q] += bv.x; v[4 * q + 1] += bv.y; v[4 * q + 2] += bv.z; v[4 * q + 3] += bv.w;
                         }
-                        if (a.ln_gamma) {
+                        if (fwd && a.ln_gamma) {
                             // the normalised values go out first (same staging, same store pattern), then v becomes
                             // gamma * xhat + beta and takes the usual path
 #pragma unroll
@@ -532,10 +569,16 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
                         const int rr = ps * 8 + rr0;
                         const long long o_r = __shfl_sync(0xffffffffu, orow, rr);
                         const int ok_r = __shfl_sync(0xffffffffu, okr, rr);
-                        if (ok_r && col + piece * 8 < ncol && c0 + piece * 8 < BN)
-                            *reinterpret_cast<uint4 *>(a.out + o_r * a.ldo + col + piece * 8) =
-                                stg[rr * 4 + (piece ^ ((rr >> 1) & 3))];
+                        if (ok_r && col + piece * 8 < ncol && c0 + piece * 8 < BN) {
+                            uint4 v4 = stg[rr * 4 + (piece ^ ((rr >> 1) & 3))];
+                            if constexpr (use_mask) {  // a comparison: minus zero, negative numbers and NaN close the gate
+                                v4.x &= gate_open(gact[ps].x); v4.y &= gate_open(gact[ps].y);
+                                v4.z &= gate_open(gact[ps].z); v4.w &= gate_open(gact[ps].w);
+                            }
+                            *reinterpret_cast<uint4 *>(a.out + o_r * a.ldo + col + piece * 8) = v4;
+                        }
                     }
+                    if constexpr (use_mask) fetch_gate(g + 1);
                     __syncwarp();
                 }
                 tc_fence_before();
@@ -553,7 +596,7 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
                 long long orow;
                 int nn;
                 if (!locate(c0, orow, nn)) continue;
-                if (a.mode == EPI_HEAD) {
+                if (fwd) {
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
                         if (nn + i < a.A) a.mean[orow * a.A + nn + i] = v[i] + pipe->bias[nn + i];
@@ -963,30 +1006,41 @@ int pick_bn(int N) {  // tile width: N split evenly into tiles of at most 256, r
     return bn < 16 ? 16 : bn;
 }
 
-// Tile width of a flat GEMM (rows x N): as pick_bn, then halved while the tiles would leave more than half of the SMs
-// without work (few rows, as in the per-step products of a recurrent layer) and the halves still divide N.
+// Tile width of a flat GEMM (rows x N): as pick_bn, then cut into twice as many tiles, down to 32 columns, while the tiles
+// would leave more than half of the SMs without work (few rows, as in the per-step products of a recurrent layer).  Forward
+// passes keep their bias in kMaxBias places, so the widened last tile has to end there.
 static int flat_bn(int N, long long rows) {
-    int bn = pick_bn(N);
+    int tiles = (N + 255) / 256, bn = pick_bn(N);
     const long long mt = (rows + 127) / 128;
-    while (bn >= 64 && bn % 32 == 0 && N % (bn / 2) == 0 && mt * ((N + bn - 1) / bn) < ppo_num_sms() / 2) bn /= 2;
+    while (bn > 32 && mt * ((N + bn - 1) / bn) < ppo_num_sms() / 2) {
+        tiles *= 2;
+        const int half = ((N + tiles - 1) / tiles + 15) / 16 * 16;
+        if (half < 32 || (N <= kMaxBias && (N + half - 1) / half * half > kMaxBias)) break;
+        bn = half;
+    }
     return bn;
 }
 
 // Grid of a flat GEMM's rows: tiles of 128, halved (down to 32) while the tiles would leave more than half of the SMs
 // without work.  A CTA's time is the length of its reduction (copies and one MMA per 16 of K, nothing amortises them), so
-// rows are better spread over idle SMs.
-static bool make_flat_grid(RowGrid &g, long long rows, int tiles_n, int row_bytes) {
-    if (!make_grid(g, (int)rows, 1, 1, row_bytes)) return false;
-    int Wt = g.Wt;
-    while (Wt % 2 == 0 && Wt / 2 >= 32 && (Wt / 2) * row_bytes % 1024 == 0 && 2ll * g.xsegs * tiles_n <= ppo_num_sms()) {
-        Wt /= 2;
-        g.Wt = Wt;
-        g.xsegs = (int)((rows + Wt - 1) / Wt);
-        g.tiles = g.xsegs;
-        g.arows = Wt;
-    }
+// rows are better spread over idle SMs.  The last tile is ragged: tiles of equal odd widths could not be halved, and 356 rows
+// of a 38400-column map took 3 CTAs 124 us.
+static bool make_flat_grid(RowGrid &g, long long rows, int tiles_n) {
+    int Wt = 128;
+    while (Wt > 32 && (Wt / 2 >= rows || 2 * ((rows + Wt - 1) / Wt) * tiles_n <= ppo_num_sms())) Wt /= 2;
+    if (rows < 32) Wt = ((int)rows + 7) / 8 * 8;
+    const long long tiles = (rows + Wt - 1) / Wt;
+    if (rows < 1 || tiles > 0x3fffffff) return false;
+    g.Wr = (int)rows; g.Hr = 1; g.Nimg = 1;
+    g.Wt = Wt; g.xsegs = g.tiles = (int)tiles; g.R = 1; g.arows = Wt;
     return true;
 }
+
+// Operands of a flat GEMM: rows of K columns, `ldx` and `ldw` elements apart.
+struct FlatOps {
+    const bf16 *X, *W;
+    long long ldx, ldw, K;
+};
 
 int ensure_smem_attrs() {
     static bool attr_set[64] = {false};
@@ -995,15 +1049,18 @@ int ensure_smem_attrs() {
     if (dev < 0 || dev >= 64) return PPO_ERR_CUDA;
     if (!attr_set[dev]) {
         const int mx = (int)(kSmemBudget + sizeof(PipeK) + 1024);
-        PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_kmajor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+        PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_kmajor_kernel<KIND_FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+        PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_kmajor_kernel<KIND_DGRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+        PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_kmajor_kernel<KIND_DGRAD_ACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
         PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
         attr_set[dev] = true;
     }
     return PPO_OK;
 }
 
-// `a.wtaps` = taps of the whole weight tensor (all classes).
-int launch_kmajor(KArgs &a, cudaStream_t st) {
+// `a.wtaps` = taps of the whole weight tensor (all classes).  ops: operands of a flat GEMM of one class, whose copies may then
+// take several chunks at a time.
+int launch_kmajor(KArgs &a, cudaStream_t st, const FlatOps *ops = nullptr) {
     int s = ensure_smem_attrs();
     if (s != PPO_OK) return s;
     a.tiles_n = (a.N + a.BN - 1) / a.BN;
@@ -1027,7 +1084,7 @@ int launch_kmajor(KArgs &a, cudaStream_t st) {
     const bool small_m = (a.grid.tiles <= 4 || (flat && total <= ppo_num_sms())) && (a.ncls == 1 || a.cls_orows != 0);
     const bool two = a.BN <= 128 && !small_m;
     a.tmem_cap = two ? 256 : 512;
-    a.nepi = (!two && a.mode == EPI_DGRAD && a.mask_bits) ? 16 : 8;
+    a.nepi = (!two && a.mode == EPI_DGRAD && (a.mask_bits || a.mask)) ? 16 : 8;
     const size_t fixed = sizeof(PipeK) + (size_t)a.nepi * 2048 + 1024;  // pipeline state, epilogue staging, alignment slack
     const size_t cta_max = two ? kSmemMax / 2 : kSmemMax;
     // (the rows an MMA reads beyond a_bytes of the last sub-block lie in the pipeline state and staging, at least 16 KB)
@@ -1037,8 +1094,22 @@ int launch_kmajor(KArgs &a, cudaStream_t st) {
     const size_t budget = cta_max - 1024 - fixed - (a.wres ? res : 0);
     int G = (int)(((small_m ? 96 : 48) * 1024) / sub);  // sub-blocks per stage: fewer barrier round trips per byte
     G = G < 1 ? 1 : (G > 8 ? 8 : G);
+    if (flat && G > a.kchunks) G = a.kchunks;
     while (G > 1 && budget / (G * sub) < (small_m ? 2 : 3)) --G;
     a.G = G;
+    // A copy costs the warp that issues it 110 to 220 cycles, and a chunk of a flat GEMM is small: where K is whole chunks they
+    // become a third axis of the map and one copy per operand fills a stage.
+    if (ops && G > 1 && ops->K % a.CB == 0 && a.grid.arows * a.row_bytes % 1024 == 0) {
+        a.batched = 1;
+        const long long da[4] = {a.CB, a.grid.Wr, a.kchunks, 1}, sa[3] = {2 * ops->ldx, 2ll * a.CB, 2 * ops->ldx * a.grid.Wr};
+        const int ba[4] = {a.CB, a.grid.Wt, G, 1};
+        PPO_TRY(make_map_strided(&a.mapA[0], ops->X, 4, da, sa, ba));
+        if (!a.wres) {
+            const long long db[4] = {a.CB, a.N, a.kchunks, 1}, sb[3] = {2 * ops->ldw, 2ll * a.CB, 2 * ops->ldw * a.N};
+            const int bb[4] = {a.CB, a.BN, G, 1};
+            PPO_TRY(make_map_strided(&a.mapB, ops->W, 4, db, sb, bb));
+        }
+    }
     a.stages = (int)(budget / (G * sub));
     if (a.stages > kMaxStages) a.stages = kMaxStages;
     if (a.stages < 2) return PPO_ERR_UNSUPPORTED;
@@ -1053,7 +1124,9 @@ int launch_kmajor(KArgs &a, cudaStream_t st) {
     const long long ctas = two ? 2ll * sms : sms;
     const unsigned grid = (unsigned)(total < ctas ? total : ctas);
     const size_t smem = (size_t)a.stages * G * sub + (a.wres ? res : 0) + fixed;
-    PPO_TRY(ppo_launch(tma_kmajor_kernel, dim3(grid), dim3((1 + a.nprod + a.nepi) * 32), smem, st, a));
+    const auto fn = a.mode != EPI_DGRAD ? tma_kmajor_kernel<KIND_FWD>
+                                        : (a.mask && !a.mask_bits ? tma_kmajor_kernel<KIND_DGRAD_ACT> : tma_kmajor_kernel<KIND_DGRAD>);
+    PPO_TRY(ppo_launch(fn, dim3(grid), dim3((1 + a.nprod + a.nepi) * 32), smem, st, a));
     return PPO_OK;
 }
 
@@ -1076,7 +1149,7 @@ int tma_gemm_fwd(const ConvGeom &g, const bf16 *X, const bf16 *W, const FwdEpilo
     a.N = g.Co;
     a.BN = flat && e.out ? flat_bn(g.Co, g.B) : pick_bn(g.Co);
     // a fully connected layer is one image with a single row of B pixels
-    const bool ok = flat ? make_flat_grid(a.grid, g.B, (a.N + a.BN - 1) / a.BN, a.row_bytes) : make_grid(a.grid, g.Wo, g.Ho, g.B, a.row_bytes);
+    const bool ok = flat ? make_flat_grid(a.grid, g.B, (a.N + a.BN - 1) / a.BN) : make_grid(a.grid, g.Wo, g.Ho, g.B, a.row_bytes);
     if (!ok) return PPO_ERR_UNSUPPORTED;
     int s = flat ? make_act_maps(a.mapA, X, g.Ci, g.Ci, g.B, 1, 1, a.grid, CB, 1)
                  : make_act_maps(a.mapA, X, g.Ci, g.Ci, g.Wi, g.Hi, g.B, a.grid, CB, 2);
@@ -1119,7 +1192,8 @@ int tma_gemm_fwd(const ConvGeom &g, const bf16 *X, const bf16 *W, const FwdEpilo
         k.taps.dx[t] = (signed char)(t % g.k);
         k.taps.wt[t] = (short)t;
     }
-    return launch_kmajor(a, st);
+    const FlatOps ops = {X, W, g.Ci, g.K(), g.Ci};
+    return launch_kmajor(a, st, flat ? &ops : nullptr);
 }
 
 static void tma_dgrad_shifts(int k, int *dmin, int *n1) {
@@ -1154,7 +1228,7 @@ int tma_gemm_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, i
     a.w_tap = wt_ld;
     const int Hr = flat ? 1 : (g.Hi + 1) / 2, Wr = flat ? g.B : (g.Wi + 1) / 2;
     const int flat_n = flat ? flat_bn(g.Ci, g.B) : 0;
-    if (!(flat && e.ksplit <= 1 ? make_flat_grid(a.grid, g.B, (g.Ci + flat_n - 1) / flat_n, a.row_bytes)
+    if (!(flat && e.ksplit <= 1 ? make_flat_grid(a.grid, g.B, (g.Ci + flat_n - 1) / flat_n)
                                 : make_grid(a.grid, Wr, Hr, flat ? 1 : g.B, a.row_bytes)))
         return PPO_ERR_UNSUPPORTED;
     int s = flat ? make_act_maps(a.mapA, dY, head ? 16 : g.Co, ldy, g.B, 1, 1, a.grid, CB, 1)
@@ -1222,7 +1296,8 @@ int tma_gemm_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, i
         k.taps.n = 1;
         k.taps.dy[0] = k.taps.dx[0] = 0;
         k.taps.wt[0] = 0;
-        return launch_kmajor(a, st);
+        const FlatOps ops = {dY, Wt, ldy, wt_ld, g.Co};
+        return launch_kmajor(a, st, &ops);
     }
     int dmin, n1;
     tma_dgrad_shifts(g.k, &dmin, &n1);
