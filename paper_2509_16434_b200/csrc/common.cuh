@@ -111,7 +111,7 @@ struct ppo_model {
     // workspace carve
     bf16 *act[PPO_MAX_CONV + 1];   // act[l], l >= 1: [mb][Ho][Wo][C] post-ReLU
     bf16 *dact[PPO_MAX_CONV + 1];  // gradient w.r.t. the pre-activation of act[l]
-    uint32_t *abits[PPO_MAX_CONV + 1];  // ReLU gate of act[l], one bit per element (layers with C % 32 == 0, else null)
+    uint32_t *abits[PPO_MAX_CONV + 1];  // ReLU gate of act[l], one bit per element (layers with C % 32 == 0 or C == 16, else null)
     bf16 *xhat[PPO_MAX_CONV + 1];   // with norm: normalised values of conv layer l, [mb][Ho][Wo][C]
     float *rstd[PPO_MAX_CONV + 1];  // with norm: 1 / sqrt(var + eps) per pixel, [mb][Ho][Wo]
     bf16 *dze;                      // with embed: gradient w.r.t. the embedding's pre-activation, [mb][E]
@@ -174,6 +174,10 @@ __device__ __forceinline__ uint32_t gate_bits_add(uint32_t gate, uint32_t pair, 
     const uint32_t on = __hgt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&pair), __float2bfloat162_rn(0.f));
     return gate | (on & (0x00010001u << j));
 }
+// The gates of a 16-channel pixel are a half word: pair j owns bits j and 8 + j.
+__device__ __forceinline__ uint16_t gate_half(uint32_t gate) { return (uint16_t)((gate & 0xFFu) | ((gate >> 8) & 0xFF00u)); }
+// Two of them as one word, the pairs of the first pixel in front: pair j owns bits j and 16 + j.
+__device__ __forceinline__ uint32_t gate_of_halves(uint32_t first, uint32_t second) { return __byte_perm(first, second, 0x5140); }
 __device__ __forceinline__ uint32_t gate_pair_mask(uint32_t gate, int j) {
     return ((gate >> j) & 0x00010001u) * 0xFFFFu;
 }

@@ -46,7 +46,7 @@ struct Args {
     const __half *depth;
     const bf16 *W;      // [C1][k*k] bf16
     const float *bias;  // [C1]
-    uint32_t *bits;     // [M][C1 / 32] or null
+    uint32_t *bits;     // [M][C1 / 32], [M] half words for C1 = 16, or null
     const float *ln_gamma, *ln_beta;  // layer normalisation over the C1 channels of a pixel (null: none; C1 = 16 or 32)
     float *ln_rstd;     // [M]
     long long M;        // output pixels
@@ -385,9 +385,12 @@ __global__ void __launch_bounds__(kThreads, 1) conv1_tc_kernel(const __grid_cons
 #pragma unroll
                 for (int j = 0; j < CW / 2; ++j) {
                     pk[j] = relu_pack_bf16x2(v[2 * j], v[2 * j + 1]);
-                    if (CW == 32) gate = gate_bits_add(gate, pk[j], j);
+                    gate = gate_bits_add(gate, pk[j], j);
                 }
-                if (CW == 32 && a.bits && m0 + lane < a.M) a.bits[(m0 + lane) * (N >> 5) + (c0 >> 5)] = gate;
+                if (a.bits && m0 + lane < a.M) {
+                    if (CW == 32) a.bits[(m0 + lane) * (N >> 5) + (c0 >> 5)] = gate;
+                    else reinterpret_cast<uint16_t *>(a.bits)[m0 + lane] = gate_half(gate);
+                }
                 emit(&a.map_out, pk, c0, m0);
             }
             tc_fence_before();
@@ -445,13 +448,13 @@ int launch_c(Args &a, cudaStream_t st) {
 
 }  // namespace
 
-// out[m][co] = relu(bias[co] + sum_tap depth(m, tap) * W[co][tap]) as bf16; `bits` (optional, C1 % 32 == 0) gets the
+// out[m][co] = relu(bias[co] + sum_tap depth(m, tap) * W[co][tap]) as bf16; `bits` (optional, C1 % 32 == 0 or C1 = 16) gets the
 // ReLU gates.  Returns PPO_ERR_UNSUPPORTED (nothing launched) for shapes it does not cover: C1 must be a multiple
-// of 16 up to 64 (of 32 when bits are wanted), k in {3, 5, 7}, the frame width even and the frames 4-byte aligned.
+// of 16 up to 64 (not 48 when bits are wanted), k in {3, 5, 7}, the frame width even and the frames 4-byte aligned.
 int conv1_tc_fwd(const __half *depth, const bf16 *W, const float *bias, bf16 *out, uint32_t *bits, int rows, int Hi,
                  int Wi, int Ho, int Wo, int C1, int ks, const float *ln_gamma, const float *ln_beta, bf16 *ln_xhat,
                  float *ln_rstd, int32_t *status, cudaStream_t st) {
-    if (!status || C1 % 16 != 0 || C1 > 64 || C1 < 16 || (bits && C1 % 32 != 0)) return PPO_ERR_UNSUPPORTED;
+    if (!status || C1 % 16 != 0 || C1 > 64 || C1 < 16 || (bits && C1 % 32 != 0 && C1 != 16)) return PPO_ERR_UNSUPPORTED;
     if (ln_gamma && ((C1 != 16 && C1 != 32) || !ln_beta || !ln_xhat || !ln_rstd)) return PPO_ERR_UNSUPPORTED;
     if (Wi % 2 != 0 || !ppo_aligned(depth, 4)) return PPO_ERR_UNSUPPORTED;
     Args a = {};

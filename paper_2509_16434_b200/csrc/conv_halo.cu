@@ -37,7 +37,7 @@ constexpr int kMaxSlots = 8;
 constexpr int kMaxOps = 9;
 constexpr size_t kSmemMax = 227 * 1024;
 
-enum { FWD = 0, FWD_LN = 1, DG_BITS = 2, DG_ACT = 3 };
+enum { FWD = 0, FWD_LN = 1, DG = 2 };
 
 // One tap of a plane: CB / 16 MMAs over the channels of a chunk.
 struct Op {
@@ -72,7 +72,6 @@ struct Args {
     uint32_t stg_bytes;     // of a staging buffer
     int stg_row;            // of a row of it, over all its output groups
     int epw;                // warps of an epilogue group
-    bool wide_gate;         // gates come as 16 activations per pixel: too many registers for a whole row per thread
     int slots, nbuf, neg;   // slots, staging buffers per epilogue group, epilogue groups
     int Wt, R, I, Wp, Rp;   // tile: Wt x R outputs of I images; cells per box row and box rows per image
     int xsegs, ysegs, tiles;
@@ -84,7 +83,6 @@ struct Args {
     int relu;
     uint32_t *out_bits;
     const uint32_t *mask_bits;
-    const bf16 *mask;
     const float *ln_gamma, *ln_beta;
     float *ln_rstd;
     int grid;
@@ -407,31 +405,22 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
         // ReLU gates of the pixels this thread's columns belong to.  They are fetched a tile ahead: this warp is what the
         // tile waits for, so a load on its own tile's path would cost its whole latency.
         uint32_t gate[4], gate_n[4];
-        uint4 act[4], act_n[4];
         auto fetch_gates = [&](const TileAt &at) {
             const int n = at.n + ci, y = at.y + cr, x = at.x + cx;
             const bool live = cell && n < a.B && y < a.Hr && x < a.Wr;
-            if (MODE == DG_BITS) {
+            if (MODE == DG) {
+                auto word = [&](int col) -> uint32_t {  // gates of the class that owns column col (a half word for 16 channels)
+                    const int grp = col / GC, iy = 2 * y + (grp >> 1), ix = 2 * x + ((grp == 1 || grp == 2) ? 1 : 0);
+                    if (col >= a.N || !live || iy >= a.Hi || ix >= a.Wi) return 0u;
+                    const long long px = ((long long)n * a.Hi + iy) * a.Wi + ix;
+                    if (GC == 16) return __ldg(reinterpret_cast<const uint16_t *>(a.mask_bits) + px);
+                    return __ldg(a.mask_bits + px * (GC / 32 > 0 ? GC / 32 : 1) + (GC == 64 ? (col >> 5) & 1 : 0));
+                };
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {  // step k / NH, half k % NH (EPW == 4: at most 128 columns)
-                    gate_n[k] = 0u;
-                    const int hh = EPW == 4 ? k % NH : h, col = (k / NH) * 64 + hh * 32, grp = col / GC;
-                    const int iy = 2 * y + (grp >> 1), ix = 2 * x + ((grp == 1 || grp == 2) ? 1 : 0);
-                    if (col < a.N && live && iy < a.Hi && ix < a.Wi)
-                        gate_n[k] = __ldg(a.mask_bits + (((long long)n * a.Hi + iy) * a.Wi + ix) * (GC / 32 > 0 ? GC / 32 : 1) + (GC == 64 ? hh : 0));
-                }
-            }
-            if (MODE == DG_ACT) {  // GC == 16: this thread's 32 columns are two classes of 16 channels
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const int grp = h * 2 + e;
-                    const int iy = 2 * y + (grp >> 1), ix = 2 * x + ((grp == 1 || grp == 2) ? 1 : 0);
-                    act_n[2 * e] = act_n[2 * e + 1] = make_uint4(0, 0, 0, 0);
-                    if (live && iy < a.Hi && ix < a.Wi) {
-                        const uint4 *mp = reinterpret_cast<const uint4 *>(a.mask + (((long long)n * a.Hi + iy) * a.Wi + ix) * 16);
-                        act_n[2 * e] = __ldg(mp);
-                        act_n[2 * e + 1] = __ldg(mp + 1);
-                    }
+                    const int col = (k / NH) * 64 + (EPW == 4 ? k % NH : h) * 32;
+                    if (GC == 16) gate_n[k] = k < NH ? gate_of_halves(word(col), word(col + 16)) : 0u;  // 64 columns: one step
+                    else gate_n[k] = word(col);
                 }
             }
         };
@@ -442,8 +431,7 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
             const bool live = cell && n < a.B && y < a.Hr && x < a.Wr;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                if (MODE == DG_BITS) gate[k] = gate_n[k];
-                if (MODE == DG_ACT) act[k] = act_n[k];
+                if (MODE == DG) gate[k] = gate_n[k];
             }
             for (int k = 0; k < a.neg; ++k) t_next.next(a);
             if (li + a.neg < nt) fetch_gates(t_next);
@@ -573,22 +561,13 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
                             uint32_t pk[4];
 #pragma unroll
                             for (int j = 0; j < 4; ++j) {
-                                const uint32_t pr = pack_bf16x2(v[8 * k + 2 * j], v[8 * k + 2 * j + 1]);
-                                if (MODE == DG_BITS) {
-                                    pk[j] = pr & gate_mask(gw, 4 * k + j);
-                                } else {
-                                    const uint4 &q4 = act[k];
-                                    const uint32_t aw = j == 0 ? q4.x : (j == 1 ? q4.y : (j == 2 ? q4.z : q4.w));
-                                    // a comparison, as wherever a gate is read: saved activations can be written from outside,
-                                    // and minus zero, negative numbers and NaN close it
-                                    pk[j] = pr & __hgt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&aw), __float2bfloat162_rn(0.f));
-                                }
+                                pk[j] = pack_bf16x2(v[8 * k + 2 * j], v[8 * k + 2 * j + 1]) & gate_mask(gw, 4 * k + j);
                             }
                             put(stg, hh * 32 + 8 * k, make_uint4(pk[0], pk[1], pk[2], pk[3]));
                         }
                     }
                 }
-                store_step(stg, s, MODE == DG_BITS || MODE == DG_ACT ? a.mapO : &a.mapO[0]);
+                store_step(stg, s, a.mapO);
             }
             acc += a.neg;
             if (acc >= nacc) { acc = eg; aph ^= 1u; }
@@ -673,7 +652,6 @@ bool plan(Args &a, int Wr, int Hr, int B) {
         // channels: 1.49 -> 1.29 ms), a single step of 32 columns and normalised rows; a plain forward tile of 64 columns and
         // more wants the room for its next two planes (1.30 against 1.48 ms).
         a.epw = a.ln_gamma || (two && (a.nloads != 4 || a.N == 32)) ? 4 : 8;
-        if (a.wide_gate) a.epw = 8;
         a.nacc = (two ? 256 : 512) / a.acc_cols;
         if (a.nacc > 4) a.nacc = 4;
         if (a.nacc < 2) continue;
@@ -728,8 +706,7 @@ int launch_epw(const Args &a, cudaStream_t st) {
 int launch(const Args &a, int mode, int GC, cudaStream_t st) {
     if (mode == FWD) return GC == 64 ? launch_epw<FWD, 64>(a, st) : launch_epw<FWD, 32>(a, st);
     if (mode == FWD_LN) return launch_ks<FWD_LN, 32, 4>(a, st);
-    if (mode == DG_BITS) return GC == 64 ? launch_epw<DG_BITS, 64>(a, st) : launch_epw<DG_BITS, 32>(a, st);
-    return launch_ks<DG_ACT, 16, 8>(a, st);
+    return GC == 64 ? launch_epw<DG, 64>(a, st) : (GC == 32 ? launch_epw<DG, 32>(a, st) : launch_epw<DG, 16>(a, st));
 }
 
 // Channels per chunk of a C-channel source, or 0.
@@ -805,7 +782,7 @@ int halo_conv_fwd(const ConvGeom &g, const bf16 *X, const bf16 *W, const FwdEpil
 static bool plan_dgrad(Args &a, const ConvGeom &g, int ldy, int wt_ld, const DgradEpilogue &e) {
     if (g.k != 3 || g.pad != 1 || g.Hi < 2 || g.Wi < 2 || ldy != g.Co || !e.out || e.out_f32 || e.ksplit > 1) return false;
     if (g.Ci != 16 && g.Ci != 32 && g.Ci != 64) return false;
-    if (g.Ci == 16 ? !e.mask_act : !e.mask_bits) return false;
+    if (!e.mask_bits) return false;
     const int CB = chunk_of(g.Co);
     if (CB == 0 || wt_ld < g.Co || wt_ld % 8 != 0 || (size_t)9 * g.Ci * g.Co * 2 > 160 * 1024) return false;
     a.CB = CB;
@@ -816,7 +793,6 @@ static bool plan_dgrad(Args &a, const ConvGeom &g, int ldy, int wt_ld, const Dgr
     a.nloads = a.nchunks;
     a.w_box = (uint32_t)(g.Ci * a.rb);
     a.w_chunk = 9u * a.w_box;
-    a.wide_gate = g.Ci == 16;
     return a.nchunks <= kMaxSlots && plan(a, (g.Wi + 1) / 2, (g.Hi + 1) / 2, g.B);
 }
 
@@ -874,7 +850,6 @@ int halo_conv_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, 
     a.Hi = g.Hi;
     a.Wi = g.Wi;
     a.mask_bits = e.mask_bits;
-    a.mask = e.mask_act;
     a.status = status;
-    return launch(a, g.Ci == 16 ? DG_ACT : DG_BITS, g.Ci, st);
+    return launch(a, DG, g.Ci, st);
 }

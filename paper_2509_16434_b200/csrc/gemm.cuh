@@ -14,7 +14,7 @@ struct FwdEpilogue {
     float *out_mean;    // head: columns 0..A-1 -> [M][A]
     float *out_value;   // head: column A -> [M]
     int A;
-    uint32_t *out_bits = nullptr;  // optional: gate bits (out > 0) of a ReLU output, [M][Co / 32]; needs Co % 32 == 0
+    uint32_t *out_bits = nullptr;  // optional: gate bits (out > 0) of a ReLU output, [M][Co / 32], or [M] half words for Co = 16
     int ldo = 0;                   // row stride of `out` in elements (0: Co)
     // Layer normalisation over the Co channels of every output row, between the bias and the ReLU (all null: none):
     // xhat = (z - mean) / sqrt(var + 1e-5), out = act(gamma * xhat + beta); xhat [M][Co] bf16 and rstd [M] fp32 are
@@ -30,7 +30,8 @@ struct DgradEpilogue {
     const bf16 *mask_act;  // [M'][Ci]: output is zeroed where this is <= 0; may be nullptr
     bf16 *out;             // [M'][Ci] bf16, or nullptr
     float *out_f32;        // [M'][Ci] fp32, or nullptr
-    const uint32_t *mask_bits = nullptr;  // the same gate as one bit per element, [M'][Ci / 32] (channel c at bit gate_bit_of_channel(c) of word c / 32);
+    const uint32_t *mask_bits = nullptr;  // the same gate as one bit per element, [M'][Ci / 32] (channel c at bit gate_bit_of_channel(c) of word c / 32),
+                                          // or [M'] half words for Ci = 16 (gate_half);
                                           // used instead of mask_act by kernels that support it
     int ksplit = 1;  // flat GEMMs with out_f32 only: the reduction is cut into ksplit (<= 8) equal slabs and slab s leaves
                      // its partial product in out_f32 + s * M' * Ci; the reader adds the slabs in order
@@ -47,7 +48,7 @@ int tc_gemm_wgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *X, flo
 
 // TMA-fed versions of the same three operations (operand tiles moved by cp.async.bulk.tensor).  They cover
 // channel counts that are multiples of 16 (any multiple of 8 that is at least 64 for a fully connected layer; a merged
-// input gradient of 16-channel layers gates by activations, not by bits);
+// input gradient gates by bits where the input channels are a multiple of 32, else by activations);
 // for anything else they return PPO_ERR_UNSUPPORTED without launching and the caller uses the tc_ versions.
 int tma_gemm_fwd(const ConvGeom &g, const bf16 *X, const bf16 *W, const FwdEpilogue &e, int32_t *status,
                  cudaStream_t st);
@@ -82,7 +83,7 @@ int wgrad_batch(F gemms, cudaStream_t st) {
 int wgrad_reduce(const float *part, int jtiles, int ctiles, int splits, int BN, int Kfwd, int Co, float *dW, float *db,
                  int ones_row, cudaStream_t st);
 
-// bits[m][c / 32] bit (c % 32) = act[m][c] > 0, for C a multiple of 32.
+// bits[m][c / 32] bit gate_bit_of_channel(c) = act[m][c] > 0, for C a multiple of 32; half words (gate_half) for C = 16.
 int relu_bits(const bf16 *act, uint32_t *bits, long long M, int C, cudaStream_t st);
 
 // First convolution (C_in = 1) as a tensor-core GEMM over thread-built im2col tiles (conv1_tc.cu).

@@ -177,8 +177,8 @@ struct KArgs {
     bf16 *out;
     float *out_f32;
     const bf16 *mask;
-    const uint32_t *mask_bits;  // merged dgrad: the gate as bits, [pixels][nq_ci / 32]
-    uint32_t *out_bits;         // forward: gate bits of the ReLU output, [pixels][N / 32]
+    const uint32_t *mask_bits;  // input gradient: the gate as bits, [pixels][nq_ci / 32], of a flat GEMM [rows][N / 32]
+    uint32_t *out_bits;         // forward: gate bits of the ReLU output, [pixels][N / 32] (half words for N = 16)
     float *mean, *value;
     const float *ln_gamma, *ln_beta;  // forward with layer normalisation over the N columns of a row (null: none)
     bf16 *ln_xhat;
@@ -548,7 +548,10 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
                                 pk[j] = relu_pack_bf16x2(v[2 * j], v[2 * j + 1]);
                                 w = gate_bits_add(w, pk[j], j);
                             }
-                            if (a.out_bits && okr) a.out_bits[orow * (a.N >> 5) + (col >> 5)] = w;
+                            if (a.out_bits && okr) {
+                                if (a.N == 16) reinterpret_cast<uint16_t *>(a.out_bits)[orow] = gate_half(w);
+                                else a.out_bits[orow * (a.N >> 5) + (col >> 5)] = w;
+                            }
                         } else {
 #pragma unroll
                             for (int j = 0; j < 16; ++j) pk[j] = pack_bf16x2(v[2 * j], v[2 * j + 1]);
@@ -1178,7 +1181,7 @@ int tma_gemm_fwd(const ConvGeom &g, const bf16 *X, const bf16 *W, const FwdEpilo
     a.bias = e.bias;
     a.out = e.out;
     a.mean = e.out_mean;
-    a.out_bits = (e.out_bits && e.relu && g.Co % 32 == 0) ? e.out_bits : nullptr;
+    a.out_bits = (e.out_bits && e.relu && (g.Co % 32 == 0 || g.Co == 16)) ? e.out_bits : nullptr;
     if (e.out_bits && !a.out_bits) return PPO_ERR_UNSUPPORTED;
     a.value = e.out_value;
     a.status = status;
@@ -1214,9 +1217,11 @@ int tma_gemm_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, i
     if (!status || g.Ci % 8 != 0 || ldy % 8 != 0 || wt_ld % 8 != 0 || ldy < wt_ld) return PPO_ERR_UNSUPPORTED;
     const bool flat = is_flat(g);
     // a 32-column group of the staged epilogue must lie inside one parity class; with 16 input channels the
-    // per-thread epilogue (16 columns = one class at a time) takes over, which needs the bf16 gate
+    // per-thread epilogue (16 columns = one class at a time) takes over, which needs the bf16 gate.  A flat GEMM has one row of
+    // bits per row of outputs.
+    const uint32_t *const bits = g.Ci % 32 == 0 ? e.mask_bits : nullptr;
     if (!flat && (g.k < 3 || g.Hi < 2 || g.Wi < 2 || !Wc)) return PPO_ERR_UNSUPPORTED;
-    if (!flat && g.Ci % 32 != 0 && (g.Ci % 16 != 0 || !e.mask_act || e.mask_bits || !e.out)) return PPO_ERR_UNSUPPORTED;
+    if (!flat && g.Ci % 32 != 0 && (g.Ci % 16 != 0 || !e.mask_act || !e.out)) return PPO_ERR_UNSUPPORTED;
     // at most 16 columns in rows padded to 16 (the head): one box, one MMA of K = 16
     const bool head = flat && g.Co <= 16 && ldy == 16 && wt_ld <= 16;
     const int CB = head ? 16 : channels_per_box(g.Co, flat);
@@ -1227,7 +1232,8 @@ int tma_gemm_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, i
     a.kchunks = (g.Co + CB - 1) / CB;
     a.w_tap = wt_ld;
     const int Hr = flat ? 1 : (g.Hi + 1) / 2, Wr = flat ? g.B : (g.Wi + 1) / 2;
-    const int flat_n = flat ? flat_bn(g.Ci, g.B) : 0;
+    int flat_n = flat ? flat_bn(g.Ci, g.B) : 0;
+    if (flat && bits) flat_n = (flat_n + 31) / 32 * 32;  // a word of gates belongs to one tile
     if (!(flat && e.ksplit <= 1 ? make_flat_grid(a.grid, g.B, (g.Ci + flat_n - 1) / flat_n)
                                 : make_grid(a.grid, Wr, Hr, flat ? 1 : g.B, a.row_bytes)))
         return PPO_ERR_UNSUPPORTED;
@@ -1243,7 +1249,7 @@ int tma_gemm_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, i
     a.out = e.out;
     a.out_f32 = e.out_f32;
     a.mask = e.mask_act;
-    a.mask_bits = flat ? nullptr : e.mask_bits;
+    a.mask_bits = bits;
     a.status = status;
     const int ks = flat && e.ksplit > 1 ? e.ksplit : 1;
     if (ks > 1) {

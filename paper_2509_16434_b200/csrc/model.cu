@@ -176,7 +176,7 @@ static size_t carve(ppo_model *m, const ppo_model *shape, int mb, char *base) {
         size_t bytes = (size_t)mb * shape->Hs[l] * shape->Ws[l] * shape->Cs[l] * sizeof(bf16);
         char *a = take(bytes), *g = take(bytes);
         if (m) { m->act[l] = (bf16 *)a; m->dact[l] = (bf16 *)g; }
-        const bool bits = shape->Cs[l] % 32 == 0 && l < shape->L;  // gate bits for the dgrad of layer l + 1
+        const bool bits = shape->Cs[l] % 32 == 0 || shape->Cs[l] == 16;  // gate bits for the gradient that arrives from above
         char *bt = bits ? take(bytes / 16) : nullptr;
         if (m) m->abits[l] = (uint32_t *)bt;
         char *xh = shape->d.norm ? take(bytes) : nullptr;
@@ -310,7 +310,7 @@ extern "C" int ppo_model_activation_ptr(const ppo_model *m, int kind, int index,
         *elems = kind == 6 ? 2 * R * H : kind == 7 ? 4 * R * H : R * H;
         return PPO_OK;
     }
-    if (kind == 2 && index >= 1 && index < m->L && m->abits[index]) {
+    if (kind == 2 && index >= 1 && index < m->L && m->Cs[index] % 32 == 0) {
         *ptr = m->abits[index];
         *elems = (size_t)m->mbmax * m->Hs[index] * m->Ws[index] * m->Cs[index] / 32;
         return PPO_OK;
@@ -389,7 +389,7 @@ extern "C" int ppo_state_reset(float *h, float *c, const uint8_t *done, int laye
 extern "C" int ppo_model_sync_masks(ppo_model *m, int rows, void *stream) {
     if (!m || !m->ws) return PPO_ERR_STATE;
     if (rows <= 0 || rows > m->mbmax) return PPO_ERR_SHAPE;
-    for (int l = 1; l < m->L; ++l)
+    for (int l = 1; l <= m->L; ++l)
         if (m->abits[l]) {
             const int s = relu_bits(m->act[l], m->abits[l], (long long)rows * m->Hs[l] * m->Ws[l], m->Cs[l],
                                     static_cast<cudaStream_t>(stream));

@@ -1,7 +1,10 @@
 """Fully connected layers at the edges of their tiles (rows and columns that no tile width divides, reductions that are no whole
-number of chunks)."""
+number of chunks), and the gates of the last convolution."""
 import pytest
+import torch
 
+import test_gpu_learner as base
+from paper_2509_16434_b200 import binding as ppo
 from paper_2509_16434_b200 import synth
 from test_gpu_conv_edges import NETS, test_conv_stack_matches_oracle as conv_stack_matches_oracle
 
@@ -17,3 +20,35 @@ def test_forward_and_gradients_match_oracle(N, T, fc, P, last, embed, monkeypatc
     w = synth.Workload("flat", N, T, 16, 24, (16, last), (3, 3), fc, 1, 2, P=P, A=3, embed=embed)
     monkeypatch.setitem(NETS, "flat", w)
     conv_stack_matches_oracle("flat", monkeypatch)  # outputs and every gradient tensor within 2e-2
+
+
+@pytest.mark.parametrize("name", ["narrow_16_32", "three_groups", "many_chunks", "small_images", "one_block"])
+def test_last_gate_is_open_for_positive_activations_only(name):
+    """The gradient of the average pool sees the last activations through their gates alone: minus zero, negative numbers and NaN
+    close them as zero does, and every gradient keeps its bits."""
+    w = NETS[name]
+    B = w.M // w.minibatches
+    L, md, lay, theta, roll, action, logp, dev = base._setup(w, B)
+    h = L.hyper
+    L.compute_gae(dev["last_value"])
+    ppo.ppo_shuffle_gather_minibatch(L.buffer, 5, 0, 0, w.minibatches, L.mb)
+    ppo.ppo_encoder_fwd(L.model, L.mb, 0, B, L.mean, L.value)
+    L.loss.zero_()
+    ppo.ppo_loss_fwd_bwd(L.model, L.mb, 0, B, B, L.mean, L.value, h.clip, h.vf_coef, h.ent_coef, L.loss, L.dmean, L.dvalue)
+    act = L.model.activation(0, len(w.conv_c)).view(torch.int16)
+    saved = act.clone()
+    where = torch.rand(act.shape, device=act.device, generator=torch.Generator(act.device).manual_seed(1)) < 0.3
+
+    def gradients(pattern):
+        act.copy_(torch.where(where, torch.tensor(pattern - 0x10000 if pattern & 0x8000 else pattern, dtype=torch.int16,
+                                                  device=act.device), saved))
+        ppo.ppo_model_sync_masks(L.model, B)
+        ppo.ppo_model_zero_grad(L.model)
+        ppo.ppo_encoder_bwd(L.model, L.mb, 0, B, L.dmean, L.dvalue, True)
+        assert ppo.ppo_poll_status() == 0
+        return L.model.grad.clone()
+
+    want = gradients(0x0000)
+    assert torch.isfinite(want).all() and float(want.norm()) > 0
+    for pattern in (0x8000, 0xBF80, 0xFF80, 0x7FC0, 0xFFC0):  # -0, -1, -inf, NaN, -NaN
+        assert torch.equal(gradients(pattern), want), hex(pattern)
