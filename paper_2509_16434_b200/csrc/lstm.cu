@@ -21,10 +21,11 @@ namespace {
 
 using namespace tc;
 
-constexpr int kCellWarps = 8;
+constexpr int kCellWarps = 16;
 constexpr int kThreads = (2 + kCellWarps) * 32;  // warp 0: TMA producer, warp 1: MMA issue and TMEM owner
 constexpr int kMaxStages = 8;
 constexpr uint32_t kABytes = 128 * 128, kBBytes = 64 * 128;  // one 64-wide chunk of the reduction: 128 envs, 64 weight rows
+constexpr uint32_t kXBytes = 128 * 64 * 4;                   // the accumulator on its way to the cell's or the store's threads
 constexpr size_t kSmemMax = 227 * 1024;
 
 struct Args {
@@ -60,6 +61,7 @@ __device__ __forceinline__ bool cell_all(bool ok) {
         : "memory");
     return r != 0;
 }
+// Between the acquire that saw other threads' plain writes and the copy that reads them through the async proxy.
 __device__ __forceinline__ void fence_proxy_all() { asm volatile("fence.proxy.async;" ::: "memory"); }
 
 // Arrival at a tile's counter, by one thread behind a barrier of the threads whose writes it publishes.
@@ -82,39 +84,48 @@ __device__ bool tile_wait(const unsigned int *counter, unsigned int target, vola
     }
 }
 
-// Eight consecutive fp32 columns of this thread's TMEM lane.
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float *v) {
-    uint32_t r[8];
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(taddr)
-                 : "memory");
-#pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+__device__ __forceinline__ void to4(const float4 &v, float *o) { o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w; }
+__device__ __forceinline__ void load4(const float *p, float *v) { to4(*reinterpret_cast<const float4 *>(p), v); }
+__device__ __forceinline__ void load4_l2(const float *p, float *v) {  // written by other CTAs of this launch
+    to4(__ldcg(reinterpret_cast<const float4 *>(p)), v);
 }
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void store4(float *p, const float *v) { *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]); }
+__device__ __forceinline__ uint2 pack4(const float *v) { return make_uint2(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3])); }
 
-__device__ __forceinline__ void load8(const float *p, float *v) {
-    const float4 a = *reinterpret_cast<const float4 *>(p), b = *reinterpret_cast<const float4 *>(p + 4);
-    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+// The exchange tile [128 rows][64 floats], 16 pieces of 16 bytes a row.  Tensor memory hands a thread a row; global memory
+// wants neighbouring lanes on one row (a lane per row made every load and store of the cell 32 lines: 9000 cycles of a
+// backward step went into the load-store unit, and polls of the counters queued behind them; 256 envs x 1024 units, 16 steps:
+// forward 187 -> 154 us, backward 258 -> 184).  Piece p of row r sits at
+// p ^ f(r), f running through eight values over eight rows with its high bit first: a row per lane on the way in, four or
+// sixteen pieces of a row on neighbouring lanes on the way out, neither meets a bank twice.
+__device__ __forceinline__ uint32_t xch_addr(uint32_t base, int row, int piece) {
+    return base + (uint32_t)row * 256u + (((uint32_t)piece ^ (((uint32_t)row & 1u) << 2 | (((uint32_t)row >> 1) & 3u))) << 4);
 }
-__device__ __forceinline__ void load8_l2(const float *p, float *v) {  // written by other CTAs of this launch
-    const float4 a = __ldcg(reinterpret_cast<const float4 *>(p)), b = __ldcg(reinterpret_cast<const float4 *>(p + 4));
-    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+// This warp's 16 accumulator columns into the tile.
+__device__ __forceinline__ void xch_put(uint32_t base, uint32_t tmem, int lg, int lane, int grp) {
+    float v[16];
+    tmem_ld16(tmem + ((uint32_t)(lg * 32) << 16) + (uint32_t)(16 * grp), v);
+    tc_fence_before();
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(xch_addr(base, lg * 32 + lane, 4 * grp + j)), "f"(v[4 * j]),
+                     "f"(v[4 * j + 1]), "f"(v[4 * j + 2]), "f"(v[4 * j + 3])
+                     : "memory");
 }
-__device__ __forceinline__ void store8(float *p, const float *v) {
-    *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
-    *reinterpret_cast<float4 *>(p + 4) = make_float4(v[4], v[5], v[6], v[7]);
-}
-__device__ __forceinline__ uint4 pack8(const float *v) {
-    return make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]), pack_bf16x2(v[6], v[7]));
+__device__ __forceinline__ float4 xch_get(uint32_t base, int row, int piece) {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"(xch_addr(base, row, piece))
+                 : "memory");
+    return v;
 }
 
 // Everything the two kernels share around the cell: barriers, tensor memory, the resident weight slice, the stream of A
 // chunks and the MMAs.
 struct Frame {
     Pipe *pipe;
-    uint32_t smem_base, b_base, tmem;
+    uint32_t smem_base, b_base, x_base, tmem;
     int warp, lane, mt, q, chunks, S;
 };
 
@@ -125,7 +136,8 @@ __device__ __forceinline__ Frame frame_begin(const Args &a, uint8_t *raw) {
     f.S = a.stages;
     f.smem_base = smem_u32(smem);
     f.b_base = f.smem_base + (uint32_t)f.S * kABytes;
-    f.pipe = reinterpret_cast<Pipe *>(smem + (size_t)f.S * kABytes + (size_t)f.chunks * kBBytes);
+    f.x_base = f.b_base + (uint32_t)f.chunks * kBBytes;
+    f.pipe = reinterpret_cast<Pipe *>(smem + (size_t)f.S * kABytes + (size_t)f.chunks * kBBytes + kXBytes);
     f.warp = warp_index();
     f.lane = threadIdx.x & 31;
     f.mt = (int)blockIdx.x / a.per_tile;
@@ -226,6 +238,7 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_fwd_kernel(const __grid_cons
             for (int t = 0; t < a.T && ok; ++t) {
                 ok = tile_wait(counter, (unsigned)(a.per_tile * (t + 1)), abort_flag, a.status);
                 if (!ok) break;
+                fence_proxy_all();
                 ok = produce_step(a, f, 0, t * a.Be + row0, s, ph, it);
             }
             if (!ok) drain(f, it);
@@ -237,71 +250,65 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_fwd_kernel(const __grid_cons
         bool ok = mbar_wait_warp(&f.pipe->wfull, 0, abort_flag, a.status);
         for (int t = 0; t < a.T && ok; ++t) ok = mma_step(a, f, s, ph);
     } else {
-        const int lg = f.warp & 3, half = (f.warp - 2) >> 2, row = lg * 32 + f.lane, e = row0 + row;
-        const bool live = e < a.Be, issuer = threadIdx.x == 64;
-        const int j0 = u0 + 8 * half;
-        const uint32_t tm = f.tmem + ((uint32_t)(lg * 32) << 16) + (uint32_t)(8 * half);
-        float cp[8], bias[4][8];
+        // thread of the cell: env `row` of the tile, units j0 .. j0 + 3
+        const int lg = f.warp & 3, grp = (f.warp - 2) >> 2, ct = (int)threadIdx.x - 64, row = ct >> 2, quad = ct & 3, e = row0 + row;
+        const bool live = e < a.Be, issuer = ct == 0;
+        const int j0 = u0 + 4 * quad;
+        float cp[4] = {0.f, 0.f, 0.f, 0.f}, bias[4][4];
 #pragma unroll
-        for (int g = 0; g < 4; ++g) load8(a.bias + g * H + j0, bias[g]);
+        for (int g = 0; g < 4; ++g) load4(a.bias + g * H + j0, bias[g]);
         if (live) {  // the state the first step starts from
             const size_t i = (size_t)e * H + j0;
-            float hv[8];
-            load8(a.h_init + i, hv);
-            load8(a.c_init + i, cp);
-            *reinterpret_cast<uint4 *>(a.hprev + i) = pack8(hv);
-            store8(a.cprev + i, cp);
-        } else {
-#pragma unroll
-            for (int k = 0; k < 8; ++k) cp[k] = 0.f;
+            float hv[4];
+            load4(a.h_init + i, hv);
+            load4(a.c_init + i, cp);
+            *reinterpret_cast<uint2 *>(a.hprev + i) = pack4(hv);
+            store4(a.cprev + i, cp);
         }
-        fence_proxy_all();
         cell_sync();
         if (issuer) tile_arrive(counter);
         for (int t = 0; t < a.T; ++t) {
             const size_t r = (size_t)t * a.Be + e;
-            float xg[4][8];
+            float xg[4][4];
             bool reset = false;
             if (live) {  // ahead of the wait: they do not depend on this step's product
 #pragma unroll
-                for (int g = 0; g < 4; ++g) load8(a.xg + r * 4 * H + g * H + j0, xg[g]);
+                for (int g = 0; g < 4; ++g) load4(a.xg + r * 4 * H + g * H + j0, xg[g]);
                 reset = a.done[r] != 0;
             }
-            if (!cell_all(mbar_wait(&f.pipe->tfull, t & 1, abort_flag, a.status))) break;
+            const bool ok = mbar_wait(&f.pipe->tfull, t & 1, abort_flag, a.status);
             tc_fence_after();
-            float hg[4][8];
-#pragma unroll
-            for (int g = 0; g < 4; ++g) tmem_ld8(tm + 16u * g, hg[g]);
-            tmem_wait_ld();
-            tc_fence_before();
-            float gi[8], gf[8], gg[8], go[8], cv[8];
-            uint4 hb = make_uint4(0, 0, 0, 0);
+            if (__all_sync(0xffffffffu, ok)) xch_put(f.x_base, f.tmem, lg, f.lane, grp);  // gate `grp` of the 16 units
+            if (!cell_all(ok)) break;
+            float gi[4], gf[4], gg[4], go[4], cv[4];
+            uint2 hb = make_uint2(0u, 0u);
             if (live) {
-                float hv[8];
+                float hg[4][4], hv[4];
 #pragma unroll
-                for (int k = 0; k < 8; ++k) {
+                for (int g = 0; g < 4; ++g) to4(xch_get(f.x_base, row, 4 * g + quad), hg[g]);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
                     lstm_cell(xg[0][k] + hg[0][k] + bias[0][k], xg[1][k] + hg[1][k] + bias[1][k], xg[2][k] + hg[2][k] + bias[2][k],
                               xg[3][k] + hg[3][k] + bias[3][k], cp[k], gi[k], gf[k], gg[k], go[k], cv[k], hv[k]);
                 }
-                hb = pack8(hv);
-                if (t + 1 < a.T) *reinterpret_cast<uint4 *>(a.hprev + (r + a.Be) * H + j0) = reset ? make_uint4(0, 0, 0, 0) : hb;
+                hb = pack4(hv);
+                if (t + 1 < a.T) *reinterpret_cast<uint2 *>(a.hprev + (r + a.Be) * H + j0) = reset ? make_uint2(0u, 0u) : hb;
             }
             if (t + 1 < a.T) {  // what the others wait for goes first, the rest behind it
-                fence_proxy_all();
                 cell_sync();
                 if (issuer) tile_arrive(counter);
             }
             if (live) {
-                *reinterpret_cast<uint4 *>(a.h + r * H + j0) = hb;
+                *reinterpret_cast<uint2 *>(a.h + r * H + j0) = hb;
                 float *gp = a.gates + r * 4 * H + j0;
-                store8(gp, gi);
-                store8(gp + H, gf);
-                store8(gp + 2 * H, gg);
-                store8(gp + 3 * H, go);
-                store8(a.c + r * H + j0, cv);
+                store4(gp, gi);
+                store4(gp + H, gf);
+                store4(gp + 2 * H, gg);
+                store4(gp + 3 * H, go);
+                store4(a.c + r * H + j0, cv);
 #pragma unroll
-                for (int k = 0; k < 8; ++k) cp[k] = reset ? 0.f : cv[k];
-                if (t + 1 < a.T) store8(a.cprev + (r + a.Be) * H + j0, cp);
+                for (int k = 0; k < 4; ++k) cp[k] = reset ? 0.f : cv[k];
+                if (t + 1 < a.T) store4(a.cprev + (r + a.Be) * H + j0, cp);
             }
         }
     }
@@ -328,6 +335,7 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_bwd_kernel(const __grid_cons
             for (int t = a.T - 1, i = 0; t > 0 && ok; --t, ++i) {
                 ok = tile_wait(counter, (unsigned)(a.per_tile * (2 * i + 1)), abort_flag, a.status);
                 if (!ok) break;
+                fence_proxy_all();
                 ok = produce_step(a, f, slab * H, t * a.Be + row0, s, ph, it);
             }
             if (!ok) drain(f, it);
@@ -339,25 +347,23 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_bwd_kernel(const __grid_cons
         bool ok = mbar_wait_warp(&f.pipe->wfull, 0, abort_flag, a.status);
         for (int t = a.T - 1; t > 0 && ok; --t) ok = mma_step(a, f, s, ph);
     } else {
-        const int lg = f.warp & 3, half = (f.warp - 2) >> 2, row = lg * 32 + f.lane, e = row0 + row;
-        const bool live = e < a.Be, issuer = threadIdx.x == 64;
-        const int j0 = f.q * 16 + 8 * half;
-        const uint32_t tm = f.tmem + ((uint32_t)(lg * 32) << 16) + (uint32_t)(32 * half);
+        // as a cell: env `row` of the tile, units j0 .. j0 + 3
+        const int lg = f.warp & 3, grp = (f.warp - 2) >> 2, ct = (int)threadIdx.x - 64, row = ct >> 2, quad = ct & 3, e = row0 + row;
+        const bool live = e < a.Be, issuer = ct == 0;
+        const int j0 = f.q * 16 + 4 * quad;
         const size_t step = (size_t)a.Be * H;
-        float dcc[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) dcc[k] = 0.f;
+        float dcc[4] = {0.f, 0.f, 0.f, 0.f};
         for (int t = a.T - 1, i = 0; t >= 0; --t, ++i) {
             const size_t r = (size_t)t * a.Be + e;
             const bool last = t == a.T - 1;
-            float dtop[8], g4[4][8], cv[8], cp[8];
+            float dtop[4], g4[4][4], cv[4], cp[4];
             bool carry = false;
             if (live) {
-                load8(a.dtop + r * H + j0, dtop);
+                load4(a.dtop + r * H + j0, dtop);
 #pragma unroll
-                for (int g = 0; g < 4; ++g) load8(a.gates + r * 4 * H + g * H + j0, g4[g]);
-                load8(a.c + r * H + j0, cv);
-                load8(a.cprev + r * H + j0, cp);
+                for (int g = 0; g < 4; ++g) load4(a.gates + r * 4 * H + g * H + j0, g4[g]);
+                load4(a.c + r * H + j0, cv);
+                load4(a.cprev + r * H + j0, cp);
                 carry = !last && a.done[r] == 0;
             }
             if (!last) {  // the partial products of the step after this one
@@ -366,43 +372,40 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_bwd_kernel(const __grid_cons
                 if (!cell_all(ok)) break;
             }
             if (live) {
-                float dhn[8];
-#pragma unroll
-                for (int k = 0; k < 8; ++k) dhn[k] = 0.f;
+                float dhn[4] = {0.f, 0.f, 0.f, 0.f};
                 if (carry) {
-                    float p[4][8];
+                    float p[4][4];
 #pragma unroll
-                    for (int s = 0; s < 4; ++s) load8_l2(a.dhc + s * step + (size_t)e * H + j0, p[s]);
+                    for (int s = 0; s < 4; ++s) load4_l2(a.dhc + s * step + (size_t)e * H + j0, p[s]);
 #pragma unroll
                     for (int s = 0; s < 4; ++s)
 #pragma unroll
-                        for (int k = 0; k < 8; ++k) dhn[k] += p[s][k];
+                        for (int k = 0; k < 4; ++k) dhn[k] += p[s][k];
                 }
-                float di[8], df[8], dgg[8], dgo[8];
+                float di[4], df[4], dgg[4], dgo[4];
 #pragma unroll
-                for (int k = 0; k < 8; ++k)
+                for (int k = 0; k < 4; ++k)
                     lstm_cell_back(dtop[k] + dhn[k], carry ? dcc[k] : 0.f, g4[0][k], g4[1][k], g4[2][k], g4[3][k], cv[k], cp[k], di[k],
                                    df[k], dgg[k], dgo[k], dcc[k]);
                 bf16 *o = a.dg + r * 4 * H + j0;
-                *reinterpret_cast<uint4 *>(o) = pack8(di);
-                *reinterpret_cast<uint4 *>(o + H) = pack8(df);
-                *reinterpret_cast<uint4 *>(o + 2 * H) = pack8(dgg);
-                *reinterpret_cast<uint4 *>(o + 3 * H) = pack8(dgo);
+                *reinterpret_cast<uint2 *>(o) = pack4(di);
+                *reinterpret_cast<uint2 *>(o + H) = pack4(df);
+                *reinterpret_cast<uint2 *>(o + 2 * H) = pack4(dgg);
+                *reinterpret_cast<uint2 *>(o + 3 * H) = pack4(dgo);
             }
             if (t == 0) break;
-            fence_proxy_all();
             cell_sync();
             if (issuer) tile_arrive(counter);
-            // this CTA's partial product
-            if (!cell_all(mbar_wait(&f.pipe->tfull, i & 1, abort_flag, a.status))) break;
+            // this CTA's partial product, 64 columns a row
+            const bool ok = mbar_wait(&f.pipe->tfull, i & 1, abort_flag, a.status);
             tc_fence_after();
-            float v[32];
-            tmem_ld32(tm, v);
-            tc_fence_before();
-            if (live) {
-                float *o = a.dhc + slab * step + (size_t)e * H + n0 + 32 * half;
+            if (__all_sync(0xffffffffu, ok)) xch_put(f.x_base, f.tmem, lg, f.lane, grp);
+            if (!cell_all(ok)) break;
 #pragma unroll
-                for (int k = 0; k < 8; ++k) __stcg(reinterpret_cast<float4 *>(o) + k, make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]));
+            for (int k = 0; k < 4; ++k) {
+                const int rr = k * 32 + (ct >> 4), piece = ct & 15;
+                if (row0 + rr < a.Be)
+                    __stcg(reinterpret_cast<float4 *>(a.dhc + slab * step + (size_t)(row0 + rr) * H + n0) + piece, xch_get(f.x_base, rr, piece));
             }
             cell_sync();
             if (issuer) tile_arrive(counter);
@@ -411,16 +414,16 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_bwd_kernel(const __grid_cons
     frame_end(a, f);
 }
 
-// Shape part; false where the layer or the sequence does not fit: a slice of W_h has to leave room for four chunks of A, and
-// all CTAs have to be resident at once.
+// Shape part; false where the layer or the sequence does not fit: a slice of W_h has to leave room for the exchange and two
+// chunks of A (four at H = 1024), and all CTAs have to be resident at once.
 bool plan(Args &a, int T, int Be, int H, int &ctas, size_t &smem) {
     if (H % 64 != 0 || T < 1 || Be < 1) return false;
     a.T = T; a.Be = Be; a.H = H;
     a.per_tile = H / 16;
     const long long n = (long long)((Be + 127) / 128) * a.per_tile;
     if (n > ppo_num_sms() || (Be + 127) / 128 + 1 > kLstmCounters) return false;
-    const size_t fixed = (size_t)(H / 64) * kBBytes + sizeof(Pipe) + 1024;
-    if (fixed + 4 * kABytes > kSmemMax) return false;
+    const size_t fixed = (size_t)(H / 64) * kBBytes + kXBytes + sizeof(Pipe) + 1024;
+    if (fixed + 2 * kABytes > kSmemMax) return false;
     a.stages = (int)((kSmemMax - fixed) / kABytes);
     if (a.stages > kMaxStages) a.stages = kMaxStages;
     smem = fixed + (size_t)a.stages * kABytes;
