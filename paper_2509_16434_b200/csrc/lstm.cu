@@ -3,9 +3,11 @@
 // A step's product with W_h is small (Be x 4H x H) and every step waits for the one before it: launch by launch the loop is
 // a chain of 13 us GEMMs and 5 us cell kernels that mostly wait, for W_h from L2, for the pipeline to fill, for the
 // launch.  Here a CTA keeps its slice of W_h in shared memory for all steps, the cell runs on the accumulator (forward) or
-// between two exchanges (backward) with c and its gradient in registers, and the CTAs of a tile of 128 envs meet at a
-// counter in global memory once (forward) or twice (backward) per step.  What a step then costs is the 256 KB of h (or of
-// one gate's gradients) a CTA pulls through L2 (2 us), the cell's memory traffic and the exchanges.
+// between two exchanges (backward) with c and its gradient in registers, and the CTAs of a tile of 128 envs exchange their
+// parts through global memory once (forward) or twice (backward) per step, with counters for each group of four of them.  What a
+// step costs (cycles of 16000, forward, 256 envs x 1024 units): 7300 for the 256 KB of h (or of one gate's gradients) a CTA
+// pulls through L2 and their MMAs (all CTAs together take 11 TB/s), 700 + 2500 for the accumulator's way to the cell and the
+// cell, 1250 until the release has seen its stores done, 2000 until the readers have seen it.
 // The arithmetic is that of the step-by-step path, sum by sum: same bits.
 //
 // All CTAs of a launch have to be resident at once (cooperative launch, one CTA per SM); every wait is bounded: on a
@@ -38,7 +40,7 @@ struct Args {
     float *gates, *c, *cprev;
     bf16 *h, *hprev, *dg;
     float *dhc;
-    unsigned int *counters;  // one per tile, 32 words apart; the last one counts the CTAs that have left
+    unsigned int *counters;  // two rows of 32 per tile (see below); the first word behind them counts the CTAs that have left
     int32_t *status;
 };
 
@@ -61,20 +63,29 @@ __device__ __forceinline__ bool cell_all(bool ok) {
         : "memory");
     return r != 0;
 }
-// Between the acquire that saw other threads' plain writes and the copy that reads them through the async proxy.
-__device__ __forceinline__ void fence_proxy_all() { asm volatile("fence.proxy.async;" ::: "memory"); }
+// Between the acquire that saw other threads' plain writes to global memory and the copy that reads them through the async
+// proxy (20 cycles; the fence over all state spaces takes 900).
+__device__ __forceinline__ void fence_proxy_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 
-// Arrival at a tile's counter, by one thread behind a barrier of the threads whose writes it publishes.
+// Counters of a tile of envs, a row of 32 for each exchange.  Word k of the first: CTAs that have published their 16 units of
+// chunk k of the reduction (64 units, four CTAs a step); of the second (backward): slabs that have published their partial
+// products of units 64 k .. 64 k + 63.  A reader waits for the four writers of what it reads next instead of for all the tile's
+// CTAs, whose slowest is some 2000 of a step's 16000 cycles behind (256 envs x 1024 units), and one row is one line to poll.
+__device__ __forceinline__ unsigned int *chunk_counters(const Args &a, int mt) { return a.counters + mt * 64; }
+__device__ __forceinline__ unsigned int *part_counters(const Args &a, int mt) { return a.counters + mt * 64 + 32; }
+// Arrival at a counter, by one thread behind a barrier of the threads whose writes it publishes.
 __device__ __forceinline__ void tile_arrive(unsigned int *counter) {
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(counter) : "memory");
 }
-// Bounded wait until a tile's counter has reached `target`.
+__device__ __forceinline__ unsigned int load_acquire(const unsigned int *p) {
+    unsigned int v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+// Bounded wait until a counter has reached `target`.
 __device__ bool tile_wait(const unsigned int *counter, unsigned int target, volatile int *abort_flag, int32_t *status) {
     const long long t0 = clock64();
-    while (true) {
-        unsigned int v;
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(counter) : "memory");
-        if (v >= target) return true;
+    while (load_acquire(counter) < target) {
         if (*abort_flag) return false;
         if (clock64() - t0 > kWaitCycles) {
             *abort_flag = 1;
@@ -82,6 +93,7 @@ __device__ bool tile_wait(const unsigned int *counter, unsigned int target, vola
             return false;
         }
     }
+    return true;
 }
 
 __device__ __forceinline__ void to4(const float4 &v, float *o) { o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w; }
@@ -167,22 +179,51 @@ __device__ __forceinline__ void frame_end(const Args &a, const Frame &f) {
         tc_fence_after();
         tmem_dealloc(f.tmem, 64);
     }
-    if (threadIdx.x == 0) {  // the last CTA to leave clears the counters for the next launch
-        const int tiles = (int)gridDim.x / a.per_tile;
+    // the last CTA to leave clears the counters for the next launch
+    const int words = (int)gridDim.x / a.per_tile * 64;
+    if (threadIdx.x == 0) {
         __threadfence();
-        if (atomicAdd(a.counters + tiles * 32, 1u) == gridDim.x - 1) {
-            for (int i = 0; i <= tiles; ++i) a.counters[i * 32] = 0u;
-            __threadfence();
-        }
+        f.pipe->tmem_slot = atomicAdd(a.counters + words, 1u) == gridDim.x - 1 ? 1u : 0u;
     }
+    __syncthreads();
+    if (f.pipe->tmem_slot)
+        for (int i = threadIdx.x; i <= words; i += kThreads) a.counters[i] = 0u;
 }
 
-// Producer: the A chunks of one step (columns col0 .. col0 + H of rows row0 .. row0 + 127).
-__device__ __forceinline__ bool produce_step(const Args &a, const Frame &f, int col0, int row0, int &s, uint32_t &ph, int &it) {
+// Producer warp: the A chunks of one step (columns col0 .. col0 + H of rows row0 .. row0 + 127), each as soon as its four CTAs
+// have published it `target / 4` times.  Lane k watches chunk k; the copies go out in order.
+__device__ __forceinline__ bool produce_step(const Args &a, const Frame &f, unsigned int target, int col0, int row0, int &s, uint32_t &ph,
+                                             int &it) {
+    volatile int *abort_flag = &f.pipe->abort_flag;
+    const unsigned int *mine = chunk_counters(a, f.mt) + f.lane;
+    bool seen = f.lane >= f.chunks;
+    uint32_t ready = 0;
+    const long long t0 = clock64();
     for (int k = 0; k < f.chunks; ++k, ++it) {
-        if (!mbar_wait(&f.pipe->empty[s], ph ^ 1u, &f.pipe->abort_flag, a.status)) return false;
-        mbar_arrive_expect_tx(&f.pipe->full[s], kABytes);
-        tma_load_2d(f.smem_base + (uint32_t)s * kABytes, &a.mapA, &f.pipe->full[s], col0 + k * 64, row0);
+        while (!((ready >> k) & 1u)) {
+            if (!seen) seen = load_acquire(mine) >= target;
+            ready = __ballot_sync(0xffffffffu, seen);
+            if ((ready >> k) & 1u) {
+                fence_proxy_global();
+                break;
+            }
+            bool stop = false;
+            if (f.lane == 0) {
+                stop = *abort_flag != 0;
+                if (!stop && clock64() - t0 > kWaitCycles) {
+                    *abort_flag = 1;
+                    ppo_report(a.status, PPO_ERR_TIMEOUT);
+                    stop = true;
+                }
+            }
+            if (__any_sync(0xffffffffu, stop)) return false;
+        }
+        if (!mbar_wait_warp(&f.pipe->empty[s], ph ^ 1u, abort_flag, a.status)) return false;
+        if (elect_one()) {
+            mbar_arrive_expect_tx(&f.pipe->full[s], kABytes);
+            tma_load_2d(f.smem_base + (uint32_t)s * kABytes, &a.mapA, &f.pipe->full[s], col0 + k * 64, row0);
+        }
+        __syncwarp();
         if (++s == f.S) { s = 0; ph ^= 1u; }
     }
     return true;
@@ -223,7 +264,7 @@ __device__ __forceinline__ bool mma_step(const Args &a, const Frame &f, int &s, 
 __global__ void __launch_bounds__(kThreads, 1) lstm_fwd_kernel(const __grid_constant__ Args a) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const Frame f = frame_begin(a, smem_raw);
-    unsigned int *counter = a.counters + f.mt * 32;
+    unsigned int *counter = chunk_counters(a, f.mt) + (f.q >> 2);  // of this CTA's units
     const int H = a.H, u0 = f.q * 16, row0 = f.mt * 128;
     volatile int *abort_flag = &f.pipe->abort_flag;
     if (f.warp == 0) {
@@ -232,17 +273,13 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_fwd_kernel(const __grid_cons
             for (int k = 0; k < f.chunks; ++k)
                 for (int g = 0; g < 4; ++g)
                     tma_load_2d(f.b_base + (uint32_t)k * kBBytes + (uint32_t)g * 2048u, &a.mapB, &f.pipe->wfull, k * 64, g * H + u0);
-            int s = 0, it = 0;
-            uint32_t ph = 0;
-            bool ok = true;
-            for (int t = 0; t < a.T && ok; ++t) {
-                ok = tile_wait(counter, (unsigned)(a.per_tile * (t + 1)), abort_flag, a.status);
-                if (!ok) break;
-                fence_proxy_all();
-                ok = produce_step(a, f, 0, t * a.Be + row0, s, ph, it);
-            }
-            if (!ok) drain(f, it);
         }
+        __syncwarp();
+        int s = 0, it = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        for (int t = 0; t < a.T && ok; ++t) ok = produce_step(a, f, 4u * (unsigned)(t + 1), 0, t * a.Be + row0, s, ph, it);
+        if (!ok && f.lane == 0) drain(f, it);
         __syncwarp();
     } else if (f.warp == 1) {
         int s = 0;
@@ -321,25 +358,22 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_fwd_kernel(const __grid_cons
 __global__ void __launch_bounds__(kThreads, 1) lstm_bwd_kernel(const __grid_constant__ Args a) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const Frame f = frame_begin(a, smem_raw);
-    unsigned int *counter = a.counters + f.mt * 32;
-    const int H = a.H, row0 = f.mt * 128, slices = H >> 6, slab = f.q / slices, n0 = (f.q - slab * slices) * 64;
+    const int H = a.H, row0 = f.mt * 128, slices = H >> 6, slab = f.q / slices, slice = f.q - slab * slices, n0 = slice * 64;
+    unsigned int *const cells = chunk_counters(a, f.mt) + (f.q >> 2);  // of this CTA's units as a cell
+    unsigned int *const parts_in = part_counters(a, f.mt) + (f.q >> 2), *const parts_out = part_counters(a, f.mt) + slice;
     volatile int *abort_flag = &f.pipe->abort_flag;
     if (f.warp == 0) {
         if (f.lane == 0) {
             mbar_arrive_expect_tx(&f.pipe->wfull, (uint32_t)f.chunks * kBBytes);
             for (int k = 0; k < f.chunks; ++k)
                 tma_load_2d(f.b_base + (uint32_t)k * kBBytes, &a.mapB, &f.pipe->wfull, slab * H + k * 64, n0);
-            int s = 0, it = 0;
-            uint32_t ph = 0;
-            bool ok = true;
-            for (int t = a.T - 1, i = 0; t > 0 && ok; --t, ++i) {
-                ok = tile_wait(counter, (unsigned)(a.per_tile * (2 * i + 1)), abort_flag, a.status);
-                if (!ok) break;
-                fence_proxy_all();
-                ok = produce_step(a, f, slab * H, t * a.Be + row0, s, ph, it);
-            }
-            if (!ok) drain(f, it);
         }
+        __syncwarp();
+        int s = 0, it = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        for (int t = a.T - 1, i = 0; t > 0 && ok; --t, ++i) ok = produce_step(a, f, 4u * (unsigned)(i + 1), slab * H, t * a.Be + row0, s, ph, it);
+        if (!ok && f.lane == 0) drain(f, it);
         __syncwarp();
     } else if (f.warp == 1) {
         int s = 0;
@@ -366,9 +400,10 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_bwd_kernel(const __grid_cons
                 load4(a.cprev + r * H + j0, cp);
                 carry = !last && a.done[r] == 0;
             }
-            if (!last) {  // the partial products of the step after this one
+            if (!last) {  // the partial products of the step after this one (their four writers had seen all cells of that step, so
+                          // the places of the step before were free)
                 bool ok = true;
-                if (issuer) ok = tile_wait(counter, (unsigned)(a.per_tile * 2 * i), abort_flag, a.status);
+                if (issuer) ok = tile_wait(parts_in, 4u * (unsigned)i, abort_flag, a.status);
                 if (!cell_all(ok)) break;
             }
             if (live) {
@@ -395,7 +430,7 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_bwd_kernel(const __grid_cons
             }
             if (t == 0) break;
             cell_sync();
-            if (issuer) tile_arrive(counter);
+            if (issuer) tile_arrive(cells);
             // this CTA's partial product, 64 columns a row
             const bool ok = mbar_wait(&f.pipe->tfull, i & 1, abort_flag, a.status);
             tc_fence_after();
@@ -408,7 +443,7 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_bwd_kernel(const __grid_cons
                     __stcg(reinterpret_cast<float4 *>(a.dhc + slab * step + (size_t)(row0 + rr) * H + n0) + piece, xch_get(f.x_base, rr, piece));
             }
             cell_sync();
-            if (issuer) tile_arrive(counter);
+            if (issuer) tile_arrive(parts_out);
         }
     }
     frame_end(a, f);
@@ -421,7 +456,7 @@ bool plan(Args &a, int T, int Be, int H, int &ctas, size_t &smem) {
     a.T = T; a.Be = Be; a.H = H;
     a.per_tile = H / 16;
     const long long n = (long long)((Be + 127) / 128) * a.per_tile;
-    if (n > ppo_num_sms() || (Be + 127) / 128 + 1 > kLstmCounters) return false;
+    if (n > ppo_num_sms() || a.H > 2048 || 2 * ((Be + 127) / 128) + 1 > kLstmCounters) return false;
     const size_t fixed = (size_t)(H / 64) * kBBytes + kXBytes + sizeof(Pipe) + 1024;
     if (fixed + 2 * kABytes > kSmemMax) return false;
     a.stages = (int)((kSmemMax - fixed) / kABytes);

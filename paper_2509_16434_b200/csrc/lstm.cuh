@@ -2,7 +2,7 @@
 #pragma once
 #include "common.cuh"
 
-constexpr int kLstmCounters = 256;  // words, 128 bytes apart, of the persistent kernels' counters
+constexpr int kLstmCounters = 256;  // rows of 32 words: counters of the persistent kernels
 
 // One layer's sequence: T steps of Be envs, H units; arrays of T * Be rows (see ppo_model).
 struct LstmSteps {
