@@ -45,7 +45,7 @@ struct Args {
 };
 
 struct Pipe {
-    uint64_t full[kMaxStages], empty[kMaxStages], tfull, wfull;
+    uint64_t full[kMaxStages], empty[kMaxStages], tfull, wfull, parts;  // parts: the cluster's partial products
     uint32_t tmem_slot;
     int abort_flag;
 };
@@ -124,12 +124,51 @@ __device__ __forceinline__ void xch_put(uint32_t base, uint32_t tmem, int lg, in
                      "f"(v[4 * j + 1]), "f"(v[4 * j + 2]), "f"(v[4 * j + 3])
                      : "memory");
 }
-__device__ __forceinline__ float4 xch_get(uint32_t base, int row, int piece) {
-    float4 v;
-    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-                 : "r"(xch_addr(base, row, piece))
+// Shared memory of CTA `rank` of the cluster at the place of this CTA's `addr`.
+__device__ __forceinline__ uint32_t in_cta(uint32_t addr, uint32_t rank) {
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+// Place of 16 bytes (piece 0 .. 3) of row `row` in slab `slab` of the partial products a CTA receives, [4][4 pieces][128 rows]:
+// a warp that sends a piece of 32 rows fills 512 bytes on end, and four pieces of a row on neighbouring lanes do not meet a
+// bank twice on the way out.
+__device__ __forceinline__ uint32_t part_addr(uint32_t base, int slab, int row, int piece) {
+    return base + (uint32_t)slab * 8192u + (uint32_t)piece * 2048u + (((uint32_t)row ^ ((uint32_t)piece << 1)) << 4);
+}
+// 16 bytes into another CTA's shared memory; its barrier counts them.
+__device__ __forceinline__ void send16(uint32_t dst, uint32_t bar, const float *v) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(dst), "f"(v[0]),
+                 "f"(v[1]), "f"(v[2]), "f"(v[3]), "r"(bar)
                  : "memory");
+}
+// Bounded wait for a phase that writes of the whole cluster complete.
+__device__ __forceinline__ bool cluster_mbar_wait(uint64_t *bar, uint32_t parity, volatile int *abort_flag, int32_t *status) {
+    const long long t0 = clock64();
+    while (true) {
+        uint32_t done;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(done)
+            : "r"(smem_u32(bar)), "r"(parity)
+            : "memory");
+        if (done) return true;
+        if (*abort_flag) return false;
+        if (clock64() - t0 > kWaitCycles) {
+            *abort_flag = 1;
+            ppo_report(status, PPO_ERR_TIMEOUT);
+            return false;
+        }
+    }
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ float4 lds16(uint32_t addr) {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
     return v;
 }
 
@@ -161,6 +200,7 @@ __device__ __forceinline__ Frame frame_begin(const Args &a, uint8_t *raw) {
         }
         mbar_init(&f.pipe->tfull, 1);
         mbar_init(&f.pipe->wfull, 1);
+        mbar_init(&f.pipe->parts, 1);
         f.pipe->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -322,7 +362,7 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_fwd_kernel(const __grid_cons
             if (live) {
                 float hg[4][4], hv[4];
 #pragma unroll
-                for (int g = 0; g < 4; ++g) to4(xch_get(f.x_base, row, 4 * g + quad), hg[g]);
+                for (int g = 0; g < 4; ++g) to4(lds16(xch_addr(f.x_base, row, 4 * g + quad)), hg[g]);
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     lstm_cell(xg[0][k] + hg[0][k] + bias[0][k], xg[1][k] + hg[1][k] + bias[1][k], xg[2][k] + hg[2][k] + bias[2][k],
@@ -353,14 +393,19 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_fwd_kernel(const __grid_cons
 }
 
 // Back-propagation through all steps of one layer: gate gradients dg of every step.  The product dg W_h of a step reduces
-// over 4 H columns in four slabs (one gate each) whose partial products are added in order: CTA q = (slab, 64 units) forms
-// one, all of them leave their partial products in global memory, and as a cell CTA q works on units 16 q .. 16 q + 15.
-__global__ void __launch_bounds__(kThreads, 1) lstm_bwd_kernel(const __grid_constant__ Args a) {
-    extern __shared__ __align__(1024) uint8_t smem_raw[];
+// over 4 H columns in four slabs (one gate each) whose partial products are added in order: CTA q = (64 units, slab) forms
+// one, and as a cell it works on units 16 q .. 16 q + 15, a quarter of the same 64.
+// CLUSTER: the four slabs of a slice are a cluster and send one another their partial products from the accumulator
+// straight into shared memory, data and signal in one; the way through global memory (store, release, poll, load) takes 9000
+// of a step's 20000 cycles, and so does shared memory that the others read behind a release (a release waits for all its
+// thread's block has under way).  A place is free again when the next product arrives: that needs gate gradients of all the
+// tile's cells, who had read it by then.
+template <bool CLUSTER>
+__device__ __forceinline__ void bwd_steps(const Args &a, uint8_t *smem_raw) {
     const Frame f = frame_begin(a, smem_raw);
-    const int H = a.H, row0 = f.mt * 128, slices = H >> 6, slab = f.q / slices, slice = f.q - slab * slices, n0 = slice * 64;
-    unsigned int *const cells = chunk_counters(a, f.mt) + (f.q >> 2);  // of this CTA's units as a cell
-    unsigned int *const parts_in = part_counters(a, f.mt) + (f.q >> 2), *const parts_out = part_counters(a, f.mt) + slice;
+    const int H = a.H, row0 = f.mt * 128, slab = f.q & 3, slice = f.q >> 2, n0 = slice * 64;
+    unsigned int *const cells = chunk_counters(a, f.mt) + slice;  // of this CTA's units as a cell
+    unsigned int *const parts = part_counters(a, f.mt) + slice;
     volatile int *abort_flag = &f.pipe->abort_flag;
     if (f.warp == 0) {
         if (f.lane == 0) {
@@ -387,23 +432,29 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_bwd_kernel(const __grid_cons
         const int j0 = f.q * 16 + 4 * quad;
         const size_t step = (size_t)a.Be * H;
         float dcc[4] = {0.f, 0.f, 0.f, 0.f};
+        float dtop[4], g4[4][4], cv[4], cp[4];
+        uint8_t done = 0;
+        // What the forward pass left for step t.  It comes from HBM in a burst of 57 KB per CTA (7 MB in all: 3500 cycles), so it is
+        // asked for while the step before multiplies.
+        auto fetch = [&](int t) {
+            if (!live) return;
+            const size_t r = (size_t)t * a.Be + e;
+            load4(a.dtop + r * H + j0, dtop);
+#pragma unroll
+            for (int g = 0; g < 4; ++g) load4(a.gates + r * 4 * H + g * H + j0, g4[g]);
+            load4(a.c + r * H + j0, cv);
+            load4(a.cprev + r * H + j0, cp);
+            done = a.done[r];
+        };
+        fetch(a.T - 1);
         for (int t = a.T - 1, i = 0; t >= 0; --t, ++i) {
             const size_t r = (size_t)t * a.Be + e;
-            const bool last = t == a.T - 1;
-            float dtop[4], g4[4][4], cv[4], cp[4];
-            bool carry = false;
-            if (live) {
-                load4(a.dtop + r * H + j0, dtop);
-#pragma unroll
-                for (int g = 0; g < 4; ++g) load4(a.gates + r * 4 * H + g * H + j0, g4[g]);
-                load4(a.c + r * H + j0, cv);
-                load4(a.cprev + r * H + j0, cp);
-                carry = !last && a.done[r] == 0;
-            }
+            const bool last = t == a.T - 1, carry = !last && done == 0;
             if (!last) {  // the partial products of the step after this one (their four writers had seen all cells of that step, so
                           // the places of the step before were free)
                 bool ok = true;
-                if (issuer) ok = tile_wait(parts_in, 4u * (unsigned)i, abort_flag, a.status);
+                if (CLUSTER) ok = cluster_mbar_wait(&f.pipe->parts, (uint32_t)(i - 1) & 1u, abort_flag, a.status);
+                else if (issuer) ok = tile_wait(parts, 4u * (unsigned)i, abort_flag, a.status);
                 if (!cell_all(ok)) break;
             }
             if (live) {
@@ -411,7 +462,10 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_bwd_kernel(const __grid_cons
                 if (carry) {
                     float p[4][4];
 #pragma unroll
-                    for (int s = 0; s < 4; ++s) load4_l2(a.dhc + s * step + (size_t)e * H + j0, p[s]);
+                    for (int s = 0; s < 4; ++s) {
+                        if (CLUSTER) to4(lds16(part_addr(f.x_base, s, row, quad)), p[s]);
+                        else load4_l2(a.dhc + s * step + (size_t)e * H + j0, p[s]);
+                    }
 #pragma unroll
                     for (int s = 0; s < 4; ++s)
 #pragma unroll
@@ -430,23 +484,57 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_bwd_kernel(const __grid_cons
             }
             if (t == 0) break;
             cell_sync();
-            if (issuer) tile_arrive(cells);
-            // this CTA's partial product, 64 columns a row
+            if (issuer) {
+                if (CLUSTER) mbar_arrive_expect_tx(&f.pipe->parts, kXBytes);  // what the four CTAs will send for this step
+                tile_arrive(cells);
+            }
+            fetch(t - 1);
+            // this CTA's partial product, 64 columns a row: columns 16 k .. 16 k + 15 are what cell k of the slice needs
             const bool ok = mbar_wait(&f.pipe->tfull, i & 1, abort_flag, a.status);
             tc_fence_after();
+            if (CLUSTER) {
+                if (__all_sync(0xffffffffu, ok)) {  // (else the abort flag ends all warps at the next wait for the parts)
+                    float v[16];
+                    tmem_ld16(f.tmem + ((uint32_t)(lg * 32) << 16) + (uint32_t)(16 * grp), v);
+                    tc_fence_before();
+                    const uint32_t bar = in_cta(smem_u32(&f.pipe->parts), (uint32_t)grp);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        send16(in_cta(part_addr(f.x_base, slab, lg * 32 + f.lane, k), (uint32_t)grp), bar, v + 4 * k);
+                }
+                continue;
+            }
             if (__all_sync(0xffffffffu, ok)) xch_put(f.x_base, f.tmem, lg, f.lane, grp);
             if (!cell_all(ok)) break;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const int rr = k * 32 + (ct >> 4), piece = ct & 15;
                 if (row0 + rr < a.Be)
-                    __stcg(reinterpret_cast<float4 *>(a.dhc + slab * step + (size_t)(row0 + rr) * H + n0) + piece, xch_get(f.x_base, rr, piece));
+                    __stcg(reinterpret_cast<float4 *>(a.dhc + slab * step + (size_t)(row0 + rr) * H + n0) + piece, lds16(xch_addr(f.x_base, rr, piece)));
             }
             cell_sync();
-            if (issuer) tile_arrive(parts_out);
+            if (issuer) tile_arrive(parts);
         }
     }
+    if (CLUSTER) {  // no CTA leaves while another may write to its shared memory
+        if (*abort_flag) {  // (sends of a step that was given up land meanwhile; a finished step has waited for its own)
+            const long long t0 = clock64();
+            while (clock64() - t0 < 100000) {
+            }
+        }
+        __syncwarp();
+        cluster_sync();
+    }
     frame_end(a, f);
+}
+
+__global__ void __launch_bounds__(kThreads, 1) lstm_bwd_kernel(const __grid_constant__ Args a) {
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    bwd_steps<false>(a, smem_raw);
+}
+__global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(kThreads, 1) lstm_bwd_cluster_kernel(const __grid_constant__ Args a) {
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    bwd_steps<true>(a, smem_raw);
 }
 
 // Shape part; false where the layer or the sequence does not fit: a slice of W_h has to leave room for the exchange and two
@@ -515,7 +603,22 @@ int lstm_bwd_steps(const LstmSteps &p, const bf16 *WhT, const float *dtop, bf16 
     a.gates = p.gates; a.c = p.c; a.cprev = p.cprev;
     a.counters = p.counters;
     a.status = status;
-    static bool set[64] = {false};
+    static bool set[64] = {false}, set_cluster[64] = {false};
+    PPO_TRY(prepare_kernel(reinterpret_cast<const void *>(lstm_bwd_cluster_kernel), set_cluster));
+    // clusters of four fit the groups of SMs less tightly than single CTAs (33 of them on 148 SMs)
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = 4;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    PPO_CUDA_CHECK(cudaOccupancyMaxActiveClusters(&clusters, lstm_bwd_cluster_kernel, &cfg));
+    if (4 * clusters >= ctas) return ppo_launch_together(lstm_bwd_cluster_kernel, dim3(ctas), dim3(kThreads), smem, st, a);
     PPO_TRY(prepare_kernel(reinterpret_cast<const void *>(lstm_bwd_kernel), set));
     return ppo_launch_together(lstm_bwd_kernel, dim3(ctas), dim3(kThreads), smem, st, a);
 }
