@@ -25,15 +25,22 @@ using namespace tc;
 
 constexpr int kCellWarps = 16;
 constexpr int kThreads = (2 + kCellWarps) * 32;  // warp 0: TMA producer, warp 1: MMA issue and TMEM owner
-constexpr int kMaxStages = 8;
-constexpr uint32_t kABytes = 128 * 128, kBBytes = 64 * 128;  // one 64-wide chunk of the reduction: 128 envs, 64 weight rows
-constexpr uint32_t kXBytes = 128 * 64 * 4;                   // the accumulator on its way to the cell's or the store's threads
+constexpr int kMaxStages = 16;
+constexpr uint32_t kBBytes = 64 * 128;  // weights of one 64-wide chunk of the reduction: 64 rows
+
+// A tile is 32 U envs, U = 1, 2 or 4: a cell thread works on U units of one env, and 512 of them on 16 units of the tile.  Fewer
+// envs per tile means more CTAs, each with less to pull, to compute and to write; the MMA takes 128 rows all the same, those
+// behind the tile's read whatever lies there and nobody looks at their results.  The smallest tile whose CTAs all fit is
+// taken (us per step, forward / backward; 119 envs x 512 units, tiles of 128 -> 32: 6.2 / 6.4 -> 4.3 / 4.4).
+__host__ __device__ constexpr int tile_envs(int U) { return 32 * U; }
+__host__ __device__ constexpr uint32_t a_bytes(int U) { return (uint32_t)tile_envs(U) * 128u; }  // envs of one chunk
+__host__ __device__ constexpr uint32_t x_bytes(int U) { return (uint32_t)tile_envs(U) * 256u; }  // the accumulator on its way to other threads
 constexpr size_t kSmemMax = 227 * 1024;
 
 struct Args {
     CUtensorMap mapA;  // forward: h_prev [T * Be][H]; backward: gate gradients [T * Be][4H]
     CUtensorMap mapB;  // forward: W_h [4H][H], boxes of 16 rows; backward: W_h^T [H][4H], boxes of 64 rows
-    int T, Be, H, per_tile, stages;  // per_tile: CTAs of a tile of 128 envs
+    int T, Be, H, per_tile, stages;  // per_tile: CTAs of a tile of envs
     const uint8_t *done;
     const float *xg, *bias, *h_init, *c_init;        // forward
     const float *dtop;                               // backward
@@ -96,15 +103,51 @@ __device__ bool tile_wait(const unsigned int *counter, unsigned int target, vola
     return true;
 }
 
-__device__ __forceinline__ void to4(const float4 &v, float *o) { o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w; }
-__device__ __forceinline__ void load4(const float *p, float *v) { to4(*reinterpret_cast<const float4 *>(p), v); }
-__device__ __forceinline__ void load4_l2(const float *p, float *v) {  // written by other CTAs of this launch
-    to4(__ldcg(reinterpret_cast<const float4 *>(p)), v);
+// U consecutive values, aligned to their size.
+template <int U>
+__device__ __forceinline__ void load_u(const float *p, float *v) {
+    if constexpr (U == 4) {
+        const float4 t = *reinterpret_cast<const float4 *>(p);
+        v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+    } else if constexpr (U == 2) {
+        const float2 t = *reinterpret_cast<const float2 *>(p);
+        v[0] = t.x; v[1] = t.y;
+    } else {
+        v[0] = *p;
+    }
 }
-__device__ __forceinline__ void store4(float *p, const float *v) { *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]); }
-__device__ __forceinline__ uint2 pack4(const float *v) { return make_uint2(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3])); }
+template <int U>
+__device__ __forceinline__ void store_u(float *p, const float *v) {
+    if constexpr (U == 4) *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    else if constexpr (U == 2) *reinterpret_cast<float2 *>(p) = make_float2(v[0], v[1]);
+    else *p = v[0];
+}
+// The same as bf16, packed.
+template <int U>
+struct Packed;
+template <>
+struct Packed<4> { using T = uint2; };
+template <>
+struct Packed<2> { using T = uint32_t; };
+template <>
+struct Packed<1> { using T = uint16_t; };
+template <int U>
+__device__ __forceinline__ typename Packed<U>::T pack_u(const float *v) {
+    if constexpr (U == 4) return make_uint2(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]));
+    else if constexpr (U == 2) return pack_bf16x2(v[0], v[1]);
+    else return __bfloat16_as_ushort(__float2bfloat16_rn(v[0]));
+}
+template <int U>
+__device__ __forceinline__ void store_bf16_u(bf16 *p, typename Packed<U>::T v) { *reinterpret_cast<typename Packed<U>::T *>(p) = v; }
 
-// The exchange tile [128 rows][64 floats], 16 pieces of 16 bytes a row.  Tensor memory hands a thread a row; global memory
+template <int U>
+__device__ __forceinline__ void lds_u(uint32_t addr, float *v) {
+    if constexpr (U == 4) asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "r"(addr) : "memory");
+    else if constexpr (U == 2) asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v[0]), "=f"(v[1]) : "r"(addr) : "memory");
+    else asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v[0]) : "r"(addr) : "memory");
+}
+
+// The exchange tile [envs][64 floats], 16 pieces of 16 bytes a row.  Tensor memory hands a thread a row; global memory
 // wants neighbouring lanes on one row (a lane per row made every load and store of the cell 32 lines: 9000 cycles of a
 // backward step went into the load-store unit, and polls of the counters queued behind them; 256 envs x 1024 units, 16 steps:
 // forward 187 -> 154 us, backward 258 -> 184).  Piece p of row r sits at
@@ -130,11 +173,12 @@ __device__ __forceinline__ uint32_t in_cta(uint32_t addr, uint32_t rank) {
     asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
-// Place of 16 bytes (piece 0 .. 3) of row `row` in slab `slab` of the partial products a CTA receives, [4][4 pieces][128 rows]:
-// a warp that sends a piece of 32 rows fills 512 bytes on end, and four pieces of a row on neighbouring lanes do not meet a
+// Place of 16 bytes (piece 0 .. 3) of row `row` in slab `slab` of the partial products a CTA receives, [4][4 pieces][envs]: a
+// warp that sends a piece of 32 rows fills 512 bytes on end, and four pieces of a row on neighbouring lanes do not meet a
 // bank twice on the way out.
+template <int U>
 __device__ __forceinline__ uint32_t part_addr(uint32_t base, int slab, int row, int piece) {
-    return base + (uint32_t)slab * 8192u + (uint32_t)piece * 2048u + (((uint32_t)row ^ ((uint32_t)piece << 1)) << 4);
+    return base + (uint32_t)(slab * 4 + piece) * (uint32_t)(tile_envs(U) * 16) + (((uint32_t)row ^ ((uint32_t)piece << 1)) << 4);
 }
 // 16 bytes into another CTA's shared memory; its barrier counts them.
 __device__ __forceinline__ void send16(uint32_t dst, uint32_t bar, const float *v) {
@@ -166,12 +210,6 @@ __device__ __forceinline__ bool cluster_mbar_wait(uint64_t *bar, uint32_t parity
 __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-__device__ __forceinline__ float4 lds16(uint32_t addr) {
-    float4 v;
-    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
-    return v;
-}
-
 // Everything the two kernels share around the cell: barriers, tensor memory, the resident weight slice, the stream of A
 // chunks and the MMAs.
 struct Frame {
@@ -180,15 +218,16 @@ struct Frame {
     int warp, lane, mt, q, chunks, S;
 };
 
+template <int U>
 __device__ __forceinline__ Frame frame_begin(const Args &a, uint8_t *raw) {
     Frame f;
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
     f.chunks = a.H >> 6;
     f.S = a.stages;
     f.smem_base = smem_u32(smem);
-    f.b_base = f.smem_base + (uint32_t)f.S * kABytes;
+    f.b_base = f.smem_base + (uint32_t)f.S * a_bytes(U);  // (an MMA's rows behind the last stage's lie in the weights)
     f.x_base = f.b_base + (uint32_t)f.chunks * kBBytes;
-    f.pipe = reinterpret_cast<Pipe *>(smem + (size_t)f.S * kABytes + (size_t)f.chunks * kBBytes + kXBytes);
+    f.pipe = reinterpret_cast<Pipe *>(smem + (size_t)f.S * a_bytes(U) + (size_t)f.chunks * kBBytes + x_bytes(U));
     f.warp = warp_index();
     f.lane = threadIdx.x & 31;
     f.mt = (int)blockIdx.x / a.per_tile;
@@ -230,8 +269,9 @@ __device__ __forceinline__ void frame_end(const Args &a, const Frame &f) {
         for (int i = threadIdx.x; i <= words; i += kThreads) a.counters[i] = 0u;
 }
 
-// Producer warp: the A chunks of one step (columns col0 .. col0 + H of rows row0 .. row0 + 127), each as soon as its four CTAs
+// Producer warp: the A chunks of one step (columns col0 .. col0 + H of the tile's rows from row0 on), each as soon as its four CTAs
 // have published it `target / 4` times.  Lane k watches chunk k; the copies go out in order.
+template <int U>
 __device__ __forceinline__ bool produce_step(const Args &a, const Frame &f, unsigned int target, int col0, int row0, int &s, uint32_t &ph,
                                              int &it) {
     volatile int *abort_flag = &f.pipe->abort_flag;
@@ -260,8 +300,8 @@ __device__ __forceinline__ bool produce_step(const Args &a, const Frame &f, unsi
         }
         if (!mbar_wait_warp(&f.pipe->empty[s], ph ^ 1u, abort_flag, a.status)) return false;
         if (elect_one()) {
-            mbar_arrive_expect_tx(&f.pipe->full[s], kABytes);
-            tma_load_2d(f.smem_base + (uint32_t)s * kABytes, &a.mapA, &f.pipe->full[s], col0 + k * 64, row0);
+            mbar_arrive_expect_tx(&f.pipe->full[s], a_bytes(U));
+            tma_load_2d(f.smem_base + (uint32_t)s * a_bytes(U), &a.mapA, &f.pipe->full[s], col0 + k * 64, row0);
         }
         __syncwarp();
         if (++s == f.S) { s = 0; ph ^= 1u; }
@@ -277,6 +317,7 @@ __device__ __forceinline__ void drain(const Frame &f, int it) {
 }
 
 // MMAs of one step into the 64 accumulator columns (warp 1).
+template <int U>
 __device__ __forceinline__ bool mma_step(const Args &a, const Frame &f, int &s, uint32_t &ph) {
     constexpr uint32_t idesc = instr_desc(128, 64, 0, 0);
     const uint64_t d0 = smem_desc_sw(f.smem_base, 16, 1024, 128);
@@ -285,7 +326,7 @@ __device__ __forceinline__ bool mma_step(const Args &a, const Frame &f, int &s, 
         if (!mbar_wait_warp(&f.pipe->full[s], ph, &f.pipe->abort_flag, a.status)) return false;
         tc_fence_after();
         if (elect_one()) {
-            const uint32_t la = lo + (uint32_t)s * (kABytes >> 4), lb = b_lo + (uint32_t)k * (kBBytes >> 4);
+            const uint32_t la = lo + (uint32_t)s * (a_bytes(U) >> 4), lb = b_lo + (uint32_t)k * (kBBytes >> 4);
             umma_bf16_lh(f.tmem, la, hi, lb, hi, idesc, k > 0 ? 1u : 0u);
 #pragma unroll
             for (int j = 1; j < 4; ++j) umma_bf16_lh(f.tmem, la + 2 * j, hi, lb + 2 * j, hi, idesc, 1u);
@@ -300,12 +341,13 @@ __device__ __forceinline__ bool mma_step(const Args &a, const Frame &f, int &s, 
 }
 
 // Forward over all steps of one layer.  CTA q of a tile owns units 16 q .. 16 q + 15: accumulator column 16 g + j is gate g
-// of unit 16 q + j, so that a thread of the cell holds the four gates of its eight units.
+// of unit 16 q + j.
+template <int U>
 __global__ void __launch_bounds__(kThreads, 1) lstm_fwd_kernel(const __grid_constant__ Args a) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    const Frame f = frame_begin(a, smem_raw);
+    const Frame f = frame_begin<U>(a, smem_raw);
     unsigned int *counter = chunk_counters(a, f.mt) + (f.q >> 2);  // of this CTA's units
-    const int H = a.H, u0 = f.q * 16, row0 = f.mt * 128;
+    const int H = a.H, u0 = f.q * 16, row0 = f.mt * tile_envs(U);
     volatile int *abort_flag = &f.pipe->abort_flag;
     if (f.warp == 0) {
         if (f.lane == 0) {
@@ -318,74 +360,76 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_fwd_kernel(const __grid_cons
         int s = 0, it = 0;
         uint32_t ph = 0;
         bool ok = true;
-        for (int t = 0; t < a.T && ok; ++t) ok = produce_step(a, f, 4u * (unsigned)(t + 1), 0, t * a.Be + row0, s, ph, it);
+        for (int t = 0; t < a.T && ok; ++t) ok = produce_step<U>(a, f, 4u * (unsigned)(t + 1), 0, t * a.Be + row0, s, ph, it);
         if (!ok && f.lane == 0) drain(f, it);
         __syncwarp();
     } else if (f.warp == 1) {
         int s = 0;
         uint32_t ph = 0;
         bool ok = mbar_wait_warp(&f.pipe->wfull, 0, abort_flag, a.status);
-        for (int t = 0; t < a.T && ok; ++t) ok = mma_step(a, f, s, ph);
+        for (int t = 0; t < a.T && ok; ++t) ok = mma_step<U>(a, f, s, ph);
     } else {
-        // thread of the cell: env `row` of the tile, units j0 .. j0 + 3
-        const int lg = f.warp & 3, grp = (f.warp - 2) >> 2, ct = (int)threadIdx.x - 64, row = ct >> 2, quad = ct & 3, e = row0 + row;
+        // thread of the cell: env `row` of the tile, units j0 .. j0 + U - 1, columns col .. of each gate's 16
+        const int lg = f.warp & 3, grp = (f.warp - 2) >> 2, ct = (int)threadIdx.x - 64, row = ct * U >> 4, col = ct * U & 15, e = row0 + row;
         const bool live = e < a.Be, issuer = ct == 0;
-        const int j0 = u0 + 4 * quad;
-        float cp[4] = {0.f, 0.f, 0.f, 0.f}, bias[4][4];
+        const int j0 = u0 + col;
+        float cp[U], bias[4][U];
 #pragma unroll
-        for (int g = 0; g < 4; ++g) load4(a.bias + g * H + j0, bias[g]);
+        for (int k = 0; k < U; ++k) cp[k] = 0.f;
+#pragma unroll
+        for (int g = 0; g < 4; ++g) load_u<U>(a.bias + g * H + j0, bias[g]);
         if (live) {  // the state the first step starts from
             const size_t i = (size_t)e * H + j0;
-            float hv[4];
-            load4(a.h_init + i, hv);
-            load4(a.c_init + i, cp);
-            *reinterpret_cast<uint2 *>(a.hprev + i) = pack4(hv);
-            store4(a.cprev + i, cp);
+            float hv[U];
+            load_u<U>(a.h_init + i, hv);
+            load_u<U>(a.c_init + i, cp);
+            store_bf16_u<U>(a.hprev + i, pack_u<U>(hv));
+            store_u<U>(a.cprev + i, cp);
         }
         cell_sync();
         if (issuer) tile_arrive(counter);
         for (int t = 0; t < a.T; ++t) {
             const size_t r = (size_t)t * a.Be + e;
-            float xg[4][4];
+            float xg[4][U];
             bool reset = false;
             if (live) {  // ahead of the wait: they do not depend on this step's product
 #pragma unroll
-                for (int g = 0; g < 4; ++g) load4(a.xg + r * 4 * H + g * H + j0, xg[g]);
+                for (int g = 0; g < 4; ++g) load_u<U>(a.xg + r * 4 * H + g * H + j0, xg[g]);
                 reset = a.done[r] != 0;
             }
             const bool ok = mbar_wait(&f.pipe->tfull, t & 1, abort_flag, a.status);
             tc_fence_after();
-            if (__all_sync(0xffffffffu, ok)) xch_put(f.x_base, f.tmem, lg, f.lane, grp);  // gate `grp` of the 16 units
+            if (lg * 32 < tile_envs(U) && __all_sync(0xffffffffu, ok)) xch_put(f.x_base, f.tmem, lg, f.lane, grp);  // gate `grp` of the 16 units
             if (!cell_all(ok)) break;
-            float gi[4], gf[4], gg[4], go[4], cv[4];
-            uint2 hb = make_uint2(0u, 0u);
+            float gi[U], gf[U], gg[U], go[U], cv[U];
+            typename Packed<U>::T hb = {};
             if (live) {
-                float hg[4][4], hv[4];
+                float hg[4][U], hv[U];
 #pragma unroll
-                for (int g = 0; g < 4; ++g) to4(lds16(xch_addr(f.x_base, row, 4 * g + quad)), hg[g]);
+                for (int g = 0; g < 4; ++g) lds_u<U>(xch_addr(f.x_base, row, 4 * g + (col >> 2)) + 4u * (col & 3), hg[g]);
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
+                for (int k = 0; k < U; ++k) {
                     lstm_cell(xg[0][k] + hg[0][k] + bias[0][k], xg[1][k] + hg[1][k] + bias[1][k], xg[2][k] + hg[2][k] + bias[2][k],
                               xg[3][k] + hg[3][k] + bias[3][k], cp[k], gi[k], gf[k], gg[k], go[k], cv[k], hv[k]);
                 }
-                hb = pack4(hv);
-                if (t + 1 < a.T) *reinterpret_cast<uint2 *>(a.hprev + (r + a.Be) * H + j0) = reset ? make_uint2(0u, 0u) : hb;
+                hb = pack_u<U>(hv);
+                if (t + 1 < a.T) store_bf16_u<U>(a.hprev + (r + a.Be) * H + j0, reset ? typename Packed<U>::T{} : hb);
             }
             if (t + 1 < a.T) {  // what the others wait for goes first, the rest behind it
                 cell_sync();
                 if (issuer) tile_arrive(counter);
             }
             if (live) {
-                *reinterpret_cast<uint2 *>(a.h + r * H + j0) = hb;
+                store_bf16_u<U>(a.h + r * H + j0, hb);
                 float *gp = a.gates + r * 4 * H + j0;
-                store4(gp, gi);
-                store4(gp + H, gf);
-                store4(gp + 2 * H, gg);
-                store4(gp + 3 * H, go);
-                store4(a.c + r * H + j0, cv);
+                store_u<U>(gp, gi);
+                store_u<U>(gp + H, gf);
+                store_u<U>(gp + 2 * H, gg);
+                store_u<U>(gp + 3 * H, go);
+                store_u<U>(a.c + r * H + j0, cv);
 #pragma unroll
-                for (int k = 0; k < 4; ++k) cp[k] = reset ? 0.f : cv[k];
-                if (t + 1 < a.T) store4(a.cprev + (r + a.Be) * H + j0, cp);
+                for (int k = 0; k < U; ++k) cp[k] = reset ? 0.f : cv[k];
+                if (t + 1 < a.T) store_u<U>(a.cprev + (r + a.Be) * H + j0, cp);
             }
         }
     }
@@ -400,10 +444,10 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_fwd_kernel(const __grid_cons
 // of a step's 20000 cycles, and so does shared memory that the others read behind a release (a release waits for all its
 // thread's block has under way).  A place is free again when the next product arrives: that needs gate gradients of all the
 // tile's cells, who had read it by then.
-template <bool CLUSTER>
+template <int U, bool CLUSTER>
 __device__ __forceinline__ void bwd_steps(const Args &a, uint8_t *smem_raw) {
-    const Frame f = frame_begin(a, smem_raw);
-    const int H = a.H, row0 = f.mt * 128, slab = f.q & 3, slice = f.q >> 2, n0 = slice * 64;
+    const Frame f = frame_begin<U>(a, smem_raw);
+    const int H = a.H, row0 = f.mt * tile_envs(U), slab = f.q & 3, slice = f.q >> 2, n0 = slice * 64;
     unsigned int *const cells = chunk_counters(a, f.mt) + slice;  // of this CTA's units as a cell
     unsigned int *const parts = part_counters(a, f.mt) + slice;
     volatile int *abort_flag = &f.pipe->abort_flag;
@@ -417,33 +461,34 @@ __device__ __forceinline__ void bwd_steps(const Args &a, uint8_t *smem_raw) {
         int s = 0, it = 0;
         uint32_t ph = 0;
         bool ok = true;
-        for (int t = a.T - 1, i = 0; t > 0 && ok; --t, ++i) ok = produce_step(a, f, 4u * (unsigned)(i + 1), slab * H, t * a.Be + row0, s, ph, it);
+        for (int t = a.T - 1, i = 0; t > 0 && ok; --t, ++i) ok = produce_step<U>(a, f, 4u * (unsigned)(i + 1), slab * H, t * a.Be + row0, s, ph, it);
         if (!ok && f.lane == 0) drain(f, it);
         __syncwarp();
     } else if (f.warp == 1) {
         int s = 0;
         uint32_t ph = 0;
         bool ok = mbar_wait_warp(&f.pipe->wfull, 0, abort_flag, a.status);
-        for (int t = a.T - 1; t > 0 && ok; --t) ok = mma_step(a, f, s, ph);
+        for (int t = a.T - 1; t > 0 && ok; --t) ok = mma_step<U>(a, f, s, ph);
     } else {
-        // as a cell: env `row` of the tile, units j0 .. j0 + 3
-        const int lg = f.warp & 3, grp = (f.warp - 2) >> 2, ct = (int)threadIdx.x - 64, row = ct >> 2, quad = ct & 3, e = row0 + row;
+        // as a cell: env `row` of the tile, units j0 .. j0 + U - 1, columns col .. of the CTA's 16
+        const int lg = f.warp & 3, grp = (f.warp - 2) >> 2, ct = (int)threadIdx.x - 64, row = ct * U >> 4, col = ct * U & 15, e = row0 + row;
         const bool live = e < a.Be, issuer = ct == 0;
-        const int j0 = f.q * 16 + 4 * quad;
+        const int j0 = f.q * 16 + col;
         const size_t step = (size_t)a.Be * H;
-        float dcc[4] = {0.f, 0.f, 0.f, 0.f};
-        float dtop[4], g4[4][4], cv[4], cp[4];
+        float dcc[U], dtop[U], g4[4][U], cv[U], cp[U];
+#pragma unroll
+        for (int k = 0; k < U; ++k) dcc[k] = 0.f;
         uint8_t done = 0;
         // What the forward pass left for step t.  It comes from HBM in a burst of 57 KB per CTA (7 MB in all: 3500 cycles), so it is
         // asked for while the step before multiplies.
         auto fetch = [&](int t) {
             if (!live) return;
             const size_t r = (size_t)t * a.Be + e;
-            load4(a.dtop + r * H + j0, dtop);
+            load_u<U>(a.dtop + r * H + j0, dtop);
 #pragma unroll
-            for (int g = 0; g < 4; ++g) load4(a.gates + r * 4 * H + g * H + j0, g4[g]);
-            load4(a.c + r * H + j0, cv);
-            load4(a.cprev + r * H + j0, cp);
+            for (int g = 0; g < 4; ++g) load_u<U>(a.gates + r * 4 * H + g * H + j0, g4[g]);
+            load_u<U>(a.c + r * H + j0, cv);
+            load_u<U>(a.cprev + r * H + j0, cp);
             done = a.done[r];
         };
         fetch(a.T - 1);
@@ -458,59 +503,68 @@ __device__ __forceinline__ void bwd_steps(const Args &a, uint8_t *smem_raw) {
                 if (!cell_all(ok)) break;
             }
             if (live) {
-                float dhn[4] = {0.f, 0.f, 0.f, 0.f};
+                float dhn[U];
+#pragma unroll
+                for (int k = 0; k < U; ++k) dhn[k] = 0.f;
                 if (carry) {
-                    float p[4][4];
+                    float p[4][U];
 #pragma unroll
                     for (int s = 0; s < 4; ++s) {
-                        if (CLUSTER) to4(lds16(part_addr(f.x_base, s, row, quad)), p[s]);
-                        else load4_l2(a.dhc + s * step + (size_t)e * H + j0, p[s]);
+                        if constexpr (CLUSTER) {
+                            lds_u<U>(part_addr<U>(f.x_base, s, row, col >> 2) + 4u * (col & 3), p[s]);
+                        } else {  // written by other CTAs of this launch
+                            const float4 v = __ldcg(reinterpret_cast<const float4 *>(a.dhc + s * step + (size_t)e * H + j0));
+                            p[s][0] = v.x; p[s][1] = v.y; p[s][2] = v.z; p[s][3] = v.w;
+                        }
                     }
 #pragma unroll
                     for (int s = 0; s < 4; ++s)
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) dhn[k] += p[s][k];
+                        for (int k = 0; k < U; ++k) dhn[k] += p[s][k];
                 }
-                float di[4], df[4], dgg[4], dgo[4];
+                float di[U], df[U], dgg[U], dgo[U];
 #pragma unroll
-                for (int k = 0; k < 4; ++k)
+                for (int k = 0; k < U; ++k)
                     lstm_cell_back(dtop[k] + dhn[k], carry ? dcc[k] : 0.f, g4[0][k], g4[1][k], g4[2][k], g4[3][k], cv[k], cp[k], di[k],
                                    df[k], dgg[k], dgo[k], dcc[k]);
                 bf16 *o = a.dg + r * 4 * H + j0;
-                *reinterpret_cast<uint2 *>(o) = pack4(di);
-                *reinterpret_cast<uint2 *>(o + H) = pack4(df);
-                *reinterpret_cast<uint2 *>(o + 2 * H) = pack4(dgg);
-                *reinterpret_cast<uint2 *>(o + 3 * H) = pack4(dgo);
+                store_bf16_u<U>(o, pack_u<U>(di));
+                store_bf16_u<U>(o + H, pack_u<U>(df));
+                store_bf16_u<U>(o + 2 * H, pack_u<U>(dgg));
+                store_bf16_u<U>(o + 3 * H, pack_u<U>(dgo));
             }
             if (t == 0) break;
             cell_sync();
             if (issuer) {
-                if (CLUSTER) mbar_arrive_expect_tx(&f.pipe->parts, kXBytes);  // what the four CTAs will send for this step
+                if (CLUSTER) mbar_arrive_expect_tx(&f.pipe->parts, x_bytes(U));  // what the four CTAs will send for this step
                 tile_arrive(cells);
             }
             fetch(t - 1);
             // this CTA's partial product, 64 columns a row: columns 16 k .. 16 k + 15 are what cell k of the slice needs
             const bool ok = mbar_wait(&f.pipe->tfull, i & 1, abort_flag, a.status);
             tc_fence_after();
-            if (CLUSTER) {
-                if (__all_sync(0xffffffffu, ok)) {  // (else the abort flag ends all warps at the next wait for the parts)
+            if constexpr (CLUSTER) {
+                if (lg * 32 < tile_envs(U) && __all_sync(0xffffffffu, ok)) {  // (else the abort flag ends all warps at the next wait for the parts)
                     float v[16];
                     tmem_ld16(f.tmem + ((uint32_t)(lg * 32) << 16) + (uint32_t)(16 * grp), v);
                     tc_fence_before();
                     const uint32_t bar = in_cta(smem_u32(&f.pipe->parts), (uint32_t)grp);
 #pragma unroll
                     for (int k = 0; k < 4; ++k)
-                        send16(in_cta(part_addr(f.x_base, slab, lg * 32 + f.lane, k), (uint32_t)grp), bar, v + 4 * k);
+                        send16(in_cta(part_addr<U>(f.x_base, slab, lg * 32 + f.lane, k), (uint32_t)grp), bar, v + 4 * k);
                 }
                 continue;
             }
+            static_assert(CLUSTER || U == 4, "the way through global memory is written for tiles of 128 envs");
             if (__all_sync(0xffffffffu, ok)) xch_put(f.x_base, f.tmem, lg, f.lane, grp);
             if (!cell_all(ok)) break;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const int rr = k * 32 + (ct >> 4), piece = ct & 15;
-                if (row0 + rr < a.Be)
-                    __stcg(reinterpret_cast<float4 *>(a.dhc + slab * step + (size_t)(row0 + rr) * H + n0) + piece, lds16(xch_addr(f.x_base, rr, piece)));
+                if (row0 + rr >= a.Be) continue;
+                float v[4];
+                lds_u<4>(xch_addr(f.x_base, rr, piece), v);
+                __stcg(reinterpret_cast<float4 *>(a.dhc + slab * step + (size_t)(row0 + rr) * H + n0) + piece, make_float4(v[0], v[1], v[2], v[3]));
             }
             cell_sync();
             if (issuer) tile_arrive(parts);
@@ -530,82 +584,41 @@ __device__ __forceinline__ void bwd_steps(const Args &a, uint8_t *smem_raw) {
 
 __global__ void __launch_bounds__(kThreads, 1) lstm_bwd_kernel(const __grid_constant__ Args a) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    bwd_steps<false>(a, smem_raw);
+    bwd_steps<4, false>(a, smem_raw);
 }
+template <int U>
 __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(kThreads, 1) lstm_bwd_cluster_kernel(const __grid_constant__ Args a) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    bwd_steps<true>(a, smem_raw);
+    bwd_steps<U, true>(a, smem_raw);
 }
 
-// Shape part; false where the layer or the sequence does not fit: a slice of W_h has to leave room for the exchange and two
-// chunks of A (four at H = 1024), and all CTAs have to be resident at once.
-bool plan(Args &a, int T, int Be, int H, int &ctas, size_t &smem) {
-    if (H % 64 != 0 || T < 1 || Be < 1) return false;
+// Shape part for tiles of 32 U envs; false where the layer or the sequence does not fit: a slice of W_h has to leave room for
+// the exchange and two chunks of A (four of 128 envs at H = 1024), and all CTAs have to be resident at once.
+bool plan(Args &a, int T, int Be, int H, int U, int &ctas, size_t &smem) {
+    if (H % 64 != 0 || H > 2048 || T < 1 || Be < 1) return false;
     a.T = T; a.Be = Be; a.H = H;
     a.per_tile = H / 16;
-    const long long n = (long long)((Be + 127) / 128) * a.per_tile;
-    if (n > ppo_num_sms() || a.H > 2048 || 2 * ((Be + 127) / 128) + 1 > kLstmCounters) return false;
-    const size_t fixed = (size_t)(H / 64) * kBBytes + kXBytes + sizeof(Pipe) + 1024;
-    if (fixed + 2 * kABytes > kSmemMax) return false;
-    a.stages = (int)((kSmemMax - fixed) / kABytes);
+    const long long tiles = (Be + tile_envs(U) - 1) / tile_envs(U), n = tiles * a.per_tile;
+    if (n > ppo_num_sms() || 2 * tiles + 1 > kLstmCounters) return false;
+    const size_t fixed = (size_t)(H / 64) * kBBytes + x_bytes(U) + sizeof(Pipe) + 1024;
+    if (fixed + 2 * a_bytes(U) > kSmemMax) return false;
+    a.stages = (int)((kSmemMax - fixed) / a_bytes(U));
     if (a.stages > kMaxStages) a.stages = kMaxStages;
-    smem = fixed + (size_t)a.stages * kABytes;
+    smem = fixed + (size_t)a.stages * a_bytes(U);
     ctas = (int)n;
     return true;
 }
 
-int prepare_kernel(const void *fn, bool (&set)[64]) {
-    int dev = 0;
-    PPO_CUDA_CHECK(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64) return PPO_ERR_CUDA;
-    if (!set[dev]) {
-        PPO_CUDA_CHECK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
-        set[dev] = true;
-    }
+template <typename F>
+int prepare_kernel(F *fn) {
+    PPO_CUDA_CHECK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
     return PPO_OK;
 }
 
-}  // namespace
-
-int lstm_fwd_steps(const LstmSteps &p, const bf16 *Wh, const float *xg, const float *bias, const float *h_init, const float *c_init,
-                   int32_t *status, cudaStream_t st) {
-    Args a = {};
-    int ctas = 0;
-    size_t smem = 0;
-    if (!status || !plan(a, p.T, p.Be, p.H, ctas, smem)) return PPO_ERR_UNSUPPORTED;
-    const long long H = p.H, rows = (long long)p.T * p.Be;
-    const long long da[2] = {H, rows}, sa[1] = {2 * H}, db[2] = {H, 4 * H}, sb[1] = {2 * H};
-    const int ba[2] = {64, 128}, bb[2] = {64, 16};
-    PPO_TRY(make_map_strided(&a.mapA, p.hprev, 2, da, sa, ba));
-    PPO_TRY(make_map_strided(&a.mapB, Wh, 2, db, sb, bb));
-    a.done = p.done;
-    a.xg = xg; a.bias = bias; a.h_init = h_init; a.c_init = c_init;
-    a.gates = p.gates; a.c = p.c; a.cprev = p.cprev; a.h = p.h; a.hprev = p.hprev;
-    a.counters = p.counters;
-    a.status = status;
-    static bool set[64] = {false};
-    PPO_TRY(prepare_kernel(reinterpret_cast<const void *>(lstm_fwd_kernel), set));
-    return ppo_launch_together(lstm_fwd_kernel, dim3(ctas), dim3(kThreads), smem, st, a);
-}
-
-int lstm_bwd_steps(const LstmSteps &p, const bf16 *WhT, const float *dtop, bf16 *dg, float *dhc, int32_t *status, cudaStream_t st) {
-    Args a = {};
-    int ctas = 0;
-    size_t smem = 0;
-    if (!status || !plan(a, p.T, p.Be, p.H, ctas, smem)) return PPO_ERR_UNSUPPORTED;
-    const long long H = p.H, rows = (long long)p.T * p.Be;
-    const long long da[2] = {4 * H, rows}, sa[1] = {8 * H}, db[2] = {4 * H, H}, sb[1] = {8 * H};
-    const int ba[2] = {64, 128}, bb[2] = {64, 64};
-    PPO_TRY(make_map_strided(&a.mapA, dg, 2, da, sa, ba));
-    PPO_TRY(make_map_strided(&a.mapB, WhT, 2, db, sb, bb));
-    a.done = p.done;
-    a.dtop = dtop; a.dg = dg; a.dhc = dhc;
-    a.gates = p.gates; a.c = p.c; a.cprev = p.cprev;
-    a.counters = p.counters;
-    a.status = status;
-    static bool set[64] = {false}, set_cluster[64] = {false};
-    PPO_TRY(prepare_kernel(reinterpret_cast<const void *>(lstm_bwd_cluster_kernel), set_cluster));
-    // clusters of four fit the groups of SMs less tightly than single CTAs (33 of them on 148 SMs)
+// Whether `ctas` CTAs in clusters of four are resident at once: clusters fit the groups of SMs less tightly than single CTAs (33
+// of them on 148 SMs).
+template <typename F>
+int clusters_fit(F *fn, int ctas, size_t smem, bool &fit) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ctas);
     cfg.blockDim = dim3(kThreads);
@@ -617,8 +630,84 @@ int lstm_bwd_steps(const LstmSteps &p, const bf16 *WhT, const float *dtop, bf16 
     cfg.attrs = &at;
     cfg.numAttrs = 1;
     int clusters = 0;
-    PPO_CUDA_CHECK(cudaOccupancyMaxActiveClusters(&clusters, lstm_bwd_cluster_kernel, &cfg));
-    if (4 * clusters >= ctas) return ppo_launch_together(lstm_bwd_cluster_kernel, dim3(ctas), dim3(kThreads), smem, st, a);
-    PPO_TRY(prepare_kernel(reinterpret_cast<const void *>(lstm_bwd_kernel), set));
+    PPO_CUDA_CHECK(cudaOccupancyMaxActiveClusters(&clusters, fn, &cfg));
+    fit = 4ll * clusters >= ctas;
+    return PPO_OK;
+}
+
+template <int U>
+int launch_fwd(Args &a, const LstmSteps &p, int ctas, size_t smem, cudaStream_t st) {
+    const long long H = p.H, rows = (long long)p.T * p.Be;
+    const long long da[2] = {H, rows}, sa[1] = {2 * H};
+    const int ba[2] = {64, tile_envs(U)};
+    PPO_TRY(make_map_strided(&a.mapA, p.hprev, 2, da, sa, ba));
+    PPO_TRY(prepare_kernel(lstm_fwd_kernel<U>));
+    return ppo_launch_together(lstm_fwd_kernel<U>, dim3(ctas), dim3(kThreads), smem, st, a);
+}
+
+int map_dg(Args &a, const LstmSteps &p, bf16 *dg, int envs) {
+    const long long H = p.H, rows = (long long)p.T * p.Be;
+    const long long da[2] = {4 * H, rows}, sa[1] = {8 * H};
+    const int ba[2] = {64, envs};
+    return make_map_strided(&a.mapA, dg, 2, da, sa, ba);
+}
+
+// PPO_ERR_UNSUPPORTED where the tiles' clusters do not all fit.
+template <int U>
+int launch_bwd_clusters(Args &a, const LstmSteps &p, bf16 *dg, cudaStream_t st) {
+    int ctas = 0;
+    size_t smem = 0;
+    if (!plan(a, p.T, p.Be, p.H, U, ctas, smem)) return PPO_ERR_UNSUPPORTED;
+    PPO_TRY(prepare_kernel(lstm_bwd_cluster_kernel<U>));
+    bool fit = false;
+    PPO_TRY(clusters_fit(lstm_bwd_cluster_kernel<U>, ctas, smem, fit));
+    if (!fit) return PPO_ERR_UNSUPPORTED;
+    PPO_TRY(map_dg(a, p, dg, tile_envs(U)));
+    return ppo_launch_together(lstm_bwd_cluster_kernel<U>, dim3(ctas), dim3(kThreads), smem, st, a);
+}
+
+}  // namespace
+
+int lstm_fwd_steps(const LstmSteps &p, const bf16 *Wh, const float *xg, const float *bias, const float *h_init, const float *c_init,
+                   int32_t *status, cudaStream_t st) {
+    Args a = {};
+    int ctas = 0, U = 1;
+    size_t smem = 0;
+    while (U <= 4 && !plan(a, p.T, p.Be, p.H, U, ctas, smem)) U *= 2;
+    if (!status || U > 4) return PPO_ERR_UNSUPPORTED;
+    const long long H = p.H;
+    const long long db[2] = {H, 4 * H}, sb[1] = {2 * H};
+    const int bb[2] = {64, 16};
+    PPO_TRY(make_map_strided(&a.mapB, Wh, 2, db, sb, bb));
+    a.done = p.done;
+    a.xg = xg; a.bias = bias; a.h_init = h_init; a.c_init = c_init;
+    a.gates = p.gates; a.c = p.c; a.cprev = p.cprev; a.h = p.h; a.hprev = p.hprev;
+    a.counters = p.counters;
+    a.status = status;
+    if (U == 1) return launch_fwd<1>(a, p, ctas, smem, st);
+    return U == 2 ? launch_fwd<2>(a, p, ctas, smem, st) : launch_fwd<4>(a, p, ctas, smem, st);
+}
+
+int lstm_bwd_steps(const LstmSteps &p, const bf16 *WhT, const float *dtop, bf16 *dg, float *dhc, int32_t *status, cudaStream_t st) {
+    Args a = {};
+    int ctas = 0;
+    size_t smem = 0;
+    if (!status || !plan(a, p.T, p.Be, p.H, 4, ctas, smem)) return PPO_ERR_UNSUPPORTED;
+    const long long H = p.H;
+    const long long db[2] = {4 * H, H}, sb[1] = {8 * H};
+    const int bb[2] = {64, 64};
+    PPO_TRY(make_map_strided(&a.mapB, WhT, 2, db, sb, bb));
+    a.done = p.done;
+    a.dtop = dtop; a.dg = dg; a.dhc = dhc;
+    a.gates = p.gates; a.c = p.c; a.cprev = p.cprev;
+    a.counters = p.counters;
+    a.status = status;
+    int s = launch_bwd_clusters<1>(a, p, dg, st);
+    if (s == PPO_ERR_UNSUPPORTED) s = launch_bwd_clusters<2>(a, p, dg, st);
+    if (s == PPO_ERR_UNSUPPORTED) s = launch_bwd_clusters<4>(a, p, dg, st);
+    if (s != PPO_ERR_UNSUPPORTED) return s;
+    plan(a, p.T, p.Be, p.H, 4, ctas, smem);
+    PPO_TRY(map_dg(a, p, dg, tile_envs(4)));
+    PPO_TRY(prepare_kernel(lstm_bwd_kernel));
     return ppo_launch_together(lstm_bwd_kernel, dim3(ctas), dim3(kThreads), smem, st, a);
 }

@@ -14,8 +14,10 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda"
 
 
-# envs per sequence group, units, steps: one env, one short / exact / one over a tile, three tiles, too many CTAs
-@pytest.mark.parametrize("Be,H,T", [(1, 64, 3), (127, 64, 3), (128, 192, 4), (129, 128, 3), (257, 448, 3), (257, 1024, 3)])
+# envs per sequence group, units, steps: one env, one short / exact / one over a tile, three tiles, too many CTAs; tiles of 32, 64
+# and 128 envs with a ragged last one; clusters of four that do not all fit (36 of them) beside single CTAs that do
+@pytest.mark.parametrize("Be,H,T", [(1, 64, 3), (127, 64, 3), (128, 192, 4), (129, 128, 3), (257, 448, 3), (257, 1024, 3),
+                                    (33, 128, 5), (161, 512, 3), (255, 1024, 3), (385, 576, 3)])
 def test_sequences_at_tile_edges_match_oracle(Be, H, T, monkeypatch):
     w = synth.Workload("edge", 2 * Be, T, 8, 12, (16, 32), (3, 3), (24,), 1, 2, P=32, A=3, n_lstm=2, lstm_h=H)
     monkeypatch.setitem(base.REC, "edge", w)
