@@ -115,7 +115,7 @@ struct ppo_model {
     bf16 *xhat[PPO_MAX_CONV + 1];   // with norm: normalised values of conv layer l, [mb][Ho][Wo][C]
     float *rstd[PPO_MAX_CONV + 1];  // with norm: 1 / sqrt(var + eps) per pixel, [mb][Ho][Wo]
     bf16 *dze;                      // with embed: gradient w.r.t. the embedding's pre-activation, [mb][E]
-    float *ln_part;                 // with norm: per-block partial sums of the gamma / beta gradients
+    float *ln_part;                 // with norm: per-block partial sums of the gamma / beta gradients, ln_cap per layer
     size_t ln_cap;
     bf16 *h[PPO_MAX_FC + 1];       // h[0] = [pooled, proprio]; h[l] post-ReLU
     bf16 *dh[PPO_MAX_FC + 2];      // dh[l]: gradient w.r.t. pre-activation of h[l]; dh[F+1]: head dout padded to 16

@@ -553,17 +553,14 @@ __global__ void __launch_bounds__(256) pack_dout_kernel(const float *__restrict_
 
 // dst[i] (i < nA: dstA[i], else dstB[i - nA]) += part[0][i] + part[1][i] + ... in that order: the second stage of the
 // reductions whose blocks leave partial sums instead of adding to the result with atomics (reproducible results).
-__global__ void __launch_bounds__(256) sum_partials_kernel(const float *__restrict__ part, int nparts, int nA,
-                                                           float *__restrict__ dstA, int nB, float *__restrict__ dstB) {
-    grid_wait();
+__device__ __forceinline__ void sum_partials_block(const float *__restrict__ part, int nparts, int nA, float *__restrict__ dstA, int nB,
+                                                   float *__restrict__ dstB, int block) {
     // 32 results per block; eight threads share a result, thread j adding the partials b = j, j + 8, ... in order, and
     // the eight sums are added in the order of j: fixed, whatever the launch.
     __shared__ float sh[8][32];
     const int o = threadIdx.x & 31, j = threadIdx.x >> 5;
-    const int i = blockIdx.x * 32 + o;
+    const int i = block * 32 + o;
     const int n = nA + nB;
-    part += (size_t)blockIdx.y * nparts * n;  // blockIdx.y: one of several independent reductions of nA results (nB = 0)
-    dstA += (size_t)blockIdx.y * nA;
     float acc = 0.f;
     if (i < n) {
         // the loads of eight partials are in flight while the sum stays in order
@@ -587,11 +584,40 @@ __global__ void __launch_bounds__(256) sum_partials_kernel(const float *__restri
         else dstB[i - nA] += v;
     }
 }
+__global__ void __launch_bounds__(256) sum_partials_kernel(const float *__restrict__ part, int nparts, int n, float *__restrict__ dst) {
+    grid_wait();  // blockIdx.y: one of several independent reductions of n results
+    sum_partials_block(part + (size_t)blockIdx.y * nparts * n, nparts, n, dst + (size_t)blockIdx.y * n, 0, nullptr, (int)blockIdx.x);
+}
+// Several reductions in one launch: those of the first layer and of the layer normalisations, whose results nothing in the
+// backward pass waits for (each in a launch of its own between the kernels of the chain cost it 6 us).
+struct SumJob {
+    const float *part;
+    int nparts, nA, nB;
+    float *dstA, *dstB;
+    int block_end;
+};
+struct SumJobs {
+    int n;
+    SumJob j[PPO_MAX_CONV + 1];
+    void add(const float *part, int nparts, int nA, float *dstA, int nB, float *dstB) {
+        j[n] = {part, nparts, nA, nB, dstA, dstB, (n ? j[n - 1].block_end : 0) + ppo_cdiv(nA + nB, 32)};
+        ++n;
+    }
+};
+__global__ void __launch_bounds__(256) sum_partials_jobs_kernel(const __grid_constant__ SumJobs jobs) {
+    grid_wait();
+    int k = 0, first = 0;
+    while ((int)blockIdx.x >= jobs.j[k].block_end) first = jobs.j[k++].block_end;
+    const SumJob &q = jobs.j[k];
+    sum_partials_block(q.part, q.nparts, q.nA, q.dstA, q.nB, q.dstB, (int)blockIdx.x - first);
+}
+static int sum_partials_jobs(const SumJobs &jobs, cudaStream_t st) {
+    if (jobs.n == 0) return PPO_OK;
+    return ppo_launch(sum_partials_jobs_kernel, dim3(jobs.j[jobs.n - 1].block_end), dim3(256), 0, st, jobs);
+}
 
-static int sum_partials(const float *part, int nparts, int nA, float *dstA, int nB, float *dstB, cudaStream_t st,
-                        int slabs = 1) {
-    PPO_TRY(ppo_launch(sum_partials_kernel, dim3(ppo_cdiv(nA + nB, 32), slabs), dim3(256), 0, st, part, nparts, nA, dstA, nB, dstB));
-    return PPO_OK;
+static int sum_partials(const float *part, int nparts, int n, float *dst, cudaStream_t st, int slabs = 1) {
+    return ppo_launch(sum_partials_kernel, dim3(ppo_cdiv(n, 32), slabs), dim3(256), 0, st, part, nparts, n, dst);
 }
 
 // part[block][n] = sum over this block's rows m of dZ[m][n]  (bias gradients, first stage), N a multiple of 8.  Threads
@@ -1035,18 +1061,18 @@ static int run_colsum(const bf16 *dZ, int ld, long long M, int N, float *db, flo
         const int rows_per_pass = 256 / (N / 8);
         const int blocks = colsum_blocks(M, (long long)rows_per_pass * 8);
         PPO_TRY(ppo_launch(colsum_kernel, dim3(blocks), dim3(256), 0, st, dZ, ld, M, N, part));
-        return sum_partials(part, blocks, N, db, 0, nullptr, st);
+        return sum_partials(part, blocks, N, db, st);
     }
     if (N > 256 && N % 256 == 0) {
         // wide layers: slabs of 256 columns along the grid's second axis
         const int blocks = colsum_blocks(M, 64);
         PPO_TRY(ppo_launch(colsum_kernel, dim3(blocks, N / 256), dim3(256), 0, st, dZ, ld, M, 256, part));
-        return sum_partials(part, blocks, 256, db, 0, nullptr, st, N / 256);
+        return sum_partials(part, blocks, 256, db, st, N / 256);
     }
     int blocks = ppo_cdiv(M, 2048);
     blocks = blocks > 64 ? 64 : (blocks < 1 ? 1 : blocks);
     PPO_TRY(ppo_launch(colsum_small_kernel, dim3(blocks, N), dim3(256), 0, st, dZ, ld, M, N, part));
-    return sum_partials(part, blocks, N, db, 0, nullptr, st);
+    return sum_partials(part, blocks, N, db, st);
 }
 
 
@@ -1337,8 +1363,8 @@ static int side_stream(ppo_model *m) {
     return PPO_OK;
 }
 
-// conv1: weight and bias gradients only (there is no dgrad into the depth image).
-static int conv1_wgrad(ppo_model *m, const ppo_minibatch *mb, int row0, int rows, cudaStream_t st) {
+// conv1: weight and bias gradients only (there is no dgrad into the depth image); their second stage goes into `sums`.
+static int conv1_wgrad(ppo_model *m, const ppo_minibatch *mb, int row0, int rows, SumJobs &sums, cudaStream_t st) {
     const ppo_model_desc &d = m->d;
     const __half *depth = static_cast<const __half *>(mb->depth_f16) + (size_t)row0 * d.H * d.W;
     const int C1 = m->Cs[1], KS = d.conv_k[0];
@@ -1373,7 +1399,8 @@ static int conv1_wgrad(ppo_model *m, const ppo_minibatch *mb, int row0, int rows
         else if (KS == 5 && nb == 6) PPO_C1W(5, 6);
         else PPO_C1W(5, 8);
 #undef PPO_C1W
-        return sum_partials(m->c1_part, blocks, C1 * KS * KS, dW, C1, db, st);
+        sums.add(m->c1_part, blocks, C1 * KS * KS, dW, C1, db);
+        return PPO_OK;
     }
     const int cpt = KS <= 3 ? 8 : (KS == 5 ? 4 : 2);
     const int lpp = C1 / cpt;
@@ -1401,7 +1428,8 @@ static int conv1_wgrad(ppo_model *m, const ppo_minibatch *mb, int row0, int rows
     else if (KS == 5) PPO_CONV1W(5, 4, 1);
     else PPO_CONV1W(7, 2, 1);
 #undef PPO_CONV1W
-    return sum_partials(m->c1_part, blocks, C1 * KS * KS, dW, C1, db, st);
+    sums.add(m->c1_part, blocks, C1 * KS * KS, dW, C1, db);
+    return PPO_OK;
 }
 
 extern "C" int ppo_encoder_bwd(ppo_model *m, const ppo_minibatch *mb, int row0, int rows, const float *dmean,
@@ -1488,7 +1516,9 @@ extern "C" int ppo_encoder_bwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
                                                            m->hw[0]));
     }
     // With layer normalisation dact[l] arrives as the gradient of the normalised, scaled and shifted value; ln_bwd
-    // turns it in place into the gradient of the convolution's output and adds the gamma and beta gradients.
+    // turns it in place into the gradient of the convolution's output and leaves partial sums of the gamma and beta gradients.
+    SumJobs sums;
+    sums.n = 0;
     auto ln_bwd = [&](int l) -> int {
         if (!d.norm) return PPO_OK;
         const int C = m->Cs[l], tc = m->ti_conv[l];
@@ -1498,10 +1528,12 @@ extern "C" int ppo_encoder_bwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
         int blocks = ppo_cdiv(M, (long long)8 * (32 / lpp) * 4);
         const int cap = ppo_num_sms() * 4;
         blocks = blocks > cap ? cap : (blocks < 1 ? 1 : blocks);
+        float *part = m->ln_part + (size_t)(l - 1) * m->ln_cap;
         if ((size_t)blocks * 2 * C > m->ln_cap) return PPO_ERR_SHAPE;
         PPO_TRY(ppo_launch(ln_bwd_kernel, dim3(blocks), dim3(256), 0, st, m->dact[l], m->xhat[l], m->rstd[l], m->master + m->tensors[tc + 2].off, M, C,
-                                              m->ln_part));
-        return sum_partials(m->ln_part, blocks, C, m->grad + m->tensors[tc + 2].off, C, m->grad + m->tensors[tc + 3].off, st);
+                                              part));
+        sums.add(part, blocks, C, m->grad + m->tensors[tc + 2].off, C, m->grad + m->tensors[tc + 3].off);
+        return PPO_OK;
     };
     // The chain of dgrads first; then the wgrads of the GEMM layers one after the other on the caller's stream
     // with conv1's wgrad beside them on the second one.  A wgrad GEMM takes most of an SM's shared memory but
@@ -1526,9 +1558,12 @@ extern "C" int ppo_encoder_bwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
     }
     if (fork && L >= 2) {
         int s = fork_here();  // dZ1 is ready
-        if (s == PPO_OK) s = conv1_wgrad(m, mb, row0, rows, leaf);
+        if (s == PPO_OK) s = conv1_wgrad(m, mb, row0, rows, sums, leaf);
+        if (s == PPO_OK) s = sum_partials_jobs(sums, leaf);
         if (s == PPO_OK) s = run_conv_wgrads(m, rows, st);
         return join(s);
     }
-    return join(conv1_wgrad(m, mb, row0, rows, st));
+    int s = conv1_wgrad(m, mb, row0, rows, sums, st);
+    if (s == PPO_OK) s = sum_partials_jobs(sums, st);
+    return join(s);
 }

@@ -668,6 +668,7 @@ struct WArgs {
     int Kfwd, Co;
     int tiles_per_split, nmma, stages;
     float *part;                    // partial tiles [split][column tile][row tile][BN][128] fp32
+    float *dW;                      // not split: the tile is added to dW right away (else null)
     // Bias gradient db[co] += sum over pixels of dY, or null.  The last column tile has an A block that no tap
     // fills; its first column is set to ones, so row ones_blk * CB of that tile's accumulator is the column
     // sum of dY: the pass over dY that a separate reduction kernel would make comes for free.
@@ -811,7 +812,8 @@ __global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_con
         if (!ok && lane == 0) drain_copies(pipe->full, kb, S, pw, NP);
         __syncwarp();
         // ---------------- epilogue: TMEM lane p is row p of this CTA's 128 x BN tile of dW^T; the whole tile goes
-        // to the CTA's slot of the scratch array, column by column (a warp's store covers 32 consecutive rows)
+        // to the CTA's slot of the scratch array, column by column (a warp's store covers 32 consecutive rows).  The only split
+        // of a reduction adds it to dW itself, the same sum without the trip (1024 x 4096 weights: a reduction of 25 us less).
         const int lg = warp & 3;
         const int p = lg * 32 + lane;
         if (nkb > 0 && ok && mbar_wait(&pipe->tfull, 0, abort_flag, a.status)) {
@@ -821,6 +823,17 @@ __global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_con
             for (int c0 = 0; c0 < BN; c0 += 16) {
                 float v[16];
                 tmem_ld16(lane_base + (uint32_t)c0, v);
+                if (a.dW) {
+                    const int jj = (int)blockIdx.x * 128 + p;
+                    float *d = a.dW + (size_t)(co0 + c0) * a.Kfwd + jj;
+                    float o[16];
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) o[i] = jj < a.Kfwd && co0 + c0 + i < a.Co ? d[(size_t)i * a.Kfwd] : 0.f;
+#pragma unroll
+                    for (int i = 0; i < 16; ++i)
+                        if (jj < a.Kfwd && co0 + c0 + i < a.Co) d[(size_t)i * a.Kfwd] = o[i] + v[i];
+                    continue;
+                }
 #pragma unroll
                 for (int i = 0; i < 16; ++i) tile[(c0 + i) * 128 + p] = v[i];
             }
@@ -1485,7 +1498,9 @@ int tma_gemm_wgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *X, fl
     a.tiles_per_split = (a.grid.tiles + splits - 1) / splits;
     splits = (a.grid.tiles + a.tiles_per_split - 1) / a.tiles_per_split;  // every split has at least one pixel tile
     dim3 grid((unsigned)jtiles, (unsigned)ctiles, (unsigned)splits);
+    if (splits == 1 && !db) a.dW = dW;
     PPO_TRY(ppo_launch(tma_wgrad_kernel, dim3(grid), dim3(kThreads), (size_t)a.stages * stage + sizeof(Pipe) + 1024, st, a));
+    if (a.dW) return PPO_OK;
     return wgrad_reduce(part, jtiles, ctiles, splits, a.BN, a.Kfwd, g.Co, dW, db,
                         db ? (jtiles - 1) * 128 + a.ones_blk * CB : 0, st);
 }

@@ -250,7 +250,7 @@ static size_t carve(ppo_model *m, const ppo_model *shape, int mb, char *base) {
             int cmax = 0;
             for (int l = 1; l <= shape->L; ++l) cmax = shape->Cs[l] > cmax ? shape->Cs[l] : cmax;
             const size_t lc = (size_t)4 * sms * 2 * cmax;
-            char *lp2 = take(lc * sizeof(float));
+            char *lp2 = take((size_t)shape->L * lc * sizeof(float));
             if (m) { m->ln_part = (float *)lp2; m->ln_cap = lc; }
         }
     }
