@@ -81,7 +81,7 @@ int wgrad_batch(F gemms, cudaStream_t st) {
     return wgrad_batch_of([](void *f) -> int { return (*static_cast<F *>(f))(); }, &gemms, st);
 }
 int wgrad_reduce(const float *part, int jtiles, int ctiles, int splits, int BN, int Kfwd, int Co, float *dW, float *db,
-                 int ones_row, cudaStream_t st);
+                 int ones_row, cudaStream_t st, int pair_ci = 0);
 
 // bits[m][c / 32] bit gate_bit_of_channel(c) = act[m][c] > 0, for C a multiple of 32; half words (gate_half) for C = 16.
 int relu_bits(const bf16 *act, uint32_t *bits, long long M, int C, cudaStream_t st);

@@ -662,7 +662,8 @@ struct WArgs {
                                     // without one are 10 to 20 % slower)
     CUtensorMap mapB[kMaxHeights];  // boxes of dY over the same pixels
     RowGrid grid;                   // output pixels
-    int s_mul, pad, ksz, ntaps;
+    int s_mul, pad, ntaps;          // source row of box kh: y * s_mul - pad + kh
+    int x_mul, x_pad, ksz;          // source column of box kw: x * x_mul - x_pad + kw, kw < ksz
     int CB, rbA, mblocks, kchunks;  // A: channels per box, row bytes, boxes per 128 columns, boxes per tap
     int CBn, rbB, nblocks, BN;      // B: likewise over the output channels of this tile
     int Kfwd, Co;
@@ -788,7 +789,7 @@ __global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_con
             while (row < a.grid.R) {
                 const int seg = min(a.grid.Hr - y, a.grid.R - row);
                 const uint32_t off = (uint32_t)(row * a.grid.Wt);
-                const int cx = x0 * a.s_mul - a.pad, cy = y * a.s_mul - a.pad;
+                const int cx = x0 * a.x_mul - a.x_pad, cy = y * a.s_mul - a.pad;
                 int kc = kc0, kh = kh0, kw = kw0;
                 for (int i = 0; sideA && i < nvalid; ++i) {
                     if (elect_one())
@@ -855,6 +856,7 @@ struct ReduceJob {
     const float *part;
     float *dW, *db;
     int jtiles, ctiles, splits, BN, Kfwd, Co, ones_row;
+    int pair_ci;    // > 0: rows of dW^T stand for pairs of pixels of this many channels (see tma_gemm_wgrad)
     int per_block;  // results per block: 128, or 32 (a warp each on more SMs) where they are few
     unsigned block_end;
 };
@@ -912,6 +914,10 @@ __global__ void __launch_bounds__(128) wgrad_reduce_kernel(const __grid_constant
         co = (int)(idx / (uint32_t)Kfwd);
         jj = (int)(idx - (uint32_t)co * (uint32_t)Kfwd);
         dst = q.dW + idx;
+        if (q.pair_ci) {  // three taps of a window row lie in four pixels, the first of which is not used
+            const int kh = jj / (3 * q.pair_ci);
+            jj += (kh + 1) * q.pair_ci;
+        }
     } else if (q.db != nullptr && idx < nW + Co) {
         co = (int)(idx - nW);
         jj = q.ones_row;
@@ -996,15 +1002,15 @@ bool make_grid(RowGrid &g, int Wr, int Hr, int Nimg, int row_bytes_min) {
 }
 
 // Maps of an activation tensor [Nimg][Hs][Ws][C, row stride ld] for boxes of CB channels, the tile width of
-// `g` and heights 1 .. min(R, Hr) rows, traversal stride es along W and H.
+// `g` and heights 1 .. min(R, Hr) rows, traversal strides ex along W and ey along H.
 int make_act_maps(CUtensorMap *maps, const bf16 *base, int C, long long ld, int Ws, int Hs, int Nimg,
-                  const RowGrid &g, int CB, int es) {
+                  const RowGrid &g, int CB, int ex, int ey) {
     const long long dims[4] = {C, Ws, Hs, Nimg};
-    const int wbox = g.Wt * es;
+    const int wbox = g.Wt * ex;
     const int maxh = g.R < g.Hr ? g.R : g.Hr;
     for (int i = 0; i < maxh; ++i) {
-        const int box[4] = {CB, wbox, (i + 1) * es, 1};
-        const int estr[4] = {1, es, es, 1};
+        const int box[4] = {CB, wbox, (i + 1) * ey, 1};
+        const int estr[4] = {1, ex, ey, 1};
         const int s = make_map(&maps[i], base, 4, dims, ld, box, estr, CB * 2);
         if (s != PPO_OK) return s;
     }
@@ -1167,8 +1173,8 @@ int tma_gemm_fwd(const ConvGeom &g, const bf16 *X, const bf16 *W, const FwdEpilo
     // a fully connected layer is one image with a single row of B pixels
     const bool ok = flat ? make_flat_grid(a.grid, g.B, (a.N + a.BN - 1) / a.BN) : make_grid(a.grid, g.Wo, g.Ho, g.B, a.row_bytes);
     if (!ok) return PPO_ERR_UNSUPPORTED;
-    int s = flat ? make_act_maps(a.mapA, X, g.Ci, g.Ci, g.B, 1, 1, a.grid, CB, 1)
-                 : make_act_maps(a.mapA, X, g.Ci, g.Ci, g.Wi, g.Hi, g.B, a.grid, CB, 2);
+    int s = flat ? make_act_maps(a.mapA, X, g.Ci, g.Ci, g.B, 1, 1, a.grid, CB, 1, 1)
+                 : make_act_maps(a.mapA, X, g.Ci, g.Ci, g.Wi, g.Hi, g.B, a.grid, CB, 2, 2);
     if (s != PPO_OK) return s;
     {
         const long long dims[2] = {g.K(), g.Co};
@@ -1250,8 +1256,8 @@ int tma_gemm_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, i
     if (!(flat && e.ksplit <= 1 ? make_flat_grid(a.grid, g.B, (g.Ci + flat_n - 1) / flat_n)
                                 : make_grid(a.grid, Wr, Hr, flat ? 1 : g.B, a.row_bytes)))
         return PPO_ERR_UNSUPPORTED;
-    int s = flat ? make_act_maps(a.mapA, dY, head ? 16 : g.Co, ldy, g.B, 1, 1, a.grid, CB, 1)
-                 : make_act_maps(a.mapA, dY, g.Co, ldy, g.Wo, g.Ho, g.B, a.grid, CB, 1);
+    int s = flat ? make_act_maps(a.mapA, dY, head ? 16 : g.Co, ldy, g.B, 1, 1, a.grid, CB, 1, 1)
+                 : make_act_maps(a.mapA, dY, g.Co, ldy, g.Wo, g.Ho, g.B, a.grid, CB, 1, 1);
     if (s != PPO_OK) return s;
     a.s_mul = 1;
     a.s_oy = a.s_ox = 0;
@@ -1406,7 +1412,7 @@ static int launch_reductions(const ReduceJobs &jobs, cudaStream_t st) {
 }
 
 int wgrad_reduce(const float *part, int jtiles, int ctiles, int splits, int BN, int Kfwd, int Co, float *dW, float *db,
-                 int ones_row, cudaStream_t st) {
+                 int ones_row, cudaStream_t st, int pair_ci) {
     const long long n = (long long)Co * Kfwd + (db ? Co : 0);
     if (n > 0xffffff00ll) return PPO_ERR_UNSUPPORTED;  // 16 GB of weights in one layer
     ReduceJobs one;
@@ -1417,7 +1423,7 @@ int wgrad_reduce(const float *part, int jtiles, int ctiles, int splits, int BN, 
         jobs.n = 0;
     }
     ReduceJob &q = jobs.j[jobs.n];
-    q = {part, dW, db, jtiles, ctiles, splits, BN, Kfwd, Co, ones_row, n < 128 * ppo_num_sms() ? 32 : 128, 0u};
+    q = {part, dW, db, jtiles, ctiles, splits, BN, Kfwd, Co, ones_row, pair_ci, n < 128 * ppo_num_sms() ? 32 : 128, 0u};
     q.block_end = (jobs.n ? jobs.j[jobs.n - 1].block_end : 0u) + (unsigned)((n + q.per_block - 1) / q.per_block);
     ++jobs.n;
     return reduce_batch ? PPO_OK : launch_reductions(jobs, st);
@@ -1439,29 +1445,37 @@ int tma_gemm_wgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *X, fl
     const int CB = channels_per_box(g.Ci, flat);
     const int CBn = g.Co % 64 == 0 ? 64 : (g.Co % 32 == 0 ? 32 : 0);
     if (CB == 0 || CBn == 0) return PPO_ERR_UNSUPPORTED;
+    // 3x3 layers of 16 channels: the copy engine takes a row of a box at a time, and 32-byte rows are a quarter of a line.  Pixels
+    // 2u and 2u + 1 lie side by side, so a window row is two boxes of pixel pairs, u - 1 and u, instead of three of pixels: half
+    // as many rows for it of twice the bytes, a quarter of which (pixel 2u - 2) nobody uses.  The tiles, and with them every
+    // sum, stay those of the single pixels.
+    const bool pair = !flat && g.Ci == 16 && g.k == 3 && g.pad == 1 && g.Wi % 2 == 0;
     WArgs a = {};
-    a.CB = CB;
-    a.rbA = CB * 2;
-    a.mblocks = 128 / CB;
-    a.kchunks = (g.Ci + CB - 1) / CB;
+    a.CB = pair ? 2 * CB : CB;
+    a.rbA = a.CB * 2;
+    a.mblocks = 128 / a.CB;
+    a.kchunks = pair ? 1 : (g.Ci + CB - 1) / CB;
     a.CBn = CBn;
     a.rbB = CBn * 2;
     a.BN = g.Co < 256 ? g.Co : 256;
     if (g.Co % a.BN != 0 || a.BN % CBn != 0) return PPO_ERR_UNSUPPORTED;
     a.nblocks = a.BN / CBn;
-    const int rb_min = a.rbA < a.rbB ? a.rbA : a.rbB;
+    const int rb_min = 2 * CB < a.rbB ? 2 * CB : a.rbB;
     const bool ok = flat ? make_grid(a.grid, g.B, 1, 1, rb_min) : make_grid(a.grid, g.Wo, g.Ho, g.B, rb_min);
     if (!ok) return PPO_ERR_UNSUPPORTED;
-    int s = flat ? make_act_maps(a.mapA, X, g.Ci, g.Ci, g.B, 1, 1, a.grid, CB, 1)
-                 : make_act_maps(a.mapA, X, g.Ci, g.Ci, g.Wi, g.Hi, g.B, a.grid, CB, 2);
+    int s = flat ? make_act_maps(a.mapA, X, g.Ci, g.Ci, g.B, 1, 1, a.grid, CB, 1, 1)
+            : pair ? make_act_maps(a.mapA, X, 2 * g.Ci, 2 * g.Ci, g.Wi / 2, g.Hi, g.B, a.grid, a.CB, 1, 2)
+                   : make_act_maps(a.mapA, X, g.Ci, g.Ci, g.Wi, g.Hi, g.B, a.grid, CB, 2, 2);
     if (s != PPO_OK) return s;
-    s = flat ? make_act_maps(a.mapB, dY, g.Co, ldy, g.B, 1, 1, a.grid, CBn, 1)
-             : make_act_maps(a.mapB, dY, g.Co, ldy, g.Wo, g.Ho, g.B, a.grid, CBn, 1);
+    s = flat ? make_act_maps(a.mapB, dY, g.Co, ldy, g.B, 1, 1, a.grid, CBn, 1, 1)
+             : make_act_maps(a.mapB, dY, g.Co, ldy, g.Wo, g.Ho, g.B, a.grid, CBn, 1, 1);
     if (s != PPO_OK) return s;
     a.s_mul = flat ? 1 : 2;
     a.pad = g.pad;
-    a.ksz = g.k;
-    a.ntaps = g.taps();
+    a.x_mul = flat || pair ? 1 : 2;
+    a.x_pad = g.pad;
+    a.ksz = pair ? 2 : g.k;
+    a.ntaps = pair ? 6 : g.taps();
     a.Kfwd = g.K();
     a.Co = g.Co;
     a.nmma = (a.grid.arows + 15) / 16;
@@ -1498,11 +1512,11 @@ int tma_gemm_wgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *X, fl
     a.tiles_per_split = (a.grid.tiles + splits - 1) / splits;
     splits = (a.grid.tiles + a.tiles_per_split - 1) / a.tiles_per_split;  // every split has at least one pixel tile
     dim3 grid((unsigned)jtiles, (unsigned)ctiles, (unsigned)splits);
-    if (splits == 1 && !db) a.dW = dW;
+    if (splits == 1 && !db && !pair) a.dW = dW;
     PPO_TRY(ppo_launch(tma_wgrad_kernel, dim3(grid), dim3(kThreads), (size_t)a.stages * stage + sizeof(Pipe) + 1024, st, a));
     if (a.dW) return PPO_OK;
     return wgrad_reduce(part, jtiles, ctiles, splits, a.BN, a.Kfwd, g.Co, dW, db,
-                        db ? (jtiles - 1) * 128 + a.ones_blk * CB : 0, st);
+                        db ? (jtiles - 1) * 128 + a.ones_blk * a.CB : 0, st, pair ? g.Ci : 0);
 }
 
 // Scratch floats that let a weight-gradient GEMM of this shape split as far as it wants: every CTA of a grid of up

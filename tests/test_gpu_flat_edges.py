@@ -52,3 +52,12 @@ def test_last_gate_is_open_for_positive_activations_only(name):
     assert torch.isfinite(want).all() and float(want.norm()) > 0
     for pattern in (0x8000, 0xBF80, 0xFF80, 0x7FC0, 0xFFC0):  # -0, -1, -inf, NaN, -NaN
         assert torch.equal(gradients(pattern), want), hex(pattern)
+
+
+# weight gradient of a 16-channel layer in pairs of pixels: even widths (one pair, a tile that ends inside a row, several tiles per
+# row), odd heights, one image and many; an odd width goes pixel by pixel
+@pytest.mark.parametrize("H,W,N,last", [(8, 4, 2, 32), (9, 12, 6, 64), (35, 44, 6, 32), (10, 532, 2, 96), (35, 46, 6, 32)])
+def test_pairs_of_pixels_match_oracle(H, W, N, last, monkeypatch):
+    w = synth.Workload("pairs", N, 2, H, W, (16, last), (3, 3), (40,), 1, 2, P=16, A=3)
+    monkeypatch.setitem(NETS, "pairs", w)
+    conv_stack_matches_oracle("pairs", monkeypatch)
