@@ -178,6 +178,10 @@ __device__ __forceinline__ uint32_t gate_bits_add(uint32_t gate, uint32_t pair, 
 __device__ __forceinline__ uint16_t gate_half(uint32_t gate) { return (uint16_t)((gate & 0xFFu) | ((gate >> 8) & 0xFF00u)); }
 // Two of them as one word, the pairs of the first pixel in front: pair j owns bits j and 16 + j.
 __device__ __forceinline__ uint32_t gate_of_halves(uint32_t first, uint32_t second) { return __byte_perm(first, second, 0x5140); }
+// All ones over each half of a bf16 pair that is > 0.
+__device__ __forceinline__ uint32_t gate_open(uint32_t pair) {
+    return __hgt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&pair), __float2bfloat162_rn(0.f));
+}
 __device__ __forceinline__ uint32_t gate_pair_mask(uint32_t gate, int j) {
     return ((gate >> j) & 0x00010001u) * 0xFFFFu;
 }

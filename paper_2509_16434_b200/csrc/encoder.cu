@@ -953,7 +953,7 @@ static int recorded(ppo_model *m, const PlanKey &key, cudaStream_t st, F &&make)
     return s;
 }
 
-enum { OP_FWD = 1, OP_DGRAD, OP_WGRAD, OP_CONV_WGRADS, OP_LSTM_FWD, OP_LSTM_BWD };
+enum { OP_FWD = 1, OP_DGRAD, OP_WGRAD, OP_CONV_WGRADS, OP_LSTM_FWD, OP_LSTM_BWD, OP_MLP_FWD, OP_MLP_BWD };
 
 static PlanKey plan_key(int op, const ConvGeom &g) {
     PlanKey k;
@@ -1297,6 +1297,23 @@ extern "C" int ppo_encoder_fwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
     }
     if (d.n_lstm > 0) PPO_TRY(lstm_forward(m, rows, st));
     int ti = m->ti_fc[1];
+    MlpLayer mlp[PPO_MAX_FC + 1] = {};
+    for (int l = 1; l <= m->F + 1; ++l) {
+        const int tl = m->ti_fc[l], K = fc_input_width(m, l);
+        const float *bias = m->master + m->tensors[tl + 1].off;
+        if (l <= m->F) mlp[l - 1] = {fc_input(m, l), K, K, m->shadow + m->tensors[tl].off, K, m->hw[l], MLP_RELU, bias, m->h[l], nullptr, nullptr, m->hw[l]};
+        else mlp[l - 1] = {fc_input(m, l), K, K, m->shadow + m->tensors[tl].off, K, d.A + 1, MLP_HEAD, bias, nullptr, nullptr, nullptr, 0};
+    }
+    if (mlp_covers(mlp, m->F + 1, rows)) {
+        PlanKey k = plan_key(OP_MLP_FWD, fc_geom(rows, 0, 0));
+        const void *p[] = {mlp[0].X, mean, value};
+        memcpy(k.p, p, sizeof(p));
+        PPO_TRY(recorded(m, k, st, [&]() -> int { return mlp_chain(mlp, m->F + 1, rows, {d.A, mean, value}, ppo_device_status_ptr(), st); }));
+        m->fwd_valid = true;
+        m->last_row0 = row0;
+        m->last_rows = rows;
+        return PPO_OK;
+    }
     for (int l = 1; l <= m->F; ++l, ti += 2) {
         ConvGeom g = fc_geom(rows, fc_input_width(m, l), m->hw[l]);
         FwdEpilogue e = {m->master + m->tensors[ti + 1].off, 1, m->h[l], nullptr, nullptr, 0};
@@ -1447,7 +1464,23 @@ extern "C" int ppo_encoder_bwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
     }
     PPO_TRY(refresh_transposed(m, st));
 
-    PPO_TRY(ppo_launch(pack_dout_kernel, dim3(ppo_cdiv((long long)rows * 16, 256)), dim3(256), 0, st, dmean, dvalue, m->dh[F + 1], rows, d.A));
+    // The input gradients of the head and the hidden layers, last to first.
+    MlpLayer mlp[PPO_MAX_FC + 1] = {};
+    for (int l = F + 1, i = 0; l >= 1; --l, ++i) {
+        const int Co = l <= F ? m->hw[l] : d.A + 1, Ci = fc_input_width(m, l);
+        const bf16 *Wt = m->wT + m->wT_off[m->ti_fc[l]];
+        if (l > 1) mlp[i] = {m->dh[l], l <= F ? Co : 16, Co, Wt, wt_ld_of(Co), Ci, MLP_GATED, nullptr, m->dh[l - 1], nullptr, m->h[l - 1], Ci};
+        else mlp[i] = {m->dh[l], l <= F ? Co : 16, Co, Wt, wt_ld_of(Co), Ci, MLP_F32, nullptr, nullptr, d.n_lstm > 0 ? m->lstm_dtop : m->dh0_f32, nullptr, Ci};
+    }
+    const bool chained = mlp_covers(mlp, F + 1, rows);
+    if (chained) {
+        PlanKey k = plan_key(OP_MLP_BWD, fc_geom(rows, 0, 0));
+        const void *p[] = {dmean, dvalue, mlp[F].out_f32};
+        memcpy(k.p, p, sizeof(p));
+        PPO_TRY(recorded(m, k, st, [&]() -> int {
+            return mlp_chain(mlp, F + 1, rows, {d.A, nullptr, nullptr, dmean, dvalue, m->dh[F + 1]}, ppo_device_status_ptr(), st);
+        }));
+    } else PPO_TRY(ppo_launch(pack_dout_kernel, dim3(ppo_cdiv((long long)rows * 16, 256)), dim3(256), 0, st, dmean, dvalue, m->dh[F + 1], rows, d.A));
     // Weight and bias gradients are leaves of the dependency graph: only the chain of dgrads has to run in order.
     // The leaves of the FC layers (small kernels on a fraction of the SMs) and, further down, conv1's wgrad go to
     // a second stream that forks from the caller's stream whenever the gradient they read is ready and joins it
@@ -1477,6 +1510,7 @@ extern "C" int ppo_encoder_bwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
         const bf16 *dY = m->dh[l];
         int s = run_wgrad(m, ti, g, dY, ldy, fc_input(m, l), leaf);
         if (s != PPO_OK) return join(s);
+        if (chained) continue;
         DgradEpilogue e;
         if (l > 1) e = {m->h[l - 1], m->dh[l - 1], nullptr};
         else e = {nullptr, nullptr, d.n_lstm > 0 ? m->lstm_dtop : m->dh0_f32};

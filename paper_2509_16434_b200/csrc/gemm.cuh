@@ -86,6 +86,32 @@ int wgrad_reduce(const float *part, int jtiles, int ctiles, int splits, int BN, 
 // bits[m][c / 32] bit gate_bit_of_channel(c) = act[m][c] > 0, for C a multiple of 32; half words (gate_half) for C = 16.
 int relu_bits(const bf16 *act, uint32_t *bits, long long M, int C, cudaStream_t st);
 
+// A chain of fully connected layers in one launch (mlp.cu).  Layer i reads X [rows][K] (row stride ldx; what layer i - 1 wrote),
+// weights W [N][K] (row stride ldw, zeros between K and ldw), and writes, by its mode: out = relu(X W^T + bias) as bf16; the
+// head's mean and value; X W^T as bf16 where the gate `mask` is > 0 (the row stride of out and mask is ldo); X W^T as fp32.
+constexpr int kMlpLayers = 5;
+enum { MLP_RELU = 0, MLP_HEAD = 1, MLP_GATED = 2, MLP_F32 = 3 };
+struct MlpLayer {
+    const bf16 *X;
+    int ldx, K;
+    const bf16 *W;
+    int ldw, N, mode;
+    const float *bias;
+    bf16 *out;
+    float *out_f32;
+    const bf16 *mask;
+    int ldo;
+};
+// mean, value: outputs of a head.  dout [rows][16] (null: none) receives dmean and dvalue as bf16 before the first layer reads it.
+struct MlpEnds {
+    int A;
+    float *mean, *value;
+    const float *dmean, *dvalue;
+    bf16 *dout;
+};
+bool mlp_covers(const MlpLayer *layers, int nl, int rows);
+int mlp_chain(const MlpLayer *layers, int nl, int rows, const MlpEnds &ends, int32_t *status, cudaStream_t st);
+
 // First convolution (C_in = 1) as a tensor-core GEMM over thread-built im2col tiles (conv1_tc.cu).
 // ln_* as in FwdEpilogue (all null: no normalisation); with them C1 must be 16 or 32.
 int conv1_tc_fwd(const __half *depth, const bf16 *W, const float *bias, bf16 *out, uint32_t *bits, int rows, int Hi,

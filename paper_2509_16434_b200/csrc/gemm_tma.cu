@@ -200,11 +200,6 @@ struct PipeK {
     // followed by the epilogue staging: per epilogue warp 32 rows x 32 bf16 columns (2 KB), 16-byte pieces swizzled
 };
 
-// All ones over each half of a bf16 pair that is > 0.
-__device__ __forceinline__ uint32_t gate_open(uint32_t pair) {
-    return __hgt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&pair), __float2bfloat162_rn(0.f));
-}
-
 // A kernel each for forward passes, input gradients and input gradients whose gate is the bf16 activation: in one, the
 // registers of the widest epilogue would spill the others'.
 enum { KIND_FWD = 0, KIND_DGRAD = 1, KIND_DGRAD_ACT = 2 };

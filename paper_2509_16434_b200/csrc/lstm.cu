@@ -70,10 +70,6 @@ __device__ __forceinline__ bool cell_all(bool ok) {
         : "memory");
     return r != 0;
 }
-// Between the acquire that saw other threads' plain writes to global memory and the copy that reads them through the async
-// proxy (20 cycles; the fence over all state spaces takes 900).
-__device__ __forceinline__ void fence_proxy_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
-
 // Counters of a tile of envs, a row of 32 for each exchange.  Word k of the first: CTAs that have published their 16 units of
 // chunk k of the reduction (64 units, four CTAs a step); of the second (backward): slabs that have published their partial
 // products of units 64 k .. 64 k + 63.  A reader waits for the four writers of what it reads next instead of for all the tile's
@@ -167,12 +163,6 @@ __device__ __forceinline__ void xch_put(uint32_t base, uint32_t tmem, int lg, in
                      "f"(v[4 * j + 1]), "f"(v[4 * j + 2]), "f"(v[4 * j + 3])
                      : "memory");
 }
-// Shared memory of CTA `rank` of the cluster at the place of this CTA's `addr`.
-__device__ __forceinline__ uint32_t in_cta(uint32_t addr, uint32_t rank) {
-    uint32_t r;
-    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-    return r;
-}
 // Place of 16 bytes (piece 0 .. 3) of row `row` in slab `slab` of the partial products a CTA receives, [4][4 pieces][envs]: a
 // warp that sends a piece of 32 rows fills 512 bytes on end, and four pieces of a row on neighbouring lanes do not meet a
 // bank twice on the way out.
@@ -185,30 +175,6 @@ __device__ __forceinline__ void send16(uint32_t dst, uint32_t bar, const float *
     asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(dst), "f"(v[0]),
                  "f"(v[1]), "f"(v[2]), "f"(v[3]), "r"(bar)
                  : "memory");
-}
-// Bounded wait for a phase that writes of the whole cluster complete.
-__device__ __forceinline__ bool cluster_mbar_wait(uint64_t *bar, uint32_t parity, volatile int *abort_flag, int32_t *status) {
-    const long long t0 = clock64();
-    while (true) {
-        uint32_t done;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(done)
-            : "r"(smem_u32(bar)), "r"(parity)
-            : "memory");
-        if (done) return true;
-        if (*abort_flag) return false;
-        if (clock64() - t0 > kWaitCycles) {
-            *abort_flag = 1;
-            ppo_report(status, PPO_ERR_TIMEOUT);
-            return false;
-        }
-    }
-}
-__device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 // Everything the two kernels share around the cell: barriers, tensor memory, the resident weight slice, the stream of A
 // chunks and the MMAs.

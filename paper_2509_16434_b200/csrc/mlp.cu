@@ -1,0 +1,444 @@
+// The fully connected layers behind the encoder as one launch per direction (sm_100a).
+//
+// Layer by layer they are a chain of kernels of 6 to 12 us that each do a microsecond of work: the rest is launching, filling a
+// pipeline, fetching weights and draining.  Rows do not depend on one another, so a tile of rows goes through all layers in one
+// cluster of 4 or 8 CTAs: a CTA owns a slice of each layer's columns, weights stream into their own ring of stages
+// without waiting for anybody, and between two layers the CTAs of the cluster exchange their columns through L2, a release, an
+// arrival at each other's barriers and an acquire: some 2500 cycles instead of a kernel boundary.
+// Measured (us, separate launches -> here): 16 rows 1024-512-512-256-13 28 -> 14; 1024 rows 96-256-13 15 -> 9; 4096 rows
+// 288-512-512-13 35 -> 21, and back 37 -> 22.
+// Sums run in the order of the separate kernels (gemm_tma.cu): same bits.
+//
+// Every wait is bounded: on a time-out the kernel records PPO_ERR_TIMEOUT, waits (bounded) for its copies, frees its
+// tensor memory and returns.
+#include "gemm.cuh"
+#include "launch.cuh"
+#include "tcgen05.cuh"
+#include "tma_host.cuh"
+
+namespace {
+
+using namespace tc;
+
+constexpr int kEpiWarps = 8;
+constexpr int kThreads = (4 + kEpiWarps) * 32;  // warp 0: rows, 1: MMA issue and TMEM owner, 2: weights, 3: maps, 4 ..: epilogue
+constexpr int kMaxStages = 16;
+constexpr int kMaxSlice = 256;                  // columns of a layer a CTA can own
+constexpr size_t kSmemMax = 227 * 1024;
+constexpr int kCopy = 16 * 1024;                // bytes of a stage, except for slices of more than 128 columns
+constexpr uint32_t kStage = 4096;               // staging of an epilogue warp: 32 rows x 128 bytes
+
+struct Layer {
+    CUtensorMap mapA, mapB;
+    int chunks, rb;       // of the reduction, and bytes of a row of one
+    int gA, gB;           // chunks a copy brings (a stage holds them): more than one where the reduction is whole chunks
+    int N, n;             // columns; of them in a CTA's slice
+    int mode, ldo;
+    const float *bias;
+    bf16 *out;
+    float *out_f32;
+    const bf16 *mask;
+};
+
+struct Args {
+    Layer l[kMlpLayers];
+    int nl, rows, Mt;          // rows of a tile: 32, 64 or 128
+    int sA, sB;                // stages
+    uint32_t a_slot, b_slot;   // their bytes
+    uint32_t tmem_cols;
+    int A;
+    float *mean, *value;       // head
+    const float *dmean, *dvalue;
+    bf16 *dout;                // gradient of the head's outputs as bf16 [rows][16] (null: forward)
+    int32_t *status;
+};
+
+struct Pipe {
+    uint64_t fullA[kMaxStages], emptyA[kMaxStages], fullB[kMaxStages], emptyB[kMaxStages], tfull, ready;
+    uint32_t tmem_slot;
+    int abort_flag;
+    alignas(16) float bias[kMlpLayers * kMaxSlice];
+};
+
+// Barrier of the epilogue that also ANDs a condition over it (a bounded wait that ran out in one warp ends all).
+__device__ __forceinline__ bool epi_all(bool ok) {
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %1, 0;\n\t"
+        "bar.red.and.pred q, 1, %2, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(r)
+        : "r"(ok ? 1u : 0u), "n"(kEpiWarps * 32)
+        : "memory");
+    return r != 0;
+}
+
+__device__ __forceinline__ void drain(uint64_t *full, int it, int S) {
+    for (int i = max(0, it - S); i < it; ++i) {
+        const long long t0 = clock64();
+        while (!mbar_try_wait(&full[i % S], (i / S) & 1))
+            if (clock64() - t0 > kWaitCycles / 4) break;
+    }
+}
+
+template <int CS>
+__device__ __forceinline__ void chain(const Args &a, uint8_t *raw) {
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
+    const uint32_t base = smem_u32(smem), b_base = base + (uint32_t)a.sA * a.a_slot;  // (an MMA's rows behind the last A stage lie in B's)
+    const uint32_t stg_off = (uint32_t)a.sA * a.a_slot + (uint32_t)a.sB * a.b_slot;
+    Pipe *pipe = reinterpret_cast<Pipe *>(smem + stg_off + kEpiWarps * kStage);
+    volatile int *abort_flag = &pipe->abort_flag;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
+    const int rank = (int)blockIdx.x % CS, row0 = (int)blockIdx.x / CS * a.Mt;
+    const int pack = a.dout ? 1 : 0;  // a step before the first layer
+    // copy of `g` chunks from chunk k of rows `row` on
+    auto copy = [](uint32_t dst, const CUtensorMap *map, uint64_t *bar, int g, int rb, int k, int row) {
+        if (g > 1) tma_load_4d(dst, map, bar, 0, row, k, 0);
+        else tma_load_4d(dst, map, bar, k * (rb >> 1), row, 0, 0);
+    };
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < a.sA; ++s) {
+            mbar_init(&pipe->fullA[s], 1);
+            mbar_init(&pipe->emptyA[s], 1);
+        }
+        for (int s = 0; s < a.sB; ++s) {
+            mbar_init(&pipe->fullB[s], 1);
+            mbar_init(&pipe->emptyB[s], 1);
+        }
+        mbar_init(&pipe->tfull, 1);
+        mbar_init(&pipe->ready, CS);
+        pipe->abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) tmem_alloc(&pipe->tmem_slot, a.tmem_cols);
+    if (warp == 3 && lane < 2 * a.nl) {
+        const CUtensorMap *m = lane & 1 ? &a.l[lane >> 1].mapB : &a.l[lane >> 1].mapA;
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(m)) : "memory");
+    }
+    __syncwarp();
+    cluster_sync();  // the barriers exist before anyone arrives at a neighbour's
+    grid_wait();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = pipe->tmem_slot;
+
+    if (warp == 0) {
+        int s = 0, it = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        for (int l = 0; l < a.nl && ok; ++l) {
+            const Layer &y = a.l[l];
+            if (l + pack > 0) {  // what the cluster has left for this layer
+                ok = cluster_mbar_wait(&pipe->ready, (uint32_t)(l + pack - 1) & 1u, abort_flag, a.status);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                fence_proxy_global();
+            }
+            if (rank * y.n >= y.N) continue;
+            for (int k = 0; k < y.chunks; k += y.gA, ++it) {
+                ok = mbar_wait_warp(&pipe->emptyA[s], ph ^ 1u, abort_flag, a.status);
+                if (!ok) break;
+                if (elect_one()) {
+                    mbar_arrive_expect_tx(&pipe->fullA[s], (uint32_t)(y.gA * a.Mt * y.rb));
+                    copy(base + (uint32_t)s * a.a_slot, &y.mapA, &pipe->fullA[s], y.gA, y.rb, k, row0);
+                }
+                __syncwarp();
+                if (++s == a.sA) { s = 0; ph ^= 1u; }
+            }
+        }
+        if (!ok && lane == 0) drain(pipe->fullA, it, a.sA);
+        __syncwarp();
+    } else if (warp == 2) {
+        int s = 0, it = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        for (int l = 0; l < a.nl && ok; ++l) {
+            const Layer &y = a.l[l];
+            if (rank * y.n >= y.N) continue;
+            for (int k = 0; k < y.chunks; k += y.gB, ++it) {
+                ok = mbar_wait_warp(&pipe->emptyB[s], ph ^ 1u, abort_flag, a.status);
+                if (!ok) break;
+                if (elect_one()) {
+                    mbar_arrive_expect_tx(&pipe->fullB[s], (uint32_t)(y.gB * y.n * y.rb));
+                    copy(b_base + (uint32_t)s * a.b_slot, &y.mapB, &pipe->fullB[s], y.gB, y.rb, k, rank * y.n);
+                }
+                __syncwarp();
+                if (++s == a.sB) { s = 0; ph ^= 1u; }
+            }
+        }
+        if (!ok && lane == 0) drain(pipe->fullB, it, a.sB);
+        __syncwarp();
+    } else if (warp == 1) {
+        // the accumulator of the layer before has been read: the rows of this one wait for the cluster's arrivals, this CTA's
+        // epilogue among them
+        int sa = 0, sb = 0;
+        uint32_t pa = 0, pb = 0;
+        bool ok = true;
+        for (int l = 0; l < a.nl && ok; ++l) {
+            const Layer &y = a.l[l];
+            if (rank * y.n >= y.N) continue;
+            const uint32_t idesc = instr_desc(128, y.n, 0, 0), rb = (uint32_t)y.rb;
+            const uint64_t d0 = smem_desc_sw(base, 16, 8u * rb, rb);
+            const uint32_t lo = (uint32_t)d0, hi = (uint32_t)(d0 >> 32), b_lo = lo + ((b_base - base) >> 4);
+            const uint32_t a16 = (uint32_t)(a.Mt * y.rb) >> 4, b16 = (uint32_t)(y.n * y.rb) >> 4;
+            int ia = 0, ib = 0;  // chunk within its stage
+            for (int k = 0; k < y.chunks; ++k) {
+                if (ib == 0) ok = mbar_wait_warp(&pipe->fullB[sb], pb, abort_flag, a.status);
+                if (ok && ia == 0) ok = mbar_wait_warp(&pipe->fullA[sa], pa, abort_flag, a.status);
+                if (!ok) break;
+                tc_fence_after();
+                const bool last = k + 1 == y.chunks, end_a = last || ia + 1 == y.gA, end_b = last || ib + 1 == y.gB;
+                if (elect_one()) {
+                    const uint32_t la = lo + (uint32_t)sa * (a.a_slot >> 4) + (uint32_t)ia * a16;
+                    const uint32_t lb = b_lo + (uint32_t)sb * (a.b_slot >> 4) + (uint32_t)ib * b16;
+                    umma_bf16_lh(tmem, la, hi, lb, hi, idesc, k > 0 ? 1u : 0u);
+                    for (int j = 1; j < (int)(rb >> 5); ++j) umma_bf16_lh(tmem, la + 2 * j, hi, lb + 2 * j, hi, idesc, 1u);
+                    if (end_a) umma_commit(&pipe->emptyA[sa]);
+                    if (end_b) umma_commit(&pipe->emptyB[sb]);
+                }
+                __syncwarp();
+                ++ia;
+                ++ib;
+                if (end_a) {
+                    ia = 0;
+                    if (++sa == a.sA) { sa = 0; pa ^= 1u; }
+                }
+                if (end_b) {
+                    ib = 0;
+                    if (++sb == a.sB) { sb = 0; pb ^= 1u; }
+                }
+            }
+            if (ok && elect_one()) umma_commit(&pipe->tfull);
+            __syncwarp();
+        }
+    } else if (warp >= 4) {
+        const int lg = warp & 3, half = (warp - 4) >> 2, et = (int)threadIdx.x - 128;
+        const int grow = row0 + lg * 32 + lane;  // this thread's row: its tensor-memory lane
+        uint4 *const stg = reinterpret_cast<uint4 *>(smem + stg_off + (uint32_t)(warp - 4) * kStage);
+        const int rr0 = lane >> 2, piece = lane & 3, sw = (lane >> 1) & 3;
+        const bool rows_here = lg * 32 < a.Mt;
+        // Behind this CTA's stores: one release, an arrival at every CTA's barrier.  before: the phase this CTA's part is made
+        // from (-1: none); a CTA without columns has not waited for it, and must not arrive a second time before it is complete.
+        auto publish = [&](bool ok, int before) -> bool {
+            if (before >= 0) ok = cluster_mbar_wait(&pipe->ready, (uint32_t)before & 1u, abort_flag, a.status) && ok;
+            if (!epi_all(ok)) return false;
+            if (warp == 4) {
+                if (lane < CS) arrive_in_cta(&pipe->ready, (uint32_t)lane);
+                __syncwarp();
+            }
+            return true;
+        };
+        {   // biases of all layers (a thread has at most one of each); the first use is behind a barrier
+            float b[kMlpLayers];
+#pragma unroll
+            for (int l = 0; l < kMlpLayers; ++l)
+                b[l] = l < a.nl && a.l[l].bias && et < a.l[l].n && rank * a.l[l].n + et < a.l[l].N ? __ldg(a.l[l].bias + rank * a.l[l].n + et) : 0.f;
+#pragma unroll
+            for (int l = 0; l < kMlpLayers; ++l) pipe->bias[l * kMaxSlice + et] = b[l];
+            epi_all(true);
+        }
+        if (pack) {
+            const int per = a.Mt / CS;
+            for (int i = et; i < per * 16; i += kEpiWarps * 32) {
+                const int r = row0 + rank * per + (i >> 4), j = i & 15;
+                if (r >= a.rows) break;
+                float v = 0.f;
+                if (j < a.A) v = a.dmean[(size_t)r * a.A + j];
+                else if (j == a.A) v = a.dvalue[r];
+                a.dout[(size_t)r * 16 + j] = __float2bfloat16_rn(v);
+            }
+            publish(true, -1);
+        }
+        uint32_t tph = 0;
+        for (int l = 0; l < a.nl; ++l) {
+            const Layer &y = a.l[l];
+            const int col0 = rank * y.n;
+            bool ok = true;
+            if (col0 < y.N && rows_here) {
+                // 16 bytes of the gate for each of this lane's four stores of a group, fetched ahead (see gemm_tma.cu)
+                uint4 gate[4];
+                auto fetch = [&](int g) {
+#pragma unroll
+                    for (int ps = 0; ps < 4; ++ps) {
+                        const int r = row0 + lg * 32 + ps * 8 + rr0, c = col0 + g + piece * 8;
+                        gate[ps] = make_uint4(0, 0, 0, 0);
+                        if (g < y.n && r < a.rows && g + piece * 8 < y.n && c < y.N)
+                            gate[ps] = __ldg(reinterpret_cast<const uint4 *>(y.mask + (size_t)r * y.ldo + c));
+                    }
+                };
+                if (y.mode == MLP_GATED) fetch(half * 32);
+                ok = mbar_wait(&pipe->tfull, tph, abort_flag, a.status);
+                ok = __all_sync(0xffffffffu, ok);
+                tc_fence_after();
+                const uint32_t tm = tmem + ((uint32_t)(lg * 32) << 16);
+#pragma unroll 1
+                for (int g = half * 32; ok && g < y.n; g += 64) {
+                    float v[32];
+                    tmem_ld16(tm + (uint32_t)g, v);
+                    if (g + 16 < y.n) {
+                        tmem_ld16(tm + (uint32_t)g + 16u, v + 16);
+                    } else {
+#pragma unroll
+                        for (int i = 16; i < 32; ++i) v[i] = 0.f;
+                    }
+                    if (y.mode == MLP_HEAD) {
+                        if (grow < a.rows) {
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) {
+                                const int c = col0 + g + i;
+                                if (c < a.A) a.mean[(size_t)grow * a.A + c] = v[i] + pipe->bias[l * kMaxSlice + g + i];
+                                else if (c == a.A) a.value[grow] = v[i] + pipe->bias[l * kMaxSlice + g + i];
+                            }
+                        }
+                        continue;
+                    }
+                    if (y.mode == MLP_F32) {  // 32 rows x 128 bytes, 16-byte pieces swizzled by the row
+#pragma unroll
+                        for (int j = 0; j < 8; ++j)
+                            stg[lane * 8 + (j ^ (lane & 7))] = make_uint4(__float_as_uint(v[4 * j]), __float_as_uint(v[4 * j + 1]),
+                                                                          __float_as_uint(v[4 * j + 2]), __float_as_uint(v[4 * j + 3]));
+                        __syncwarp();
+#pragma unroll
+                        for (int ps = 0; ps < 8; ++ps) {
+                            const int rr = ps * 4 + (lane >> 3), p8 = lane & 7, r = row0 + lg * 32 + rr, c = col0 + g + p8 * 4;
+                            if (r < a.rows && g + p8 * 4 < y.n && c < y.N)
+                                *reinterpret_cast<uint4 *>(y.out_f32 + (size_t)r * y.ldo + c) = stg[rr * 8 + (p8 ^ (rr & 7))];
+                        }
+                        __syncwarp();
+                        continue;
+                    }
+                    uint32_t pk[16];
+                    if (y.mode == MLP_RELU) {
+                        const float *bp = pipe->bias + l * kMaxSlice + g;
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) {
+                            const bool in = j < 8 || g + 16 < y.n;
+                            pk[j] = relu_pack_bf16x2(v[2 * j] + (in ? bp[2 * j] : 0.f), v[2 * j + 1] + (in ? bp[2 * j + 1] : 0.f));
+                        }
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) pk[j] = pack_bf16x2(v[2 * j], v[2 * j + 1]);
+                    }
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) stg[lane * 4 + (j ^ sw)] = make_uint4(pk[4 * j], pk[4 * j + 1], pk[4 * j + 2], pk[4 * j + 3]);
+                    __syncwarp();
+#pragma unroll
+                    for (int ps = 0; ps < 4; ++ps) {
+                        const int rr = ps * 8 + rr0, r = row0 + lg * 32 + rr, c = col0 + g + piece * 8;
+                        if (r < a.rows && g + piece * 8 < y.n && c < y.N) {
+                            uint4 o = stg[rr * 4 + (piece ^ ((rr >> 1) & 3))];
+                            if (y.mode == MLP_GATED) {
+                                o.x &= gate_open(gate[ps].x); o.y &= gate_open(gate[ps].y);
+                                o.z &= gate_open(gate[ps].z); o.w &= gate_open(gate[ps].w);
+                            }
+                            *reinterpret_cast<uint4 *>(y.out + (size_t)r * y.ldo + c) = o;
+                        }
+                    }
+                    if (y.mode == MLP_GATED) fetch(g + 64);
+                    __syncwarp();
+                }
+                tc_fence_before();
+            }
+            if (col0 < y.N) tph ^= 1u;
+            if (l + 1 < a.nl && !publish(ok, l + pack - 1)) break;
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync();  // no CTA leaves while a neighbour may arrive at its barriers
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem, a.tmem_cols);
+    }
+}
+
+__global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(kThreads, 1) mlp_chain4_kernel(const __grid_constant__ Args a) {
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    chain<4>(a, smem_raw);
+}
+__global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(kThreads, 1) mlp_chain8_kernel(const __grid_constant__ Args a) {
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    chain<8>(a, smem_raw);
+}
+
+// CTAs per cluster and rows per tile, or false.  Clusters of eight cut the columns finer, but only 15 of them are resident on 148
+// SMs (33 of four); a second wave would cost as much as it saves.  Below that the smallest tile that still leaves one wave.
+bool shape(int rows, int &cs, int &Mt) {
+    cs = 8;
+    for (Mt = 32; Mt <= 128; Mt *= 2)
+        if ((rows + Mt - 1) / Mt <= 15) return true;
+    cs = 4;
+    Mt = 128;
+    return (rows + 127) / 128 <= 33;
+}
+
+}  // namespace
+
+bool mlp_covers(const MlpLayer *layers, int nl, int rows) {
+    int cs, Mt;
+    if (nl < 1 || nl > kMlpLayers || rows < 1 || !shape(rows, cs, Mt)) return false;
+    for (int i = 0; i < nl; ++i) {
+        const MlpLayer &y = layers[i];
+        const bool narrow = y.ldx == 16 && y.K <= 16;
+        if (!narrow && (y.K < 64 || y.K % 8 != 0 || y.ldx % 8 != 0)) return false;
+        if (y.ldw % 8 != 0 || (y.mode == MLP_HEAD ? y.N > 16 : y.N % 8 != 0)) return false;
+        if ((y.N + cs - 1) / cs > kMaxSlice - 15) return false;
+    }
+    return true;
+}
+
+int mlp_chain(const MlpLayer *layers, int nl, int rows, const MlpEnds &ends, int32_t *status, cudaStream_t st) {
+    if (!status || !mlp_covers(layers, nl, rows)) return PPO_ERR_UNSUPPORTED;
+    Args a = {};
+    int cs;
+    shape(rows, cs, a.Mt);
+    a.nl = nl;
+    a.rows = rows;
+    a.A = ends.A;
+    a.mean = ends.mean; a.value = ends.value;
+    a.dmean = ends.dmean; a.dvalue = ends.dvalue; a.dout = ends.dout;
+    a.status = status;
+    int n_max = 0;
+    for (int i = 0; i < nl; ++i) {
+        const MlpLayer &x = layers[i];
+        Layer &y = a.l[i];
+        const bool narrow = x.ldx == 16 && x.K <= 16;  // the head's gradient, rows padded to 16
+        const int CB = narrow ? 16 : 64;
+        y.rb = 2 * CB;
+        y.chunks = (x.K + CB - 1) / CB;
+        y.N = x.N;
+        y.n = ((x.N + cs - 1) / cs + 15) / 16 * 16;
+        y.mode = x.mode; y.ldo = x.ldo;
+        y.bias = x.bias;
+        y.out = x.out; y.out_f32 = x.out_f32; y.mask = x.mask;
+        // a copy costs its warp some 150 cycles: chunks of a few KB go out several at a time
+        const bool whole = x.K % CB == 0;
+        auto fill = [&](int bytes) { const int g = kCopy / bytes; return !whole || g < 1 ? 1 : (g < y.chunks ? g : y.chunks); };
+        y.gA = fill(a.Mt * y.rb);
+        y.gB = fill(y.n * y.rb);
+        const long long da[4] = {y.gA > 1 ? CB : (narrow ? 16 : x.K), rows, y.gA > 1 ? y.chunks : 1, 1};
+        const long long db[4] = {y.gB > 1 ? CB : x.ldw, x.N, y.gB > 1 ? y.chunks : 1, 1};
+        const long long sa[3] = {2ll * x.ldx, 2ll * CB, 2ll * x.ldx * rows}, sb[3] = {2ll * x.ldw, 2ll * CB, 2ll * x.ldw * x.N};
+        const int ba[4] = {CB, a.Mt, y.gA, 1}, bb[4] = {CB, y.n, y.gB, 1};
+        PPO_TRY(make_map_strided(&y.mapA, x.X, 4, da, sa, ba));
+        PPO_TRY(make_map_strided(&y.mapB, x.W, 4, db, sb, bb));
+        n_max = y.n > n_max ? y.n : n_max;
+    }
+    a.tmem_cols = 32;
+    while ((int)a.tmem_cols < n_max) a.tmem_cols *= 2;
+    a.a_slot = kCopy;  // 128 rows of a chunk at most
+    a.b_slot = n_max * 128 > kCopy ? (uint32_t)n_max * 128u : kCopy;
+    const size_t room = kSmemMax - sizeof(Pipe) - kEpiWarps * kStage - 1024;
+    a.sA = (int)((80 * 1024) / a.a_slot);
+    if (a.sA > kMaxStages) a.sA = kMaxStages;
+    a.sB = (int)((room - (size_t)a.sA * a.a_slot) / a.b_slot);
+    if (a.sB > kMaxStages) a.sB = kMaxStages;
+    if (a.sB < 2) return PPO_ERR_UNSUPPORTED;
+    const size_t smem = (size_t)a.sA * a.a_slot + (size_t)a.sB * a.b_slot + kEpiWarps * kStage + sizeof(Pipe) + 1024;
+    const auto fn = cs == 8 ? mlp_chain8_kernel : mlp_chain4_kernel;
+    PPO_CUDA_CHECK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+    return ppo_launch(fn, dim3((unsigned)((rows + a.Mt - 1) / a.Mt * cs)), dim3(kThreads), smem, st, a);
+}
