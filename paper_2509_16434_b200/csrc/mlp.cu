@@ -91,12 +91,6 @@ __device__ __forceinline__ void chain(const Args &a, uint8_t *raw) {
     volatile int *abort_flag = &pipe->abort_flag;
     const int warp = warp_index(), lane = threadIdx.x & 31;
     const int rank = (int)blockIdx.x % CS, row0 = (int)blockIdx.x / CS * a.Mt;
-    const int pack = a.dout ? 1 : 0;  // a step before the first layer
-    // copy of `g` chunks from chunk k of rows `row` on
-    auto copy = [](uint32_t dst, const CUtensorMap *map, uint64_t *bar, int g, int rb, int k, int row) {
-        if (g > 1) tma_load_4d(dst, map, bar, 0, row, k, 0);
-        else tma_load_4d(dst, map, bar, k * (rb >> 1), row, 0, 0);
-    };
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < a.sA; ++s) {
@@ -118,32 +112,41 @@ __device__ __forceinline__ void chain(const Args &a, uint8_t *raw) {
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(m)) : "memory");
     }
     __syncwarp();
-    cluster_sync();  // the barriers exist before anyone arrives at a neighbour's
+    cluster_arrive();  // the barriers exist before anyone arrives at a neighbour's: all threads wait for it once, later
     grid_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = pipe->tmem_slot;
 
+    // (what a layer's loops need is taken out of the parameters before them: indexed by layer and read in the loop, they made a copy
+    // cost 430 cycles and a chunk's MMAs 570)
     if (warp == 0) {
         int s = 0, it = 0;
         uint32_t ph = 0;
         bool ok = true;
         for (int l = 0; l < a.nl && ok; ++l) {
-            const Layer &y = a.l[l];
-            if (l + pack > 0) {  // what the cluster has left for this layer
-                ok = cluster_mbar_wait(&pipe->ready, (uint32_t)(l + pack - 1) & 1u, abort_flag, a.status);
+            const int chunks = a.l[l].chunks, rb = a.l[l].rb, g = a.l[l].gA, N = a.l[l].N, n = a.l[l].n;
+            const CUtensorMap *const map = &a.l[l].mapA;
+            if (l > 0) {  // what the cluster has left for this layer
+                ok = cluster_mbar_wait(&pipe->ready, (uint32_t)(l - 1) & 1u, abort_flag, a.status);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 fence_proxy_global();
             }
-            if (rank * y.n >= y.N) continue;
-            for (int k = 0; k < y.chunks; k += y.gA, ++it) {
+            if (rank * n >= N) continue;
+            if (l == 0 && a.dout) {  // the epilogue fills the first stage
+                it = s = 1;
+                continue;
+            }
+            const uint32_t bytes = (uint32_t)(g * a.Mt * rb);
+            for (int k = 0; k < chunks; k += g, ++it) {
                 ok = mbar_wait_warp(&pipe->emptyA[s], ph ^ 1u, abort_flag, a.status);
                 if (!ok) break;
+                const int c0 = g > 1 ? 0 : k * (rb >> 1), c2 = g > 1 ? k : 0;
                 if (elect_one()) {
-                    mbar_arrive_expect_tx(&pipe->fullA[s], (uint32_t)(y.gA * a.Mt * y.rb));
-                    copy(base + (uint32_t)s * a.a_slot, &y.mapA, &pipe->fullA[s], y.gA, y.rb, k, row0);
+                    mbar_arrive_expect_tx(&pipe->fullA[s], bytes);
+                    tma_load_4d(base + (uint32_t)s * a.a_slot, map, &pipe->fullA[s], c0, row0, c2, 0);
                 }
                 __syncwarp();
                 if (++s == a.sA) { s = 0; ph ^= 1u; }
@@ -156,14 +159,17 @@ __device__ __forceinline__ void chain(const Args &a, uint8_t *raw) {
         uint32_t ph = 0;
         bool ok = true;
         for (int l = 0; l < a.nl && ok; ++l) {
-            const Layer &y = a.l[l];
-            if (rank * y.n >= y.N) continue;
-            for (int k = 0; k < y.chunks; k += y.gB, ++it) {
+            const int chunks = a.l[l].chunks, rb = a.l[l].rb, g = a.l[l].gB, n = a.l[l].n, col0 = rank * n;
+            const CUtensorMap *const map = &a.l[l].mapB;
+            if (col0 >= a.l[l].N) continue;
+            const uint32_t bytes = (uint32_t)(g * n * rb);
+            for (int k = 0; k < chunks; k += g, ++it) {
                 ok = mbar_wait_warp(&pipe->emptyB[s], ph ^ 1u, abort_flag, a.status);
                 if (!ok) break;
+                const int c0 = g > 1 ? 0 : k * (rb >> 1), c2 = g > 1 ? k : 0;
                 if (elect_one()) {
-                    mbar_arrive_expect_tx(&pipe->fullB[s], (uint32_t)(y.gB * y.n * y.rb));
-                    copy(b_base + (uint32_t)s * a.b_slot, &y.mapB, &pipe->fullB[s], y.gB, y.rb, k, rank * y.n);
+                    mbar_arrive_expect_tx(&pipe->fullB[s], bytes);
+                    tma_load_4d(b_base + (uint32_t)s * a.b_slot, map, &pipe->fullB[s], c0, col0, c2, 0);
                 }
                 __syncwarp();
                 if (++s == a.sB) { s = 0; ph ^= 1u; }
@@ -178,24 +184,29 @@ __device__ __forceinline__ void chain(const Args &a, uint8_t *raw) {
         uint32_t pa = 0, pb = 0;
         bool ok = true;
         for (int l = 0; l < a.nl && ok; ++l) {
-            const Layer &y = a.l[l];
-            if (rank * y.n >= y.N) continue;
-            const uint32_t idesc = instr_desc(128, y.n, 0, 0), rb = (uint32_t)y.rb;
+            const int chunks = a.l[l].chunks, n = a.l[l].n, gA = a.l[l].gA, gB = a.l[l].gB;
+            if (rank * n >= a.l[l].N) continue;
+            const uint32_t rb = (uint32_t)a.l[l].rb, idesc = instr_desc(128, n, 0, 0);
             const uint64_t d0 = smem_desc_sw(base, 16, 8u * rb, rb);
             const uint32_t lo = (uint32_t)d0, hi = (uint32_t)(d0 >> 32), b_lo = lo + ((b_base - base) >> 4);
-            const uint32_t a16 = (uint32_t)(a.Mt * y.rb) >> 4, b16 = (uint32_t)(y.n * y.rb) >> 4;
+            const uint32_t a16 = (uint32_t)a.Mt * rb >> 4, b16 = (uint32_t)n * rb >> 4;
+            const bool wide = rb == 128;
             int ia = 0, ib = 0;  // chunk within its stage
-            for (int k = 0; k < y.chunks; ++k) {
+            for (int k = 0; k < chunks; ++k) {
                 if (ib == 0) ok = mbar_wait_warp(&pipe->fullB[sb], pb, abort_flag, a.status);
                 if (ok && ia == 0) ok = mbar_wait_warp(&pipe->fullA[sa], pa, abort_flag, a.status);
                 if (!ok) break;
                 tc_fence_after();
-                const bool last = k + 1 == y.chunks, end_a = last || ia + 1 == y.gA, end_b = last || ib + 1 == y.gB;
+                const bool last = k + 1 == chunks, end_a = last || ia + 1 == gA, end_b = last || ib + 1 == gB;
                 if (elect_one()) {
                     const uint32_t la = lo + (uint32_t)sa * (a.a_slot >> 4) + (uint32_t)ia * a16;
                     const uint32_t lb = b_lo + (uint32_t)sb * (a.b_slot >> 4) + (uint32_t)ib * b16;
                     umma_bf16_lh(tmem, la, hi, lb, hi, idesc, k > 0 ? 1u : 0u);
-                    for (int j = 1; j < (int)(rb >> 5); ++j) umma_bf16_lh(tmem, la + 2 * j, hi, lb + 2 * j, hi, idesc, 1u);
+                    if (wide) {  // unrolled: a loop here would take the operands out of the uniform registers
+                        umma_bf16_lh(tmem, la + 2, hi, lb + 2, hi, idesc, 1u);
+                        umma_bf16_lh(tmem, la + 4, hi, lb + 4, hi, idesc, 1u);
+                        umma_bf16_lh(tmem, la + 6, hi, lb + 6, hi, idesc, 1u);
+                    }
                     if (end_a) umma_commit(&pipe->emptyA[sa]);
                     if (end_b) umma_commit(&pipe->emptyB[sb]);
                 }
@@ -220,11 +231,14 @@ __device__ __forceinline__ void chain(const Args &a, uint8_t *raw) {
         uint4 *const stg = reinterpret_cast<uint4 *>(smem + stg_off + (uint32_t)(warp - 4) * kStage);
         const int rr0 = lane >> 2, piece = lane & 3, sw = (lane >> 1) & 3;
         const bool rows_here = lg * 32 < a.Mt;
+        bool joined = false;  // waited for the cluster's start
         // Behind this CTA's stores: one release, an arrival at every CTA's barrier.  before: the phase this CTA's part is made
         // from (-1: none); a CTA without columns has not waited for it, and must not arrive a second time before it is complete.
         auto publish = [&](bool ok, int before) -> bool {
             if (before >= 0) ok = cluster_mbar_wait(&pipe->ready, (uint32_t)before & 1u, abort_flag, a.status) && ok;
             if (!epi_all(ok)) return false;
+            if (!joined) cluster_wait();
+            joined = true;
             if (warp == 4) {
                 if (lane < CS) arrive_in_cta(&pipe->ready, (uint32_t)lane);
                 __syncwarp();
@@ -240,24 +254,38 @@ __device__ __forceinline__ void chain(const Args &a, uint8_t *raw) {
             for (int l = 0; l < kMlpLayers; ++l) pipe->bias[l * kMaxSlice + et] = b[l];
             epi_all(true);
         }
-        if (pack) {
+        if (a.dout) {
+            // The head's gradient as bf16: every CTA makes the tile's rows for itself, straight into the first stage (32-byte rows,
+            // their two pieces swapped in every other four), and its share of them for the weight gradient.
             const int per = a.Mt / CS;
-            for (int i = et; i < per * 16; i += kEpiWarps * 32) {
-                const int r = row0 + rank * per + (i >> 4), j = i & 15;
-                if (r >= a.rows) break;
-                float v = 0.f;
-                if (j < a.A) v = a.dmean[(size_t)r * a.A + j];
-                else if (j == a.A) v = a.dvalue[r];
-                a.dout[(size_t)r * 16 + j] = __float2bfloat16_rn(v);
+            for (int i = et; i < a.Mt * 2; i += kEpiWarps * 32) {
+                const int row = i >> 1, p = i & 1, r = row0 + row;
+                float v[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const int j = 8 * p + k;
+                    v[k] = 0.f;
+                    if (r < a.rows && j < a.A) v[k] = __ldg(a.dmean + (size_t)r * a.A + j);
+                    else if (r < a.rows && j == a.A) v[k] = __ldg(a.dvalue + r);
+                }
+                const uint4 o = make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]), pack_bf16x2(v[6], v[7]));
+                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(base + (uint32_t)row * 32u + (((uint32_t)p ^ (((uint32_t)row >> 2) & 1u)) << 4)),
+                             "r"(o.x), "r"(o.y), "r"(o.z), "r"(o.w)
+                             : "memory");
+                if (r < a.rows && row / per == rank) *reinterpret_cast<uint4 *>(a.dout + (size_t)r * 16 + 8 * p) = o;
             }
-            publish(true, -1);
+            fence_async_smem();
+            epi_all(true);
+            if (et == 0 && rank * a.l[0].n < a.l[0].N) mbar_arrive(&pipe->fullA[0]);
         }
         uint32_t tph = 0;
         for (int l = 0; l < a.nl; ++l) {
-            const Layer &y = a.l[l];
-            const int col0 = rank * y.n;
+            const int N = a.l[l].N, n = a.l[l].n, mode = a.l[l].mode, ldo = a.l[l].ldo, col0 = rank * n;
+            bf16 *const out = a.l[l].out;
+            float *const out_f32 = a.l[l].out_f32;
+            const bf16 *const mask = a.l[l].mask;
             bool ok = true;
-            if (col0 < y.N && rows_here) {
+            if (col0 < N && rows_here) {
                 // 16 bytes of the gate for each of this lane's four stores of a group, fetched ahead (see gemm_tma.cu)
                 uint4 gate[4];
                 auto fetch = [&](int g) {
@@ -265,26 +293,21 @@ __device__ __forceinline__ void chain(const Args &a, uint8_t *raw) {
                     for (int ps = 0; ps < 4; ++ps) {
                         const int r = row0 + lg * 32 + ps * 8 + rr0, c = col0 + g + piece * 8;
                         gate[ps] = make_uint4(0, 0, 0, 0);
-                        if (g < y.n && r < a.rows && g + piece * 8 < y.n && c < y.N)
-                            gate[ps] = __ldg(reinterpret_cast<const uint4 *>(y.mask + (size_t)r * y.ldo + c));
+                        if (g < n && r < a.rows && g + piece * 8 < n && c < N)
+                            gate[ps] = __ldg(reinterpret_cast<const uint4 *>(mask + (size_t)r * ldo + c));
                     }
                 };
-                if (y.mode == MLP_GATED) fetch(half * 32);
+                if (mode == MLP_GATED) fetch(half * 32);
                 ok = mbar_wait(&pipe->tfull, tph, abort_flag, a.status);
                 ok = __all_sync(0xffffffffu, ok);
                 tc_fence_after();
                 const uint32_t tm = tmem + ((uint32_t)(lg * 32) << 16);
 #pragma unroll 1
-                for (int g = half * 32; ok && g < y.n; g += 64) {
-                    float v[32];
+                for (int g = half * 32; ok && g < n; g += 64) {
+                    float v[32] = {};
                     tmem_ld16(tm + (uint32_t)g, v);
-                    if (g + 16 < y.n) {
-                        tmem_ld16(tm + (uint32_t)g + 16u, v + 16);
-                    } else {
-#pragma unroll
-                        for (int i = 16; i < 32; ++i) v[i] = 0.f;
-                    }
-                    if (y.mode == MLP_HEAD) {
+                    if (g + 16 < n) tmem_ld16(tm + (uint32_t)g + 16u, v + 16);  // (else nothing made of those is stored)
+                    if (mode == MLP_HEAD) {
                         if (grow < a.rows) {
 #pragma unroll
                             for (int i = 0; i < 16; ++i) {
@@ -295,7 +318,7 @@ __device__ __forceinline__ void chain(const Args &a, uint8_t *raw) {
                         }
                         continue;
                     }
-                    if (y.mode == MLP_F32) {  // 32 rows x 128 bytes, 16-byte pieces swizzled by the row
+                    if (mode == MLP_F32) {  // 32 rows x 128 bytes, 16-byte pieces swizzled by the row
 #pragma unroll
                         for (int j = 0; j < 8; ++j)
                             stg[lane * 8 + (j ^ (lane & 7))] = make_uint4(__float_as_uint(v[4 * j]), __float_as_uint(v[4 * j + 1]),
@@ -304,19 +327,20 @@ __device__ __forceinline__ void chain(const Args &a, uint8_t *raw) {
 #pragma unroll
                         for (int ps = 0; ps < 8; ++ps) {
                             const int rr = ps * 4 + (lane >> 3), p8 = lane & 7, r = row0 + lg * 32 + rr, c = col0 + g + p8 * 4;
-                            if (r < a.rows && g + p8 * 4 < y.n && c < y.N)
-                                *reinterpret_cast<uint4 *>(y.out_f32 + (size_t)r * y.ldo + c) = stg[rr * 8 + (p8 ^ (rr & 7))];
+                            if (r < a.rows && g + p8 * 4 < n && c < N)
+                                *reinterpret_cast<uint4 *>(out_f32 + (size_t)r * ldo + c) = stg[rr * 8 + (p8 ^ (rr & 7))];
                         }
                         __syncwarp();
                         continue;
                     }
                     uint32_t pk[16];
-                    if (y.mode == MLP_RELU) {
-                        const float *bp = pipe->bias + l * kMaxSlice + g;
+                    if (mode == MLP_RELU) {
+                        const float4 *bp = reinterpret_cast<const float4 *>(pipe->bias + l * kMaxSlice + g);
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            const bool in = j < 8 || g + 16 < y.n;
-                            pk[j] = relu_pack_bf16x2(v[2 * j] + (in ? bp[2 * j] : 0.f), v[2 * j + 1] + (in ? bp[2 * j + 1] : 0.f));
+                        for (int q = 0; q < 8; ++q) {
+                            const float4 b = bp[q];
+                            pk[2 * q] = relu_pack_bf16x2(v[4 * q] + b.x, v[4 * q + 1] + b.y);
+                            pk[2 * q + 1] = relu_pack_bf16x2(v[4 * q + 2] + b.z, v[4 * q + 3] + b.w);
                         }
                     } else {
 #pragma unroll
@@ -328,23 +352,29 @@ __device__ __forceinline__ void chain(const Args &a, uint8_t *raw) {
 #pragma unroll
                     for (int ps = 0; ps < 4; ++ps) {
                         const int rr = ps * 8 + rr0, r = row0 + lg * 32 + rr, c = col0 + g + piece * 8;
-                        if (r < a.rows && g + piece * 8 < y.n && c < y.N) {
+                        if (r < a.rows && g + piece * 8 < n && c < N) {
                             uint4 o = stg[rr * 4 + (piece ^ ((rr >> 1) & 3))];
-                            if (y.mode == MLP_GATED) {
+                            if (mode == MLP_GATED) {
                                 o.x &= gate_open(gate[ps].x); o.y &= gate_open(gate[ps].y);
                                 o.z &= gate_open(gate[ps].z); o.w &= gate_open(gate[ps].w);
                             }
-                            *reinterpret_cast<uint4 *>(y.out + (size_t)r * y.ldo + c) = o;
+                            *reinterpret_cast<uint4 *>(out + (size_t)r * ldo + c) = o;
                         }
                     }
-                    if (y.mode == MLP_GATED) fetch(g + 64);
+                    if (mode == MLP_GATED) fetch(g + 64);
                     __syncwarp();
                 }
                 tc_fence_before();
             }
-            if (col0 < y.N) tph ^= 1u;
-            if (l + 1 < a.nl && !publish(ok, l + pack - 1)) break;
+            if (col0 < N) tph ^= 1u;
+            if (l + 1 < a.nl && !publish(ok, l - 1)) break;
         }
+        __syncwarp();
+        if (!joined) cluster_wait();
+    }
+    if (warp < 4) {
+        __syncwarp();
+        cluster_wait();
     }
     tc_fence_before();
     __syncthreads();
