@@ -31,7 +31,7 @@ constexpr uint32_t kStage = 4096;               // staging of an epilogue warp: 
 struct Layer {
     CUtensorMap mapA, mapB;
     int chunks, rb;       // of the reduction, and bytes of a row of one
-    int gA, gB;           // chunks a copy brings (a stage holds them): more than one where the reduction is whole chunks
+    int g;                // chunks of a stage (a copy brings them): more than one where the reduction is whole chunks
     int N, n;             // columns; of them in a CTA's slice
     int mode, ldo;
     const float *bias;
@@ -126,7 +126,7 @@ __device__ __forceinline__ void chain(const Args &a, uint8_t *raw) {
         uint32_t ph = 0;
         bool ok = true;
         for (int l = 0; l < a.nl && ok; ++l) {
-            const int chunks = a.l[l].chunks, rb = a.l[l].rb, g = a.l[l].gA, N = a.l[l].N, n = a.l[l].n;
+            const int chunks = a.l[l].chunks, rb = a.l[l].rb, g = a.l[l].g, N = a.l[l].N, n = a.l[l].n;
             const CUtensorMap *const map = &a.l[l].mapA;
             if (l > 0) {  // what the cluster has left for this layer
                 ok = cluster_mbar_wait(&pipe->ready, (uint32_t)(l - 1) & 1u, abort_flag, a.status);
@@ -159,7 +159,7 @@ __device__ __forceinline__ void chain(const Args &a, uint8_t *raw) {
         uint32_t ph = 0;
         bool ok = true;
         for (int l = 0; l < a.nl && ok; ++l) {
-            const int chunks = a.l[l].chunks, rb = a.l[l].rb, g = a.l[l].gB, n = a.l[l].n, col0 = rank * n;
+            const int chunks = a.l[l].chunks, rb = a.l[l].rb, g = a.l[l].g, n = a.l[l].n, col0 = rank * n;
             const CUtensorMap *const map = &a.l[l].mapB;
             if (col0 >= a.l[l].N) continue;
             const uint32_t bytes = (uint32_t)(g * n * rb);
@@ -180,47 +180,46 @@ __device__ __forceinline__ void chain(const Args &a, uint8_t *raw) {
     } else if (warp == 1) {
         // the accumulator of the layer before has been read: the rows of this one wait for the cluster's arrivals, this CTA's
         // epilogue among them
+        const int sA = a.sA, sB = a.sB;
+        const uint32_t a_slot16 = a.a_slot >> 4, b_slot16 = a.b_slot >> 4;
         int sa = 0, sb = 0;
         uint32_t pa = 0, pb = 0;
         bool ok = true;
         for (int l = 0; l < a.nl && ok; ++l) {
-            const int chunks = a.l[l].chunks, n = a.l[l].n, gA = a.l[l].gA, gB = a.l[l].gB;
+            const int chunks = a.l[l].chunks, n = a.l[l].n, g = a.l[l].g;
             if (rank * n >= a.l[l].N) continue;
             const uint32_t rb = (uint32_t)a.l[l].rb, idesc = instr_desc(128, n, 0, 0);
             const uint64_t d0 = smem_desc_sw(base, 16, 8u * rb, rb);
             const uint32_t lo = (uint32_t)d0, hi = (uint32_t)(d0 >> 32), b_lo = lo + ((b_base - base) >> 4);
             const uint32_t a16 = (uint32_t)a.Mt * rb >> 4, b16 = (uint32_t)n * rb >> 4;
             const bool wide = rb == 128;
-            int ia = 0, ib = 0;  // chunk within its stage
-            for (int k = 0; k < chunks; ++k) {
-                if (ib == 0) ok = mbar_wait_warp(&pipe->fullB[sb], pb, abort_flag, a.status);
-                if (ok && ia == 0) ok = mbar_wait_warp(&pipe->fullA[sa], pa, abort_flag, a.status);
+            uint32_t accum = 0;
+            for (int k = 0; k < chunks; k += g) {
+                ok = mbar_wait_warp(&pipe->fullB[sb], pb, abort_flag, a.status);
+                if (!ok) break;
+                ok = mbar_wait_warp(&pipe->fullA[sa], pa, abort_flag, a.status);
                 if (!ok) break;
                 tc_fence_after();
-                const bool last = k + 1 == chunks, end_a = last || ia + 1 == gA, end_b = last || ib + 1 == gB;
-                if (elect_one()) {
-                    const uint32_t la = lo + (uint32_t)sa * (a.a_slot >> 4) + (uint32_t)ia * a16;
-                    const uint32_t lb = b_lo + (uint32_t)sb * (a.b_slot >> 4) + (uint32_t)ib * b16;
-                    umma_bf16_lh(tmem, la, hi, lb, hi, idesc, k > 0 ? 1u : 0u);
-                    if (wide) {  // unrolled: a loop here would take the operands out of the uniform registers
-                        umma_bf16_lh(tmem, la + 2, hi, lb + 2, hi, idesc, 1u);
-                        umma_bf16_lh(tmem, la + 4, hi, lb + 4, hi, idesc, 1u);
-                        umma_bf16_lh(tmem, la + 6, hi, lb + 6, hi, idesc, 1u);
+                const int nval = min(g, chunks - k);
+                uint32_t la = lo + (uint32_t)sa * a_slot16, lb = b_lo + (uint32_t)sb * b_slot16;
+                for (int c = 0; c < nval; ++c, la += a16, lb += b16) {
+                    if (elect_one()) {
+                        umma_bf16_lh(tmem, la, hi, lb, hi, idesc, accum);
+                        if (wide) {
+                            umma_bf16_lh(tmem, la + 2, hi, lb + 2, hi, idesc, 1u);
+                            umma_bf16_lh(tmem, la + 4, hi, lb + 4, hi, idesc, 1u);
+                            umma_bf16_lh(tmem, la + 6, hi, lb + 6, hi, idesc, 1u);
+                        }
                     }
-                    if (end_a) umma_commit(&pipe->emptyA[sa]);
-                    if (end_b) umma_commit(&pipe->emptyB[sb]);
+                    accum = 1u;
+                }
+                if (elect_one()) {
+                    umma_commit(&pipe->emptyA[sa]);
+                    umma_commit(&pipe->emptyB[sb]);
                 }
                 __syncwarp();
-                ++ia;
-                ++ib;
-                if (end_a) {
-                    ia = 0;
-                    if (++sa == a.sA) { sa = 0; pa ^= 1u; }
-                }
-                if (end_b) {
-                    ib = 0;
-                    if (++sb == a.sB) { sb = 0; pb ^= 1u; }
-                }
+                if (++sa == sA) { sa = 0; pa ^= 1u; }
+                if (++sb == sB) { sb = 0; pb ^= 1u; }
             }
             if (ok && elect_one()) umma_commit(&pipe->tfull);
             __syncwarp();
@@ -446,13 +445,12 @@ int mlp_chain(const MlpLayer *layers, int nl, int rows, const MlpEnds &ends, int
         y.out = x.out; y.out_f32 = x.out_f32; y.mask = x.mask;
         // a copy costs its warp some 150 cycles: chunks of a few KB go out several at a time
         const bool whole = x.K % CB == 0;
-        auto fill = [&](int bytes) { const int g = kCopy / bytes; return !whole || g < 1 ? 1 : (g < y.chunks ? g : y.chunks); };
-        y.gA = fill(a.Mt * y.rb);
-        y.gB = fill(y.n * y.rb);
-        const long long da[4] = {y.gA > 1 ? CB : (narrow ? 16 : x.K), rows, y.gA > 1 ? y.chunks : 1, 1};
-        const long long db[4] = {y.gB > 1 ? CB : x.ldw, x.N, y.gB > 1 ? y.chunks : 1, 1};
+        y.g = whole ? kCopy / ((a.Mt > y.n ? a.Mt : y.n) * y.rb) : 1;
+        y.g = y.g < 1 ? 1 : (y.g < y.chunks ? y.g : y.chunks);
+        const long long da[4] = {y.g > 1 ? CB : (narrow ? 16 : x.K), rows, y.g > 1 ? y.chunks : 1, 1};
+        const long long db[4] = {y.g > 1 ? CB : x.ldw, x.N, y.g > 1 ? y.chunks : 1, 1};
         const long long sa[3] = {2ll * x.ldx, 2ll * CB, 2ll * x.ldx * rows}, sb[3] = {2ll * x.ldw, 2ll * CB, 2ll * x.ldw * x.N};
-        const int ba[4] = {CB, a.Mt, y.gA, 1}, bb[4] = {CB, y.n, y.gB, 1};
+        const int ba[4] = {CB, a.Mt, y.g, 1}, bb[4] = {CB, y.n, y.g, 1};
         PPO_TRY(make_map_strided(&y.mapA, x.X, 4, da, sa, ba));
         PPO_TRY(make_map_strided(&y.mapB, x.W, 4, db, sb, bb));
         n_max = y.n > n_max ? y.n : n_max;
