@@ -484,6 +484,50 @@ __global__ void __launch_bounds__(256) pool_concat_kernel(const bf16 *__restrict
     h0[b * (C + P) + C + j] = __float2bfloat16_rn(proprio[i]);
 }
 
+// The same for few rows of large maps, where a thread's chain of loads (32 pixels a trip) is all the time there is: a block
+// takes 32 channels of a row, brings kPoolPx pixels at a time into shared memory with every thread's loads in flight at once, and
+// 16 threads add two channels each, pixel by pixel as above: the same sums.  The last block of a row copies its proprioception.
+constexpr int kPoolPx = 512;
+__global__ void __launch_bounds__(256) pool_concat_tall_kernel(const bf16 *__restrict__ act, const float *__restrict__ proprio,
+                                                               bf16 *__restrict__ h0, int npx, int C, int P) {
+    grid_wait();
+    __shared__ __align__(16) uint4 px[kPoolPx * 4];  // [pixel][32 channels]
+    const int b = blockIdx.y, c0 = blockIdx.x * 32, t = threadIdx.x;
+    const uint4 *src = reinterpret_cast<const uint4 *>(act + (size_t)b * npx * C + c0);
+    const int row16 = C >> 3;  // 16-byte pieces from pixel to pixel
+    float s0 = 0.f, s1 = 0.f;
+    for (int p0 = 0; p0 < npx; p0 += kPoolPx) {
+        const int n = min(kPoolPx, npx - p0);
+        uint4 v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int i = t + u * 256, p = i >> 2;
+            if (p < n) v[u] = __ldcs(src + (size_t)(p0 + p) * row16 + (i & 3));
+        }
+        if (p0 > 0) __syncthreads();
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int i = t + u * 256;
+            if ((i >> 2) < n) px[i] = v[u];
+        }
+        __syncthreads();
+        if (t < 16) {
+            const uint32_t *w = reinterpret_cast<const uint32_t *>(px) + t;
+#pragma unroll 16
+            for (int p = 0; p < n; ++p) {
+                const uint32_t r = w[p * 16];
+                const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&r));
+                s0 += f.x;
+                s1 += f.y;
+            }
+        }
+    }
+    const float inv = 1.f / (float)npx;
+    if (t < 16) *reinterpret_cast<uint32_t *>(h0 + (size_t)b * (C + P) + c0 + 2 * t) = pack_bf16x2(s0 * inv, s1 * inv);
+    if (blockIdx.x == gridDim.x - 1)
+        for (int j = t; j < P; j += 256) h0[(size_t)b * (C + P) + C + j] = __float2bfloat16_rn(proprio[(size_t)b * P + j]);
+}
+
 // dact[b][px][c] = dh0[b][c] / npx where act > 0, else 0; 8 channels per thread.  I: index type, 32 bits where they do (two
 // 64-bit divisions per thread cost as much as its memory traffic).
 template <typename I>
@@ -1291,6 +1335,14 @@ extern "C" int ppo_encoder_fwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
     } else {
         const int C = m->Cs[m->L];
         const bool few = (long long)rows * (C / 8) < 512LL * ppo_num_sms();  // not two blocks of threads of 8 channels per SM
+        const int npx = m->Hs[m->L] * m->Ws[m->L];
+        // One wave of its blocks (six or seven per SM), and a chain of more than four trips otherwise (us, threads of 2 channels ->
+        // blocks): 850 pixels x 64 channels, 16 rows 30.8 -> 10.3; 221 x 128, 140 rows 10.9 -> 5.4, 384 rows 11.4 and 12.7, 768
+        // rows 13.2 and 22.5.
+        if (C % 32 == 0 && npx > 128 && (long long)rows * C <= 192LL * ppo_num_sms() && rows <= 65535)
+            PPO_TRY(ppo_launch(pool_concat_tall_kernel, dim3(C / 32, rows), dim3(256), 0, st, m->act[m->L], mb->proprio + (size_t)row0 * d.P,
+                               m->h[0], npx, C, d.P));
+        else
         PPO_TRY(ppo_launch(few ? pool_concat_kernel<2> : pool_concat_kernel<8>,
                            dim3(ppo_cdiv((long long)rows * (C / (few ? 2 : 8) + d.P), 256)), dim3(256), 0, st,
                            m->act[m->L], mb->proprio + (size_t)row0 * d.P, m->h[0], rows, m->Hs[m->L] * m->Ws[m->L], C, d.P));

@@ -54,6 +54,24 @@ def test_last_gate_is_open_for_positive_activations_only(name):
         assert torch.equal(gradients(pattern), want), hex(pattern)
 
 
+# average pool of few rows with many pixels (one and several loads into shared memory, exactly full ones, 32 and 96 channels) beside
+# the sum in fp64, rounded to bf16: n sums in fp32 are within n 2^-24 of the sum of the magnitudes, the rounding within 2^-8
+@pytest.mark.parametrize("H,W,last,rows", [(44, 48, 32, 1), (64, 128, 96, 3), (90, 92, 32, 5), (45, 47, 64, 200), (130, 140, 64, 2)])
+def test_pool_of_large_maps(H, W, last, rows):
+    w = synth.Workload("pool", 2 * rows, 1, H, W, (16, last), (3, 3), (40,), 1, 2, P=24, A=3)
+    L, md, lay, theta, roll, action, logp, dev = base._setup(w, rows)
+    L.compute_gae(dev["last_value"])
+    ppo.ppo_shuffle_gather_minibatch(L.buffer, 5, 0, 0, w.minibatches, L.mb)
+    ppo.ppo_encoder_fwd(L.model, L.mb, 0, rows, L.mean, L.value)
+    npx = ((H + 3) // 4) * ((W + 3) // 4)
+    act = L.model.activation(0, 2)[:rows * npx * last].double().view(rows, npx, last)
+    h0 = L.model.activation(1, 0)[:rows * (last + 24)].double().view(rows, last + 24)
+    want = act.mean(1)
+    assert bool(((h0[:, :last] - want).abs() <= want.abs() * 2.0 ** -8 + act.abs().sum(1) * 2.0 ** -24).all())
+    assert torch.equal(h0[:, last:], L.mb.proprio[:rows].to(torch.bfloat16).double())
+    assert ppo.ppo_poll_status() == 0
+
+
 # weight gradient of a 16-channel layer in pairs of pixels: even widths (one pair, a tile that ends inside a row, several tiles per
 # row), odd heights, one image and many; an odd width goes pixel by pixel
 @pytest.mark.parametrize("H,W,N,last", [(8, 4, 2, 32), (9, 12, 6, 64), (35, 44, 6, 32), (10, 532, 2, 96), (35, 46, 6, 32)])
