@@ -22,8 +22,8 @@ namespace {
 
 using namespace tc;
 
-constexpr int kProducers = 128;       // 4 warps: gather, then epilogue
-constexpr int kThreads = 160;         // wgrad kernel: + 1 warp issuing the MMAs
+constexpr int kProducers = 256;       // wgrad kernel, 8 warps: gather; the first four then do the epilogue
+constexpr int kThreads = 288;         // + 1 warp issuing the MMAs
 constexpr int kMaxTaps = 49;
 // ------------------------------------------------------------------ K-major ----
 
@@ -402,7 +402,7 @@ __global__ void __launch_bounds__(kThreads) igemm_wgrad_kernel(const __grid_cons
         pipe->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 4) tmem_alloc(&pipe->tmem_slot, ncols);
+    if (warp == 8) tmem_alloc(&pipe->tmem_slot, ncols);
     grid_wait();
     tc_fence_before();
     __syncthreads();
@@ -416,9 +416,9 @@ __global__ void __launch_bounds__(kThreads) igemm_wgrad_kernel(const __grid_cons
     const int nkb = (int)((m_hi - m_lo + 63) >> 6);
     const uint32_t smem_base = smem_u32(smem);
 
-    if (warp < 4) {
+    if (warp < 8) {
         // Thread p owns 16-byte chunk column c16 = p % 16 of the 128-column A tile (and of each pair of
-        // 64-column B blocks) and rows p / 16 + 8 i, so that the lanes of a row read contiguous bytes.
+        // 64-column B blocks) and rows p / 16 + 16 i, so that the lanes of a row read contiguous bytes.
         const int p = threadIdx.x;
         const int c16 = p & 15, rg = p >> 4, half = c16 >> 3, q = c16 & 7;
         int a_off = -1, a_dy = 0, a_dx = 0;   // this thread's column: offset inside a source pixel and its tap
@@ -432,11 +432,11 @@ __global__ void __launch_bounds__(kThreads) igemm_wgrad_kernel(const __grid_cons
             }
         }
         const uint32_t dst0 = (uint32_t)half * 8192u + (uint32_t)rg * 128u + (((uint32_t)q ^ ((uint32_t)rg & 7u)) << 4);
-        // output pixel of each of the 8 rows, advanced by 64 rows per K block without divisions
-        int ow[8], oh[8], ob[8];
+        // output pixel of each of the 4 rows, advanced by 64 rows per K block without divisions
+        int ow[4], oh[4], ob[4];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const long long m = m_lo + rg + 8 * i;
+        for (int i = 0; i < 4; ++i) {
+            const long long m = m_lo + rg + 16 * i;
             ow[i] = (int)(m % a.Wo);
             const long long t = m / a.Wo;
             oh[i] = (int)(t % a.Ho);
@@ -451,18 +451,18 @@ __global__ void __launch_bounds__(kThreads) igemm_wgrad_kernel(const __grid_cons
             const uint32_t sa = smem_base + s * stage_bytes + dst0, sb = sa + 16384u - (uint32_t)half * 8192u;
             const long long mb = m_lo + (long long)kb * 64 + rg;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const long long m = mb + 8 * i;
+            for (int i = 0; i < 4; ++i) {
+                const long long m = mb + 16 * i;
                 const bool row_ok = m < m_hi;
                 const int yy = 2 * oh[i] + a_dy, xx = 2 * ow[i] + a_dx;
                 const bool v = row_ok && a_off >= 0 && (unsigned)yy < (unsigned)a.Hi && (unsigned)xx < (unsigned)a.Wi;
                 const bf16 *src = v ? a.X + (((long long)ob[i] * a.Hi + yy) * a.Wi + xx) * a.Ci + a_off : a.X;
-                cp_async16_ca(sa + (uint32_t)i * 1024u, src, v);
+                cp_async16_ca(sa + (uint32_t)i * 2048u, src, v);
                 const bf16 *dyrow = a.dY + m * a.ldy;
                 for (int blk = half; blk < nblkB; blk += 2) {
                     const int co = co0 + blk * 64 + q * 8;
                     const bool vb = row_ok && co < co_lim;
-                    cp_async16(sb + (uint32_t)blk * 8192u + (uint32_t)i * 1024u, vb ? dyrow + co : a.dY, vb);
+                    cp_async16(sb + (uint32_t)blk * 8192u + (uint32_t)i * 2048u, vb ? dyrow + co : a.dY, vb);
                 }
                 // next K block: 64 rows further
                 ow[i] += a.dow64;
@@ -477,9 +477,9 @@ __global__ void __launch_bounds__(kThreads) igemm_wgrad_kernel(const __grid_cons
         cp_async_wait<0>();
 
         // ---------------- epilogue: TMEM lane p is column j0 + p of dW^T
-        if (ok && nkb > 0) ok = mbar_wait(&pipe->tfull[0], 0, abort_flag, a.status);
+        if (warp < 4 && ok && nkb > 0) ok = mbar_wait(&pipe->tfull[0], 0, abort_flag, a.status);
         tc_fence_after();
-        if (ok && nkb > 0) {
+        if (warp < 4 && ok && nkb > 0) {
             float *tile = a.part + ((size_t)(blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * (size_t)(128 * BN);
             const uint32_t lane_base = tmem_d + ((uint32_t)(warp * 32) << 16);
             for (int c0 = 0; c0 < BN; c0 += 16) {
@@ -513,7 +513,7 @@ __global__ void __launch_bounds__(kThreads) igemm_wgrad_kernel(const __grid_cons
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 4) {
+    if (warp == 8) {
         tc_fence_after();
         tmem_dealloc(tmem_d, ncols);
     }
@@ -532,8 +532,13 @@ int kmajor_stages(int BN) {
     return s > kMaxStagesK ? kMaxStagesK : (s < 3 ? 3 : s);
 }
 size_t kmajor_smem(int BN) { return (size_t)kmajor_stages(BN) * (16384 + (size_t)BN * 128) + sizeof(PipeK) + 1024; }
+// Two CTAs on an SM where three stages of each fit: a grid is two CTAs per SM (the sums are cut that way), and gathering is a
+// matter of loads in flight and of warps to issue them, not of stages (32 -> 48 channels, 1024 rows of 31 x 38 pixels, one CTA
+// of 4 gathering warps -> two of 8: 171 -> 94 us).
 int wgrad_stages(int BN) {
-    int s = (int)((200 * 1024) / (16384 + (size_t)((BN + 63) / 64) * 8192));
+    const size_t stage = 16384 + (size_t)((BN + 63) / 64) * 8192;
+    int s = (int)((108 * 1024) / stage);
+    if (s < 3) s = (int)((200 * 1024) / stage);
     return s > kMaxStagesK ? kMaxStagesK : (s < 3 ? 3 : s);
 }
 size_t wgrad_smem(int BN) {
