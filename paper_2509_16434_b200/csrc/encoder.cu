@@ -884,14 +884,18 @@ __global__ void __launch_bounds__(256) ln_bwd_kernel(bf16 *__restrict__ d, const
 
 // ------------------------------------------------------------ recurrent trunk ----
 
-// State the first step of a sequence starts from: h_prev[0] = bf16(h_init), c_prev[0] = c_init (rows of one step, Be x H).
-__global__ void __launch_bounds__(256) lstm_init_kernel(const float *__restrict__ h_init, const float *__restrict__ c_init,
-                                                        bf16 *__restrict__ hprev, float *__restrict__ cprev, int n) {
+// State the first step of a sequence starts from: h_prev[0] = bf16(h_init), c_prev[0] = c_init (rows of one step, n = Be x H),
+// of gridDim.y layers whose h_init and c_init follow one another.
+struct InitJobs {
+    bf16 *hprev[PPO_MAX_LSTM];
+    float *cprev[PPO_MAX_LSTM];
+};
+__global__ void __launch_bounds__(256) lstm_init_kernel(const float *__restrict__ h_init, const float *__restrict__ c_init, InitJobs jobs, int n) {
     grid_wait();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, l = blockIdx.y;
     if (i >= n) return;
-    hprev[i] = __float2bfloat16_rn(h_init[i]);
-    cprev[i] = c_init[i];
+    jobs.hprev[l][i] = __float2bfloat16_rn(h_init[(size_t)l * n + i]);
+    jobs.cprev[l][i] = c_init[(size_t)l * n + i];
 }
 
 // One time step of one LSTM layer for Be envs, element-wise part: gate pre-activations = xg + hg + b,
@@ -997,7 +1001,7 @@ static int recorded(ppo_model *m, const PlanKey &key, cudaStream_t st, F &&make)
     return s;
 }
 
-enum { OP_FWD = 1, OP_DGRAD, OP_WGRAD, OP_CONV_WGRADS, OP_LSTM_FWD, OP_LSTM_BWD, OP_MLP_FWD, OP_MLP_BWD };
+enum { OP_FWD = 1, OP_DGRAD, OP_WGRAD, OP_CONV_WGRADS, OP_LSTM_FWD, OP_LSTM_BWD, OP_LSTM_STEP, OP_MLP_FWD, OP_MLP_BWD };
 
 static PlanKey plan_key(int op, const ConvGeom &g) {
     PlanKey k;
@@ -1179,10 +1183,30 @@ static int lstm_forward(ppo_model *m, int rows, cudaStream_t st) {
     const ppo_model_desc &d = m->d;
     const int T = m->seq_T, Be = m->seq_Be, H = d.lstm_h;
     if (T <= 0 || T * Be != rows || !m->seq_done) return PPO_ERR_STATE;
+    bool started = false;  // the states of all layers are in place
     for (int l = 0; l < d.n_lstm; ++l) {
         const int in = l == 0 ? m->hw[0] : H, ti = m->ti_lstm[l];
         const bf16 *X = l == 0 ? m->h[0] : m->lstm_hs[l - 1];
         float *cprev = m->lstm_c[l] + (size_t)m->mbmax * H;
+        if (T == 1) {
+            if (!started) {
+                InitJobs jobs;
+                for (int k = 0; k < d.n_lstm; ++k) {
+                    jobs.hprev[k] = m->lstm_hprev[k];
+                    jobs.cprev[k] = m->lstm_c[k] + (size_t)m->mbmax * H;
+                }
+                PPO_TRY(ppo_launch(lstm_init_kernel, dim3(ppo_cdiv((long long)Be * H, 256), d.n_lstm), dim3(256), 0, st, m->seq_h_init, m->seq_c_init,
+                                   jobs, Be * H));
+                started = true;
+            }
+            PlanKey k = plan_key(OP_LSTM_STEP, fc_geom(Be, in, l));
+            const int one = recorded(m, k, st, [&]() -> int {
+                return lstm_one_step(lstm_steps(m, l), X, in, m->shadow + m->tensors[ti].off, m->shadow + m->tensors[ti + 1].off,
+                                     m->master + m->tensors[ti + 2].off, ppo_device_status_ptr(), st);
+            });
+            if (one == PPO_OK) continue;
+            if (one != PPO_ERR_UNSUPPORTED) return one;
+        }
         PPO_TRY(gemm_nt_f32(m, rows, 4 * H, in, X, in, m->shadow + m->tensors[ti].off, m->lstm_xg, st));
         const int one = lstm_persistent(m, OP_LSTM_FWD, l, st, [&]() -> int {
             return lstm_fwd_steps(lstm_steps(m, l), m->shadow + m->tensors[ti + 1].off, m->lstm_xg, m->master + m->tensors[ti + 2].off,
@@ -1190,9 +1214,13 @@ static int lstm_forward(ppo_model *m, int rows, cudaStream_t st) {
         });
         if (one == PPO_OK) continue;
         if (one != PPO_ERR_UNSUPPORTED) return one;
-        PPO_TRY(ppo_launch(lstm_init_kernel, dim3(ppo_cdiv((long long)Be * H, 256)), dim3(256), 0, st, m->seq_h_init + (size_t)l * Be * H,
-                                                                          m->seq_c_init + (size_t)l * Be * H,
-                                                                          m->lstm_hprev[l], cprev, Be * H));
+        if (!started) {
+            InitJobs job;
+            job.hprev[0] = m->lstm_hprev[l];
+            job.cprev[0] = cprev;
+            PPO_TRY(ppo_launch(lstm_init_kernel, dim3(ppo_cdiv((long long)Be * H, 256)), dim3(256), 0, st, m->seq_h_init + (size_t)l * Be * H,
+                               m->seq_c_init + (size_t)l * Be * H, job, Be * H));
+        }
         for (int t = 0; t < T; ++t) {
             const size_t r0 = (size_t)t * Be;
             PPO_TRY(gemm_nt_f32(m, Be, 4 * H, H, m->lstm_hprev[l] + r0 * H, H, m->shadow + m->tensors[ti + 1].off, m->lstm_hg, st));

@@ -558,6 +558,171 @@ __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(kThreads, 1) lstm_bw
     bwd_steps<U, true>(a, smem_raw);
 }
 
+// ---- one step: acting ----
+
+// A sequence of one step has nothing to keep resident and nobody to exchange with: x W_x^T and h W_h^T of M envs and U units
+// (4 U columns, gate g of unit j at g U + j) run through one pipeline into two accumulators, and the cell works on their sum.
+// Separate launches for W_x x and the step had each its own pipeline to fill, and 512 envs x 1024 units, too many for the
+// time loop, took four of them.  What bounds it: the bytes a CTA pulls through L2 (M + 4 U rows of every chunk).
+// Measured (us per layer): 16 envs x 1024 units 16.7 -> 7.4; 512 envs x 1024 units 32 -> 19.
+struct StepArgs {
+    CUtensorMap mapX, mapH, mapWx, mapWh;
+    int Be, H;
+    int chunksX, gX, chunksH, gH;  // chunks of the two reductions, and of them in a copy
+    int stages;
+    const float *bias, *cprev;
+    float *gates, *c;
+    bf16 *h;
+    int32_t *status;
+};
+constexpr int kStepG = 2;  // chunks of a stage
+
+template <int M, int U>
+__global__ void __launch_bounds__(kThreads, 1) lstm_step_kernel(const __grid_constant__ StepArgs a) {
+    constexpr uint32_t kA = M * 128u, kB = 4u * U * 128u, kStageBytes = kStepG * (kA + kB);
+    constexpr int W = M * U >= 2048 ? 4 : (M * U >= 1024 ? 2 : 1);  // units of a thread in a pass over the cells
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    const int S = a.stages, H = a.H;
+    const uint32_t base = smem_u32(smem), x_base = base + (uint32_t)S * kStageBytes;  // (an MMA's rows behind M lie in what follows)
+    Pipe *pipe = reinterpret_cast<Pipe *>(smem + (size_t)S * kStageBytes + (size_t)M * U * 16);
+    volatile int *abort_flag = &pipe->abort_flag;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
+    const int slices = H / U, mt = (int)blockIdx.x / slices, u0 = ((int)blockIdx.x - mt * slices) * U, row0 = mt * M;
+    constexpr uint32_t ncols = 8 * U < 32 ? 32 : 8 * U;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < S; ++s) {
+            mbar_init(&pipe->full[s], 1);
+            mbar_init(&pipe->empty[s], 1);
+        }
+        mbar_init(&pipe->tfull, 1);
+        pipe->abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) tmem_alloc(&pipe->tmem_slot, ncols);
+    grid_wait();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = pipe->tmem_slot;
+
+    if (warp == 0) {
+        int s = 0, it = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        for (int part = 0; part < 2 && ok; ++part) {
+            const int chunks = part ? a.chunksH : a.chunksX, g = part ? a.gH : a.gX;
+            const CUtensorMap *const ma = part ? &a.mapH : &a.mapX, *const mb = part ? &a.mapWh : &a.mapWx;
+            for (int k = 0; k < chunks; k += g, ++it) {
+                ok = mbar_wait_warp(&pipe->empty[s], ph ^ 1u, abort_flag, a.status);
+                if (!ok) break;
+                const uint32_t dst = base + (uint32_t)s * kStageBytes;
+                const int c0 = g > 1 ? 0 : k * 64, ck = g > 1 ? k : 0;
+                if (elect_one()) {
+                    mbar_arrive_expect_tx(&pipe->full[s], (uint32_t)g * (kA + kB));
+                    tma_load_4d(dst, ma, &pipe->full[s], c0, row0, ck, 0);
+                    tma_load_4d(dst + kStepG * kA, mb, &pipe->full[s], c0, u0, 0, ck);
+                }
+                __syncwarp();
+                if (++s == S) { s = 0; ph ^= 1u; }
+            }
+        }
+        if (!ok && lane == 0)
+            for (int i = max(0, it - S); i < it; ++i) {
+                const long long t0 = clock64();
+                while (!mbar_try_wait(&pipe->full[i % S], (i / S) & 1))
+                    if (clock64() - t0 > kWaitCycles / 4) break;
+            }
+        __syncwarp();
+    } else if (warp == 1) {
+        constexpr uint32_t idesc = instr_desc(128, 4 * U, 0, 0);
+        const uint64_t d0 = smem_desc_sw(base, 16, 1024, 128);
+        const uint32_t lo = (uint32_t)d0, hi = (uint32_t)(d0 >> 32);
+        int s = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        for (int part = 0; part < 2 && ok; ++part) {
+            const int chunks = part ? a.chunksH : a.chunksX, g = part ? a.gH : a.gX;
+            const uint32_t td = tmem + (part ? 4u * U : 0u);
+            uint32_t accum = 0;
+            for (int k = 0; k < chunks; k += g) {
+                ok = mbar_wait_warp(&pipe->full[s], ph, abort_flag, a.status);
+                if (!ok) break;
+                tc_fence_after();
+                const int nval = min(g, chunks - k);
+                uint32_t la = lo + (uint32_t)s * (kStageBytes >> 4), lb = la + (kStepG * kA >> 4);
+                for (int c = 0; c < nval; ++c, la += kA >> 4, lb += kB >> 4) {
+                    if (elect_one()) {
+                        umma_bf16_lh(td, la, hi, lb, hi, idesc, accum);
+                        umma_bf16_lh(td, la + 2, hi, lb + 2, hi, idesc, 1u);
+                        umma_bf16_lh(td, la + 4, hi, lb + 4, hi, idesc, 1u);
+                        umma_bf16_lh(td, la + 6, hi, lb + 6, hi, idesc, 1u);
+                    }
+                    accum = 1u;
+                }
+                if (elect_one()) umma_commit(&pipe->empty[s]);
+                __syncwarp();
+                if (++s == S) { s = 0; ph ^= 1u; }
+            }
+        }
+        if (ok && elect_one()) umma_commit(&pipe->tfull);
+        __syncwarp();
+    } else {
+        const int lg = warp & 3, grp = (warp - 2) >> 2, ct = (int)threadIdx.x - 64;
+        auto place = [&](int row, int col) {  // of a float of the exchange tile [M][4 U] (see xch_addr)
+            return x_base + (uint32_t)row * (16u * U) +
+                   ((((uint32_t)col >> 2) ^ (((uint32_t)row & 1u) << 2 | (((uint32_t)row >> 1) & 3u))) << 4) + 4u * ((uint32_t)col & 3u);
+        };
+        const bool ok = mbar_wait(&pipe->tfull, 0, abort_flag, a.status);
+        tc_fence_after();
+        if (lg * 32 < M && __all_sync(0xffffffffu, ok)) {
+            const uint32_t tm = tmem + ((uint32_t)(lg * 32) << 16);
+#pragma unroll
+            for (int b = grp; b < U / 4; b += 4) {
+                float x[16], h[16];
+                tmem_ld16(tm + 16u * b, x);
+                tmem_ld16(tm + 4u * U + 16u * b, h);
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(place(lg * 32 + lane, 16 * b + 4 * j)), "f"(x[4 * j] + h[4 * j]),
+                                 "f"(x[4 * j + 1] + h[4 * j + 1]), "f"(x[4 * j + 2] + h[4 * j + 2]), "f"(x[4 * j + 3] + h[4 * j + 3])
+                                 : "memory");
+            }
+            tc_fence_before();
+        }
+        if (cell_all(ok)) {
+#pragma unroll 1
+            for (int i = ct * W; i < M * U; i += kCellWarps * 32 * W) {
+                const int row = i / U, col = i - row * U, e = row0 + row, j = u0 + col;
+                if (e >= a.Be) break;
+                const size_t r = (size_t)e * H + j, r4 = (size_t)e * 4 * H + j;
+                float p[4][W], b[4][W], cp[W], gi[W], gf[W], gg[W], go[W], cv[W], hv[W];
+                load_u<W>(a.cprev + r, cp);
+#pragma unroll
+                for (int g = 0; g < 4; ++g) {
+                    load_u<W>(a.bias + g * H + j, b[g]);
+                    lds_u<W>(place(row, g * U + col), p[g]);
+                }
+#pragma unroll
+                for (int k = 0; k < W; ++k)
+                    lstm_cell(p[0][k] + b[0][k], p[1][k] + b[1][k], p[2][k] + b[2][k], p[3][k] + b[3][k], cp[k], gi[k], gf[k], gg[k], go[k], cv[k], hv[k]);
+                store_u<W>(a.gates + r4, gi);
+                store_u<W>(a.gates + r4 + H, gf);
+                store_u<W>(a.gates + r4 + 2 * H, gg);
+                store_u<W>(a.gates + r4 + 3 * H, go);
+                store_u<W>(a.c + r, cv);
+                store_bf16_u<W>(a.h + r, pack_u<W>(hv));
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem, ncols);
+    }
+}
+
 // Shape part for tiles of 32 U envs; false where the layer or the sequence does not fit: a slice of W_h has to leave room for
 // the exchange and two chunks of A (four of 128 envs at H = 1024), and all CTAs have to be resident at once.
 bool plan(Args &a, int T, int Be, int H, int U, int &ctas, size_t &smem) {
@@ -579,6 +744,29 @@ template <typename F>
 int prepare_kernel(F *fn) {
     PPO_CUDA_CHECK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
     return PPO_OK;
+}
+
+template <int M, int U>
+int launch_step(StepArgs &a, int in, const LstmSteps &p, const bf16 *X, const bf16 *Wx, const bf16 *Wh, cudaStream_t st) {
+    const long long H = p.H, Be = p.Be;
+    auto maps = [&](CUtensorMap &ma, CUtensorMap &mb, const bf16 *A, const bf16 *B, int K, int &chunks, int &g) -> int {
+        chunks = (K + 63) / 64;
+        g = K % 64 == 0 && chunks > 1 ? kStepG : 1;
+        const bool many = g > 1;
+        const long long da[4] = {many ? 64 : K, Be, many ? chunks : 1, 1}, sa[3] = {2ll * K, 128, 2ll * K * Be};
+        const long long db[4] = {many ? 64 : K, H, 4, many ? chunks : 1}, sb[3] = {2ll * K, 2ll * K * H, 128};
+        const int ba[4] = {64, M, g, 1}, bb[4] = {64, U, 4, g};
+        PPO_TRY(make_map_strided(&ma, A, 4, da, sa, ba));
+        return make_map_strided(&mb, B, 4, db, sb, bb);
+    };
+    PPO_TRY(maps(a.mapX, a.mapWx, X, Wx, in, a.chunksX, a.gX));
+    PPO_TRY(maps(a.mapH, a.mapWh, p.hprev, Wh, (int)H, a.chunksH, a.gH));
+    const size_t stage = (size_t)kStepG * (M + 4 * U) * 128, fixed = (size_t)M * U * 16 + sizeof(Pipe) + 1024;
+    a.stages = (int)((kSmemMax - fixed) / stage);
+    if (a.stages > kMaxStages) a.stages = kMaxStages;
+    PPO_TRY(prepare_kernel(lstm_step_kernel<M, U>));
+    const unsigned ctas = (unsigned)((Be + M - 1) / M * (H / U));
+    return ppo_launch(lstm_step_kernel<M, U>, dim3(ctas), dim3(kThreads), (size_t)a.stages * stage + fixed, st, a);
 }
 
 // Whether `ctas` CTAs in clusters of four are resident at once: clusters fit the groups of SMs less tightly than single CTAs (33
@@ -676,4 +864,22 @@ int lstm_bwd_steps(const LstmSteps &p, const bf16 *WhT, const float *dtop, bf16 
     PPO_TRY(map_dg(a, p, dg, tile_envs(4)));
     PPO_TRY(prepare_kernel(lstm_bwd_kernel));
     return ppo_launch_together(lstm_bwd_kernel, dim3(ctas), dim3(kThreads), smem, st, a);
+}
+
+int lstm_one_step(const LstmSteps &p, const bf16 *X, int in, const bf16 *Wx, const bf16 *Wh, const float *bias, int32_t *status, cudaStream_t st) {
+    if (!status || p.T != 1 || p.H % 64 != 0 || in < 64 || in % 8 != 0) return PPO_ERR_UNSUPPORTED;
+    StepArgs a = {};
+    a.Be = p.Be; a.H = p.H;
+    a.bias = bias; a.cprev = p.cprev;
+    a.gates = p.gates; a.c = p.c; a.h = p.h;
+    a.status = status;
+    // the shape with the fewest bytes per CTA whose CTAs all run at once; the largest up to two waves
+    const long long sms = ppo_num_sms();
+    auto ctas = [&](int M, int U) { return (long long)((p.Be + M - 1) / M) * (p.H / U); };
+    if (ctas(32, 8) <= sms) return launch_step<32, 8>(a, in, p, X, Wx, Wh, st);
+    if (ctas(32, 16) <= sms) return launch_step<32, 16>(a, in, p, X, Wx, Wh, st);
+    if (ctas(64, 16) <= sms) return launch_step<64, 16>(a, in, p, X, Wx, Wh, st);
+    if (ctas(128, 16) <= sms) return launch_step<128, 16>(a, in, p, X, Wx, Wh, st);
+    if (ctas(128, 32) <= 2 * sms) return launch_step<128, 32>(a, in, p, X, Wx, Wh, st);
+    return PPO_ERR_UNSUPPORTED;
 }
