@@ -885,17 +885,31 @@ __global__ void __launch_bounds__(256) ln_bwd_kernel(bf16 *__restrict__ d, const
 // ------------------------------------------------------------ recurrent trunk ----
 
 // State the first step of a sequence starts from: h_prev[0] = bf16(h_init), c_prev[0] = c_init (rows of one step, n = Be x H),
-// of gridDim.y layers whose h_init and c_init follow one another.
+// of gridDim.y layers whose h_init and c_init follow one another; V elements per thread (four where h_init and c_init are aligned
+// for it, 512 envs x 2 x 1024 units: 11.9 -> 5 us).
 struct InitJobs {
     bf16 *hprev[PPO_MAX_LSTM];
     float *cprev[PPO_MAX_LSTM];
 };
+template <int V>
 __global__ void __launch_bounds__(256) lstm_init_kernel(const float *__restrict__ h_init, const float *__restrict__ c_init, InitJobs jobs, int n) {
     grid_wait();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x, l = blockIdx.y;
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) * V, l = blockIdx.y;
     if (i >= n) return;
-    jobs.hprev[l][i] = __float2bfloat16_rn(h_init[(size_t)l * n + i]);
-    jobs.cprev[l][i] = c_init[(size_t)l * n + i];
+    const float *h = h_init + (size_t)l * n + i, *c = c_init + (size_t)l * n + i;
+    if constexpr (V == 4) {
+        const float4 hv = *reinterpret_cast<const float4 *>(h);
+        *reinterpret_cast<uint2 *>(jobs.hprev[l] + i) = make_uint2(pack_bf16x2(hv.x, hv.y), pack_bf16x2(hv.z, hv.w));
+        *reinterpret_cast<float4 *>(jobs.cprev[l] + i) = *reinterpret_cast<const float4 *>(c);
+    } else {
+        jobs.hprev[l][i] = __float2bfloat16_rn(*h);
+        jobs.cprev[l][i] = *c;
+    }
+}
+static int lstm_init(const float *h_init, const float *c_init, const InitJobs &jobs, int layers, int n, cudaStream_t st) {
+    const bool wide = n % 4 == 0 && ppo_aligned(h_init, 16) && ppo_aligned(c_init, 16);
+    return ppo_launch(wide ? lstm_init_kernel<4> : lstm_init_kernel<1>, dim3(ppo_cdiv(n, wide ? 1024 : 256), layers), dim3(256), 0, st, h_init,
+                      c_init, jobs, n);
 }
 
 // One time step of one LSTM layer for Be envs, element-wise part: gate pre-activations = xg + hg + b,
@@ -1195,8 +1209,7 @@ static int lstm_forward(ppo_model *m, int rows, cudaStream_t st) {
                     jobs.hprev[k] = m->lstm_hprev[k];
                     jobs.cprev[k] = m->lstm_c[k] + (size_t)m->mbmax * H;
                 }
-                PPO_TRY(ppo_launch(lstm_init_kernel, dim3(ppo_cdiv((long long)Be * H, 256), d.n_lstm), dim3(256), 0, st, m->seq_h_init, m->seq_c_init,
-                                   jobs, Be * H));
+                PPO_TRY(lstm_init(m->seq_h_init, m->seq_c_init, jobs, d.n_lstm, Be * H, st));
                 started = true;
             }
             PlanKey k = plan_key(OP_LSTM_STEP, fc_geom(Be, in, l));
@@ -1218,8 +1231,7 @@ static int lstm_forward(ppo_model *m, int rows, cudaStream_t st) {
             InitJobs job;
             job.hprev[0] = m->lstm_hprev[l];
             job.cprev[0] = cprev;
-            PPO_TRY(ppo_launch(lstm_init_kernel, dim3(ppo_cdiv((long long)Be * H, 256)), dim3(256), 0, st, m->seq_h_init + (size_t)l * Be * H,
-                               m->seq_c_init + (size_t)l * Be * H, job, Be * H));
+            PPO_TRY(lstm_init(m->seq_h_init + (size_t)l * Be * H, m->seq_c_init + (size_t)l * Be * H, job, 1, Be * H, st));
         }
         for (int t = 0; t < T; ++t) {
             const size_t r0 = (size_t)t * Be;

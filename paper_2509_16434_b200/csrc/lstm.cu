@@ -828,7 +828,7 @@ int lstm_fwd_steps(const LstmSteps &p, const bf16 *Wh, const float *xg, const fl
     int ctas = 0, U = 1;
     size_t smem = 0;
     while (U <= 4 && !plan(a, p.T, p.Be, p.H, U, ctas, smem)) U *= 2;
-    if (!status || U > 4) return PPO_ERR_UNSUPPORTED;
+    if (!status || U > 4 || !ppo_aligned(h_init, 16) || !ppo_aligned(c_init, 16)) return PPO_ERR_UNSUPPORTED;
     const long long H = p.H;
     const long long db[2] = {H, 4 * H}, sb[1] = {2 * H};
     const int bb[2] = {64, 16};
