@@ -673,6 +673,9 @@ struct WArgs {
     int32_t *status;
 };
 
+// ADD: the reduction is not split, and the epilogue adds the tile to dW itself (a kernel of its own: its registers would take the
+// place of the first layer's gradient, which runs beside the split ones).
+template <bool ADD>
 __global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_constant__ WArgs a) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -809,27 +812,44 @@ __global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_con
         __syncwarp();
         // ---------------- epilogue: TMEM lane p is row p of this CTA's 128 x BN tile of dW^T; the whole tile goes
         // to the CTA's slot of the scratch array, column by column (a warp's store covers 32 consecutive rows).  The only split
-        // of a reduction adds it to dW itself, the same sum without the trip (1024 x 4096 weights: a reduction of 25 us less).
+        // of a reduction adds it to dW itself, the same sum without the trip (1024 x 4096 weights of 4096 rows: 35 us and a reduction
+        // of 25 -> 46).
         const int lg = warp & 3;
         const int p = lg * 32 + lane;
-        if (nkb > 0 && ok && mbar_wait(&pipe->tfull, 0, abort_flag, a.status)) {
+        if constexpr (ADD) {
+            // 64 columns of dW a trip, fetched a trip ahead (16 at a time, when they are needed, take 4 us longer)
+            const int jj = (int)blockIdx.x * 128 + p;
+            float *const d = a.dW + (size_t)co0 * a.Kfwd + jj;
+            const int cols = jj < a.Kfwd ? min(BN, a.Co - co0) : 0;
+            float o[64];
+            auto fetch = [&](int c0) {
+#pragma unroll
+                for (int i = 0; i < 64; ++i) o[i] = c0 + i < cols ? __ldcg(d + (size_t)(c0 + i) * a.Kfwd) : 0.f;
+            };
+            fetch(0);
+            if (nkb > 0 && ok && mbar_wait(&pipe->tfull, 0, abort_flag, a.status)) {
+                tc_fence_after();
+                const uint32_t lane_base = tmem_d + ((uint32_t)(lg * 32) << 16);
+                for (int c0 = 0; c0 < BN; c0 += 64) {
+                    float v[64];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (c0 + 16 * q < BN) tmem_ld16(lane_base + (uint32_t)(c0 + 16 * q), v + 16 * q);
+#pragma unroll
+                    for (int i = 0; i < 64; ++i) v[i] += o[i];
+                    if (c0 + 64 < BN) fetch(c0 + 64);
+#pragma unroll
+                    for (int i = 0; i < 64; ++i)
+                        if (c0 + i < cols) d[(size_t)(c0 + i) * a.Kfwd] = v[i];
+                }
+            }
+        } else if (nkb > 0 && ok && mbar_wait(&pipe->tfull, 0, abort_flag, a.status)) {
             tc_fence_after();
             float *tile = a.part + ((size_t)(blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * (size_t)(128 * BN);
             const uint32_t lane_base = tmem_d + ((uint32_t)(lg * 32) << 16);
             for (int c0 = 0; c0 < BN; c0 += 16) {
                 float v[16];
                 tmem_ld16(lane_base + (uint32_t)c0, v);
-                if (a.dW) {
-                    const int jj = (int)blockIdx.x * 128 + p;
-                    float *d = a.dW + (size_t)(co0 + c0) * a.Kfwd + jj;
-                    float o[16];
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) o[i] = jj < a.Kfwd && co0 + c0 + i < a.Co ? d[(size_t)i * a.Kfwd] : 0.f;
-#pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        if (jj < a.Kfwd && co0 + c0 + i < a.Co) d[(size_t)i * a.Kfwd] = o[i] + v[i];
-                    continue;
-                }
 #pragma unroll
                 for (int i = 0; i < 16; ++i) tile[(c0 + i) * 128 + p] = v[i];
             }
@@ -1069,7 +1089,8 @@ int ensure_smem_attrs() {
         PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_kmajor_kernel<KIND_FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
         PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_kmajor_kernel<KIND_DGRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
         PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_kmajor_kernel<KIND_DGRAD_ACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
-        PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
+        PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_wgrad_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
+        PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_wgrad_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
         attr_set[dev] = true;
     }
     return PPO_OK;
@@ -1507,8 +1528,10 @@ int tma_gemm_wgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *X, fl
     a.tiles_per_split = (a.grid.tiles + splits - 1) / splits;
     splits = (a.grid.tiles + a.tiles_per_split - 1) / a.tiles_per_split;  // every split has at least one pixel tile
     dim3 grid((unsigned)jtiles, (unsigned)ctiles, (unsigned)splits);
-    if (splits == 1 && !db && !pair) a.dW = dW;
-    PPO_TRY(ppo_launch(tma_wgrad_kernel, dim3(grid), dim3(kThreads), (size_t)a.stages * stage + sizeof(Pipe) + 1024, st, a));
+    // Not split because there are tiles enough: added right away.  Not split because there are few rows: the reduction is a launch
+    // of 3 us, and a lone tile's trips to dW take longer (2 x 4 tiles of 72 rows 7 + 3 us, added 16).
+    if (splits == 1 && !db && !pair && 2 * jtiles * ctiles >= ppo_num_sms()) a.dW = dW;
+    PPO_TRY(ppo_launch(a.dW ? tma_wgrad_kernel<true> : tma_wgrad_kernel<false>, dim3(grid), dim3(kThreads), (size_t)a.stages * stage + sizeof(Pipe) + 1024, st, a));
     if (a.dW) return PPO_OK;
     return wgrad_reduce(part, jtiles, ctiles, splits, a.BN, a.Kfwd, g.Co, dW, db,
                         db ? (jtiles - 1) * 128 + a.ones_blk * a.CB : 0, st, pair ? g.Ci : 0);
