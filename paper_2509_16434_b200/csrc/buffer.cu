@@ -668,17 +668,28 @@ __device__ __forceinline__ uint32_t gather_sample(const GatherArgs &g, const Per
     return t * g.N + perm_apply(p, g.start + e);
 }
 
-// The row's small fields, by one CTA of the row.
-__device__ __forceinline__ void gather_small(const GatherArgs &g, uint32_t row, uint32_t s) {
+// The row's small fields, by one CTA of the row: a thread's value of sample s, and its place in row `row`.
+__device__ __forceinline__ float small_load(const GatherArgs &g, uint32_t s) {
     const int t = threadIdx.x;
-    if (t < g.P) g.o_proprio[(size_t)row * g.P + t] = g.proprio[(size_t)s * g.P + t];
-    if (t >= 64 && t < 64 + g.A) g.o_action[(size_t)row * g.A + (t - 64)] = g.action[(size_t)s * g.A + (t - 64)];
-    if (t == 128) g.o_logp[row] = g.logp[s];
-    if (t == 129) g.o_value[row] = g.value[s];
-    if (t == 130) g.o_adv[row] = g.adv[s];
-    if (t == 131) g.o_ret[row] = g.ret[s];
+    if (t < g.P) return g.proprio[(size_t)s * g.P + t];
+    if (t >= 64 && t < 64 + g.A) return g.action[(size_t)s * g.A + (t - 64)];
+    if (t == 128) return g.logp[s];
+    if (t == 129) return g.value[s];
+    if (t == 130) return g.adv[s];
+    if (t == 131) return g.ret[s];
+    if (t == 133 && g.o_done) return __uint_as_float(g.done[s]);
+    return 0.f;
+}
+__device__ __forceinline__ void small_store(const GatherArgs &g, uint32_t row, uint32_t s, float v) {
+    const int t = threadIdx.x;
+    if (t < g.P) g.o_proprio[(size_t)row * g.P + t] = v;
+    if (t >= 64 && t < 64 + g.A) g.o_action[(size_t)row * g.A + (t - 64)] = v;
+    if (t == 128) g.o_logp[row] = v;
+    if (t == 129) g.o_value[row] = v;
+    if (t == 130) g.o_adv[row] = v;
+    if (t == 131) g.o_ret[row] = v;
     if (t == 132 && g.o_index) g.o_index[row] = s;
-    if (t == 133 && g.o_done) g.o_done[row] = g.done[s];
+    if (t == 133 && g.o_done) g.o_done[row] = (uint8_t)__float_as_uint(v);
 }
 
 // Bytes Q * 4 + h / 8 .. + 16 of the 32 bytes a | b (h = 0 or 16 bits).
@@ -701,13 +712,13 @@ constexpr uint32_t kGatherUnits = 1024;  // 16-byte units a CTA moves: four per 
 // the CTA.  Measured: 5.9 -> 6.4 TB/s at 32768 rows of 160 x 120; persistent CTAs that work out the next sample between
 // loads and stores, or several chunks per CTA, are slower.
 // RAGGED: frames whose byte count is no multiple of 16.  Source and destination of a row are then misaligned against
-// each other by some even number of bytes: every aligned unit of the destination is assembled from two aligned loads
-// (the second one hits L1: the neighbouring thread fetched it), counted from a 128-byte line so that a warp stores whole
-// lines; the few bytes in front of the first and behind the last whole unit go as single pixels.  The loads stay inside
+// each other by some even number of bytes: every aligned unit of the destination is assembled from two aligned units of
+// the source (the second one is the neighbouring lane's, for the last lane a load that hits L1), counted from a 128-byte line so
+// that a warp stores whole lines; the few bytes in front of the first and behind the last whole unit go as single pixels.  The loads stay inside
 // the depth slab, which is padded to 256 bytes and followed by others.  Measured: 82 -> 61 us for 6700 rows of 90 x 122
-// against a pixel per access.
+// against a pixel per access, 50 with eight blocks per SM (the second unit in registers of its own made it five).
 template <bool RAGGED>
-__global__ void __launch_bounds__(256) gather_kernel(const __grid_constant__ GatherArgs g, const __grid_constant__ PermParams p) {
+__global__ void __launch_bounds__(256, 8) gather_kernel(const __grid_constant__ GatherArgs g, const __grid_constant__ PermParams p) {
     grid_wait();
     const uint32_t row = blockIdx.x / g.chunks, chunk = blockIdx.x - row * g.chunks;
     __shared__ uint32_t s_sample;
@@ -734,32 +745,44 @@ __global__ void __launch_bounds__(256) gather_kernel(const __grid_constant__ Gat
     const uint4 *src16 = reinterpret_cast<const uint4 *>(src + lead - shift);
     uint4 *dst16 = reinterpret_cast<uint4 *>(dst + lead);
     const int t0 = u0 + (int)threadIdx.x;
-    uint4 a[4], b[4];
+    uint4 a[4];
+    const int last = RAGGED && shift ? hi : hi - 1;  // the unit behind the last one supplies its rest
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const int u = t0 + 256 * k;
-        if (u >= lo && u < hi) {
-            if (RAGGED) {
-                a[k] = __ldg(src16 + u);
-                if (shift) b[k] = __ldg(src16 + u + 1);
-            } else {
-                a[k] = __ldcs(src16 + u);
-            }
-        }
+        if (u >= lo && u <= last) a[k] = RAGGED ? __ldg(src16 + u) : __ldcs(src16 + u);
+    }
+    // Ragged frames are small ones as well: the small fields and the ends of the frame are under way with the rest, behind it they
+    // would be another trip to memory (4.35 -> 4.57 TB/s for 49 x 66).  Whole ones are bound by HBM and lose 1 %.
+    const int t = threadIdx.x;
+    const size_t done = (size_t)lead + (size_t)units * 16;
+    float small = 0.f;
+    uint32_t ends = 0;  // a pixel of the head and one of the tail
+    if (RAGGED && chunk == 0) {
+        small = small_load(g, s);
+        if (2 * t < lead) ends = reinterpret_cast<const uint16_t *>(src)[t];
+        if (2 * t < tail) ends |= (uint32_t)reinterpret_cast<const uint16_t *>(src + done)[t] << 16;
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const int u = t0 + 256 * k;
-        if (u >= lo && u < hi) __stcs(dst16 + u, RAGGED && shift ? window16(a[k], b[k], shift >> 2, (shift & 2u) * 8u) : a[k]);
+        if (RAGGED && shift) {
+            uint4 b = make_uint4(__shfl_down_sync(0xffffffffu, a[k].x, 1), __shfl_down_sync(0xffffffffu, a[k].y, 1),
+                                 __shfl_down_sync(0xffffffffu, a[k].z, 1), __shfl_down_sync(0xffffffffu, a[k].w, 1));
+            if (u >= lo && u < hi) {
+                if ((threadIdx.x & 31) == 31) b = __ldg(src16 + u + 1);
+                __stcs(dst16 + u, window16(a[k], b, shift >> 2, (shift & 2u) * 8u));
+            }
+        } else if (u >= lo && u < hi) {
+            __stcs(dst16 + u, a[k]);
+        }
     }
     if (chunk == 0) {
         if (RAGGED) {
-            const int t = threadIdx.x;
-            if (2 * t < lead) reinterpret_cast<uint16_t *>(dst)[t] = reinterpret_cast<const uint16_t *>(src)[t];
-            const size_t done = (size_t)lead + (size_t)units * 16;
-            if (2 * t < tail) reinterpret_cast<uint16_t *>(dst + done)[t] = reinterpret_cast<const uint16_t *>(src + done)[t];
+            if (2 * t < lead) reinterpret_cast<uint16_t *>(dst)[t] = (uint16_t)ends;
+            if (2 * t < tail) reinterpret_cast<uint16_t *>(dst + done)[t] = (uint16_t)(ends >> 16);
         }
-        gather_small(g, row, s);
+        small_store(g, row, s, RAGGED ? small : small_load(g, s));
     }
 }
 
