@@ -704,7 +704,7 @@ int launch_epw(const Args &a, cudaStream_t st) {
 }
 
 int launch(const Args &a, int mode, int GC, cudaStream_t st) {
-    if (mode == FWD) return GC == 64 ? launch_epw<FWD, 64>(a, st) : launch_epw<FWD, 32>(a, st);
+    if (mode == FWD) return GC == 64 ? launch_epw<FWD, 64>(a, st) : (GC == 32 ? launch_epw<FWD, 32>(a, st) : launch_epw<FWD, 16>(a, st));
     if (mode == FWD_LN) return launch_ks<FWD_LN, 32, 4>(a, st);
     return GC == 64 ? launch_epw<DG, 64>(a, st) : (GC == 32 ? launch_epw<DG, 32>(a, st) : launch_epw<DG, 16>(a, st));
 }
@@ -716,7 +716,10 @@ int chunk_of(int C) { return C % 64 == 0 ? 64 : (C % 32 == 0 ? 32 : (C % 16 == 0
 
 int halo_conv_fwd(const ConvGeom &g, const bf16 *X, const bf16 *W, const FwdEpilogue &e, int32_t *status, cudaStream_t st) {
     if (!status || g.k != 3 || g.pad != 1 || g.Hi < 2 || g.Wi < 2) return PPO_ERR_UNSUPPORTED;
-    if (!e.out || (e.ldo && e.ldo != g.Co) || g.Co % 32 != 0 || g.Co > 256) return PPO_ERR_UNSUPPORTED;
+    if (!e.out || (e.ldo && e.ldo != g.Co) || g.Co % 16 != 0 || g.Co > 256) return PPO_ERR_UNSUPPORTED;
+    // Outputs that are no multiple of 32 leave in groups of 16 columns; gate bits and layer normalisation work on 32.  (32 -> 48
+    // channels, 1024 rows of 31 x 38: tap boxes 36 us, here 21; 16 -> 48, 384 rows of 96 x 117: 104 and 52.)
+    if (g.Co % 32 != 0 && (e.out_bits || e.ln_gamma)) return PPO_ERR_UNSUPPORTED;
     const int CB = chunk_of(g.Ci);
     if (CB == 0 || CB != g.Ci || (size_t)9 * g.Ci * g.Co * 2 > 160 * 1024) return PPO_ERR_UNSUPPORTED;
     Args a = {};
@@ -757,7 +760,7 @@ int halo_conv_fwd(const ConvGeom &g, const bf16 *X, const bf16 *W, const FwdEpil
         const int s = make_map_strided(&a.mapW, W, 2, dims, str, box);
         if (s != PPO_OK) return s;
     }
-    const int GC = g.Co % 64 == 0 && !e.ln_gamma ? 64 : 32;
+    const int GC = g.Co % 64 == 0 && !e.ln_gamma ? 64 : (g.Co % 32 == 0 ? 32 : 16);
     const long long dims[4] = {g.Co, g.Wo, g.Ho, g.B};
     const long long str[3] = {2ll * g.Co, 2ll * g.Wo * g.Co, 2ll * g.Ho * g.Wo * g.Co};
     const int box[4] = {GC, a.Wt, a.R, a.I};
