@@ -199,15 +199,17 @@ class Buffer:
         if v is not None:
             return v.detach()
         d = self.desc
-        ptr = lib().ppo_buffer_field_ptr(self.handle, f)
-        off = ptr - self.storage.data_ptr()
-        nbytes = ppo_buffer_field_bytes(d, f)
-        raw = self.storage[off:off + nbytes]
+        off = lib().ppo_buffer_field_ptr(self.handle, f) - self.storage.data_ptr()
         dt = self._DT.get(f, torch.float32)
-        shape = {FIELD_DEPTH: (d.T, d.N, d.H, d.W), FIELD_PROPRIO: (d.T, d.N, d.P), FIELD_ACTION: (d.T, d.N, d.A),
-                 FIELD_SCRATCH: (-1,)}.get(f, (d.T, d.N))
-        self._slabs[f] = raw.view(dt).view(shape)
-        return self._slabs[f].detach()
+        if f == FIELD_DEPTH:
+            shape = (d.T, d.N, d.H, d.W)
+        elif f == FIELD_SCRATCH:
+            shape = (ppo_buffer_field_bytes(d, f) // dt.itemsize,)
+        else:
+            shape = (d.T, d.N, d.P) if f == FIELD_PROPRIO else (d.T, d.N, d.A) if f == FIELD_ACTION else (d.T, d.N)
+        v = torch.empty(0, dtype=dt, device=self.storage.device).set_(self.storage.untyped_storage(), off // dt.itemsize, shape)
+        self._slabs[f] = v
+        return v.detach()
 
 
 def ppo_buffer_write_step(buf: Buffer, t: int, depth, proprio, action, logp, value, reward, done, stream=None):

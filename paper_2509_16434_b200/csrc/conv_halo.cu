@@ -718,7 +718,7 @@ int halo_conv_fwd(const ConvGeom &g, const bf16 *X, const bf16 *W, const FwdEpil
     if (!status || g.k != 3 || g.pad != 1 || g.Hi < 2 || g.Wi < 2) return PPO_ERR_UNSUPPORTED;
     if (!e.out || (e.ldo && e.ldo != g.Co) || g.Co % 16 != 0 || g.Co > 256) return PPO_ERR_UNSUPPORTED;
     // Outputs that are no multiple of 32 leave in groups of 16 columns; gate bits and layer normalisation work on 32.  (32 -> 48
-    // channels, 1024 rows of 31 x 38: tap boxes 36 us, here 21; 16 -> 48, 384 rows of 96 x 117: 104 and 52.)
+    // channels, 1024 rows of 31 x 38: tap boxes 37 us, here 25; 16 -> 48, 384 rows of 96 x 117: 92 and 53.)
     if (g.Co % 32 != 0 && (e.out_bits || e.ln_gamma)) return PPO_ERR_UNSUPPORTED;
     const int CB = chunk_of(g.Ci);
     if (CB == 0 || CB != g.Ci || (size_t)9 * g.Ci * g.Co * 2 > 160 * 1024) return PPO_ERR_UNSUPPORTED;

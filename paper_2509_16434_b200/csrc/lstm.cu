@@ -741,8 +741,14 @@ bool plan(Args &a, int T, int Be, int H, int U, int &ctas, size_t &smem) {
 }
 
 template <typename F>
-int prepare_kernel(F *fn) {
-    PPO_CUDA_CHECK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+int prepare_kernel(F *fn, bool (&set)[64]) {
+    int dev = 0;
+    PPO_CUDA_CHECK(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= 64) return PPO_ERR_CUDA;
+    if (!set[dev]) {
+        PPO_CUDA_CHECK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+        set[dev] = true;
+    }
     return PPO_OK;
 }
 
@@ -764,7 +770,8 @@ int launch_step(StepArgs &a, int in, const LstmSteps &p, const bf16 *X, const bf
     const size_t stage = (size_t)kStepG * (M + 4 * U) * 128, fixed = (size_t)M * U * 16 + sizeof(Pipe) + 1024;
     a.stages = (int)((kSmemMax - fixed) / stage);
     if (a.stages > kMaxStages) a.stages = kMaxStages;
-    PPO_TRY(prepare_kernel(lstm_step_kernel<M, U>));
+    static bool set[64] = {false};
+    PPO_TRY(prepare_kernel(lstm_step_kernel<M, U>, set));
     const unsigned ctas = (unsigned)((Be + M - 1) / M * (H / U));
     return ppo_launch(lstm_step_kernel<M, U>, dim3(ctas), dim3(kThreads), (size_t)a.stages * stage + fixed, st, a);
 }
@@ -795,7 +802,8 @@ int launch_fwd(Args &a, const LstmSteps &p, int ctas, size_t smem, cudaStream_t 
     const long long da[2] = {H, rows}, sa[1] = {2 * H};
     const int ba[2] = {64, tile_envs(U)};
     PPO_TRY(make_map_strided(&a.mapA, p.hprev, 2, da, sa, ba));
-    PPO_TRY(prepare_kernel(lstm_fwd_kernel<U>));
+    static bool set[64] = {false};
+    PPO_TRY(prepare_kernel(lstm_fwd_kernel<U>, set));
     return ppo_launch_together(lstm_fwd_kernel<U>, dim3(ctas), dim3(kThreads), smem, st, a);
 }
 
@@ -812,7 +820,8 @@ int launch_bwd_clusters(Args &a, const LstmSteps &p, bf16 *dg, cudaStream_t st) 
     int ctas = 0;
     size_t smem = 0;
     if (!plan(a, p.T, p.Be, p.H, U, ctas, smem)) return PPO_ERR_UNSUPPORTED;
-    PPO_TRY(prepare_kernel(lstm_bwd_cluster_kernel<U>));
+    static bool set[64] = {false};
+    PPO_TRY(prepare_kernel(lstm_bwd_cluster_kernel<U>, set));
     bool fit = false;
     PPO_TRY(clusters_fit(lstm_bwd_cluster_kernel<U>, ctas, smem, fit));
     if (!fit) return PPO_ERR_UNSUPPORTED;
@@ -862,7 +871,8 @@ int lstm_bwd_steps(const LstmSteps &p, const bf16 *WhT, const float *dtop, bf16 
     if (s != PPO_ERR_UNSUPPORTED) return s;
     plan(a, p.T, p.Be, p.H, 4, ctas, smem);
     PPO_TRY(map_dg(a, p, dg, tile_envs(4)));
-    PPO_TRY(prepare_kernel(lstm_bwd_kernel));
+    static bool set[64] = {false};
+    PPO_TRY(prepare_kernel(lstm_bwd_kernel, set));
     return ppo_launch_together(lstm_bwd_kernel, dim3(ctas), dim3(kThreads), smem, st, a);
 }
 
