@@ -79,3 +79,21 @@ def test_pairs_of_pixels_match_oracle(H, W, N, last, monkeypatch):
     w = synth.Workload("pairs", N, 2, H, W, (16, last), (3, 3), (40,), 1, 2, P=16, A=3)
     monkeypatch.setitem(NETS, "pairs", w)
     conv_stack_matches_oracle("pairs", monkeypatch)
+
+
+# the dense chain at its lines: 32 | 64 | 128 rows per tile in clusters of eight, clusters of four, the most rows it takes and one
+# more (layer by layer); the widest slices it takes (240 columns of a CTA) and the next width, which it leaves to single layers
+@pytest.mark.parametrize("B,fc", [(480, (72, 40)), (481, (200, 120)), (961, (72, 504)), (1921, (960,)), (1921, (968,)), (4224, (40,)),
+                                  (4225, (40,))])
+def test_dense_chain_at_its_lines_matches_oracle(B, fc, monkeypatch):
+    w = synth.Workload("chain", 2 * B, 1, 8, 12, (16, 32), (3, 3), fc, 1, 2, P=40, A=3)
+    monkeypatch.setitem(NETS, "chain", w)
+    conv_stack_matches_oracle("chain", monkeypatch)
+
+
+# 48 outputs: behind 16, 32 and 48 channels, odd extents, rows of several segments, many small images, as the last layer
+@pytest.mark.parametrize("H,W,N,conv", [(17, 22, 6, (16, 48, 32)), (35, 54, 4, (32, 48, 64)), (12, 530, 2, (16, 48)), (14, 18, 60, (48, 48, 16))])
+def test_48_channels_from_halo_tiles_match_oracle(H, W, N, conv, monkeypatch):
+    w = synth.Workload("c48", N, 2, H, W, conv, (3,) * len(conv), (40,), 1, 2, P=16, A=3)
+    monkeypatch.setitem(NETS, "c48", w)
+    conv_stack_matches_oracle("c48", monkeypatch)

@@ -115,3 +115,31 @@ def test_recurrent_acting_stays_within_a_rounding_of_the_sequence():
     assert float(max(d)) <= 2.0 ** -8
     assert torch.equal(got_lp, lp)  # of the action under its own mean: noise and log-sigma only
     assert ppo.ppo_poll_status() == 0
+
+
+# one launch per layer and step in every shape (32 x 8, 32 x 16, 64 x 16, 128 x 16, 128 x 32 envs x units, the last in one wave and in
+# two), ragged tiles, inputs of one, two and three chunks; two launches where the state's pointers are odd
+@pytest.mark.parametrize("n,H,P", [(1, 64, 32), (33, 512, 160), (65, 512, 96), (161, 512, 32), (300, 512, 160), (600, 512, 96), (700, 1024, 32)])
+def test_steps_one_by_one_give_the_bits_of_the_sequence(n, H, P):
+    w = synth.Workload("one", n, 2, 8, 12, (16, 32), (3, 3), (24,), 1, 1, P=P, A=3, n_lstm=2, lstm_h=H)
+    L, md, lay, theta, roll, action, logp, dev = base._setup(w, w.B)
+    ppo = base.ppo
+    roll["done"][0, 1::3] = 1
+    dev["done"] = torch.as_tensor(roll["done"]).to(DEV)
+    zero = torch.zeros_like(dev["eps"][0])  # actions are then the means
+    got = []
+    for t in range(w.T):
+        got.append(L.act(dev["depth"][t], dev["proprio"][t], zero))
+        L.reset_rollout_state(n, dev["done"][t])
+    mean, value = (torch.cat([g[i] for g in got]) for i in (0, 2))
+    rows = w.T * n
+    seq = ppo.Minibatch(dev["depth"].data_ptr(), dev["proprio"].data_ptr(), None, None, None, None, None, None, rows)
+    odd = [torch.zeros(L.h_init.numel() + 1, device=DEV)[1:].view_as(L.h_init) for _ in range(2)]
+    for h0, c0 in ((torch.zeros_like(L.h_init), torch.zeros_like(L.c_init)), odd):
+        ppo.ppo_model_set_sequence(L.model, w.T, n, dev["done"], h0, c0)
+        ppo.ppo_encoder_fwd(L.model, seq, 0, rows, L.mean, L.value)
+        assert torch.equal(mean, L.mean[:rows]) and torch.equal(value, L.value[:rows])
+    zero_state = np.zeros((w.n_lstm, n, H), np.float32)
+    mu, V, _, _ = orc.encoder_fwd_seq(md, orc.round_weights(md, theta), roll["depth"], roll["proprio"], roll["done"], zero_state, zero_state, True)
+    assert ppo.ppo_poll_status() == 0
+    assert rel_l2(mean.cpu().numpy(), mu) <= ENC_TOL and rel_l2(value.cpu().numpy(), V) <= ENC_TOL
