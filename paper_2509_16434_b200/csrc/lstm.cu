@@ -564,7 +564,7 @@ __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(kThreads, 1) lstm_bw
 // (4 U columns, gate g of unit j at g U + j) run through one pipeline into two accumulators, and the cell works on their sum.
 // Separate launches for W_x x and the step had each its own pipeline to fill, and 512 envs x 1024 units, too many for the
 // time loop, took four of them.  What bounds it: the bytes a CTA pulls through L2 (M + 4 U rows of every chunk).
-// Measured (us per layer): 16 envs x 1024 units 16.7 -> 7.4; 512 envs x 1024 units 32 -> 19.
+// Measured (us per layer): 16 envs x 1024 units 16.7 -> 7.7; 512 envs x 1024 units 32 -> 19.
 struct StepArgs {
     CUtensorMap mapX, mapH, mapWx, mapWh;
     int Be, H;

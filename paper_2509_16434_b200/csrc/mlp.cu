@@ -5,8 +5,8 @@
 // cluster of 4 or 8 CTAs: a CTA owns a slice of each layer's columns, weights stream into their own ring of stages
 // without waiting for anybody, and between two layers the CTAs of the cluster exchange their columns through L2, a release, an
 // arrival at each other's barriers and an acquire: some 2500 cycles instead of a kernel boundary.
-// Measured (us, separate launches -> here): 16 rows 1024-512-512-256-13 28 -> 14; 1024 rows 96-256-13 15 -> 9; 4096 rows
-// 288-512-512-13 35 -> 21, and back 37 -> 22.
+// Measured (us, separate launches -> here): 16 rows 1024-512-512-256-13 25 -> 16.5; 1024 rows 96-256-13 15 -> 8.7, and back
+// 13 -> 8.2; 4096 rows 64-512-512-256-13 37 -> 21 each way.
 // Sums run in the order of the separate kernels (gemm_tma.cu): same bits.
 //
 // Every wait is bounded: on a time-out the kernel records PPO_ERR_TIMEOUT, waits (bounded) for its copies, frees its
