@@ -662,7 +662,7 @@ struct WArgs {
     int CB, rbA, mblocks, kchunks;  // A: channels per box, row bytes, boxes per 128 columns, boxes per tap
     int CBn, rbB, nblocks, BN;      // B: likewise over the output channels of this tile
     int Kfwd, Co;
-    int tiles_per_split, nmma, stages;
+    int tiles_per_split, nmma, stages, jtiles;
     float *part;                    // partial tiles [split][column tile][row tile][BN][128] fp32
     float *dW;                      // not split: the tile is added to dW right away (else null)
     // Bias gradient db[co] += sum over pixels of dY, or null.  The last column tile has an A block that no tap
@@ -675,14 +675,21 @@ struct WArgs {
 
 // ADD: the reduction is not split, and the epilogue adds the tile to dW itself (a kernel of its own: its registers would take the
 // place of the first layer's gradient, which runs beside the split ones).
-template <bool ADD>
-__global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_constant__ WArgs a) {
-    extern __shared__ __align__(1024) uint8_t smem_raw[];
+//
+// PAIR: two CTAs of a cluster take neighbouring column tiles as one 256-row product (cta_group::2): each fetches its 128 columns of
+// X and half of dY's BN, and the MMAs, issued by the first CTA, read both halves.  What bounds the single form at BN = 256: a trip
+// of 16 pixels reads 12 KB of shared memory in the 128 cycles of its MMA while as much comes in, 1.5 times what it delivers,
+// and an SM takes in some 50 bytes a clock where 96 would be used up; half of dY less makes both 64.  The sums keep their order.
+// Measured (us, single -> pair): 128 -> 256 channels, 4096 rows of 8 x 10 outputs 208 -> 135, of 15 x 20 704 -> 532; 256 -> 256
+// of 8 x 10 394 -> 290; 128 -> 128, 1024 rows of 15 x 20 132 -> 114; 1024 x 4096 weights of 4096 rows 46 -> 40.
+template <bool ADD, bool PAIR>
+__device__ __forceinline__ void wgrad_body(const WArgs &a, uint8_t *smem_raw) {
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int BN = a.BN, S = a.stages;
     const uint32_t rbA = (uint32_t)a.rbA, rbB = (uint32_t)a.rbB;
     const uint32_t a_bytes = 128u * 256u;                 // 128 pixel rows x 128 columns of bf16
-    const uint32_t stage_bytes = a_bytes + 128u * 2u * (uint32_t)BN;
+    const uint32_t stage_bytes = a_bytes + 128u * (PAIR ? 1u : 2u) * (uint32_t)BN;
+    const uint32_t rank = PAIR ? blockIdx.x & 1u : 0u;
     Pipe *pipe = reinterpret_cast<Pipe *>(smem + (size_t)S * stage_bytes);
     volatile int *abort_flag = &pipe->abort_flag;
     const int warp = warp_index(), lane = threadIdx.x & 31;
@@ -703,7 +710,7 @@ __global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_con
         const uint32_t n16 = (uint32_t)S * stage_bytes / 16u;
         for (uint32_t i = threadIdx.x; i < n16; i += kThreads) z[i] = make_uint4(0, 0, 0, 0);
     }
-    const bool ones_tile = a.has_db && blockIdx.x == gridDim.x - 1;
+    const bool ones_tile = a.has_db && (int)blockIdx.x == a.jtiles - 1;
     if (ones_tile) {
         // channel 0 of block ones_blk, all 128 pixel rows of every stage: the first element of 16-byte piece 0,
         // which the swizzle moves to piece (row & 7) of a 128-byte row, ((row >> 1) & 3) of a 64-byte row,
@@ -717,10 +724,18 @@ __global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_con
         }
     }
     fence_async_smem();
-    if (warp == 0) tmem_alloc(&pipe->tmem_slot, ncols);
+    if (warp == 0) {
+        if constexpr (PAIR) tmem_alloc_pair(&pipe->tmem_slot, ncols);
+        else tmem_alloc(&pipe->tmem_slot, ncols);
+    }
     grid_wait();
     tc_fence_before();
-    __syncthreads();
+    if constexpr (PAIR) {
+        __syncthreads();
+        cluster_sync();
+    } else {
+        __syncthreads();
+    }
     tc_fence_after();
     const uint32_t tmem_d = pipe->tmem_slot;
     const uint32_t smem_base = smem_u32(smem);
@@ -734,8 +749,10 @@ __global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_con
     for (int i = 0; i < a.mblocks; ++i)
         if ((jb0 + i) / a.kchunks < a.ntaps) ++nvalid;
 
-    if (warp == 0) {
-        const uint32_t idesc = instr_desc(128, BN, 1, 1);
+    if (PAIR && warp == 0 && rank != 0) {
+        // the other CTA issues for both
+    } else if (warp == 0) {
+        const uint32_t idesc = instr_desc(PAIR ? 256 : 128, BN, 1, 1);
         const uint64_t dA = smem_desc_sw(smem_base, 128u * rbA, 8u * rbA, rbA);
         const uint64_t dB = smem_desc_sw(smem_base + a_bytes, 128u * rbB, 8u * rbB, rbB);
         const uint32_t a_hi = (uint32_t)(dA >> 32), b_hi = (uint32_t)(dB >> 32);
@@ -750,16 +767,21 @@ __global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_con
             if (elect_one()) {
                 uint32_t la = (uint32_t)dA + (uint32_t)s * (stage_bytes >> 4), lb = (uint32_t)dB + (uint32_t)s * (stage_bytes >> 4);
                 for (int k = 0; k < a.nmma; ++k, la += stepA, lb += stepB) {
-                    umma_bf16_lh(tmem_d, la, a_hi, lb, b_hi, idesc, accum);
+                    if constexpr (PAIR) umma_bf16_pair(tmem_d, la, a_hi, lb, b_hi, idesc, accum);
+                    else umma_bf16_lh(tmem_d, la, a_hi, lb, b_hi, idesc, accum);
                     accum = 1u;
                 }
-                umma_commit(&pipe->empty[s]);
+                if constexpr (PAIR) umma_commit_pair(&pipe->empty[s]);
+                else umma_commit(&pipe->empty[s]);
             }
             accum = 1u;
             __syncwarp();
             if (++s == S) { s = 0; ph ^= 1u; }
         }
-        if (ok && nkb > 0 && elect_one()) umma_commit(&pipe->tfull);
+        if (ok && nkb > 0 && elect_one()) {
+            if constexpr (PAIR) umma_commit_pair(&pipe->tfull);
+            else umma_commit(&pipe->tfull);
+        }
         __syncwarp();
     } else {
         // ---------------- TMA producers: two warps for A and two for B, each with every second stage (S >= 2).  All lanes
@@ -769,7 +791,13 @@ __global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_con
         constexpr int NP = 2;
         const int pw = (warp - 1) & 1;
         const bool sideA = warp <= NP;
-        const uint32_t tx_bytes = (uint32_t)a.grid.arows * (sideA ? (uint32_t)nvalid * rbA : (uint32_t)a.nblocks * rbB);
+        // (a pair's copies all count at the first CTA's barriers, which expect both CTAs' bytes)
+        int nboth = nvalid;
+        if constexpr (PAIR)
+            for (int i = 0; i < a.mblocks; ++i)
+                if ((((int)blockIdx.x ^ 1) * a.mblocks + i) / a.kchunks < a.ntaps) ++nboth;
+        const uint32_t tx_bytes = (uint32_t)a.grid.arows * (sideA ? (uint32_t)nboth * rbA : (uint32_t)a.nblocks * rbB);
+        const int nb = PAIR ? a.nblocks / 2 : a.nblocks, c0b = co0 + (PAIR ? (int)rank * (BN / 2) : 0);
         const int tap0 = jb0 / a.kchunks, kc0 = jb0 - tap0 * a.kchunks, kh0 = tap0 / a.ksz, kw0 = tap0 - kh0 * a.ksz;
         bool ok = true;
         int kb = pw, s = pw;
@@ -782,7 +810,8 @@ __global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_con
             const int x0 = pt.xs * a.grid.Wt;
             ok = mbar_wait_warp(&pipe->empty[s], ph ^ 1u, abort_flag, a.status);
             if (!ok) break;
-            if (elect_one()) mbar_arrive_expect_tx(&pipe->full[s], tx_bytes);
+            if (rank == 0 && elect_one()) mbar_arrive_expect_tx(&pipe->full[s], tx_bytes);
+            const uint32_t full = PAIR ? in_cta(smem_u32(&pipe->full[s]), 0) : smem_u32(&pipe->full[s]);
             int n = pt.n, y = pt.y, row = 0;
             while (row < a.grid.R) {
                 const int seg = min(a.grid.Hr - y, a.grid.R - row);
@@ -791,15 +820,15 @@ __global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_con
                 int kc = kc0, kh = kh0, kw = kw0;
                 for (int i = 0; sideA && i < nvalid; ++i) {
                     if (elect_one())
-                        tma_load_4d(st + ((uint32_t)i * 128u + off) * rbA, &a.mapA[seg - 1], &pipe->full[s], kc * a.CB, cx + kw, cy + kh, n);
+                        tma_load_at<PAIR>(st + ((uint32_t)i * 128u + off) * rbA, &a.mapA[seg - 1], full, kc * a.CB, cx + kw, cy + kh, n);
                     if (++kc == a.kchunks) {
                         kc = 0;
                         if (++kw == a.ksz) { kw = 0; ++kh; }
                     }
                 }
-                for (int i = 0; !sideA && i < a.nblocks; ++i)
+                for (int i = 0; !sideA && i < nb; ++i)
                     if (elect_one())
-                        tma_load_4d(st + a_bytes + ((uint32_t)i * 128u + off) * rbB, &a.mapB[seg - 1], &pipe->full[s], co0 + i * a.CBn, x0, y, n);
+                        tma_load_at<PAIR>(st + a_bytes + ((uint32_t)i * 128u + off) * rbB, &a.mapB[seg - 1], full, c0b + i * a.CBn, x0, y, n);
                 row += seg;
                 y += seg;
                 if (y >= a.grid.Hr) { y = 0; ++n; }
@@ -808,7 +837,15 @@ __global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_con
             s += NP;
             if (s >= S) { s -= S; ph ^= 1u; }
         }
-        if (!ok && lane == 0) drain_copies(pipe->full, kb, S, pw, NP);
+        if constexpr (PAIR) {
+            if (!ok) {  // copies in flight count at the other CTA: they land meanwhile
+                const long long t0 = clock64();
+                while (clock64() - t0 < 200000) {
+                }
+            }
+        } else {
+            if (!ok && lane == 0) drain_copies(pipe->full, kb, S, pw, NP);
+        }
         __syncwarp();
         // ---------------- epilogue: TMEM lane p is row p of this CTA's 128 x BN tile of dW^T; the whole tile goes
         // to the CTA's slot of the scratch array, column by column (a warp's store covers 32 consecutive rows).  The only split
@@ -843,9 +880,9 @@ __global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_con
                         if (c0 + i < cols) d[(size_t)(c0 + i) * a.Kfwd] = v[i];
                 }
             }
-        } else if (nkb > 0 && ok && mbar_wait(&pipe->tfull, 0, abort_flag, a.status)) {
+        } else if (nkb > 0 && ok && mbar_wait(&pipe->tfull, 0, abort_flag, a.status) && (!PAIR || (int)blockIdx.x < a.jtiles)) {
             tc_fence_after();
-            float *tile = a.part + ((size_t)(blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * (size_t)(128 * BN);
+            float *tile = a.part + ((size_t)(blockIdx.z * gridDim.y + blockIdx.y) * (size_t)a.jtiles + blockIdx.x) * (size_t)(128 * BN);
             const uint32_t lane_base = tmem_d + ((uint32_t)(lg * 32) << 16);
             for (int c0 = 0; c0 < BN; c0 += 16) {
                 float v[16];
@@ -857,10 +894,22 @@ __global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_con
     }
     tc_fence_before();
     __syncthreads();
+    if constexpr (PAIR) cluster_sync();
     if (warp == 0) {
         tc_fence_after();
-        tmem_dealloc(tmem_d, ncols);
+        if constexpr (PAIR) tmem_dealloc_pair(tmem_d, ncols);
+        else tmem_dealloc(tmem_d, ncols);
     }
+}
+template <bool ADD>
+__global__ void __launch_bounds__(kThreads, 1) tma_wgrad_kernel(const __grid_constant__ WArgs a) {
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    wgrad_body<ADD, false>(a, smem_raw);
+}
+template <bool ADD>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) tma_wgrad_pair_kernel(const __grid_constant__ WArgs a) {
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    wgrad_body<ADD, true>(a, smem_raw);
 }
 
 // dW[co][jj] += sum over the splits, in their order, of the partial tiles a split-K weight-gradient kernel left
@@ -1091,6 +1140,8 @@ int ensure_smem_attrs() {
         PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_kmajor_kernel<KIND_DGRAD_ACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
         PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_wgrad_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
         PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_wgrad_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
+        PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_wgrad_pair_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
+        PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_wgrad_pair_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
         attr_set[dev] = true;
     }
     return PPO_OK;
@@ -1528,10 +1579,22 @@ int tma_gemm_wgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *X, fl
     a.tiles_per_split = (a.grid.tiles + splits - 1) / splits;
     splits = (a.grid.tiles + a.tiles_per_split - 1) / a.tiles_per_split;  // every split has at least one pixel tile
     dim3 grid((unsigned)jtiles, (unsigned)ctiles, (unsigned)splits);
+    a.jtiles = jtiles;
     // Not split because there are tiles enough: added right away.  Not split because there are few rows: the reduction is a launch
     // of 3 us, and a lone tile's trips to dW take longer (2 x 4 tiles of 72 rows 7 + 3 us, added 16).
     if (splits == 1 && !db && !pair && 2 * jtiles * ctiles >= ppo_num_sms()) a.dW = dW;
-    PPO_TRY(ppo_launch(a.dW ? tma_wgrad_kernel<true> : tma_wgrad_kernel<false>, dim3(grid), dim3(kThreads), (size_t)a.stages * stage + sizeof(Pipe) + 1024, st, a));
+    // In pairs where their CTAs still fit at once (an odd number of column tiles adds an empty one; the splits stay, for the order of
+    // the sums) and there is something to save: with 5 tiles of pixels per CTA both take 10 us, with one or two a pair is 1 us longer.
+    const int jpairs = (jtiles + 1) / 2;
+    if (!two && a.BN >= 128 && a.nblocks % 2 == 0 && a.tiles_per_split >= 16 && 2ll * jpairs * ctiles * splits <= ppo_num_sms()) {
+        const size_t half = (size_t)128 * 256 + (size_t)128 * a.BN;
+        a.stages = stages_for(half);
+        if (a.stages > kMaxStages) a.stages = kMaxStages;
+        grid.x = 2u * (unsigned)jpairs;
+        PPO_TRY(ppo_launch(a.dW ? tma_wgrad_pair_kernel<true> : tma_wgrad_pair_kernel<false>, dim3(grid), dim3(kThreads), (size_t)a.stages * half + sizeof(Pipe) + 1024, st, a));
+    } else {
+        PPO_TRY(ppo_launch(a.dW ? tma_wgrad_kernel<true> : tma_wgrad_kernel<false>, dim3(grid), dim3(kThreads), (size_t)a.stages * stage + sizeof(Pipe) + 1024, st, a));
+    }
     if (a.dW) return PPO_OK;
     return wgrad_reduce(part, jtiles, ctiles, splits, a.BN, a.Kfwd, g.Co, dW, db,
                         db ? (jtiles - 1) * 128 + a.ones_blk * a.CB : 0, st, pair ? g.Ci : 0);

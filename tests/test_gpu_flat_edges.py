@@ -97,3 +97,13 @@ def test_48_channels_from_halo_tiles_match_oracle(H, W, N, conv, monkeypatch):
     w = synth.Workload("c48", N, 2, H, W, conv, (3,) * len(conv), (40,), 1, 2, P=16, A=3)
     monkeypatch.setitem(NETS, "c48", w)
     conv_stack_matches_oracle("c48", monkeypatch)
+
+
+# weight gradients in pairs of column tiles (148 SMs): 15 tiles of pixels per CTA (single) and 16 (pairs) with a ragged last one, the
+# bias in a tile of its own, in a free block (192 inputs) and beside an empty tile (256), two groups of output columns (512)
+@pytest.mark.parametrize("H,N,conv", [(64, 420, (32, 128, 128)), (64, 421, (32, 128, 128)), (32, 1290, (64, 192, 128)),
+                                      (64, 215, (32, 128, 512)), (64, 850, (32, 64, 256, 256))])
+def test_pairs_of_column_tiles_match_oracle(H, N, conv, monkeypatch):
+    w = synth.Workload("cpairs", N, 1, H, H, conv, (3,) * len(conv), (40,), 1, 1, P=16, A=3)
+    monkeypatch.setitem(NETS, "cpairs", w)
+    conv_stack_matches_oracle("cpairs", monkeypatch)
