@@ -118,8 +118,8 @@ __device__ void drain_copies(uint64_t *full, int it, int S, int first, int np) {
 // that consecutive tiles of a CTA share their pixel tile (the classes of a dgrad) or at least neighbour it.
 struct TileCursor {
     int g, g_end, mt, nt, c;
-    __device__ void init(int total, int tiles_n, int ncls) {
-        const int q = total / (int)gridDim.x, r = total - q * (int)gridDim.x, b = (int)blockIdx.x;
+    __device__ void init(int total, int tiles_n, int ncls, int b, int ctas) {
+        const int q = total / ctas, r = total - q * ctas;
         g = b * q + (b < r ? b : r);
         g_end = g + q + (b < r ? 1 : 0);
         c = g % ncls;
@@ -167,6 +167,7 @@ struct KArgs {
     int tmem_cap;           // tensor-memory columns this CTA may take: 512, or 256 when two CTAs share an SM
     int nepi;               // epilogue warps: 8, or 16 where the epilogue is the heavier side (dgrad with gates)
     int nprod;              // producer warps: 1 .. min(kProducers, stages)
+    int pair;               // tiles in pairs, see the kernel
     int wres, wtaps;        // weights resident in shared memory (all wtaps * kchunks boxes, loaded once)
     int N, BN, tiles_n, total_tiles, ncls, stages;  // tile g = ((mt * tiles_n) + nt) * ncls + class
     int Hout, Wout, ldo;
@@ -204,13 +205,22 @@ struct PipeK {
 // registers of the widest epilogue would spill the others'.
 enum { KIND_FWD = 0, KIND_DGRAD = 1, KIND_DGRAD_ACT = 2 };
 
-template <int KIND>
-__global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_constant__ KArgs a) {
-    extern __shared__ __align__(1024) uint8_t smem_raw[];
+//
+// PAIR: two CTAs of a cluster take neighbouring pixel tiles and the same columns as one 256-row product (cta_group::2): each fetches
+// its own pixels and half of the BN weight rows, the MMAs, issued by the first CTA, read both halves, and each drains its own
+// rows.  An odd last tile is paired with one behind the grid, whose copies are zeros and whose rows nobody stores.  Half of the weight
+// rows less in and out of each CTA's shared memory, whose bandwidth is the single form's bound at these widths.  Measured (us,
+// single -> pair): forward 128 -> 256 channels, 4096 rows of 8 x 10 outputs 168 -> 147, of 15 x 20 645 -> 558, 256 -> 256 of 8 x 10
+// 344 -> 288, its input gradient 460 -> 379; forward 128 -> 128, 1024 rows of 15 x 20 135 -> 99.
+template <int KIND, bool PAIR>
+__device__ __forceinline__ void kmajor_body(const KArgs &a, uint8_t *smem_raw) {
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int BN = a.BN, S = a.stages, G = a.G;
     const uint32_t rb = (uint32_t)a.row_bytes;
-    const uint32_t a_bytes = a.a_bytes, b_bytes = (uint32_t)BN * rb;
+    const uint32_t a_bytes = a.a_bytes, b_bytes = (uint32_t)BN * rb / (PAIR ? 2u : 1u);
+    const int rank = PAIR ? (int)blockIdx.x & 1 : 0;
+    const int cta = PAIR ? (int)blockIdx.x >> 1 : (int)blockIdx.x, ctas = PAIR ? (int)gridDim.x >> 1 : (int)gridDim.x;  // of the tile cursor
+    auto tile_of = [&](int mt) { return PAIR ? 2 * mt + rank : mt; };
     const uint32_t sub_bytes = a_bytes + (a.wres ? 0u : b_bytes);
     const uint32_t stage_bytes = (uint32_t)G * sub_bytes;
     // a stage is A and B of sub-block after sub-block, or (batched) all A and behind them all B
@@ -231,13 +241,16 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
         }
         for (int i = 0; i < nacc; ++i) {
             mbar_init(&pipe->tfull[i], 1);
-            mbar_init(&pipe->tempty[i], a.nepi * 32);
+            mbar_init(&pipe->tempty[i], PAIR ? a.nepi * 2 : a.nepi * 32);  // (pair: a thread of each warp of both CTAs)
         }
         mbar_init(&pipe->wfull, 1);
         pipe->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 1) tmem_alloc(&pipe->tmem_slot, ncols);
+    if (warp == 1) {
+        if constexpr (PAIR) tmem_alloc_pair(&pipe->tmem_slot, ncols);
+        else tmem_alloc(&pipe->tmem_slot, ncols);
+    }
     grid_wait();
     if (KIND == KIND_FWD)
         for (int i = threadIdx.x; i < a.tiles_n * BN; i += (int)blockDim.x) pipe->bias[i] = i < a.N ? a.bias[i] : 0.f;
@@ -248,6 +261,7 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
         }
     tc_fence_before();
     __syncthreads();
+    if constexpr (PAIR) cluster_sync();
     tc_fence_after();
     const uint32_t tmem_base = pipe->tmem_slot;
     const uint32_t smem_base = smem_u32(smem);
@@ -256,7 +270,7 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
     if (warp == 0 || warp >= 2 + a.nepi) {
         // ---------------- TMA producers
         const int pw = warp == 0 ? 0 : warp - 1 - a.nepi, np = a.nprod;
-        if (a.wres && pw == 0) {
+        if (!PAIR && a.wres && pw == 0) {
             const int nw = a.wtaps * a.kchunks;
             if (lane == 0) mbar_arrive_expect_tx(&pipe->wfull, (uint32_t)nw * b_bytes);
             __syncwarp();
@@ -266,18 +280,20 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
             }
         }
         // All lanes walk the tiles together, one elected lane issues (see tcgen05.cuh).
-        const uint32_t tx_sub = (uint32_t)a.grid.arows * rb + (a.wres ? 0u : b_bytes);
+        // (a pair's copies all count at the first CTA's barriers, which expect both CTAs' bytes)
+        const uint32_t tx_sub = ((uint32_t)a.grid.arows * rb + (a.wres ? 0u : b_bytes)) * (PAIR ? 2u : 1u);
+        const uint32_t full0 = PAIR ? in_cta(smem_u32(pipe->full), 0) : smem_u32(pipe->full);
         int it = pw, s = pw, it0 = 0;  // it, s: this warp's next stage of the whole run and its slot; it0: first of the tile
         uint32_t ph = 0;
         bool ok = true;
         TileCursor tc_;
-        tc_.init(a.total_tiles, a.tiles_n, a.ncls);
+        tc_.init(a.total_tiles, a.tiles_n, a.ncls, cta, ctas);
         PixTile pt;
-        pt.init(a.grid, tc_.mt);
+        pt.init(a.grid, tile_of(tc_.mt));
         for (; tc_.valid() && ok; tc_.next(a.tiles_n, a.ncls)) {
             const KClass &k = a.cls[tc_.c];
-            pt.advance_to(a.grid, tc_.mt);
-            const int brow = tc_.nt * BN + k.b_row0, ntaps = k.taps.n, nsub = ntaps * a.kchunks;
+            pt.advance_to(a.grid, tile_of(tc_.mt));
+            const int brow = tc_.nt * BN + k.b_row0 + (PAIR ? rank * (BN / 2) : 0), ntaps = k.taps.n, nsub = ntaps * a.kchunks;
             const int cx = pt.xs * a.grid.Wt * a.s_mul + a.s_ox;
             int tap = 0, kc = (it - it0) * G;
             while (!a.batched && kc >= a.kchunks) { kc -= a.kchunks; ++tap; }
@@ -285,9 +301,10 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
                 ok = mbar_wait_warp(&pipe->empty[s], ph ^ 1u, abort_flag, a.status);
                 if (!ok) break;
                 const int nval = a.batched ? 0 : min(G, nsub - q0);
-                if (elect_one()) mbar_arrive_expect_tx(&pipe->full[s], (uint32_t)(a.batched ? G : nval) * tx_sub);
+                if (rank == 0 && elect_one()) mbar_arrive_expect_tx(&pipe->full[s], (uint32_t)(a.batched ? G : nval) * tx_sub);
+                const uint32_t full = full0 + 8u * (uint32_t)s;
                 uint32_t dst = smem_base + (uint32_t)s * stage_bytes;
-                if (a.batched) {  // chunks behind the last arrive as zeros; one kernel tap, one pixel row
+                if (!PAIR && a.batched) {  // chunks behind the last arrive as zeros; one kernel tap, one pixel row
                     if (elect_one()) tma_load_4d(dst, &a.mapA[0], &pipe->full[s], 0, cx, kc, 0);
                     if (!a.wres && elect_one()) tma_load_4d(dst + b_off, &a.mapB, &pipe->full[s], 0, brow, kc, 0);
                     kc += G;
@@ -298,14 +315,14 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
                     while (row < a.grid.R) {  // one box per image the tile touches
                         const int seg = min(a.grid.Hr - y, a.grid.R - row);
                         if (elect_one())
-                            tma_load_4d(dst + (uint32_t)(row * a.grid.Wt) * rb, &a.mapA[seg - 1], &pipe->full[s], kc * a.CB, cx + dx,
-                                        y * a.s_mul + a.s_oy + dy, n);
+                            tma_load_at<PAIR>(dst + (uint32_t)(row * a.grid.Wt) * rb, &a.mapA[seg - 1], full, kc * a.CB, cx + dx,
+                                              y * a.s_mul + a.s_oy + dy, n);
                         row += seg;
                         y += seg;
                         if (y >= a.grid.Hr) { y = 0; ++n; }
                     }
                     if (!a.wres && elect_one())
-                        tma_load_2d(dst + a_bytes, &a.mapB, &pipe->full[s], (int)k.taps.wt[tap] * a.w_tap + kc * a.CB, brow);
+                        tma_load_at<PAIR>(dst + a_bytes, &a.mapB, full, (int)k.taps.wt[tap] * a.w_tap + kc * a.CB, brow);
                     if (++kc == a.kchunks) { kc = 0; ++tap; }
                 }
                 __syncwarp();
@@ -318,12 +335,22 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
             }
             it0 += (nsub + G - 1) / G;
         }
-        if (!ok && lane == 0) drain_copies(pipe->full, it, S, pw, np);
+        if constexpr (PAIR) {
+            if (!ok) {  // copies in flight count at the other CTA: they land meanwhile
+                const long long t0 = clock64();
+                while (clock64() - t0 < 200000) {
+                }
+            }
+        } else {
+            if (!ok && lane == 0) drain_copies(pipe->full, it, S, pw, np);
+        }
         __syncwarp();
+    } else if (PAIR && warp == 1 && rank != 0) {
+        // the other CTA issues for both
     } else if (warp == 1) {
         // ---------------- MMA issue: one elected thread feeds the tensor core; the descriptors are built once and
         // advanced by adds
-        const uint32_t idesc = instr_desc(128, BN, 0, 0);
+        const uint32_t idesc = instr_desc(PAIR ? 256 : 128, BN, 0, 0);
         const uint32_t sbo = 8u * rb;
         const uint64_t d0 = smem_desc_sw(smem_base, 16, sbo, rb);
         const uint32_t d_lo0 = (uint32_t)d0, d_hi = (uint32_t)(d0 >> 32);
@@ -336,7 +363,7 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
         bool ok = true;
         if (a.wres) ok = mbar_wait_warp(&pipe->wfull, 0, abort_flag, a.status);
         TileCursor tc_;
-        for (tc_.init(a.total_tiles, a.tiles_n, a.ncls); tc_.valid() && ok; tc_.next(a.tiles_n, a.ncls), ++ti) {
+        for (tc_.init(a.total_tiles, a.tiles_n, a.ncls, cta, ctas); tc_.valid() && ok; tc_.next(a.tiles_n, a.ncls), ++ti) {
             const int c = tc_.c;
             const int nsub = a.cls[c].taps.n * a.kchunks;
             const int acc = ti & (nacc - 1);
@@ -359,22 +386,33 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
                         if (++kc == a.kchunks) { kc = 0; ++tap; }
                     }
                     if (elect_one()) {
-                        umma_bf16_lh(tmem_d, la, d_hi, lb, d_hi, idesc, accum);
-                        if (ksteps >= 2) umma_bf16_lh(tmem_d, la + 2, d_hi, lb + 2, d_hi, idesc, 1u);
-                        if (ksteps == 4) {
-                            umma_bf16_lh(tmem_d, la + 4, d_hi, lb + 4, d_hi, idesc, 1u);
-                            umma_bf16_lh(tmem_d, la + 6, d_hi, lb + 6, d_hi, idesc, 1u);
+                        if constexpr (PAIR) {  // (rows of 128 bytes)
+                            umma_bf16_pair(tmem_d, la, d_hi, lb, d_hi, idesc, accum);
+                            umma_bf16_pair(tmem_d, la + 2, d_hi, lb + 2, d_hi, idesc, 1u);
+                            umma_bf16_pair(tmem_d, la + 4, d_hi, lb + 4, d_hi, idesc, 1u);
+                            umma_bf16_pair(tmem_d, la + 6, d_hi, lb + 6, d_hi, idesc, 1u);
+                        } else {
+                            umma_bf16_lh(tmem_d, la, d_hi, lb, d_hi, idesc, accum);
+                            if (ksteps >= 2) umma_bf16_lh(tmem_d, la + 2, d_hi, lb + 2, d_hi, idesc, 1u);
+                            if (ksteps == 4) {
+                                umma_bf16_lh(tmem_d, la + 4, d_hi, lb + 4, d_hi, idesc, 1u);
+                                umma_bf16_lh(tmem_d, la + 6, d_hi, lb + 6, d_hi, idesc, 1u);
+                            }
                         }
                     }
                     accum = 1u;
                 }
                 if (elect_one()) {
-                    umma_commit(&pipe->empty[s]);
+                    if constexpr (PAIR) umma_commit_pair(&pipe->empty[s]);
+                    else umma_commit(&pipe->empty[s]);
                 }
                 __syncwarp();
                 if (++s == S) { s = 0; ph ^= 1u; }
             }
-            if (ok && elect_one()) umma_commit(&pipe->tfull[acc]);
+            if (ok && elect_one()) {
+                if constexpr (PAIR) umma_commit_pair(&pipe->tfull[acc]);
+                else umma_commit(&pipe->tfull[acc]);
+            }
             __syncwarp();
         }
     } else {
@@ -385,10 +423,20 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
         const RowGrid &gr = a.grid;
         int ti = 0;
         bool ok = true;
+        // This warp is done with an accumulator.
+        auto release = [&](int acc) {
+            tc_fence_before();
+            if constexpr (PAIR) {
+                __syncwarp();
+                if (lane == 0) arrive_at(in_cta(smem_u32(&pipe->tempty[acc]), 0));
+            } else {
+                mbar_arrive(&pipe->tempty[acc]);
+            }
+        };
         TileCursor tc_;
-        tc_.init(a.total_tiles, a.tiles_n, a.ncls);
+        tc_.init(a.total_tiles, a.tiles_n, a.ncls, cta, ctas);
         PixTile pt;
-        pt.init(gr, tc_.mt);
+        pt.init(gr, tile_of(tc_.mt));
         int last_mt = -1;
         bool pix_ok = false;  // tile row p is a pixel of the grid
         int n = 0, y = 0, x = 0;
@@ -398,7 +446,7 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
             const KClass &k = a.cls[tc_.c];
             if (tc_.mt != last_mt) {  // pixel of tile row p
                 last_mt = tc_.mt;
-                pt.advance_to(gr, tc_.mt);
+                pt.advance_to(gr, tile_of(tc_.mt));
                 x = pt.xs * gr.Wt + xx;
                 n = pt.n;
                 y = pt.y + fr;
@@ -579,8 +627,7 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
                     if constexpr (use_mask) fetch_gate(g + 1);
                     __syncwarp();
                 }
-                tc_fence_before();
-                mbar_arrive(&pipe->tempty[acc]);
+                release(acc);
                 continue;
             }
             // ---- head and fp32 outputs (small): every thread stores its own row
@@ -638,16 +685,27 @@ __global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_c
                         if (nn + q * 4 < ncol) op[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
                 }
             }
-            tc_fence_before();
-            mbar_arrive(&pipe->tempty[acc]);
+            release(acc);
         }
     }
     tc_fence_before();
     __syncthreads();
+    if constexpr (PAIR) cluster_sync();
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, ncols);
+        if constexpr (PAIR) tmem_dealloc_pair(tmem_base, ncols);
+        else tmem_dealloc(tmem_base, ncols);
     }
+}
+template <int KIND>
+__global__ void __launch_bounds__(kKThreads, 1) tma_kmajor_kernel(const __grid_constant__ KArgs a) {
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    kmajor_body<KIND, false>(a, smem_raw);
+}
+template <int KIND>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KIND == KIND_FWD ? (1 + kProducers + 8) * 32 : kKThreads, 1) tma_kmajor_pair_kernel(const __grid_constant__ KArgs a) {
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    kmajor_body<KIND, true>(a, smem_raw);
 }
 
 // -------------------------------------------------------------------- wgrad ----
@@ -1140,6 +1198,8 @@ int ensure_smem_attrs() {
         PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_kmajor_kernel<KIND_DGRAD_ACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
         PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_wgrad_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
         PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_wgrad_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
+        PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_kmajor_pair_kernel<KIND_FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+        PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_kmajor_pair_kernel<KIND_DGRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
         PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_wgrad_pair_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
         PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_wgrad_pair_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
         attr_set[dev] = true;
@@ -1149,18 +1209,29 @@ int ensure_smem_attrs() {
 
 // `a.wtaps` = taps of the whole weight tensor (all classes).  ops: operands of a flat GEMM of one class, whose copies may then
 // take several chunks at a time.
+// Whether a convolution's tiles go in pairs; its weight boxes are then BN / 2 rows high.  Input gradients of 128 columns do not gain:
+// their tiles are short and their epilogues long, which two CTAs on an SM overlap better (single / pair, us: 128 <- 256 channels, 4096
+// rows of 8 x 10 outputs 225 / 217, of 15 x 20 936 / 947; 128 <- 128, 1024 rows of 15 x 20 135 / 156).  Fewer tiles than SMs take
+// one CTA each.
+static bool kmajor_pair(const KArgs &a, int ncls) {
+    const long long tiles = (long long)a.grid.tiles * ((a.N + a.BN - 1) / a.BN) * ncls;
+    const size_t weights = (size_t)a.wtaps * a.kchunks * a.BN * a.row_bytes;
+    return (a.mode == EPI_DGRAD ? a.BN > 128 : a.BN >= 128) && a.row_bytes == 128 && weights > kMaxResident && a.mode != EPI_HEAD && !(a.mask && !a.mask_bits) &&
+           tiles >= ppo_num_sms();
+}
+
 int launch_kmajor(KArgs &a, cudaStream_t st, const FlatOps *ops = nullptr) {
     int s = ensure_smem_attrs();
     if (s != PPO_OK) return s;
     a.tiles_n = (a.N + a.BN - 1) / a.BN;
     if (a.mode != EPI_DGRAD && a.tiles_n * a.BN > kMaxBias) return PPO_ERR_UNSUPPORTED;  // bias staged in shared memory
-    const long long per = (long long)a.grid.tiles * a.tiles_n;
+    const long long per = (long long)(a.pair ? (a.grid.tiles + 1) / 2 : a.grid.tiles) * a.tiles_n;
     const long long total = per * a.ncls;
     if (total <= 0) return PPO_OK;
     if (total > 0x7fffffffll) return PPO_ERR_UNSUPPORTED;
     a.total_tiles = (int)total;
-    const size_t b_bytes = (size_t)a.BN * a.row_bytes;
-    const size_t res = (size_t)a.wtaps * a.kchunks * b_bytes;
+    const size_t b_bytes = (size_t)a.BN * a.row_bytes / (a.pair ? 2 : 1);
+    const size_t res = (size_t)a.wtaps * a.kchunks * a.BN * a.row_bytes;
     // resident weights only while they leave most of the shared memory to the A stages: the bytes in flight
     // are what hides the copy latency
     a.wres = (a.tiles_n == 1 && a.ncls == 1 && res <= kMaxResident) ? 1 : 0;
@@ -1170,8 +1241,8 @@ int launch_kmajor(KArgs &a, cudaStream_t st, const FlatOps *ops = nullptr) {
     // A GEMM of a few row tiles gives a CTA one or two tiles: nothing amortises the copy latency, so such a CTA takes the
     // SM alone, with stages of up to 96 KB (fewer, larger hand-overs), and the narrow-tile rule below does not apply.
     const bool flat = a.grid.Hr == 1 && a.grid.Nimg == 1;
-    const bool small_m = (a.grid.tiles <= 4 || (flat && total <= ppo_num_sms())) && (a.ncls == 1 || a.cls_orows != 0);
-    const bool two = a.BN <= 128 && !small_m;
+    const bool small_m = !a.pair && (a.grid.tiles <= 4 || (flat && total <= ppo_num_sms())) && (a.ncls == 1 || a.cls_orows != 0);
+    const bool two = a.BN <= 128 && !small_m && !a.pair;
     a.tmem_cap = two ? 256 : 512;
     a.nepi = (!two && a.mode == EPI_DGRAD && (a.mask_bits || a.mask)) ? 16 : 8;
     const size_t fixed = sizeof(PipeK) + (size_t)a.nepi * 2048 + 1024;  // pipeline state, epilogue staging, alignment slack
@@ -1208,11 +1279,16 @@ int launch_kmajor(KArgs &a, cudaStream_t st, const FlatOps *ops = nullptr) {
     // (forward 128 -> 256 on 20 x 15 195 us with one, 178 with two; 256 -> 256 359 and 338).  Several classes alone on an SM
     // (merged input gradients wider than 128 columns, split reductions) keep one, which is not the faster choice: 256 -> 256 on
     // 20 x 15 432 us with one and 416 with two, 96 -> 128 on 40 x 30 487 and 476, 8 slabs of 16 x 10240 9.1 and 8.4.
-    a.nprod = two || a.ncls > 1 ? 1 : (a.stages < kProducers ? a.stages : kProducers);
+    a.nprod = !a.pair && (two || a.ncls > 1) ? 1 : (a.stages < kProducers ? a.stages : kProducers);
     const int sms = ppo_num_sms();
     const long long ctas = two ? 2ll * sms : sms;
-    const unsigned grid = (unsigned)(total < ctas ? total : ctas);
     const size_t smem = (size_t)a.stages * G * sub + (a.wres ? res : 0) + fixed;
+    if (a.pair) {
+        const unsigned pairs = (unsigned)(total < sms / 2 ? total : sms / 2);
+        return ppo_launch(a.mode != EPI_DGRAD ? tma_kmajor_pair_kernel<KIND_FWD> : tma_kmajor_pair_kernel<KIND_DGRAD>, dim3(2 * pairs),
+                          dim3((1 + a.nprod + a.nepi) * 32), smem, st, a);
+    }
+    const unsigned grid = (unsigned)(total < ctas ? total : ctas);
     const auto fn = a.mode != EPI_DGRAD ? tma_kmajor_kernel<KIND_FWD>
                                         : (a.mask && !a.mask_bits ? tma_kmajor_kernel<KIND_DGRAD_ACT> : tma_kmajor_kernel<KIND_DGRAD>);
     PPO_TRY(ppo_launch(fn, dim3(grid), dim3((1 + a.nprod + a.nepi) * 32), smem, st, a));
@@ -1243,9 +1319,11 @@ int tma_gemm_fwd(const ConvGeom &g, const bf16 *X, const bf16 *W, const FwdEpilo
     int s = flat ? make_act_maps(a.mapA, X, g.Ci, g.Ci, g.B, 1, 1, a.grid, CB, 1, 1)
                  : make_act_maps(a.mapA, X, g.Ci, g.Ci, g.Wi, g.Hi, g.B, a.grid, CB, 2, 2);
     if (s != PPO_OK) return s;
+    a.mode = e.out ? EPI_FWD : EPI_HEAD;
+    a.pair = !flat && kmajor_pair(a, 1);
     {
         const long long dims[2] = {g.K(), g.Co};
-        const int box[2] = {CB, a.BN}, es[2] = {1, 1};
+        const int box[2] = {CB, a.pair ? a.BN / 2 : a.BN}, es[2] = {1, 1};
         s = make_map(&a.mapB, W, 2, dims, g.K(), box, es, a.row_bytes);
         if (s != PPO_OK) return s;
     }
@@ -1254,7 +1332,6 @@ int tma_gemm_fwd(const ConvGeom &g, const bf16 *X, const bf16 *W, const FwdEpilo
     a.Hout = flat ? 1 : g.Ho;
     a.Wout = flat ? g.B : g.Wo;
     a.ldo = e.ldo ? e.ldo : g.Co;
-    a.mode = e.out ? EPI_FWD : EPI_HEAD;
     if (e.ln_gamma) {
         if (!e.ln_beta || !e.ln_xhat || !e.ln_rstd || !e.out || g.Co > 256 || g.Co % 32 != 0 || a.ldo != g.Co) return PPO_ERR_UNSUPPORTED;
         a.ln_gamma = e.ln_gamma;
@@ -1403,9 +1480,10 @@ int tma_gemm_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, i
     a.N = a.BN;  // every group is one full tile of columns
     a.nq_ci = g.Ci;
     a.wtaps = nshift;
+    a.pair = kmajor_pair(a, Ntot / a.BN);
     {
         const long long dims[2] = {(long long)nshift * wt_ld, Ntot};
-        const int box[2] = {CB, a.BN}, es[2] = {1, 1};
+        const int box[2] = {CB, a.pair ? a.BN / 2 : a.BN}, es[2] = {1, 1};
         s = make_map(&a.mapB, Wc, 2, dims, (long long)nshift * wt_ld, box, es, a.row_bytes);
         if (s != PPO_OK) return s;
     }

@@ -339,4 +339,18 @@ __device__ __forceinline__ void tma_load_at(uint32_t dst, const void *map, uint3
             : "memory");
 }
 
+template <bool PAIR>
+__device__ __forceinline__ void tma_load_at(uint32_t dst, const void *map, uint32_t bar, int c0, int c1) {
+    if constexpr (PAIR)
+        asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::"r"(dst),
+                     "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1)
+                     : "memory");
+    else
+        asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::"r"(dst),
+                     "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1)
+                     : "memory");
+}
+// Arrival at a barrier of the cluster, for order with tensor memory only: nothing this thread wrote is released to the other CTA.
+__device__ __forceinline__ void arrive_at(uint32_t bar) { asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory"); }
+
 }  // namespace tc

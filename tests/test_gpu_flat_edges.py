@@ -107,3 +107,13 @@ def test_pairs_of_column_tiles_match_oracle(H, N, conv, monkeypatch):
     w = synth.Workload("cpairs", N, 1, H, H, conv, (3,) * len(conv), (40,), 1, 1, P=16, A=3)
     monkeypatch.setitem(NETS, "cpairs", w)
     conv_stack_matches_oracle("cpairs", monkeypatch)
+
+
+# convolutions whose pixel tiles go in pairs: fewer tiles than SMs (147, single) and as many, odd numbers of tiles, rows of two tiles
+# each, tiles of several images; 128, 192 (above) and 256 columns forward, 4 x 256 back
+@pytest.mark.parametrize("H,W,N,conv", [(64, 64, 294, (32, 128, 128)), (64, 64, 296, (32, 128, 128)), (8, 532, 41, (64, 128)),
+                                        (34, 30, 601, (64, 256, 256))])
+def test_pairs_of_pixel_tiles_match_oracle(H, W, N, conv, monkeypatch):
+    w = synth.Workload("ppairs", N, 1, H, W, conv, (3,) * len(conv), (40,), 1, 1, P=16, A=3)
+    monkeypatch.setitem(NETS, "ppairs", w)
+    conv_stack_matches_oracle("ppairs", monkeypatch)
