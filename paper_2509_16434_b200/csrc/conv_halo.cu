@@ -722,6 +722,10 @@ int halo_conv_fwd(const ConvGeom &g, const bf16 *X, const bf16 *W, const FwdEpil
     if (g.Co % 32 != 0 && (e.out_bits || e.ln_gamma)) return PPO_ERR_UNSUPPORTED;
     const int CB = chunk_of(g.Ci);
     if (CB == 0 || CB != g.Ci || (size_t)9 * g.Ci * g.Co * 2 > 160 * 1024) return PPO_ERR_UNSUPPORTED;
+    // 128 outputs of 64 channels: the weights leave no room for the next tile's planes, and tap boxes whose tiles go in pairs are shorter
+    // (4096 rows of 15 x 20 outputs 253 us here, 221 there; of 30 x 40 1043 and 900).  With layer normalisation it is the other way
+    // round (512 rows of 8 x 10 outputs 22 and 28 us: their epilogue walks each row three times and is the longer side there).
+    if (CB == 64 && g.Co >= 128 && !e.ln_gamma && tma_fwd_in_pairs(g)) return PPO_ERR_UNSUPPORTED;
     Args a = {};
     a.CB = CB;
     a.rb = CB * 2;

@@ -52,6 +52,8 @@ int tc_gemm_wgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *X, flo
 // for anything else they return PPO_ERR_UNSUPPORTED without launching and the caller uses the tc_ versions.
 int tma_gemm_fwd(const ConvGeom &g, const bf16 *X, const bf16 *W, const FwdEpilogue &e, int32_t *status,
                  cudaStream_t st);
+// Whether tma_gemm_fwd takes a convolution's pixel tiles in pairs of CTAs.
+bool tma_fwd_in_pairs(const ConvGeom &g);
 // Wc: the layer's weights regrouped by tma_dgrad_weights for the merged four-class dgrad (convolutions only;
 // fully connected layers read Wt).
 int tma_gemm_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, int wt_ld, const bf16 *Wc,

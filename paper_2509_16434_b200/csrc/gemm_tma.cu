@@ -1299,6 +1299,18 @@ bool is_flat(const ConvGeom &g) { return g.Hi == 1 && g.Wi == 1 && g.Ho == 1 && 
 
 }  // namespace
 
+bool tma_fwd_in_pairs(const ConvGeom &g) {
+    KArgs a = {};
+    const int CB = is_flat(g) ? 0 : channels_per_box(g.Ci, false);
+    if (CB == 0 || !make_grid(a.grid, g.Wo, g.Ho, g.B, CB * 2)) return false;
+    a.row_bytes = CB * 2;
+    a.kchunks = (g.Ci + CB - 1) / CB;
+    a.wtaps = g.taps();
+    a.N = g.Co;
+    a.BN = pick_bn(g.Co);
+    return kmajor_pair(a, 1);
+}
+
 int tma_gemm_fwd(const ConvGeom &g, const bf16 *X, const bf16 *W, const FwdEpilogue &e, int32_t *status,
                  cudaStream_t st) {
     if (!status || g.taps() > kMaxTaps || g.Ci % 8 != 0) return PPO_ERR_UNSUPPORTED;
