@@ -1275,11 +1275,10 @@ int launch_kmajor(KArgs &a, cudaStream_t st, const FlatOps *ops = nullptr) {
     if (a.stages < 2) return PPO_ERR_UNSUPPORTED;
     // Producers.  Two CTAs on an SM are two producers already, and a second one in each costs the other CTA its place: 352
     // threads of 96 registers do not fit twice (input gradient 256 -> 128 channels of 4096 images of 20 x 15: 252 us with one,
-    // 365 with two; forward 96 -> 128 on 40 x 30 413 and 646).  Alone on its SM a CTA of a single class takes two
-    // (forward 128 -> 256 on 20 x 15 195 us with one, 178 with two; 256 -> 256 359 and 338).  Several classes alone on an SM
-    // (merged input gradients wider than 128 columns, split reductions) keep one, which is not the faster choice: 256 -> 256 on
-    // 20 x 15 432 us with one and 416 with two, 96 -> 128 on 40 x 30 487 and 476, 8 slabs of 16 x 10240 9.1 and 8.4.
-    a.nprod = !a.pair && (two || a.ncls > 1) ? 1 : (a.stages < kProducers ? a.stages : kProducers);
+    // 365 with two; forward 96 -> 128 on 40 x 30 413 and 646).  Alone on its SM a CTA takes two (single CTAs, forward 128 -> 256 on
+    // 20 x 15 195 us with one, 178 with two; input gradient 256 -> 256 432 and 416, 96 -> 128 on 40 x 30 487 and 476; 8 slabs of
+    // 16 x 10240 9.1 and 8.4).
+    a.nprod = two ? 1 : (a.stages < kProducers ? a.stages : kProducers);
     const int sms = ppo_num_sms();
     const long long ctas = two ? 2ll * sms : sms;
     const size_t smem = (size_t)a.stages * G * sub + (a.wres ? res : 0) + fixed;
