@@ -33,11 +33,11 @@ sys.path.insert(0, ROOT)
 # sample row, from ncu captures of small twins of the workloads (traffic grows in proportion to the rows): workload
 # -> (bytes per row, capture).  An entry is dropped (traffic: null) as soon as a kernel it covers changes.
 NCU_DRAM_BYTES_PER_ROW = {
-    "cfg2": (2.5673e6, "ncu capture of cfg2_prof at 512 rows, scaled by rows: profiles/ncu_main_kernels_cfg2_prof.txt"),
-    "cfg3": (2.5673e6, "ncu capture of cfg2_prof at 512 rows, scaled by rows: profiles/ncu_main_kernels_cfg2_prof.txt"),
-    "cfg2_prof": (2.5673e6, "ncu capture of cfg2_prof at 512 rows: profiles/ncu_main_kernels_cfg2_prof.txt"),
-    "cfg4": (10.9533e6, "ncu capture of cfg4_prof at 128 rows, scaled by rows: profiles/ncu_main_kernels_cfg4_prof.txt"),
-    "cfg4_prof": (10.9533e6, "ncu capture of cfg4_prof at 128 rows: profiles/ncu_main_kernels_cfg4_prof.txt"),
+    "cfg2": (2.6872e6, "ncu capture of cfg2_prof at 512 rows, scaled by rows: profiles/ncu_main_kernels_cfg2_prof.txt"),
+    "cfg3": (2.6872e6, "ncu capture of cfg2_prof at 512 rows, scaled by rows: profiles/ncu_main_kernels_cfg2_prof.txt"),
+    "cfg2_prof": (2.6872e6, "ncu capture of cfg2_prof at 512 rows: profiles/ncu_main_kernels_cfg2_prof.txt"),
+    "cfg4": (11.1422e6, "ncu capture of cfg4_prof at 128 rows, scaled by rows: profiles/ncu_main_kernels_cfg4_prof.txt"),
+    "cfg4_prof": (11.1422e6, "ncu capture of cfg4_prof at 128 rows: profiles/ncu_main_kernels_cfg4_prof.txt"),
 }
 METRIC = "ppo_learner_env_steps_trained_per_sec"
 UNIT = "env-steps/s"
@@ -360,7 +360,7 @@ def run_ours(args):
         gather_gbs = 2 * (rows if w.n_lstm else w.B) * record_bytes(w) / (gat_ms * 1e-3) / 1e9
         gae_gbs = (17 + 8) * w.M / (gae_ms * 1e-3) / 1e9
         adam_gbs = 30 * L.model.arena / (adam_ms * 1e-3) / 1e9
-        # DRAM bytes of the encoder's GEMM and conv1 kernels per sample row (dram__bytes_read + write summed over the 18
+        # DRAM bytes of the encoder's GEMM and conv1 kernels per sample row (dram__bytes_read + write summed over the 15
         # launches of one forward + backward, ncu capture of the cfg2 network at 512 rows: profiles/ncu_main_kernels_cfg2_prof.txt);
         # traffic grows in proportion to the rows.  Valid for the cfg2/cfg3 network only, and only while those kernels are unchanged.
         per_row, capture = NCU_DRAM_BYTES_PER_ROW.get(w.name, (None, "no ncu capture of the current kernels at this workload"))

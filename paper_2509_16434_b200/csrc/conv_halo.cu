@@ -17,7 +17,7 @@
 // order as in gemm_tma.cu: the results are the same bits.
 // Measured, 4096 rows alone (tap boxes -> here; in brackets the HBM time of inputs, gates and outputs): 32 -> 64 channels on
 // 160 x 120 forward 2.22 -> 1.25 ms (1.17), input gradient 3.25 -> 1.28 (1.2); 64 -> 128 on 80 x 60 forward 1.20 -> 0.98
-// (0.58), input gradient 1.58 -> 1.01 to 1.07 (0.6).
+// (0.58; tap boxes whose tiles go in pairs of CTAs take 0.90, and that forward pass), input gradient 1.58 -> 1.01 to 1.07 (0.6).
 #include <cuda.h>
 
 #include "gemm.cuh"

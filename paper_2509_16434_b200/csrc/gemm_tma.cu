@@ -15,6 +15,7 @@
 //      and plain boxes of dY, read with the pixel index as the reduction; split over pixel tiles across
 //      CTAs, each of which leaves its partial tile in scratch memory; wgrad_reduce_kernel adds the partial
 //      tiles to dW in a fixed order, so that the result does not depend on which CTA finishes first.
+//  tma_kmajor_pair_kernel, tma_wgrad_pair_kernel : the same for wide layers, two CTAs of a cluster as one tensor core.
 //
 // Tiles follow the pixel grid instead of cutting the flattened pixel index every 128: a tile is a
 // rectangle of Wt pixels by R rows of the (image, row) sequence (Wt * R <= 128, chosen to fill most of
