@@ -11,6 +11,7 @@
 //
 // Every wait is bounded: on a time-out the kernel records PPO_ERR_TIMEOUT, waits (bounded) for its copies, frees its
 // tensor memory and returns.
+#include "exchange.h"
 #include "gemm.cuh"
 #include "launch.cuh"
 #include "tcgen05.cuh"
@@ -54,7 +55,8 @@ struct Args {
 };
 
 struct Pipe {
-    uint64_t fullA[kMaxStages], emptyA[kMaxStages], fullB[kMaxStages], emptyB[kMaxStages], tfull, ready;
+    uint64_t fullA[kMaxStages], emptyA[kMaxStages], fullB[kMaxStages], emptyB[kMaxStages], tfull;
+    uint64_t ready[ChainExchange::barriers(kMlpLayers)];  // of the exchange behind each layer
     uint32_t tmem_slot;
     int abort_flag;
     alignas(16) float bias[kMlpLayers * kMaxSlice];
@@ -102,7 +104,7 @@ __device__ __forceinline__ void chain(const Args &a, uint8_t *raw) {
             mbar_init(&pipe->emptyB[s], 1);
         }
         mbar_init(&pipe->tfull, 1);
-        mbar_init(&pipe->ready, CS);
+        for (int i = 0; i < ChainExchange::barriers(kMlpLayers); ++i) mbar_init(&pipe->ready[i], CS);
         pipe->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -129,7 +131,7 @@ __device__ __forceinline__ void chain(const Args &a, uint8_t *raw) {
             const int chunks = a.l[l].chunks, rb = a.l[l].rb, g = a.l[l].g, N = a.l[l].N, n = a.l[l].n;
             const CUtensorMap *const map = &a.l[l].mapA;
             if (l > 0) {  // what the cluster has left for this layer
-                ok = cluster_mbar_wait(&pipe->ready, (uint32_t)(l - 1) & 1u, abort_flag, a.status);
+                ok = cluster_mbar_wait(&pipe->ready[ChainExchange::barrier(l - 1)], ChainExchange::parity(l - 1), abort_flag, a.status);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 fence_proxy_global();
@@ -231,15 +233,13 @@ __device__ __forceinline__ void chain(const Args &a, uint8_t *raw) {
         const int rr0 = lane >> 2, piece = lane & 3, sw = (lane >> 1) & 3;
         const bool rows_here = lg * 32 < a.Mt;
         bool joined = false;  // waited for the cluster's start
-        // Behind this CTA's stores: one release, an arrival at every CTA's barrier.  before: the phase this CTA's part is made
-        // from (-1: none); a CTA without columns has not waited for it, and must not arrive a second time before it is complete.
-        auto publish = [&](bool ok, int before) -> bool {
-            if (before >= 0) ok = cluster_mbar_wait(&pipe->ready, (uint32_t)before & 1u, abort_flag, a.status) && ok;
+        // Behind this CTA's stores: one release, an arrival at every CTA's barrier of the exchange behind layer l.
+        auto publish = [&](bool ok, int l) -> bool {
             if (!epi_all(ok)) return false;
             if (!joined) cluster_wait();
             joined = true;
             if (warp == 4) {
-                if (lane < CS) arrive_in_cta(&pipe->ready, (uint32_t)lane);
+                if (lane < CS) arrive_in_cta(&pipe->ready[ChainExchange::barrier(l)], (uint32_t)lane);
                 __syncwarp();
             }
             return true;
@@ -366,7 +366,7 @@ __device__ __forceinline__ void chain(const Args &a, uint8_t *raw) {
                 tc_fence_before();
             }
             if (col0 < N) tph ^= 1u;
-            if (l + 1 < a.nl && !publish(ok, l - 1)) break;
+            if (l + 1 < a.nl && !publish(ok, l)) break;
         }
         __syncwarp();
         if (!joined) cluster_wait();

@@ -82,8 +82,9 @@ def test_pairs_of_pixels_match_oracle(H, W, N, last, monkeypatch):
 
 
 # the dense chain at its lines: 32 | 64 | 128 rows per tile in clusters of eight, clusters of four, the most rows it takes and one
-# more (layer by layer); the widest slices it takes (240 columns of a CTA) and the next width, which it leaves to single layers
-@pytest.mark.parametrize("B,fc", [(480, (72, 40)), (481, (200, 120)), (961, (72, 504)), (1921, (960,)), (1921, (968,)), (4224, (40,)),
+# more (layer by layer); the widest slices it takes (240 columns of a CTA) and the next width, which it leaves to single layers; a
+# CTA without columns of a layer between two of which it has some (120, 200, 120 in slices of 16, 32, 16)
+@pytest.mark.parametrize("B,fc", [(33, (120, 200, 120)), (480, (72, 40)), (481, (200, 120)), (961, (72, 504)), (1921, (960,)), (1921, (968,)), (4224, (40,)),
                                   (4225, (40,))])
 def test_dense_chain_at_its_lines_matches_oracle(B, fc, monkeypatch):
     w = synth.Workload("chain", 2 * B, 1, 8, 12, (16, 32), (3, 3), fc, 1, 2, P=40, A=3)
