@@ -1,11 +1,13 @@
 """CPU-only checks of the CUDA library's host side: it loads, exports what the header declares, sizes and layouts
 agree with the definitions, and bad arguments are refused before anything is launched."""
 import ctypes as C
+import mmap
 import os
 import re
 
 import numpy as np
 import pytest
+import torch
 
 from oracle import oracle as orc
 from paper_2509_16434_b200 import binding as ppo
@@ -155,3 +157,47 @@ def test_synth_is_seeded_and_shaped():
     nz = d[d > 0]
     assert 0.07 < np.mean(d == 0) < 0.13 and nz.min() >= 0.1 and nz.max() <= 2.0
     assert a["done"].dtype == np.uint8 and a["proprio"].shape == (4, 8, 32) and a["eps"].shape == (4, 8, 12)
+
+
+# ------------------------------------------------------------------ views of the slabs
+
+def _cpu_buffer():
+    with pytest.MonkeyPatch.context() as patch:  # host memory of whole pages: slabs want 256-byte alignment
+        patch.setattr(torch, "empty", lambda n, dtype, device: torch.frombuffer(mmap.mmap(-1, n), dtype=dtype))
+        return ppo.Buffer(ppo.buffer_desc(3, 2, 4, 6, 5, 2), "cpu")
+
+
+def test_slab_first_looked_at_in_inference_mode_stays_usable():
+    buf = _cpu_buffer()
+    with torch.inference_mode():  # the ordinary way to run a rollout
+        first = buf.field(ppo.FIELD_REWARD)
+        first.fill_(1.0)
+    view = buf.field(ppo.FIELD_REWARD)
+    assert not view.is_inference() and torch.equal(view, torch.ones(2, 3))
+    view[1].copy_(torch.full((3,), 2.0))
+    w = torch.ones(2, 3, requires_grad=True)
+    (w * buf.field(ppo.FIELD_REWARD)).sum().backward()  # saved for backward
+    assert torch.equal(w.grad, torch.tensor([[1.0] * 3, [2.0] * 3])) and torch.equal(first, w.grad)
+
+
+def test_slab_views_cover_the_storage_and_count_as_its_writes():
+    buf = _cpu_buffer()
+    d, at = buf.desc, 0
+    for f, (dt, shape) in enumerate([(torch.float16, (2, 3, 4, 6)), (torch.float32, (2, 3, 5)), (torch.float32, (2, 3, 2))]
+                                    + [(torch.float32, (2, 3))] * 3 + [(torch.uint8, (2, 3))] + [(torch.float32, (2, 3))] * 2):
+        v = buf.field(f)
+        assert v.dtype == dt and tuple(v.shape) == shape and v.is_contiguous()
+        assert v.data_ptr() == buf.storage.data_ptr() + at and v.numel() * v.element_size() == ppo.ppo_buffer_field_bytes(d, f)
+        at += -(-v.numel() * v.element_size() // 256) * 256
+    scratch = buf.field(ppo.FIELD_SCRATCH)
+    assert scratch.dim() == 1 and scratch.numel() * 4 == ppo.ppo_buffer_field_bytes(d, ppo.FIELD_SCRATCH)
+    a, before = buf.field(ppo.FIELD_ADV), buf.storage._version
+    a.zero_()
+    assert buf.storage._version > before and buf.field(ppo.FIELD_ADV)._version == buf.storage._version  # autograd sees the write
+    a.resize_(0)  # a caller's own tensor: the next look is whole again
+    assert tuple(buf.field(ppo.FIELD_ADV).shape) == (2, 3)
+    with pytest.raises(TypeError):
+        buf.field(99)
+    buf.close()
+    with pytest.raises(TypeError):
+        buf.field(ppo.FIELD_ADV)
