@@ -1001,12 +1001,12 @@ static ConvGeom fc_geom(int rows, int in, int out) {
 }
 
 // Runs `make` the first time an operation is called with this key and remembers its launches; later calls only enqueue
-// them.
+// them.  last: see ppo_replay.
 template <typename F>
-static int recorded(ppo_model *m, const PlanKey &key, cudaStream_t st, F &&make) {
+static int recorded(ppo_model *m, const PlanKey &key, cudaStream_t st, F &&make, const void *last = nullptr, size_t last_bytes = 0) {
     if (!m->plans) m->plans = new (std::nothrow) ppo_plans();
     if (!m->plans) return make();
-    if (const Launches *known = m->plans->find(key)) return ppo_replay(*known, st);
+    if (const Launches *known = m->plans->find(key)) return ppo_replay(*known, st, last, last_bytes);
     Recording made, *outer = ppo_recording;
     ppo_recording = &made;
     const int s = make();
@@ -1398,9 +1398,9 @@ extern "C" int ppo_encoder_fwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
     }
     if (mlp_covers(mlp, m->F + 1, rows)) {
         PlanKey k = plan_key(OP_MLP_FWD, fc_geom(rows, 0, 0));
-        const void *p[] = {mlp[0].X, mean, value};
-        memcpy(k.p, p, sizeof(p));
-        PPO_TRY(recorded(m, k, st, [&]() -> int { return mlp_chain(mlp, m->F + 1, rows, {d.A, mean, value}, ppo_device_status_ptr(), st); }));
+        k.p[0] = mlp[0].X;
+        const MlpEnds ends = {d.A, mean, value, nullptr, nullptr, nullptr};
+        PPO_TRY(recorded(m, k, st, [&]() -> int { return mlp_chain(mlp, m->F + 1, rows, ends, ppo_device_status_ptr(), st); }, &ends, sizeof(ends)));
         m->fwd_valid = true;
         m->last_row0 = row0;
         m->last_rows = rows;
@@ -1567,11 +1567,9 @@ extern "C" int ppo_encoder_bwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
     const bool chained = mlp_covers(mlp, F + 1, rows);
     if (chained) {
         PlanKey k = plan_key(OP_MLP_BWD, fc_geom(rows, 0, 0));
-        const void *p[] = {dmean, dvalue, mlp[F].out_f32};
-        memcpy(k.p, p, sizeof(p));
-        PPO_TRY(recorded(m, k, st, [&]() -> int {
-            return mlp_chain(mlp, F + 1, rows, {d.A, nullptr, nullptr, dmean, dvalue, m->dh[F + 1]}, ppo_device_status_ptr(), st);
-        }));
+        k.p[0] = mlp[F].out_f32;
+        const MlpEnds ends = {d.A, nullptr, nullptr, dmean, dvalue, m->dh[F + 1]};
+        PPO_TRY(recorded(m, k, st, [&]() -> int { return mlp_chain(mlp, F + 1, rows, ends, ppo_device_status_ptr(), st); }, &ends, sizeof(ends)));
     } else PPO_TRY(ppo_launch(pack_dout_kernel, dim3(ppo_cdiv((long long)rows * 16, 256)), dim3(256), 0, st, dmean, dvalue, m->dh[F + 1], rows, d.A));
     // Weight and bias gradients are leaves of the dependency graph: only the chain of dgrads has to run in order.
     // The leaves of the FC layers (small kernels on a fraction of the SMs) and, further down, conv1's wgrad go to

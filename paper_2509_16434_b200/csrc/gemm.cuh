@@ -104,7 +104,8 @@ struct MlpLayer {
     const bf16 *mask;
     int ldo;
 };
-// mean, value: outputs of a head.  dout [rows][16] (null: none) receives dmean and dvalue as bf16 before the first layer reads it.
+// mean, value: outputs of a head.  dout [rows][16] (null: none) receives dmean and dvalue as bf16 before the first layer reads it.  The last
+// argument of the kernel: a chain prepared once is launched again with other ends (ppo_replay).
 struct MlpEnds {
     int A;
     float *mean, *value;

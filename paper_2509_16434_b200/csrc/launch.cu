@@ -43,12 +43,16 @@ int ppo_enqueue(const void *fn, dim3 grid, dim3 block, size_t smem, bool togethe
     return PPO_OK;
 }
 
-int ppo_replay(const Launches &launches, cudaStream_t st) {
+int ppo_replay(const Launches &launches, cudaStream_t st, const void *last, size_t last_bytes) {
     for (const LaunchRecord &r : launches) {
         void *argv[32];
         const size_t n = r.offset.size();
         if (n > 32) return PPO_ERR_CUDA;
         for (size_t i = 0; i < n; ++i) argv[i] = const_cast<char *>(r.bytes.data()) + r.offset[i];
+        if (last) {
+            if (n == 0 || r.bytes.size() - r.offset[n - 1] != last_bytes) return PPO_ERR_CUDA;
+            argv[n - 1] = const_cast<void *>(last);
+        }
         const int s = ppo_enqueue(r.fn, r.grid, r.block, r.smem, r.together, st, argv);
         if (s != PPO_OK) return s;
     }

@@ -77,5 +77,6 @@ int ppo_launch_together(void (*fn)(P...), dim3 grid, dim3 block, size_t smem, cu
     return ppo_launch_as(true, fn, grid, block, smem, st, args...);
 }
 
-// Enqueues a recorded operation.
-int ppo_replay(const Launches &launches, cudaStream_t st);
+// Enqueues a recorded operation.  last (null: none): what takes the place of the last argument of every launch, last_bytes long; for
+// arguments that are no part of the preparation, such as the addresses of results, and of the key neither.
+int ppo_replay(const Launches &launches, cudaStream_t st, const void *last = nullptr, size_t last_bytes = 0);

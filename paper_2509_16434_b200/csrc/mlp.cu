@@ -47,10 +47,6 @@ struct Args {
     int sA, sB;                // stages
     uint32_t a_slot, b_slot;   // their bytes
     uint32_t tmem_cols;
-    int A;
-    float *mean, *value;       // head
-    const float *dmean, *dvalue;
-    bf16 *dout;                // gradient of the head's outputs as bf16 [rows][16] (null: forward)
     int32_t *status;
 };
 
@@ -85,7 +81,7 @@ __device__ __forceinline__ void drain(uint64_t *full, int it, int S) {
 }
 
 template <int CS>
-__device__ __forceinline__ void chain(const Args &a, uint8_t *raw) {
+__device__ __forceinline__ void chain(const Args &a, const MlpEnds &e, uint8_t *raw) {
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
     const uint32_t base = smem_u32(smem), b_base = base + (uint32_t)a.sA * a.a_slot;  // (an MMA's rows behind the last A stage lie in B's)
     const uint32_t stg_off = (uint32_t)a.sA * a.a_slot + (uint32_t)a.sB * a.b_slot;
@@ -137,7 +133,7 @@ __device__ __forceinline__ void chain(const Args &a, uint8_t *raw) {
                 fence_proxy_global();
             }
             if (rank * n >= N) continue;
-            if (l == 0 && a.dout) {  // the epilogue fills the first stage
+            if (l == 0 && e.dout) {  // the epilogue fills the first stage
                 it = s = 1;
                 continue;
             }
@@ -253,7 +249,7 @@ __device__ __forceinline__ void chain(const Args &a, uint8_t *raw) {
             for (int l = 0; l < kMlpLayers; ++l) pipe->bias[l * kMaxSlice + et] = b[l];
             epi_all(true);
         }
-        if (a.dout) {
+        if (e.dout) {
             // The head's gradient as bf16: every CTA makes the tile's rows for itself, straight into the first stage (32-byte rows,
             // their two pieces swapped in every other four), and its share of them for the weight gradient.
             const int per = a.Mt / CS;
@@ -264,14 +260,14 @@ __device__ __forceinline__ void chain(const Args &a, uint8_t *raw) {
                 for (int k = 0; k < 8; ++k) {
                     const int j = 8 * p + k;
                     v[k] = 0.f;
-                    if (r < a.rows && j < a.A) v[k] = __ldg(a.dmean + (size_t)r * a.A + j);
-                    else if (r < a.rows && j == a.A) v[k] = __ldg(a.dvalue + r);
+                    if (r < a.rows && j < e.A) v[k] = __ldg(e.dmean + (size_t)r * e.A + j);
+                    else if (r < a.rows && j == e.A) v[k] = __ldg(e.dvalue + r);
                 }
                 const uint4 o = make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]), pack_bf16x2(v[6], v[7]));
                 asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(base + (uint32_t)row * 32u + (((uint32_t)p ^ (((uint32_t)row >> 2) & 1u)) << 4)),
                              "r"(o.x), "r"(o.y), "r"(o.z), "r"(o.w)
                              : "memory");
-                if (r < a.rows && row / per == rank) *reinterpret_cast<uint4 *>(a.dout + (size_t)r * 16 + 8 * p) = o;
+                if (r < a.rows && row / per == rank) *reinterpret_cast<uint4 *>(e.dout + (size_t)r * 16 + 8 * p) = o;
             }
             fence_async_smem();
             epi_all(true);
@@ -311,8 +307,8 @@ __device__ __forceinline__ void chain(const Args &a, uint8_t *raw) {
 #pragma unroll
                             for (int i = 0; i < 16; ++i) {
                                 const int c = col0 + g + i;
-                                if (c < a.A) a.mean[(size_t)grow * a.A + c] = v[i] + pipe->bias[l * kMaxSlice + g + i];
-                                else if (c == a.A) a.value[grow] = v[i] + pipe->bias[l * kMaxSlice + g + i];
+                                if (c < e.A) e.mean[(size_t)grow * e.A + c] = v[i] + pipe->bias[l * kMaxSlice + g + i];
+                                else if (c == e.A) e.value[grow] = v[i] + pipe->bias[l * kMaxSlice + g + i];
                             }
                         }
                         continue;
@@ -384,13 +380,13 @@ __device__ __forceinline__ void chain(const Args &a, uint8_t *raw) {
     }
 }
 
-__global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(kThreads, 1) mlp_chain4_kernel(const __grid_constant__ Args a) {
+__global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(kThreads, 1) mlp_chain4_kernel(const __grid_constant__ Args a, const __grid_constant__ MlpEnds e) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    chain<4>(a, smem_raw);
+    chain<4>(a, e, smem_raw);
 }
-__global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(kThreads, 1) mlp_chain8_kernel(const __grid_constant__ Args a) {
+__global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(kThreads, 1) mlp_chain8_kernel(const __grid_constant__ Args a, const __grid_constant__ MlpEnds e) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    chain<8>(a, smem_raw);
+    chain<8>(a, e, smem_raw);
 }
 
 // CTAs per cluster and rows per tile, or false.  Clusters of eight cut the columns finer, but only 15 of them are resident on 148
@@ -426,9 +422,6 @@ int mlp_chain(const MlpLayer *layers, int nl, int rows, const MlpEnds &ends, int
     shape(rows, cs, a.Mt);
     a.nl = nl;
     a.rows = rows;
-    a.A = ends.A;
-    a.mean = ends.mean; a.value = ends.value;
-    a.dmean = ends.dmean; a.dvalue = ends.dvalue; a.dout = ends.dout;
     a.status = status;
     int n_max = 0;
     for (int i = 0; i < nl; ++i) {
@@ -475,5 +468,5 @@ int mlp_chain(const MlpLayer *layers, int nl, int rows, const MlpEnds &ends, int
         PPO_CUDA_CHECK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
         set[cs == 8][dev] = true;
     }
-    return ppo_launch(fn, dim3((unsigned)((rows + a.Mt - 1) / a.Mt * cs)), dim3(kThreads), smem, st, a);
+    return ppo_launch(fn, dim3((unsigned)((rows + a.Mt - 1) / a.Mt * cs)), dim3(kThreads), smem, st, a, ends);
 }

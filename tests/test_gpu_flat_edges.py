@@ -1,5 +1,7 @@
 """Fully connected layers at the edges of their tiles (rows and columns that no tile width divides, reductions that are no whole
 number of chunks), and the gates of the last convolution."""
+import ctypes as C
+
 import pytest
 import torch
 
@@ -90,6 +92,53 @@ def test_dense_chain_at_its_lines_matches_oracle(B, fc, monkeypatch):
     w = synth.Workload("chain", 2 * B, 1, 8, 12, (16, 32), (3, 3), fc, 1, 2, P=40, A=3)
     monkeypatch.setitem(NETS, "chain", w)
     conv_stack_matches_oracle("chain", monkeypatch)
+
+
+class _Mallinfo2(C.Structure):
+    _fields_ = [(n, C.c_size_t) for n in ("arena", "ordblks", "smblks", "hblks", "hblkhd", "usmblks", "fsmblks", "uordblks", "fordblks", "keepcost")]
+
+
+def _heap_bytes():
+    libc = C.CDLL(None)
+    libc.mallinfo2.restype = _Mallinfo2
+    m = libc.mallinfo2()
+    return m.uordblks + m.hblkhd
+
+
+def test_a_chain_with_other_ends_is_the_chain_that_was_prepared():
+    """Mean and value, and their gradients, at addresses that no call has seen: every call writes to and reads from its own, and none is
+    prepared (or remembered: a prepared chain is 2 KB) again."""
+    w = synth.Workload("ends", 64, 1, 8, 12, (16, 32), (3, 3), (504, 72), 1, 1, P=40, A=3)
+    n, B = 256, 64
+    L = base._setup(w, B)[0]
+    L.compute_gae(torch.zeros(64, device="cuda"))
+    ppo.ppo_shuffle_gather_minibatch(L.buffer, 5, 0, 0, 1, L.mb)
+    mean, value = torch.full((n, B, 3), -9.0, device="cuda"), torch.full((n, B), -9.0, device="cuda")
+    ppo.ppo_encoder_fwd(L.model, L.mb, 0, B, L.mean, L.value)
+    g = torch.Generator("cuda").manual_seed(2)
+    L.dmean.copy_(torch.randn((B, 3), device="cuda", generator=g))
+    L.dvalue.copy_(torch.randn(B, device="cuda", generator=g))
+    dmean, dvalue = torch.zeros_like(mean), torch.zeros_like(value)
+    dmean[n - 1], dvalue[n - 1] = L.dmean, L.dvalue
+
+    def gradients(dm, dv):
+        ppo.ppo_model_zero_grad(L.model)
+        ppo.ppo_encoder_bwd(L.model, L.mb, 0, B, dm, dv, True)
+
+    gradients(L.dmean, L.dvalue)
+    want = L.model.grad.clone()
+    for i in range(8):
+        ppo.ppo_encoder_fwd(L.model, L.mb, 0, B, mean[i], value[i])
+        gradients(dmean[i], dvalue[i])
+    before = _heap_bytes()
+    for i in range(8, n):
+        ppo.ppo_encoder_fwd(L.model, L.mb, 0, B, mean[i], value[i])
+        gradients(dmean[i], dvalue[i])
+    grown = _heap_bytes() - before
+    assert ppo.ppo_poll_status() == 0
+    assert bool((mean == L.mean).all()) and bool((value == L.value).all())
+    assert torch.equal(L.model.grad, want) and float(want.norm()) > 0
+    assert grown < 64 * 1024, grown
 
 
 # 48 outputs: behind 16, 32 and 48 channels, odd extents, rows of several segments, many small images, as the last layer
