@@ -250,6 +250,7 @@ __device__ __forceinline__ bool produce_step(const Args &a, const Frame &f, unsi
             if (!seen) seen = load_acquire(mine) >= target;
             ready = __ballot_sync(0xffffffffu, seen);
             if ((ready >> k) & 1u) {
+                __syncwarp();  // a vote orders no memory: what lane k has acquired is passed on to the lane that issues the copy
                 fence_proxy_global();
                 break;
             }
