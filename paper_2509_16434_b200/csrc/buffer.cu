@@ -11,15 +11,13 @@
 static __device__ int32_t g_ppo_status;
 
 int32_t *ppo_device_status_ptr() {
-    static int32_t *ptrs[64] = {nullptr};
+    static PerDevice<int32_t *> ptrs;
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
-    if (!ptrs[dev]) {
+    if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+    return ptrs.get(dev, []() -> int32_t * {
         void *p = nullptr;
-        if (cudaGetSymbolAddress(&p, g_ppo_status) != cudaSuccess) return nullptr;
-        ptrs[dev] = static_cast<int32_t *>(p);
-    }
-    return ptrs[dev];
+        return cudaGetSymbolAddress(&p, g_ppo_status) == cudaSuccess ? static_cast<int32_t *>(p) : nullptr;
+    });
 }
 
 static std::atomic<unsigned long long> g_launches{0};
@@ -29,15 +27,13 @@ void ppo_count_launches(int n) { g_launches.fetch_add((unsigned long long)n, std
 extern "C" uint64_t ppo_launch_count(void) { return g_launches.load(std::memory_order_relaxed); }
 
 int ppo_num_sms() {
-    static int sms[64] = {0};
+    static PerDevice<int> sms;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
-    if (!sms[dev]) {
+    return sms.get(dev, [dev] {
         int n = 0;
-        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 148;
-        sms[dev] = n;
-    }
-    return sms[dev];
+        return cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0 ? n : 148;
+    });
 }
 
 int ppo_work_sequence(cudaStream_t st, uint64_t *seq) {
@@ -487,18 +483,16 @@ __global__ void __launch_bounds__(128) gae_fused_kernel(const float *__restrict_
 
 // Blocks of gae_fused_kernel that can be resident at once on the current device (0: cooperative launch unavailable).
 static int gae_fused_capacity() {
-    static int cap[64] = {0};
-    static bool known[64] = {false};
+    static PerDevice<int> cap;  // + 1
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-    if (!known[dev]) {
+    return cap.get(dev, [dev] {
         int coop = 0, per_sm = 0;
         if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gae_fused_kernel, 128, 0) == cudaSuccess)
-            cap[dev] = per_sm * ppo_num_sms();
-        known[dev] = true;
-    }
-    return cap[dev];
+            return per_sm * ppo_num_sms() + 1;
+        return 1;
+    }) - 1;
 }
 
 extern "C" int ppo_compute_gae(ppo_buffer *b, const float *last_value, float gamma, float lambda, int normalize,
@@ -560,15 +554,13 @@ static __device__ __align__(256) double g_gae_static_scratch[2 * kMaxGaeBlocks];
 // Device address of the scratch array on the current device (nullptr on error).  The array's name is
 // only a host-side handle; kernels must be given the address cudaGetSymbolAddress returns.
 static double *gae_static_scratch_ptr() {
-    static double *ptrs[64] = {nullptr};
+    static PerDevice<double *> ptrs;
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
-    if (!ptrs[dev]) {
-        double *p = nullptr;
-        if (cudaGetSymbolAddress((void **)&p, g_gae_static_scratch) != cudaSuccess) return nullptr;
-        ptrs[dev] = p;
-    }
-    return ptrs[dev];
+    if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+    return ptrs.get(dev, []() -> double * {
+        void *p = nullptr;
+        return cudaGetSymbolAddress(&p, g_gae_static_scratch) == cudaSuccess ? static_cast<double *>(p) : nullptr;
+    });
 }
 
 extern "C" int ppo_gae_static(const float *reward, const float *value, const uint8_t *done, const float *last_value,

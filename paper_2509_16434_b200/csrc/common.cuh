@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "../../include/ppo_b200.h"
+#include "per_device.h"
 
 typedef __nv_bfloat16 bf16;
 
@@ -40,6 +41,19 @@ int32_t *ppo_device_status_ptr();
 // Adds n to the process-wide count of kernels and memsets this library has enqueued.
 void ppo_count_launches(int n);
 int ppo_num_sms();
+// Runs setup() (a status) on the current device unless it has succeeded there before.
+template <typename F>
+int ppo_once_per_device(PerDevice<bool> &done, F &&setup) {
+    int dev = 0, s = PPO_ERR_CUDA;
+    PPO_CUDA_CHECK(cudaGetDevice(&dev));
+    return done.get(dev, [&]() -> bool { return (s = setup()) == PPO_OK; }) ? PPO_OK : s;
+}
+// Lets a kernel have `bytes` of dynamic shared memory.
+template <typename F>
+int ppo_allow_smem(F *fn, size_t bytes) {
+    PPO_CUDA_CHECK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    return PPO_OK;
+}
 
 // Device state that a handle makes once and relies on from then on (cleared counters) is remembered together with the
 // sequence of work that makes it: eager work has run by the time later eager work does, but work that is captured runs when

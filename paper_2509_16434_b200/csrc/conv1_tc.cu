@@ -408,15 +408,9 @@ __global__ void __launch_bounds__(kThreads, 1) conv1_tc_kernel(const __grid_cons
 
 template <int KS, int T, bool DIRECT, int CW, bool LN>
 int launch_one(const Args &a, size_t smem, cudaStream_t st) {
-    static bool attr_set[64] = {false};
-    int dev = 0;
-    PPO_CUDA_CHECK(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64) return PPO_ERR_CUDA;
+    static PerDevice<bool> set;
     const auto fn = conv1_tc_kernel<KS, T, DIRECT, CW, LN>;
-    if (!attr_set[dev]) {
-        PPO_CUDA_CHECK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
-        attr_set[dev] = true;
-    }
+    PPO_TRY(ppo_once_per_device(set, [&] { return ppo_allow_smem(fn, kSmemMax); }));
     const int sms = ppo_num_sms(), nstage = (a.tiles + T - 1) / T;
     return ppo_launch(fn, dim3(nstage < sms ? nstage : sms), dim3(kThreads), smem, st, a);
 }

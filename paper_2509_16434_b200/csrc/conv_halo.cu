@@ -679,15 +679,9 @@ bool plan(Args &a, int Wr, int Hr, int B) {
 
 template <int MODE, int GC, int KS, int EPW>
 int launch_one(const Args &a, cudaStream_t st) {
-    static bool attr_set[64] = {false};
-    int dev = 0;
-    PPO_CUDA_CHECK(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64) return PPO_ERR_CUDA;
+    static PerDevice<bool> set;
     const auto fn = conv_halo_kernel<MODE, GC, KS, EPW>;
-    if (!attr_set[dev]) {
-        PPO_CUDA_CHECK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
-        attr_set[dev] = true;
-    }
+    PPO_TRY(ppo_once_per_device(set, [&] { return ppo_allow_smem(fn, kSmemMax); }));
     return ppo_launch(fn, dim3((unsigned)a.grid), dim3((2 + a.neg * EPW) * 32), a.smem, st, a);
 }
 

@@ -547,20 +547,16 @@ size_t wgrad_smem(int BN) {
 
 // Opts both kernels into their largest dynamic shared memory footprint, once per device.
 int ensure_smem_attrs() {
-    static bool attr_set[64] = {false};
-    int dev = 0;
-    PPO_CUDA_CHECK(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64) return PPO_ERR_CUDA;
-    if (!attr_set[dev]) {
-        size_t mx = 0;
-        for (int bn = 16; bn <= 256; bn += 16) mx = kmajor_smem(bn) > mx ? kmajor_smem(bn) : mx;
-        PPO_CUDA_CHECK(cudaFuncSetAttribute(igemm_kmajor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mx));
-        size_t mw = 0;
-        for (int bn = 16; bn <= 256; bn += 16) mw = wgrad_smem(bn) > mw ? wgrad_smem(bn) : mw;
-        PPO_CUDA_CHECK(cudaFuncSetAttribute(igemm_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mw));
-        attr_set[dev] = true;
-    }
-    return PPO_OK;
+    static PerDevice<bool> set;
+    return ppo_once_per_device(set, []() -> int {
+        size_t mx = 0, mw = 0;
+        for (int bn = 16; bn <= 256; bn += 16) {
+            mx = kmajor_smem(bn) > mx ? kmajor_smem(bn) : mx;
+            mw = wgrad_smem(bn) > mw ? wgrad_smem(bn) : mw;
+        }
+        PPO_TRY(ppo_allow_smem(igemm_kmajor_kernel, mx));
+        return ppo_allow_smem(igemm_wgrad_kernel, mw);
+    });
 }
 
 // Fills the tile bookkeeping of a.cls[0 .. ncls) (Mrows, taps set by the caller) and launches.

@@ -1188,24 +1188,19 @@ struct FlatOps {
 };
 
 int ensure_smem_attrs() {
-    static bool attr_set[64] = {false};
-    int dev = 0;
-    PPO_CUDA_CHECK(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64) return PPO_ERR_CUDA;
-    if (!attr_set[dev]) {
-        const int mx = (int)(kSmemBudget + sizeof(PipeK) + 1024);
-        PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_kmajor_kernel<KIND_FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
-        PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_kmajor_kernel<KIND_DGRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
-        PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_kmajor_kernel<KIND_DGRAD_ACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
-        PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_wgrad_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
-        PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_wgrad_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
-        PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_kmajor_pair_kernel<KIND_FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
-        PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_kmajor_pair_kernel<KIND_DGRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
-        PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_wgrad_pair_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
-        PPO_CUDA_CHECK(cudaFuncSetAttribute(tma_wgrad_pair_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
-        attr_set[dev] = true;
-    }
-    return PPO_OK;
+    static PerDevice<bool> set;
+    return ppo_once_per_device(set, []() -> int {
+        const size_t mx = kSmemBudget + sizeof(PipeK) + 1024;
+        PPO_TRY(ppo_allow_smem(tma_kmajor_kernel<KIND_FWD>, kSmemMax));
+        PPO_TRY(ppo_allow_smem(tma_kmajor_kernel<KIND_DGRAD>, kSmemMax));
+        PPO_TRY(ppo_allow_smem(tma_kmajor_kernel<KIND_DGRAD_ACT>, kSmemMax));
+        PPO_TRY(ppo_allow_smem(tma_wgrad_kernel<true>, mx));
+        PPO_TRY(ppo_allow_smem(tma_wgrad_kernel<false>, mx));
+        PPO_TRY(ppo_allow_smem(tma_kmajor_pair_kernel<KIND_FWD>, kSmemMax));
+        PPO_TRY(ppo_allow_smem(tma_kmajor_pair_kernel<KIND_DGRAD>, kSmemMax));
+        PPO_TRY(ppo_allow_smem(tma_wgrad_pair_kernel<true>, mx));
+        return ppo_allow_smem(tma_wgrad_pair_kernel<false>, mx);
+    });
 }
 
 // `a.wtaps` = taps of the whole weight tensor (all classes).  ops: operands of a flat GEMM of one class, whose copies may then

@@ -741,18 +741,6 @@ bool plan(Args &a, int T, int Be, int H, int U, int &ctas, size_t &smem) {
     return true;
 }
 
-template <typename F>
-int prepare_kernel(F *fn, bool (&set)[64]) {
-    int dev = 0;
-    PPO_CUDA_CHECK(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64) return PPO_ERR_CUDA;
-    if (!set[dev]) {
-        PPO_CUDA_CHECK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
-        set[dev] = true;
-    }
-    return PPO_OK;
-}
-
 template <int M, int U>
 int launch_step(StepArgs &a, int in, const LstmSteps &p, const bf16 *X, const bf16 *Wx, const bf16 *Wh, cudaStream_t st) {
     const long long H = p.H, Be = p.Be;
@@ -771,8 +759,8 @@ int launch_step(StepArgs &a, int in, const LstmSteps &p, const bf16 *X, const bf
     const size_t stage = (size_t)kStepG * (M + 4 * U) * 128, fixed = (size_t)M * U * 16 + sizeof(Pipe) + 1024;
     a.stages = (int)((kSmemMax - fixed) / stage);
     if (a.stages > kMaxStages) a.stages = kMaxStages;
-    static bool set[64] = {false};
-    PPO_TRY(prepare_kernel(lstm_step_kernel<M, U>, set));
+    static PerDevice<bool> set;
+    PPO_TRY(ppo_once_per_device(set, [] { return ppo_allow_smem(lstm_step_kernel<M, U>, kSmemMax); }));
     const unsigned ctas = (unsigned)((Be + M - 1) / M * (H / U));
     return ppo_launch(lstm_step_kernel<M, U>, dim3(ctas), dim3(kThreads), (size_t)a.stages * stage + fixed, st, a);
 }
@@ -803,8 +791,8 @@ int launch_fwd(Args &a, const LstmSteps &p, int ctas, size_t smem, cudaStream_t 
     const long long da[2] = {H, rows}, sa[1] = {2 * H};
     const int ba[2] = {64, tile_envs(U)};
     PPO_TRY(make_map_strided(&a.mapA, p.hprev, 2, da, sa, ba));
-    static bool set[64] = {false};
-    PPO_TRY(prepare_kernel(lstm_fwd_kernel<U>, set));
+    static PerDevice<bool> set;
+    PPO_TRY(ppo_once_per_device(set, [] { return ppo_allow_smem(lstm_fwd_kernel<U>, kSmemMax); }));
     return ppo_launch_together(lstm_fwd_kernel<U>, dim3(ctas), dim3(kThreads), smem, st, a);
 }
 
@@ -821,8 +809,8 @@ int launch_bwd_clusters(Args &a, const LstmSteps &p, bf16 *dg, cudaStream_t st) 
     int ctas = 0;
     size_t smem = 0;
     if (!plan(a, p.T, p.Be, p.H, U, ctas, smem)) return PPO_ERR_UNSUPPORTED;
-    static bool set[64] = {false};
-    PPO_TRY(prepare_kernel(lstm_bwd_cluster_kernel<U>, set));
+    static PerDevice<bool> set;
+    PPO_TRY(ppo_once_per_device(set, [] { return ppo_allow_smem(lstm_bwd_cluster_kernel<U>, kSmemMax); }));
     bool fit = false;
     PPO_TRY(clusters_fit(lstm_bwd_cluster_kernel<U>, ctas, smem, fit));
     if (!fit) return PPO_ERR_UNSUPPORTED;
@@ -872,8 +860,8 @@ int lstm_bwd_steps(const LstmSteps &p, const bf16 *WhT, const float *dtop, bf16 
     if (s != PPO_ERR_UNSUPPORTED) return s;
     plan(a, p.T, p.Be, p.H, 4, ctas, smem);
     PPO_TRY(map_dg(a, p, dg, tile_envs(4)));
-    static bool set[64] = {false};
-    PPO_TRY(prepare_kernel(lstm_bwd_kernel, set));
+    static PerDevice<bool> set;
+    PPO_TRY(ppo_once_per_device(set, [] { return ppo_allow_smem(lstm_bwd_kernel, kSmemMax); }));
     return ppo_launch_together(lstm_bwd_kernel, dim3(ctas), dim3(kThreads), smem, st, a);
 }
 

@@ -460,13 +460,7 @@ int mlp_chain(const MlpLayer *layers, int nl, int rows, const MlpEnds &ends, int
     if (a.sB < 2) return PPO_ERR_UNSUPPORTED;
     const size_t smem = (size_t)a.sA * a.a_slot + (size_t)a.sB * a.b_slot + kEpiWarps * kStage + sizeof(Pipe) + 1024;
     const auto fn = cs == 8 ? mlp_chain8_kernel : mlp_chain4_kernel;
-    static bool set[2][64] = {};
-    int dev = 0;
-    PPO_CUDA_CHECK(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64) return PPO_ERR_CUDA;
-    if (!set[cs == 8][dev]) {
-        PPO_CUDA_CHECK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
-        set[cs == 8][dev] = true;
-    }
+    static PerDevice<bool> set[2];
+    PPO_TRY(ppo_once_per_device(set[cs == 8], [&] { return ppo_allow_smem(fn, kSmemMax); }));
     return ppo_launch(fn, dim3((unsigned)((rows + a.Mt - 1) / a.Mt * cs)), dim3(kThreads), smem, st, a, ends);
 }
