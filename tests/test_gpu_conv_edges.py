@@ -74,8 +74,8 @@ def test_gate_bits_are_the_signs_of_the_activations():
             assert np.array_equal(bits != 0, act > 0), (name, l)
 
 
-# layers whose gate the input gradient reads as activations in the halo kernel (16 channels), as activations in the generic
-# one (48) and as bits (32)
+# layers whose gate the input gradient reads as half words of bits (16 channels, halo kernel), as activations (48, generic kernel)
+# and as bits (32)
 @pytest.mark.parametrize("name", ["narrow_16_32", "ln_odd", "chunks_of_16", "two_chunks"])
 def test_gate_is_open_for_positive_activations_only(name):
     """Saved activations written from outside may be anything: minus zero, negative numbers and NaN close the gate as zero

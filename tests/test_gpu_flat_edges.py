@@ -2,15 +2,37 @@
 number of chunks), and the gates of the last convolution."""
 import ctypes as C
 
+import numpy as np
 import pytest
 import torch
 
 import test_gpu_learner as base
+from helpers import rel_l2
 from paper_2509_16434_b200 import binding as ppo
 from paper_2509_16434_b200 import synth
 from test_gpu_conv_edges import NETS, test_conv_stack_matches_oracle as conv_stack_matches_oracle
 
 pytestmark = pytest.mark.gpu
+
+
+def _all_rows_match_oracle(w):
+    """The forward of a whole minibatch in one call, row by row: a row is within the encoder's tolerance of itself, or of a row of
+    average size where it is smaller."""
+    B = w.M // w.minibatches
+    L, md, lay, theta, roll, action, logp, dev = base._setup(w, B, theta_scale_head=20.0)
+    L.compute_gae(dev["last_value"])
+    f, _, _, mu_o, V_o = base._oracle_minibatch(md, lay, theta, roll, action, logp, w, L.hyper, 5, 0, 0, w.minibatches)
+    ppo.ppo_shuffle_gather_minibatch(L.buffer, 5, 0, 0, w.minibatches, L.mb)
+    L.mean.fill_(-9.0)
+    L.value.fill_(-9.0)
+    ppo.ppo_encoder_fwd(L.model, L.mb, 0, B, L.mean, L.value)
+    assert ppo.ppo_poll_status() == 0
+    got = np.concatenate([L.mean[:B].cpu().numpy(), L.value[:B, None].cpu().numpy()], 1).astype(np.float64)
+    want = np.concatenate([mu_o, np.asarray(V_o).reshape(-1, 1)], 1)
+    norm = np.linalg.norm(want, axis=1)
+    err = np.linalg.norm(got - want, axis=1) / np.maximum(norm, np.sqrt(np.mean(norm ** 2)))
+    print(f"rows of {B}: largest error {err.max():.2e}")
+    assert err.max() <= base.ENC_TOL, int(err.argmax())
 
 
 # minibatches of 1, 33, 129 and 300 rows: one row, one past a tile of 32, one past a tile of 128, many ragged tiles; widths that are
@@ -22,6 +44,7 @@ def test_forward_and_gradients_match_oracle(N, T, fc, P, last, embed, monkeypatc
     w = synth.Workload("flat", N, T, 16, 24, (16, last), (3, 3), fc, 1, 2, P=P, A=3, embed=embed)
     monkeypatch.setitem(NETS, "flat", w)
     conv_stack_matches_oracle("flat", monkeypatch)  # outputs and every gradient tensor within 2e-2
+    _all_rows_match_oracle(w)
 
 
 @pytest.mark.parametrize("name", ["narrow_16_32", "three_groups", "many_chunks", "small_images", "one_block"])
@@ -86,12 +109,61 @@ def test_pairs_of_pixels_match_oracle(H, W, N, last, monkeypatch):
 # the dense chain at its lines: 32 | 64 | 128 rows per tile in clusters of eight, clusters of four, the most rows it takes and one
 # more (layer by layer); the widest slices it takes (240 columns of a CTA) and the next width, which it leaves to single layers; a
 # CTA without columns of a layer between two of which it has some (120, 200, 120 in slices of 16, 32, 16)
-@pytest.mark.parametrize("B,fc", [(33, (120, 200, 120)), (480, (72, 40)), (481, (200, 120)), (961, (72, 504)), (1921, (960,)), (1921, (968,)), (4224, (40,)),
-                                  (4225, (40,))])
+CHAIN_LINES = [(33, (120, 200, 120)), (480, (72, 40)), (481, (200, 120)), (961, (72, 504)), (1921, (960,)), (1921, (968,)), (4224, (40,)),
+               (4225, (40,))]
+
+
+@pytest.mark.parametrize("B,fc", CHAIN_LINES)
 def test_dense_chain_at_its_lines_matches_oracle(B, fc, monkeypatch):
     w = synth.Workload("chain", 2 * B, 1, 8, 12, (16, 32), (3, 3), fc, 1, 2, P=40, A=3)
     monkeypatch.setitem(NETS, "chain", w)
     conv_stack_matches_oracle("chain", monkeypatch)
+    _all_rows_match_oracle(w)
+
+
+# (widths that the chain takes: a layer reads 64 values or more)
+@pytest.mark.parametrize("B,fc", [(1, (72,)), (33, (120, 200, 120)), (480, (72, 72)), (481, (200, 120)), (960, (504, 72)), (961, (72, 504)), (1920, (120,)),
+                                  (1921, (960,)), (1921, (968,)), (4224, (64,)), (4225, (64,))])
+def test_dense_chain_gives_the_bits_of_single_layers(B, fc):
+    """B rows in one call against the same rows among 4226, which no chain takes, and (forward) in pieces of 480, which clusters of
+    eight take: outputs and hidden layers are the same bits.  Back, only the rows of the last tile of 32 carry a gradient, so that
+    none of it can be lost in the rest; the input gradients are the same bits, and the weight gradients sum the same terms (at most 32
+    rows x 24 pixels) in other groups: 768 roundings of 2^-24 are 4.6e-5 of the sum of their sizes."""
+    R = 4226
+    w = synth.Workload("bits", R, 1, 8, 12, (16, 32), (3, 3), fc, 1, 1, P=40, A=3)
+    L = base.Learner(w, R, "cuda")
+    shapes, gammas = synth.param_shapes(w)
+    L.model.load(synth.init_params(L.model.arena, [o for o, _ in L.model.tensors()], shapes, 3, ones=gammas))
+    r = synth.rollout_torch(w, "cuda", 3)
+    rows = ppo.Minibatch(r["depth"].data_ptr(), r["proprio"].data_ptr(), None, None, None, None, None, None, R)
+    g = torch.Generator("cuda").manual_seed(4)
+    first = (B - 1) // 32 * 32
+    dmean, dvalue = torch.zeros((R, 3), device="cuda"), torch.zeros(R, device="cuda")
+    dmean[first:B] = torch.randn((B - first, 3), device="cuda", generator=g)
+    dvalue[first:B] = torch.randn(B - first, device="cuda", generator=g)
+
+    def run(n):
+        L.mean.fill_(-9.0)
+        L.value.fill_(-9.0)
+        ppo.ppo_encoder_fwd(L.model, rows, 0, n, L.mean, L.value)
+        out = [L.mean.clone(), L.value.clone()] + [L.model.activation(1, l)[:B * k].clone() for l, k in enumerate([72] + list(fc))]
+        ppo.ppo_model_zero_grad(L.model)
+        ppo.ppo_encoder_bwd(L.model, rows, 0, n, dmean, dvalue, True)
+        return out, L.model.grad.clone()
+
+    (mean, value, *hidden), grad = run(B)
+    (mean_all, value_all, *hidden_all), grad_all = run(R)
+    assert bool((mean[B:] == -9.0).all()) and bool((value[B:] == -9.0).all())
+    assert torch.equal(mean[:B], mean_all[:B]) and torch.equal(value[:B], value_all[:B])
+    assert all(torch.equal(a, b) for a, b in zip(hidden, hidden_all))
+    for r0 in range(0, B, 480):
+        n = min(480, B - r0)
+        ppo.ppo_encoder_fwd(L.model, rows, r0, n, L.mean, L.value)
+        assert torch.equal(L.mean[:n], mean[r0:r0 + n]) and torch.equal(L.value[:n], value[r0:r0 + n])
+    assert ppo.ppo_poll_status() == 0
+    errs = [rel_l2(grad[o:o + s].cpu().numpy(), grad_all[o:o + s].cpu().numpy()) for o, s in L.model.tensors()[:-1]]
+    print(f"gradients of rows {first} to {B}: largest difference {max(errs):.1e}")
+    assert float(grad.norm()) > 0 and max(errs) <= 5e-5
 
 
 class _Mallinfo2(C.Structure):
