@@ -7,6 +7,7 @@ The library must exist (build with `python -m paper_2509_16434_b200.build` or
 from __future__ import annotations
 
 import ctypes as C
+import math
 import os
 from typing import Optional, Sequence
 
@@ -181,12 +182,15 @@ class Buffer:
 
     def _views(self):
         d = self.desc
-        shapes = {FIELD_DEPTH: (d.T, d.N, d.H, d.W), FIELD_PROPRIO: (d.T, d.N, d.P), FIELD_ACTION: (d.T, d.N, d.A), FIELD_SCRATCH: (-1,)}
+        shapes = {FIELD_DEPTH: (d.T, d.N, d.H, d.W), FIELD_PROPRIO: (d.T, d.N, d.P), FIELD_ACTION: (d.T, d.N, d.A),
+                  FIELD_SCRATCH: (ppo_buffer_field_bytes(d, FIELD_SCRATCH) // 4,)}
+        typed = {dt: self.storage.view(dt) for dt in (torch.float32, torch.float16, torch.uint8)}
+        ptr, start = lib().ppo_buffer_field_ptr, self.storage.data_ptr()
         views = {}
         for f in range(NUM_FIELDS):
-            off = lib().ppo_buffer_field_ptr(self.handle, f) - self.storage.data_ptr()
-            raw = self.storage[off:off + ppo_buffer_field_bytes(d, f)]
-            views[f] = raw.view(self._DT.get(f, torch.float32)).view(shapes.get(f, (d.T, d.N)))
+            dt, shape = self._DT.get(f, torch.float32), shapes.get(f, (d.T, d.N))
+            stride = tuple(math.prod(shape[i + 1:]) for i in range(len(shape)))
+            views[f] = typed[dt].as_strided(shape, stride, (ptr(self.handle, f) - start) // dt.itemsize)
         return views
 
     def close(self):
