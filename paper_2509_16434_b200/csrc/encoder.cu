@@ -557,7 +557,7 @@ __global__ void __launch_bounds__(256) unpool_kernel(const float *__restrict__ d
 
 // The same from the gate bits (C a multiple of 32): block (row b, run of `per` pixels), a thread owns 8 channels, whose gradient
 // it converts once, and every rpb-th pixel of the run.  The kernel writes what it must and reads a sixteenth of it: 4096
-// rows of 80 pixels x 256 channels 57 -> 29 us against reading the activations.
+// rows of 80 pixels x 256 channels 57 -> 30 us (ncu) against reading the activations.
 __global__ void __launch_bounds__(256) unpool_bits_kernel(const float *__restrict__ dh0, const uint32_t *__restrict__ bits,
                                                           bf16 *__restrict__ dact, int npx, int C, int ld_h0, int runs, int per) {
     grid_wait();
@@ -886,7 +886,7 @@ __global__ void __launch_bounds__(256) ln_bwd_kernel(bf16 *__restrict__ d, const
 
 // State the first step of a sequence starts from: h_prev[0] = bf16(h_init), c_prev[0] = c_init (rows of one step, n = Be x H),
 // of gridDim.y layers whose h_init and c_init follow one another; V elements per thread (four where h_init and c_init are aligned
-// for it, 512 envs x 2 x 1024 units: 11.9 -> 5 us).
+// for it).  512 envs x 2 layers of 1024 units, kernel times under ncu: a launch and an element each 4.7 + 4.3 us, this 6.6.
 struct InitJobs {
     bf16 *hprev[PPO_MAX_LSTM];
     float *cprev[PPO_MAX_LSTM];

@@ -3,9 +3,10 @@
 // A step's product with W_h is small (Be x 4H x H) and every step waits for the one before it: launch by launch the loop is
 // a chain of 13 us GEMMs and 5 us cell kernels that mostly wait, for W_h from L2, for the pipeline to fill, for the
 // launch.  Here a CTA keeps its slice of W_h in shared memory for all steps, the cell runs on the accumulator (forward) or
-// between two exchanges (backward) with c and its gradient in registers, and the CTAs of a tile of 128 envs exchange their
-// parts through global memory once (forward) or twice (backward) per step, with counters for each group of four of them.  What a
-// step costs (cycles of 16000, forward, 256 envs x 1024 units): 7300 for the 256 KB of h (or of one gate's gradients) a CTA
+// between two exchanges (backward) with c and its gradient in registers, and the CTAs of a tile of 32, 64 or 128 envs exchange
+// h (or the gate gradients) through global memory once per step, with counters for each group of four of them.  Backward's other
+// exchange, the partial products of the four slabs of a reduction, goes by st.async into shared memory of the cluster the four
+// form; through global memory only where tiles of 128 envs fit but not as clusters.  What a step costs (cycles of 16000, forward, 256 envs x 1024 units): 7300 for the 256 KB of h (or of one gate's gradients) a CTA
 // pulls through L2 and their MMAs (all CTAs together take 11 TB/s), 700 + 2500 for the accumulator's way to the cell and the
 // cell, 1250 until the release has seen its stores done, 2000 until the readers have seen it.
 // The arithmetic is that of the step-by-step path, sum by sum: same bits.

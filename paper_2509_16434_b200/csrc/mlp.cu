@@ -389,8 +389,9 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(kThreads, 1) mlp_cha
     chain<8>(a, e, smem_raw);
 }
 
-// CTAs per cluster and rows per tile, or false.  Clusters of eight cut the columns finer, but only 15 of them are resident on 148
-// SMs (33 of four); a second wave would cost as much as it saves.  Below that the smallest tile that still leaves one wave.
+// CTAs per cluster and rows per tile, or false.  Clusters of eight cut the columns finer, but cudaOccupancyMaxActiveClusters gives 15
+// of them on a B200's 148 SMs (33 of four); a second wave would cost as much as it saves.  Below that the smallest tile that still
+// leaves one wave.  The two counts are the part's, not asked for in every call: where fewer fit, clusters run one after another.
 bool shape(int rows, int &cs, int &Mt) {
     cs = 8;
     for (Mt = 32; Mt <= 128; Mt *= 2)

@@ -343,7 +343,7 @@ struct LstmStates {
 };
 
 // h (bf16 -> fp32) and c of the last time step, zero where done: one thread per V state elements, blockIdx.y is the layer.  Four
-// at a time where the caller's arrays are aligned for it (512 envs x 2 x 1024 units: 6.3 -> 4.0 us).
+// at a time where the caller's arrays are aligned for it (512 envs x 2 x 1024 units: 9.0 -> 4.8 us under ncu).
 template <int V>
 __global__ void __launch_bounds__(256) lstm_read_state_kernel(const __grid_constant__ LstmStates s, const uint8_t *__restrict__ done,
                                                               float *__restrict__ h_out, float *__restrict__ c_out, int Be, int H) {

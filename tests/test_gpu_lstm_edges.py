@@ -1,4 +1,4 @@
-"""Recurrent layers as one kernel per direction at the edges of their tiles (128 envs, 16 units per CTA), the step-by-step
+"""Recurrent layers as one kernel per direction at the edges of their tiles (32, 64 or 128 envs, 16 units per CTA), the step-by-step
 path where not all CTAs fit the GPU, and what acting does differently: the embedding in slabs and the state reset."""
 import numpy as np
 import pytest
