@@ -34,6 +34,10 @@ using namespace tc;
 // and two staging buffers, a group has eight warps, two per lane quarter, which share out the columns.
 
 constexpr int kMaxSlots = 8;
+constexpr int kMaxGroups = 8;   // row groups of the ring between the input gradient and the first layer's weight gradient
+constexpr int kWinStages = 4;   // stages of window tiles, of four trips of 32 pixels each
+constexpr int kTrip = 32, kStagePx = 4 * kTrip;
+constexpr int kBuildWarps = 8;  // in two sets of four
 constexpr int kMaxOps = 9;
 constexpr size_t kSmemMax = 227 * 1024;
 
@@ -90,7 +94,19 @@ struct Args {
     int32_t *status;
 };
 
+// The first layer's weight gradient behind the input gradient of the second (see first_sums).
+struct First {
+    int Hf, Wh;             // frame rows, and 32-bit words of one
+    int M, px_per_warp;     // pixels of the first layer's output; of one of the eight runs that make a block of partial sums
+    int blocks;             // blocks of partial sums, dealt out over the CTAs
+    int groups, ring_px;    // row groups in flight, pixels of the ring
+    int group_px, last_px;  // pixels of a group of 2 R rows, and of the last one of an image
+    uint32_t ring_bytes;
+    float *part;            // [block][C1 k k (dW order) | C1 (db)]
+};
+
 struct Pipe {
+    uint64_t gfull[kMaxGroups], gempty[kMaxGroups], pfull[kWinStages], pempty[kWinStages];
     uint64_t full[kMaxSlots], empty[kMaxSlots], tfull[4], tempty[4], wfull;
     uint32_t tmem_slot;
     int abort_flag;
@@ -168,20 +184,287 @@ __device__ __forceinline__ bool epi_all(bool ok, int eg) {
     return r != 0;
 }
 
+// A kernel parameter in a register: several roles that each read theirs in their loops evict one another's from the constant
+// cache, and a reading then takes a few hundred cycles.
+__device__ __forceinline__ int held(int v) {
+    asm volatile("" : "+r"(v));
+    return v;
+}
+
+// A walk through the row groups of a CTA: the barriers' index and parity, the group's place in its image, and the ring slot of its first
+// pixel (negative while that lies in front of the CTA's run).
+struct GroupWalk {
+    int groups, ysegs, group_px, last_px, ring_px;
+    int i, k, slot;
+    uint32_t ph;
+    __device__ void init(const Args &a, const First &f, int k0, int slot0) {
+        groups = held(f.groups); ysegs = held(a.ysegs); group_px = held(f.group_px); last_px = held(f.last_px); ring_px = held(f.ring_px);
+        i = 0; k = k0; slot = slot0; ph = 0;
+    }
+    __device__ int px() const { return k == ysegs - 1 ? last_px : group_px; }
+    __device__ void next() {
+        slot += px();
+        if (slot >= ring_px) slot -= ring_px;
+        if (++i == groups) { i = 0; ph ^= 1u; }
+        if (++k == ysegs) k = 0;
+    }
+};
+
+// Window of the first layer as aligned pairs of fp16 frame pixels, one row of the weight gradient per pair element and one for the bias.
+template <int K1>
+struct Win {
+    static constexpr int P = K1 / 2, ODD = P & 1, NP = (K1 + ODD + 1) / 2, KW = K1 * NP;
+    static constexpr int TP = (2 * KW + 1 + 15) / 16 * 16, MB = TP / 16;
+};
+
+// Place of the 16-byte piece `piece` of ring pixel `row` (C1 channels).  Neighbouring lanes of the epilogue write every second pixel,
+// ldmatrix reads eight in a row: both go to eight different 16-byte columns of the 128-byte lines.
+template <int C1>
+__device__ __forceinline__ uint32_t ring_offset(int row, int piece) {
+    constexpr int per = 64 / C1, lg = per == 4 ? 2 : 1;  // pixels per line
+    const int line = row >> lg, q = (row & (per - 1)) * (8 / per) + piece;
+    return (uint32_t)line * 128u + ((uint32_t)(q ^ (line & 7)) << 4);
+}
+
+__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t addr, uint32_t &r0, uint32_t &r1, uint32_t &r2, uint32_t &r3) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// Builder warp bw: the window tiles of the pixels p0 .. p1, [32 px][TP] bf16, four trips to a stage; trip bw % 4 of every second
+// stage.
+// The builders also stand between ring and sums, whose loop is the kernel's longest chain: a stage is handed over when its pixels
+// have arrived in the ring, and a row group is given back by the builder that sees the stage it ends in summed.
+template <int K1>
+__device__ __forceinline__ void first_windows(const First &f, int H1, int W1, const __half *depth, int p0, int p1, const GroupWalk &at, int bw,
+                                              uint8_t *patch, Pipe *pipe, int32_t *status) {
+    using WN = Win<K1>;
+    constexpr int TP = WN::TP, KW = WN::KW, NP = WN::NP, P = WN::P, ODD = WN::ODD;
+    const int lane = threadIdx.x & 31, nstages = (p1 - p0 + kStagePx - 1) / kStagePx;
+    const uint32_t *const frames = reinterpret_cast<const uint32_t *>(depth);
+    const int Hf = held(f.Hf), Wh = held(f.Wh);
+    H1 = held(H1);
+    W1 = held(W1);
+    int m = p0 + (bw >> 2) * kStagePx + (bw & 3) * kTrip + lane;
+    int ow = m % W1, oh = m / W1 % H1;
+    long long b = m / W1 / H1;
+    const int d_oh = 2 * kStagePx / W1, d_ow = 2 * kStagePx - d_oh * W1;
+    uint32_t raw[KW];
+    bool live = false;
+    // A trip's loads are issued a turn ahead of their use.  A pair outside the frame is a predicated load that leaves its zero.
+    auto fetch = [&]() {
+        live = m < p1;
+        const int pw0 = ow - (P + ODD) / 2, ih0 = 2 * oh - P;
+        const uint32_t *row = frames + ((b * Hf + ih0) * Wh + pw0);
+        bool cok[NP];
+#pragma unroll
+        for (int q = 0; q < NP; ++q) cok[q] = live && (unsigned)(pw0 + q) < (unsigned)Wh;
+#pragma unroll
+        for (int kh = 0; kh < K1; ++kh) {
+            const bool rok = (unsigned)(ih0 + kh) < (unsigned)Hf;
+#pragma unroll
+            for (int q = 0; q < NP; ++q) {
+                raw[kh * NP + q] = 0u;
+                if (rok && cok[q]) raw[kh * NP + q] = __ldg(row + q);
+            }
+            row += Wh;
+        }
+        m += 2 * kStagePx;
+        ow += d_ow;
+        if (ow >= W1) { ow -= W1; ++oh; }
+        oh += d_oh;
+        while (oh >= H1) { oh -= H1; ++b; }
+    };
+    fetch();
+    uint8_t *const mine = patch + (size_t)((bw & 3) * kTrip + lane) * (TP * 2);
+    const int sw = TP == 32 ? (lane >> 1) & 3 : (lane >> 2) & 1;
+    GroupWalk seen = at, done = at;
+    int avail = at.slot, ended = at.slot + at.px();  // pixels of the run that have arrived; end of group `done`
+    for (int s = bw >> 2; s < nstages; s += 2) {
+        uint32_t wv[TP / 2];
+#pragma unroll
+        for (int k = 0; k < TP / 2; ++k) wv[k] = 0u;
+#pragma unroll
+        for (int k = 0; k < KW; ++k) {
+            const float2 v = __half22float2(*reinterpret_cast<const __half2 *>(&raw[k]));
+            wv[k] = pack_bf16x2(v.x, v.y);
+        }
+        if (live) wv[KW] = 0x00003F80u;  // (1.0, 0) as bf16: the bias-gradient column
+        fetch();
+        const int slot = s & (kWinStages - 1);
+        if (!mbar_wait_warp(&pipe->pempty[slot], (uint32_t)(s / kWinStages & 1) ^ 1u, &pipe->abort_flag, status)) return;
+        uint8_t *const row = mine + (size_t)slot * (kStagePx * TP * 2);
+#pragma unroll
+        for (int c = 0; c < TP / 8; ++c)
+            *reinterpret_cast<uint4 *>(row + ((c ^ sw) << 4)) = make_uint4(wv[4 * c], wv[4 * c + 1], wv[4 * c + 2], wv[4 * c + 3]);
+        if ((bw & 3) == 0) {
+            const int summed = (s - kWinStages + 1) * kStagePx;  // (the first stages have nothing before them)
+            for (; ended <= summed; ended += done.px()) {
+                if (ended > summed - kStagePx && lane == 0) mbar_arrive(&pipe->gempty[done.i]);
+                done.next();
+            }
+        }
+        const int end = min(p1 - p0, s * kStagePx + (bw & 3) * kTrip + kTrip);
+        while (avail < end) {
+            if (!mbar_wait_warp(&pipe->gfull[seen.i], seen.ph, &pipe->abort_flag, status)) return;
+            avail += seen.px();
+            seen.next();
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&pipe->pfull[slot]);
+    }
+}
+
+// dW1[co][tap] = sum over pixels dZ1[px][co] x[px][tap] as mma.sync m16n8k16 with the pixel as K, dZ1 from the ring in which the
+// epilogue leaves it and x from the builders' window tiles.  The pixels are summed in the runs, the trips of 32 and the blocks
+// of conv1_wgrad_mma_kernel: the same bits.  A run is one chain of dependent products, 25 cycles for 16 pixels, and a fragment load
+// takes its warp 16 to 20: a unit of 16 rows (pair elements of the window) x 16 channels per warp, its fragments two trips ahead.  Finer
+// units make shorter chains of more shared-memory reads: 8 channels a unit 490 us, 16 channels 450 to 475.
+template <int K1, int C1>
+constexpr int kUnits = Win<K1>::MB * (C1 / 16);
+template <int K1, int C1>
+__device__ __forceinline__ void first_sums(const First &f, int p0, int p1, int block0, int ring_px, int unit, uint32_t ring, uint32_t patch,
+                                           Pipe *pipe, int32_t *status) {
+    using WN = Win<K1>;
+    constexpr int TP = WN::TP, KW = WN::KW, NP = WN::NP, ODD = WN::ODD, K2 = K1 * K1;
+    const int lane = threadIdx.x & 31, mi = lane >> 3, r = lane & 7;
+    const int ui = unit / (C1 / 16), uj = unit % (C1 / 16) * 2;
+    uint32_t a_off[2], b_off[2];
+#pragma unroll
+    for (int ks = 0; ks < 2; ++ks) {
+        const int ar = 16 * ks + r + (mi >= 2 ? 8 : 0), sw = TP == 32 ? (ar >> 1) & 3 : (ar >> 2) & 1;
+        a_off[ks] = (uint32_t)(ar * (TP * 2) + (((2 * ui + (mi & 1)) ^ sw) << 4));
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) b_off[j] = ring_offset<C1>(lane, uj + j);  // (a trip starts at a multiple of 32 pixels)
+    const int total = p1 - p0, nstages = (total + kStagePx - 1) / kStagePx;
+    const int run_trips = held(f.px_per_warp / kTrip);
+    const uint32_t ring_end = ring + (uint32_t)ring_px * (C1 * 2);  // (whole stages)
+    float *out = f.part + (size_t)block0 * (C1 * (K2 + 1));
+    float acc[2][4] = {}, sum[2][4] = {};
+    int left = run_trips, run = 0;
+    // The end of a run: eight of them, in order, make a block.
+    auto flush = [&](bool last) {
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                sum[j][q] += acc[j][q];
+                acc[j][q] = 0.f;
+            }
+        left = run_trips;
+        if (++run < 8 && !last) return;
+        const int g = lane >> 2, c = lane & 3;
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int t = 16 * ui + g + (q & 2 ? 8 : 0), co = 8 * (uj + j) + 2 * c + (q & 1);
+                const int kh = (t >> 1) / NP, kw = 2 * ((t >> 1) - kh * NP) + (t & 1) - ODD;
+                if (t < 2 * KW && kw >= 0 && kw < K1) out[co * K2 + kh * K1 + kw] = sum[j][q];
+                else if (t == 2 * KW) out[C1 * K2 + co] = sum[j][q];
+                sum[j][q] = 0.f;
+            }
+        run = 0;
+        out += C1 * (K2 + 1);
+    };
+    constexpr uint32_t kX = kTrip * TP * 2, kZ = kTrip * C1 * 2;  // bytes of a trip
+    constexpr int LA = 2;                            // trips that are fetched ahead
+    uint32_t af[2 * LA][2][4], bf[2 * LA][2][4];     // fragments
+    auto fetch_z = [&](int b, uint32_t zs) {
+#pragma unroll
+        for (int j = 0; j < 2; ++j) ldmatrix_x4_trans(zs + b_off[j], bf[b][j][0], bf[b][j][1], bf[b][j][2], bf[b][j][3]);
+    };
+    auto fetch_x = [&](int b, int ks, uint32_t xs) {
+        ldmatrix_x4_trans(xs + a_off[ks], af[b][ks][0], af[b][ks][1], af[b][ks][2], af[b][ks][3]);
+    };
+    auto products = [&](int b, int ks) {
+#pragma unroll
+        for (int j = 0; j < 2; ++j) mma_bf16_16816(acc[j], af[b][ks], bf[b][j][2 * ks], bf[b][j][2 * ks + 1]);
+    };
+    uint32_t xs = patch, zs = ring, ph = 0;
+    int ps = 0;
+    if (!mbar_wait_warp(&pipe->pfull[0], 0, &pipe->abort_flag, status)) return;
+    if (nstages > 1) {
+#pragma unroll
+        for (int t = 0; t < LA; ++t) {
+            fetch_z(t, zs + t * kZ);
+            fetch_x(t, 0, xs + t * kX);
+            fetch_x(t, 1, xs + t * kX);
+        }
+    }
+#pragma unroll 1
+    for (int s = 0; s + 1 < nstages; ++s) {
+        const int old = ps;
+        uint32_t xn = xs, zn = zs;  // of the stage that trip t + LA is in
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const int b = t % (2 * LA), n = (t + LA) % (2 * LA), u = (t + LA) & 3;
+            products(b, 0);
+            if (t + LA == 4) {
+                zn = zs + 4 * kZ;
+                if (zn == ring_end) zn = ring;
+                xn = xs + 4 * kX;
+                if (++ps == kWinStages) {
+                    ps = 0;
+                    xn = patch;
+                    ph ^= 1u;
+                }
+                if (!mbar_wait_warp(&pipe->pfull[ps], ph, &pipe->abort_flag, status)) return;
+            }
+            fetch_z(n, zn + u * kZ);
+            fetch_x(n, 0, xn + u * kX);
+            products(b, 1);
+            fetch_x(n, 1, xn + u * kX);
+            if (t < 3 && --left == 0) flush(false);
+        }
+        xs = xn;
+        zs = zn;
+        if (lane == 0) mbar_arrive(&pipe->pempty[old]);
+        __syncwarp();
+        if (--left == 0) flush(false);
+    }
+    // the last stage, trip by trip
+#pragma unroll 1
+    for (int px = (nstages - 1) * kStagePx; px < total; px += kTrip, xs += kX, zs += kZ) {
+        fetch_z(0, zs);
+        fetch_x(0, 0, xs);
+        fetch_x(0, 1, xs);
+        const int rest = total - px;
+        if (rest < kTrip) {  // behind the last pixel the ring holds something else
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int k = 8 * q + 2 * (lane & 3);
+#pragma unroll
+                for (int j = 0; j < 2; ++j) bf[0][j][q] &= (k < rest ? 0xFFFFu : 0u) | (k + 1 < rest ? 0xFFFF0000u : 0u);
+            }
+        }
+        products(0, 0);
+        products(0, 1);
+        if (--left == 0 || rest <= kTrip) flush(rest <= kTrip);
+    }
+}
+
 // GC: columns of an output group, i.e. of one pixel of one store (16, 32 or 64; its bytes are the swizzled row).
 // KS: K = 16 steps per channel chunk (1, 2 or 4: rows of 32, 64 or 128 bytes).
 // EPW: warps of an epilogue group, 4 or 8.
-template <int MODE, int GC, int KS, int EPW>
-__global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a) {
+// K1: kernel size of the first layer whose weight gradient takes the place of the output (0: none; input gradient, EPW 4, GC = C1).
+template <int MODE, int GC, int KS, int EPW, int K1>
+__device__ __forceinline__ void halo_body(const Args &a, const First &f, const __half *depth, uint8_t *smem_raw) {
     constexpr int NH = EPW == 4 ? 2 : 1;  // halves of 64 columns a warp works on
-    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    constexpr uint32_t kPatchBytes = K1 > 0 ? kWinStages * kStagePx * Win<K1 ? K1 : 3>::TP * 2 : 0;
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t smem_base = smem_u32(smem);
     // A slots, then weights (reads of the last slot's halo rows may run on into them), output staging, pipeline state
     const uint32_t w_base = smem_base + a.slots_bytes;
     const uint32_t w_bytes = (uint32_t)a.nchunks * a.w_chunk;
     const uint32_t stg_off = (a.slots_bytes + w_bytes + 1023u) & ~1023u;
-    Pipe *pipe = reinterpret_cast<Pipe *>(smem + stg_off + (size_t)(a.nbuf * a.neg) * a.stg_bytes);
+    Pipe *pipe = reinterpret_cast<Pipe *>(smem + stg_off + (K1 > 0 ? (size_t)f.ring_bytes + kPatchBytes : (size_t)(a.nbuf * a.neg) * a.stg_bytes));
     volatile int *abort_flag = &pipe->abort_flag;
     const int warp = warp_index(), lane = threadIdx.x & 31;
     const int nacc = a.nacc;
@@ -197,6 +480,16 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
             mbar_init(&pipe->tempty[i], EPW * 32);
         }
         mbar_init(&pipe->wfull, 1);
+        if constexpr (K1 > 0) {
+            for (int i = 0; i < f.groups; ++i) {
+                mbar_init(&pipe->gfull[i], (uint32_t)(a.xsegs * EPW * 32));
+                mbar_init(&pipe->gempty[i], 1);
+            }
+            for (int i = 0; i < kWinStages; ++i) {
+                mbar_init(&pipe->pfull[i], kStagePx / kTrip);
+                mbar_init(&pipe->pempty[i], kUnits<K1, GC>);
+            }
+        }
         pipe->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -217,7 +510,27 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
 
     // contiguous run of tiles for this CTA
     const int q = a.tiles / (int)gridDim.x, rem = a.tiles - q * (int)gridDim.x, bid = (int)blockIdx.x;
-    const int t0 = bid * q + (bid < rem ? bid : rem), nt = q + (bid < rem ? 1 : 0);
+    int t0 = bid * q + (bid < rem ? bid : rem), nt = q + (bid < rem ? 1 : 0);
+    // with the first layer's sums: the tiles of the row groups that hold the pixels of its blocks
+    int p0 = 0, p1 = 0, block0 = 0;
+    GroupWalk first_group;
+    if constexpr (K1 > 0) {
+        const int bq = f.blocks / (int)gridDim.x, br = f.blocks - bq * (int)gridDim.x, nb = bq + (bid < br ? 1 : 0);
+        block0 = bid * bq + (bid < br ? bid : br);
+        p0 = block0 * 8 * f.px_per_warp;
+        p1 = (int)min((long long)f.M, (long long)(block0 + nb) * 8 * f.px_per_warp);
+        auto group_of = [&](int px, int &k, int &start) -> int {  // its number over all images, and where it starts
+            const int img = px / (a.Hi * a.Wi), in = px - img * a.Hi * a.Wi;
+            k = in / f.group_px;
+            start = img * a.Hi * a.Wi + k * f.group_px;
+            return img * a.ysegs + k;
+        };
+        int k, start, k1, start1;
+        const int g0 = group_of(p0, k, start), g1 = group_of(p1 - 1, k1, start1);
+        first_group.init(a, f, k, start - p0);
+        t0 = g0 * a.xsegs;
+        nt = (g1 - g0 + 1) * a.xsegs;
+    }
 
     if (warp == 0) {
         {
@@ -353,6 +666,12 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
             __syncwarp();
             if (++acc == nacc) { acc = 0; aph ^= 1u; }
         }
+    } else if (K1 > 0 && warp >= 10) {
+        if constexpr (K1 > 0) {
+            const uint32_t patch_off = stg_off + f.ring_bytes;
+            if (warp < 10 + kBuildWarps) first_windows<K1>(f, a.Hi, a.Wi, depth, p0, p1, first_group, warp - 10, smem + patch_off, pipe, a.status);
+            else first_sums<K1, GC>(f, p0, p1, block0, first_group.ring_px, warp - 10 - kBuildWarps, smem_base + stg_off, smem_base + patch_off, pipe, a.status);
+        }
     } else {
         // ---------------- epilogue: warp reads TMEM lanes 32 (warp % 4) .. +31 and, of every 64 columns, half `h`
         const int lg = warp & 3, eg = (warp - 2) / EPW, h = EPW == 4 ? 0 : ((warp - 2) >> 2) & 1;
@@ -426,6 +745,66 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
         };
         TileAt t_next = t;
         if (eg < nt) fetch_gates(t);
+        if constexpr (K1 > 0) {
+            // The input gradient of the first layer's output goes into the ring its weight gradient is summed from, pixel by pixel.
+            GroupWalk grp = first_group;
+            const int xsegs = held(a.xsegs), Hi = held(a.Hi), Wi = held(a.Wi), B = held(a.B), Hr = held(a.Hr), Wr = held(a.Wr);
+            int xs = 0;  // of the tile in its row group
+            auto next_tile = [&]() {
+                if (++xs == xsegs) {
+                    xs = 0;
+                    grp.next();
+                }
+            };
+            for (int k = 0; k < eg; ++k) next_tile();
+            const uint32_t ring = smem_base + stg_off;
+            for (int li = eg; li < nt; li += a.neg, t = t_next) {
+                const int n = t.n + ci, y = t.y + cr, x = t.x + cx;
+                const bool live = cell && n < B && y < Hr && x < Wr;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) gate[k] = gate_n[k];
+                for (int k = 0; k < a.neg; ++k) t_next.next(a);
+                if (li + a.neg < nt) fetch_gates(t_next);
+                const int gi = grp.i, slot = grp.slot;
+                const uint32_t gph = grp.ph;
+                for (int k = 0; k < a.neg; ++k) next_tile();
+                if (!mbar_wait_warp(&pipe->gempty[gi], gph ^ 1u, abort_flag, a.status)) break;
+                if (!mbar_wait_warp(&pipe->tfull[acc], aph, abort_flag, a.status)) break;
+                tc_fence_after();
+                const uint32_t lane_base = tmem_base + (uint32_t)(acc * a.acc_cols) + ((uint32_t)(lg * 32) << 16);
+#pragma unroll 1
+                for (int q = 0; q < GC / 8; ++q) {  // (rolled: the roles' loops share the instruction cache)
+                    float v[32];
+                    tmem_ld32(lane_base + (uint32_t)(32 * q), v);
+                    if (q == GC / 8 - 1) {
+                        tc_fence_before();
+                        mbar_arrive(&pipe->tempty[acc]);
+                    }
+                    const uint32_t gw = q == 0 ? gate[0] : (q == 1 ? gate[1] : (q == 2 ? gate[2] : gate[3]));
+#pragma unroll
+                    for (int h16 = 0; h16 < 32; h16 += GC) {
+                        const int cls = GC == 32 ? q : 2 * q + h16 / 16, ph = cls >> 1, pw = (cls ^ ph) & 1;
+                        int row = slot + (2 * cr + ph) * Wi + 2 * x + pw;
+                        const bool put_it = live && row >= 0 && 2 * y + ph < Hi && 2 * x + pw < Wi;
+                        if (row >= grp.ring_px) row -= grp.ring_px;
+                        uint32_t pk[GC / 2];
+#pragma unroll
+                        for (int j = 0; j < GC / 2; ++j)
+                            pk[j] = pack_bf16x2(v[h16 + 2 * j], v[h16 + 2 * j + 1]) & gate_mask(gw, h16 / 2 + j);
+                        if (put_it) {
+#pragma unroll
+                            for (int c = 0; c < GC / 8; ++c)
+                                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(ring + ring_offset<GC>(row, c)), "r"(pk[4 * c]),
+                                             "r"(pk[4 * c + 1]), "r"(pk[4 * c + 2]), "r"(pk[4 * c + 3])
+                                             : "memory");
+                        }
+                    }
+                }
+                mbar_arrive(&pipe->gfull[gi]);
+                acc += a.neg;
+                if (acc >= nacc) { acc = eg; aph ^= 1u; }
+            }
+        } else
         for (int li = eg; li < nt; li += a.neg, t = t_next) {
             const int n = t.n + ci, y = t.y + cr, x = t.x + cx;
             const bool live = cell && n < a.B && y < a.Hr && x < a.Wr;
@@ -580,6 +959,28 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
         tc_fence_after();
         tmem_dealloc(tmem_base, ncols);
     }
+}
+
+template <int MODE, int GC, int KS, int EPW>
+__global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a) {
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    halo_body<MODE, GC, KS, EPW, 0>(a, First{}, nullptr, smem_raw);
+}
+
+// The input gradient of the second convolution and from it, on chip, the weight gradient of the first one, which is all it is for: the
+// gradient of the first layer's output, the largest of all, does not go through HBM (2.5 GB of writes and reads at 4096 rows of
+// 160 x 120 and 32 channels).  Its tiles' rows go into a ring of pixels in the order of the image, builder warps make the windows
+// of the frames, and two warps sum runs of pixels (mma.sync, as conv1_wgrad_mma_kernel: same bits).  What bounds it: the chain of
+// a run (500 cycles for 128 pixels by itself) and shared memory's bandwidth, which tensor core, fragments, windows and ring have to
+// share (800 cycles in place; tensor core alone 215 of them, epilogue 720 on two groups).  Measured at that size: 330 + 290 us -> 460, a
+// minibatch 3.22 -> 3.12 ms.
+// (depth is the last argument: a prepared launch is made again with other frames.)
+template <int GC, int K1>
+constexpr int kFirstThreads = (10 + kBuildWarps + kUnits<K1, GC>) * 32;
+template <int GC, int KS, int K1>
+__global__ void __launch_bounds__(kFirstThreads<GC, K1>, 1) conv_halo_first_kernel(const __grid_constant__ Args a, const __grid_constant__ First f, const __half *depth) {
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    halo_body<DG, GC, KS, 4, K1>(a, f, depth, smem_raw);
 }
 
 // --------------------------------------------------------------------- host ----
@@ -780,10 +1181,9 @@ int halo_conv_fwd(const ConvGeom &g, const bf16 *X, const bf16 *W, const FwdEpil
 }
 
 // Shape part of the input gradient's arguments; false where the layer is not covered.
-static bool plan_dgrad(Args &a, const ConvGeom &g, int ldy, int wt_ld, const DgradEpilogue &e) {
-    if (g.k != 3 || g.pad != 1 || g.Hi < 2 || g.Wi < 2 || ldy != g.Co || !e.out || e.out_f32 || e.ksplit > 1) return false;
+static bool dgrad_shape(Args &a, const ConvGeom &g, int ldy, int wt_ld) {
+    if (g.k != 3 || g.pad != 1 || g.Hi < 2 || g.Wi < 2 || ldy != g.Co) return false;
     if (g.Ci != 16 && g.Ci != 32 && g.Ci != 64) return false;
-    if (!e.mask_bits) return false;
     const int CB = chunk_of(g.Co);
     if (CB == 0 || wt_ld < g.Co || wt_ld % 8 != 0 || (size_t)9 * g.Ci * g.Co * 2 > 160 * 1024) return false;
     a.CB = CB;
@@ -794,7 +1194,11 @@ static bool plan_dgrad(Args &a, const ConvGeom &g, int ldy, int wt_ld, const Dgr
     a.nloads = a.nchunks;
     a.w_box = (uint32_t)(g.Ci * a.rb);
     a.w_chunk = 9u * a.w_box;
-    return a.nchunks <= kMaxSlots && plan(a, (g.Wi + 1) / 2, (g.Hi + 1) / 2, g.B);
+    return a.nchunks <= kMaxSlots;
+}
+static bool plan_dgrad(Args &a, const ConvGeom &g, int ldy, int wt_ld, const DgradEpilogue &e) {
+    if (!e.out || e.out_f32 || e.ksplit > 1 || !e.mask_bits) return false;
+    return dgrad_shape(a, g, ldy, wt_ld) && plan(a, (g.Wi + 1) / 2, (g.Hi + 1) / 2, g.B);
 }
 
 bool halo_dgrad_covers(const ConvGeom &g, int ldy, int wt_ld, const DgradEpilogue &e) {
@@ -806,12 +1210,11 @@ bool halo_dgrad_covers(const ConvGeom &g, int ldy, int wt_ld, const DgradEpilogu
 // The four parity classes (ph, pw) of input pixels (2y + ph, 2x + pw) side by side in the order 00, 01, 11, 10: the
 // classes that have a tap at a given shift of dY are then neighbours (all four at (0, 0), 01 | 11 at (0, 1), 11 | 10 at
 // (1, 0), 11 at (1, 1)), so every shift is one MMA of just those columns and no product with a zero weight is formed.
-int halo_conv_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, int wt_ld, const DgradEpilogue &e,
-                    int32_t *status, cudaStream_t st) {
-    Args a = {};
-    if (!status || !plan_dgrad(a, g, ldy, wt_ld, e)) return PPO_ERR_UNSUPPORTED;
+static constexpr int cls_ph[4] = {0, 0, 1, 1}, cls_pw[4] = {0, 1, 1, 0};
+
+// What the planned tiles read.
+static int dgrad_operands(Args &a, const ConvGeom &g, const bf16 *dY, const bf16 *Wt, int wt_ld) {
     const int CB = a.CB;
-    const int cls_ph[4] = {0, 0, 1, 1}, cls_pw[4] = {0, 1, 1, 0};
     int nb = 0, no = 0;
     for (int dy = 0; dy < 2; ++dy)
         for (int dx = 0; dx < 2; ++dx) {
@@ -840,6 +1243,16 @@ int halo_conv_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, 
         s = make_map_strided(&a.mapW, Wt, 2, wd, ws, wb);
         if (s != PPO_OK) return s;
     }
+    a.Hi = g.Hi;
+    a.Wi = g.Wi;
+    return PPO_OK;
+}
+
+int halo_conv_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, int wt_ld, const DgradEpilogue &e,
+                    int32_t *status, cudaStream_t st) {
+    Args a = {};
+    if (!status || !plan_dgrad(a, g, ldy, wt_ld, e)) return PPO_ERR_UNSUPPORTED;
+    PPO_TRY(dgrad_operands(a, g, dY, Wt, wt_ld));
     for (int c = 0; c < 4; ++c) {
         const int ph = cls_ph[c], pw = cls_pw[c];
         const long long dims[4] = {g.Ci, (g.Wi - pw + 1) / 2, (g.Hi - ph + 1) / 2, g.B};
@@ -848,9 +1261,122 @@ int halo_conv_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, 
         const int s = make_map_strided(&a.mapO[c], e.out + ((size_t)ph * g.Wi + pw) * g.Ci, 4, dims, str, box);
         if (s != PPO_OK) return s;
     }
-    a.Hi = g.Hi;
-    a.Wi = g.Wi;
     a.mask_bits = e.mask_bits;
     a.status = status;
     return launch(a, DG, g.Ci, st);
+}
+
+// Division of shared memory and the tile for the input gradient whose output stays on chip: room for the loads of a tile and one more,
+// and a ring of at least two row groups; fewest tiles, then the lowest groups.
+static bool plan_first(Args &a, First &f, const ConvGeom &g) {
+    const int Wr = (g.Wi + 1) / 2, Hr = (g.Hi + 1) / 2, C1 = g.Ci;
+    const size_t w = ((size_t)a.nchunks * a.w_chunk + 1023) & ~size_t(1023);
+    const size_t patch = (size_t)kWinStages * kStagePx * Win<3>::TP * 2;
+    const size_t fixed = w + patch + sizeof(Pipe) + 2048;
+    if (fixed >= kSmemMax) return false;
+    const size_t room = kSmemMax - fixed;
+    auto ring_of = [&](int groups, int R) -> size_t {  // whole stages
+        return (size_t)((groups * 2 * R * g.Wi + kStagePx - 1) / kStagePx * kStagePx) * C1 * 2;
+    };
+    auto slot_of = [&](int R, int Wp) -> size_t { return ((size_t)(R + 1) * Wp * a.rb + 127) & ~size_t(127); };
+    long long best_t = -1;
+    int least = 0;
+    for (int xs = 1; xs <= Wr && xs <= 64; ++xs) {
+        const int Wt = (Wr + xs - 1) / xs, Wp = Wt + 1;
+        if (Wt > 128) continue;
+        int top = (128 - Wt) / Wp + 1;
+        if (top > Hr) top = Hr;
+        for (int R = top; R >= 1; --R) {
+            const int ysegs = (Hr + R - 1) / R, Re = (Hr + ysegs - 1) / ysegs;
+            if ((Hr + Re - 1) / Re != ysegs) continue;
+            // Groups in flight: a builder that waits for one has by then given back all that ended kWinStages stages before its own.
+            const int ahead = kWinStages + 1;
+            int touch = 2;
+            for (int i = 0; i < ysegs; ++i) {
+                int sum = 0, n = 2;
+                for (int k = i;; k = k + 1 == ysegs ? 0 : k + 1, ++n) {
+                    sum += (k == ysegs - 1 ? g.Hi - 2 * Re * (ysegs - 1) : 2 * Re) * g.Wi;
+                    if (sum > ahead * kStagePx) break;
+                }
+                touch = n > touch ? n : touch;
+            }
+            if (touch > kMaxGroups) continue;
+            if ((size_t)(a.nloads + 1) * slot_of(Re, Wp) + 1024 + ring_of(touch, Re) > room) continue;
+            const long long tiles = (long long)g.B * ysegs * ((Wr + Wt - 1) / Wt);
+            if (best_t < 0 || tiles < best_t || (tiles == best_t && Re < a.R)) {
+                best_t = tiles;
+                a.Wt = Wt; a.R = Re;
+                least = touch;
+            }
+        }
+    }
+    if (best_t < 0 || best_t > 0x3fffffff) return false;
+    a.I = 1;
+    a.Wp = a.Wt + 1;
+    a.Rp = a.R + 1;
+    a.xsegs = (Wr + a.Wt - 1) / a.Wt;
+    a.ysegs = (Hr + a.R - 1) / a.R;
+    a.tiles = (int)best_t;
+    a.Hr = Hr; a.Wr = Wr; a.B = g.B;
+    a.epw = 4;
+    a.neg = 2;
+    a.acc_cols = a.N;
+    a.nacc = 4;
+    a.slot_bytes = (uint32_t)slot_of(a.R, a.Wp);
+    f.groups = least;
+    while (f.groups < 3 && (size_t)(a.nloads + 1) * a.slot_bytes + 1024 + ring_of(f.groups + 1, a.R) <= room) ++f.groups;
+    f.group_px = 2 * a.R * g.Wi;
+    f.last_px = (g.Hi - 2 * a.R * (a.ysegs - 1)) * g.Wi;
+    f.ring_bytes = (uint32_t)ring_of(f.groups, a.R);
+    f.ring_px = (int)(f.ring_bytes / (C1 * 2));
+    a.slots = (int)((room - 1024 - f.ring_bytes) / a.slot_bytes);
+    if (a.slots > kMaxSlots) a.slots = kMaxSlots;
+    a.slots_bytes = ((uint32_t)a.slots * a.slot_bytes + 1023u) & ~1023u;
+    a.smem = a.slots_bytes + w + f.ring_bytes + patch + sizeof(Pipe) + 1024;
+    return true;
+}
+
+// Where it pays (us of a backward pass's share, the two kernels by themselves -> here; 3x3, 32 -> 64 channels): 4096 rows of 160 x 120 (19.7 M
+// pixels of the first layer) 620 -> 460, 2048 rows of 240 x 180 (22 M) the same share, 2048 rows of 130 x 100 (6.7 M) 10 less of a
+// minibatch of 870, 1024 rows of 84 x 64 (1.4 M) 6 more of 280.  5x5 windows (twice the fragments, 2.5 times the loads of a builder)
+// take longer than the two kernels at all sizes, 16 channels too: half as much dX to keep out of HBM for the same chain.
+static bool first_shape(Args &a, First &f, const ConvGeom &g, int ldy, int wt_ld, const uint32_t *mask_bits, const FirstGrad &q) {
+    if (q.k != 3 || g.Ci != 32 || !mask_bits || q.Wf % 2 != 0) return false;
+    const long long M = (long long)g.B * g.Hi * g.Wi;
+    if (M < 4000000 || M > 0x7fff0000ll) return false;  // (pixels are 32-bit numbers here)
+    return dgrad_shape(a, g, ldy, wt_ld) && plan_first(a, f, g);
+}
+
+bool halo_first_covers(const ConvGeom &g, int ldy, int wt_ld, const uint32_t *mask_bits, const FirstGrad &q) {
+    Args a = {};
+    First f = {};
+    return first_shape(a, f, g, ldy, wt_ld, mask_bits, q);
+}
+
+template <int KS>
+static int launch_first(const Args &a, const First &f, const __half *depth, cudaStream_t st) {
+    static PerDevice<bool> set;
+    const auto fn = conv_halo_first_kernel<32, KS, 3>;
+    PPO_TRY(ppo_once_per_device(set, [&] { return ppo_allow_smem(fn, kSmemMax); }));
+    return ppo_launch(fn, dim3((unsigned)a.grid), dim3(kFirstThreads<32, 3>), a.smem, st, a, f, depth);
+}
+
+int halo_dgrad_first(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, int wt_ld, const uint32_t *mask_bits, const FirstGrad &q,
+                     const __half *depth, int32_t *status, cudaStream_t st) {
+    Args a = {};
+    First f = {};
+    if (!status || !ppo_aligned(depth, 4) || !first_shape(a, f, g, ldy, wt_ld, mask_bits, q)) return PPO_ERR_UNSUPPORTED;
+    PPO_TRY(dgrad_operands(a, g, dY, Wt, wt_ld));
+    a.mask_bits = mask_bits;
+    a.status = status;
+    f.Hf = q.Hf;
+    f.Wh = q.Wf / 2;
+    f.M = g.B * g.Hi * g.Wi;
+    f.px_per_warp = q.px_per_warp;
+    f.blocks = q.blocks;
+    f.part = q.part;
+    a.grid = q.blocks < ppo_num_sms() ? q.blocks : ppo_num_sms();
+    const int ks = a.CB >> 4;
+    if (ks == 4) return launch_first<4>(a, f, depth, st);
+    return ks == 2 ? launch_first<2>(a, f, depth, st) : launch_first<1>(a, f, depth, st);
 }

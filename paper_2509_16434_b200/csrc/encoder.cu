@@ -1015,7 +1015,7 @@ static int recorded(ppo_model *m, const PlanKey &key, cudaStream_t st, F &&make,
     return s;
 }
 
-enum { OP_FWD = 1, OP_DGRAD, OP_WGRAD, OP_CONV_WGRADS, OP_LSTM_FWD, OP_LSTM_BWD, OP_LSTM_STEP, OP_MLP_FWD, OP_MLP_BWD };
+enum { OP_FWD = 1, OP_DGRAD, OP_WGRAD, OP_CONV_WGRADS, OP_LSTM_FWD, OP_LSTM_BWD, OP_LSTM_STEP, OP_MLP_FWD, OP_MLP_BWD, OP_DGRAD_FIRST };
 
 static PlanKey plan_key(int op, const ConvGeom &g) {
     PlanKey k;
@@ -1472,22 +1472,56 @@ static int side_stream(ppo_model *m) {
     return PPO_OK;
 }
 
+// Whether conv1's weight gradient is reduced on the tensor cores, and into how many blocks of eight runs of how many pixels.
+static bool conv1_runs(const ppo_model *m, const __half *depth, int rows, int &blocks, long long &per_warp) {
+    const int C1 = m->Cs[1], KS = m->d.conv_k[0];
+    const long long M = (long long)rows * m->Hs[1] * m->Ws[1];
+    blocks = ppo_cdiv(M, 8 * 16 * 8);
+    const int cap = ppo_num_sms() * 4;
+    blocks = blocks > cap ? cap : (blocks < 1 ? 1 : blocks);
+    per_warp = (M + (long long)blocks * 8 - 1) / ((long long)blocks * 8);
+    per_warp = (per_warp + 31) / 32 * 32;
+    return C1 % 16 == 0 && C1 <= 64 && (KS == 3 || KS == 5) && m->d.W % 2 == 0 && ppo_aligned(depth, 4);
+}
+
+// conv2's input gradient and conv1's weight gradient in one launch, where the first is read by nothing but the second (no layer
+// normalisation between them); PPO_ERR_UNSUPPORTED (nothing launched) otherwise.  The second stage goes into `sums`.
+static int conv1_fused(ppo_model *m, const ppo_minibatch *mb, int row0, int rows, SumJobs &sums, cudaStream_t st) {
+    const ppo_model_desc &d = m->d;
+    const __half *depth = static_cast<const __half *>(mb->depth_f16) + (size_t)row0 * d.H * d.W;
+    const int C1 = m->Cs[1], KS = d.conv_k[0], ti = m->ti_conv[2];
+    int blocks;
+    long long per_warp;
+    if (d.norm || !conv1_runs(m, depth, rows, blocks, per_warp)) return PPO_ERR_UNSUPPORTED;
+    const long long M = (long long)rows * m->Hs[1] * m->Ws[1];
+    blocks = ppo_cdiv(M, 8 * per_warp);  // those behind the last pixel would add zeros
+    if ((size_t)blocks * C1 * (KS * KS + 1) > m->c1_cap) return PPO_ERR_SHAPE;
+    const ConvGeom g = conv_geom(m, 2, rows);
+    const FirstGrad q = {d.H, d.W, KS, blocks, (int)per_warp, m->c1_part};
+    const bf16 *Wt = m->wT + m->wT_off[ti];
+    PlanKey k = plan_key(OP_DGRAD_FIRST, g);
+    const void *p[] = {m->dact[2], Wt, m->abits[1], m->c1_part};
+    memcpy(k.p, p, sizeof(p));
+    const int s = recorded(m, k, st, [&]() -> int {
+        return halo_dgrad_first(g, m->dact[2], g.Co, Wt, wt_ld_of(g.Co), m->abits[1], q, depth, ppo_device_status_ptr(), st);
+    }, &depth, sizeof(depth));
+    if (s == PPO_OK) sums.add(m->c1_part, blocks, C1 * KS * KS, m->grad + m->tensors[0].off, C1, m->grad + m->tensors[1].off);
+    return s;
+}
+
 // conv1: weight and bias gradients only (there is no dgrad into the depth image); their second stage goes into `sums`.
 static int conv1_wgrad(ppo_model *m, const ppo_minibatch *mb, int row0, int rows, SumJobs &sums, cudaStream_t st) {
     const ppo_model_desc &d = m->d;
     const __half *depth = static_cast<const __half *>(mb->depth_f16) + (size_t)row0 * d.H * d.W;
     const int C1 = m->Cs[1], KS = d.conv_k[0];
     const long long M = (long long)rows * m->Hs[1] * m->Ws[1];
-    if (C1 % 16 == 0 && C1 <= 64 && (KS == 3 || KS == 5) && d.W % 2 == 0 && ppo_aligned(depth, 4)) {
+    int blocks;
+    long long per_warp;
+    if (conv1_runs(m, depth, rows, blocks, per_warp)) {
         // tensor-core reduction
         const int TP = KS == 3 ? 16 : 32;
         const size_t tile = (size_t)32 * TP * 2 + (size_t)32 * C1 * 2, redb = (size_t)TP * C1 * sizeof(float);
         const size_t smem = 8 * (tile > redb ? tile : redb);
-        int blocks = ppo_cdiv(M, 8 * 16 * 8);
-        const int cap = ppo_num_sms() * 4;
-        blocks = blocks > cap ? cap : (blocks < 1 ? 1 : blocks);
-        long long per_warp = (M + (long long)blocks * 8 - 1) / ((long long)blocks * 8);
-        per_warp = (per_warp + 31) / 32 * 32;
         float *dW = m->grad + m->tensors[0].off, *db = m->grad + m->tensors[1].off;
         if ((size_t)blocks * C1 * (KS * KS + 1) > m->c1_cap) return PPO_ERR_SHAPE;
 #define PPO_C1W(KS_, NB_)                                                                                    \
@@ -1516,10 +1550,10 @@ static int conv1_wgrad(ppo_model *m, const ppo_minibatch *mb, int row0, int rows
     if (C1 % cpt != 0 || lpp > 32 || (lpp & (lpp - 1)) != 0) return PPO_ERR_UNSUPPORTED;
     const int ppi = 32 / lpp;
     const size_t smem = (size_t)4 * C1 * (KS * KS + 1) * sizeof(float);
-    int blocks = ppo_cdiv(M, 4 * 256);
+    blocks = ppo_cdiv(M, 4 * 256);
     const int cap = ppo_num_sms() * 6;
     blocks = blocks > cap ? cap : (blocks < 1 ? 1 : blocks);
-    long long per_warp = (M + (long long)blocks * 4 - 1) / ((long long)blocks * 4);
+    per_warp = (M + (long long)blocks * 4 - 1) / ((long long)blocks * 4);
     per_warp = (per_warp + ppi - 1) / ppi * ppi;
     float *dW = m->grad + m->tensors[0].off, *db = m->grad + m->tensors[1].off;
     if ((size_t)blocks * C1 * (KS * KS + 1) > m->c1_cap) return PPO_ERR_SHAPE;
@@ -1664,6 +1698,7 @@ extern "C" int ppo_encoder_bwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
     // few registers and threads, conv1's wgrad the opposite, and both leave most issue slots and half the DRAM
     // bandwidth unused on their own, so they share the SMs.  (The dgrad kernels take whole SMs: nothing fits
     // beside them.)  Without a second stream the order is the plain one: wgrad, dgrad, layer by layer.
+    bool first_done = false;  // conv1's weight gradient has been formed on the way
     for (int l = L; l >= 2; --l) {
         const int ti = m->ti_conv[l];
         ConvGeom g = conv_geom(m, l, rows);
@@ -1672,6 +1707,12 @@ extern "C" int ppo_encoder_bwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
         int s = ln_bwd(l);
         if (s == PPO_OK && !fork)
             s = run_wgrad(m, ti, g, m->dact[l], g.Co, m->act[l - 1], st);
+        if (s == PPO_OK && l == 2) {
+            s = conv1_fused(m, mb, row0, rows, sums, st);
+            first_done = s == PPO_OK;
+            if (first_done) continue;
+            if (s == PPO_ERR_UNSUPPORTED) s = PPO_OK;
+        }
         if (s == PPO_OK)
             s = run_dgrad(m, g, m->dact[l], g.Co, m->wT + m->wT_off[ti], wt_ld_of(g.Co), l, e, st);
         if (s != PPO_OK) return join(s);
@@ -1682,12 +1723,12 @@ extern "C" int ppo_encoder_bwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
     }
     if (fork && L >= 2) {
         int s = fork_here();  // dZ1 is ready
-        if (s == PPO_OK) s = conv1_wgrad(m, mb, row0, rows, sums, leaf);
+        if (s == PPO_OK && !first_done) s = conv1_wgrad(m, mb, row0, rows, sums, leaf);
         if (s == PPO_OK) s = sum_partials_jobs(sums, leaf);
         if (s == PPO_OK) s = run_conv_wgrads(m, rows, st);
         return join(s);
     }
-    int s = conv1_wgrad(m, mb, row0, rows, sums, st);
+    int s = first_done ? PPO_OK : conv1_wgrad(m, mb, row0, rows, sums, st);
     if (s == PPO_OK) s = sum_partials_jobs(sums, st);
     return join(s);
 }

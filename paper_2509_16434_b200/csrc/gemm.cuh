@@ -65,6 +65,17 @@ int halo_conv_fwd(const ConvGeom &g, const bf16 *X, const bf16 *W, const FwdEpil
 bool halo_dgrad_covers(const ConvGeom &g, int ldy, int wt_ld, const DgradEpilogue &e);
 int halo_conv_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, int wt_ld, const DgradEpilogue &e,
                     int32_t *status, cudaStream_t st);
+// The input gradient of the second convolution (g) kept on chip, and the first convolution's weight gradient formed from it: `blocks` sets
+// of partial sums, each of eight runs of px_per_warp (a multiple of 32) pixels, in part[block][C1 k k (dW order) | C1 (db)], the bits
+// that conv1_wgrad_mma_kernel leaves.  Frames [B][Hf][Wf]; every block holds a pixel.
+struct FirstGrad {
+    int Hf, Wf, k;
+    int blocks, px_per_warp;
+    float *part;
+};
+bool halo_first_covers(const ConvGeom &g, int ldy, int wt_ld, const uint32_t *mask_bits, const FirstGrad &q);
+int halo_dgrad_first(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, int wt_ld, const uint32_t *mask_bits, const FirstGrad &q,
+                     const __half *depth, int32_t *status, cudaStream_t st);
 size_t tma_dgrad_weight_elems(int Ci, int k, int wt_ld);
 int tma_dgrad_weights(const bf16 *W, bf16 *Wc, int Co, int k, int Ci, int wt_ld, cudaStream_t st);
 // db (may be null; convolutions only): the bias gradient db[co] += sum over pixels of dY[.][co], taken from a

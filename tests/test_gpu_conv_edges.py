@@ -109,3 +109,42 @@ def test_gate_is_open_for_positive_activations_only(name):
     assert torch.isfinite(want).all() and float(want.norm()) > 0
     for pattern in closed[1:]:
         assert torch.equal(first_layer(pattern), want), hex(pattern)
+
+
+# Calls of 4 M pixels of the first layer and more keep the second layer's input gradient on chip (3x3, 32 channels): odd grids, a last
+# trip of fewer than 32 pixels, rows wider than a tile, several small images in flight, one and two chunks of output channels.
+@pytest.mark.parametrize("rows,H,W,C2", [(2901, 61, 90, 64), (953, 31, 530, 32), (15701, 30, 34, 48), (1301, 112, 110, 128)])
+def test_first_layer_gradient_of_a_whole_call_is_that_of_its_pieces(rows, H, W, C2):
+    """One backward call against the same rows in four: fp32 sums of the same products in another grouping.  A sum of 4 M terms
+    runs through chains of at most 200 additions, 200 x 2^-24 = 1.2e-5 of its parts; one trip of 32 pixels left out is 3e-3."""
+    w = synth.Workload("whole", rows, 1, H, W, (32, C2), (3, 3), (32,), 1, 1, P=16, A=3)
+    L, md, lay, theta, roll, action, logp, dev = base._setup(w, rows)
+    h = L.hyper
+    L.compute_gae(dev["last_value"])
+    ppo.ppo_shuffle_gather_minibatch(L.buffer, 5, 0, 0, 1, L.mb)
+    n = sum(s for _, s in L.model.tensors()[:2])
+    o0 = L.model.tensors()[0][0]
+
+    def gradients(pieces, dmean=None, dvalue=None):
+        ppo.ppo_model_zero_grad(L.model)
+        step = -(-rows // pieces)
+        for r0 in range(0, rows, step):
+            k = min(step, rows - r0)
+            ppo.ppo_encoder_fwd(L.model, L.mb, r0, k, L.mean, L.value)
+            if dmean is None:
+                L.loss.zero_()
+                ppo.ppo_loss_fwd_bwd(L.model, L.mb, 0, rows, rows, L.mean, L.value, h.clip, h.vf_coef, h.ent_coef, L.loss, L.dmean,
+                                     L.dvalue)
+                dm, dv = L.dmean, L.dvalue
+            else:
+                dm, dv = dmean[r0:r0 + k].contiguous(), dvalue[r0:r0 + k].contiguous()
+            ppo.ppo_encoder_bwd(L.model, L.mb, r0, k, dm, dv, True)
+        assert ppo.ppo_poll_status() == 0
+        return L.model.grad[o0:o0 + n].clone()
+
+    whole = gradients(1)
+    again = gradients(1)
+    pieces = gradients(4, L.dmean.clone(), L.dvalue.clone())
+    assert torch.equal(whole, again)
+    assert torch.isfinite(whole).all() and float(whole.norm()) > 0
+    assert float((whole - pieces).norm() / pieces.norm()) <= 5e-5
