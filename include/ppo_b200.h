@@ -365,6 +365,13 @@ int ppo_shuffle_gather_sequences(const ppo_buffer *buf, uint64_t seed, uint32_t 
 int ppo_policy_sample(const ppo_model *m, int rows, const float *dev_mean, const float *dev_eps, float *dev_action,
                       float *dev_logp, void *stream);
 
+/* One decision of `rows` envs: ppo_encoder_fwd on rows 0 .. rows-1 of `obs`, then ppo_policy_sample with its mean, in fewer launches.  A
+ * recurrent model first takes the one-step sequence (done uint8 [rows], h and c fp32 [n_lstm][rows][lstm_h]) as ppo_model_set_sequence
+ * with T = 1 does, and leaves in h and c, in place, what ppo_model_read_state gives afterwards; otherwise done, h and c are NULL
+ * (else INVALID_ARG).  Results and later calls are those of the separate ones. */
+int ppo_policy_step(ppo_model *m, const ppo_minibatch *obs, int rows, const uint8_t *dev_done, float *dev_h, float *dev_c,
+                    const float *dev_eps, float *dev_mean, float *dev_value, float *dev_action, float *dev_logp, void *stream);
+
 /* actions <- pi(stack(obs)) followed by D <- D U {...} without a copy in between (Algorithm 2): runs the
  * encoder on the observation already stored in slab row t of `buf` (all N envs, in micro-batches of the bound
  * size), draws action = mu + exp(logsigma) * eps from caller-supplied standard-normal noise dev_eps [N][A],

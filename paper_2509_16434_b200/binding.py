@@ -30,7 +30,7 @@ EXPORTS = [
     "ppo_adam_step", "ppo_policy_sample", "ppo_poll_status", "ppo_model_activation_ptr", "ppo_gae_static",
     "ppo_model_sync_masks", "ppo_buffer_write_obs", "ppo_buffer_write_outcome", "ppo_policy_act", "ppo_launch_count",
     "ppo_selftest_wait_timeout", "ppo_buffer_render_depth", "ppo_model_set_sequence", "ppo_shuffle_gather_sequences",
-    "ppo_model_read_state", "ppo_state_reset",
+    "ppo_model_read_state", "ppo_state_reset", "ppo_policy_step",
 ]
 
 
@@ -103,6 +103,7 @@ def lib():
         L.ppo_adam_step.argtypes = [C.c_void_p, C.c_float, C.c_float, C.c_float, C.c_float, C.c_int64, C.c_void_p]
         L.ppo_policy_sample.argtypes = [C.c_void_p, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p,
                                         C.c_void_p]
+        L.ppo_policy_step.argtypes = [C.c_void_p, C.POINTER(Minibatch), C.c_int] + [C.c_void_p] * 9
         L.ppo_poll_status.argtypes = [C.c_void_p]
         L.ppo_buffer_write_obs.argtypes = [C.c_void_p, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p]
         L.ppo_buffer_write_outcome.argtypes = [C.c_void_p, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p]
@@ -423,6 +424,12 @@ def ppo_encoder_bwd(m: Model, mb: MinibatchArrays, row0: int, rows: int, dmean, 
 
 def ppo_adam_step(m: Model, lr: float, beta1: float, beta2: float, eps: float, step: int, stream=None):
     _check(lib().ppo_adam_step(m.handle, lr, beta1, beta2, eps, step, _stream(stream)), "ppo_adam_step")
+
+
+def ppo_policy_step(m: Model, obs: Minibatch, rows: int, done, h, c, eps, mean, value, action, logp, stream=None):
+    """One decision: forward pass, sampling and, for a recurrent model (else done, h, c are None), the state in place."""
+    _check(lib().ppo_policy_step(m.handle, _mbref(obs), rows, _ptr(done), _ptr(h), _ptr(c), _ptr(eps), _ptr(mean), _ptr(value),
+                                 _ptr(action), _ptr(logp), _stream(stream)), "ppo_policy_step")
 
 
 def ppo_policy_act(m: Model, buf: Buffer, t: int, eps, stream=None):

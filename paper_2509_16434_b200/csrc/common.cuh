@@ -90,6 +90,14 @@ struct ppo_tensor {
 
 struct ppo_plans;  // recorded launches of a model (launch.cuh)
 
+// What a decision wants of a forward pass besides mean and value; the kernels that can write it say so, the rest is made behind them.
+struct ActTail {
+    const float *eps;
+    float *action, *logp;      // the sampled action and its log-density
+    float *h_out, *c_out;      // state of a one-step sequence (null: feed-forward), as ppo_model_read_state gives it
+    bool sampled, state_read;  // set by the forward pass
+};
+
 struct ppo_model {
     ppo_model_desc d;
     int L, F;
@@ -157,11 +165,19 @@ struct ppo_model {
     // forward/backward pairing
     int last_row0, last_rows;
     bool fwd_valid;
+    ActTail *tail = nullptr;  // of the decision whose forward pass this is
     ppo_plans *plans = nullptr;
     // second stream of the backward pass with its fork and join events (made on first use)
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
 };
+
+// action = mean + exp(logsigma) eps and one component's share of its log-density.
+#define PPO_HALF_LOG_2PI 0.91893853320467274178f
+__device__ __forceinline__ float sample_action(float mean, float logsigma, float eps, float &logp) {
+    logp += -0.5f * eps * eps - logsigma - PPO_HALF_LOG_2PI;
+    return mean + expf(logsigma) * eps;
+}
 
 __device__ __forceinline__ float bf2f(bf16 x) { return __bfloat162float(x); }
 

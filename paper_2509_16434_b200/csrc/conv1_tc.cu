@@ -43,7 +43,6 @@ constexpr int kStgBytes = 2048;  // an epilogue warp's staging tile; it has two
 
 struct Args {
     CUtensorMap map_out, map_xhat;
-    const __half *depth;
     const bf16 *W;      // [C1][k*k] bf16
     const float *bias;  // [C1]
     uint32_t *bits;     // [M][C1 / 32], [M] half words for C1 = 16, or null
@@ -114,8 +113,9 @@ struct PixAt {
 // T: tiles per stage (one barrier round trip and one accumulator hand-over each).
 // DIRECT: builders read the frames from global memory themselves; for frames so wide that a run does not fit.
 // CW: channels of an epilogue group, 32 or (C1 no multiple of 32) 16.  LN: layer normalisation (C1 == CW).
+// (depth is the last argument: a prepared launch is made again with other frames.)
 template <int KS, int T, bool DIRECT, int CW, bool LN>
-__global__ void __launch_bounds__(kThreads, 1) conv1_tc_kernel(const __grid_constant__ Args a) {
+__global__ void __launch_bounds__(kThreads, 1) conv1_tc_kernel(const __grid_constant__ Args a, const __half *depth) {
     using WN = Win<KS>;
     constexpr int K2 = KS * KS, KP = WN::KP, P = WN::P, ODD = WN::ODD, NP = WN::NP, KW = WN::KW;
     constexpr uint32_t kTileBytes = 128u * KP * 2u, kStageBytes = T * kTileBytes;
@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv1_tc_kernel(const __grid_cons
         // ---------------- loader: one bulk copy per stage.  The few words in front of the first or behind the last
         // 16-byte unit of all frames (where the unit would reach outside them) are copied by hand.
         if (!DIRECT && lane == 0) {
-            const uint32_t *frames = reinterpret_cast<const uint32_t *>(a.depth);
+            const uint32_t *frames = reinterpret_cast<const uint32_t *>(depth);
             const uintptr_t lo_all = reinterpret_cast<uintptr_t>(frames), hi_all = lo_all + (uintptr_t)a.words * 4;
             PixAt first, last;
             first.init(a, (long long)s0 * T * 128);
@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv1_tc_kernel(const __grid_cons
     } else if (warp < kBuildWarps) {
         // ---------------- builders: thread r of group q fills row r of tiles q, q + 2, .. of every stage
         const int grp = threadIdx.x >> 7, r = threadIdx.x & 127;
-        const uint32_t *frames = reinterpret_cast<const uint32_t *>(a.depth);
+        const uint32_t *frames = reinterpret_cast<const uint32_t *>(depth);
         const int d_w = 256 % a.Wo, d_h = 256 / a.Wo;
         long long m = ((long long)s0 * T + grp) * 128 + r;
         PixAt at;
@@ -407,16 +407,16 @@ __global__ void __launch_bounds__(kThreads, 1) conv1_tc_kernel(const __grid_cons
 }
 
 template <int KS, int T, bool DIRECT, int CW, bool LN>
-int launch_one(const Args &a, size_t smem, cudaStream_t st) {
+int launch_one(const Args &a, const __half *depth, size_t smem, cudaStream_t st) {
     static PerDevice<bool> set;
     const auto fn = conv1_tc_kernel<KS, T, DIRECT, CW, LN>;
     PPO_TRY(ppo_once_per_device(set, [&] { return ppo_allow_smem(fn, kSmemMax); }));
     const int sms = ppo_num_sms(), nstage = (a.tiles + T - 1) / T;
-    return ppo_launch(fn, dim3(nstage < sms ? nstage : sms), dim3(kThreads), smem, st, a);
+    return ppo_launch(fn, dim3(nstage < sms ? nstage : sms), dim3(kThreads), smem, st, a, depth);
 }
 
 template <int KS, int T, int CW>
-int launch(Args &a, cudaStream_t st) {
+int launch(Args &a, const __half *depth, cudaStream_t st) {
     constexpr int KP = Win<KS>::KP;
     constexpr size_t stage = (size_t)T * 128 * KP * 2;
     a.stages = (int)(96 * 1024 / stage);
@@ -430,14 +430,14 @@ int launch(Args &a, cudaStream_t st) {
     const bool direct = fixed + kRaw * (size_t)raw > kSmemMax;
     a.raw_bytes = direct ? 0u : (uint32_t)raw;
     const size_t smem = fixed + kRaw * (size_t)a.raw_bytes;
-    if (a.ln_gamma) return direct ? launch_one<KS, T, true, CW, true>(a, smem, st) : launch_one<KS, T, false, CW, true>(a, smem, st);
-    return direct ? launch_one<KS, T, true, CW, false>(a, smem, st) : launch_one<KS, T, false, CW, false>(a, smem, st);
+    if (a.ln_gamma) return direct ? launch_one<KS, T, true, CW, true>(a, depth, smem, st) : launch_one<KS, T, false, CW, true>(a, depth, smem, st);
+    return direct ? launch_one<KS, T, true, CW, false>(a, depth, smem, st) : launch_one<KS, T, false, CW, false>(a, depth, smem, st);
 }
 
 template <int KS>
-int launch_c(Args &a, cudaStream_t st) {
-    if (a.C1 % 32 == 0) return launch<KS, 4, 32>(a, st);
-    return a.C1 == 16 ? launch<KS, 8, 16>(a, st) : launch<KS, 4, 16>(a, st);  // 8 tiles: 128 accumulator columns
+int launch_c(Args &a, const __half *depth, cudaStream_t st) {
+    if (a.C1 % 32 == 0) return launch<KS, 4, 32>(a, depth, st);
+    return a.C1 == 16 ? launch<KS, 8, 16>(a, depth, st) : launch<KS, 4, 16>(a, depth, st);  // 8 tiles: 128 accumulator columns
 }
 
 }  // namespace
@@ -452,7 +452,7 @@ int conv1_tc_fwd(const __half *depth, const bf16 *W, const float *bias, bf16 *ou
     if (ln_gamma && ((C1 != 16 && C1 != 32) || !ln_beta || !ln_xhat || !ln_rstd)) return PPO_ERR_UNSUPPORTED;
     if (Wi % 2 != 0 || !ppo_aligned(depth, 4)) return PPO_ERR_UNSUPPORTED;
     Args a = {};
-    a.depth = depth; a.W = W; a.bias = bias; a.bits = bits;
+    a.W = W; a.bias = bias; a.bits = bits;
     a.ln_gamma = ln_gamma; a.ln_beta = ln_beta; a.ln_rstd = ln_rstd;
     a.M = (long long)rows * Ho * Wo;
     a.words = (long long)rows * Hi * (Wi / 2);
@@ -467,8 +467,8 @@ int conv1_tc_fwd(const __half *depth, const bf16 *W, const float *bias, bf16 *ou
     const int box[2] = {CW, 32};
     PPO_TRY(make_map_strided(&a.map_out, out, 2, dims, str, box));
     if (ln_gamma) PPO_TRY(make_map_strided(&a.map_xhat, ln_xhat, 2, dims, str, box));
-    if (ks == 3) return launch_c<3>(a, st);
-    if (ks == 5) return launch_c<5>(a, st);
-    if (ks == 7) return launch_c<7>(a, st);
+    if (ks == 3) return launch_c<3>(a, depth, st);
+    if (ks == 5) return launch_c<5>(a, depth, st);
+    if (ks == 7) return launch_c<7>(a, depth, st);
     return PPO_ERR_UNSUPPORTED;
 }

@@ -775,22 +775,24 @@ __global__ void __launch_bounds__(256) concat_proprio_kernel(const float *__rest
 }
 
 // h0[b] = [ReLU(bias + the slabs' partial products in order), proprio[b]] as bf16: second stage of a split embedding.
-__global__ void __launch_bounds__(256) embed_finish_kernel(const float *__restrict__ part, int slabs, const float *__restrict__ bias,
-                                                           const float *__restrict__ proprio, bf16 *__restrict__ h0, int rows,
-                                                           int E, int P) {
-    grid_wait();
-    const int ld = E + P, i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= rows * ld) return;
+struct EmbedFinish {
+    const float *part, *bias, *proprio;
+    bf16 *h0;
+    int slabs, rows, E, P;
+};
+__device__ __forceinline__ void embed_finish_at(const EmbedFinish &q, int i) {
+    const int ld = q.E + q.P;
+    if (i >= q.rows * ld) return;
     const int b = i / ld, j = i - b * ld;
     float v;
-    if (j < E) {
-        v = bias[j];
-        for (int s = 0; s < slabs; ++s) v += part[((size_t)s * rows + b) * E + j];
+    if (j < q.E) {
+        v = q.bias[j];
+        for (int s = 0; s < q.slabs; ++s) v += q.part[((size_t)s * q.rows + b) * q.E + j];
         v = fmaxf(v, 0.f);
     } else {
-        v = proprio[(size_t)b * P + j - E];
+        v = q.proprio[(size_t)b * q.P + j - q.E];
     }
-    h0[i] = __float2bfloat16_rn(v);
+    q.h0[i] = __float2bfloat16_rn(v);
 }
 
 // dz[b][e] = dh0[b][e] where the embedding h0[b][e] is > 0, else 0 (back through its ReLU), as a bf16 GEMM operand.
@@ -891,10 +893,17 @@ struct InitJobs {
     bf16 *hprev[PPO_MAX_LSTM];
     float *cprev[PPO_MAX_LSTM];
 };
+// The last blocks (behind the gridDim.x - init_blocks ones of the states) finish the split embedding q of an acting step, which the state
+// does not depend on: a launch less in a decision.
 template <int V>
-__global__ void __launch_bounds__(256) lstm_init_kernel(const float *__restrict__ h_init, const float *__restrict__ c_init, InitJobs jobs, int n) {
+__global__ void __launch_bounds__(256) lstm_init_kernel(const float *__restrict__ h_init, const float *__restrict__ c_init, InitJobs jobs, int n,
+                                                        int init_blocks, EmbedFinish q) {
     grid_wait();
-    const int i = (blockIdx.x * blockDim.x + threadIdx.x) * V, l = blockIdx.y;
+    if ((int)blockIdx.x >= init_blocks) {
+        embed_finish_at(q, ((int)blockIdx.x - init_blocks) * (int)blockDim.x + (int)threadIdx.x);
+        return;
+    }
+    const int per = (n + 256 * V - 1) / (256 * V), l = (int)blockIdx.x / per, i = (((int)blockIdx.x - l * per) * 256 + (int)threadIdx.x) * V;
     if (i >= n) return;
     const float *h = h_init + (size_t)l * n + i, *c = c_init + (size_t)l * n + i;
     if constexpr (V == 4) {
@@ -906,10 +915,20 @@ __global__ void __launch_bounds__(256) lstm_init_kernel(const float *__restrict_
         jobs.cprev[l][i] = *c;
     }
 }
-static int lstm_init(const float *h_init, const float *c_init, const InitJobs &jobs, int layers, int n, cudaStream_t st) {
+static int lstm_init(const float *h_init, const float *c_init, const InitJobs &jobs, int layers, int n, cudaStream_t st, const EmbedFinish &q = {}) {
     const bool wide = n % 4 == 0 && ppo_aligned(h_init, 16) && ppo_aligned(c_init, 16);
-    return ppo_launch(wide ? lstm_init_kernel<4> : lstm_init_kernel<1>, dim3(ppo_cdiv(n, wide ? 1024 : 256), layers), dim3(256), 0, st, h_init,
-                      c_init, jobs, n);
+    const int init_blocks = ppo_cdiv(n, wide ? 1024 : 256) * layers, embed_blocks = q.part ? ppo_cdiv((long long)q.rows * (q.E + q.P), 256) : 0;
+    return ppo_launch(wide ? lstm_init_kernel<4> : lstm_init_kernel<1>, dim3(init_blocks + embed_blocks), dim3(256), 0, st, h_init, c_init, jobs, n,
+                      init_blocks, q);
+}
+// The states all layers of a one-step sequence start from.
+static int lstm_init_all(ppo_model *m, cudaStream_t st, const EmbedFinish &q = {}) {
+    InitJobs jobs;
+    for (int k = 0; k < m->d.n_lstm; ++k) {
+        jobs.hprev[k] = m->lstm_hprev[k];
+        jobs.cprev[k] = m->lstm_c[k] + (size_t)m->mbmax * m->d.lstm_h;
+    }
+    return lstm_init(m->seq_h_init, m->seq_c_init, jobs, m->d.n_lstm, m->seq_Be * m->d.lstm_h, st, q);
 }
 
 // One time step of one LSTM layer for Be envs, element-wise part: gate pre-activations = xg + hg + b,
@@ -1015,7 +1034,7 @@ static int recorded(ppo_model *m, const PlanKey &key, cudaStream_t st, F &&make,
     return s;
 }
 
-enum { OP_FWD = 1, OP_DGRAD, OP_WGRAD, OP_CONV_WGRADS, OP_LSTM_FWD, OP_LSTM_BWD, OP_LSTM_STEP, OP_MLP_FWD, OP_MLP_BWD, OP_DGRAD_FIRST };
+enum { OP_FWD = 1, OP_DGRAD, OP_WGRAD, OP_CONV_WGRADS, OP_LSTM_FWD, OP_LSTM_BWD, OP_LSTM_STEP, OP_MLP_FWD, OP_MLP_BWD, OP_DGRAD_FIRST, OP_CONV1 };
 
 static PlanKey plan_key(int op, const ConvGeom &g) {
     PlanKey k;
@@ -1192,32 +1211,32 @@ static int lstm_persistent(ppo_model *m, int op, int l, cudaStream_t st, F &&mak
 }
 
 // Forward of the recurrent trunk over the announced sequence (rows = T * Be, time-major): per layer one GEMM for
-// W_x x of all rows, then per step the GEMM W_h h_prev and the element-wise cell.
-static int lstm_forward(ppo_model *m, int rows, cudaStream_t st) {
+// W_x x of all rows, then per step the GEMM W_h h_prev and the element-wise cell.  started: the states of all layers are in place.
+static int lstm_forward(ppo_model *m, int rows, bool started, cudaStream_t st) {
     const ppo_model_desc &d = m->d;
     const int T = m->seq_T, Be = m->seq_Be, H = d.lstm_h;
     if (T <= 0 || T * Be != rows || !m->seq_done) return PPO_ERR_STATE;
-    bool started = false;  // the states of all layers are in place
+    int steps = 0;  // layers that were one launch and wrote the decision's state
     for (int l = 0; l < d.n_lstm; ++l) {
         const int in = l == 0 ? m->hw[0] : H, ti = m->ti_lstm[l];
         const bf16 *X = l == 0 ? m->h[0] : m->lstm_hs[l - 1];
         float *cprev = m->lstm_c[l] + (size_t)m->mbmax * H;
         if (T == 1) {
-            if (!started) {
-                InitJobs jobs;
-                for (int k = 0; k < d.n_lstm; ++k) {
-                    jobs.hprev[k] = m->lstm_hprev[k];
-                    jobs.cprev[k] = m->lstm_c[k] + (size_t)m->mbmax * H;
-                }
-                PPO_TRY(lstm_init(m->seq_h_init, m->seq_c_init, jobs, d.n_lstm, Be * H, st));
-                started = true;
-            }
+            if (!started) PPO_TRY(lstm_init_all(m, st));
+            started = true;
             PlanKey k = plan_key(OP_LSTM_STEP, fc_geom(Be, in, l));
+            LstmStepEnds ends = {nullptr, nullptr, nullptr};
+            if (m->tail && m->tail->h_out && ppo_aligned(m->tail->h_out, 16) && ppo_aligned(m->tail->c_out, 16))
+                ends = {m->tail->h_out + (size_t)l * Be * H, m->tail->c_out + (size_t)l * Be * H, m->seq_done};
             const int one = recorded(m, k, st, [&]() -> int {
                 return lstm_one_step(lstm_steps(m, l), X, in, m->shadow + m->tensors[ti].off, m->shadow + m->tensors[ti + 1].off,
-                                     m->master + m->tensors[ti + 2].off, ppo_device_status_ptr(), st);
-            });
-            if (one == PPO_OK) continue;
+                                     m->master + m->tensors[ti + 2].off, ends, ppo_device_status_ptr(), st);
+            }, &ends, sizeof(ends));
+            if (one == PPO_OK) {
+                if (m->tail && l == d.n_lstm - 1) m->tail->state_read = ends.h_out != nullptr && steps == l;
+                ++steps;
+                continue;
+            }
             if (one != PPO_ERR_UNSUPPORTED) return one;
         }
         PPO_TRY(gemm_nt_f32(m, rows, 4 * H, in, X, in, m->shadow + m->tensors[ti].off, m->lstm_xg, st));
@@ -1302,11 +1321,19 @@ extern "C" int ppo_encoder_fwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
         const int C1 = m->Cs[1], KS = d.conv_k[0];
         const long long M = (long long)rows * m->Hs[1] * m->Ws[1];
         const bool norm = d.norm != 0;
-        const int tcs = conv1_tc_fwd(depth, m->shadow + m->tensors[0].off, m->master + m->tensors[1].off, m->act[1],
-                                     m->abits[1], rows, d.H, d.W, m->Hs[1], m->Ws[1], C1, KS,
-                                     norm ? m->master + m->tensors[2].off : nullptr,
-                                     norm ? m->master + m->tensors[3].off : nullptr, norm ? m->xhat[1] : nullptr,
-                                     norm ? m->rstd[1] : nullptr, ppo_device_status_ptr(), st);
+        int tcs = PPO_ERR_UNSUPPORTED;
+        if (ppo_aligned(depth, 4)) {
+            PlanKey k = plan_key(OP_CONV1, fc_geom(rows, 0, 0));
+            const void *p[] = {m->shadow, m->master, m->act[1], m->abits[1], m->xhat[1], m->rstd[1]};
+            memcpy(k.p, p, sizeof(p));
+            tcs = recorded(m, k, st, [&]() -> int {
+                return conv1_tc_fwd(depth, m->shadow + m->tensors[0].off, m->master + m->tensors[1].off, m->act[1],
+                                    m->abits[1], rows, d.H, d.W, m->Hs[1], m->Ws[1], C1, KS,
+                                    norm ? m->master + m->tensors[2].off : nullptr,
+                                    norm ? m->master + m->tensors[3].off : nullptr, norm ? m->xhat[1] : nullptr,
+                                    norm ? m->rstd[1] : nullptr, ppo_device_status_ptr(), st);
+            }, &depth, sizeof(depth));
+        }
         if (tcs != PPO_OK && (tcs != PPO_ERR_UNSUPPORTED || norm)) return tcs;  // only the tensor-core kernel normalises
         const int CH = C1 / 8;
         const bool stage = CH == 1 || CH == 2 || CH == 4 || CH == 8;
@@ -1343,6 +1370,7 @@ extern "C" int ppo_encoder_fwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
         }
         PPO_TRY(run_fwd(m, g, m->act[l - 1], m->shadow + m->tensors[tc].off, e, st));
     }
+    bool started = false;  // the recurrent layers' states are in place
     if (m->ti_embed >= 0) {
         // flatten -> fully connected -> ReLU into the first E columns of h_0, proprio behind them
         const int K = m->Hs[m->L] * m->Ws[m->L] * m->Cs[m->L];
@@ -1363,8 +1391,10 @@ extern "C" int ppo_encoder_fwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
             (size_t)slabs * rows * d.embed <= m->wg_cap[m->ti_embed]) {
             PPO_TRY(gemm_nt_f32(m, rows, d.embed, K, m->act[m->L], K, m->shadow + m->tensors[m->ti_embed].off, m->wg_part[m->ti_embed],
                                 st, slabs));
-            PPO_TRY(ppo_launch(embed_finish_kernel, dim3(ppo_cdiv((long long)rows * m->hw[0], 256)), dim3(256), 0, st, part, slabs,
-                               m->master + m->tensors[m->ti_embed + 1].off, mb->proprio + (size_t)row0 * d.P, m->h[0], rows, d.embed, d.P));
+            const EmbedFinish q = {part, m->master + m->tensors[m->ti_embed + 1].off, mb->proprio + (size_t)row0 * d.P, m->h[0], slabs, rows, d.embed, d.P};
+            if (m->seq_Be != rows || !m->seq_done) return PPO_ERR_STATE;
+            PPO_TRY(lstm_init_all(m, st, q));
+            started = true;
         } else {
         FwdEpilogue e = {m->master + m->tensors[m->ti_embed + 1].off, 1, m->h[0], nullptr, nullptr, 0};
         e.ldo = m->hw[0];
@@ -1387,7 +1417,7 @@ extern "C" int ppo_encoder_fwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
                            dim3(ppo_cdiv((long long)rows * (C / (few ? 2 : 8) + d.P), 256)), dim3(256), 0, st,
                            m->act[m->L], mb->proprio + (size_t)row0 * d.P, m->h[0], rows, m->Hs[m->L] * m->Ws[m->L], C, d.P));
     }
-    if (d.n_lstm > 0) PPO_TRY(lstm_forward(m, rows, st));
+    if (d.n_lstm > 0) PPO_TRY(lstm_forward(m, rows, started, st));
     int ti = m->ti_fc[1];
     MlpLayer mlp[PPO_MAX_FC + 1] = {};
     for (int l = 1; l <= m->F + 1; ++l) {
@@ -1399,7 +1429,14 @@ extern "C" int ppo_encoder_fwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
     if (mlp_covers(mlp, m->F + 1, rows)) {
         PlanKey k = plan_key(OP_MLP_FWD, fc_geom(rows, 0, 0));
         k.p[0] = mlp[0].X;
-        const MlpEnds ends = {d.A, mean, value, nullptr, nullptr, nullptr};
+        MlpEnds ends = {d.A, mean, value, nullptr, nullptr, nullptr};
+        if (m->tail) {
+            ends.logsigma = m->master + m->tensors.back().off;
+            ends.eps = m->tail->eps;
+            ends.action = m->tail->action;
+            ends.logp = m->tail->logp;
+            m->tail->sampled = true;
+        }
         PPO_TRY(recorded(m, k, st, [&]() -> int { return mlp_chain(mlp, m->F + 1, rows, ends, ppo_device_status_ptr(), st); }, &ends, sizeof(ends)));
         m->fwd_valid = true;
         m->last_row0 = row0;

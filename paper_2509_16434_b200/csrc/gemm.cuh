@@ -122,6 +122,8 @@ struct MlpEnds {
     float *mean, *value;
     const float *dmean, *dvalue;
     bf16 *dout;
+    const float *logsigma = nullptr, *eps = nullptr;  // a head that also samples (eps null: none)
+    float *action = nullptr, *logp = nullptr;
 };
 bool mlp_covers(const MlpLayer *layers, int nl, int rows);
 int mlp_chain(const MlpLayer *layers, int nl, int rows, const MlpEnds &ends, int32_t *status, cudaStream_t st);

@@ -580,7 +580,7 @@ struct StepArgs {
 constexpr int kStepG = 2;  // chunks of a stage
 
 template <int M, int U>
-__global__ void __launch_bounds__(kThreads, 1) lstm_step_kernel(const __grid_constant__ StepArgs a) {
+__global__ void __launch_bounds__(kThreads, 1) lstm_step_kernel(const __grid_constant__ StepArgs a, const __grid_constant__ LstmStepEnds ends) {
     constexpr uint32_t kA = M * 128u, kB = 4u * U * 128u, kStageBytes = kStepG * (kA + kB);
     constexpr int W = M * U >= 2048 ? 4 : (M * U >= 1024 ? 2 : 1);  // units of a thread in a pass over the cells
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -714,6 +714,16 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_step_kernel(const __grid_con
                 store_u<W>(a.gates + r4 + 3 * H, go);
                 store_u<W>(a.c + r, cv);
                 store_bf16_u<W>(a.h + r, pack_u<W>(hv));
+                if (ends.h_out) {
+                    const bool reset = ends.done[e] != 0;
+#pragma unroll
+                    for (int k = 0; k < W; ++k) {
+                        hv[k] = reset ? 0.f : bf2f(__float2bfloat16_rn(hv[k]));
+                        cv[k] = reset ? 0.f : cv[k];
+                    }
+                    store_u<W>(ends.h_out + r, hv);
+                    store_u<W>(ends.c_out + r, cv);
+                }
             }
         }
     }
@@ -743,7 +753,7 @@ bool plan(Args &a, int T, int Be, int H, int U, int &ctas, size_t &smem) {
 }
 
 template <int M, int U>
-int launch_step(StepArgs &a, int in, const LstmSteps &p, const bf16 *X, const bf16 *Wx, const bf16 *Wh, cudaStream_t st) {
+int launch_step(StepArgs &a, int in, const LstmSteps &p, const bf16 *X, const bf16 *Wx, const bf16 *Wh, const LstmStepEnds &ends, cudaStream_t st) {
     const long long H = p.H, Be = p.Be;
     auto maps = [&](CUtensorMap &ma, CUtensorMap &mb, const bf16 *A, const bf16 *B, int K, int &chunks, int &g) -> int {
         chunks = (K + 63) / 64;
@@ -763,7 +773,7 @@ int launch_step(StepArgs &a, int in, const LstmSteps &p, const bf16 *X, const bf
     static PerDevice<bool> set;
     PPO_TRY(ppo_once_per_device(set, [] { return ppo_allow_smem(lstm_step_kernel<M, U>, kSmemMax); }));
     const unsigned ctas = (unsigned)((Be + M - 1) / M * (H / U));
-    return ppo_launch(lstm_step_kernel<M, U>, dim3(ctas), dim3(kThreads), (size_t)a.stages * stage + fixed, st, a);
+    return ppo_launch(lstm_step_kernel<M, U>, dim3(ctas), dim3(kThreads), (size_t)a.stages * stage + fixed, st, a, ends);
 }
 
 // Whether `ctas` CTAs in clusters of four are resident at once: clusters fit the groups of SMs less tightly than single CTAs (33
@@ -866,7 +876,8 @@ int lstm_bwd_steps(const LstmSteps &p, const bf16 *WhT, const float *dtop, bf16 
     return ppo_launch_together(lstm_bwd_kernel, dim3(ctas), dim3(kThreads), smem, st, a);
 }
 
-int lstm_one_step(const LstmSteps &p, const bf16 *X, int in, const bf16 *Wx, const bf16 *Wh, const float *bias, int32_t *status, cudaStream_t st) {
+int lstm_one_step(const LstmSteps &p, const bf16 *X, int in, const bf16 *Wx, const bf16 *Wh, const float *bias, const LstmStepEnds &ends,
+                  int32_t *status, cudaStream_t st) {
     if (!status || p.T != 1 || p.H % 64 != 0 || in < 64 || in % 8 != 0) return PPO_ERR_UNSUPPORTED;
     StepArgs a = {};
     a.Be = p.Be; a.H = p.H;
@@ -876,10 +887,10 @@ int lstm_one_step(const LstmSteps &p, const bf16 *X, int in, const bf16 *Wx, con
     // the shape with the fewest bytes per CTA whose CTAs all run at once; the largest up to two waves
     const long long sms = ppo_num_sms();
     auto ctas = [&](int M, int U) { return (long long)((p.Be + M - 1) / M) * (p.H / U); };
-    if (ctas(32, 8) <= sms) return launch_step<32, 8>(a, in, p, X, Wx, Wh, st);
-    if (ctas(32, 16) <= sms) return launch_step<32, 16>(a, in, p, X, Wx, Wh, st);
-    if (ctas(64, 16) <= sms) return launch_step<64, 16>(a, in, p, X, Wx, Wh, st);
-    if (ctas(128, 16) <= sms) return launch_step<128, 16>(a, in, p, X, Wx, Wh, st);
-    if (ctas(128, 32) <= 2 * sms) return launch_step<128, 32>(a, in, p, X, Wx, Wh, st);
+    if (ctas(32, 8) <= sms) return launch_step<32, 8>(a, in, p, X, Wx, Wh, ends, st);
+    if (ctas(32, 16) <= sms) return launch_step<32, 16>(a, in, p, X, Wx, Wh, ends, st);
+    if (ctas(64, 16) <= sms) return launch_step<64, 16>(a, in, p, X, Wx, Wh, ends, st);
+    if (ctas(128, 16) <= sms) return launch_step<128, 16>(a, in, p, X, Wx, Wh, ends, st);
+    if (ctas(128, 32) <= 2 * sms) return launch_step<128, 32>(a, in, p, X, Wx, Wh, ends, st);
     return PPO_ERR_UNSUPPORTED;
 }

@@ -17,7 +17,14 @@ struct LstmSteps {
 int lstm_fwd_steps(const LstmSteps &p, const bf16 *Wh, const float *xg, const float *bias, const float *h_init, const float *c_init,
                    int32_t *status, cudaStream_t st);
 // A sequence of one step, W_x x included (X [Be][in]); hprev and cprev hold the state it starts from.
-int lstm_one_step(const LstmSteps &p, const bf16 *X, int in, const bf16 *Wx, const bf16 *Wh, const float *bias, int32_t *status, cudaStream_t st);
+// ends: where the state after the step goes as well, fp32 and zero where done (null: nowhere; 16-byte aligned).  The last argument of the
+// kernel: a step prepared once is launched again with others.
+struct LstmStepEnds {
+    float *h_out, *c_out;
+    const uint8_t *done;
+};
+int lstm_one_step(const LstmSteps &p, const bf16 *X, int in, const bf16 *Wx, const bf16 *Wh, const float *bias, const LstmStepEnds &ends,
+                  int32_t *status, cudaStream_t st);
 // WhT: W_h^T [H][4H].  dhc: 4 * Be * H floats of scratch.
 int lstm_bwd_steps(const LstmSteps &p, const bf16 *WhT, const float *dtop, bf16 *dg, float *dhc, int32_t *status, cudaStream_t st);
 

@@ -307,8 +307,16 @@ __device__ __forceinline__ void chain(const Args &a, const MlpEnds &e, uint8_t *
 #pragma unroll
                             for (int i = 0; i < 16; ++i) {
                                 const int c = col0 + g + i;
-                                if (c < e.A) e.mean[(size_t)grow * e.A + c] = v[i] + pipe->bias[l * kMaxSlice + g + i];
-                                else if (c == e.A) e.value[grow] = v[i] + pipe->bias[l * kMaxSlice + g + i];
+                                v[i] += pipe->bias[l * kMaxSlice + g + i];
+                                if (c < e.A) e.mean[(size_t)grow * e.A + c] = v[i];
+                                else if (c == e.A) e.value[grow] = v[i];
+                            }
+                            if (e.eps && col0 + g == 0) {  // (at most 16 columns: they are all here)
+                                float lp = 0.f;
+#pragma unroll
+                                for (int i = 0; i < 15; ++i)
+                                    if (i < e.A) e.action[(size_t)grow * e.A + i] = sample_action(v[i], __ldg(e.logsigma + i), __ldg(e.eps + (size_t)grow * e.A + i), lp);
+                                e.logp[grow] = lp;
                             }
                         }
                         continue;

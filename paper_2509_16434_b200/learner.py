@@ -84,12 +84,8 @@ class Learner:
         if self.recurrent and (self.roll_h is None or self.roll_h.shape[1] != n):
             self.reset_rollout_state(n)
         if n <= self.microbatch:  # all envs at once: the state is read and written where it is kept
-            if self.recurrent:
-                ppo.ppo_model_set_sequence(self.model, 1, n, self.roll_done, self.roll_h, self.roll_c)
-            ppo.ppo_encoder_fwd(self.model, obs, 0, n, self.mean, value)
-            ppo.ppo_policy_sample(self.model, n, self.mean, eps, action, logp)
-            if self.recurrent:
-                ppo.ppo_model_read_state(self.model, self.roll_h, self.roll_c)
+            state = (self.roll_done, self.roll_h, self.roll_c) if self.recurrent else (None, None, None)
+            ppo.ppo_policy_step(self.model, obs, n, *state, eps, self.mean, value, action, logp)
             return action, logp, value
         for r0 in range(0, n, self.microbatch):
             rows = min(self.microbatch, n - r0)

@@ -288,3 +288,49 @@ def test_state_after_a_sequence_matches_oracle_and_chains():
         ppo.ppo_model_read_state(L.model, hs, cs)
     assert torch.equal(hs, h_out) and torch.equal(cs, c_out)
     assert ppo.ppo_poll_status() == 0
+
+
+@pytest.mark.parametrize("family", ["recurrent", "recurrent_split", "recurrent_many", "plain", "plain_wide"])
+def test_one_decision_call_is_the_separate_calls(family):
+    """ppo_policy_step against set_sequence, encoder_fwd, policy_sample and read_state: the same bits in every output and in the state, for
+    done flags of both kinds, several decisions in a row, and where the kernels that end the pass do not cover the shapes."""
+    kw = dict(norm=True, embed=32, n_lstm=2, lstm_h=128) if family.startswith("recurrent") else {}
+    n, H, W = {"recurrent": (16, 48, 64), "recurrent_split": (21, 96, 128), "recurrent_many": (301, 33, 46), "plain": (37, 40, 50),
+               "plain_wide": (5, 40, 50)}[family]
+    conv = (16, 32, 64, 128) if kw else (16, 32)
+    fc = (2000,) if family == "plain_wide" else (72, 120)  # (2000 columns: layer by layer)
+    w = synth.Workload("step", n, 2, H, W, conv, (3,) * len(conv), fc, 1, 1, P=32 if kw else 16, A=5, **kw)
+    dev = "cuda"
+    L = Learner(w, 2 * n, dev)
+    shapes, gammas = synth.param_shapes(w)
+    L.model.load(synth.init_params(L.model.arena, [o for o, _ in L.model.tensors()], shapes, 3, ones=gammas))
+    r = synth.rollout_torch(w, dev, 4)
+    g = torch.Generator(dev).manual_seed(5)
+
+    def arrays():
+        return [torch.full((n, w.A), 7.0, device=dev), torch.full((n,), 7.0, device=dev), torch.full((n, w.A), 7.0, device=dev),
+                torch.full((n,), 7.0, device=dev)]
+
+    state = [torch.randn((2, n, 128), generator=g, device=dev) for _ in range(2)] if kw else None
+    for t in range(2):
+        depth, proprio, eps = r["depth"][t], r["proprio"][t], r["eps"][t]
+        done = (torch.arange(n, device=dev) % 3 == t).to(torch.uint8) if kw else None
+        obs = ppo.Minibatch(depth.data_ptr(), proprio.data_ptr(), None, None, None, None, None, None, n)
+        mean, value, action, logp = arrays()
+        mine = [s.clone() for s in state] if kw else [None, None]
+        ppo.ppo_policy_step(L.model, obs, n, done, mine[0], mine[1], eps, mean, value, action, logp)
+        mean2, value2, action2, logp2 = arrays()
+        if kw:
+            ppo.ppo_model_set_sequence(L.model, 1, n, done, state[0], state[1])
+        ppo.ppo_encoder_fwd(L.model, obs, 0, n, mean2, value2)
+        ppo.ppo_policy_sample(L.model, n, mean2, eps, action2, logp2)
+        if kw:
+            ppo.ppo_model_read_state(L.model, state[0], state[1])
+            assert torch.equal(mine[0], state[0]) and torch.equal(mine[1], state[1])
+            assert not bool(state[0][:, done != 0].any()) and bool(state[0][:, done == 0].any())
+        assert ppo.ppo_poll_status() == 0
+        for a, b in ((mean, mean2), (value, value2), (action, action2), (logp, logp2)):
+            assert torch.equal(a, b)
+    with pytest.raises(ppo.PpoError):
+        z = torch.zeros((2, n, 128), device=dev)
+        ppo.ppo_policy_step(L.model, obs, n, None, z, None, eps, mean, value, action, logp)
