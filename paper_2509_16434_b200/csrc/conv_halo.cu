@@ -21,6 +21,7 @@
 #include <cuda.h>
 
 #include "gemm.cuh"
+#include "halo_plan.h"
 #include "launch.cuh"
 #include "tcgen05.cuh"
 #include "tma_host.cuh"
@@ -28,90 +29,13 @@
 namespace {
 
 using namespace tc;
+using namespace halo;
 
 // An epilogue group works on a tile, the groups of a CTA on alternate ones.  A group has four warps, one per TMEM lane
 // quarter: fewer meet at its barriers, and two tiles are drained at a time.  Where shared memory holds only one CTA per SM
 // and two staging buffers, a group has eight warps, two per lane quarter, which share out the columns.
 
-constexpr int kMaxSlots = 8;
-constexpr int kMaxGroups = 8;   // row groups of the ring between the input gradient and the first layer's weight gradient
-constexpr int kWinStages = 4;   // stages of window tiles, of four trips of 32 pixels each
-constexpr int kTrip = 32, kStagePx = 4 * kTrip;
-constexpr int kBuildWarps = 8;  // in two sets of four
-constexpr int kMaxOps = 9;
-constexpr size_t kSmemMax = 227 * 1024;
-
 enum { FWD = 0, FWD_LN = 1, DG = 2 };
-
-// One tap of a plane: CB / 16 MMAs over the channels of a chunk.
-struct Op {
-    uint32_t a16;    // start of the A rows inside the plane's box, in 16-byte units
-    uint32_t b16;    // start of the weights of chunk 0, in 16-byte units
-    uint32_t dcol;   // first accumulator column
-    uint32_t idesc;  // instruction descriptor (column count)
-};
-
-struct Plane {
-    int ox, oy;      // box origin relative to the tile's first output cell
-    uint32_t bytes;  // of its box
-};
-
-struct WLoad {       // one box of weights: rows of one tap (all chunks loaded one after the other)
-    int k0;          // column of the weight matrix, without the chunk
-    uint32_t off;    // destination of chunk 0
-};
-
-struct Args {
-    CUtensorMap mapA[4];    // planes
-    CUtensorMap mapW;
-    CUtensorMap mapO[4];    // output groups (forward: one map, the group is the first coordinate)
-    CUtensorMap mapX;       // normalised values
-    Op ops[kMaxOps];
-    Plane planes[4];
-    WLoad wl[kMaxOps];
-    int nplanes, nwl, nchunks, nloads, CB, rb;
-    uint32_t w_chunk;       // bytes of the weights of one chunk
-    uint32_t w_box;         // bytes of one box of weights
-    uint32_t slot_bytes, slots_bytes;  // of one slot; of all of them, rounded up
-    uint32_t stg_bytes;     // of a staging buffer
-    int stg_row;            // of a row of it, over all its output groups
-    int epw;                // warps of an epilogue group
-    int slots, nbuf, neg;   // slots, staging buffers per epilogue group, epilogue groups
-    int Wt, R, I, Wp, Rp;   // tile: Wt x R outputs of I images; cells per box row and box rows per image
-    int xsegs, ysegs, tiles;
-    int Hr, Wr, B;          // grid of outputs (forward) or of 2x2 input blocks (input gradient)
-    int N;                  // accumulator columns
-    int acc_cols, nacc;
-    int Hi, Wi;             // input gradient: the image that is written
-    const float *bias;
-    int relu;
-    uint32_t *out_bits;
-    const uint32_t *mask_bits;
-    const float *ln_gamma, *ln_beta;
-    float *ln_rstd;
-    int grid;
-    size_t smem;
-    int32_t *status;
-};
-
-// The first layer's weight gradient behind the input gradient of the second (see first_sums).
-struct First {
-    int Hf, Wh;             // frame rows, and 32-bit words of one
-    int M, px_per_warp;     // pixels of the first layer's output; of one of the eight runs that make a block of partial sums
-    int blocks;             // blocks of partial sums, dealt out over the CTAs
-    int groups, ring_px;    // row groups in flight, pixels of the ring
-    int group_px, last_px;  // pixels of a group of 2 R rows, and of the last one of an image
-    uint32_t ring_bytes;
-    float *part;            // [block][C1 k k (dW order) | C1 (db)]
-};
-
-struct Pipe {
-    uint64_t gfull[kMaxGroups], gempty[kMaxGroups], pfull[kWinStages], pempty[kWinStages];
-    uint64_t full[kMaxSlots], empty[kMaxSlots], tfull[4], tempty[4], wfull;
-    uint32_t tmem_slot;
-    int abort_flag;
-    alignas(16) float bias[256], gamma[256], beta[256];
-};
 
 template <int EPW>
 __device__ __forceinline__ void epi_sync(int eg) { asm volatile("bar.sync %0, %1;" ::"r"(1 + eg), "n"(EPW * 32) : "memory"); }
@@ -210,13 +134,6 @@ struct GroupWalk {
     }
 };
 
-// Window of the first layer as aligned pairs of fp16 frame pixels, one row of the weight gradient per pair element and one for the bias.
-template <int K1>
-struct Win {
-    static constexpr int P = K1 / 2, ODD = P & 1, NP = (K1 + ODD + 1) / 2, KW = K1 * NP;
-    static constexpr int TP = (2 * KW + 1 + 15) / 16 * 16, MB = TP / 16;
-};
-
 // Place of the 16-byte piece `piece` of ring pixel `row` (C1 channels).  Neighbouring lanes of the epilogue write every second pixel,
 // ldmatrix reads eight in a row: both go to eight different 16-byte columns of the 128-byte lines.
 template <int C1>
@@ -242,7 +159,7 @@ __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const uint32_t (&a
 // have arrived in the ring, and a row group is given back by the builder that sees the stage it ends in summed.
 template <int K1>
 __device__ __forceinline__ void first_windows(const First &f, int H1, int W1, const __half *depth, int p0, int p1, const GroupWalk &at, int bw,
-                                              uint8_t *patch, Pipe *pipe, int32_t *status) {
+                                              uint8_t *patch, FirstPipe *pipe, int32_t *status) {
     using WN = Win<K1>;
     constexpr int TP = WN::TP, KW = WN::KW, NP = WN::NP, P = WN::P, ODD = WN::ODD;
     const int lane = threadIdx.x & 31, nstages = (p1 - p0 + kStagePx - 1) / kStagePx;
@@ -329,7 +246,7 @@ template <int K1, int C1>
 constexpr int kUnits = Win<K1>::MB * (C1 / 16);
 template <int K1, int C1>
 __device__ __forceinline__ void first_sums(const First &f, int p0, int p1, int block0, int ring_px, int unit, uint32_t ring, uint32_t patch,
-                                           Pipe *pipe, int32_t *status) {
+                                           FirstPipe *pipe, int32_t *status) {
     using WN = Win<K1>;
     constexpr int TP = WN::TP, KW = WN::KW, NP = WN::NP, ODD = WN::ODD, K2 = K1 * K1;
     const int lane = threadIdx.x & 31, mi = lane >> 3, r = lane & 7;
@@ -465,6 +382,7 @@ __device__ __forceinline__ void halo_body(const Args &a, const First &f, const _
     const uint32_t w_bytes = (uint32_t)a.nchunks * a.w_chunk;
     const uint32_t stg_off = (a.slots_bytes + w_bytes + 1023u) & ~1023u;
     Pipe *pipe = reinterpret_cast<Pipe *>(smem + stg_off + (K1 > 0 ? (size_t)f.ring_bytes + kPatchBytes : (size_t)(a.nbuf * a.neg) * a.stg_bytes));
+    [[maybe_unused]] FirstPipe *const hand = static_cast<FirstPipe *>(pipe);  // (K1 > 0)
     volatile int *abort_flag = &pipe->abort_flag;
     const int warp = warp_index(), lane = threadIdx.x & 31;
     const int nacc = a.nacc;
@@ -482,12 +400,12 @@ __device__ __forceinline__ void halo_body(const Args &a, const First &f, const _
         mbar_init(&pipe->wfull, 1);
         if constexpr (K1 > 0) {
             for (int i = 0; i < f.groups; ++i) {
-                mbar_init(&pipe->gfull[i], (uint32_t)(a.xsegs * EPW * 32));
-                mbar_init(&pipe->gempty[i], 1);
+                mbar_init(&hand->gfull[i], (uint32_t)(a.xsegs * EPW * 32));
+                mbar_init(&hand->gempty[i], 1);
             }
             for (int i = 0; i < kWinStages; ++i) {
-                mbar_init(&pipe->pfull[i], kStagePx / kTrip);
-                mbar_init(&pipe->pempty[i], kUnits<K1, GC>);
+                mbar_init(&hand->pfull[i], kStagePx / kTrip);
+                mbar_init(&hand->pempty[i], kUnits<K1, GC>);
             }
         }
         pipe->abort_flag = 0;
@@ -669,8 +587,8 @@ __device__ __forceinline__ void halo_body(const Args &a, const First &f, const _
     } else if (K1 > 0 && warp >= 10) {
         if constexpr (K1 > 0) {
             const uint32_t patch_off = stg_off + f.ring_bytes;
-            if (warp < 10 + kBuildWarps) first_windows<K1>(f, a.Hi, a.Wi, depth, p0, p1, first_group, warp - 10, smem + patch_off, pipe, a.status);
-            else first_sums<K1, GC>(f, p0, p1, block0, first_group.ring_px, warp - 10 - kBuildWarps, smem_base + stg_off, smem_base + patch_off, pipe, a.status);
+            if (warp < 10 + kBuildWarps) first_windows<K1>(f, a.Hi, a.Wi, depth, p0, p1, first_group, warp - 10, smem + patch_off, hand, a.status);
+            else first_sums<K1, GC>(f, p0, p1, block0, first_group.ring_px, warp - 10 - kBuildWarps, smem_base + stg_off, smem_base + patch_off, hand, a.status);
         }
     } else {
         // ---------------- epilogue: warp reads TMEM lanes 32 (warp % 4) .. +31 and, of every 64 columns, half `h`
@@ -768,7 +686,7 @@ __device__ __forceinline__ void halo_body(const Args &a, const First &f, const _
                 const int gi = grp.i, slot = grp.slot;
                 const uint32_t gph = grp.ph;
                 for (int k = 0; k < a.neg; ++k) next_tile();
-                if (!mbar_wait_warp(&pipe->gempty[gi], gph ^ 1u, abort_flag, a.status)) break;
+                if (!mbar_wait_warp(&hand->gempty[gi], gph ^ 1u, abort_flag, a.status)) break;
                 if (!mbar_wait_warp(&pipe->tfull[acc], aph, abort_flag, a.status)) break;
                 tc_fence_after();
                 const uint32_t lane_base = tmem_base + (uint32_t)(acc * a.acc_cols) + ((uint32_t)(lg * 32) << 16);
@@ -800,7 +718,7 @@ __device__ __forceinline__ void halo_body(const Args &a, const First &f, const _
                         }
                     }
                 }
-                mbar_arrive(&pipe->gfull[gi]);
+                mbar_arrive(&hand->gfull[gi]);
                 acc += a.neg;
                 if (acc >= nacc) { acc = eg; aph ^= 1u; }
             }
@@ -985,105 +903,13 @@ __global__ void __launch_bounds__(kFirstThreads<GC, K1>, 1) conv_halo_first_kern
 
 // --------------------------------------------------------------------- host ----
 
-uint32_t stage_rows_bytes(int rows, int row_bytes) { return ((uint32_t)(rows * row_bytes) + 1023u) & ~1023u; }
-
-// Tile rectangle whose loads (`loads` slots) and staging buffers (`bufs`) fit into `room` bytes: fewest tiles over the
-// whole grid, then fewest loaded cells.  The M rows of a tile (halo cells included, except behind its last row) have to
-// fit into the 128 rows of an MMA.
-bool choose_tile(Args &a, int Wr, int Hr, int B, size_t room, int loads, int bufs) {
-    long long best_t = -1, best_c = 0;
-    for (int xs = 1; xs <= Wr && xs <= 64; ++xs) {
-        const int Wt = (Wr + xs - 1) / xs, Wp = Wt + 1;
-        if (Wt > 128) continue;
-        int top = (128 - Wt) / Wp + 1;
-        if (top > Hr) top = Hr;
-        for (int R = top; R >= 1; --R) {
-            const int ysegs = (Hr + R - 1) / R;
-            if (R < top && (Hr + R) / (R + 1) == ysegs) continue;  // a taller tile makes as few segments
-            const int Re = (Hr + ysegs - 1) / ysegs;
-            int I = 1;
-            if (ysegs == 1 && xs == 1) {
-                const int per = (Re + 1) * Wp, last = (Re - 1) * Wp + Wt;
-                I = 1 + (128 - last) / per;
-                if (I > B) I = B;
-            }
-            auto fits = [&](int img) {
-                const size_t slot = ((size_t)img * (Re + 1) * Wp * a.rb + 127) & ~size_t(127);
-                return (size_t)loads * slot + (size_t)bufs * stage_rows_bytes(img * Re * Wt, a.stg_row) <= room;
-            };
-            while (I > 1 && !fits(I)) --I;
-            if (!fits(I)) continue;
-            const long long tiles = (long long)((B + I - 1) / I) * ysegs * ((Wr + Wt - 1) / Wt);
-            const long long cells = tiles * I * (Re + 1) * Wp;
-            if (best_t < 0 || tiles < best_t || (tiles == best_t && cells < best_c)) {
-                best_t = tiles; best_c = cells;
-                a.Wt = Wt; a.R = Re; a.I = I;
-            }
-        }
-    }
-    if (best_t < 0 || best_t > 0x3fffffff) return false;
-    a.Wp = a.Wt + 1;
-    a.Rp = a.R + 1;
-    a.xsegs = (Wr + a.Wt - 1) / a.Wt;
-    a.ysegs = (Hr + a.R - 1) / a.R;
-    a.tiles = (int)best_t;
-    a.Hr = Hr; a.Wr = Wr; a.B = B;
-    return true;
-}
-
-// Division of shared and tensor memory, and the tile that goes with it.  A tile's loads (four planes, or one box per chunk)
-// are all held at once.  Two CTAs per SM, one epilogue group each, where the weights and a full-sized tile's loads and
-// staging fit into half of it; else one CTA with two epilogue groups, if need be with a smaller tile.  The epilogue is
-// the longest chain of a tile (read the accumulator, convert, stage, hand over, wait until the copy engine has read the
-// buffer), so it is what the second CTA or group is for; a CTA's only group stages into two buffers if they fit.  What
-// room is left goes to more slots, for the next tile's loads.
-bool plan(Args &a, int Wr, int Hr, int B) {
-    const size_t w = ((size_t)a.nchunks * a.w_chunk + 1023) & ~size_t(1023);
-    const size_t fixed = w + sizeof(Pipe) + 1024 + 1024;  // alignment of the base and behind the slots
-    a.stg_row = a.N == 32 && !a.ln_gamma ? 64 : 128;  // 64 columns, or 32 and the normalised values beside the outputs
-    a.acc_cols = 32;
-    while (a.acc_cols < a.N) a.acc_cols *= 2;
-    const size_t half = kSmemMax / 2 - 512;
-    Args best = a;
-    if (!choose_tile(best, Wr, Hr, B, size_t(1) << 30, a.nloads, 1)) return false;
-    for (int two = a.N <= 128 ? 1 : 0; two >= 0; --two) {
-        const size_t room = two ? half : kSmemMax;
-        if (fixed >= room) continue;
-        // Four-warp groups (see the top of the file) cost a second staging buffer: worth it for the input gradient (32
-        // channels: 1.49 -> 1.29 ms), a single step of 32 columns and normalised rows; a plain forward tile of 64 columns and
-        // more wants the room for its next two planes (1.30 against 1.48 ms).
-        a.epw = a.ln_gamma || (two && (a.nloads != 4 || a.N == 32)) ? 4 : 8;
-        a.nacc = (two ? 256 : 512) / a.acc_cols;
-        if (a.nacc > 4) a.nacc = 4;
-        if (a.nacc < 2) continue;
-        a.neg = two ? 8 / a.epw : 2;
-        if (a.neg > a.nacc) a.neg = a.nacc;  // a group has accumulators of its own
-        const int least = a.nloads == 4 || two ? a.nloads : a.nloads + 1;
-        if (!choose_tile(a, Wr, Hr, B, room - fixed, least, a.neg)) continue;
-        if (two && a.tiles > best.tiles) continue;  // no smaller tile for the sake of a second CTA
-        a.slot_bytes = (uint32_t)(a.I * a.Rp * a.Wp * a.rb + 127) & ~127u;
-        a.stg_bytes = stage_rows_bytes(a.I * a.R * a.Wt, a.stg_row);
-        // a second staging buffer comes before more slots where a step stages twice (normalised values, then outputs) or a
-        // tile is one load; a plain forward tile wants its next two planes first (32 -> 64 channels: 1.45 -> 1.29 ms)
-        const int before = a.nloads == 4 && !a.ln_gamma ? a.nloads + 2 : least;
-        a.nbuf = two && (size_t)before * a.slot_bytes + 2 * (size_t)(a.neg * a.stg_bytes) <= room - fixed ? 2 : 1;
-        a.slots = (int)((room - fixed - (size_t)(a.nbuf * a.neg) * a.stg_bytes) / a.slot_bytes);
-        if (a.slots > kMaxSlots) a.slots = kMaxSlots;
-        a.slots_bytes = ((uint32_t)a.slots * a.slot_bytes + 1023u) & ~1023u;
-        a.smem = a.slots_bytes + w + (size_t)(a.nbuf * a.neg) * a.stg_bytes + sizeof(Pipe) + 1024;
-        const int ctas = ppo_num_sms() * (two ? 2 : 1);
-        a.grid = a.tiles < ctas ? a.tiles : ctas;
-        return true;
-    }
-    return false;
-}
-
 template <int MODE, int GC, int KS, int EPW>
 int launch_one(const Args &a, cudaStream_t st) {
     static PerDevice<bool> set;
     const auto fn = conv_halo_kernel<MODE, GC, KS, EPW>;
     PPO_TRY(ppo_once_per_device(set, [&] { return ppo_allow_smem(fn, kSmemMax); }));
-    return ppo_launch(fn, dim3((unsigned)a.grid), dim3((2 + a.neg * EPW) * 32), a.smem, st, a);
+    const int ctas = ppo_num_sms() * a.per_sm;
+    return ppo_launch(fn, dim3((unsigned)(a.tiles < ctas ? a.tiles : ctas)), dim3((2 + a.neg * EPW) * 32), a.smem, st, a);
 }
 
 template <int MODE, int GC, int EPW>
@@ -1266,76 +1092,6 @@ int halo_conv_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, 
     return launch(a, DG, g.Ci, st);
 }
 
-// Division of shared memory and the tile for the input gradient whose output stays on chip: room for the loads of a tile and one more,
-// and a ring of at least two row groups; fewest tiles, then the lowest groups.
-static bool plan_first(Args &a, First &f, const ConvGeom &g) {
-    const int Wr = (g.Wi + 1) / 2, Hr = (g.Hi + 1) / 2, C1 = g.Ci;
-    const size_t w = ((size_t)a.nchunks * a.w_chunk + 1023) & ~size_t(1023);
-    const size_t patch = (size_t)kWinStages * kStagePx * Win<3>::TP * 2;
-    const size_t fixed = w + patch + sizeof(Pipe) + 2048;
-    if (fixed >= kSmemMax) return false;
-    const size_t room = kSmemMax - fixed;
-    auto ring_of = [&](int groups, int R) -> size_t {  // whole stages
-        return (size_t)((groups * 2 * R * g.Wi + kStagePx - 1) / kStagePx * kStagePx) * C1 * 2;
-    };
-    auto slot_of = [&](int R, int Wp) -> size_t { return ((size_t)(R + 1) * Wp * a.rb + 127) & ~size_t(127); };
-    long long best_t = -1;
-    int least = 0;
-    for (int xs = 1; xs <= Wr && xs <= 64; ++xs) {
-        const int Wt = (Wr + xs - 1) / xs, Wp = Wt + 1;
-        if (Wt > 128) continue;
-        int top = (128 - Wt) / Wp + 1;
-        if (top > Hr) top = Hr;
-        for (int R = top; R >= 1; --R) {
-            const int ysegs = (Hr + R - 1) / R, Re = (Hr + ysegs - 1) / ysegs;
-            if ((Hr + Re - 1) / Re != ysegs) continue;
-            // Groups in flight: a builder that waits for one has by then given back all that ended kWinStages stages before its own.
-            const int ahead = kWinStages + 1;
-            int touch = 2;
-            for (int i = 0; i < ysegs; ++i) {
-                int sum = 0, n = 2;
-                for (int k = i;; k = k + 1 == ysegs ? 0 : k + 1, ++n) {
-                    sum += (k == ysegs - 1 ? g.Hi - 2 * Re * (ysegs - 1) : 2 * Re) * g.Wi;
-                    if (sum > ahead * kStagePx) break;
-                }
-                touch = n > touch ? n : touch;
-            }
-            if (touch > kMaxGroups) continue;
-            if ((size_t)(a.nloads + 1) * slot_of(Re, Wp) + 1024 + ring_of(touch, Re) > room) continue;
-            const long long tiles = (long long)g.B * ysegs * ((Wr + Wt - 1) / Wt);
-            if (best_t < 0 || tiles < best_t || (tiles == best_t && Re < a.R)) {
-                best_t = tiles;
-                a.Wt = Wt; a.R = Re;
-                least = touch;
-            }
-        }
-    }
-    if (best_t < 0 || best_t > 0x3fffffff) return false;
-    a.I = 1;
-    a.Wp = a.Wt + 1;
-    a.Rp = a.R + 1;
-    a.xsegs = (Wr + a.Wt - 1) / a.Wt;
-    a.ysegs = (Hr + a.R - 1) / a.R;
-    a.tiles = (int)best_t;
-    a.Hr = Hr; a.Wr = Wr; a.B = g.B;
-    a.epw = 4;
-    a.neg = 2;
-    a.acc_cols = a.N;
-    a.nacc = 4;
-    a.slot_bytes = (uint32_t)slot_of(a.R, a.Wp);
-    f.groups = least;
-    while (f.groups < 3 && (size_t)(a.nloads + 1) * a.slot_bytes + 1024 + ring_of(f.groups + 1, a.R) <= room) ++f.groups;
-    f.group_px = 2 * a.R * g.Wi;
-    f.last_px = (g.Hi - 2 * a.R * (a.ysegs - 1)) * g.Wi;
-    f.ring_bytes = (uint32_t)ring_of(f.groups, a.R);
-    f.ring_px = (int)(f.ring_bytes / (C1 * 2));
-    a.slots = (int)((room - 1024 - f.ring_bytes) / a.slot_bytes);
-    if (a.slots > kMaxSlots) a.slots = kMaxSlots;
-    a.slots_bytes = ((uint32_t)a.slots * a.slot_bytes + 1023u) & ~1023u;
-    a.smem = a.slots_bytes + w + f.ring_bytes + patch + sizeof(Pipe) + 1024;
-    return true;
-}
-
 // Where it pays (us of a backward pass's share, the two kernels by themselves -> here; 3x3, 32 -> 64 channels): 4096 rows of 160 x 120 (19.7 M
 // pixels of the first layer) 620 -> 460, 2048 rows of 240 x 180 (22 M) the same share, 2048 rows of 130 x 100 (6.7 M) 10 less of a
 // minibatch of 870, 1024 rows of 84 x 64 (1.4 M) 6 more of 280.  5x5 windows (twice the fragments, 2.5 times the loads of a builder)
@@ -1344,7 +1100,7 @@ static bool first_shape(Args &a, First &f, const ConvGeom &g, int ldy, int wt_ld
     if (q.k != 3 || g.Ci != 32 || !mask_bits || q.Wf % 2 != 0) return false;
     const long long M = (long long)g.B * g.Hi * g.Wi;
     if (M < 4000000 || M > 0x7fff0000ll) return false;  // (pixels are 32-bit numbers here)
-    return dgrad_shape(a, g, ldy, wt_ld) && plan_first(a, f, g);
+    return dgrad_shape(a, g, ldy, wt_ld) && plan_first(a, f, g.Hi, g.Wi, g.Ci, g.B);
 }
 
 bool halo_first_covers(const ConvGeom &g, int ldy, int wt_ld, const uint32_t *mask_bits, const FirstGrad &q) {
@@ -1355,10 +1111,11 @@ bool halo_first_covers(const ConvGeom &g, int ldy, int wt_ld, const uint32_t *ma
 
 template <int KS>
 static int launch_first(const Args &a, const First &f, const __half *depth, cudaStream_t st) {
+    const int sms = ppo_num_sms();
     static PerDevice<bool> set;
     const auto fn = conv_halo_first_kernel<32, KS, 3>;
     PPO_TRY(ppo_once_per_device(set, [&] { return ppo_allow_smem(fn, kSmemMax); }));
-    return ppo_launch(fn, dim3((unsigned)a.grid), dim3(kFirstThreads<32, 3>), a.smem, st, a, f, depth);
+    return ppo_launch(fn, dim3((unsigned)(f.blocks < sms ? f.blocks : sms)), dim3(kFirstThreads<32, 3>), a.smem, st, a, f, depth);
 }
 
 int halo_dgrad_first(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, int wt_ld, const uint32_t *mask_bits, const FirstGrad &q,
@@ -1375,7 +1132,6 @@ int halo_dgrad_first(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt,
     f.px_per_warp = q.px_per_warp;
     f.blocks = q.blocks;
     f.part = q.part;
-    a.grid = q.blocks < ppo_num_sms() ? q.blocks : ppo_num_sms();
     const int ks = a.CB >> 4;
     if (ks == 4) return launch_first<4>(a, f, depth, st);
     return ks == 2 ? launch_first<2>(a, f, depth, st) : launch_first<1>(a, f, depth, st);
