@@ -156,7 +156,7 @@ __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const uint32_t (&a
 // Builder warp bw: the window tiles of the pixels p0 .. p1, [32 px][TP] bf16, four trips to a stage; trip bw % 4 of every second
 // stage.
 // The builders also stand between ring and sums, whose loop is the kernel's longest chain: a stage is handed over when its pixels
-// have arrived in the ring, and a row group is given back by the builder that sees the stage it ends in summed.
+// have arrived in the ring, and the first of them gives a row group back when it has seen the stage it ends in summed.
 template <int K1>
 __device__ __forceinline__ void first_windows(const First &f, int H1, int W1, const __half *depth, int p0, int p1, const GroupWalk &at, int bw,
                                               uint8_t *patch, FirstPipe *pipe, int32_t *status) {
@@ -219,14 +219,12 @@ __device__ __forceinline__ void first_windows(const First &f, int H1, int W1, co
 #pragma unroll
         for (int c = 0; c < TP / 8; ++c)
             *reinterpret_cast<uint4 *>(row + ((c ^ sw) << 4)) = make_uint4(wv[4 * c], wv[4 * c + 1], wv[4 * c + 2], wv[4 * c + 3]);
-        if ((bw & 3) == 0) {
-            const int summed = (s - kWinStages + 1) * kStagePx;  // (the first stages have nothing before them)
-            for (; ended <= summed; ended += done.px()) {
-                if (ended > summed - kStagePx && lane == 0) mbar_arrive(&pipe->gempty[done.i]);
+        if (ring_gives_back(bw))
+            for (; ended <= ring_summed(s); ended += done.px()) {  // (the first stages have nothing before them)
+                if (lane == 0) mbar_arrive(&pipe->gempty[done.i]);
                 done.next();
             }
-        }
-        const int end = min(p1 - p0, s * kStagePx + (bw & 3) * kTrip + kTrip);
+        const int end = ring_needs(s, bw & 3, p1 - p0);
         while (avail < end) {
             if (!mbar_wait_warp(&pipe->gfull[seen.i], seen.ph, &pipe->abort_flag, status)) return;
             avail += seen.px();

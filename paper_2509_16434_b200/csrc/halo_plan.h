@@ -4,6 +4,12 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#ifdef __CUDACC__
+#define PPO_HALO_FN __host__ __device__ constexpr
+#else
+#define PPO_HALO_FN constexpr
+#endif
+
 namespace halo {
 
 constexpr int kMaxSlots = 8;
@@ -188,6 +194,21 @@ inline bool plan(Args &a, int Wr, int Hr, int B) {
     return false;
 }
 
+// Hand-overs of the ring.  A wait by parity sees a phase only until the next one of the same barrier is complete, and takes the phase
+// before the last for it: a waiter may be neither two phases behind nor two ahead.
+//
+// Row groups are given back by one builder, in order.  An epilogue group that has tiles in every second row group only (one tile each)
+// looks at a barrier at every second use where the number of row groups in flight is odd, and leans on this: what it saw given back
+// for its last tile came behind all that was given back before.
+PPO_HALO_FN bool ring_gives_back(int builder) { return builder == 0; }
+// End of what has been summed, in pixels of the run, when a builder is let into stage s.
+PPO_HALO_FN int ring_summed(int s) { return (s - kWinStages + 1) * kStagePx; }
+// Pixels of the run that trip `trip` of stage s waits for.
+PPO_HALO_FN int ring_needs(int s, int trip, int total) {
+    const int end = s * kStagePx + trip * kTrip + kTrip;
+    return end < total ? end : total;
+}
+
 // Division of shared memory and the tile for the input gradient whose output stays on chip: room for the loads of a tile and one more,
 // and a ring of at least two row groups; fewest tiles, then the lowest groups.
 inline bool plan_first(Args &a, First &f, int Hi, int Wi, int C1, int B) {
@@ -211,7 +232,8 @@ inline bool plan_first(Args &a, First &f, int Hi, int Wi, int C1, int B) {
         for (int R = top; R >= 1; --R) {
             const int ysegs = (Hr + R - 1) / R, Re = (Hr + ysegs - 1) / ysegs;
             if ((Hr + Re - 1) / Re != ysegs) continue;
-            // Groups in flight: a builder that waits for one has by then given back all that ended kWinStages stages before its own.
+            // Groups in flight.  A builder that waits in stage s stands behind a stage (s or, of the other set, s - 1) in which all was
+            // given back that ended kWinStages stages before that: at most this many stages' pixels, of whole groups, are not.
             const int ahead = kWinStages + 1;
             int touch = 2;
             for (int i = 0; i < ysegs; ++i) {
