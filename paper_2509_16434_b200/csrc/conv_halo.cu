@@ -224,7 +224,7 @@ __device__ __forceinline__ void first_windows(const First &f, int H1, int W1, co
                 if (lane == 0) mbar_arrive(&pipe->gempty[done.i]);
                 done.next();
             }
-        const int end = ring_needs(s, bw & 3, p1 - p0);
+        const int end = ring_needs(s, p1 - p0);
         while (avail < end) {
             if (!mbar_wait_warp(&pipe->gfull[seen.i], seen.ph, &pipe->abort_flag, status)) return;
             avail += seen.px();

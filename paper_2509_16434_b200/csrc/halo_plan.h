@@ -203,9 +203,11 @@ inline bool plan(Args &a, int Wr, int Hr, int B) {
 PPO_HALO_FN bool ring_gives_back(int builder) { return builder == 0; }
 // End of what has been summed, in pixels of the run, when a builder is let into stage s.
 PPO_HALO_FN int ring_summed(int s) { return (s - kWinStages + 1) * kStagePx; }
-// Pixels of the run that trip `trip` of stage s waits for.
-PPO_HALO_FN int ring_needs(int s, int trip, int total) {
-    const int end = s * kStagePx + trip * kTrip + kTrip;
+// Pixels of the run that a builder waits for before it hands its trip of stage s over: those of the whole stage, which is handed over with
+// the last of its four trips anyway.  With its own trip's alone a row group behind them that ends in the same stage could be summed,
+// given back and filled again before this builder, by then stages behind, looked at it for the first time.
+PPO_HALO_FN int ring_needs(int s, int total) {
+    const int end = (s + 1) * kStagePx;
     return end < total ? end : total;
 }
 

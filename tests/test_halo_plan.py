@@ -2,6 +2,8 @@
 import os
 import subprocess
 
+import pytest
+
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 # Forward passes (Ci -> Co) and input gradients (Co -> Ci) on grids of w x h: the slots a CTA has against those that fit beside what the
@@ -59,7 +61,7 @@ def test_the_ring_takes_no_room_from_kernels_without_one(tmp_path):
 # Every interleaving of the ring's hand-overs for runs that cross ends of images, on planned grids: two epilogue groups on alternate
 # tiles, builders of both sets, and the sums.  A wait that a barrier's parity lets pass before its time, or one that never passes
 # although nothing else can move, is an error.  FAULT plants one: 1, each set's first builder gives back the row groups that end in the
-# stages of its own set.
+# stages of its own set; 2, a builder waits for the pixels of its own trip only.
 RING = r"""
 #include <cstdio>
 #include <cstdlib>
@@ -71,6 +73,12 @@ using namespace halo;
 static bool gives_back(int builder, int s, int end) {
     if (FAULT == 1) return (builder & 3) == 0 && end > ring_summed(s) - kStagePx;
     return ring_gives_back(builder);
+}
+
+static int needs(int builder, int s, int total) {
+    const int end = s * kStagePx + ((builder & 3) + 1) * kTrip;
+    if (FAULT == 2) return end < total ? end : total;
+    return ring_needs(s, total);
 }
 
 struct Run {
@@ -172,7 +180,7 @@ static const char *follow(const Run &r, long &states) {
                 go(n);
             } else {
                 const int g = s.seen[b];
-                if (g == 0 || r.end[g - 1] < ring_needs(k, r.builder[b] & 3, r.total)) {
+                if (g == 0 || r.end[g - 1] < needs(r.builder[b], k, r.total)) {
                     if (!passes(full(g % G), g / G & 1)) continue;
                     if (tiles_done(g) < r.xsegs) return "a builder takes pixels for written that are not";
                     ++n.seen[b];
@@ -245,11 +253,17 @@ def _ring(tmp_path, fault, builders):
     return found
 
 
-def test_the_ring_is_handed_over_in_order(tmp_path):
-    assert all(": ok" in o for o in _ring(tmp_path, 0, (0, 4)))
+@pytest.mark.parametrize("builders", [(0, 4), (0, 4, 1), (0, 4, 2, 5)])
+def test_the_ring_is_handed_over_in_order(tmp_path, builders):
+    assert all(": ok" in o for o in _ring(tmp_path, 0, builders))
 
 
 def test_two_that_give_back_are_found_out(tmp_path):
     """Released by two builders, a row group can be given back before the one in front of it."""
     found = _ring(tmp_path, 1, (0, 4))
     assert all("not been given back" in o for o in found[:3]) and all("nothing can move" in o for o in found[3:5]), found
+
+
+def test_a_builder_that_falls_behind_is_found_out(tmp_path):
+    """Builder 1, waiting for its own trip's pixels alone, misses a row group of 48 pixels that is filled twice meanwhile."""
+    assert "nothing can move" in _ring(tmp_path, 2, (0, 4, 1))[5]
