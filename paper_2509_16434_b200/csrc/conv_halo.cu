@@ -340,8 +340,8 @@ __device__ __forceinline__ void first_sums(const First &f, int p0, int p1, int b
         }
         xs = xn;
         zs = zn;
+        __syncwarp();  // (the release covers what all lanes read)
         if (lane == 0) mbar_arrive(&pipe->pempty[old]);
-        __syncwarp();
         if (--left == 0) flush(false);
     }
     // the last stage, trip by trip
