@@ -393,6 +393,12 @@ uint64_t ppo_launch_count(void);
  * ppo_poll_status returns PPO_ERR_TIMEOUT and clears it; the device stays usable. */
 int ppo_selftest_wait_timeout(long long limit_cycles, int *dev_gave_up, void *stream);
 
+/* Self-test of the first convolution's gradients (no counterpart in the paper): adds them to the model's gradients once more, behind an
+ * ppo_encoder_bwd of the same arguments, from the gradient that call left for the second convolution's output.  one_launch 1: by the
+ * kernel that keeps the second convolution's input gradient on chip, as large calls do (PPO_ERR_UNSUPPORTED where that call did
+ * not); 0: by the two kernels it stands for, whose bits it gives. */
+int ppo_selftest_first_gradient(ppo_model *m, const ppo_minibatch *mb, int row0, int rows, int one_launch, void *stream);
+
 /* Synchronises `stream`, then returns the first error a kernel recorded in the library's
  * device status word since the last poll (PPO_OK if none), or PPO_ERR_CUDA if the stream
  * reports a CUDA error. */

@@ -30,7 +30,7 @@ EXPORTS = [
     "ppo_adam_step", "ppo_policy_sample", "ppo_poll_status", "ppo_model_activation_ptr", "ppo_gae_static",
     "ppo_model_sync_masks", "ppo_buffer_write_obs", "ppo_buffer_write_outcome", "ppo_policy_act", "ppo_launch_count",
     "ppo_selftest_wait_timeout", "ppo_buffer_render_depth", "ppo_model_set_sequence", "ppo_shuffle_gather_sequences",
-    "ppo_model_read_state", "ppo_state_reset", "ppo_policy_step",
+    "ppo_model_read_state", "ppo_state_reset", "ppo_policy_step", "ppo_selftest_first_gradient",
 ]
 
 
@@ -118,6 +118,7 @@ def lib():
         L.ppo_launch_count.restype = C.c_uint64
         L.ppo_launch_count.argtypes = []
         L.ppo_selftest_wait_timeout.argtypes = [C.c_longlong, C.c_void_p, C.c_void_p]
+        L.ppo_selftest_first_gradient.argtypes = [C.c_void_p, C.POINTER(Minibatch), C.c_int, C.c_int, C.c_int, C.c_void_p]
         L.ppo_gae_static.argtypes = [C.c_void_p] * 4 + [C.c_int, C.c_int, C.c_float, C.c_float, C.c_int] + [C.c_void_p] * 4
         L.ppo_model_activation_ptr.argtypes = [C.c_void_p, C.c_int, C.c_int, C.POINTER(C.c_void_p),
                                                C.POINTER(C.c_size_t)]
@@ -246,6 +247,11 @@ def ppo_launch_count() -> int:
 def ppo_selftest_wait_timeout(limit_cycles: int, gave_up, stream=None):
     _check(lib().ppo_selftest_wait_timeout(limit_cycles, _ptr(gave_up), _stream(stream)),
            "ppo_selftest_wait_timeout")
+
+
+def ppo_selftest_first_gradient(m: Model, mb: MinibatchArrays, row0: int, rows: int, one_launch: bool, stream=None):
+    _check(lib().ppo_selftest_first_gradient(m.handle, _mbref(mb), row0, rows, int(one_launch), _stream(stream)),
+           "ppo_selftest_first_gradient")
 
 
 def ppo_compute_gae(buf: Buffer, last_value, gamma: float, lam: float, normalize=True, stats_out=None,

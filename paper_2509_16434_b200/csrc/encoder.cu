@@ -1769,3 +1769,22 @@ extern "C" int ppo_encoder_bwd(ppo_model *m, const ppo_minibatch *mb, int row0, 
     if (s == PPO_OK) s = sum_partials_jobs(sums, st);
     return join(s);
 }
+
+extern "C" int ppo_selftest_first_gradient(ppo_model *m, const ppo_minibatch *mb, int row0, int rows, int one_launch, void *stream) {
+    PPO_TRY(check_rows(m, mb, row0, rows));
+    if (!m->fwd_valid || m->last_row0 != row0 || m->last_rows != rows) return PPO_ERR_STATE;
+    if (m->L < 2 || m->d.norm) return PPO_ERR_UNSUPPORTED;
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    PPO_TRY(refresh_transposed(m, st));
+    SumJobs sums;
+    sums.n = 0;
+    if (one_launch) PPO_TRY(conv1_fused(m, mb, row0, rows, sums, st));
+    else {
+        const ConvGeom g = conv_geom(m, 2, rows);
+        DgradEpilogue e = {m->act[1], m->dact[1], nullptr};
+        e.mask_bits = m->abits[1];
+        PPO_TRY(run_dgrad(m, g, m->dact[2], g.Co, m->wT + m->wT_off[m->ti_conv[2]], wt_ld_of(g.Co), 2, e, st));
+        PPO_TRY(conv1_wgrad(m, mb, row0, rows, sums, st));
+    }
+    return sum_partials_jobs(sums, st);
+}

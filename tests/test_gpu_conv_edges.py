@@ -148,3 +148,36 @@ def test_first_layer_gradient_of_a_whole_call_is_that_of_its_pieces(rows, H, W, 
     assert torch.equal(whole, again)
     assert torch.isfinite(whole).all() and float(whole.norm()) > 0
     assert float((whole - pieces).norm() / pieces.norm()) <= 5e-5
+
+
+# as above, and an odd number of row groups in flight with short last ones (124 x 164, 69 x 90: of 164 and 225 pixels; 122 x 96: of 48)
+@pytest.mark.parametrize("rows,H,W,C2", [(2901, 61, 90, 64), (953, 31, 530, 32), (15701, 30, 34, 48), (1301, 112, 110, 128),
+                                         (801, 124, 164, 64), (2541, 69, 90, 64), (1367, 122, 96, 128)])
+def test_first_layer_gradient_is_that_of_the_two_kernels(rows, H, W, C2):
+    """The same bits from the one launch as from input gradient and weight gradient by themselves, time and again; a backward call
+    of this size makes the one."""
+    w = synth.Workload("first", rows, 1, H, W, (32, C2), (3, 3), (32,), 1, 1, P=16, A=3)
+    L, md, lay, theta, roll, action, logp, dev = base._setup(w, rows)
+    L.compute_gae(dev["last_value"])
+    ppo.ppo_shuffle_gather_minibatch(L.buffer, 5, 0, 0, 1, L.mb)
+    ppo.ppo_encoder_fwd(L.model, L.mb, 0, rows, L.mean, L.value)
+    g = torch.Generator("cuda").manual_seed(1)
+    L.dmean.normal_(generator=g)
+    L.dvalue.normal_(generator=g)
+    (o0, _), (o1, s1) = L.model.tensors()[:2]
+
+    def gradients(call, *args):
+        ppo.ppo_model_zero_grad(L.model)
+        before = ppo.ppo_launch_count()
+        call(L.model, L.mb, 0, rows, *args)
+        launches = ppo.ppo_launch_count() - before
+        assert ppo.ppo_poll_status() == 0
+        return L.model.grad[o0:o1 + s1].clone(), launches
+
+    whole, _ = gradients(ppo.ppo_encoder_bwd, L.dmean, L.dvalue, True)
+    two, launches = gradients(ppo.ppo_selftest_first_gradient, False)
+    assert torch.isfinite(two).all() and float(two.norm()) > 0
+    assert launches == 3 and torch.equal(two, whole)
+    for _ in range(5):
+        one, launches = gradients(ppo.ppo_selftest_first_gradient, True)  # (refused where the backward call takes the two kernels)
+        assert launches == 2 and torch.equal(one, two)
