@@ -334,3 +334,39 @@ def test_one_decision_call_is_the_separate_calls(family):
     with pytest.raises(ppo.PpoError):
         z = torch.zeros((2, n, 128), device=dev)
         ppo.ppo_policy_step(L.model, obs, n, None, z, None, eps, mean, value, action, logp)
+
+
+@pytest.mark.parametrize("family", ["unaligned", "unaligned_split", "many_units"])
+def test_one_decision_call_where_a_step_kernel_does_not_leave_the_state(family):
+    """States that are not 16-byte aligned (with the embedding split and not), more step CTAs than two waves: the call
+    reads the state behind the pass instead.  The same bits as the separate calls, in place, twice in a row."""
+    n, H, W, lstm_h = {"unaligned": (16, 48, 64, 128), "unaligned_split": (21, 96, 128, 128), "many_units": (1281, 33, 46, 1024)}[family]
+    w = synth.Workload("step", n, 2, H, W, (16, 32, 64, 128), (3, 3, 3, 3), (72, 120), 1, 1, P=32, A=5, norm=True, embed=32, n_lstm=2,
+                       lstm_h=lstm_h)
+    dev = "cuda"
+    L = Learner(w, 2 * n, dev)
+    shapes, gammas = synth.param_shapes(w)
+    L.model.load(synth.init_params(L.model.arena, [o for o, _ in L.model.tensors()], shapes, 3, ones=gammas))
+    r = synth.rollout_torch(w, dev, 4)
+    shift = 1 if family.startswith("unaligned") else 0
+
+    def states(seed):
+        g = torch.Generator(dev).manual_seed(seed)
+        return [torch.randn(2 * n * lstm_h + shift, generator=g, device=dev)[shift:].view(2, n, lstm_h) for _ in range(2)]
+
+    mine, theirs = states(5), states(5)
+    for t in range(2):
+        depth, proprio, eps = r["depth"][t], r["proprio"][t], r["eps"][t]
+        done = (torch.arange(n, device=dev) % 3 == t).to(torch.uint8)
+        obs = ppo.Minibatch(depth.data_ptr(), proprio.data_ptr(), None, None, None, None, None, None, n)
+        one, two = [[torch.full(s, 7.0, device=dev) for s in ((n, w.A), (n,), (n, w.A), (n,))] for _ in range(2)]
+        ppo.ppo_policy_step(L.model, obs, n, done, mine[0], mine[1], eps, *one)
+        ppo.ppo_model_set_sequence(L.model, 1, n, done, theirs[0], theirs[1])
+        mean, value, action, logp = two
+        ppo.ppo_encoder_fwd(L.model, obs, 0, n, mean, value)
+        ppo.ppo_policy_sample(L.model, n, mean, eps, action, logp)
+        ppo.ppo_model_read_state(L.model, theirs[0], theirs[1])
+        assert ppo.ppo_poll_status() == 0
+        for a, b in zip(one + mine, two + theirs):
+            assert torch.equal(a, b)
+        assert all(torch.isfinite(s).all() for s in mine) and not bool(mine[0][:, done != 0].any()) and bool(mine[0][:, done == 0].any())
