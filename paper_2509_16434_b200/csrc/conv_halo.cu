@@ -1090,15 +1090,23 @@ int halo_conv_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, 
     return launch(a, DG, g.Ci, st);
 }
 
-// Where it pays (us of a backward pass's share, the two kernels by themselves -> here; 3x3, 32 -> 64 channels): 4096 rows of 160 x 120 (19.7 M
-// pixels of the first layer) 620 -> 460, 2048 rows of 240 x 180 (22 M) the same share, 2048 rows of 130 x 100 (6.7 M) 10 less of a
-// minibatch of 870, 1024 rows of 84 x 64 (1.4 M) 6 more of 280.  5x5 windows (twice the fragments, 2.5 times the loads of a builder)
-// take longer than the two kernels at all sizes, 16 channels too: half as much dX to keep out of HBM for the same chain.
+// Where it pays: first layers of 3x3 and 32 channels, second ones of 64 or 32 (one chunk), from 4 M pixels of the first layer, in tiles of
+// that many of them on average.  Backward passes of three layers, us, the two kernels -> this one, by output channels of the second:
+//   channels, 4 M pixels of 160 x 120 and of 320 x 240 frames   64: 350 -> 321, 356 -> 326; 32: 258 -> 245, 256 -> 242; 16: 404 -> 414,
+//            408 -> 412; 48 (three chunks): 555 -> 565, 597 -> 598; 128 (two, in smaller tiles): 485 -> 500, 495 -> 626
+//   tiles, 4 M pixels   64: 255 to 262 pixels (258 x 182, 262 x 196) 361 -> 367, 367 -> 369; 336 and 344 (84 x 64, 86 x 63) 367 -> 373, 367
+//            -> 369; from 350 on 3 to 14 % less (30 sizes of frames; one alike).  32: 286 to 345 (52 x 44, 60 x 45, 310 x 230) 307 -> 315,
+//            287 -> 305, 260 -> 270; 353 to 360 (530 x 31, 92 x 61, 60 x 48) 270 -> 287, 273 -> 283, 285 -> 293; 380 and 385 (100 x 75,
+//            88 x 70) 281 -> 281, 275 -> 277; from 390 on 0 to 8 % less.  An epilogue group takes its time per tile, the two kernels
+//            theirs per pixel.
+//   pixels, 64   19.7 M (160 x 120) 1460 -> 1330, 6.7 M (130 x 100) 10 less of a minibatch of 870, 1.4 M (84 x 64) 6 more of 280
+// 5x5 windows (twice the fragments, 2.5 times the loads of a builder) take longer than the two kernels at all sizes, and so do 16 channels
+// of the first layer: half as much dX to keep out of HBM for the same chain.
 static bool first_shape(Args &a, First &f, const ConvGeom &g, int ldy, int wt_ld, const uint32_t *mask_bits, const FirstGrad &q) {
-    if (q.k != 3 || g.Ci != 32 || !mask_bits || q.Wf % 2 != 0) return false;
+    if (q.k != 3 || g.Ci != 32 || (g.Co != 32 && g.Co != 64) || !mask_bits || q.Wf % 2 != 0) return false;
     const long long M = (long long)g.B * g.Hi * g.Wi;
     if (M < 4000000 || M > 0x7fff0000ll) return false;  // (pixels are 32-bit numbers here)
-    return dgrad_shape(a, g, ldy, wt_ld) && plan_first(a, f, g.Hi, g.Wi, g.Ci, g.B);
+    return dgrad_shape(a, g, ldy, wt_ld) && plan_first(a, f, g.Hi, g.Wi, g.Ci, g.B) && M >= (g.Co == 64 ? 350ll : 390ll) * a.tiles;
 }
 
 bool halo_first_covers(const ConvGeom &g, int ldy, int wt_ld, const uint32_t *mask_bits, const FirstGrad &q) {
