@@ -225,7 +225,7 @@ int main(int argc, char **argv) {
     for (int end = -v[4]; r.end.empty() || r.end.back() < r.total; k = (k + 1) % a.ysegs)
         r.end.push_back(end += k % a.ysegs == a.ysegs - 1 ? f.last_px : f.group_px);
     r.ntiles = (int)r.end.size() * r.xsegs;
-    if (r.end.size() > 60 || r.ntiles > 250 || r.builder.size() > kMost) return 2;
+    if (r.end[0] <= 0 || r.end.size() > 60 || r.ntiles > 250 || r.builder.size() > kMost) return 2;
     long states = 0;
     const char *wrong = follow(r, states);
     printf("%d row groups, %d in flight, of %d px, the last of an image %d, %d tiles each: %s (%ld states)\n", (int)r.end.size(), r.groups,
@@ -235,9 +235,9 @@ int main(int argc, char **argv) {
 """
 
 # frames, channels, row groups of the run's first image, pixels in front of the run: odd and even numbers of row groups in flight, short
-# last ones, runs that start in and at row groups
-RUNS = [(124, 164, 64, 2, 16), (180, 240, 64, 2, 80), (69, 90, 64, 1, 16), (112, 110, 128, 1, 112), (113, 114, 128, 1, 64),
-        (122, 96, 128, 2, 112), (154, 192, 128, 1, 96), (61, 90, 64, 2, 0), (31, 530, 32, 2, 0), (30, 34, 48, 1, 0)]
+# last ones, several tiles each, runs that start in and at row groups
+RUNS = [(124, 164, 64, 2, 16), (180, 240, 64, 2, 80), (69, 90, 64, 1, 16), (162, 108, 64, 2, 112), (205, 126, 64, 1, 16), (84, 112, 64, 1, 64),
+        (110, 146, 64, 3, 8), (240, 320, 64, 2, 0), (201, 268, 32, 2, 100), (120, 160, 64, 1, 0)]
 
 
 def _ring(tmp_path, fault, builders):
@@ -259,11 +259,10 @@ def test_the_ring_is_handed_over_in_order(tmp_path, builders):
 
 
 def test_two_that_give_back_are_found_out(tmp_path):
-    """Released by two builders, a row group can be given back before the one in front of it."""
-    found = _ring(tmp_path, 1, (0, 4))
-    assert all("not been given back" in o for o in found[:3]) and all("nothing can move" in o for o in found[3:5]), found
+    """Released by two builders, a row group can be given back before the one in front of it: seen where their number is odd."""
+    assert all("not been given back" in o for o in _ring(tmp_path, 1, (0, 4))[:3])
 
 
 def test_a_builder_that_falls_behind_is_found_out(tmp_path):
-    """Builder 1, waiting for its own trip's pixels alone, misses a row group of 48 pixels that is filled twice meanwhile."""
-    assert "nothing can move" in _ring(tmp_path, 2, (0, 4, 1))[5]
+    """Builder 1, waiting for its own trip's pixels alone, misses a row group of 54 pixels that is filled twice meanwhile."""
+    assert "nothing can move" in _ring(tmp_path, 2, (0, 4, 1))[3]
