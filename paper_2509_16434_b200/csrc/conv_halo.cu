@@ -134,12 +134,10 @@ struct GroupWalk {
     }
 };
 
-// Place of the 16-byte piece `piece` of ring pixel `row` (C1 channels).  Neighbouring lanes of the epilogue write every second pixel,
+// Place of the 16-byte piece `piece` of ring pixel `row`, two to a line.  Neighbouring lanes of the epilogue write every second pixel,
 // ldmatrix reads eight in a row: both go to eight different 16-byte columns of the 128-byte lines.
-template <int C1>
 __device__ __forceinline__ uint32_t ring_offset(int row, int piece) {
-    constexpr int per = 64 / C1, lg = per == 4 ? 2 : 1;  // pixels per line
-    const int line = row >> lg, q = (row & (per - 1)) * (8 / per) + piece;
+    const int line = row >> 1, q = (row & 1) * 4 + piece;
     return (uint32_t)line * 128u + ((uint32_t)(q ^ (line & 7)) << 4);
 }
 
@@ -157,11 +155,9 @@ __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const uint32_t (&a
 // stage.
 // The builders also stand between ring and sums, whose loop is the kernel's longest chain: a stage is handed over when its pixels
 // have arrived in the ring, and the first of them gives a row group back when it has seen the stage it ends in summed.
-template <int K1>
 __device__ __forceinline__ void first_windows(const First &f, int H1, int W1, const __half *depth, int p0, int p1, const GroupWalk &at, int bw,
                                               uint8_t *patch, FirstPipe *pipe, int32_t *status) {
-    using WN = Win<K1>;
-    constexpr int TP = WN::TP, KW = WN::KW, NP = WN::NP, P = WN::P, ODD = WN::ODD;
+    constexpr int TP = Win::TP, KW = Win::KW, NP = Win::NP, P = Win::P, ODD = Win::ODD;
     const int lane = threadIdx.x & 31, nstages = (p1 - p0 + kStagePx - 1) / kStagePx;
     const uint32_t *const frames = reinterpret_cast<const uint32_t *>(depth);
     const int Hf = held(f.Hf), Wh = held(f.Wh);
@@ -182,7 +178,7 @@ __device__ __forceinline__ void first_windows(const First &f, int H1, int W1, co
 #pragma unroll
         for (int q = 0; q < NP; ++q) cok[q] = live && (unsigned)(pw0 + q) < (unsigned)Wh;
 #pragma unroll
-        for (int kh = 0; kh < K1; ++kh) {
+        for (int kh = 0; kh < Win::K; ++kh) {
             const bool rok = (unsigned)(ih0 + kh) < (unsigned)Hf;
 #pragma unroll
             for (int q = 0; q < NP; ++q) {
@@ -199,7 +195,7 @@ __device__ __forceinline__ void first_windows(const First &f, int H1, int W1, co
     };
     fetch();
     uint8_t *const mine = patch + (size_t)((bw & 3) * kTrip + lane) * (TP * 2);
-    const int sw = TP == 32 ? (lane >> 1) & 3 : (lane >> 2) & 1;
+    const int sw = (lane >> 2) & 1;
     GroupWalk seen = at, done = at;
     int avail = at.slot, ended = at.slot + at.px();  // pixels of the run that have arrived; end of group `done`
     for (int s = bw >> 2; s < nstages; s += 2) {
@@ -238,25 +234,20 @@ __device__ __forceinline__ void first_windows(const First &f, int H1, int W1, co
 // dW1[co][tap] = sum over pixels dZ1[px][co] x[px][tap] as mma.sync m16n8k16 with the pixel as K, dZ1 from the ring in which the
 // epilogue leaves it and x from the builders' window tiles.  The pixels are summed in the runs, the trips of 32 and the blocks
 // of conv1_wgrad_mma_kernel: the same bits.  A run is one chain of dependent products, 25 cycles for 16 pixels, and a fragment load
-// takes its warp 16 to 20: a unit of 16 rows (pair elements of the window) x 16 channels per warp, its fragments two trips ahead.  Finer
+// takes its warp 16 to 20: a unit of all 16 rows (pair elements of the window) x 16 channels per warp, its fragments two trips ahead.  Finer
 // units make shorter chains of more shared-memory reads: 8 channels a unit 490 us, 16 channels 450 to 475.
-template <int K1, int C1>
-constexpr int kUnits = Win<K1>::MB * (C1 / 16);
-template <int K1, int C1>
 __device__ __forceinline__ void first_sums(const First &f, int p0, int p1, int block0, int ring_px, int unit, uint32_t ring, uint32_t patch,
                                            FirstPipe *pipe, int32_t *status) {
-    using WN = Win<K1>;
-    constexpr int TP = WN::TP, KW = WN::KW, NP = WN::NP, ODD = WN::ODD, K2 = K1 * K1;
-    const int lane = threadIdx.x & 31, mi = lane >> 3, r = lane & 7;
-    const int ui = unit / (C1 / 16), uj = unit % (C1 / 16) * 2;
+    constexpr int TP = Win::TP, KW = Win::KW, NP = Win::NP, ODD = Win::ODD, K1 = Win::K, K2 = K1 * K1, C1 = kFirstC;
+    const int lane = threadIdx.x & 31, mi = lane >> 3, r = lane & 7, uj = 2 * unit;
     uint32_t a_off[2], b_off[2];
 #pragma unroll
     for (int ks = 0; ks < 2; ++ks) {
-        const int ar = 16 * ks + r + (mi >= 2 ? 8 : 0), sw = TP == 32 ? (ar >> 1) & 3 : (ar >> 2) & 1;
-        a_off[ks] = (uint32_t)(ar * (TP * 2) + (((2 * ui + (mi & 1)) ^ sw) << 4));
+        const int ar = 16 * ks + r + (mi >= 2 ? 8 : 0), sw = (ar >> 2) & 1;
+        a_off[ks] = (uint32_t)(ar * (TP * 2) + (((mi & 1) ^ sw) << 4));
     }
 #pragma unroll
-    for (int j = 0; j < 2; ++j) b_off[j] = ring_offset<C1>(lane, uj + j);  // (a trip starts at a multiple of 32 pixels)
+    for (int j = 0; j < 2; ++j) b_off[j] = ring_offset(lane, uj + j);  // (a trip starts at a multiple of 32 pixels)
     const int total = p1 - p0, nstages = (total + kStagePx - 1) / kStagePx;
     const int run_trips = held(f.px_per_warp / kTrip);
     const uint32_t ring_end = ring + (uint32_t)ring_px * (C1 * 2);  // (whole stages)
@@ -279,7 +270,7 @@ __device__ __forceinline__ void first_sums(const First &f, int p0, int p1, int b
         for (int j = 0; j < 2; ++j)
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const int t = 16 * ui + g + (q & 2 ? 8 : 0), co = 8 * (uj + j) + 2 * c + (q & 1);
+                const int t = g + (q & 2 ? 8 : 0), co = 8 * (uj + j) + 2 * c + (q & 1);
                 const int kh = (t >> 1) / NP, kw = 2 * ((t >> 1) - kh * NP) + (t & 1) - ODD;
                 if (t < 2 * KW && kw >= 0 && kw < K1) out[co * K2 + kh * K1 + kw] = sum[j][q];
                 else if (t == 2 * KW) out[C1 * K2 + co] = sum[j][q];
@@ -368,19 +359,20 @@ __device__ __forceinline__ void first_sums(const First &f, int p0, int p1, int b
 // GC: columns of an output group, i.e. of one pixel of one store (16, 32 or 64; its bytes are the swizzled row).
 // KS: K = 16 steps per channel chunk (1, 2 or 4: rows of 32, 64 or 128 bytes).
 // EPW: warps of an epilogue group, 4 or 8.
-// K1: kernel size of the first layer whose weight gradient takes the place of the output (0: none; input gradient, EPW 4, GC = C1).
-template <int MODE, int GC, int KS, int EPW, int K1>
+// FIRST: the first layer's weight gradient takes the place of the output (input gradient, EPW 4, GC = kFirstC).
+template <int MODE, int GC, int KS, int EPW, bool FIRST>
 __device__ __forceinline__ void halo_body(const Args &a, const First &f, const __half *depth, uint8_t *smem_raw) {
     constexpr int NH = EPW == 4 ? 2 : 1;  // halves of 64 columns a warp works on
-    constexpr uint32_t kPatchBytes = K1 > 0 ? kWinStages * kStagePx * Win<K1 ? K1 : 3>::TP * 2 : 0;
+    constexpr uint32_t kPatchBytes = kWinStages * kStagePx * Win::TP * 2;
+    static_assert(!FIRST || (MODE == DG && GC == kFirstC && EPW == 4), "");
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t smem_base = smem_u32(smem);
     // A slots, then weights (reads of the last slot's halo rows may run on into them), output staging, pipeline state
     const uint32_t w_base = smem_base + a.slots_bytes;
     const uint32_t w_bytes = (uint32_t)a.nchunks * a.w_chunk;
     const uint32_t stg_off = (a.slots_bytes + w_bytes + 1023u) & ~1023u;
-    Pipe *pipe = reinterpret_cast<Pipe *>(smem + stg_off + (K1 > 0 ? (size_t)f.ring_bytes + kPatchBytes : (size_t)(a.nbuf * a.neg) * a.stg_bytes));
-    [[maybe_unused]] FirstPipe *const hand = static_cast<FirstPipe *>(pipe);  // (K1 > 0)
+    Pipe *pipe = reinterpret_cast<Pipe *>(smem + stg_off + (FIRST ? (size_t)f.ring_bytes + kPatchBytes : (size_t)(a.nbuf * a.neg) * a.stg_bytes));
+    [[maybe_unused]] FirstPipe *const hand = static_cast<FirstPipe *>(pipe);  // (FIRST)
     volatile int *abort_flag = &pipe->abort_flag;
     const int warp = warp_index(), lane = threadIdx.x & 31;
     const int nacc = a.nacc;
@@ -396,14 +388,14 @@ __device__ __forceinline__ void halo_body(const Args &a, const First &f, const _
             mbar_init(&pipe->tempty[i], EPW * 32);
         }
         mbar_init(&pipe->wfull, 1);
-        if constexpr (K1 > 0) {
+        if constexpr (FIRST) {
             for (int i = 0; i < f.groups; ++i) {
                 mbar_init(&hand->gfull[i], (uint32_t)(a.xsegs * EPW * 32));
                 mbar_init(&hand->gempty[i], 1);
             }
             for (int i = 0; i < kWinStages; ++i) {
                 mbar_init(&hand->pfull[i], kStagePx / kTrip);
-                mbar_init(&hand->pempty[i], kUnits<K1, GC>);
+                mbar_init(&hand->pempty[i], kUnits);
             }
         }
         pipe->abort_flag = 0;
@@ -430,7 +422,7 @@ __device__ __forceinline__ void halo_body(const Args &a, const First &f, const _
     // with the first layer's sums: the tiles of the row groups that hold the pixels of its blocks
     int p0 = 0, p1 = 0, block0 = 0;
     GroupWalk first_group;
-    if constexpr (K1 > 0) {
+    if constexpr (FIRST) {
         const int bq = f.blocks / (int)gridDim.x, br = f.blocks - bq * (int)gridDim.x, nb = bq + (bid < br ? 1 : 0);
         block0 = bid * bq + (bid < br ? bid : br);
         p0 = block0 * 8 * f.px_per_warp;
@@ -582,11 +574,11 @@ __device__ __forceinline__ void halo_body(const Args &a, const First &f, const _
             __syncwarp();
             if (++acc == nacc) { acc = 0; aph ^= 1u; }
         }
-    } else if (K1 > 0 && warp >= 10) {
-        if constexpr (K1 > 0) {
+    } else if (FIRST && warp >= 10) {
+        if constexpr (FIRST) {
             const uint32_t patch_off = stg_off + f.ring_bytes;
-            if (warp < 10 + kBuildWarps) first_windows<K1>(f, a.Hi, a.Wi, depth, p0, p1, first_group, warp - 10, smem + patch_off, hand, a.status);
-            else first_sums<K1, GC>(f, p0, p1, block0, first_group.ring_px, warp - 10 - kBuildWarps, smem_base + stg_off, smem_base + patch_off, hand, a.status);
+            if (warp < 10 + kBuildWarps) first_windows(f, a.Hi, a.Wi, depth, p0, p1, first_group, warp - 10, smem + patch_off, hand, a.status);
+            else first_sums(f, p0, p1, block0, first_group.ring_px, warp - 10 - kBuildWarps, smem_base + stg_off, smem_base + patch_off, hand, a.status);
         }
     } else {
         // ---------------- epilogue: warp reads TMEM lanes 32 (warp % 4) .. +31 and, of every 64 columns, half `h`
@@ -661,7 +653,7 @@ __device__ __forceinline__ void halo_body(const Args &a, const First &f, const _
         };
         TileAt t_next = t;
         if (eg < nt) fetch_gates(t);
-        if constexpr (K1 > 0) {
+        if constexpr (FIRST) {
             // The input gradient of the first layer's output goes into the ring its weight gradient is summed from, pixel by pixel.
             GroupWalk grp = first_group;
             const int xsegs = held(a.xsegs), Hi = held(a.Hi), Wi = held(a.Wi), B = held(a.B), Hr = held(a.Hr), Wr = held(a.Wr);
@@ -689,31 +681,27 @@ __device__ __forceinline__ void halo_body(const Args &a, const First &f, const _
                 tc_fence_after();
                 const uint32_t lane_base = tmem_base + (uint32_t)(acc * a.acc_cols) + ((uint32_t)(lg * 32) << 16);
 #pragma unroll 1
-                for (int q = 0; q < GC / 8; ++q) {  // (rolled: the roles' loops share the instruction cache)
+                for (int q = 0; q < 4; ++q) {  // classes (rolled: the roles' loops share the instruction cache)
                     float v[32];
                     tmem_ld32(lane_base + (uint32_t)(32 * q), v);
-                    if (q == GC / 8 - 1) {
+                    if (q == 3) {
                         tc_fence_before();
                         mbar_arrive(&pipe->tempty[acc]);
                     }
                     const uint32_t gw = q == 0 ? gate[0] : (q == 1 ? gate[1] : (q == 2 ? gate[2] : gate[3]));
+                    const int ph = q >> 1, pw = (q ^ ph) & 1;
+                    int row = slot + (2 * cr + ph) * Wi + 2 * x + pw;
+                    const bool put_it = live && row >= 0 && 2 * y + ph < Hi && 2 * x + pw < Wi;
+                    if (row >= grp.ring_px) row -= grp.ring_px;
+                    uint32_t pk[16];
 #pragma unroll
-                    for (int h16 = 0; h16 < 32; h16 += GC) {
-                        const int cls = GC == 32 ? q : 2 * q + h16 / 16, ph = cls >> 1, pw = (cls ^ ph) & 1;
-                        int row = slot + (2 * cr + ph) * Wi + 2 * x + pw;
-                        const bool put_it = live && row >= 0 && 2 * y + ph < Hi && 2 * x + pw < Wi;
-                        if (row >= grp.ring_px) row -= grp.ring_px;
-                        uint32_t pk[GC / 2];
+                    for (int j = 0; j < 16; ++j) pk[j] = pack_bf16x2(v[2 * j], v[2 * j + 1]) & gate_mask(gw, j);
+                    if (put_it) {
 #pragma unroll
-                        for (int j = 0; j < GC / 2; ++j)
-                            pk[j] = pack_bf16x2(v[h16 + 2 * j], v[h16 + 2 * j + 1]) & gate_mask(gw, h16 / 2 + j);
-                        if (put_it) {
-#pragma unroll
-                            for (int c = 0; c < GC / 8; ++c)
-                                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(ring + ring_offset<GC>(row, c)), "r"(pk[4 * c]),
-                                             "r"(pk[4 * c + 1]), "r"(pk[4 * c + 2]), "r"(pk[4 * c + 3])
-                                             : "memory");
-                        }
+                        for (int c = 0; c < 4; ++c)
+                            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(ring + ring_offset(row, c)), "r"(pk[4 * c]),
+                                         "r"(pk[4 * c + 1]), "r"(pk[4 * c + 2]), "r"(pk[4 * c + 3])
+                                         : "memory");
                     }
                 }
                 mbar_arrive(&hand->gfull[gi]);
@@ -880,7 +868,7 @@ __device__ __forceinline__ void halo_body(const Args &a, const First &f, const _
 template <int MODE, int GC, int KS, int EPW>
 __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    halo_body<MODE, GC, KS, EPW, 0>(a, First{}, nullptr, smem_raw);
+    halo_body<MODE, GC, KS, EPW, false>(a, First{}, nullptr, smem_raw);
 }
 
 // The input gradient of the second convolution and from it, on chip, the weight gradient of the first one, which is all it is for: the
@@ -891,12 +879,11 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
 // share (800 cycles in place; tensor core alone 215 of them, epilogue 720 on two groups).  Measured at that size: 330 + 290 us -> 460, a
 // minibatch 3.22 -> 3.12 ms.
 // (depth is the last argument: a prepared launch is made again with other frames.)
-template <int GC, int K1>
-constexpr int kFirstThreads = (10 + kBuildWarps + kUnits<K1, GC>) * 32;
-template <int GC, int KS, int K1>
-__global__ void __launch_bounds__(kFirstThreads<GC, K1>, 1) conv_halo_first_kernel(const __grid_constant__ Args a, const __grid_constant__ First f, const __half *depth) {
+constexpr int kFirstThreads = (10 + kBuildWarps + kUnits) * 32;
+template <int KS>
+__global__ void __launch_bounds__(kFirstThreads, 1) conv_halo_first_kernel(const __grid_constant__ Args a, const __grid_constant__ First f, const __half *depth) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    halo_body<DG, GC, KS, 4, K1>(a, f, depth, smem_raw);
+    halo_body<DG, kFirstC, KS, 4, true>(a, f, depth, smem_raw);
 }
 
 // --------------------------------------------------------------------- host ----
@@ -1103,25 +1090,19 @@ int halo_conv_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, 
 // 5x5 windows (twice the fragments, 2.5 times the loads of a builder) take longer than the two kernels at all sizes, and so do 16 channels
 // of the first layer: half as much dX to keep out of HBM for the same chain.
 static bool first_shape(Args &a, First &f, const ConvGeom &g, int ldy, int wt_ld, const uint32_t *mask_bits, const FirstGrad &q) {
-    if (q.k != 3 || g.Ci != 32 || (g.Co != 32 && g.Co != 64) || !mask_bits || q.Wf % 2 != 0) return false;
+    if (q.k != Win::K || g.Ci != kFirstC || (g.Co != 32 && g.Co != 64) || !mask_bits || q.Wf % 2 != 0) return false;
     const long long M = (long long)g.B * g.Hi * g.Wi;
     if (M < 4000000 || M > 0x7fff0000ll) return false;  // (pixels are 32-bit numbers here)
-    return dgrad_shape(a, g, ldy, wt_ld) && plan_first(a, f, g.Hi, g.Wi, g.Ci, g.B) && M >= (g.Co == 64 ? 350ll : 390ll) * a.tiles;
-}
-
-bool halo_first_covers(const ConvGeom &g, int ldy, int wt_ld, const uint32_t *mask_bits, const FirstGrad &q) {
-    Args a = {};
-    First f = {};
-    return first_shape(a, f, g, ldy, wt_ld, mask_bits, q);
+    return dgrad_shape(a, g, ldy, wt_ld) && plan_first(a, f, g.Hi, g.Wi, g.B) && M >= (g.Co == 64 ? 350ll : 390ll) * a.tiles;
 }
 
 template <int KS>
 static int launch_first(const Args &a, const First &f, const __half *depth, cudaStream_t st) {
     const int sms = ppo_num_sms();
     static PerDevice<bool> set;
-    const auto fn = conv_halo_first_kernel<32, KS, 3>;
+    const auto fn = conv_halo_first_kernel<KS>;
     PPO_TRY(ppo_once_per_device(set, [&] { return ppo_allow_smem(fn, kSmemMax); }));
-    return ppo_launch(fn, dim3((unsigned)(f.blocks < sms ? f.blocks : sms)), dim3(kFirstThreads<32, 3>), a.smem, st, a, f, depth);
+    return ppo_launch(fn, dim3((unsigned)(f.blocks < sms ? f.blocks : sms)), dim3(kFirstThreads), a.smem, st, a, f, depth);
 }
 
 int halo_dgrad_first(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, int wt_ld, const uint32_t *mask_bits, const FirstGrad &q,
@@ -1138,7 +1119,5 @@ int halo_dgrad_first(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt,
     f.px_per_warp = q.px_per_warp;
     f.blocks = q.blocks;
     f.part = q.part;
-    const int ks = a.CB >> 4;
-    if (ks == 4) return launch_first<4>(a, f, depth, st);
-    return ks == 2 ? launch_first<2>(a, f, depth, st) : launch_first<1>(a, f, depth, st);
+    return a.CB == 64 ? launch_first<4>(a, f, depth, st) : launch_first<2>(a, f, depth, st);
 }

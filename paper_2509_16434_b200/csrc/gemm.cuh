@@ -73,7 +73,6 @@ struct FirstGrad {
     int blocks, px_per_warp;
     float *part;
 };
-bool halo_first_covers(const ConvGeom &g, int ldy, int wt_ld, const uint32_t *mask_bits, const FirstGrad &q);
 int halo_dgrad_first(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, int wt_ld, const uint32_t *mask_bits, const FirstGrad &q,
                      const __half *depth, int32_t *status, cudaStream_t st);
 size_t tma_dgrad_weight_elems(int Ci, int k, int wt_ld);

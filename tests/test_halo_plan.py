@@ -216,7 +216,7 @@ int main(int argc, char **argv) {
     a.nloads = a.nchunks = Co / a.CB;
     a.N = 128;
     a.w_chunk = 9u * 32 * a.rb;
-    if (!plan_first(a, f, Hi, Wi, 32, 512)) return printf("no plan\n"), 2;
+    if (!plan_first(a, f, Hi, Wi, 512)) return printf("no plan\n"), 2;
     r.groups = f.groups;
     r.xsegs = a.xsegs;
     r.nstages = v[5];
