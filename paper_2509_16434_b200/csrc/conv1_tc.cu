@@ -23,6 +23,7 @@
 // 0.41 -> 0.25 (0.22); 160x120 3x3 16 filters normalised 0.51 -> 0.29 (0.22).
 // Frames must hold finite values (an Inf or NaN beside a window would meet a zero weight) and have an even
 // width.
+#include "conv1_window.h"
 #include "gemm.cuh"
 #include "launch.cuh"
 #include "tcgen05.cuh"
@@ -83,14 +84,11 @@ __host__ __device__ constexpr uint32_t idesc_f16(int M, int N) {
     return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-// K layout of a window of size KS: window row kh holds NP pairs; pair q covers frame columns
-// 2 ow - P - ODD + 2 q (+1), element e of it is kernel column 2 q + e - ODD (outside 0 .. KS-1: zero filter entry).
-// Halves 2 KS NP and 2 KS NP + 1 carry the constant 1 for the two bias parts; the rest up to KP are zero.
+// K layout of a window (conv1_window.h): halves 2 KS NP and 2 KS NP + 1 carry the constant 1 for the two bias parts; the rest up to KP are
+// zero, as are the filter entries of kernel columns outside 0 .. KS-1.
 template <int KS>
-struct Win {
-    static constexpr int P = KS / 2, ODD = P & 1, NP = (KS + ODD + 1) / 2;
-    static constexpr int KW = KS * NP;                     // 32-bit words of window data
-    static constexpr int KP = (2 * KW + 2 + 15) / 16 * 16; // halves per im2col row
+struct Win : Window<KS> {
+    static constexpr int KP = (2 * Window<KS>::KW + 2 + 15) / 16 * 16;  // halves per im2col row
 };
 
 // Output pixel of a walk through the frames, advanced without divisions.

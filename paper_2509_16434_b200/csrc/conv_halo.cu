@@ -20,6 +20,7 @@
 // (0.58; tap boxes whose tiles go in pairs of CTAs take 0.90, and that forward pass), input gradient 1.58 -> 1.01 to 1.07 (0.6).
 #include <cuda.h>
 
+#include "conv1_window.h"
 #include "gemm.cuh"
 #include "halo_plan.h"
 #include "launch.cuh"
@@ -141,80 +142,41 @@ __device__ __forceinline__ uint32_t ring_offset(int row, int piece) {
     return (uint32_t)line * 128u + ((uint32_t)(q ^ (line & 7)) << 4);
 }
 
-__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t addr, uint32_t &r0, uint32_t &r1, uint32_t &r2, uint32_t &r3) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(addr) : "memory");
-}
-__device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
 // Builder warp bw: the window tiles of the pixels p0 .. p1, [32 px][TP] bf16, four trips to a stage; trip bw % 4 of every second
 // stage.
 // The builders also stand between ring and sums, whose loop is the kernel's longest chain: a stage is handed over when its pixels
 // have arrived in the ring, and the first of them gives a row group back when it has seen the stage it ends in summed.
 __device__ __forceinline__ void first_windows(const First &f, int H1, int W1, const __half *depth, int p0, int p1, const GroupWalk &at, int bw,
                                               uint8_t *patch, FirstPipe *pipe, int32_t *status) {
-    constexpr int TP = Win::TP, KW = Win::KW, NP = Win::NP, P = Win::P, ODD = Win::ODD;
+    constexpr int TP = Window<kFirstK>::TP;
     const int lane = threadIdx.x & 31, nstages = (p1 - p0 + kStagePx - 1) / kStagePx;
     const uint32_t *const frames = reinterpret_cast<const uint32_t *>(depth);
     const int Hf = held(f.Hf), Wh = held(f.Wh);
     H1 = held(H1);
     W1 = held(W1);
     int m = p0 + (bw >> 2) * kStagePx + (bw & 3) * kTrip + lane;
-    int ow = m % W1, oh = m / W1 % H1;
-    long long b = m / W1 / H1;
+    WindowWalk<kFirstK> px;
+    px.init(m, W1, H1);
     const int d_oh = 2 * kStagePx / W1, d_ow = 2 * kStagePx - d_oh * W1;
-    uint32_t raw[KW];
+    uint32_t raw[Window<kFirstK>::KW];
     bool live = false;
-    // A trip's loads are issued a turn ahead of their use.  A pair outside the frame is a predicated load that leaves its zero.
-    auto fetch = [&]() {
+    auto fetch = [&]() {  // a trip's loads, a turn ahead of their use
         live = m < p1;
-        const int pw0 = ow - (P + ODD) / 2, ih0 = 2 * oh - P;
-        const uint32_t *row = frames + ((b * Hf + ih0) * Wh + pw0);
-        bool cok[NP];
-#pragma unroll
-        for (int q = 0; q < NP; ++q) cok[q] = live && (unsigned)(pw0 + q) < (unsigned)Wh;
-#pragma unroll
-        for (int kh = 0; kh < Win::K; ++kh) {
-            const bool rok = (unsigned)(ih0 + kh) < (unsigned)Hf;
-#pragma unroll
-            for (int q = 0; q < NP; ++q) {
-                raw[kh * NP + q] = 0u;
-                if (rok && cok[q]) raw[kh * NP + q] = __ldg(row + q);
-            }
-            row += Wh;
-        }
+        px.fetch(frames, Hf, Wh, live, raw);
         m += 2 * kStagePx;
-        ow += d_ow;
-        if (ow >= W1) { ow -= W1; ++oh; }
-        oh += d_oh;
-        while (oh >= H1) { oh -= H1; ++b; }
+        px.advance(d_ow, d_oh, W1, H1);
     };
     fetch();
     uint8_t *const mine = patch + (size_t)((bw & 3) * kTrip + lane) * (TP * 2);
-    const int sw = (lane >> 2) & 1;
     GroupWalk seen = at, done = at;
     int avail = at.slot, ended = at.slot + at.px();  // pixels of the run that have arrived; end of group `done`
     for (int s = bw >> 2; s < nstages; s += 2) {
         uint32_t wv[TP / 2];
-#pragma unroll
-        for (int k = 0; k < TP / 2; ++k) wv[k] = 0u;
-#pragma unroll
-        for (int k = 0; k < KW; ++k) {
-            const float2 v = __half22float2(*reinterpret_cast<const __half2 *>(&raw[k]));
-            wv[k] = pack_bf16x2(v.x, v.y);
-        }
-        if (live) wv[KW] = 0x00003F80u;  // (1.0, 0) as bf16: the bias-gradient column
+        window_row<kFirstK>(raw, live, wv);
         fetch();
         const int slot = s & (kWinStages - 1);
         if (!mbar_wait_warp(&pipe->pempty[slot], (uint32_t)(s / kWinStages & 1) ^ 1u, &pipe->abort_flag, status)) return;
-        uint8_t *const row = mine + (size_t)slot * (kStagePx * TP * 2);
-#pragma unroll
-        for (int c = 0; c < TP / 8; ++c)
-            *reinterpret_cast<uint4 *>(row + ((c ^ sw) << 4)) = make_uint4(wv[4 * c], wv[4 * c + 1], wv[4 * c + 2], wv[4 * c + 3]);
+        put_row(mine + (size_t)slot * (kStagePx * TP * 2), lane, wv);
         if (ring_gives_back(bw))
             for (; ended <= ring_summed(s); ended += done.px()) {  // (the first stages have nothing before them)
                 if (lane == 0) mbar_arrive(&pipe->gempty[done.i]);
@@ -238,13 +200,14 @@ __device__ __forceinline__ void first_windows(const First &f, int H1, int W1, co
 // units make shorter chains of more shared-memory reads: 8 channels a unit 490 us, 16 channels 450 to 475.
 __device__ __forceinline__ void first_sums(const First &f, int p0, int p1, int block0, int ring_px, int unit, uint32_t ring, uint32_t patch,
                                            FirstPipe *pipe, int32_t *status) {
-    constexpr int TP = Win::TP, KW = Win::KW, NP = Win::NP, ODD = Win::ODD, K1 = Win::K, K2 = K1 * K1, C1 = kFirstC;
+    using WN = Window<kFirstK>;
+    constexpr int TP = WN::TP, KW = WN::KW, NP = WN::NP, ODD = WN::ODD, K1 = kFirstK, K2 = K1 * K1, C1 = kFirstC;
     const int lane = threadIdx.x & 31, mi = lane >> 3, r = lane & 7, uj = 2 * unit;
     uint32_t a_off[2], b_off[2];
 #pragma unroll
     for (int ks = 0; ks < 2; ++ks) {
-        const int ar = 16 * ks + r + (mi >= 2 ? 8 : 0), sw = (ar >> 2) & 1;
-        a_off[ks] = (uint32_t)(ar * (TP * 2) + (((mi & 1) ^ sw) << 4));
+        const int ar = 16 * ks + r + (mi >= 2 ? 8 : 0), c = (mi & 1) ^ piece_swizzle(ar, TP * 2);
+        a_off[ks] = (uint32_t)(ar * (TP * 2) + (c << 4));
     }
 #pragma unroll
     for (int j = 0; j < 2; ++j) b_off[j] = ring_offset(lane, uj + j);  // (a trip starts at a multiple of 32 pixels)
@@ -363,7 +326,7 @@ __device__ __forceinline__ void first_sums(const First &f, int p0, int p1, int b
 template <int MODE, int GC, int KS, int EPW, bool FIRST>
 __device__ __forceinline__ void halo_body(const Args &a, const First &f, const __half *depth, uint8_t *smem_raw) {
     constexpr int NH = EPW == 4 ? 2 : 1;  // halves of 64 columns a warp works on
-    constexpr uint32_t kPatchBytes = kWinStages * kStagePx * Win::TP * 2;
+    constexpr uint32_t kPatchBytes = kWinStages * kStagePx * Window<kFirstK>::TP * 2;
     static_assert(!FIRST || (MODE == DG && GC == kFirstC && EPW == 4), "");
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t smem_base = smem_u32(smem);
@@ -1090,7 +1053,7 @@ int halo_conv_dgrad(const ConvGeom &g, const bf16 *dY, int ldy, const bf16 *Wt, 
 // 5x5 windows (twice the fragments, 2.5 times the loads of a builder) take longer than the two kernels at all sizes, and so do 16 channels
 // of the first layer: half as much dX to keep out of HBM for the same chain.
 static bool first_shape(Args &a, First &f, const ConvGeom &g, int ldy, int wt_ld, const uint32_t *mask_bits, const FirstGrad &q) {
-    if (q.k != Win::K || g.Ci != kFirstC || (g.Co != 32 && g.Co != 64) || !mask_bits || q.Wf % 2 != 0) return false;
+    if (q.k != kFirstK || g.Ci != kFirstC || (g.Co != 32 && g.Co != 64) || !mask_bits || q.Wf % 2 != 0) return false;
     const long long M = (long long)g.B * g.Hi * g.Wi;
     if (M < 4000000 || M > 0x7fff0000ll) return false;  // (pixels are 32-bit numbers here)
     return dgrad_shape(a, g, ldy, wt_ld) && plan_first(a, f, g.Hi, g.Wi, g.B) && M >= (g.Co == 64 ? 350ll : 390ll) * a.tiles;

@@ -3,6 +3,7 @@
 #include <new>
 
 #include "common.cuh"
+#include "conv1_window.h"
 #include "launch.cuh"
 #include "gemm.cuh"
 #include "lstm.cuh"
@@ -221,32 +222,16 @@ __global__ void __launch_bounds__(128) conv1_wgrad_kernel(const __half *__restri
 // outside the window and its row of D is dropped -- followed by a column of ones whose product is the bias gradient,
 // zero padded to TP.  About 3 instructions per pixel and channel-independent instead of C1 (k*k + 1) / 32 multiply-adds
 // plus their loads: the kernel becomes a stream over dZ.  C1 must be a multiple of 16 and the frame width even.
-__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t addr, uint32_t &r0, uint32_t &r1, uint32_t &r2, uint32_t &r3) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
-                 : "r"(addr));
-}
-__device__ __forceinline__ void mma_bf16_16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
-                                               uint32_t b0, uint32_t b1) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
 template <int KS, int NB>  // NB = C1 / 8 column blocks
 __global__ void __launch_bounds__(256) conv1_wgrad_mma_kernel(const __half *__restrict__ depth,
                                                               const bf16 *__restrict__ dZ, float *__restrict__ part,
                                                               int rows, int Hi, int Wi,
                                                               int Ho, int Wo, long long px_per_warp) {
     grid_wait();
-    constexpr int K2 = KS * KS, P = KS / 2, ODD = P & 1, NP = (KS + ODD + 1) / 2, KW = KS * NP;
-    constexpr int TP = (2 * KW + 1 + 15) / 16 * 16, MB = TP / 16, C1 = NB * 8;
+    using WN = Window<KS>;
+    constexpr int K2 = KS * KS, ODD = WN::ODD, NP = WN::NP, KW = WN::KW, TP = WN::TP, MB = TP / 16, C1 = NB * 8;
     constexpr int PX = 32;  // pixels per trip: one per lane, two K = 16 steps of the MMA
     constexpr int kXBytes = PX * TP * 2, kZBytes = PX * C1 * 2;
-    // 16-byte piece c of row r of a tile sits at piece c ^ f(r): rows of 32, 64 or 128 bytes would otherwise put the
-    // same piece of several rows into the same banks, on the way in as on the way out (ldmatrix reads a column of pieces)
-    auto swz = [](int r, int row_bytes) { return row_bytes == 128 ? r & 7 : (row_bytes == 64 ? (r >> 1) & 3 : (row_bytes == 32 ? (r >> 2) & 1 : 0)); };
     extern __shared__ __align__(16) uint8_t smw[];  // per warp: X tile [32 px][TP], dZ tile [32 px][C1]; later the reduction
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint8_t *xs = smw + (size_t)warp * (kXBytes + kZBytes), *zs = xs + kXBytes;
@@ -262,42 +247,21 @@ __global__ void __launch_bounds__(256) conv1_wgrad_mma_kernel(const __half *__re
     const long long gw = (long long)blockIdx.x * 8 + warp;
     long long m0 = gw * px_per_warp;                       // px_per_warp is a multiple of 32
     const long long m_end = min(M, m0 + px_per_warp);
-    int ow = 0, oh = 0;  // this lane's pixel m0 + lane
-    long long b = 0;
-    if (m0 < m_end) {
-        const long long m = m0 + lane;
-        ow = (int)(m % Wo);
-        const long long t = m / Wo;
-        oh = (int)(t % Ho);
-        b = t / Ho;
-    }
+    WindowWalk<KS> at = {0, 0, 0};  // this lane's pixel m0 + lane
+    if (m0 < m_end) at.init(m0 + lane, Wo, Ho);
     const int d_oh = PX / Wo, d_ow = PX % Wo;  // 32 pixels further (Wo >= 1)
     constexpr int ZP = PX * C1 / 8 / 32;       // 16-byte pieces of the gradient tile per lane
     uint32_t raw[KW];                          // this lane's window, zero outside the frame
     bool live = false;
     uint4 zreg[ZP];
     // Loads of the tile that starts at pixel mt into registers; they are issued one trip ahead, so that their
-    // latency overlaps the previous tile's MMAs.  The kernel is bound by its instructions as much as by HBM: a pair outside
-    // the frame is a predicated load that leaves its zero, a full tile takes its gradient rows without tests.
+    // latency overlaps the previous tile's MMAs.  The kernel is bound by its instructions as much as by HBM: a full tile takes
+    // its gradient rows without tests.
     const int Wh = Wi >> 1;  // 32-bit words per frame row
     const uint32_t *const frames = reinterpret_cast<const uint32_t *>(depth);
     auto prefetch = [&](long long mt) {
         live = mt + lane < m_end;
-        const int pw0 = ow - (P + ODD) / 2, ih0 = 2 * oh - P;
-        const uint32_t *row = frames + ((b * Hi + ih0) * Wh + pw0);
-        bool cok[NP];
-#pragma unroll
-        for (int q = 0; q < NP; ++q) cok[q] = live && (unsigned)(pw0 + q) < (unsigned)Wh;
-#pragma unroll
-        for (int kh = 0; kh < KS; ++kh) {
-            const bool rok = (unsigned)(ih0 + kh) < (unsigned)Hi;
-#pragma unroll
-            for (int q = 0; q < NP; ++q) {
-                raw[kh * NP + q] = 0u;
-                if (rok && cok[q]) raw[kh * NP + q] = __ldg(row + q);
-            }
-            row += Wh;
-        }
+        at.fetch(frames, Hi, Wh, live, raw);
         if (mt + PX <= m_end) {
 #pragma unroll
             for (int z = 0; z < ZP; ++z) zreg[z] = __ldcs(reinterpret_cast<const uint4 *>(dZ + mt * C1) + lane + 32 * z);
@@ -312,31 +276,16 @@ __global__ void __launch_bounds__(256) conv1_wgrad_mma_kernel(const __half *__re
     };
     if (m0 < m_end) prefetch(m0);
     for (; m0 < m_end; m0 += PX) {
-        {   // conversion here, a trip after the loads were issued: at their side it would wait for them on the spot
-            uint32_t wv[TP / 2];
-#pragma unroll
-            for (int k = 0; k < TP / 2; ++k) wv[k] = 0u;
-#pragma unroll
-            for (int k = 0; k < KW; ++k) {
-                const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&raw[k]));
-                wv[k] = pack_bf16x2(f.x, f.y);
-            }
-            if (live) wv[KW] = 0x00003F80u;  // (1.0, 0) as bf16: the bias-gradient column
-#pragma unroll
-            for (int c = 0; c < TP / 8; ++c)
-                *reinterpret_cast<uint4 *>(xs + lane * (TP * 2) + ((c ^ swz(lane, TP * 2)) * 16)) =
-                    make_uint4(wv[4 * c], wv[4 * c + 1], wv[4 * c + 2], wv[4 * c + 3]);
-        }
+        uint32_t wv[TP / 2];  // converted here, a trip after the loads were issued: at their side it would wait for them
+        window_row<KS>(raw, live, wv);
+        put_row(xs + lane * (TP * 2), lane, wv);
 #pragma unroll
         for (int z = 0; z < ZP; ++z) {
             const int i = lane + 32 * z, zr = i / (C1 / 8), zc = i % (C1 / 8);
-            reinterpret_cast<uint4 *>(zs)[zr * (C1 / 8) + (zc ^ swz(zr, C1 * 2))] = zreg[z];
+            reinterpret_cast<uint4 *>(zs)[zr * (C1 / 8) + (zc ^ piece_swizzle(zr, C1 * 2))] = zreg[z];
         }
         __syncwarp();
-        ow += d_ow;
-        if (ow >= Wo) { ow -= Wo; ++oh; }
-        oh += d_oh;
-        while (oh >= Ho) { oh -= Ho; ++b; }
+        at.advance(d_ow, d_oh, Wo, Ho);
         if (m0 + PX < m_end) prefetch(m0 + PX);
         // ---- fragments and MMAs, 16 pixels per K step
 #pragma unroll
@@ -347,20 +296,20 @@ __global__ void __launch_bounds__(256) conv1_wgrad_mma_kernel(const __half *__re
             for (int i = 0; i < MB; ++i) {
                 // matrices: (taps 16i..+7, px 0-7), (taps 16i+8.., px 0-7), (taps 16i.., px 8-15), (taps 16i+8.., px 8-15)
                 const int row = 16 * ks + r + (mi >= 2 ? 8 : 0);
-                const uint32_t addr = xs_a + (uint32_t)(row * (TP * 2) + ((2 * i + (mi & 1)) ^ swz(row, TP * 2)) * 16);
+                const uint32_t addr = xs_a + (uint32_t)(row * (TP * 2) + ((2 * i + (mi & 1)) ^ piece_swizzle(row, TP * 2)) * 16);
                 ldmatrix_x4_trans(addr, af[i][0], af[i][1], af[i][2], af[i][3]);
             }
 #pragma unroll
             for (int j = 0; j < NB; j += 2) {
                 // matrices: (px 0-7, co 8j..), (px 8-15, co 8j..), (px 0-7, co 8j+8..), (px 8-15, co 8j+8..)
                 const int row = 16 * ks + r + (mi & 1) * 8;
-                const uint32_t addr = zs_a + (uint32_t)(row * (C1 * 2) + ((j + (mi >> 1)) ^ swz(row, C1 * 2)) * 16);
+                const uint32_t addr = zs_a + (uint32_t)(row * (C1 * 2) + ((j + (mi >> 1)) ^ piece_swizzle(row, C1 * 2)) * 16);
                 uint32_t b0, b1, b2, b3;
                 ldmatrix_x4_trans(addr, b0, b1, b2, b3);
 #pragma unroll
                 for (int i = 0; i < MB; ++i) {
-                    mma_bf16_16816(acc[i][j], af[i][0], af[i][1], af[i][2], af[i][3], b0, b1);
-                    mma_bf16_16816(acc[i][j + 1], af[i][0], af[i][1], af[i][2], af[i][3], b2, b3);
+                    mma_bf16_16816(acc[i][j], af[i], b0, b1);
+                    mma_bf16_16816(acc[i][j + 1], af[i], b2, b3);
                 }
             }
         }

@@ -4,6 +4,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include "conv1_window.h"
+
 #ifdef __CUDACC__
 #define PPO_HALO_FN __host__ __device__ constexpr
 #else
@@ -17,7 +19,8 @@ constexpr int kMaxGroups = 8;   // row groups of the ring between the input grad
 constexpr int kWinStages = 4;   // stages of window tiles, of four trips of 32 pixels each
 constexpr int kTrip = 32, kStagePx = 4 * kTrip;
 constexpr int kBuildWarps = 8;  // in two sets of four
-constexpr int kFirstC = 32;     // channels of the first layer
+constexpr int kFirstK = 3, kFirstC = 32;  // of the first layer: 3x3, 32 channels
+static_assert(Window<kFirstK>::TP == 16, "one row of fragments");
 constexpr int kUnits = kFirstC / 16;  // warps that sum
 constexpr int kMaxOps = 9;
 constexpr size_t kSmemMax = 227 * 1024;
@@ -96,14 +99,6 @@ struct FirstPipe : Pipe {
     uint64_t gfull[kMaxGroups], gempty[kMaxGroups], pfull[kWinStages], pempty[kWinStages];
 };
 
-
-// Window of the first layer (3x3) as aligned pairs of fp16 frame pixels, one row of the weight gradient per pair element and one for the
-// bias.
-struct Win {
-    static constexpr int K = 3, P = K / 2, ODD = P & 1, NP = (K + ODD + 1) / 2, KW = K * NP;
-    static constexpr int TP = (2 * KW + 1 + 15) / 16 * 16;
-    static_assert(TP == 16, "one row of fragments");
-};
 
 inline uint32_t stage_rows_bytes(int rows, int row_bytes) { return ((uint32_t)(rows * row_bytes) + 1023u) & ~1023u; }
 
@@ -219,7 +214,7 @@ PPO_HALO_FN int ring_needs(int s, int total) {
 inline bool plan_first(Args &a, First &f, int Hi, int Wi, int B) {
     const int Wr = (Wi + 1) / 2, Hr = (Hi + 1) / 2, C1 = kFirstC;
     const size_t w = ((size_t)a.nchunks * a.w_chunk + 1023) & ~size_t(1023);
-    const size_t patch = (size_t)kWinStages * kStagePx * Win::TP * 2;
+    const size_t patch = (size_t)kWinStages * kStagePx * Window<kFirstK>::TP * 2;
     const size_t fixed = w + patch + sizeof(FirstPipe) + 2048;
     if (fixed >= kSmemMax) return false;
     const size_t room = kSmemMax - fixed;
