@@ -30,11 +30,11 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of the encoder kernels of one forward + backward per
-# sample row, from ncu captures of small twins of the workloads (traffic grows in proportion to the rows): workload
+# sample row, from ncu captures of small twins or micro-batches of the workloads (traffic grows in proportion to the rows): workload
 # -> (bytes per row, capture).  An entry is dropped (traffic: null) as soon as a kernel it covers changes.
 NCU_DRAM_BYTES_PER_ROW = {
-    "cfg2": (2.6872e6, "ncu capture of cfg2_prof at 512 rows, scaled by rows: profiles/ncu_main_kernels_cfg2_prof.txt"),
-    "cfg3": (2.6872e6, "ncu capture of cfg2_prof at 512 rows, scaled by rows: profiles/ncu_main_kernels_cfg2_prof.txt"),
+    "cfg2": (2.3645e6, "ncu capture of cfg2 in micro-batches of 1024 rows, scaled by rows: profiles/ncu_main_kernels_cfg2.txt"),
+    "cfg3": (2.3645e6, "ncu capture of cfg2 in micro-batches of 1024 rows, scaled by rows: profiles/ncu_main_kernels_cfg2.txt"),
     "cfg2_prof": (2.6872e6, "ncu capture of cfg2_prof at 512 rows: profiles/ncu_main_kernels_cfg2_prof.txt"),
     "cfg4": (11.1422e6, "ncu capture of cfg4_prof at 128 rows, scaled by rows: profiles/ncu_main_kernels_cfg4_prof.txt"),
     "cfg4_prof": (11.1422e6, "ncu capture of cfg4_prof at 128 rows: profiles/ncu_main_kernels_cfg4_prof.txt"),
@@ -360,9 +360,9 @@ def run_ours(args):
         gather_gbs = 2 * (rows if w.n_lstm else w.B) * record_bytes(w) / (gat_ms * 1e-3) / 1e9
         gae_gbs = (17 + 8) * w.M / (gae_ms * 1e-3) / 1e9
         adam_gbs = 30 * L.model.arena / (adam_ms * 1e-3) / 1e9
-        # DRAM bytes of the encoder's GEMM and conv1 kernels per sample row (dram__bytes_read + write summed over the 15
-        # launches of one forward + backward, ncu capture of the cfg2 network at 512 rows: profiles/ncu_main_kernels_cfg2_prof.txt);
-        # traffic grows in proportion to the rows.  Valid for the cfg2/cfg3 network only, and only while those kernels are unchanged.
+        # DRAM bytes of the encoder's GEMM and conv1 kernels per sample row (dram__bytes_read + write summed over the launches of
+        # one forward + backward); traffic grows in proportion to the rows.  Valid only while those kernels are unchanged, and for
+        # the cfg2 network in micro-batches of at least 834 rows (4 M pixels of the first layer).
         per_row, capture = NCU_DRAM_BYTES_PER_ROW.get(w.name, (None, "no ncu capture of the current kernels at this workload"))
         traffic = per_row * mean_rows if per_row else None
         roofline = {"bound": "tensor",

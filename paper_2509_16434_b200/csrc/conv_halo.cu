@@ -839,10 +839,10 @@ __global__ void __maxnreg__(96) conv_halo_kernel(const __grid_constant__ Args a)
 // The input gradient of the second convolution and from it, on chip, the weight gradient of the first one, which is all it is for: the
 // gradient of the first layer's output, the largest of all, does not go through HBM (2.5 GB of writes and reads at 4096 rows of
 // 160 x 120 and 32 channels).  Its tiles' rows go into a ring of pixels in the order of the image, builder warps make the windows
-// of the frames, and two warps sum runs of pixels (mma.sync, as conv1_wgrad_mma_kernel: same bits).  What bounds it: the chain of
-// a run (500 cycles for 128 pixels by itself) and shared memory's bandwidth, which tensor core, fragments, windows and ring have to
-// share (800 cycles in place; tensor core alone 215 of them, epilogue 720 on two groups).  Measured at that size: 330 + 290 us -> 460, a
-// minibatch 3.22 -> 3.12 ms.
+// of the frames, and two warps sum runs of pixels (mma.sync, as conv1_wgrad_mma_kernel: same bits).  What bounds it: the epilogue,
+// whose two groups need 720 of the 800 cycles that 128 pixels take; the chain of a run needs 500, the tensor core 215.  Nothing is near
+// a limit of the chip (counters at 1024 rows: 2.0 instructions per cycle, shared memory's pipe 30 %, tensor pipe 25 %, DRAM 21 %).
+// Measured at that size: 330 + 290 us -> 460, a minibatch 3.22 -> 3.12 ms.
 // (depth is the last argument: a prepared launch is made again with other frames.)
 constexpr int kFirstThreads = (10 + kBuildWarps + kUnits) * 32;
 template <int KS>

@@ -669,7 +669,8 @@ extern "C" int ppo_policy_sample(const ppo_model *m, int rows, const float *mean
 // The forward pass of a decision and what follows it: in the kernels that end the pass where they can, else in launches of their own.  A
 // launch costs the host 4 to 6 us and a small kernel the GPU 2, and a decision of few envs is bound by both: with the sampling in
 // the head's kernel, the states in the step kernels and the first layer's launch prepared once, the paper's policy takes 10 launches
-// instead of 13: 16 envs 84 -> 77 us, 64 92.5 -> 89, 512 206.5 -> 200.5.
+// instead of 13: 16 envs 84.5 -> 81.4 us, 512 205.6 -> 201.0.  (The head's kernel pays 2 us of that back: it samples behind its last
+// accumulator.)
 static int decide(ppo_model *m, const ppo_minibatch *obs, int row0, int rows, float *mean, float *value, ActTail tail, void *stream) {
     m->tail = &tail;
     const int s = ppo_encoder_fwd(m, obs, row0, rows, mean, value, stream);
